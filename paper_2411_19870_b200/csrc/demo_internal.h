@@ -27,6 +27,7 @@ struct DemoCompressArgs {
     const DemoTensorEntry *entries;  // device
     int n_entries;
     long long n_chunks;
+    int k;                      // k_eff of the list's tensors (one chunk size per list, so one k_eff)
     const void *const *g_ptrs;  // device array indexed by DemoTensorEntry::tensor
     float *const *m_ptrs;       // device array
     DemoRecord *payload;        // device, whole payload of this worker

@@ -675,6 +675,7 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
         a.entries = ctx->d_entries1d;
         a.n_entries = ctx->n1d;
         a.n_chunks = ctx->chunks1d;
+        a.k = ctx->cfg.topk < s ? ctx->cfg.topk : s;
         err = demo_launch_compress_generic(s, 0, a, ctx->sm_count, side);
         ctx->launches += 1;
     }
@@ -682,6 +683,7 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
         a.entries = ctx->d_entries2d;
         a.n_entries = ctx->n2d;
         a.n_chunks = ctx->chunks2d;
+        a.k = ctx->cfg.topk;  // <= s * s
         a.momentum_dct = ctx->momentum_dct ? 1 : 0;
         if (use_fast_path(ctx))
             err = demo_launch_compress_fast(s, a, ctx->sm_count, stream);

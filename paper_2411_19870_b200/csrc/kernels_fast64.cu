@@ -38,17 +38,23 @@ constexpr int CAPWP = CAPW + 4;
 constexpr int WCAP = 512;     // capacity of the wide candidate list (out-of-line path)
 constexpr int TMEM_COLS_PER_GROUP = 64;  // one column block per four warps (two slots)
 constexpr int ROW_AHEAD = 8;              // entries of the row-stage list fetched ahead
+// Up to this k the k-th largest of the 64 row maxima bounds the top-k well enough (k = 48: about 90 candidates in a dense
+// tile, k = 64: about 260) and the row stage of the inverse is cheaper from the list of records; above it the kernel
+// variant with a bound from 256 quarter rows and a dense row stage takes over.  Measured, 4096 x 4096, one compress call:
+// k = 40 / 48 from the list 53.7 / 57.2 us, k = 49 / 64 / 96 / 128 with the dense row stage 56.9 / 57.4 / 58.5 / 59.5 us
+// (59 / 80 / 102 / 120 us from a list with the selection out of line); 8192 x 8192, k = 128: 430 -> 205 us.
+constexpr int MAX_K_LISTED = 48;
 
 // Tile area of a slot:  [0, 64*68*4)  the padded transpose / coefficient / row-stage tile X; its first 16 KB double as
 // the landing area of the m tile and as the source of the TMA store of the new momentum;  behind it the landing
-// area of the g tile, which between its two uses holds the lists of the selection: wide candidate list, big-k list, and -- at its
-// end -- the row-stage list.
+// area of the g tile, which between its two uses holds the lists of the selection: wide candidate list and -- at its end -- the
+// row-stage list.
 constexpr size_t TILE_X_BYTES = (size_t)S * XS * sizeof(float);
 template <typename GT>
 constexpr size_t region_bytes()
 {
     constexpr size_t g_bytes = (size_t)S * S * sizeof(GT);
-    constexpr size_t lists = (size_t)(WCAP + 4) * 8 + 256 * 8 + 65 * 16;  // wide list + big-k list + row-stage list
+    constexpr size_t lists = (size_t)(WCAP + 4) * 8 + 65 * 16;  // wide list + row-stage list
     static_assert(lists <= g_bytes, "the selection's lists live in the g landing area");
     return TILE_X_BYTES + g_bytes;
 }
@@ -72,14 +78,77 @@ struct SlotMem {
     unsigned *misc;      // [16]
     unsigned *wkey;      // [WCAP + 4] wide list, behind the tile
     unsigned *widx;      // [WCAP + 4]
-    uint2 *rbig;         // [256] kept records for 64 < k <= 256: (row << 16 | column, alpha * value), behind the wide list
 };
 
+// How the selection leaves the kept coefficients besides the records: as the list of the sparse row stage, in the
+// coefficient tile as q - alpha q (momentum in the transform domain), or as the tile itself with alpha q at the kept
+// places and zero elsewhere.
+enum { SELECT_LISTED, SELECT_QDOM, SELECT_DENSE };
+
 // ------------------------------------------------------------------------------------------------
-// Out-of-line selection for the chunks the in-line path does not take: more than 64 candidates in a
-// warp's list (tiles of low rank or with a concentrated spectrum, tied or degenerate chunks), fewer
-// candidates than k (NaN coefficients) or k > 64 (for 64 < k <= 256 the bound comes from step 2 alone).  Works from the coefficient tile in X (row t is
-// this thread's), writes the records to `rec` and, for k <= 64, the pre-decoded list for the row stage.
+// Exact 4 x 8-bit radix select over the coefficient tile in X (complete for every thread of the slot), any k: the
+// last resort of both variants below (tied or degenerate chunks, non-finite values, k > 256).
+// ------------------------------------------------------------------------------------------------
+__device__ __noinline__ void select_radix(const SlotMem sm, int k_eff, DemoRecord *rec, float alpha, int t, int bar_id, int mode)
+{
+    const SlotBarrier<S> sb{bar_id};
+    const int lane = t & 31, warp = t >> 5;
+    float *X = sm.X;
+    unsigned *misc = sm.misc;
+    unsigned thr, need_eq;
+    sb.sync();
+    radix_select_tile<S, XS>(X, k_eff, sm.hist, misc, &thr, &need_eq, t, sb);
+    unsigned gt = 0, eq = 0;
+#pragma unroll 1
+    for (int v = 0; v < S; ++v) {
+        const unsigned key = mag_key(X[t * XS + v]);
+        gt += key > thr;
+        eq += key == thr;
+    }
+    const unsigned packed = gt | (eq << 16);
+    const unsigned inc = warp_inclusive_scan(packed, lane);
+    sb.sync();  // radix_select_tile's last reads of misc are done
+    if (lane == 31) misc[warp] = inc;
+    sb.sync();
+    unsigned before = inc - packed;
+    if (warp == 1) before += misc[0];
+    unsigned gb = before & 0xffffu, eb = before >> 16;
+#pragma unroll 1
+    for (int v = 0; v < S; ++v) {
+        const float val = X[t * XS + v];
+        const unsigned key = mag_key(val);
+        bool s = false;
+        unsigned pos = 0;
+        if (key > thr) {
+            pos = gb + min(eb, need_eq);
+            ++gb;
+            s = true;
+        } else if (key == thr) {
+            if (eb < need_eq) {
+                pos = gb + eb;
+                s = true;
+            }
+            ++eb;
+        }
+        if (s) {
+            DemoRecord r;
+            r.idx = t * S + v;
+            r.val = val;
+            rec[pos] = r;
+            if (mode == SELECT_QDOM)
+                X[t * XS + v] = fmaf(-alpha, val, val);
+            else if (mode == SELECT_LISTED)
+                sm.recs4[pos] = make_int4(t * XS, v * S, __float_as_int(alpha * val), 0);
+        }
+        if (mode == SELECT_DENSE) X[t * XS + v] = s ? alpha * val : 0.f;
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Out-of-line selection (k <= MAX_K_LISTED) for the chunks the in-line path does not take: more than 64 candidates in
+// a warp's list (tiles of low rank or with a concentrated spectrum, tied or degenerate chunks) or fewer
+// candidates than k (NaN coefficients).  Works from the coefficient tile in X (row t is
+// this thread's), writes the records to `rec` and the pre-decoded list for the row stage.
 //   1. wide list: up to WCAP candidates under the bound `lmin` (the k-th largest of the 64 row maxima),
 //      every warp takes the whole list into registers and finds the exact k-th largest key by a
 //      bit-by-bit ballot search;
@@ -88,7 +157,7 @@ struct SlotMem {
 //   3. otherwise an exact 4 x 8-bit radix select over the whole tile.
 // ------------------------------------------------------------------------------------------------
 __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord *rec, float alpha, int t, int bar_id,
-                                         unsigned lmin_w, bool bound_valid, bool qdom)
+                                         unsigned lmin_w, bool qdom)
 {
     const SlotBarrier<S> sb{bar_id};
     const int lane = t & 31, warp = t >> 5;
@@ -98,7 +167,7 @@ __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord
     sb.sync();  // the coefficient tile is complete; the in-line path is done with its lists
 
     bool done = false;
-    if (k_eff <= 256) {  // (the finer bound below needs at least k groups: 256 quarter rows / quarter columns)
+    {
         unsigned long long mask = 0ull;
         unsigned off = 0, n_all = 0xffffffffu;
         auto count_under = [&](unsigned bound) {
@@ -114,10 +183,7 @@ __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord
             n_all = n0 + misc[1];
             off = inc - cnt + (warp ? n0 : 0u);
         };
-        if (bound_valid)
-            count_under(lmin_w);
-        else
-            lmin_w = 0u;  // k > 64: the row maxima give no bound, the finer partition does
+        count_under(lmin_w);
         if (n_all > (unsigned)WCAP) {
             // tighter bound: the k_eff-th largest of the 256 quarter-row maxima and of the 256 quarter-column maxima
             unsigned rk[4], ck[4];
@@ -132,15 +198,12 @@ __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord
                 }
                 rk[g] = m;
             }
-            // (the quarter-column maxima matter for tiles with a few active columns; with k > 64, where this is the
-            // ordinary path of every chunk, the quarter rows alone give the bound)
+            // (the quarter-column maxima matter for tiles with a few active columns)
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 unsigned m = 0u;
-                if (bound_valid) {
 #pragma unroll 4
-                    for (int u = 0; u < 16; ++u) m = max(m, mag_key(X[(16 * g + u) * XS + t]));
-                }
+                for (int u = 0; u < 16; ++u) m = max(m, mag_key(X[(16 * g + u) * XS + t]));
                 ck[g] = m;
             }
             unsigned *gq = sm.wkey;  // [8][64], behind the tile
@@ -179,10 +242,9 @@ __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord
                 }
                 return pre;
             };
-            unsigned l2 = kth_of_256(rk, prk);
-            if (bound_valid) l2 = max(l2, kth_of_256(ck, pck));
+            const unsigned l2 = max(kth_of_256(rk, prk), kth_of_256(ck, pck));
             sb.sync();  // gq is read; the wide list may overwrite it
-            if (l2 > lmin_w || !bound_valid) {
+            if (l2 > lmin_w) {
                 lmin_w = l2;
                 count_under(lmin_w);
             }
@@ -248,10 +310,8 @@ __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord
                             rec[pos] = r;
                             if (qdom)  // transform-domain momentum: what stays of a transmitted coefficient
                                 X[uo + v] = fmaf(-alpha, r.val, r.val);
-                            else if (k_eff <= 64)
-                                recs4[pos] = make_int4(uo, v * S, __float_as_int(alpha * r.val), 0);
                             else
-                                sm.rbig[pos] = make_uint2(((unsigned)r.idx >> LOG2S) << 16 | (unsigned)v, __float_as_uint(alpha * r.val));
+                                recs4[pos] = make_int4(uo, v * S, __float_as_int(alpha * r.val), 0);
                         }
                     }
                     gt_before += __popc(gtb);
@@ -265,56 +325,7 @@ __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord
             done = true;
         }
     }
-    if (!done) {
-        unsigned thr, need_eq;
-        sb.sync();
-        radix_select_tile<S, XS>(X, k_eff, sm.hist, misc, &thr, &need_eq, t, sb);
-        unsigned gt = 0, eq = 0;
-#pragma unroll 1
-        for (int v = 0; v < S; ++v) {
-            const unsigned key = mag_key(X[t * XS + v]);
-            gt += key > thr;
-            eq += key == thr;
-        }
-        const unsigned packed = gt | (eq << 16);
-        const unsigned inc = warp_inclusive_scan(packed, lane);
-        sb.sync();  // radix_select_tile's last reads of misc are done
-        if (lane == 31) misc[warp] = inc;
-        sb.sync();
-        unsigned before = inc - packed;
-        if (warp == 1) before += misc[0];
-        unsigned gb = before & 0xffffu, eb = before >> 16;
-#pragma unroll 1
-        for (int v = 0; v < S; ++v) {
-            const float val = X[t * XS + v];
-            const unsigned key = mag_key(val);
-            bool s = false;
-            unsigned pos = 0;
-            if (key > thr) {
-                pos = gb + min(eb, need_eq);
-                ++gb;
-                s = true;
-            } else if (key == thr) {
-                if (eb < need_eq) {
-                    pos = gb + eb;
-                    s = true;
-                }
-                ++eb;
-            }
-            if (s) {
-                DemoRecord r;
-                r.idx = t * S + v;
-                r.val = val;
-                rec[pos] = r;
-                if (qdom)
-                    X[t * XS + v] = fmaf(-alpha, val, val);
-                else if (k_eff <= 64)
-                    recs4[pos] = make_int4(t * XS, v * S, __float_as_int(alpha * val), 0);
-                else if (k_eff <= 256)
-                    sm.rbig[pos] = make_uint2((unsigned)t << 16 | (unsigned)v, __float_as_uint(alpha * val));
-            }
-        }
-    }
+    if (!done) select_radix(sm, k_eff, rec, alpha, t, bar_id, qdom ? SELECT_QDOM : SELECT_LISTED);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -445,11 +456,10 @@ __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], i
         recs4[t] = make_int4(pad_row, 0, 0, 0);  // list padding (ordered before the record writes by the barriers below)
         if (t == 0) recs4[64] = make_int4(pad_row, 0, 0, 0);
     }
-    bool slow = (k_eff > S);
-    bool bound_valid = false;
+    bool slow = false;
     bool zero_chunk = false;
     unsigned n_cw = 0, off = 0, mlo = 0u, mhi = 0u, lmin_w = 0u;
-    if (!slow) {
+    {
         // per-thread maximum magnitude (independent chains of 16, 3-input max)
         float tm = 0.f;
 #pragma unroll
@@ -480,7 +490,6 @@ __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], i
             prefix = (cnt >= (unsigned)k_eff) ? cand : prefix;
         }
         lmin_w = prefix;
-        bound_valid = true;
         if (!zero_chunk) {
             // candidates: |q| >= L  <=>  |q| > Lm (the float just below L); the sign bit of Lm - |q|
             // is funnel-shifted into a bit mask (independent chains of 16)
@@ -518,7 +527,7 @@ __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], i
     } else {
         // stash the coefficients of row t (own row: no hazard with other threads)
         stash_row(std::integral_constant<bool, CORE_STASH>{});
-        if (!slow) {
+        {
             const unsigned lbase = warp * CAPWP;
             if (n_cw <= CAPW) {
                 // each warp compacts its candidates into its own list (rows of warp 0 precede rows of
@@ -551,9 +560,205 @@ __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], i
         }
         if (slow) {
             if (CORE_STASH) stash_row(std::false_type{});  // the out-of-line selection reads the tile in index order
-            select_slow(sm, k_eff, rec, alpha, t, bar_id, lmin_w, bound_valid, QDOM);
+            select_slow(sm, k_eff, rec, alpha, t, bar_id, lmin_w, QDOM);
             sb.sync();  // every thread is done with the coefficient tile
             zero_row();
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Exact top-k for k > MAX_K_LISTED; same contract as select_chunk, except that with the momentum in the spatial domain
+// it leaves row t of X ready for the dense row stage: alpha * q at the kept places, zero elsewhere, position p of the
+// row holding coefficient core_index(p).  Ends before the barrier that makes records and tile visible.
+// The bound is the k-th largest of the 256 quarter-row maxima (16 coefficients each): for a dense tile about 55
+// candidates at k = 49, 175 at k = 128, 245 at k = 160.  Both warps take all candidates into registers and find the
+// kept set by the same ballot search as the list variant.
+// ------------------------------------------------------------------------------------------------
+constexpr int MAX_K_QUARTERS = 192;  // above it the bound admits too many candidates (k = 192: 340 of 512 places)
+
+template <bool QDOM>
+__device__ __forceinline__ void select_chunk_big(const SlotMem &sm, float (&q)[S], int k_eff, DemoRecord *rec, float alpha,
+                                                 int t, const SlotBarrier<S> &sb, int bar_id)
+{
+    float *X = sm.X;
+    unsigned *misc = sm.misc;
+    const int lane = t & 31, warp = t >> 5;
+    float *my_row = X + t * XS;
+    auto stash_row = [&]() {
+        float4 *row = reinterpret_cast<float4 *>(my_row);
+#pragma unroll
+        for (int v4 = 0; v4 < S / 4; ++v4) row[v4] = make_float4(q[4 * v4], q[4 * v4 + 1], q[4 * v4 + 2], q[4 * v4 + 3]);
+    };
+    auto zero_row = [&]() {
+        float4 *row = reinterpret_cast<float4 *>(my_row);
+#pragma unroll
+        for (int v4 = 0; v4 < S / 4; ++v4) row[v4] = make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    // position of coefficient v in core order: v = (2j + 1) << s sits at (32 >> s) + j, v = 0 at 0
+    auto core_pos = [](int v) {
+        const int sft = __ffs(v | S) - 1;
+        return ((S / 2) >> sft) + (v >> (sft + 1));
+    };
+    bool slow = k_eff > MAX_K_QUARTERS;
+    bool zero_chunk = false;
+    if (!slow) {
+        unsigned own[4], oth[4];
+        unsigned *gq = sm.wkey;  // [4][64]
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const int b0 = 16 * g;
+            float cm = max3abs(q[b0], q[b0 + 1], q[b0 + 2]);
+#pragma unroll
+            for (int j = 3; j + 1 < 16; j += 2) cm = max3f(cm, fabsf(q[b0 + j]), fabsf(q[b0 + j + 1]));
+            own[g] = __float_as_uint(fmaxf(cm, fabsf(q[b0 + 15])));
+            gq[g * 64 + t] = own[g];
+        }
+        sb.sync();  // (row t of the tile is this thread's: every thread has read its row of the transposed tile too)
+#pragma unroll
+        for (int g = 0; g < 4; ++g) oth[g] = gq[g * 64 + (t ^ 32)];
+        unsigned lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            lo = min(lo, min(own[g], oth[g]));
+            hi = max(hi, max(own[g], oth[g]));
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        zero_chunk = (hi == 0u);
+        const int c0 = 31 - __clz((lo ^ hi) | 0x8000u);
+        unsigned bound = lo & ~((2u << c0) - 1u);
+#pragma unroll 1
+        for (int b = zero_chunk ? 14 : c0; b >= 15; --b) {
+            const unsigned cand = bound | (1u << b);
+            unsigned cnt = 0;
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+                cnt += __popc(__ballot_sync(0xffffffffu, own[g] >= cand)) + __popc(__ballot_sync(0xffffffffu, oth[g] >= cand));
+            bound = (cnt >= (unsigned)k_eff) ? cand : bound;
+        }
+        if (zero_chunk) {
+            // all coefficients zero: the tie rule gives the records 0 .. k_eff-1 with value 0
+            for (int r = t; r < k_eff; r += S) {
+                DemoRecord z;
+                z.idx = r;
+                z.val = 0.f;
+                rec[r] = z;
+            }
+            zero_row();
+            return;
+        }
+        // candidates: |q| >= bound, i.e. |q| > the float just below it (see select_chunk)
+        const float Lm = bound ? __uint_as_float(bound - 1u) : -1.f;
+        unsigned mc[S / 16];
+#pragma unroll
+        for (int ch = 0; ch < S / 16; ++ch) {
+            unsigned mm = 0u;
+#pragma unroll
+            for (int j = 15; j >= 0; --j) mm = __funnelshift_l(__float_as_uint(Lm - fabsf(q[16 * ch + j])), mm, 1);
+            mc[ch] = mm;
+        }
+        unsigned long long mask = ((unsigned long long)(mc[2] | (mc[3] << 16)) << 32) | (mc[0] | (mc[1] << 16));
+        const unsigned cnt = (unsigned)__popcll(mask);
+        const unsigned inc = warp_inclusive_scan(cnt, lane);
+        if (lane == 31) misc[warp] = inc;
+        stash_row();
+        sb.sync();  // counts visible; the maxima in the list area are read
+        const unsigned n_w0 = misc[0], n_all = n_w0 + misc[1];
+        slow = n_all > (unsigned)WCAP || n_all < (unsigned)k_eff;  // (fewer than k: NaN coefficients)
+        if (!slow) {
+            unsigned *wval = sm.wkey, *widx = sm.widx;
+            unsigned o = inc - cnt + (warp ? n_w0 : 0u);
+            while (mask) {
+                const int v = __ffsll((long long)mask) - 1;
+                mask &= mask - 1ull;
+                widx[o] = t * S + v;
+                wval[o] = __float_as_uint(my_row[v]);
+                ++o;
+            }
+            if (!QDOM) zero_row();
+            sb.sync();  // the list is complete, the tile cleared
+            auto pick = [&](auto wk_tag) {
+                constexpr int WK = decltype(wk_tag)::value;
+                unsigned keys[WK];
+                unsigned top = 0u;
+#pragma unroll
+                for (int j = 0; j < WK; ++j) {
+                    const unsigned i = (unsigned)j * 32u + lane;
+                    keys[j] = (i < n_all) ? (wval[i] & 0x7fffffffu) : 0u;
+                    top = max(top, keys[j]);
+                }
+                top = __reduce_max_sync(0xffffffffu, top);
+                const int wb0 = 31 - __clz((bound ^ top) | 1u);
+                unsigned thr = bound & ~((2u << wb0) - 1u);
+                unsigned n_ge = n_all;  // every entry is >= the bound >= thr; the search stops at exactly k_eff
+#pragma unroll 1
+                for (int b = wb0; b >= 0 && n_ge != (unsigned)k_eff; --b) {
+                    const unsigned cand = thr | (1u << b);
+                    unsigned n = 0;
+#pragma unroll
+                    for (int j = 0; j < WK; ++j) n += __popc(__ballot_sync(0xffffffffu, keys[j] >= cand));
+                    if (n >= (unsigned)k_eff) {
+                        thr = cand;
+                        n_ge = n;
+                    }
+                }
+                unsigned n_gt = 0;
+#pragma unroll
+                for (int j = 0; j < WK; ++j) n_gt += __popc(__ballot_sync(0xffffffffu, keys[j] > thr));
+                const unsigned need_eq = (unsigned)k_eff - n_gt;
+                const unsigned lt = (1u << lane) - 1u;
+                unsigned gt_before = 0, eq_before = 0;
+#pragma unroll
+                for (int j = 0; j < WK; ++j) {
+                    const unsigned gtb = __ballot_sync(0xffffffffu, keys[j] > thr);
+                    const unsigned eqb = __ballot_sync(0xffffffffu, keys[j] == thr);
+                    if ((j & 1) == warp) {
+                        const unsigned e = eq_before + __popc(eqb & lt);
+                        if ((keys[j] > thr) || (keys[j] == thr && e < need_eq)) {
+                            const unsigned pos = gt_before + __popc(gtb & lt) + min(e, need_eq);
+                            DemoRecord r;
+                            r.idx = (int)widx[j * 32 + lane];
+                            r.val = __uint_as_float(wval[j * 32 + lane]);
+                            rec[pos] = r;
+                            float *row = X + (r.idx >> LOG2S) * XS;
+                            const int v = r.idx & (S - 1);
+                            if (QDOM)
+                                row[v] = fmaf(-alpha, r.val, r.val);
+                            else
+                                row[core_pos(v)] = alpha * r.val;
+                        }
+                    }
+                    gt_before += __popc(gtb);
+                    eq_before += __popc(eqb);
+                }
+            };
+            if (n_all <= 256u)
+                pick(std::integral_constant<int, 8>{});
+            else
+                pick(std::integral_constant<int, WCAP / 32>{});
+        }
+    } else {
+        sb.sync();  // every thread has read its row of the transposed tile
+        stash_row();
+    }
+    if (slow) {
+        select_radix(sm, k_eff, rec, alpha, t, bar_id, QDOM ? SELECT_QDOM : SELECT_DENSE);
+        if (!QDOM) {  // index order -> core order (this thread's row)
+            float4 *row = reinterpret_cast<float4 *>(my_row);
+#pragma unroll
+            for (int v4 = 0; v4 < S / 4; ++v4) {
+                const float4 f = row[v4];
+                q[4 * v4] = f.x;
+                q[4 * v4 + 1] = f.y;
+                q[4 * v4 + 2] = f.z;
+                q[4 * v4 + 3] = f.w;
+            }
+            fdct::static_for<0, S / 4>([&](auto i) {
+                constexpr int v4 = decltype(i)::value;
+                row[v4] = make_float4(q[fdct::core_index<S>(4 * v4)], q[fdct::core_index<S>(4 * v4 + 1)],
+                                      q[fdct::core_index<S>(4 * v4 + 2)], q[fdct::core_index<S>(4 * v4 + 3)]);
+            });
         }
     }
 }
@@ -562,7 +767,9 @@ __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], i
 // demo_set_momentum_domain): they hold its chunk-wise DCT, tile by tile and transposed (element (r, c) of a tile
 // is coefficient (c, r)): the step is then Q = beta*Qm + DCT(g), top-k, Qm <- Q - alpha*Q_kept -- one forward
 // transform of the gradient, no inverse transform, no row stage.
-template <typename GT, int THREADS, bool QDOM>
+// BIGK (k > MAX_K_LISTED): the selection is select_chunk_big and the row stage of the inverse is dense -- a fourth trip
+// through the transform core along row t, k of whose coefficients are not zero -- instead of k rank-1 updates.
+template <typename GT, int THREADS, bool QDOM, bool BIGK>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(DemoCompressArgs a)
 {
     constexpr int NCH = THREADS / S;
@@ -580,7 +787,6 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
     sm.X = Ms;
     sm.wkey = reinterpret_cast<unsigned *>(sm.raw + TILE_X_BYTES);
     sm.widx = sm.wkey + WCAP + 4;
-    sm.rbig = reinterpret_cast<uint2 *>(sm.widx + WCAP + 4);
     sm.tmax = reinterpret_cast<float *>(sm.raw + region_bytes<GT>());
     sm.cand_idx = reinterpret_cast<int *>(sm.tmax + S);
     sm.cand_val = reinterpret_cast<float *>(sm.cand_idx + CAP + 8);
@@ -678,9 +884,11 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
 
         // Three passes through one copy of the transform core: 0 = DCT-II down column t of B = beta*m + g,
         // 1 = DCT-II along row t (followed by the selection and the sparse row stage of the inverse),
-        // 2 = DCT-III down column t of the row-stage tile (followed by the residual).
+        // 2 = DCT-III down column t of the row-stage tile (followed by the residual).  BIGK: 2 = DCT-III along row t of
+        // the kept coefficients, 3 = DCT-III down column t.
+        constexpr int PASSES = QDOM ? 2 : (BIGK ? 4 : 3);
 #pragma unroll 1
-        for (int ph = 0; ph < (QDOM ? 2 : 3); ++ph) {
+        for (int ph = 0; ph < PASSES; ++ph) {
             float w[S], y[S];
             if (ph < 2) {
                 float x[S];
@@ -722,11 +930,23 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
                     }
                 }
                 fdct::dct2_pre_paired<S>(x, w);
+            } else if (BIGK && ph == 2) {
+                const float4 *row = reinterpret_cast<const float4 *>(X + t * XS);
+#pragma unroll
+                for (int v4 = 0; v4 < S / 4; ++v4) {  // (the selection left the kept coefficients in core order)
+                    const float4 f = row[v4];
+                    w[4 * v4 + 0] = f.x;
+                    w[4 * v4 + 1] = f.y;
+                    w[4 * v4 + 2] = f.z;
+                    w[4 * v4 + 3] = f.w;
+                }
             } else {
-                // column t of the row-stage tile was written by this thread only: no barrier before reading it
+                // column t of the row-stage tile: written by this thread only (no barrier before reading it), or, in pair
+                // order within each row, by the dense row stage
+                const float *Xt = X + (BIGK ? fdct::pair_order(t) : t);
                 fdct::static_for<0, S>([&](auto i) {
                     constexpr int p = decltype(i)::value;
-                    w[p] = X[fdct::core_index<S>(p) * XS + t];
+                    w[p] = Xt[fdct::core_index<S>(p) * XS];
                 });
             }
 
@@ -741,7 +961,16 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
                     Xc[fdct::core_index<S>(p) * XS] = y[p];
                 });
                 sb.sync();
-            } else if (ph == 2) {
+            } else if (BIGK && !QDOM && ph == 2) {
+                fdct::F2 rp[S / 2];  // the row of the row-stage tile in pair order
+                fdct::dct3_post_pairs<S>(y, rp);
+                float4 *row = reinterpret_cast<float4 *>(X + t * XS);
+#pragma unroll
+                for (int v4 = 0; v4 < S / 4; ++v4)
+                    row[v4] = make_float4(fdct::f2_lo(rp[2 * v4]), fdct::f2_hi(rp[2 * v4]), fdct::f2_lo(rp[2 * v4 + 1]),
+                                          fdct::f2_hi(rp[2 * v4 + 1]));
+                sb.sync();
+            } else if (ph == PASSES - 1 && !QDOM) {
                 // m <- B - alpha * IDCT(kept): column t of the new momentum goes into a dense tile (the m staging
                 // area; the row-stage tile it overlaps is dead for every thread only after the barrier below, so the
                 // column is formed in registers first), which one TMA store writes out; the next chunk's tiles are
@@ -790,7 +1019,10 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
 #pragma unroll
                         for (int j = 0; j < 32; ++j) q[32 * h + j] = fmaf(a.beta, mq[j], q[32 * h + j]);
                     }
-                    select_chunk<true>(sm, q, k_eff, rec, a.alpha, t, sb, slot + 1, PAD_ROW);
+                    if constexpr (BIGK)
+                        select_chunk_big<true>(sm, q, k_eff, rec, a.alpha, t, sb, slot + 1);
+                    else
+                        select_chunk<true>(sm, q, k_eff, rec, a.alpha, t, sb, slot + 1, PAD_ROW);
                     sb.sync();  // the tile holds Q - alpha * Q_kept (kept entries were patched by the record writers)
                     float4 rowv[S / 4];
                     {
@@ -816,81 +1048,41 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
                     }
                     continue;
                 }
+                if constexpr (BIGK) {
+                    select_chunk_big<false>(sm, q, k_eff, rec, a.alpha, t, sb, slot + 1);
+                    sb.sync();  // records complete, kept coefficients in the tile
+                    continue;
+                }
                 select_chunk<false>(sm, q, k_eff, rec, a.alpha, t, sb, slot + 1, PAD_ROW);
                 sb.sync();  // records complete (shared list and global payload), tile zeroed
 
                 // ---- residual: row stage of the inverse from the k_eff records, sparse --------------
                 {
                     // T[u][t] = sum over kept (u, v) of alpha * val * C[v][t]; the basis is read through L1
-                    const float *Ct = a.C + t;
                     float acc = 0.f;
-                    if (k_eff <= 64) {
-                        // The running sum of a row is stored after every entry (the last store of a row carries the
-                        // whole sum) and starts again from zero when the next entry belongs to another row: no branch in
-                        // the loop.  The list is padded with zero-valued entries (entry 64 is always one) whose "row" is
-                        // a scratch line outside the tile.  Entries and their cosines are fetched ahead of the
-                        // dependent accumulation.
-                        float *Xt = X + t;
-                        int4 nx = recs4[0];
+                    // The running sum of a row is stored after every entry (the last store of a row carries the
+                    // whole sum) and starts again from zero when the next entry belongs to another row: no branch in
+                    // the loop.  The list is padded with zero-valued entries (entry 64 is always one) whose "row" is
+                    // a scratch line outside the tile.  Entries and their cosines are fetched ahead of the
+                    // dependent accumulation.
+                    float *Xt = X + t;
+                    int4 nx = recs4[0];
 #pragma unroll 1
-                        for (int r0 = 0; r0 < k_eff; r0 += ROW_AHEAD) {
-                            int4 rc[ROW_AHEAD + 1];
-                            float cv[ROW_AHEAD];
-                            rc[0] = nx;
+                    for (int r0 = 0; r0 < k_eff; r0 += ROW_AHEAD) {
+                        int4 rc[ROW_AHEAD + 1];
+                        float cv[ROW_AHEAD];
+                        rc[0] = nx;
 #pragma unroll
-                            for (int j = 1; j < ROW_AHEAD + 1; ++j) rc[j] = recs4[r0 + j];
-                            nx = rc[ROW_AHEAD];
+                        for (int j = 1; j < ROW_AHEAD + 1; ++j) rc[j] = recs4[r0 + j];
+                        nx = rc[ROW_AHEAD];
 #pragma unroll
-                            for (int j = 0; j < ROW_AHEAD; ++j) cv[j] = __ldg(a.C + (unsigned)(rc[j].y + t));
+                        for (int j = 0; j < ROW_AHEAD; ++j) cv[j] = __ldg(a.C + (unsigned)(rc[j].y + t));
 #pragma unroll
-                            for (int j = 0; j < ROW_AHEAD; ++j) {
-                                acc = fmaf(__int_as_float(rc[j].z), cv[j], acc);
-                                Xt[rc[j].x] = acc;
-                                acc = (rc[j].x != rc[j + 1].x) ? 0.f : acc;
-                            }
+                        for (int j = 0; j < ROW_AHEAD; ++j) {
+                            acc = fmaf(__int_as_float(rc[j].z), cv[j], acc);
+                            Xt[rc[j].x] = acc;
+                            acc = (rc[j].x != rc[j + 1].x) ? 0.f : acc;
                         }
-                    } else {
-                        // k > 64: up to 256 kept records come from a compact shared list, more from the payload
-                        // itself; four cosines are fetched ahead
-                        const bool listed = k_eff <= 256;
-                        int cur_u = -1;
-#pragma unroll 1
-                        for (int r0 = 0; r0 < k_eff; r0 += 4) {
-                            int u[4];
-                            float z[4], cv[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                u[j] = -1;
-                                z[j] = 0.f;
-                                int v = 0;
-                                if (r0 + j < k_eff) {
-                                    if (listed) {
-                                        const uint2 e = sm.rbig[r0 + j];
-                                        u[j] = (int)(e.x >> 16) * XS;
-                                        v = (int)(e.x & 0xffffu);
-                                        z[j] = __uint_as_float(e.y);
-                                    } else {
-                                        const DemoRecord rc = rec[r0 + j];
-                                        u[j] = (rc.idx >> LOG2S) * XS;
-                                        v = rc.idx & (S - 1);
-                                        z[j] = a.alpha * rc.val;
-                                    }
-                                }
-                                cv[j] = __ldg(Ct + v * S);
-                            }
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                if (u[j] >= 0) {
-                                    if (u[j] != cur_u) {
-                                        if (cur_u >= 0) X[cur_u + t] = acc;
-                                        acc = 0.f;
-                                        cur_u = u[j];
-                                    }
-                                    acc = fmaf(z[j], cv[j], acc);
-                                }
-                            }
-                        }
-                        if (cur_u >= 0) X[cur_u + t] = acc;
                     }
                 }
             }
@@ -904,11 +1096,11 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
 }
 
-template <typename GT, int THREADS, bool QDOM>
+template <typename GT, int THREADS, bool QDOM, bool BIGK>
 cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
 {
     constexpr int NCH = THREADS / S;
-    auto kernel = compress64_kernel<GT, THREADS, QDOM>;
+    auto kernel = compress64_kernel<GT, THREADS, QDOM, BIGK>;
     const size_t smem = slot_bytes<GT>() * NCH + 16;
     if (a.n_chunks <= 0) return cudaSuccess;
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -935,12 +1127,12 @@ cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t strea
 cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
 {
     if (a.tmap_m == nullptr || a.tmap_g == nullptr) return cudaErrorNotSupported;
-#ifndef DEMO_T64
-#define DEMO_T64 64
-#endif
+    auto pick = [&](auto gt, auto qdom) {
+        using GT = decltype(gt);
+        constexpr bool Q = decltype(qdom)::value;
+        return a.k > MAX_K_LISTED ? launch64<GT, 64, Q, true>(a, sm_count, stream) : launch64<GT, 64, Q, false>(a, sm_count, stream);
+    };
     if (a.momentum_dct)
-        return a.grad_bf16 ? launch64<__nv_bfloat16, DEMO_T64, true>(a, sm_count, stream)
-                           : launch64<float, DEMO_T64, true>(a, sm_count, stream);
-    return a.grad_bf16 ? launch64<__nv_bfloat16, DEMO_T64, false>(a, sm_count, stream)
-                       : launch64<float, DEMO_T64, false>(a, sm_count, stream);
+        return a.grad_bf16 ? pick(__nv_bfloat16{}, std::true_type{}) : pick(float{}, std::true_type{});
+    return a.grad_bf16 ? pick(__nv_bfloat16{}, std::false_type{}) : pick(float{}, std::false_type{});
 }
