@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 // One payload record: flat index inside the chunk + fp32 coefficient (8 bytes, little-endian).
 struct DemoRecord {
     int32_t idx;
@@ -97,10 +99,11 @@ cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *flag
 
 // ---- tensors of any order with rectangular chunks (appendix of the paper: blocking operator and
 // multilinear product; kernels_nd.cu) ---------------------------------------------------------------
-constexpr int DEMO_ND_DIMS = 4;  // lower orders are padded on the left with axes of extent 1
+constexpr int DEMO_ND_DIMS = 4;         // lower orders are padded on the left with axes of extent 1
+constexpr int DEMO_ND_MAX_ROWS = 1024;  // contiguous rows of a chunk whose offsets the kernels tabulate
 
 struct DemoNdEntry {
-    long long chunk_begin;           // id of this tensor's first chunk inside the work list
+    long long chunk_begin;           // id of this tensor's first chunk inside its class
     long long chunk_end;             // chunk_begin + number of chunks of this tensor
     long long rec_begin;             // index of this tensor's first record inside a payload
     long long stride[DEMO_ND_DIMS];  // element stride of each axis of the (contiguous) tensor
@@ -110,33 +113,59 @@ struct DemoNdEntry {
     int s[DEMO_ND_DIMS];             // chunk shape
     int c[DEMO_ND_DIMS];             // chunk grid
     unsigned inv[DEMO_ND_DIMS];      // ceil(2^32 / s[a]) for s[a] > 1 (division by multiplication), else 0
-    int basis[DEMO_ND_DIMS];         // offset (floats, multiple of 4) of axis a's [C | C^T] inside the table
+    int basis[DEMO_ND_DIMS];         // offset (floats, multiple of 8) of axis a's table, where it is a dense contraction
+    // filled in by demo_nd_plan and demo_nd_classify (kernels_nd.cu)
+    int p[DEMO_ND_DIMS];             // element strides of the padded tile in shared memory
+    int tile;                        // its floats, a multiple of 4
+    int tail;                        // > 0: the last two axes are both of this extent and transformed together
+    int row;                         // elements that are contiguous both in the tensor and in the tile
+    unsigned inv_row;                // ceil(2^32 / row) for row > 1, else 0
+    int row_table;                   // 1: the chunk's rows are few and their offsets fit 32 bits
+    int threads;                     // CTA size this chunk would choose
+    int layout;                      // same number: same strides in the tensor and in the tile
 };
 
+// Tensors that share a kernel variant: one launch.
+struct DemoNdClass {
+    int first, n;        // entries first .. first + n - 1 of the context's list
+    long long n_chunks;  // chunk ids run over the class
+    int threads;         // CTA size
+    int max_M, tile;     // largest chunk / padded tile (floats, multiples of 4)
+    int rows;            // longest row table
+    int dense_axes;      // some extent is a dense contraction from a table (second tile)
+    int big;             // some extent is 128: the variant with 64 registers per half line
+};
+// Coefficient tables of the dense extents in use.
+struct DemoNdTables {
+    std::vector<float> data;
+    int of[129];
+    DemoNdTables() { for (int &v : of) v = -1; }
+    int get(int s);  // offset of the tables of extent s (made on first use)
+};
+void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables);
+// Sorts `entries` by class, sets their chunk ranges (chunk_end holds the number of chunks before) and lists the classes.
+void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vector<DemoNdClass> *classes);
+
 struct DemoNdCompressArgs {
-    const DemoNdEntry *entries;  // device
-    int n_entries;
-    long long n_chunks;
+    const DemoNdEntry *entries;  // device, the class's first
+    DemoNdClass cls;
     const void *const *g_ptrs;
     float *const *m_ptrs;
     DemoRecord *payload;
-    const float *tables;  // device: per chunk extent s in use, C (s x s, C[u*s + n]) followed by C^T
+    const float *tables;  // device: DemoNdTables::data
     float beta, alpha;
     int grad_bf16;
-    int max_M;  // largest chunk of the list (sizes the shared-memory buffers)
     int *status;
 };
 
 struct DemoNdDecodeArgs {
-    const DemoNdEntry *entries;
-    int n_entries;
-    long long n_chunks;
+    const DemoNdEntry *entries;  // device, the class's first
+    DemoNdClass cls;
     const DemoRecord *const *payloads;
     int W;
     float *const *x_ptrs;
     const float *tables;
     float lr, wd;
-    int max_M;
     int *status;
     int agg, phi;
     float agg_scale;

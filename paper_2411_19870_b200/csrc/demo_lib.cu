@@ -36,8 +36,7 @@ struct demo_ctx {
     // contexts made by demo_init_nd: one work list of rectangular chunks of any order, the DCT matrices
     // of every chunk extent in one table; the square-chunk lists above stay empty
     bool nd = false;
-    int n_nd = 0, max_M = 0;
-    long long chunks_nd = 0;
+    std::vector<DemoNdClass> nd_classes;  // one kernel launch each; entries of a class are neighbours
     DemoNdEntry *d_entries_nd = nullptr;
     float *d_tables = nullptr;
 
@@ -444,13 +443,10 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
         return DEMO_ERR_CUDA;
     }
 
-    // planner: the work list (axes padded on the left to DEMO_ND_DIMS), payload offsets, and one
-    // orthonormal DCT-II matrix per distinct chunk extent
+    // planner: the work list (axes padded on the left to DEMO_ND_DIMS), payload offsets, tile layouts and tables
     std::vector<DemoNdEntry> entries;
-    std::vector<float> tables;
+    DemoNdTables tables;
     try {
-        int table_of[DEMO_ND_MAX_EXTENT + 1];
-        for (int &v : table_of) v = -1;
         c->first_record.resize(n_tensors);
         c->n_chunks.resize(n_tensors);
         c->n_elems.resize(n_tensors);
@@ -458,7 +454,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
         long long rec = 0;
         for (int t = 0; t < n_tensors; ++t) {
             const demo_nd_tensor_desc &d = tensors[t];
-            DemoNdEntry e;
+            DemoNdEntry e{};
             const int pad = DEMO_ND_DIMS - d.ndim;
             long long stride = 1, M = 1, n_ch = 1;
             for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
@@ -471,35 +467,14 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
                 stride *= n;
                 M *= s;
                 n_ch *= n / s;
-                e.basis[a] = 0;
                 e.inv[a] = s > 1 ? (unsigned)(((1ULL << 32) + (unsigned)s - 1) / (unsigned)s) : 0u;
-                if (s > 1) {
-                    if (table_of[s] < 0) {
-                        // C then C^T, each s x s; every table starts on a 16-byte boundary
-                        table_of[s] = (int)tables.size();
-                        const double pi = 3.141592653589793238462643383279502884;
-                        std::vector<float> C((size_t)s * s);
-                        for (int u = 0; u < s; ++u)
-                            for (int n2 = 0; n2 < s; ++n2) {
-                                const double au = (u == 0) ? std::sqrt(1.0 / s) : std::sqrt(2.0 / s);
-                                C[(size_t)u * s + n2] = (float)(au * std::cos(pi * (2.0 * n2 + 1.0) * u / (2.0 * s)));
-                            }
-                        tables.insert(tables.end(), C.begin(), C.end());
-                        for (int n2 = 0; n2 < s; ++n2)
-                            for (int u = 0; u < s; ++u) tables.push_back(C[(size_t)u * s + n2]);
-                        while (tables.size() % 4) tables.push_back(0.f);
-                    }
-                    e.basis[a] = table_of[s];
-                }
             }
             e.tensor = t;
             e.M = (int)M;
             e.k_eff = (int)(cfg->topk < M ? cfg->topk : M);
             e.rec_begin = rec;
-            e.chunk_begin = c->chunks_nd;
-            c->chunks_nd += n_ch;
-            e.chunk_end = c->chunks_nd;
-            if (((e.M + 3) & ~3) > c->max_M) c->max_M = (e.M + 3) & ~3;  // buffers stay 16-byte aligned
+            e.chunk_end = n_ch;  // (the classes below set the ranges)
+            demo_nd_plan(&e, &tables);
             entries.push_back(e);
             c->first_record[t] = rec;
             c->n_chunks[t] = n_ch;
@@ -508,7 +483,8 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
             rec += n_ch * e.k_eff;
         }
         c->total_records = rec;
-        if (tables.empty()) tables.push_back(1.0f);  // every extent is 1: no matrix is ever read
+        demo_nd_classify(entries, c->sm_count, &c->nd_classes);
+        if (tables.data.empty()) tables.data.push_back(1.0f);  // no dense extent: never read
         const size_t W = (size_t)cfg->num_workers, T = (size_t)n_tensors;
         c->h_g.assign(W * T, nullptr);
         c->h_m.assign(W * T, nullptr);
@@ -520,11 +496,9 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
         release(c);
         return DEMO_ERR_ALLOC;
     }
-    c->n_nd = n_tensors;
-
     const size_t W = (size_t)cfg->num_workers, T = (size_t)n_tensors;
     bool ok = true;
-    ok = ok && cudaMalloc(&c->d_tables, tables.size() * sizeof(float)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_tables, tables.data.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_entries_nd, entries.size() * sizeof(DemoNdEntry)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_status, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_g, W * T * sizeof(void *)) == cudaSuccess;
@@ -536,7 +510,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
         release(c);
         return DEMO_ERR_ALLOC;
     }
-    ok = ok && cudaMemcpy(c->d_tables, tables.data(), tables.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+    ok = ok && cudaMemcpy(c->d_tables, tables.data.data(), tables.data.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemcpy(c->d_entries_nd, entries.data(), entries.size() * sizeof(DemoNdEntry),
                           cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess;
@@ -636,9 +610,6 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
 
     if (ctx->nd) {
         DemoNdCompressArgs n;
-        n.entries = ctx->d_entries_nd;
-        n.n_entries = ctx->n_nd;
-        n.n_chunks = ctx->chunks_nd;
         n.g_ptrs = ctx->d_g + row;
         n.m_ptrs = ctx->d_m + row;
         n.payload = static_cast<DemoRecord *>(payload_out);
@@ -646,13 +617,16 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
         n.beta = ctx->cfg.beta;
         n.alpha = ctx->alpha;
         n.grad_bf16 = ctx->cfg.grad_dtype == DEMO_BF16;
-        n.max_M = ctx->max_M;
         n.status = ctx->d_status;
-        if (demo_launch_compress_nd(n, ctx->sm_count, stream) != cudaSuccess) {
-            cudaGetLastError();
-            return DEMO_ERR_CUDA;
+        for (const DemoNdClass &k : ctx->nd_classes) {
+            n.entries = ctx->d_entries_nd + k.first;
+            n.cls = k;
+            if (demo_launch_compress_nd(n, ctx->sm_count, stream) != cudaSuccess) {
+                cudaGetLastError();
+                return DEMO_ERR_CUDA;
+            }
+            ctx->launches += 1;
         }
-        ctx->launches += 1;
         return DEMO_OK;
     }
 
@@ -790,26 +764,26 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
 
     if (ctx->nd) {
         DemoNdDecodeArgs n;
-        n.entries = ctx->d_entries_nd;
-        n.n_entries = ctx->n_nd;
-        n.n_chunks = ctx->chunks_nd;
         n.payloads = ctx->d_p;
         n.W = W;
         n.x_ptrs = ctx->d_x;
         n.tables = ctx->d_tables;
         n.lr = ctx->cfg.lr;
         n.wd = ctx->cfg.weight_decay;
-        n.max_M = ctx->max_M;
         n.status = ctx->d_status;
         n.agg = ctx->aggregation;
         n.phi = ctx->phi;
         n.agg_scale = (ctx->aggregation == DEMO_AGG_MEAN) ? 1.0f / (float)W : 1.0f;
         n.sign_ptrs = signs ? ctx->d_s : nullptr;
-        if (demo_launch_decode_nd(n, ctx->sm_count, stream) != cudaSuccess) {
-            cudaGetLastError();
-            return DEMO_ERR_CUDA;
+        for (const DemoNdClass &k : ctx->nd_classes) {
+            n.entries = ctx->d_entries_nd + k.first;
+            n.cls = k;
+            if (demo_launch_decode_nd(n, ctx->sm_count, stream) != cudaSuccess) {
+                cudaGetLastError();
+                return DEMO_ERR_CUDA;
+            }
+            ctx->launches += 1;
         }
-        ctx->launches += 1;
         return DEMO_OK;
     }
 

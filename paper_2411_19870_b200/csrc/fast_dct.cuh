@@ -584,4 +584,119 @@ FDCT_HD void dct3_post_pairs(const float (&y)[N], F2 (&xp)[N / 2])
 // Position of element v in the "pair order" (neighbours of odd pairs swapped); its own inverse.
 constexpr int pair_order(int v) { return v ^ ((v >> 1) & 1); }
 
+// ------------------------------------------------------------------------------------------------
+// DCT-II / DCT-III with the butterflies of the factorisation above, but the DCT-IV blocks of up to 16 points as plain
+// products with immediate constants (larger ones take one rotation stage and go on with DCT-II): about 12 operations per
+// element at 32 points instead of 9, and the rounding of a dense product where the input is sparse.  Root mean square error
+// on unit-variance data, 32 points: forward 7.5e-8 (fully factorised 7.6e-8, dense product 1.05e-7), inverse of two
+// non-zero coefficients 1.0e-8 (1.4e-8, 0.9e-8).  For kernels whose result is compared with dense transforms.
+// ------------------------------------------------------------------------------------------------
+constexpr int DENSE4_MAX = 16;
+
+template <int N, class SC>
+FDCT_HD void dct4_dense(const float (&v)[N], float (&V)[N]);
+
+template <int N, class SC>
+FDCT_HD void dct2_dense4(const float (&x)[N], float (&X)[N])
+{
+    if constexpr (N == 1) {
+        X[0] = x[0] * (float)SC::value;
+    } else {
+        constexpr int H = N / 2;
+        float u[H], v[H], E[H], O[H];
+        static_for<0, H>([&](auto i) {
+            constexpr int n = decltype(i)::value;
+            u[n] = x[n] + x[N - 1 - n];
+            v[n] = x[n] - x[N - 1 - n];
+        });
+        dct2_dense4<H, SC>(u, E);
+        dct4_dense<H, SC>(v, O);
+        static_for<0, H>([&](auto i) {
+            constexpr int j = decltype(i)::value;
+            X[2 * j] = E[j];
+            X[2 * j + 1] = O[j];
+        });
+    }
+}
+template <int N, class SC>
+FDCT_HD void dct4_dense(const float (&v)[N], float (&V)[N])
+{
+    if constexpr (N <= DENSE4_MAX) {
+        static_for<0, N>([&](auto i) {
+            constexpr int u = decltype(i)::value;
+            float acc = 0.f;
+            static_for<0, N>([&](auto j) {
+                constexpr int n = decltype(j)::value;
+                // cos(m pi / 4N) with the angle reduced to [0, pi/2] in whole numbers
+                constexpr int m0 = ((2 * n + 1) * (2 * u + 1)) % (8 * N), m1 = m0 > 4 * N ? 8 * N - m0 : m0;
+                constexpr double c = m1 > 2 * N ? -c_cos(kPi * (4 * N - m1) / (4.0 * N)) : c_cos(kPi * m1 / (4.0 * N));
+                acc = n == 0 ? (float)(SC::value * c) * v[0] : fmaf((float)(SC::value * c), v[n], acc);
+            });
+            V[u] = acc;
+        });
+    } else {
+        constexpr int H = N / 2;
+        float a[H], b[H], A[H], Bt[H];
+        static_for<0, H>([&](auto i) {
+            constexpr int n = decltype(i)::value;
+            constexpr double th = (2.0 * n + 1.0) * kPi / (4.0 * N);
+            constexpr double sg = (n % 2 == 0) ? 1.0 : -1.0;
+            constexpr float c = (float)(SC::value * c_cos(th));
+            constexpr float s = (float)(SC::value * c_sin(th));
+            constexpr float cb = (float)(SC::value * sg * c_cos(th));
+            constexpr float sb = (float)(SC::value * sg * c_sin(th));
+            a[n] = fmaf(v[N - 1 - n], s, v[n] * c);
+            b[n] = fmaf(v[N - 1 - n], cb, -(v[n] * sb));
+        });
+        dct2_dense4<H, ScaleOne>(a, A);
+        dct2_dense4<H, ScaleOne>(b, Bt);
+        V[0] = A[0];
+        V[N - 1] = -Bt[0];
+        static_for<1, H>([&](auto i) {
+            constexpr int p = decltype(i)::value;
+            V[2 * p - 1] = A[p] - Bt[H - p];
+            V[2 * p] = A[p] + Bt[H - p];
+        });
+    }
+}
+template <int N, class SC>
+FDCT_HD void dct3_dense4(const float (&X)[N], float (&x)[N])
+{
+    if constexpr (N == 1) {
+        x[0] = X[0] * (float)SC::value;
+    } else {
+        constexpr int H = N / 2;
+        float Xe[H], Xo[H], e[H], o[H];
+        static_for<0, H>([&](auto i) {
+            constexpr int j = decltype(i)::value;
+            Xe[j] = X[2 * j];
+            Xo[j] = X[2 * j + 1];
+        });
+        dct3_dense4<H, SC>(Xe, e);
+        dct4_dense<H, SC>(Xo, o);
+        static_for<0, H>([&](auto i) {
+            constexpr int n = decltype(i)::value;
+            x[n] = e[n] + o[n];
+            x[N - 1 - n] = e[n] - o[n];
+        });
+    }
+}
+// Orthonormal forms, in place.
+template <int N>
+FDCT_HD void dct2_ortho_dense4(float (&x)[N])
+{
+    float X[N];
+    dct2_dense4<N, ScaleOrtho<N>>(x, X);
+    X[0] *= (float)c_sqrt(0.5);
+    static_for<0, N>([&](auto i) { x[decltype(i)::value] = X[decltype(i)::value]; });
+}
+template <int N>
+FDCT_HD void dct3_ortho_dense4(float (&X)[N])
+{
+    float x[N];
+    X[0] *= (float)c_sqrt(0.5);
+    dct3_dense4<N, ScaleOrtho<N>>(X, x);
+    static_for<0, N>([&](auto i) { X[decltype(i)::value] = x[decltype(i)::value]; });
+}
+
 }  // namespace fdct

@@ -2,16 +2,41 @@
 // s_0 x ... x s_{d-1}: the general statement of the method in the paper's appendix ("Multilinear
 // Transforms and Chunk-wise Tensor Blocking").  The chunk transform is the multilinear product
 // T(B; C_0, ..., C_{d-1}) with the DCT matrix of dimension s_a on axis a, applied one axis after the
-// other as dense contractions on the CUDA cores; chunk extents are run-time values.  One CTA works on
-// one chunk at a time and keeps it in shared memory from the momentum update to the residual
-// write-back, so HBM is touched once per operand, as in the kernels for square chunks.  Selection,
-// record layout and update are those of kernels_generic.cu.
+// other; chunk extents are run-time values.  One CTA works on one chunk at a time and keeps it in shared
+// memory from the momentum update to the residual write-back, so HBM is touched once per operand.
+//
+// What bounds these kernels is instruction issue and latency, with barriers between the phases, so the work per element
+// and the number of phases are what the design cuts:
+//   * an axis is transformed line by line, in place, in registers: extents up to 8 and 16 / 32 one line per thread, 64 / 128
+//     two threads per line (fast_dct.cuh, dct2_dense4); two equal small last axes (a convolution's kernel window)
+//     together; only the other extents are dense contractions from a table, even and odd outputs apart (half the
+//     products), into a second tile;
+//   * the tile's strides are padded on the host so that neighbouring lines do not share banks, and a line's elements are a
+//     constant stride apart; the padding is always zero, so that sweeps over the tile run over plain memory, 16 bytes at a
+//     time;
+//   * global offsets come from a table of the chunk's contiguous rows, not from four divisions per element, and the loads
+//     of eight elements per thread are issued together;
+//   * top-k: the k-th largest of the threads' maxima (from a histogram relative to the largest) bounds the k-th coefficient;
+//     the few dozen to few hundred coefficients above it are listed, one warp finds the k-th among them, and the kept ones
+//     are put in index order by counting; radix select only when the list overflows (chunks with many equal magnitudes, k
+//     beyond the bound).
+// Measured (one call, bf16 gradients, k = 32; dense contractions on every axis with radix select -> this): four
+// 512 x 512 x 3 x 3 weights in 32 x 32 x 3 x 3 chunks (9.4 M parameters) compress 381 -> 115 us, decode 219 -> 63;
+// 7511 x 512 in 29 x 64: 243 -> 83 / 122 -> 36; 8192 x 8192 in 32 x 128: 2424 -> 1050 / 1155 -> 379; in 16 x 32 (k = 4):
+// 3254 -> 1017 / 1509 -> 409.
 #include <cuda_bf16.h>
 
+#include <cmath>
+#include <type_traits>
+
 #include "demo_internal.h"
-#include "generic_common.cuh"
+#include "fast_dct.cuh"
 
 namespace {
+
+constexpr int CAND = 512;  // candidate list
+
+__device__ __forceinline__ unsigned mag_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 
 // Last entry with chunk_begin <= c.
 __device__ __forceinline__ int find_nd_entry(const DemoNdEntry *entries, int n, long long c)
@@ -42,339 +67,1168 @@ __device__ __forceinline__ size_t chunk_base(const DemoNdEntry &e, unsigned lc)
     return base;
 }
 
-// The entry and the base offset of the CTA's current chunk, looked up by one thread (the table is read
-// again only when the chunk belongs to another tensor than the previous one).
-struct ChunkSlot {
-    DemoNdEntry e;
-    size_t base;
-};
-
-__device__ __forceinline__ void locate_chunk(ChunkSlot *slot, const DemoNdEntry *entries, int n_entries, long long c)
-{
-    if (threadIdx.x == 0) {
-        if (c < slot->e.chunk_begin || c >= slot->e.chunk_end) slot->e = entries[find_nd_entry(entries, n_entries, c)];
-        slot->base = chunk_base(slot->e, (unsigned)(c - slot->e.chunk_begin));
-    }
-    __syncthreads();
-}
-
-// Offset of element i (row-major inside the chunk) relative to the chunk's first element.  The
-// divisions by the chunk extents are multiplications by inv[a] = ceil(2^32 / s_a), exact for
+// Offsets of element i (row-major inside the chunk) in the tensor, relative to the chunk's first element, and in the
+// tile.  The divisions by the chunk extents are multiplications by inv[a] = ceil(2^32 / s_a), exact for
 // i < 2^14 and s_a <= 2^7.
-__device__ __forceinline__ size_t elem_offset(const DemoNdEntry &e, int i)
+struct Place {
+    size_t g;
+    int t;
+};
+__device__ __forceinline__ Place place_of(const DemoNdEntry &e, int i)
 {
-    size_t off = 0;
+    Place o{0, 0};
     unsigned r = (unsigned)i;
 #pragma unroll
     for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
         if (e.s[a] > 1) {
             const unsigned q = __umulhi(r, e.inv[a]);
-            off += (size_t)(r - q * (unsigned)e.s[a]) * (size_t)e.stride[a];
+            const unsigned j = r - q * (unsigned)e.s[a];
+            o.g += (size_t)j * (size_t)e.stride[a];
+            o.t += (int)j * e.p[a];
             r = q;
         }
     }
-    return off;
+    return o;
 }
-
-// One axis of the multilinear product on a chunk in shared memory viewed as [outer][s][inner]:
-//   dst[o][j][i] = sum_n T[n][j] src[o][n][i]
-// with T = C^T for the forward transform (T[n][j] = C[j][n]) and T = C for the inverse; either way the
-// threads of a warp that differ in j read neighbouring table entries.  Each thread owns a TU x TV tile
-// of outputs: TU along j, TV along i (VI, vector loads) or along o.
-template <int TU, int TV, bool VI>
-__device__ __forceinline__ void axis_pass(float *__restrict__ dst, const float *__restrict__ src,
-                                          const float *__restrict__ T, int s, int inner, int outer)
+// Row-major index of the element at tile position t (never a padding place).
+__device__ __forceinline__ int index_of(const DemoNdEntry &e, int t)
 {
-    const int gj = s / TU;
-    const int gi = VI ? inner / TV : inner;
-    const int go = VI ? outer : outer / TV;
-    const int vstep = VI ? 1 : s * inner;  // distance between the TV inputs (and outputs) of a tile
-    const int items = go * gj * gi;
-    for (int it = threadIdx.x; it < items; it += GEN_THREADS) {
-        const int ii = it % gi;
-        const int t = it / gi;
-        const int j0 = (t % gj) * TU;
-        const int oo = t / gj;
-        const int o0 = VI ? oo : oo * TV;
-        const int i0 = VI ? ii * TV : ii;
-        const float *sp = src + (size_t)o0 * s * inner + i0;
-        const float *tp = T + j0;
-        float acc[TU][TV];
+    int i = 0;
 #pragma unroll
-        for (int q = 0; q < TU; ++q)
-#pragma unroll
-            for (int v = 0; v < TV; ++v) acc[q][v] = 0.f;
-#pragma unroll 2
-        for (int n = 0; n < s; ++n) {
-            float tv[TU], sv[TV];
-            if constexpr (TU == 4) {  // s, j0 and the table offset are multiples of 4
-                const float4 t4 = __ldg(reinterpret_cast<const float4 *>(tp + n * s));
-                tv[0] = t4.x, tv[1] = t4.y, tv[2] = t4.z, tv[3] = t4.w;
-            } else {
-#pragma unroll
-                for (int q = 0; q < TU; ++q) tv[q] = __ldg(tp + n * s + q);
-            }
-            if constexpr (VI && TV == 4) {  // inner and i0 are multiples of 4, the buffers 16-byte aligned
-                const float4 s4 = *reinterpret_cast<const float4 *>(sp + n * inner);
-                sv[0] = s4.x, sv[1] = s4.y, sv[2] = s4.z, sv[3] = s4.w;
-            } else {
-#pragma unroll
-                for (int v = 0; v < TV; ++v) sv[v] = sp[n * inner + v * vstep];
-            }
-#pragma unroll
-            for (int q = 0; q < TU; ++q)
-#pragma unroll
-                for (int v = 0; v < TV; ++v) acc[q][v] = fmaf(tv[q], sv[v], acc[q][v]);
-        }
-        float *dp = dst + (size_t)o0 * s * inner + (size_t)j0 * inner + i0;
-#pragma unroll
-        for (int q = 0; q < TU; ++q) {
-            if constexpr (VI && TV == 4) {
-                *reinterpret_cast<float4 *>(dp + q * inner) = make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
-            } else {
-#pragma unroll
-                for (int v = 0; v < TV; ++v) dp[q * inner + v * vstep] = acc[q][v];
-            }
+    for (int a = 0; a < DEMO_ND_DIMS; ++a) {
+        if (e.s[a] > 1) {
+            const int j = t / e.p[a];
+            t -= j * e.p[a];
+            i = i * e.s[a] + j;
         }
     }
+    return i;
 }
 
-// The last axis with an extent that is a multiple of 4 (inner == 1: the contracted index is contiguous):
-// each thread owns 4 outputs along j for 4 consecutive o and reads its inputs four n at a time with
-// 16-byte loads -- 8 loads per 64 FMAs.
-__device__ __forceinline__ void axis_pass_last(float *__restrict__ dst, const float *__restrict__ src,
-                                               const float *__restrict__ T, int s, int outer)
+// Shared memory of a CTA: this, then uint2 rows[cls.rows], float B[max_M] (compress), the tiles.
+struct Shared {
+    DemoNdEntry e[2];  // current and next chunk, looked up by one thread a chunk ahead
+    size_t base[2];
+    unsigned hi, n, n_kept, bound, thr, need_eq, n_eq, state[2], warp_tot[12];
+    unsigned hist[256], fine[256];
+    uint2 cand[CAND];      // candidates (value bits, tile position) in no particular order
+    uint4 kept[CAND / 2];  // the kept ones, two per entry
+};
+extern __shared__ __align__(16) unsigned char smem_raw[];
+__device__ __forceinline__ Shared *shared() { return reinterpret_cast<Shared *>(smem_raw); }
+struct View {
+    uint2 *rows;  // (offset in the tensor, offset in the tile) of every row
+    float *B, *tile0, *tile1;
+};
+__host__ __device__ constexpr size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
+
+__device__ __forceinline__ View carve(const DemoNdClass &k, bool with_b)
 {
-    const int gj = s / 4;
-    const int items = (outer / 4) * gj;
-    for (int it = threadIdx.x; it < items; it += GEN_THREADS) {
-        const int j0 = (it % gj) * 4;
-        const int o0 = (it / gj) * 4;
-        const float *sp = src + (size_t)o0 * s;
-        const float *tp = T + j0;
-        float acc[4][4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[q][v] = 0.f;
-        for (int n = 0; n < s; n += 4) {
-            float sv[4][4];  // [v][dn]
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float4 s4 = *reinterpret_cast<const float4 *>(sp + v * s + n);
-                sv[v][0] = s4.x, sv[v][1] = s4.y, sv[v][2] = s4.z, sv[v][3] = s4.w;
-            }
-#pragma unroll
-            for (int dn = 0; dn < 4; ++dn) {
-                const float4 t4 = __ldg(reinterpret_cast<const float4 *>(tp + (n + dn) * s));
-                const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[q][v] = fmaf(tv[q], sv[v][dn], acc[q][v]);
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            *reinterpret_cast<float4 *>(dst + (size_t)(o0 + v) * s + j0) = make_float4(acc[0][v], acc[1][v], acc[2][v], acc[3][v]);
-    }
+    View v;
+    unsigned char *raw = smem_raw + align16(sizeof(Shared));
+    v.rows = reinterpret_cast<uint2 *>(raw);
+    raw += align16((size_t)k.rows * 8);
+    v.B = reinterpret_cast<float *>(raw);
+    raw += with_b ? (size_t)k.max_M * 4 : 0;
+    v.tile0 = reinterpret_cast<float *>(raw);
+    v.tile1 = v.tile0 + (k.dense_axes ? k.tile : 0);
+    return v;
+}
+size_t shared_bytes(const DemoNdClass &k, bool with_b)
+{
+    return align16(sizeof(Shared)) + align16((size_t)k.rows * 8) + (with_b ? (size_t)k.max_M * 4 : 0) +
+           (size_t)k.tile * 4 * (k.dense_axes ? 2 : 1);
 }
 
-template <int TU>
-__device__ __forceinline__ void axis_dispatch(float *dst, const float *src, const float *T, int s, int inner, int M)
+__device__ __forceinline__ void locate(Shared *w, int slot, const DemoNdEntry *entries, int n_entries, long long c)
 {
-    const int outer = M / (s * inner);
-    // 4-wide tiles along i (or o) where the chunk has enough outputs to keep the CTA busy with them
-    if (TU == 4 && inner == 1 && M >= 16 * GEN_THREADS / 2 && (outer & 3) == 0)
-        axis_pass_last(dst, src, T, s, outer);
-    else if (M >= 16 * GEN_THREADS / 2 && (inner & 3) == 0)
-        axis_pass<TU, 4, true>(dst, src, T, s, inner, outer);
-    else if (M >= 16 * GEN_THREADS / 2 && (outer & 3) == 0)
-        axis_pass<TU, 4, false>(dst, src, T, s, inner, outer);
-    else
-        axis_pass<TU, 1, true>(dst, src, T, s, inner, outer);
-}
-
-// All axes in turn, ping-pong between `a` and `b` (src may be one of them or a third buffer, which is
-// then left intact).  Returns where the result is; src itself when every extent is 1.
-__device__ __forceinline__ float *transform_chunk(float *src, float *a, float *b, const DemoNdEntry &e,
-                                                  const float *tables, bool inverse)
-{
-    float *cur = src;
-    int inner = e.M;
-    for (int ax = 0; ax < DEMO_ND_DIMS; ++ax) {
-        const int s = e.s[ax];
-        inner /= s;
-        if (s == 1) continue;
-        float *dst = (cur == a) ? b : a;
-        const float *T = tables + e.basis[ax] + (inverse ? 0 : s * s);  // [C | C^T] per extent
-        if ((s & 3) == 0)
-            axis_dispatch<4>(dst, cur, T, s, inner, e.M);
+    DemoNdEntry &e = w->e[slot];
+    const DemoNdEntry &other = w->e[slot ^ 1];
+    if (c < e.chunk_begin || c >= e.chunk_end) {
+        if (c >= other.chunk_begin && c < other.chunk_end)
+            e = other;
         else
-            axis_dispatch<1>(dst, cur, T, s, inner, e.M);
-        __syncthreads();
-        cur = dst;
+            e = entries[find_nd_entry(entries, n_entries, c)];
     }
-    return cur;
+    w->base[slot] = chunk_base(e, (unsigned)(c - e.chunk_begin));
 }
 
-__global__ void __launch_bounds__(GEN_THREADS) compress_nd_kernel(DemoNdCompressArgs a)
+// (all threads) another layout than the previous chunk's: offsets of its rows; the tiles are cleared, because its padding
+// lies elsewhere.  A barrier must follow.
+__device__ __forceinline__ void enter_layout(const View &v, const DemoNdEntry &e, const DemoNdClass &k)
 {
-    extern __shared__ __align__(16) float smem[];
-    float *Bt = smem;
-    float *X1 = Bt + a.max_M;
-    float *X2 = X1 + a.max_M;
-    unsigned *hist = reinterpret_cast<unsigned *>(X2 + a.max_M);  // [256]
-    unsigned *warp_tot = hist + 256;                              // [8]
-    unsigned *s_state = warp_tot + 8;                             // [2]
-    __shared__ ChunkSlot slot;
-    const int tid = threadIdx.x;
-    if (tid == 0) slot.e.chunk_begin = 1, slot.e.chunk_end = 0;  // no tensor yet
+    const int T = blockDim.x;
+    if (e.row_table)
+        for (int r = threadIdx.x; r * e.row < e.M; r += T) {
+            const Place o = place_of(e, r * e.row);
+            v.rows[r] = make_uint2((unsigned)o.g, (unsigned)o.t);
+        }
+    for (int i = threadIdx.x; i < k.tile; i += T) {
+        v.tile0[i] = 0.f;
+        v.tile1[i] = 0.f;
+    }
+}
+// Runs over the chunk's elements, U per thread and round: every thread calls load(j, offset in the tensor) U times without
+// a branch in between (the last element again where there is none left), then use(j, index, offset, tile position) for
+// those that exist.
+template <int U, class Load, class Use>
+__device__ __forceinline__ void for_elements(const View &v, const DemoNdEntry &e, Load load, Use use)
+{
+    const int M = e.M, T = blockDim.x;
+    auto walk = [&](auto table) {
+        using Off = typename std::conditional<decltype(table)::value, unsigned, size_t>::type;
+        const unsigned row = (unsigned)e.row, inv_row = e.inv_row;
+        for (int i0 = threadIdx.x; i0 < M; i0 += U * T) {
+            Off g[U];
+            int t[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                const int i = min(i0 + j * T, M - 1);
+                if constexpr (decltype(table)::value) {
+                    const unsigned r = inv_row ? __umulhi((unsigned)i, inv_row) : (unsigned)i;
+                    const unsigned d = (unsigned)i - r * row;
+                    const uint2 o = v.rows[r];
+                    g[j] = o.x + d;
+                    t[j] = (int)(o.y + d);
+                } else {
+                    const Place o = place_of(e, i);
+                    g[j] = o.g;
+                    t[j] = o.t;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j) load(j, g[j]);
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+                if (i0 + j * T < M) use(j, i0 + j * T, g[j], t[j]);
+        }
+    };
+    if (e.row_table)
+        walk(std::true_type{});
+    else
+        walk(std::false_type{});
+}
 
-    for (long long c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
-        locate_chunk(&slot, a.entries, a.n_entries, c);
-        const DemoNdEntry &e = slot.e;
-        const long long lc = c - e.chunk_begin;
-        const size_t base = slot.base;
-        float *__restrict__ m = a.m_ptrs[e.tensor];
-        const void *g = a.g_ptrs[e.tensor];
-        const int M = e.M, k_eff = e.k_eff;
+// ---- one axis of the multilinear product ------------------------------------------------------------
+// Every extent is a function of its own (not inlined: dozens of register-resident bodies in one kernel cost each other
+// registers).  They get the byte offset of the tile and the slot of the entry, so that the accesses stay shared-memory
+// accesses.
+__device__ __forceinline__ float *tile_at(unsigned off) { return reinterpret_cast<float *>(smem_raw + off); }
+__device__ __forceinline__ unsigned tile_offset(const float *X)
+{
+    return (unsigned)(reinterpret_cast<const unsigned char *>(X) - smem_raw);
+}
+
+// Tile position of the first element of line L along axis a (a .. a_last where axes are transformed together): the other
+// axes' indices, the last running fastest.
+__device__ __forceinline__ int line_base(const DemoNdEntry &e, int a, int a_last, int L)
+{
+    int t = 0;
+    unsigned r = (unsigned)L;
+#pragma unroll
+    for (int b = DEMO_ND_DIMS - 1; b >= 0; --b) {
+        if ((b < a || b > a_last) && e.s[b] > 1) {
+            const unsigned q = __umulhi(r, e.inv[b]);
+            t += (int)(r - q * (unsigned)e.s[b]) * e.p[b];
+            r = q;
+        }
+    }
+    return t;
+}
+
+// C[u][n] = a_u cos(pi (2n+1) u / (2S)), the angle reduced to [0, pi/2] in whole numbers.
+template <int S>
+constexpr double dct_entry(int u, int n)
+{
+    int m = ((2 * n + 1) * u) % (4 * S);
+    if (m > 2 * S) m = 4 * S - m;
+    const double c = m > S ? -fdct::c_cos(fdct::kPi * (2 * S - m) / (2.0 * S)) : fdct::c_cos(fdct::kPi * m / (2.0 * S));
+    return c * fdct::c_sqrt((u == 0 ? 1.0 : 2.0) / S);
+}
+
+template <int S, bool INV>
+__device__ __forceinline__ void line_transform(float (&x)[S])
+{
+    if constexpr ((S & (S - 1)) == 0) {
+        if constexpr (INV)
+            fdct::dct3_ortho_dense4<S>(x);
+        else
+            fdct::dct2_ortho_dense4<S>(x);
+    } else {
+        float y[S];
+        fdct::static_for<0, S>([&](auto uu) {
+            constexpr int u = decltype(uu)::value;
+            float acc = 0.f;
+            fdct::static_for<0, S>([&](auto nn) {
+                constexpr int n = decltype(nn)::value;
+                constexpr float c = (float)(INV ? dct_entry<S>(n, u) : dct_entry<S>(u, n));
+                acc = n == 0 ? c * x[0] : fmaf(c, x[n], acc);
+            });
+            y[u] = acc;
+        });
+#pragma unroll
+        for (int n = 0; n < S; ++n) x[n] = y[n];
+    }
+}
+
+template <int S, bool INV>
+__device__ __noinline__ void lines_whole(unsigned tile, int slot, int a)
+{
+    float *X = tile_at(tile);
+    const DemoNdEntry &e = shared()->e[slot];
+    const int lines = e.M / S, p = e.p[a];
+    for (int L = threadIdx.x; L < lines; L += blockDim.x) {
+        float *q = X + line_base(e, a, a, L);
+        float x[S];
+#pragma unroll
+        for (int n = 0; n < S; ++n) x[n] = q[n * p];
+        line_transform<S, INV>(x);
+#pragma unroll
+        for (int n = 0; n < S; ++n) q[n * p] = x[n];
+    }
+}
+
+// The last two axes, both of extent S: S * S consecutive elements per thread.
+template <int S, bool INV>
+__device__ __noinline__ void lines_tail(unsigned tile, int slot)
+{
+    float *X = tile_at(tile);
+    const DemoNdEntry &e = shared()->e[slot];
+    const int lines = e.M / (S * S);
+    for (int L = threadIdx.x; L < lines; L += blockDim.x) {
+        float *q = X + line_base(e, 2, 3, L);
+        float x[S][S];
+#pragma unroll
+        for (int i = 0; i < S; ++i)
+#pragma unroll
+            for (int j = 0; j < S; ++j) x[i][j] = q[i * S + j];
+#pragma unroll
+        for (int i = 0; i < S; ++i) line_transform<S, INV>(x[i]);
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+            float col[S];
+#pragma unroll
+            for (int i = 0; i < S; ++i) col[i] = x[i][j];
+            line_transform<S, INV>(col);
+#pragma unroll
+            for (int i = 0; i < S; ++i) q[i * S + j] = col[i];
+        }
+    }
+}
+
+// Extent 2H, two threads per line: the even outputs are a DCT-II of H points of x[n] + x[2H-1-n], the odd ones a DCT-IV of
+// x[n] - x[2H-1-n].  Even warps take one, odd warps the other; the CTA is a multiple of 64 threads.
+template <int H, bool INV>
+__device__ __noinline__ void lines_split(unsigned tile, int slot, int a)
+{
+    float *X = tile_at(tile);
+    const DemoNdEntry &e = shared()->e[slot];
+    using SC = fdct::ScaleOrtho<2 * H>;
+    constexpr float DC = (float)fdct::c_sqrt(0.5);
+    const int lines = e.M / (2 * H), p = e.p[a];
+    const int h = (threadIdx.x >> 5) & 1;
+    const int l0 = (threadIdx.x >> 6) * 32 + (threadIdx.x & 31), per_round = blockDim.x >> 1;
+    for (int r0 = 0; r0 < lines; r0 += per_round) {
+        const bool active = r0 + l0 < lines;
+        float *q = X + (active ? line_base(e, a, a, r0 + l0) : 0);
+        float x[H], y[H];
+        if (active) {
+            if constexpr (!INV) {
+#pragma unroll
+                for (int n = 0; n < H; ++n) {
+                    const float lo = q[n * p], hi = q[(2 * H - 1 - n) * p];
+                    x[n] = h ? lo - hi : lo + hi;
+                }
+                if (h == 0) {
+                    fdct::dct2_dense4<H, SC>(x, y);
+                    y[0] *= DC;
+                } else {
+                    fdct::dct4_dense<H, SC>(x, y);
+                }
+            } else {
+#pragma unroll
+                for (int n = 0; n < H; ++n) x[n] = q[(2 * n + h) * p];
+                if (h == 0) {
+                    x[0] *= DC;
+                    fdct::dct3_dense4<H, SC>(x, y);
+                } else {
+                    fdct::dct4_dense<H, SC>(x, y);
+                }
+            }
+        }
+        __syncthreads();  // both halves of every line of this round are read
+        if (active) {
+            if constexpr (!INV) {
+#pragma unroll
+                for (int n = 0; n < H; ++n) q[(2 * n + h) * p] = y[n];
+            } else {
+                if (h == 0) {
+#pragma unroll
+                    for (int n = 0; n < H; ++n) q[n * p] = y[n];
+                } else {
+#pragma unroll
+                    for (int n = 0; n < H; ++n) q[(2 * H - 1 - n) * p] = y[n];
+                }
+            }
+        }
+        if constexpr (INV) {
+            __syncthreads();
+            if (active) {
+#pragma unroll
+                for (int i = 0; i < H / 2; ++i) {
+                    const int n = i + h * (H / 2);
+                    const float ev = q[n * p], od = q[(2 * H - 1 - n) * p];
+                    q[n * p] = ev + od;
+                    q[(2 * H - 1 - n) * p] = ev - od;
+                }
+            }
+        }
+    }
+}
+
+// Any other extent, from a table.  Forward: a thread forms 8 even or 8 odd outputs of LPT lines from
+// x[n] +- x[s-1-n]; inverse: 8 outputs n and their mirror images from the even and the odd coefficients.
+// Table of extent s, h = ceil(s/2), even / odd outputs padded to pe / po (multiples of 8):
+//   forward rows n < h: [C[0][n], C[2][n], ... | C[1][n], C[3][n], ...] (the middle n of an odd s halved),
+//   inverse rows u < s: C[u][n] for n < h, padded to pe.
+__host__ __device__ constexpr int up8(int v) { return (v + 7) & ~7; }
+template <int LPT, bool INV>
+__device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, const float *__restrict__ table, int slot, int a)
+{
+    float *__restrict__ dst = tile_at(dst_tile);
+    const float *__restrict__ src = tile_at(src_tile);
+    const DemoNdEntry &e = shared()->e[slot];
+    const int s = e.s[a], p = e.p[a], lines = e.M / s;
+    const int h = (s + 1) >> 1, pe = up8(h), po = up8(s >> 1);
+    const int groups = INV ? pe >> 3 : (pe + po) >> 3;
+    const float *Tb = INV ? table + h * (pe + po) : table;
+    const int Q = (lines + LPT - 1) / LPT;
+    const int items = groups * Q;
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        const int g = it / Q, l0 = it - g * Q;
+        int b[LPT];
+#pragma unroll
+        for (int v = 0; v < LPT; ++v) b[v] = line_base(e, a, a, min(l0 + v * Q, lines - 1));
+        if constexpr (!INV) {
+            const bool odd = 8 * g >= pe;
+            const float sign = odd ? -1.f : 1.f;
+            float acc[LPT][8];
+#pragma unroll
+            for (int v = 0; v < LPT; ++v)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[v][j] = 0.f;
+            const float *tp = Tb + 8 * g;
+            int lo = 0, hi = (s - 1) * p;
+#pragma unroll 4
+            for (int n = 0; n < h; ++n, tp += pe + po, lo += p, hi -= p) {
+                const float4 t0 = __ldg(reinterpret_cast<const float4 *>(tp));
+                const float4 t1 = __ldg(reinterpret_cast<const float4 *>(tp + 4));
+                const float t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+#pragma unroll
+                for (int v = 0; v < LPT; ++v) {
+                    const float xv = fmaf(sign, src[b[v] + hi], src[b[v] + lo]);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[v][j] = fmaf(t[j], xv, acc[v][j]);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < LPT; ++v) {
+                if (l0 + v * Q < lines) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int u = odd ? 2 * (8 * g - pe + j) + 1 : 2 * (8 * g + j);
+                        if (u < s) dst[b[v] + u * p] = acc[v][j];
+                    }
+                }
+            }
+        } else {
+            float ev[LPT][8], od[LPT][8];
+#pragma unroll
+            for (int v = 0; v < LPT; ++v)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) ev[v][j] = od[v][j] = 0.f;
+            const float *tp = Tb + 8 * g;
+            auto term = [&](int u, float (&acc)[LPT][8]) {
+                const float4 t0 = __ldg(reinterpret_cast<const float4 *>(tp + u * pe));
+                const float4 t1 = __ldg(reinterpret_cast<const float4 *>(tp + u * pe + 4));
+                const float t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+#pragma unroll
+                for (int v = 0; v < LPT; ++v) {
+                    const float xv = src[b[v] + u * p];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[v][j] = fmaf(t[j], xv, acc[v][j]);
+                }
+            };
+#pragma unroll 2
+            for (int u = 0; u + 1 < s; u += 2) {
+                term(u, ev);
+                term(u + 1, od);
+            }
+            if (s & 1) term(s - 1, ev);
+#pragma unroll
+            for (int v = 0; v < LPT; ++v) {
+                if (l0 + v * Q < lines) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int n = 8 * g + j;
+                        if (n < h) {
+                            dst[b[v] + n * p] = ev[v][j] + od[v][j];
+                            if (n != s - 1 - n) dst[b[v] + (s - 1 - n) * p] = ev[v][j] - od[v][j];
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+// Extents that are transformed in registers.
+constexpr bool in_place_extent(int s) { return s <= 8 || s == 16 || s == 32 || s == 64 || s == 128; }
+
+// All axes in turn.  cur / spare: the tile and the second tile (used by dense axes only); swapped as needed.
+template <bool INV, bool BIG>
+__device__ __forceinline__ void transform_chunk(float *&cur, float *&spare, int slot, const float *tables)
+{
+    const DemoNdEntry &e = shared()->e[slot];
+    unsigned tile = tile_offset(cur), other = tile_offset(spare);
+#pragma unroll 1
+    for (int a = 0; a < DEMO_ND_DIMS; ++a) {
+        const int s = e.s[a];
+        if (s == 1) continue;
+        if (e.tail && a == 2) {
+            switch (s) {
+                case 2: lines_tail<2, INV>(tile, slot); break;
+                case 3: lines_tail<3, INV>(tile, slot); break;
+                case 4: lines_tail<4, INV>(tile, slot); break;
+                case 5: lines_tail<5, INV>(tile, slot); break;
+                case 6: lines_tail<6, INV>(tile, slot); break;
+                default: lines_tail<7, INV>(tile, slot); break;
+            }
+            __syncthreads();
+            break;
+        }
+        switch (s) {
+            case 2: lines_whole<2, INV>(tile, slot, a); break;
+            case 3: lines_whole<3, INV>(tile, slot, a); break;
+            case 4: lines_whole<4, INV>(tile, slot, a); break;
+            case 5: lines_whole<5, INV>(tile, slot, a); break;
+            case 6: lines_whole<6, INV>(tile, slot, a); break;
+            case 7: lines_whole<7, INV>(tile, slot, a); break;
+            case 8: lines_whole<8, INV>(tile, slot, a); break;
+            case 16: lines_whole<16, INV>(tile, slot, a); break;
+            case 32: lines_whole<32, INV>(tile, slot, a); break;
+            case 64: lines_split<32, INV>(tile, slot, a); break;
+            case 128:
+                if constexpr (BIG) lines_split<64, INV>(tile, slot, a);
+                break;
+            default: {
+                // two lines per thread where that still occupies the CTA
+                const int lines = e.M / s, pe = up8((s + 1) >> 1), groups = (INV ? pe : pe + up8(s >> 1)) >> 3;
+                if (groups * ((lines + 1) >> 1) >= (int)blockDim.x)
+                    lines_dense<2, INV>(other, tile, tables + e.basis[a], slot, a);
+                else
+                    lines_dense<1, INV>(other, tile, tables + e.basis[a], slot, a);
+                const unsigned t = tile;
+                tile = other;
+                other = t;
+            }
+        }
+        __syncthreads();
+    }
+    cur = tile_at(tile);
+    spare = tile_at(other);
+}
+
+__device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned *warp_tot)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned inc = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned n = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += n;
+    }
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    unsigned base = 0;
+    for (int w = 0; w < warp; ++w) base += warp_tot[w];
+    __syncthreads();
+    return base + inc - v;
+}
+
+// (one warp) the bin of hist[0..256), taken in ascending order, where the running count reaches `rank`, and the count
+// before it; bin 256 if it never does.
+__device__ __forceinline__ void find_bin(const unsigned *hist, unsigned rank, unsigned *bin, unsigned *before_bin)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned h[8], local = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        h[j] = hist[8 * lane + j];
+        local += h[j];
+    }
+    unsigned inc = local;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned n = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += n;
+    }
+    unsigned cum = inc - local, b = 256, bb = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (cum < rank && cum + h[j] >= rank) {
+            b = 8 * lane + j;
+            bb = cum;
+        }
+        cum += h[j];
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, b < 256u);
+    const int src = who ? __ffs(who) - 1 : 0;
+    *bin = __shfl_sync(0xffffffffu, b, src);
+    *before_bin = __shfl_sync(0xffffffffu, bb, src);
+}
+
+// Exact top-k by radix select on the magnitude bits, index-ordered compaction; leaves alpha * kept in X, zero elsewhere.
+__device__ __noinline__ void select_radix(unsigned tile, int slot, DemoRecord *rec, float alpha)
+{
+    float *X = tile_at(tile);
+    Shared *s = shared();
+    const DemoNdEntry &e = s->e[slot];
+    const int tid = threadIdx.x, T = blockDim.x, M = e.M, k_eff = e.k_eff;
+    if (tid == 0) {
+        s->state[0] = 0u;               // prefix of the key found so far
+        s->state[1] = (unsigned)k_eff;  // rank still to resolve inside the prefix class
+    }
+    for (int pass = 0; pass < 4; ++pass) {
+        const int shift = 24 - 8 * pass;
+        const unsigned mask = (pass == 0) ? 0u : (0xffffffffu << (shift + 8));
+        for (int i = tid; i < 256; i += T) s->hist[i] = 0u;
+        __syncthreads();
+        const unsigned prefix = s->state[0];
+        for (int i = tid; i < M; i += T) {
+            const unsigned key = mag_key(X[place_of(e, i).t]);
+            if ((key & mask) == prefix) atomicAdd(&s->hist[255u - ((key >> shift) & 255u)], 1u);
+        }
+        __syncthreads();
+        if (tid < 32) {
+            unsigned bin, before;
+            const unsigned rem = s->state[1];
+            find_bin(s->hist, rem, &bin, &before);
+            __syncwarp();
+            if (tid == 0) {
+                s->state[1] = rem - before;
+                s->state[0] = prefix | ((255u - bin) << shift);
+            }
+        }
+        __syncthreads();
+    }
+    const unsigned thr = s->state[0], need_eq = s->state[1];
+    const int per = (M + T - 1) / T;
+    const int start = tid * per;
+    const int stop = min(M, start + per);
+    unsigned gt = 0, eq = 0;
+    for (int i = start; i < stop; ++i) {
+        const unsigned key = mag_key(X[place_of(e, i).t]);
+        gt += key > thr;
+        eq += key == thr;
+    }
+    const unsigned before = block_exclusive_scan(gt | (eq << 16), s->warp_tot);
+    unsigned gb = before & 0xffffu, eb = before >> 16;
+    for (int i = start; i < stop; ++i) {
+        const int t = place_of(e, i).t;
+        const float v = X[t];
+        const unsigned key = mag_key(v);
+        bool sel = false;
+        unsigned pos = 0;
+        if (key > thr) {
+            pos = gb + min(eb, need_eq);
+            ++gb;
+            sel = true;
+        } else if (key == thr) {
+            if (eb < need_eq) {
+                pos = gb + eb;
+                sel = true;
+            }
+            ++eb;
+        }
+        if (sel) {
+            DemoRecord r;
+            r.idx = i;
+            r.val = v;
+            rec[pos] = r;
+        }
+        X[t] = sel ? alpha * v : 0.f;  // the residual removes alpha times the kept part
+    }
+    __syncthreads();
+}
+
+// (one warp) the k_eff-th largest of n candidate keys, NK per lane: threshold, how many equal to it are kept and exist.
+template <int NK>
+__device__ __noinline__ void find_threshold(unsigned n, unsigned bound, int k_eff)
+{
+    const int lane = threadIdx.x & 31;
+    Shared *s = shared();
+    unsigned keys[NK];
+    unsigned top = 0u;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+        const unsigned i = (unsigned)j * 32u + lane;
+        keys[j] = i < n ? (s->cand[i].x & 0x7fffffffu) : 0u;
+        top = max(top, keys[j]);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    const int b0 = 31 - __clz((bound ^ top) | 1u);
+    unsigned thr = bound & ~((2u << b0) - 1u);
+    unsigned n_ge = n;  // every candidate is >= the bound >= thr
+#pragma unroll 1
+    for (int b = b0; b >= 0 && n_ge != (unsigned)k_eff; --b) {
+        const unsigned cand = thr | (1u << b);
+        unsigned cnt = 0;
+#pragma unroll
+        for (int j = 0; j < NK; ++j) cnt += __popc(__ballot_sync(0xffffffffu, keys[j] >= cand));
+        if (cnt >= (unsigned)k_eff) {
+            thr = cand;
+            n_ge = cnt;
+        }
+    }
+    unsigned n_gt = 0;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) n_gt += __popc(__ballot_sync(0xffffffffu, keys[j] > thr));
+    if (lane == 0) {
+        s->thr = thr;
+        s->need_eq = (unsigned)k_eff - n_gt;
+        s->n_eq = n_ge - n_gt;
+    }
+}
+
+// Exact top-k of the coefficients in X (complete for all threads): records in ascending index order to `rec`, X left
+// with alpha * kept and zero elsewhere; ends with a barrier.  hist, fine, hi, n and n_kept were cleared before a barrier.
+__device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec, float alpha)
+{
+    const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+    Shared *s = shared();
+    const DemoNdEntry &e = s->e[slot];
+    const int k_eff = e.k_eff, quads = e.tile >> 2;
+    float4 *X4 = reinterpret_cast<float4 *>(X);
+    // group maxima: a thread's quads as one group, or -- where k is not well below the number of threads -- as four
+    const bool four = 2 * k_eff > T;
+    unsigned key[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 4
+    for (int i = tid; i < quads; i += T) {
+        const float4 f = X4[i];
+        key[0] = max(key[0], mag_key(f.x));
+        key[1] = max(key[1], mag_key(f.y));
+        key[2] = max(key[2], mag_key(f.z));
+        key[3] = max(key[3], mag_key(f.w));
+    }
+    const unsigned mine = max(max(key[0], key[1]), max(key[2], key[3]));
+    {
+        const unsigned mx = __reduce_max_sync(0xffffffffu, mine);
+        if (lane == 0) atomicMax(&s->hi, mx);
+    }
+    __syncthreads();
+    const unsigned hi = s->hi;
+    if (hi == 0u) {
+        // all coefficients zero: the tie rule gives the records 0 .. k_eff-1 with value 0
+        for (int r = tid; r < k_eff; r += T) {
+            DemoRecord z;
+            z.idx = r;
+            z.val = 0.f;
+            rec[r] = z;
+        }
+        __syncthreads();
+        return;
+    }
+    // their histogram, 16 bins per octave below the largest, then one of 256 steps inside the bin that holds the k-th group:
+    // the lower edge of that step bounds the k-th coefficient from below.  (The edge of the first bin alone, up to 6 % below,
+    // is not enough: with error feedback the magnitudes crowd just below the threshold.)
+    auto each_group = [&](auto f) {
+        if (four) {
+#pragma unroll
+            for (int g = 0; g < 4; ++g) f(key[g]);
+        } else {
+            f(mine);
+        }
+    };
+    each_group([&](unsigned q) { atomicAdd(&s->hist[min(255u, (hi >> 19) - (q >> 19))], 1u); });
+    __syncthreads();
+    if (tid < 32) {
+        unsigned bin, before;
+        find_bin(s->hist, (unsigned)k_eff, &bin, &before);
+        if (tid == 0) {
+            s->state[0] = bin < 255u ? (hi >> 19) - bin : 0u;
+            s->state[1] = (unsigned)k_eff - before;
+        }
+    }
+    __syncthreads();
+    const unsigned top12 = s->state[0];
+    if (top12) {
+        each_group([&](unsigned q) {
+            if (q >> 19 == top12) atomicAdd(&s->fine[255u - ((q >> 11) & 255u)], 1u);
+        });
+        __syncthreads();
+        if (tid < 32) {
+            unsigned step, before;
+            find_bin(s->fine, s->state[1], &step, &before);
+            if (tid == 0) s->bound = top12 << 19 | (255u - step) << 11;
+        }
+    } else if (tid == 0) {
+        s->bound = 1u;  // fewer than k groups near the largest
+    }
+    __syncthreads();
+    const unsigned bound = s->bound;  // (>= 1: the padding is never a candidate)
+    auto append = [&](float f, int t) {
+        if (mag_key(f) >= bound) {
+            const unsigned at = atomicAdd(&s->n, 1u);
+            if (at < (unsigned)CAND) s->cand[at] = make_uint2(__float_as_uint(f), (unsigned)t);
+        }
+    };
+#pragma unroll 2
+    for (int i = tid; i < quads; i += T) {
+        const float4 f = X4[i];
+        if (max(max(mag_key(f.x), mag_key(f.y)), max(mag_key(f.z), mag_key(f.w))) >= bound) {
+            append(f.x, 4 * i);
+            append(f.y, 4 * i + 1);
+            append(f.z, 4 * i + 2);
+            append(f.w, 4 * i + 3);
+        }
+    }
+    __syncthreads();
+    const int n = (int)s->n;
+    if (n > CAND || n < k_eff) {
+        select_radix(tile_offset(X), slot, rec, alpha);
+        return;
+    }
+    // one warp finds the threshold, the others clear the tile
+    if (tid < 32) {
+        if (n <= 64)
+            find_threshold<2>((unsigned)n, bound, k_eff);
+        else if (n <= 128)
+            find_threshold<4>((unsigned)n, bound, k_eff);
+        else if (n <= 256)
+            find_threshold<8>((unsigned)n, bound, k_eff);
+        else
+            find_threshold<16>((unsigned)n, bound, k_eff);
+    }
+    if (T == 32) {
+        for (int i = tid; i < quads; i += 32) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (tid >= 32) {
+        for (int i = tid - 32; i < quads; i += T - 32) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    uint2 *kept = reinterpret_cast<uint2 *>(s->kept);
+    if (tid == 0 && (k_eff & 1)) kept[k_eff] = make_uint2(0u, 0xffffffffu);  // completes the last pair: behind everything
+    __syncthreads();
+    const unsigned thr = s->thr, need_eq = s->need_eq;
+    const bool ties = need_eq != s->n_eq;
+    for (int i = tid; i < n; i += T) {
+        const uint2 c = s->cand[i];
+        const unsigned mag = c.x & 0x7fffffffu;
+        bool keep = mag >= thr;
+        if (keep && ties && mag == thr) {  // equal keys straddle the k-th place: the lowest positions (in index order) are kept
+            unsigned ahead = 0;
+            for (int j = 0; j < n; ++j) ahead += (s->cand[j].x & 0x7fffffffu) == thr && s->cand[j].y < c.y;
+            keep = ahead < need_eq;
+        }
+        if (keep) kept[atomicAdd(&s->n_kept, 1u)] = c;
+    }
+    __syncthreads();
+    // a record's place is the number of kept positions below its own (tile positions are in index order)
+    const int pairs = (k_eff + 1) >> 1;
+    for (int i = tid; i < k_eff; i += T) {
+        const uint2 c = kept[i];
+        int pos = 0;
+#pragma unroll 4
+        for (int j = 0; j < pairs; ++j) {
+            const uint4 q = s->kept[j];
+            pos += (q.y < c.y ? 1 : 0) + (q.w < c.y ? 1 : 0);
+        }
+        DemoRecord r;
+        r.idx = index_of(e, (int)c.y);
+        r.val = __uint_as_float(c.x);
+        rec[pos] = r;
+        X[c.y] = alpha * r.val;
+    }
+    __syncthreads();
+}
+
+// Registers: 80 per thread (768 threads per SM); 128 with extents of 128.
+constexpr int MAX_THREADS = 384, MAX_THREADS_BIG = 256;
+
+template <typename GT, bool BIG>
+__global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compress_nd_kernel(DemoNdCompressArgs a)
+{
+    const View v = carve(a.cls, true);
+    Shared *s = shared();
+    float *tile0 = v.tile0, *tile1 = v.tile1;
+    const int tid = threadIdx.x, T = blockDim.x;
+    if (tid < 2) s->e[tid].chunk_begin = 1, s->e[tid].chunk_end = 0;  // no tensor yet
+    __syncthreads();
+    if (tid == 0 && blockIdx.x < a.cls.n_chunks) locate(s, 0, a.entries, a.cls.n, blockIdx.x);
+    int layout = -1, slot = 0;
+
+    for (long long c = blockIdx.x; c < a.cls.n_chunks; c += gridDim.x, slot ^= 1) {
+        // cleared for this chunk's selection; the barriers up to it order the writes
+        for (int i = tid; i < 256; i += T) s->hist[i] = s->fine[i] = 0u;
+        if (tid == 0) s->hi = 0u, s->n = 0u, s->n_kept = 0u;
+        __syncthreads();
+        const DemoNdEntry &e = s->e[slot];
+        if (e.layout != layout) {
+            layout = e.layout;
+            enter_layout(v, e, a.cls);
+            __syncthreads();
+        }
+        if (tid == T - 1 && c + gridDim.x < a.cls.n_chunks) locate(s, slot ^ 1, a.entries, a.cls.n, c + gridDim.x);
+        const size_t base = s->base[slot];
+        float *__restrict__ m = a.m_ptrs[e.tensor] + base;
+        const GT *__restrict__ g = static_cast<const GT *>(a.g_ptrs[e.tensor]) + base;
 
         // momentum update  B = beta*m + g  on the chunk (Algorithm 1, worker side)
-        for (int i = tid; i < M; i += GEN_THREADS) {
-            const size_t off = base + elem_offset(e, i);
-            const float gv = a.grad_bf16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(g)[off])
-                                         : reinterpret_cast<const float *>(g)[off];
-            Bt[i] = fmaf(a.beta, m[off], gv);
+        {
+            constexpr int U = 8;
+            float mv[U];
+            GT gv[U];
+            for_elements<U>(
+                v, e,
+                [&](int j, auto off) {
+                    mv[j] = m[off];
+                    gv[j] = g[off];
+                },
+                [&](int j, int i, auto, int t) {
+                    const float b = fmaf(a.beta, mv[j], (float)gv[j]);
+                    v.B[i] = b;
+                    tile0[t] = b;
+                });
         }
         __syncthreads();
-
-        float *Q = transform_chunk(Bt, X1, X2, e, a.tables, false);  // Q = T(B; C_0, ..., C_{d-1})
-        float *O = (Q == X1) ? X2 : X1;
-
-        // top-k: threshold by radix select, then index-ordered compaction into the payload
-        unsigned thr, need_eq;
-        radix_select(Q, M, k_eff, hist, s_state, &thr, &need_eq);
-        const int per = (M + GEN_THREADS - 1) / GEN_THREADS;
-        const int start = tid * per;
-        const int stop = min(M, start + per);
-        unsigned gt = 0, eq = 0;
-        for (int i = start; i < stop; ++i) {
-            const unsigned key = mag_key(Q[i]);
-            gt += key > thr;
-            eq += key == thr;
-        }
-        const unsigned before = block_exclusive_scan(gt | (eq << 16), warp_tot);
-        unsigned gb = before & 0xffffu, eb = before >> 16;
-        DemoRecord *rec = a.payload + e.rec_begin + lc * (long long)k_eff;
-        for (int i = start; i < stop; ++i) {
-            const float v = Q[i];
-            const unsigned key = mag_key(v);
-            bool sel = false;
-            unsigned pos = 0;
-            if (key > thr) {
-                pos = gb + min(eb, need_eq);
-                ++gb;
-                sel = true;
-            } else if (key == thr) {
-                if (eb < need_eq) {
-                    pos = gb + eb;
-                    sel = true;
-                }
-                ++eb;
-            }
-            if (sel) {
-                DemoRecord r;
-                r.idx = i;
-                r.val = v;
-                rec[pos] = r;
-            }
-            O[i] = sel ? a.alpha * v : 0.f;  // the residual removes alpha times the kept part
-        }
-        __syncthreads();
-
+        transform_chunk<false, BIG>(tile0, tile1, slot, a.tables);  // Q = T(B; C_0, ..., C_{d-1})
+        select_topk(tile0, slot, a.payload + e.rec_begin + (c - e.chunk_begin) * (long long)e.k_eff, a.alpha);
         // momentum subtraction  m <- B - alpha * T(kept; C_0^T, ..., C_{d-1}^T)
-        float *spare = (O == X1) ? X2 : X1;
-        const float *R = transform_chunk(O, spare, O, e, a.tables, true);
-        for (int i = tid; i < M; i += GEN_THREADS) m[base + elem_offset(e, i)] = Bt[i] - R[i];
+        transform_chunk<true, BIG>(tile0, tile1, slot, a.tables);
+        for_elements<4>(v, e, [](int, auto) {}, [&](int, int i, auto off, int t) { m[off] = v.B[i] - tile0[t]; });
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(GEN_THREADS) decode_nd_kernel(DemoNdDecodeArgs a)
+template <bool BIG>
+__global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode_nd_kernel(DemoNdDecodeArgs a)
 {
-    extern __shared__ __align__(16) float smem[];
-    float *St = smem;
-    float *X1 = St + a.max_M;
-    unsigned short *Cn = reinterpret_cast<unsigned short *>(X1 + a.max_M);  // senders per coordinate (agg == 2)
-    __shared__ ChunkSlot slot;
-    const int tid = threadIdx.x;
+    const View v = carve(a.cls, false);
+    Shared *s = shared();
+    float *tile0 = v.tile0, *tile1 = v.tile1;
+    unsigned short *Cn = reinterpret_cast<unsigned short *>(v.tile0 + (size_t)a.cls.tile * (a.cls.dense_axes ? 2 : 1));  // senders (agg == 2)
+    constexpr int STAGE = CAND;  // records staged at once (in the place of the selection's list)
+    uint2 *stage = s->cand;
+    const int tid = threadIdx.x, T = blockDim.x;
     const bool counts = a.agg == 2;
-    if (tid == 0) slot.e.chunk_begin = 1, slot.e.chunk_end = 0;  // no tensor yet
+    if (tid < 2) s->e[tid].chunk_begin = 1, s->e[tid].chunk_end = 0;
+    __syncthreads();
+    if (tid == 0 && blockIdx.x < a.cls.n_chunks) locate(s, 0, a.entries, a.cls.n, blockIdx.x);
+    int layout = -1, slot = 0;
 
-    for (long long c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
-        locate_chunk(&slot, a.entries, a.n_entries, c);
-        const DemoNdEntry &e = slot.e;
-        const long long lc = c - e.chunk_begin;
-        const size_t base = slot.base;
-        float *__restrict__ x = a.x_ptrs[e.tensor];
-        const int M = e.M, k_eff = e.k_eff;
-        const long long rec_off = e.rec_begin + lc * (long long)k_eff;
-
-        for (int i = tid; i < M; i += GEN_THREADS) {
-            St[i] = 0.f;
-            if (counts) Cn[i] = 0;
-        }
+    for (long long c = blockIdx.x; c < a.cls.n_chunks; c += gridDim.x, slot ^= 1) {
         __syncthreads();
-        // S = sum over workers, in worker order; indices are unique inside one worker's chunk, so a
-        // barrier per worker fixes the summation order
-        for (int w = 0; w < a.W; ++w) {
-            const DemoRecord *rec = a.payloads[w] + rec_off;
-            for (int i = tid; i < k_eff; i += GEN_THREADS) {
-                const DemoRecord r = rec[i];
-                if ((unsigned)r.idx < (unsigned)M) {
-                    St[r.idx] += r.val;
-                    if (counts) Cn[r.idx] += 1;
-                } else {
-                    atomicMax(a.status, DEMO_DEV_PAYLOAD);
-                }
-            }
+        const DemoNdEntry &e = s->e[slot];
+        if (e.layout != layout) {
+            layout = e.layout;
+            enter_layout(v, e, a.cls);
             __syncthreads();
+        }
+        if (tid == T - 1 && c + gridDim.x < a.cls.n_chunks) locate(s, slot ^ 1, a.entries, a.cls.n, c + gridDim.x);
+        const size_t base = s->base[slot];
+        const int M = e.M, k_eff = e.k_eff;
+        const long long rec_off = e.rec_begin + (c - e.chunk_begin) * (long long)k_eff;
+
+        for (int i = tid; i < e.tile >> 2; i += T) reinterpret_cast<float4 *>(tile0)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (counts)
+            for (int i = tid; i < M; i += T) Cn[i] = 0;
+        // S = sum over workers, in worker order: batches of records are staged by all threads, the first warp adds them
+        // worker after worker (indices are unique inside one worker's chunk)
+        auto add = [&](int idx, float val) {
+            if ((unsigned)idx < (unsigned)M) {
+                tile0[place_of(e, idx).t] += val;
+                if (counts) Cn[idx] += 1;
+            } else {
+                atomicMax(a.status, DEMO_DEV_PAYLOAD);
+            }
+        };
+        if (k_eff <= STAGE) {
+            const int wb = STAGE / k_eff;
+            for (int w0 = 0; w0 < a.W; w0 += wb) {
+                const int nw = min(wb, a.W - w0);
+                for (int r = tid; r < nw * k_eff; r += T) {
+                    const int w = r / k_eff;
+                    const DemoRecord rc = a.payloads[w0 + w][rec_off + (r - w * k_eff)];
+                    stage[r] = make_uint2((unsigned)rc.idx, __float_as_uint(rc.val));
+                }
+                __syncthreads();
+                if (tid < 32) {
+                    for (int w = 0; w < nw; ++w) {
+                        for (int i = tid; i < k_eff; i += 32) {
+                            const uint2 r = stage[w * k_eff + i];
+                            add((int)r.x, __uint_as_float(r.y));
+                        }
+                        __syncwarp();
+                    }
+                }
+                __syncthreads();
+            }
+        } else {
+            __syncthreads();
+            for (int w = 0; w < a.W; ++w) {
+                const DemoRecord *rec = a.payloads[w] + rec_off;
+                for (int i = tid; i < k_eff; i += T) add(rec[i].idx, rec[i].val);
+                __syncthreads();
+            }
         }
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
-            for (int i = tid; i < M; i += GEN_THREADS) {
+            for (int i = tid; i < M; i += T) {
                 const unsigned short n = Cn[i];
-                if (n > 1) St[i] = St[i] / (float)n;
+                const int t = place_of(e, i).t;
+                if (n > 1) tile0[t] = tile0[t] / (float)n;
             }
             __syncthreads();
         }
-        const float *R = transform_chunk(St, X1, St, e, a.tables, true);
-        // x <- x - lr * (phi(R) + wd * x), sign(0) = 0
-        for (int i = tid; i < M; i += GEN_THREADS) {
-            const size_t off = base + elem_offset(e, i);
-            const float rv = R[i];
-            if (a.sign_ptrs) {  // parameter-server form: hand out sign(R), the workers apply it
-                a.sign_ptrs[e.tensor][off] = (signed char)((rv > 0.f) - (rv < 0.f));
-                continue;
-            }
-            const float sg = a.phi ? rv * a.agg_scale : (float)((rv > 0.f) - (rv < 0.f));
-            const float xv = x[off];
-            x[off] = fmaf(-a.lr, fmaf(a.wd, xv, sg), xv);
+        transform_chunk<true, BIG>(tile0, tile1, slot, a.tables);
+        if (a.sign_ptrs) {  // parameter-server form: hand out sign(R), the workers apply it
+            signed char *__restrict__ sg = a.sign_ptrs[e.tensor] + base;
+            for_elements<4>(v, e, [](int, auto) {}, [&](int, int, auto off, int t) {
+                const float rv = tile0[t];
+                sg[off] = (signed char)((rv > 0.f) - (rv < 0.f));
+            });
+            continue;
         }
-        __syncthreads();
+        // x <- x - lr * (phi(R) + wd * x), sign(0) = 0
+        float *__restrict__ x = a.x_ptrs[e.tensor] + base;
+        constexpr int U = 8;
+        float xv[U];
+        for_elements<U>(
+            v, e, [&](int j, auto off) { xv[j] = x[off]; },
+            [&](int j, int, auto off, int t) {
+                const float rv = tile0[t];
+                const float sg = a.phi ? rv * a.agg_scale : (float)((rv > 0.f) - (rv < 0.f));
+                x[off] = fmaf(-a.lr, fmaf(a.wd, xv[j], sg), xv[j]);
+            });
     }
+}
+
+template <typename K>
+cudaError_t launch_nd(K kernel, size_t smem, const DemoNdClass &cls, int sm_count, cudaStream_t stream, const void *args)
+{
+    if (cls.n_chunks <= 0) return cudaSuccess;
+    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    int per_sm = 0;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, cls.threads, smem);
+    if (err != cudaSuccess) return err;
+    if (per_sm < 1) per_sm = 1;
+    long long grid = (long long)sm_count * per_sm;
+    if (grid > cls.n_chunks) grid = cls.n_chunks;
+    void *params[] = {const_cast<void *>(args)};
+    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)grid), dim3((unsigned)cls.threads), params, smem, stream);
 }
 
 }  // namespace
 
+int DemoNdTables::get(int s)
+{
+    if (of[s] >= 0) return of[s];
+    of[s] = (int)data.size();
+    const double pi = 3.141592653589793238462643383279502884;
+    const int h = (s + 1) / 2, pe = up8(h), po = up8(s / 2);
+    auto C = [&](int u, int n) {
+        if ((u & 1) && 2 * n == s - 1) return 0.0;
+        return std::sqrt((u == 0 ? 1.0 : 2.0) / s) * std::cos(pi * (2.0 * n + 1.0) * u / (2.0 * s));
+    };
+    for (int n = 0; n < h; ++n) {
+        for (int j = 0; j < pe; ++j) data.push_back(2 * j < s ? (float)(C(2 * j, n) * (2 * n == s - 1 ? 0.5 : 1.0)) : 0.f);
+        for (int j = 0; j < po; ++j) data.push_back(2 * j + 1 < s ? (float)C(2 * j + 1, n) : 0.f);
+    }
+    for (int u = 0; u < s; ++u)
+        for (int n = 0; n < pe; ++n) data.push_back(n < h ? (float)C(u, n) : 0.f);
+    return of[s];
+}
+
+// Tile strides: the innermost axis is dense, every outer stride may be padded by a few words.  The padding is the one with
+// the fewest bank conflicts of a warp's accesses over the axis passes (32 neighbouring lines at a time), the smaller tile
+// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it.
+void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
+{
+    const int *s = e->s;
+    e->tail = s[2] == s[3] && s[3] >= 2 && s[3] <= 7 ? s[3] : 0;
+    auto conflicts = [&](const int *p) {
+        long long cost = 0;
+        for (int a = 0; a < DEMO_ND_DIMS; ++a) {
+            if (s[a] == 1 || (e->tail && a == 3)) continue;
+            const int last = e->tail && a == 2 ? 3 : a;
+            const int lines = e->M / (s[a] * (last > a ? s[last] : 1));
+            for (int w = 0; w < 3 && w * 32 < lines; ++w) {  // the first, second and third warp's lines
+                int bank[32] = {0}, worst = 0;
+                for (int l = 32 * w; l < lines && l < 32 * w + 32; ++l) {
+                    int r = l, t = 0;
+                    for (int b = DEMO_ND_DIMS - 1; b >= 0; --b)
+                        if (b < a || b > last) {
+                            t += (r % s[b]) * p[b];
+                            r /= s[b];
+                        }
+                    const int v = ++bank[t & 31];
+                    worst = worst > v ? worst : v;
+                }
+                cost += worst * (last > a ? 2 : 1);
+            }
+        }
+        return cost;
+    };
+    const int room = e->M / 16 > 64 ? e->M / 16 : 64;
+    long long best = -1;
+    int p[DEMO_ND_DIMS];
+    p[3] = 1;
+    for (int pad2 = 0; pad2 <= (s[2] > 1 && !e->tail ? 8 : 0); ++pad2) {
+        p[2] = s[3] + pad2;
+        for (int pad1 = 0; pad1 <= (s[1] > 1 && s[2] * s[3] > 1 ? 8 : 0); ++pad1) {
+            p[1] = p[2] * s[2] + pad1;
+            for (int pad0 = 0; pad0 <= (s[0] > 1 && s[1] * s[2] * s[3] > 1 ? 31 : 0); ++pad0) {
+                p[0] = p[1] * s[1] + pad0;
+                const int floats = p[0] * s[0];
+                if (floats > e->M + room) break;
+                const long long cost = conflicts(p) * (1LL << 20) + floats;
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    for (int a = 0; a < DEMO_ND_DIMS; ++a) e->p[a] = p[a];
+                    e->tile = (floats + 3) & ~3;
+                }
+            }
+        }
+    }
+    // rows: the trailing elements that follow one another in the tensor and in the tile
+    long long run = 1, span = 0;
+    bool joined = true;
+    for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
+        if (joined && (s[a] == 1 || (e->stride[a] == run && e->p[a] == run)))
+            run *= s[a];
+        else
+            joined = joined && s[a] == 1;
+        span += (s[a] - 1) * e->stride[a];
+    }
+    e->row = (int)run;
+    e->inv_row = run > 1 ? (unsigned)(((1ULL << 32) + (unsigned long long)run - 1) / (unsigned long long)run) : 0u;
+    e->row_table = e->M / run <= DEMO_ND_MAX_ROWS && span < (1LL << 32);
+    // threads: enough for every pass over the long axes in whole rounds, and for 32 elements each
+    int threads = (e->M + 31) / 32;
+    for (int a = 0; a < DEMO_ND_DIMS; ++a) {
+        if (!in_place_extent(s[a])) e->basis[a] = tables->get(s[a]);
+        if (s[a] <= 8) continue;
+        int n = e->M / s[a];
+        if (s[a] == 64 || s[a] == 128) n = (n + 31) / 32 * 64;
+        if (!in_place_extent(s[a])) n = n * (up8((s[a] + 1) / 2) + up8(s[a] / 2)) / 8 / 2;
+        const int rounds = (n + MAX_THREADS - 1) / MAX_THREADS;
+        n = (n + rounds - 1) / rounds;
+        threads = threads > n ? threads : n;
+    }
+    threads = (threads + 31) / 32 * 32;
+    e->threads = threads > MAX_THREADS ? MAX_THREADS : threads;
+}
+
+// A class is a size bucket with or without extents of 128 (registers) and with or without dense axes (shared memory), so
+// that a few chunks of one kind do not set the resources of all others.  Classes that would not fill the device (fewer than
+// two chunks per SM) are merged, with one another and, where it has all that they need, with the largest of the others:
+// a launch of its own costs more than the wider variant.
+void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vector<DemoNdClass> *classes)
+{
+    struct Group {
+        std::vector<DemoNdEntry> list;
+        long long chunks = 0, elems = 0;
+        DemoNdClass k{};
+        void widen(const DemoNdClass &o)
+        {
+            k.max_M = k.max_M > o.max_M ? k.max_M : o.max_M;
+            k.tile = k.tile > o.tile ? k.tile : o.tile;
+            k.rows = k.rows > o.rows ? k.rows : o.rows;
+            k.dense_axes |= o.dense_axes;
+            k.big |= o.big;
+        }
+        void take(Group &o)
+        {
+            if (o.list.empty()) return;
+            list.insert(list.end(), o.list.begin(), o.list.end());
+            if (o.elems > elems) k.threads = o.k.threads;  // the CTA size of the larger
+            chunks += o.chunks;
+            elems += o.elems;
+            widen(o.k);
+            o = Group();
+        }
+    };
+    Group g[16], rest;
+    for (const DemoNdEntry &e : entries) {
+        Group one;
+        one.list.push_back(e);
+        one.chunks = e.chunk_end;
+        one.elems = e.chunk_end * e.M;
+        one.k.threads = e.threads;
+        one.k.max_M = (e.M + 3) & ~3;
+        one.k.tile = e.tile;
+        one.k.rows = e.row_table ? e.M / e.row : 0;
+        for (int s : e.s) {
+            one.k.big |= s == 128;
+            one.k.dense_axes |= !in_place_extent(s);
+        }
+        const int bucket = e.M <= 512 ? 0 : e.M <= 2048 ? 1 : e.M <= 4096 ? 2 : 3;
+        g[bucket * 4 + one.k.big * 2 + one.k.dense_axes].take(one);
+    }
+    Group *largest = nullptr;
+    for (Group &d : g) {
+        if (d.list.empty()) continue;
+        if (d.chunks < 2LL * sm_count)
+            rest.take(d);
+        else if (!largest || d.elems > largest->elems)
+            largest = &d;
+    }
+    if (largest && largest->k.max_M >= rest.k.max_M && largest->k.tile >= rest.k.tile && largest->k.big >= rest.k.big &&
+        largest->k.dense_axes >= rest.k.dense_axes)
+        largest->take(rest);
+    entries.clear();
+    classes->clear();
+    auto same_layout = [](const DemoNdEntry &x, const DemoNdEntry &y) {
+        for (int a = 0; a < DEMO_ND_DIMS; ++a)
+            if (x.s[a] != y.s[a] || x.stride[a] != y.stride[a]) return false;  // (the tile follows from these)
+        return true;
+    };
+    auto emit = [&](Group &d) {
+        if (d.list.empty()) return;
+        DemoNdClass k = d.k;
+        k.first = (int)entries.size();
+        k.n = (int)d.list.size();
+        k.n_chunks = 0;
+        bool split = false;
+        for (DemoNdEntry e : d.list) {
+            const long long n = e.chunk_end;
+            e.chunk_begin = k.n_chunks;
+            k.n_chunks += n;
+            e.chunk_end = k.n_chunks;
+            for (int s : e.s) split = split || s == 64 || s == 128;
+            e.layout = k.n_chunks > n && same_layout(entries.back(), e) ? entries.back().layout : (int)entries.size();
+            entries.push_back(e);
+        }
+        if (split) k.threads = (k.threads + 63) / 64 * 64;  // two warps per 32 lines
+        if (k.big && k.threads > MAX_THREADS_BIG) k.threads = MAX_THREADS_BIG;
+        classes->push_back(k);
+    };
+    for (Group &d : g) emit(d);
+    emit(rest);
+}
+
 cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, cudaStream_t stream)
 {
-    const size_t smem = 3 * (size_t)a.max_M * sizeof(float) + (256 + 8 + 2) * sizeof(unsigned);
-    return launch_persistent(compress_nd_kernel, smem, a.n_chunks, sm_count, stream, &a);
+    const size_t smem = shared_bytes(a.cls, true);
+    if (a.cls.big)
+        return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, true>, smem, a.cls, sm_count, stream, &a)
+                           : launch_nd(compress_nd_kernel<float, true>, smem, a.cls, sm_count, stream, &a);
+    return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, false>, smem, a.cls, sm_count, stream, &a)
+                       : launch_nd(compress_nd_kernel<float, false>, smem, a.cls, sm_count, stream, &a);
 }
 
 cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
-    const size_t smem = 2 * (size_t)a.max_M * sizeof(float) + (((size_t)a.max_M * 2 + 15) & ~(size_t)15);
-    return launch_persistent(decode_nd_kernel, smem, a.n_chunks, sm_count, stream, &a);
+    const size_t smem = shared_bytes(a.cls, false) + (a.agg == 2 ? align16((size_t)a.cls.max_M * 2) : 0);
+    return a.cls.big ? launch_nd(decode_nd_kernel<true>, smem, a.cls, sm_count, stream, &a)
+                     : launch_nd(decode_nd_kernel<false>, smem, a.cls, sm_count, stream, &a);
 }

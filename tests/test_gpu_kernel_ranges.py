@@ -1,9 +1,10 @@
 """Edges of the size ranges the kernel variants are chosen by, against the fp64 oracle (rules and tolerances of
 tests/parity.py, every chunk)."""
+import types
+
 import pytest
 import torch
 
-import paper_2411_19870_b200 as demo
 from paper_2411_19870_b200 import inputs
 from tests import parity
 
@@ -25,4 +26,35 @@ def test_s64_list_and_dense_row_stage(k, kind):
             g[0][64:128, :64] = 0
             g[0][70, 5] = 0.5
         r.step(grads=grads)
+    r.close()
+
+
+@pytest.mark.parametrize("shapes,chunks,k", [
+    ([(64, 32, 7, 7), (32,)], [(32, 4, 7, 7), (32,)], 40),         # kernel windows of 7 x 7; a lossless vector
+    ([(32, 16, 2, 2), (24, 4, 6, 6)], [(16, 16, 2, 2), (8, 4, 6, 6)], 17),
+    ([(32, 48, 3)], [(32, 48, 1)], 33),                            # 1536 rows of one element: no row table
+    ([(128, 64), (64, 384)], [(64, 32), (32, 128)], 64),           # two threads per line; two classes in one context
+    ([(58, 128), (62, 93)], [(29, 64), (31, 31)], 32),             # odd dense extents, one and two lines per thread
+    ([(127, 127)], [(127, 127)], 300),                             # the largest dense chunk: both tiles and B fill the SM
+    ([(64, 96)], [(16, 32)], 400),                                 # k close to the chunk: the list overflows
+])
+def test_nd_extents(shapes, chunks, k):
+    r = parity.NdRunner(shapes, chunks, topk=k, num_workers=2, grad_std=0.02)
+    for _ in range(2):
+        r.step()
+    r.close()
+
+
+def test_nd_ties_and_untouched_chunks():
+    """Equal magnitudes straddling the k-th place inside the candidate list (a few equal coefficients) and beyond it
+    (+-a everywhere), a constant chunk, an all-zero chunk."""
+    r = parity.NdRunner([(64, 48)], [(32, 24)], topk=20, num_workers=1, grad_dtype=torch.float32)
+    g = torch.zeros(64, 48, device="cuda")
+    g[:32, 24:] = 0.25
+    sign = torch.where(torch.rand(32, 24, device="cuda", generator=torch.Generator("cuda").manual_seed(3)) < 0.5, -1.0, 1.0)
+    g[32:, :24] = 0.125 * sign
+    g[32, 24] = 1.0
+    r.inputs = types.SimpleNamespace(random_tensor=lambda *a: g)  # the gradient of every step
+    for _ in range(2):
+        r.step()
     r.close()
