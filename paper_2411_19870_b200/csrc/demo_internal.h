@@ -29,7 +29,7 @@ struct DemoCompressArgs {
     const DemoTensorEntry *entries;  // device
     int n_entries;
     long long n_chunks;
-    int k;                      // k_eff of the list's tensors (one chunk size per list, so one k_eff)
+    int k;                      // k_eff of the list's tensors (all of one kind and chunk size)
     const void *const *g_ptrs;  // device array indexed by DemoTensorEntry::tensor
     float *const *m_ptrs;       // device array
     DemoRecord *payload;        // device, whole payload of this worker
@@ -67,12 +67,17 @@ struct DemoDecodeArgs {
     signed char *const *sign_ptrs = nullptr;
 };
 
-// Launchers (defined in the kernel translation units).  `s` is the chunk size, `two_d` selects
-// s x s tiles (1) or length-s segments (0).  Return the CUDA error of the launch.
-cudaError_t demo_launch_compress_generic(int s, int two_d, const DemoCompressArgs &a, int sm_count,
-                                         cudaStream_t stream);
-cudaError_t demo_launch_decode_generic(int s, int two_d, const DemoDecodeArgs &a, int sm_count,
+// Launchers (defined in the kernel translation units).  `s` is the chunk size.  Return the CUDA error of the launch.
+// Dense transforms of s x s tiles, any basis (kernels_generic.cu).
+cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
+// Segments of 1-D tensors (any s, any basis) and, where `demo_small_tiles_supported` and the basis is the DCT, s x s tiles, in
+// one launch (kernels_small.cu).  Either list may be NULL.
+bool demo_small_tiles_supported(int s);
+cudaError_t demo_launch_compress_small(int s, const DemoCompressArgs *segs, const DemoCompressArgs *tiles, int sm_count,
                                        cudaStream_t stream);
+cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count,
+                                     cudaStream_t stream);
 // Fast-DCT kernels for 2-D tensors; `supported` tells whether chunk size s has one.
 bool demo_fast_supported(int s);
 cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, int sm_count, cudaStream_t stream);

@@ -562,6 +562,11 @@ static bool use_fast_path(const demo_ctx *ctx)
     return ctx->path == DEMO_PATH_AUTO && !ctx->custom_basis && demo_fast_supported(s) && (s != 128 || ctx->encode);
 }
 
+static bool use_small_tiles(const demo_ctx *ctx)
+{
+    return ctx->path == DEMO_PATH_AUTO && !ctx->custom_basis && demo_small_tiles_supported(ctx->cfg.chunk);
+}
+
 // A caller-supplied basis has no fast factorisation: its dense transforms run on the tensor cores where
 // there is a kernel for the chunk size, else on the CUDA cores.
 static bool use_tc_path(const demo_ctx *ctx)
@@ -642,29 +647,31 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
     a.tmap_m = ctx->encode ? ctx->d_tm_m + row : nullptr;
     a.tmap_g = ctx->encode ? ctx->d_tm_g + row : nullptr;
     const int s = ctx->cfg.chunk;
+    DemoCompressArgs a1 = a;  // the 1-D tensors
+    a1.entries = ctx->d_entries1d;
+    a1.n_entries = ctx->n1d;
+    a1.n_chunks = ctx->chunks1d;
+    a1.k = ctx->cfg.topk < s ? ctx->cfg.topk : s;
+    a1.momentum_dct = 0;  // they keep the momentum itself
+    a.entries = ctx->d_entries2d;
+    a.n_entries = ctx->n2d;
+    a.n_chunks = ctx->chunks2d;
+    a.k = ctx->cfg.topk;  // <= s * s
+    a.momentum_dct = ctx->momentum_dct ? 1 : 0;
+    const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     cudaStream_t side = stream;
-    if (ctx->n1d) {
-        side = fork_side(ctx, stream);
-        a.momentum_dct = 0;  // 1-D tensors keep the momentum itself
-        a.entries = ctx->d_entries1d;
-        a.n_entries = ctx->n1d;
-        a.n_chunks = ctx->chunks1d;
-        a.k = ctx->cfg.topk < s ? ctx->cfg.topk : s;
-        err = demo_launch_compress_generic(s, 0, a, ctx->sm_count, side);
+    if (ctx->n1d || small_tiles) {
+        if (!small_tiles) side = fork_side(ctx, stream);
+        err = demo_launch_compress_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, side);
         ctx->launches += 1;
     }
-    if (err == cudaSuccess && ctx->n2d) {
-        a.entries = ctx->d_entries2d;
-        a.n_entries = ctx->n2d;
-        a.n_chunks = ctx->chunks2d;
-        a.k = ctx->cfg.topk;  // <= s * s
-        a.momentum_dct = ctx->momentum_dct ? 1 : 0;
+    if (err == cudaSuccess && ctx->n2d && !small_tiles) {
         if (use_fast_path(ctx))
             err = demo_launch_compress_fast(s, a, ctx->sm_count, stream);
         else if (use_tc_path(ctx))
             err = demo_launch_compress_tc(a, ctx->sm_count, stream);
         else
-            err = demo_launch_compress_generic(s, 1, a, ctx->sm_count, stream);
+            err = demo_launch_compress_generic(s, a, ctx->sm_count, stream);
         ctx->launches += 1;
     }
     {
@@ -801,26 +808,28 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.agg_scale = (ctx->aggregation == DEMO_AGG_MEAN) ? 1.0f / (float)W : 1.0f;
     a.sign_ptrs = signs ? ctx->d_s : nullptr;
     const int s = ctx->cfg.chunk;
+    DemoDecodeArgs a1 = a;  // the 1-D tensors
+    a1.entries = ctx->d_entries1d;
+    a1.n_entries = ctx->n1d;
+    a1.n_chunks = ctx->chunks1d;
+    a.entries = ctx->d_entries2d;
+    a.n_entries = ctx->n2d;
+    a.n_chunks = ctx->chunks2d;
+    const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     cudaStream_t side = stream;
-    if (ctx->n1d) {
-        side = fork_side(ctx, stream);
-        a.entries = ctx->d_entries1d;
-        a.n_entries = ctx->n1d;
-        a.n_chunks = ctx->chunks1d;
-        err = demo_launch_decode_generic(s, 0, a, ctx->sm_count, side);
+    if (ctx->n1d || small_tiles) {
+        if (!small_tiles) side = fork_side(ctx, stream);
+        err = demo_launch_decode_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, side);
         ctx->launches += 1;
     }
-    if (err == cudaSuccess && ctx->n2d) {
-        a.entries = ctx->d_entries2d;
-        a.n_entries = ctx->n2d;
-        a.n_chunks = ctx->chunks2d;
+    if (err == cudaSuccess && ctx->n2d && !small_tiles) {
         // (a caller-supplied basis: the signs come from the dense kernels, there is no tensor-core variant)
         if (use_fast_path(ctx))
             err = demo_launch_decode_fast(s, a, ctx->sm_count, stream);
         else if (use_tc_path(ctx) && !signs)
             err = demo_launch_decode_tc(a, ctx->sm_count, stream);
         else
-            err = demo_launch_decode_generic(s, 1, a, ctx->sm_count, stream);
+            err = demo_launch_decode_generic(s, a, ctx->sm_count, stream);
         ctx->launches += 1;
     }
     {

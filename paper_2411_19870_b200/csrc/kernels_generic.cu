@@ -1,10 +1,10 @@
-// Generic kernels of the DeMo optimizer transform: any chunk size s in {8,16,32,64,128}, 2-D tiles
-// and 1-D segments, any k <= M.  One CTA works on one chunk at a time; the chunk stays in shared
+// Generic kernels of the DeMo optimizer transform: s x s tiles of any chunk size s in {8,16,32,64,128}, any basis,
+// any k <= M.  One CTA works on one chunk at a time; the chunk stays in shared
 // memory from the momentum update to the residual write-back, so HBM is touched once per operand.
 // The chunk DCT here is the dense contraction with the precomputed basis (the paper's own cost
-// model, Section 2.1 "Complexity Analysis"); the register-resident fast-DCT kernels for the common
-// sizes live in kernels_fast.cu.  These kernels are the path for 1-D tensors, for s in {8,16,128}
-// and the cross-check of the fast path.
+// model, Section 2.1 "Complexity Analysis"); the register-resident fast-DCT kernels live in kernels_fast*.cu and
+// kernels_small.cu.  These kernels are the path for caller-supplied bases where there is no tensor-core kernel and the
+// cross-check of the fast path (DEMO_PATH_GENERIC).
 #include <cuda_bf16.h>
 
 #include "demo_internal.h"
@@ -47,38 +47,30 @@ __device__ __forceinline__ void mm(float *__restrict__ out, const float *__restr
     }
 }
 
-// Forward chunk DCT: 2-D  Q = C B C^T,  1-D  q = C b.  Result in `q_out`, `tmp` is scratch.
-template <int S, int ROWS>
+// Forward chunk transform  Q = C B C^T.  Result in `q_out`, `tmp` is scratch.
+template <int S>
 __device__ __forceinline__ void forward_dct(const float *Bt, float *tmp, float *q_out, const float *C)
 {
-    if (ROWS > 1) {
-        mm<ROWS, S, S>(tmp, Bt, S, 1, C, 1, S);  // tmp[i][v] = sum_j B[i][j] C[v][j]
-        __syncthreads();
-        mm<S, S, S>(q_out, C, S, 1, tmp, S, 1);  // Q[u][v] = sum_i C[u][i] tmp[i][v]
-    } else {
-        mm<ROWS, S, S>(q_out, Bt, S, 1, C, 1, S);
-    }
+    mm<S, S, S>(tmp, Bt, S, 1, C, 1, S);  // tmp[i][v] = sum_j B[i][j] C[v][j]
+    __syncthreads();
+    mm<S, S, S>(q_out, C, S, 1, tmp, S, 1);  // Q[u][v] = sum_i C[u][i] tmp[i][v]
     __syncthreads();
 }
 
-// Inverse chunk DCT: 2-D  R = C^T Q C,  1-D  r = C^T q.  Result in `r_out`, `tmp` is scratch.
-template <int S, int ROWS>
+// Inverse chunk transform  R = C^T Q C.  Result in `r_out`, `tmp` is scratch.
+template <int S>
 __device__ __forceinline__ void inverse_dct(const float *Qt, float *tmp, float *r_out, const float *C)
 {
-    if (ROWS > 1) {
-        mm<ROWS, S, S>(tmp, Qt, S, 1, C, S, 1);   // tmp[u][j] = sum_v Q[u][v] C[v][j]
-        __syncthreads();
-        mm<S, S, S>(r_out, C, 1, S, tmp, S, 1);   // R[i][j] = sum_u C[u][i] tmp[u][j]
-    } else {
-        mm<ROWS, S, S>(r_out, Qt, S, 1, C, S, 1);
-    }
+    mm<S, S, S>(tmp, Qt, S, 1, C, S, 1);   // tmp[u][j] = sum_v Q[u][v] C[v][j]
+    __syncthreads();
+    mm<S, S, S>(r_out, C, 1, S, tmp, S, 1);   // R[i][j] = sum_u C[u][i] tmp[u][j]
     __syncthreads();
 }
 
-template <int S, int ROWS>
+template <int S>
 __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompressArgs a)
 {
-    constexpr int M = ROWS * S;
+    constexpr int M = S * S;
     extern __shared__ float smem[];
     float *Bt = smem;
     float *X1 = Bt + M;
@@ -93,7 +85,7 @@ __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompr
         const long long lc = c - te.chunk_begin;
         const long long k0 = lc / te.c1;
         const int k1 = (int)(lc - k0 * te.c1);
-        const size_t base = (size_t)k0 * ROWS * (size_t)te.n1 + (size_t)k1 * S;
+        const size_t base = (size_t)k0 * S * (size_t)te.n1 + (size_t)k1 * S;
         float *__restrict__ m = a.m_ptrs[te.tensor];
         const void *g = a.g_ptrs[te.tensor];
         const int k_eff = te.k_eff;
@@ -108,9 +100,9 @@ __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompr
         }
         __syncthreads();
 
-        float *Q = (ROWS > 1) ? X2 : X1;   // coefficients
-        float *O = (ROWS > 1) ? X1 : X2;   // the other buffer
-        forward_dct<S, ROWS>(Bt, X1, Q, a.C);
+        float *Q = X2;  // coefficients
+        float *O = X1;  // the other buffer
+        forward_dct<S>(Bt, X1, Q, a.C);
 
         // top-k: threshold by radix select, then index-ordered compaction into the payload
         unsigned thr, need_eq;
@@ -161,8 +153,8 @@ __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompr
         __syncthreads();
 
         // momentum subtraction  m <- B - IDCT(kept coefficients)
-        float *R = (ROWS > 1) ? O : Q;
-        inverse_dct<S, ROWS>(O, Q, R, a.C);
+        float *R = O;
+        inverse_dct<S>(O, Q, R, a.C);
         for (int i = tid; i < M; i += GEN_THREADS) {
             const int r = i / S, j = i - r * S;
             m[base + (size_t)r * te.n1 + j] = Bt[i] - R[i];
@@ -171,10 +163,10 @@ __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompr
     }
 }
 
-template <int S, int ROWS>
+template <int S>
 __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeArgs a)
 {
-    constexpr int M = ROWS * S;
+    constexpr int M = S * S;
     extern __shared__ float smem[];
     float *St = smem;
     float *X1 = St + M;
@@ -187,7 +179,7 @@ __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeA
         const long long lc = c - te.chunk_begin;
         const long long k0 = lc / te.c1;
         const int k1 = (int)(lc - k0 * te.c1);
-        const size_t base = (size_t)k0 * ROWS * (size_t)te.n1 + (size_t)k1 * S;
+        const size_t base = (size_t)k0 * S * (size_t)te.n1 + (size_t)k1 * S;
         float *__restrict__ x = a.x_ptrs[te.tensor];
         const int k_eff = te.k_eff;
         const long long rec_off = te.rec_begin + lc * (long long)k_eff;
@@ -219,8 +211,8 @@ __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeA
             }
             __syncthreads();
         }
-        float *R = (ROWS > 1) ? St : X1;
-        inverse_dct<S, ROWS>(St, X1, R, a.C);
+        float *R = St;
+        inverse_dct<S>(St, X1, R, a.C);
         // x <- x - lr * (sign(R) + wd * x), sign(0) = 0
         for (int i = tid; i < M; i += GEN_THREADS) {
             const int r = i / S, j = i - r * S;
@@ -274,36 +266,29 @@ __global__ void __launch_bounds__(GEN_THREADS) apply_signs_kernel(DemoApplySigns
 }
 
 template <int S>
-cudaError_t compress_dispatch(int two_d, const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t compress_dispatch(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
 {
     const size_t extra = (256 + 8 + 2) * sizeof(unsigned);
-    if (two_d)
-        return launch_persistent(compress_generic_kernel<S, S>, 3 * S * S * sizeof(float) + extra, a.n_chunks,
-                                 sm_count, stream, &a);
-    return launch_persistent(compress_generic_kernel<S, 1>, 3 * S * sizeof(float) + extra, a.n_chunks, sm_count,
-                             stream, &a);
+    return launch_persistent(compress_generic_kernel<S>, 3 * S * S * sizeof(float) + extra, a.n_chunks, sm_count, stream, &a);
 }
 
 template <int S>
-cudaError_t decode_dispatch(int two_d, const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t decode_dispatch(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
-    if (two_d)
-        return launch_persistent(decode_generic_kernel<S, S>, 2 * S * S * sizeof(float) + S * S * 2, a.n_chunks, sm_count,
-                                 stream, &a);
-    return launch_persistent(decode_generic_kernel<S, 1>, 2 * S * sizeof(float) + S * 2, a.n_chunks, sm_count, stream, &a);
+    return launch_persistent(decode_generic_kernel<S>, 2 * S * S * sizeof(float) + S * S * 2, a.n_chunks, sm_count, stream, &a);
 }
 
 }  // namespace
 
-cudaError_t demo_launch_compress_generic(int s, int two_d, const DemoCompressArgs &a, int sm_count,
+cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, int sm_count,
                                          cudaStream_t stream)
 {
     switch (s) {
-        case 8: return compress_dispatch<8>(two_d, a, sm_count, stream);
-        case 16: return compress_dispatch<16>(two_d, a, sm_count, stream);
-        case 32: return compress_dispatch<32>(two_d, a, sm_count, stream);
-        case 64: return compress_dispatch<64>(two_d, a, sm_count, stream);
-        case 128: return compress_dispatch<128>(two_d, a, sm_count, stream);
+        case 8: return compress_dispatch<8>(a, sm_count, stream);
+        case 16: return compress_dispatch<16>(a, sm_count, stream);
+        case 32: return compress_dispatch<32>(a, sm_count, stream);
+        case 64: return compress_dispatch<64>(a, sm_count, stream);
+        case 128: return compress_dispatch<128>(a, sm_count, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -318,15 +303,15 @@ cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, c
     return cudaGetLastError();
 }
 
-cudaError_t demo_launch_decode_generic(int s, int two_d, const DemoDecodeArgs &a, int sm_count,
+cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, int sm_count,
                                        cudaStream_t stream)
 {
     switch (s) {
-        case 8: return decode_dispatch<8>(two_d, a, sm_count, stream);
-        case 16: return decode_dispatch<16>(two_d, a, sm_count, stream);
-        case 32: return decode_dispatch<32>(two_d, a, sm_count, stream);
-        case 64: return decode_dispatch<64>(two_d, a, sm_count, stream);
-        case 128: return decode_dispatch<128>(two_d, a, sm_count, stream);
+        case 8: return decode_dispatch<8>(a, sm_count, stream);
+        case 16: return decode_dispatch<16>(a, sm_count, stream);
+        case 32: return decode_dispatch<32>(a, sm_count, stream);
+        case 64: return decode_dispatch<64>(a, sm_count, stream);
+        case 128: return decode_dispatch<128>(a, sm_count, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -590,13 +575,13 @@ extern "C" demo_status demo_decode_apply_static(const demo_config *cfg, const de
             a.entries = reinterpret_cast<const DemoTensorEntry *>(base + OFF_ENTRIES);
             a.n_entries = n2d;
             a.n_chunks = chunks2d;
-            err = demo_launch_decode_generic(s, 1, a, sm_count, stream);
+            err = demo_launch_decode_generic(s, a, sm_count, stream);
         }
         if (err == cudaSuccess && n1d) {
             a.entries = reinterpret_cast<const DemoTensorEntry *>(base + OFF_ENTRIES) + n2d;
             a.n_entries = n1d;
             a.n_chunks = chunks1d;
-            err = demo_launch_decode_generic(s, 0, a, sm_count, stream);
+            err = demo_launch_decode_small(s, &a, nullptr, sm_count, stream);
         }
         if (err != cudaSuccess) {
             cudaGetLastError();

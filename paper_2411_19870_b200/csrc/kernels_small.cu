@@ -1,0 +1,578 @@
+// Kernels for the small chunks: length-s segments of 1-D tensors (any s and basis; one warp per segment) and s x s tiles with
+// s in {8, 16} (s lanes per tile, 4 or 2 tiles per warp).  A launch takes both lists: the tensors of a small model are done in
+// one launch per call, and the norm vectors of a large one beside its tiles.
+//
+// What bounds them is latency: a chunk holds 8 to 256 elements, so nothing is gained by more threads per chunk (the dense
+// kernels, a 256-thread CTA per chunk with radix select and a barrier between all steps, spent 24 us on 2048 tiles of 8 x 8
+// and 13 us on 1024 segments), and a warp needs no block barrier from the loads to the stores:
+//   * segments: every lane forms s/32 coefficients by reading rows of the basis through L1 (the sums run over n in order, so
+//     the results are those of the dense kernels bit for bit); keys in registers, the k-th by a bit-by-bit ballot search;
+//   * tiles: lane j holds column j, then row j, in registers (fast_dct.cuh); the transposes go through a tile of the
+//     warp's own shared memory; the k-th key by a bit-by-bit search with counts added up over the tile's lanes.
+// Measured: 256 x 512 in 8 x 8 tiles plus a vector of 512, two compress calls and a decode: 60.7 -> 30.4 us (the tiles and
+// the segments of a call were two launches on two streams).
+#include <cuda_bf16.h>
+
+#include <type_traits>
+
+#include "demo_internal.h"
+#include "fast_dct.cuh"
+
+namespace {
+
+constexpr int THREADS = 128, WARPS = THREADS / 32;
+constexpr unsigned FULL = 0xffffffffu;
+
+__device__ __forceinline__ unsigned mag_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+
+// (warp) the tensor that owns chunk id c: the last entry with chunk_begin <= c.
+__device__ __forceinline__ int find_entry_warp(const DemoTensorEntry *entries, int n, long long c)
+{
+    const int lane = threadIdx.x & 31;
+    int count = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const bool below = i0 + lane < n && entries[i0 + lane].chunk_begin <= c;
+        const int b = __popc(__ballot_sync(FULL, below));
+        count += b;
+        if (b < 32) break;  // (chunk_begin ascends)
+    }
+    return count - 1;
+}
+
+// ---- segments -------------------------------------------------------------------------------------------
+// Lane l holds elements l, l + 32, ... (E = s/32 of them, one for s < 32, where the upper lanes idle).
+template <int S>
+struct Seg {
+    static constexpr int E = S < 32 ? 1 : S / 32;
+    static constexpr int PAD = S + 4;
+};
+
+// r[n] = sum_u C[u][n] line[u], u in order.
+template <int S>
+__device__ __forceinline__ void inverse_segment(const float *line, const float *__restrict__ C, float (&r)[Seg<S>::E], int lane)
+{
+    constexpr int E = Seg<S>::E;
+#pragma unroll
+    for (int e = 0; e < E; ++e) r[e] = 0.f;
+    if (lane >= S) return;
+#pragma unroll 8
+    for (int u = 0; u < S; ++u) {
+        const float q = line[u];
+#pragma unroll
+        for (int e = 0; e < E; ++e) r[e] = fmaf(q, __ldg(C + u * S + lane + 32 * e), r[e]);
+    }
+}
+
+template <int S>
+__device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long long c, float *line)
+{
+    constexpr int E = Seg<S>::E;
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < S;
+    const DemoTensorEntry te = a.entries[find_entry_warp(a.entries, a.n_entries, c)];
+    const long long lc = c - te.chunk_begin;
+    const size_t base = (size_t)lc * S + lane;
+    float *__restrict__ m = a.m_ptrs[te.tensor];
+    const void *g = a.g_ptrs[te.tensor];
+    const int k = te.k_eff;
+
+    // momentum update  b = beta*m + g  (Algorithm 1, worker side)
+    float b[E], q[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        b[e] = 0.f;
+        if (on) {
+            const size_t off = base + 32 * e;
+            const float gv = a.grad_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(g)[off])
+                                         : static_cast<const float *>(g)[off];
+            b[e] = fmaf(a.beta, m[off], gv);
+            line[lane + 32 * e] = b[e];
+        }
+        q[e] = 0.f;
+    }
+    __syncwarp();
+    // q = C b
+    if (on) {
+#pragma unroll 4
+        for (int n = 0; n < S; n += 4) {
+            const float4 x = *reinterpret_cast<const float4 *>(line + n);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const float4 t = __ldg(reinterpret_cast<const float4 *>(a.C + (lane + 32 * e) * S + n));
+                q[e] = fmaf(x.x, t.x, q[e]);
+                q[e] = fmaf(x.y, t.y, q[e]);
+                q[e] = fmaf(x.z, t.z, q[e]);
+                q[e] = fmaf(x.w, t.w, q[e]);
+            }
+        }
+    }
+    __syncwarp();
+    // exact top-k: threshold by ballots from the highest bit any key has; keys equal to it are kept in index order
+    unsigned key[E], hi = 0u;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        key[e] = on ? mag_key(q[e]) : 0u;
+        hi = max(hi, key[e]);
+    }
+    unsigned thr = 0u;
+    int need_eq = S;  // k = s: everything is kept
+    if (k < S) {
+        hi = __reduce_max_sync(FULL, hi);
+        int n_ge = S;
+#pragma unroll 1
+        for (int bit = 31 - __clz(hi | 1u); bit >= 0 && n_ge != k; --bit) {
+            const unsigned cand = thr | (1u << bit);
+            int cnt = 0;
+#pragma unroll
+            for (int e = 0; e < E; ++e) cnt += __popc(__ballot_sync(FULL, key[e] >= cand));
+            if (cnt >= k) {
+                thr = cand;
+                n_ge = cnt;
+            }
+        }
+        int n_gt = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) n_gt += __popc(__ballot_sync(FULL, key[e] > thr));
+        need_eq = k - n_gt;
+    }
+    DemoRecord *rec = a.payload + te.rec_begin + lc * (long long)k;
+    const unsigned lt = (1u << lane) - 1u;
+    int gt_before = 0, eq_before = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const unsigned gtb = __ballot_sync(FULL, on && key[e] > thr), eqb = __ballot_sync(FULL, on && key[e] == thr);
+        const int eq = eq_before + __popc(eqb & lt);
+        const bool keep = on && (key[e] > thr || (key[e] == thr && eq < need_eq));
+        if (keep) {
+            DemoRecord r;
+            r.idx = lane + 32 * e;
+            r.val = q[e];
+            rec[gt_before + __popc(gtb & lt) + min(eq, need_eq)] = r;
+        }
+        if (on) line[lane + 32 * e] = keep ? a.alpha * q[e] : 0.f;
+        gt_before += __popc(gtb);
+        eq_before += __popc(eqb);
+    }
+    __syncwarp();
+    // m <- b - alpha C^T (kept)
+    float r[E];
+    inverse_segment<S>(line, a.C, r, lane);
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (on) m[base + 32 * e] = b[e] - r[e];
+    __syncwarp();
+}
+
+template <int S>
+__device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long long c, float *line, unsigned short *senders)
+{
+    constexpr int E = Seg<S>::E;
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < S, counts = a.agg == 2;
+    const DemoTensorEntry te = a.entries[find_entry_warp(a.entries, a.n_entries, c)];
+    const long long lc = c - te.chunk_begin;
+    const size_t base = (size_t)lc * S + lane;
+    const int k = te.k_eff;
+    const long long rec_off = te.rec_begin + lc * (long long)k;
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (on) {
+            line[lane + 32 * e] = 0.f;
+            if (counts) senders[lane + 32 * e] = 0;
+        }
+    __syncwarp();
+    // sum over workers in worker order; eight records per lane are fetched together
+    constexpr int WB = 8 / E;
+    for (int w0 = 0; w0 < a.W; w0 += WB) {
+        DemoRecord rc[WB][E];
+#pragma unroll
+        for (int w = 0; w < WB; ++w)
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                rc[w][e] = (lane + 32 * e < k && w0 + w < a.W) ? a.payloads[w0 + w][rec_off + lane + 32 * e] : DemoRecord{-1, 0.f};
+#pragma unroll
+        for (int w = 0; w < WB; ++w) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (lane + 32 * e < k && w0 + w < a.W) {
+                    if ((unsigned)rc[w][e].idx < (unsigned)S) {
+                        line[rc[w][e].idx] += rc[w][e].val;
+                        if (counts) senders[rc[w][e].idx] += 1;
+                    } else {
+                        atomicMax(a.status, DEMO_DEV_PAYLOAD);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (on) {
+                const unsigned short n = senders[lane + 32 * e];
+                if (n > 1) line[lane + 32 * e] = line[lane + 32 * e] / (float)n;
+            }
+        __syncwarp();
+    }
+    float r[E];
+    inverse_segment<S>(line, a.C, r, lane);
+    if (on) {
+        if (a.sign_ptrs) {
+            signed char *__restrict__ sg = a.sign_ptrs[te.tensor];
+#pragma unroll
+            for (int e = 0; e < E; ++e) sg[base + 32 * e] = (signed char)((r[e] > 0.f) - (r[e] < 0.f));
+        } else {
+            float *__restrict__ x = a.x_ptrs[te.tensor];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const float sg = a.phi ? r[e] * a.agg_scale : (float)((r[e] > 0.f) - (r[e] < 0.f));
+                const float xv = x[base + 32 * e];
+                x[base + 32 * e] = fmaf(-a.lr, fmaf(a.wd, xv, sg), xv);
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// ---- tiles of 8 x 8 and 16 x 16 ----------------------------------------------------------------------------
+template <int S>
+struct Tile {
+    static constexpr int PER_WARP = 32 / S;
+    static constexpr int XS = S + 1;  // row stride: a lane walks a row or a column without bank conflicts among its tile
+    static constexpr int FLOATS = PER_WARP * S * XS + 32;  // tiles of a warp start a bank apart
+};
+template <int S>
+__device__ __forceinline__ int segment_sum(int v)
+{
+#pragma unroll
+    for (int d = 1; d < S; d <<= 1) v += __shfl_xor_sync(FULL, v, d);
+    return v;
+}
+// Exclusive prefix sum over the lanes of a tile.
+template <int S>
+__device__ __forceinline__ int segment_before(int v, int j)
+{
+    int inc = v;
+#pragma unroll
+    for (int d = 1; d < S; d <<= 1) {
+        const int n = __shfl_up_sync(FULL, inc, d, S);
+        if (j >= d) inc += n;
+    }
+    return inc - v;
+}
+template <int S>
+struct TileRef {
+    DemoTensorEntry te;
+    long long lc;
+    size_t base;  // of this lane's column
+};
+template <int S>
+__device__ __forceinline__ TileRef<S> tile_ref(const DemoTensorEntry *entries, int n, long long c, int j)
+{
+    TileRef<S> t;
+    t.te = entries[demo_find_entry(entries, n, c)];
+    t.lc = c - t.te.chunk_begin;
+    const long long k0 = t.lc / t.te.c1;
+    t.base = (size_t)k0 * S * (size_t)t.te.n1 + (size_t)(t.lc - k0 * t.te.c1) * S + j;
+    return t;
+}
+// Row j of the kept coefficients in q -> column j of C^T Q C in q.
+template <int S>
+__device__ __forceinline__ void inverse_tile(float (&q)[S], float *X, int j)
+{
+    constexpr int XS = Tile<S>::XS;
+    fdct::dct3_ortho_dense4<S>(q);
+#pragma unroll
+    for (int v = 0; v < S; ++v) X[j * XS + v] = q[v];
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < S; ++u) q[u] = X[u * XS + j];
+    __syncwarp();
+    fdct::dct3_ortho_dense4<S>(q);
+}
+
+template <int S, typename GT>
+__device__ __forceinline__ void compress_tiles(const DemoCompressArgs &a, long long group, float *warp_mem)
+{
+    constexpr int XS = Tile<S>::XS, M = S * S;
+    const int lane = threadIdx.x & 31, j = lane % S, sub = lane / S;
+    float *X = warp_mem + sub * (S * XS + S);
+    const long long c_own = group * Tile<S>::PER_WARP + sub;
+    const bool on = c_own < a.n_chunks;
+    const TileRef<S> t = tile_ref<S>(a.entries, a.n_entries, on ? c_own : a.n_chunks - 1, j);
+    const int n1 = t.te.n1, k = t.te.k_eff;
+    float *__restrict__ m = a.m_ptrs[t.te.tensor] + t.base;
+    const GT *__restrict__ g = static_cast<const GT *>(a.g_ptrs[t.te.tensor]) + t.base;
+
+    // momentum update  B = beta*m + g, column j  (Algorithm 1, worker side)
+    float B[S], q[S];
+    {
+        GT gv[S];
+#pragma unroll
+        for (int i = 0; i < S; ++i) {
+            B[i] = m[(size_t)i * n1];
+            gv[i] = g[(size_t)i * n1];
+        }
+#pragma unroll
+        for (int i = 0; i < S; ++i) q[i] = B[i] = fmaf(a.beta, B[i], (float)gv[i]);
+    }
+    fdct::dct2_ortho_dense4<S>(q);
+#pragma unroll
+    for (int u = 0; u < S; ++u) X[u * XS + j] = q[u];
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < S; ++v) q[v] = X[j * XS + v];
+    __syncwarp();
+    fdct::dct2_ortho_dense4<S>(q);  // row j of Q
+
+    // exact top-k: bit-by-bit search for a threshold with exactly k keys at or above it, all tiles of the warp together
+    unsigned thr = 0u;
+    int need_eq = M;  // k = M: everything is kept
+    if (__any_sync(FULL, k < M)) {
+        unsigned hi = 0u;
+#pragma unroll
+        for (int v = 0; v < S; ++v) hi = max(hi, mag_key(q[v]));
+        hi = __reduce_max_sync(FULL, hi);
+        int n_ge = M;
+#pragma unroll 1
+        for (int bit = 31 - __clz(hi | 1u); bit >= 0 && __any_sync(FULL, n_ge != k); --bit) {
+            const unsigned cand = thr | (1u << bit);
+            int cnt = 0;
+#pragma unroll
+            for (int v = 0; v < S; ++v) cnt += mag_key(q[v]) >= cand;
+            cnt = segment_sum<S>(cnt);
+            if (cnt >= k && n_ge != k) {
+                thr = cand;
+                n_ge = cnt;
+            }
+        }
+        int n_gt = 0;
+#pragma unroll
+        for (int v = 0; v < S; ++v) n_gt += mag_key(q[v]) > thr;
+        need_eq = k - segment_sum<S>(n_gt);
+    }
+    // records in ascending index order (row after row); equal keys in index order until k are reached
+    int gt = 0, eq = 0;
+#pragma unroll
+    for (int v = 0; v < S; ++v) {
+        gt += mag_key(q[v]) > thr;
+        eq += mag_key(q[v]) == thr;
+    }
+    const int before = segment_before<S>(gt | eq << 16, j);
+    gt = before & 0xffff;
+    eq = before >> 16;
+    DemoRecord *rec = a.payload + t.te.rec_begin + t.lc * (long long)k;
+#pragma unroll
+    for (int v = 0; v < S; ++v) {
+        const unsigned key = mag_key(q[v]);
+        const bool keep = key > thr || (key == thr && eq < need_eq);
+        if (keep && on) {
+            DemoRecord r;
+            r.idx = j * S + v;
+            r.val = q[v];
+            rec[gt + min(eq, need_eq)] = r;
+        }
+        gt += key > thr;
+        eq += key == thr;
+        q[v] = keep ? a.alpha * q[v] : 0.f;
+    }
+    // m <- B - alpha * IDCT(kept)
+    inverse_tile<S>(q, X, j);
+    if (on) {
+#pragma unroll
+        for (int i = 0; i < S; ++i) m[(size_t)i * n1] = B[i] - q[i];
+    }
+}
+
+template <int S>
+__device__ __forceinline__ void decode_tiles(const DemoDecodeArgs &a, long long group, float *warp_mem, unsigned short *warp_counts)
+{
+    constexpr int XS = Tile<S>::XS, M = S * S;
+    const int lane = threadIdx.x & 31, j = lane % S, sub = lane / S;
+    float *X = warp_mem + sub * (S * XS + S);
+    unsigned short *senders = warp_counts + sub * M;
+    const bool counts = a.agg == 2;
+    const long long c_own = group * Tile<S>::PER_WARP + sub;
+    const bool on = c_own < a.n_chunks;
+    const TileRef<S> t = tile_ref<S>(a.entries, a.n_entries, on ? c_own : a.n_chunks - 1, j);
+    const int n1 = t.te.n1, k = t.te.k_eff;
+    const long long rec_off = t.te.rec_begin + t.lc * (long long)k;
+#pragma unroll
+    for (int v = 0; v < S; ++v) {
+        X[j * XS + v] = 0.f;
+        if (counts) senders[j * S + v] = 0;
+    }
+    __syncwarp();
+    // sum over workers in worker order; the records of eight workers are fetched together, or, for k > S, eight rounds of
+    // one worker's
+    auto add = [&](DemoRecord r) {
+        if ((unsigned)r.idx < (unsigned)M) {
+            X[(r.idx / S) * XS + r.idx % S] += r.val;
+            if (counts) senders[r.idx] += 1;
+        } else if (on) {
+            atomicMax(a.status, DEMO_DEV_PAYLOAD);
+        }
+    };
+    if (__all_sync(FULL, k <= S)) {
+        for (int w0 = 0; w0 < a.W; w0 += 8) {
+            DemoRecord rc[8];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) rc[w] = (j < k && w0 + w < a.W) ? a.payloads[w0 + w][rec_off + j] : DemoRecord{-1, 0.f};
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                if (j < k && w0 + w < a.W) add(rc[w]);
+                __syncwarp();
+            }
+        }
+    } else {
+        for (int w = 0; w < a.W; ++w) {
+            for (int r0 = 0; r0 < M; r0 += 8 * S) {  // (k <= M)
+                DemoRecord rc[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int i = r0 + r * S + j;
+                    rc[r] = i < k ? a.payloads[w][rec_off + i] : DemoRecord{-1, 0.f};
+                }
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+                    if (r0 + r * S + j < k) add(rc[r]);
+            }
+            __syncwarp();
+        }
+    }
+    float q[S];
+#pragma unroll
+    for (int v = 0; v < S; ++v) {
+        q[v] = X[j * XS + v];
+        if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
+            const unsigned short n = senders[j * S + v];
+            if (n > 1) q[v] = q[v] / (float)n;
+        }
+    }
+    __syncwarp();
+    inverse_tile<S>(q, X, j);
+    if (!on) return;
+    if (a.sign_ptrs) {  // parameter-server form: hand out sign(R), the workers apply it
+        signed char *__restrict__ sg = a.sign_ptrs[t.te.tensor] + t.base;
+#pragma unroll
+        for (int i = 0; i < S; ++i) sg[(size_t)i * n1] = (signed char)((q[i] > 0.f) - (q[i] < 0.f));
+        return;
+    }
+    // x <- x - lr * (phi(R) + wd * x), sign(0) = 0
+    float *__restrict__ x = a.x_ptrs[t.te.tensor] + t.base;
+    float xv[S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) xv[i] = x[(size_t)i * n1];
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+        const float sg = a.phi ? q[i] * a.agg_scale : (float)((q[i] > 0.f) - (q[i] < 0.f));
+        x[(size_t)i * n1] = fmaf(-a.lr, fmaf(a.wd, xv[i], sg), xv[i]);
+    }
+}
+
+// ---- kernels: blocks below `seg_blocks` walk the segments, the others the tiles (TILES only) ------------------
+template <int S, bool TILES>
+constexpr int warp_floats() { return TILES && Tile<S>::FLOATS > Seg<S>::PAD ? Tile<S>::FLOATS : Seg<S>::PAD; }
+
+template <int S, typename GT, bool TILES>
+__global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArgs segs, DemoCompressArgs tiles, int seg_blocks)
+{
+    __shared__ __align__(16) float mem[WARPS][warp_floats<S, TILES>()];
+    const int warp = threadIdx.x >> 5;
+    if (!TILES || (int)blockIdx.x < seg_blocks) {
+        for (long long c = (long long)blockIdx.x * WARPS + warp; c < segs.n_chunks; c += (long long)seg_blocks * WARPS)
+            compress_segment<S>(segs, c, mem[warp]);
+    } else if constexpr (TILES) {
+        const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
+        const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
+        for (long long p = (long long)(blockIdx.x - seg_blocks) * WARPS + warp; p < groups; p += stride)
+            compress_tiles<S, GT>(tiles, p, mem[warp]);
+    }
+}
+
+template <int S, bool TILES>
+__global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs segs, DemoDecodeArgs tiles, int seg_blocks)
+{
+    __shared__ __align__(16) float mem[WARPS][warp_floats<S, TILES>()];
+    __shared__ unsigned short counts[WARPS][TILES ? Tile<S>::PER_WARP * S * S : S];
+    const int warp = threadIdx.x >> 5;
+    if (!TILES || (int)blockIdx.x < seg_blocks) {
+        for (long long c = (long long)blockIdx.x * WARPS + warp; c < segs.n_chunks; c += (long long)seg_blocks * WARPS)
+            decode_segment<S>(segs, c, mem[warp], counts[warp]);
+    } else if constexpr (TILES) {
+        const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
+        const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
+        for (long long p = (long long)(blockIdx.x - seg_blocks) * WARPS + warp; p < groups; p += stride)
+            decode_tiles<S>(tiles, p, mem[warp], counts[warp]);
+    }
+}
+
+// One warp per segment or group of tiles, up to eight blocks per SM for each list (what 64 registers per thread allow).
+int blocks_for(long long warps, int sm_count)
+{
+    const long long b = (warps + WARPS - 1) / WARPS, cap = 8LL * sm_count;
+    return (int)(b < cap ? b : cap);
+}
+template <class A>
+cudaError_t launch(const void *kernel, int per_warp, const A *segs, const A *tiles, int sm_count, cudaStream_t stream)
+{
+    A none{};
+    const A &sa = segs ? *segs : none, &ta = tiles ? *tiles : none;
+    int seg_blocks = segs ? blocks_for(sa.n_chunks, sm_count) : 0;
+    const int tile_blocks = tiles ? blocks_for((ta.n_chunks + per_warp - 1) / per_warp, sm_count) : 0;
+    if (seg_blocks + tile_blocks == 0) return cudaSuccess;
+    void *params[] = {const_cast<A *>(&sa), const_cast<A *>(&ta), &seg_blocks};
+    return cudaLaunchKernel(kernel, dim3((unsigned)(seg_blocks + tile_blocks)), dim3(THREADS), params, 0, stream);
+}
+
+template <int S>
+cudaError_t compress_small(const DemoCompressArgs *segs, const DemoCompressArgs *tiles, int sm_count, cudaStream_t stream)
+{
+    if constexpr (S <= 16) {
+        if (tiles)
+            return launch(tiles->grad_bf16 ? (const void *)compress_small_kernel<S, __nv_bfloat16, true>
+                                           : (const void *)compress_small_kernel<S, float, true>,
+                          Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
+    }
+    return launch((const void *)compress_small_kernel<S, float, false>, 1, segs, (const DemoCompressArgs *)nullptr, sm_count, stream);
+}
+template <int S>
+cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count, cudaStream_t stream)
+{
+    if constexpr (S <= 16) {
+        if (tiles)
+            return launch((const void *)decode_small_kernel<S, true>, Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
+    }
+    return launch((const void *)decode_small_kernel<S, false>, 1, segs, (const DemoDecodeArgs *)nullptr, sm_count, stream);
+}
+
+}  // namespace
+
+bool demo_small_tiles_supported(int s) { return s == 8 || s == 16; }
+
+cudaError_t demo_launch_compress_small(int s, const DemoCompressArgs *segs, const DemoCompressArgs *tiles, int sm_count,
+                                       cudaStream_t stream)
+{
+    switch (s) {
+        case 8: return compress_small<8>(segs, tiles, sm_count, stream);
+        case 16: return compress_small<16>(segs, tiles, sm_count, stream);
+        case 32: return compress_small<32>(segs, nullptr, sm_count, stream);
+        case 64: return compress_small<64>(segs, nullptr, sm_count, stream);
+        case 128: return compress_small<128>(segs, nullptr, sm_count, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count,
+                                     cudaStream_t stream)
+{
+    switch (s) {
+        case 8: return decode_small<8>(segs, tiles, sm_count, stream);
+        case 16: return decode_small<16>(segs, tiles, sm_count, stream);
+        case 32: return decode_small<32>(segs, nullptr, sm_count, stream);
+        case 64: return decode_small<64>(segs, nullptr, sm_count, stream);
+        case 128: return decode_small<128>(segs, nullptr, sm_count, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}

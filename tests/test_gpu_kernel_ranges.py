@@ -58,3 +58,34 @@ def test_nd_ties_and_untouched_chunks():
     for _ in range(2):
         r.step()
     r.close()
+
+
+@pytest.mark.parametrize("k", [1, 4, 8, 9, 63, 64])
+def test_small_tiles_8(k):
+    """s = 8: four tiles per warp, an odd number of them, records beyond one round of lanes, lossless."""
+    wl = inputs.Workload("s8", [(3 * 8, 7 * 8), (8, 8), (5 * 8,)], chunk=8, topk=k, num_workers=9, grad_kind="student_t_ties")
+    r = parity.Runner(wl, max_chunks=10**9, seed=k)
+    for _ in range(2):
+        r.step()
+    r.close()
+
+
+@pytest.mark.parametrize("k,agg", [(2, 0), (16, 2), (17, 1), (130, 2), (256, 0)])
+def test_small_tiles_16(k, agg):
+    wl = inputs.Workload("s16", [(3 * 16, 3 * 16), (16, 32)], chunk=16, topk=k, num_workers=3, grad_kind="student_t_ties",
+                         grad_dtype=torch.float32)
+    r = parity.Runner(wl, max_chunks=10**9, seed=k, agg=agg)
+    for _ in range(2):
+        r.step()
+    r.close()
+
+
+@pytest.mark.parametrize("s,k,workers", [(8, 3, 2), (16, 16, 9), (32, 5, 17), (64, 33, 5), (128, 1, 3), (128, 97, 2)])
+def test_segments(s, k, workers):
+    """1-D tensors alone, more than one tensor per warp's search (33 and up), tied and zero segments among them."""
+    shapes = [(s * (1 + t % 3),) for t in range(37)]
+    wl = inputs.Workload("seg", shapes, chunk=s, topk=k, num_workers=workers, grad_kind="student_t_ties")
+    r = parity.Runner(wl, max_chunks=10**9, seed=s + k)
+    for _ in range(2):
+        r.step()
+    r.close()
