@@ -232,7 +232,7 @@ class DemoTransform:
     def _array(self, key, tensors, check=None):
         """Pointer array for a list of tensors, cached per key and data pointers.  ``check`` = (shapes,
         dtype, on_device) is verified whenever the pointers are new."""
-        ptrs = tuple(_tensor_ptrs(tensors))
+        ptrs = [t.data_ptr() for t in tensors]
         hit = self._ptr_cache.get(key)
         if hit is None or hit[0] != ptrs:
             if check is not None:
@@ -258,10 +258,8 @@ class DemoTransform:
 
     @staticmethod
     def _stream(stream) -> ctypes.c_void_p:
-        if stream is None:
-            import torch
-
-            stream = torch.cuda.current_stream()
+        if stream is None:  # the current stream's handle, without building a Stream object around it
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
         return ctypes.c_void_p(int(getattr(stream, "cuda_stream", stream)))
 
     # --- the ABI calls -------------------------------------------------------------------------

@@ -7,6 +7,8 @@
 
 #include <vector>
 
+struct DemoTickets;  // launch.cuh
+
 // One payload record: flat index inside the chunk + fp32 coefficient (8 bytes, little-endian).
 struct DemoRecord {
     int32_t idx;
@@ -42,6 +44,8 @@ struct DemoCompressArgs {
     // pointer arrays; box = one s x s tile).  NULL: tiles are staged row by row with 1-D bulk copies.
     const void *tmap_m;
     const void *tmap_g;
+    int wait_first = 1;  // see StreamOrder (launch.cuh)
+    DemoTickets *tickets = nullptr;  // device; the counter of this kernel's chunks
     // 1: the momentum tensors hold the chunk-wise DCT of the momentum (tiles transposed); only the s = 64 tile
     // kernel with tensor maps implements it
     int momentum_dct = 0;
@@ -58,13 +62,15 @@ struct DemoDecodeArgs {
     float lr;
     float wd;
     int *status;
-    const void *tmap_x;  // optional tensor maps of the parameter tensors (see DemoCompressArgs)
+    const void *tmap_x;  // optional tensor maps of the parameter tensors (see DemoCompressArgs); s = 128 only
     int agg;          // 0 sum, 1 mean over workers, 2 per-coordinate count-normalised mean (0/0 = 0)
     int phi;          // 0 sign, 1 identity
     float agg_scale;  // 1/W for the mean, else 1 (only the identity update sees it)
     // Parameter-server form: when not NULL, write sign(R) in {-1, 0, +1} per element to these int8 tensors
     // (device array indexed like x_ptrs) instead of updating the parameters.
     signed char *const *sign_ptrs = nullptr;
+    int wait_first = 1;  // see StreamOrder (launch.cuh)
+    DemoTickets *tickets = nullptr;  // device; the counter of this kernel's chunks
 };
 
 // Launchers (defined in the kernel translation units).  `s` is the chunk size.  Return the CUDA error of the launch.
@@ -161,6 +167,8 @@ struct DemoNdCompressArgs {
     float beta, alpha;
     int grad_bf16;
     int *status;
+    int wait_first = 1;  // see StreamOrder (launch.cuh)
+    DemoTickets *tickets = nullptr;  // device; the counter of this kernel's chunks
 };
 
 struct DemoNdDecodeArgs {
@@ -175,6 +183,8 @@ struct DemoNdDecodeArgs {
     int agg, phi;
     float agg_scale;
     signed char *const *sign_ptrs = nullptr;  // see DemoDecodeArgs
+    int wait_first = 1;
+    DemoTickets *tickets = nullptr;
 };
 
 // x <- x - lr (sign + wd x) from int8 signs, over every tensor of a context (kernels_generic.cu).

@@ -10,6 +10,9 @@
 
 #include "../../include/demo.h"
 #include "demo_internal.h"
+#include "launch.cuh"
+
+constexpr int TICKETS = 32;  // one per kernel of a call that may run beside another: tiles, N-D classes
 
 struct demo_ctx {
     demo_config cfg;
@@ -30,6 +33,7 @@ struct demo_ctx {
     long long chunks2d = 0, chunks1d = 0;
     DemoTensorEntry *d_entries2d = nullptr, *d_entries1d = nullptr;
 
+    DemoTickets *d_tickets = nullptr;  // [TICKETS] chunk counters, zero between launches
     float *d_C = nullptr;
     int *d_status = nullptr;
 
@@ -67,13 +71,8 @@ struct demo_ctx {
     // the caller's pointers change.  NULL when the driver entry point is unavailable.
     PFN_cuTensorMapEncodeTiled encode = nullptr;
     CUtensorMap *d_tm_g = nullptr, *d_tm_m = nullptr;  // [W][T]
-    CUtensorMap *d_tm_x = nullptr;                     // [T]
+    CUtensorMap *d_tm_x = nullptr;                     // [T], s = 128 only
     std::vector<CUtensorMap> h_tm;                     // staging, [T]
-
-    // The small kernel of the 1-D tensors runs on a side stream beside the kernel of the 2-D tensors
-    // (fork / join by events; also legal inside a stream capture).  NULL: both on the caller's stream.
-    cudaStream_t side_stream = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 
     // demo_step_host: host->device gradient copies run on their own stream so that the copy of worker
     // w+1 overlaps the compress of worker w (created on first use)
@@ -147,6 +146,7 @@ void release(demo_ctx *c)
     if (!c) return;
     cudaFree(c->d_entries2d);
     cudaFree(c->d_entries1d);
+    cudaFree(c->d_tickets);
     cudaFree(c->d_C);
     cudaFree(c->d_entries_nd);
     cudaFree(c->d_tables);
@@ -166,9 +166,6 @@ void release(demo_ctx *c)
     for (cudaEvent_t e : c->ev_copied)
         if (e) cudaEventDestroy(e);
     if (c->ev_start) cudaEventDestroy(c->ev_start);
-    if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-    if (c->ev_join) cudaEventDestroy(c->ev_join);
-    if (c->side_stream) cudaStreamDestroy(c->side_stream);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     delete c;
 }
@@ -295,6 +292,7 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     bool ok = true;
     ok = ok && cudaMalloc(&c->d_C, C.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_status, sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_tickets, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_P, C.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_P_stage, 2 * C.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_basis_flag, sizeof(int)) == cudaSuccess;
@@ -318,7 +316,7 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
             }
             ok = ok && cudaMalloc(&c->d_tm_g, W * T * sizeof(CUtensorMap)) == cudaSuccess;
             ok = ok && cudaMalloc(&c->d_tm_m, W * T * sizeof(CUtensorMap)) == cudaSuccess;
-            ok = ok && cudaMalloc(&c->d_tm_x, T * sizeof(CUtensorMap)) == cudaSuccess;
+            if (s == 128) ok = ok && cudaMalloc(&c->d_tm_x, T * sizeof(CUtensorMap)) == cudaSuccess;
         } else {
             cudaGetLastError();
         }
@@ -330,16 +328,7 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     }
     ok = ok && cudaMemcpy(c->d_C, C.data(), C.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess;
-    if (ok && c->n2d && c->n1d) {
-        // optional: without them the two kernels of a call simply run one after the other
-        if (cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            if (c->side_stream) cudaStreamDestroy(c->side_stream);
-            c->side_stream = nullptr;
-        }
-    }
+    ok = ok && cudaMemset(c->d_tickets, 0, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     if (ok && c->n2d)
         ok = cudaMemcpy(c->d_entries2d, e2d.data(), e2d.size() * sizeof(DemoTensorEntry), cudaMemcpyHostToDevice) ==
              cudaSuccess;
@@ -385,7 +374,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
     // Square chunks of one size: when every tensor is cut into s x s tiles of its last two axes or into length-s
     // segments of its last axis (all leading chunk extents 1, so the leading axes merely stack rows), for one s
     // that demo_init knows, the layout of chunks and records is that of demo_init on the flattened tensors -- the
-    // context is built by it and runs its kernels (fast DCT, tensor maps, side stream).
+    // context is built by it and runs its kernels (fast DCT, tensor maps).
     {
         int s_common = 0;
         bool regular = true;
@@ -501,6 +490,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
     ok = ok && cudaMalloc(&c->d_tables, tables.data.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_entries_nd, entries.size() * sizeof(DemoNdEntry)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_status, sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_tickets, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_g, W * T * sizeof(void *)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_m, W * T * sizeof(void *)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_x, T * sizeof(void *)) == cudaSuccess;
@@ -514,6 +504,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
     ok = ok && cudaMemcpy(c->d_entries_nd, entries.data(), entries.size() * sizeof(DemoNdEntry),
                           cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMemset(c->d_tickets, 0, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         release(c);
@@ -533,26 +524,6 @@ demo_status demo_payload_layout(const demo_ctx *ctx, int32_t tensor, int64_t *fi
     if (n_chunks) *n_chunks = ctx->n_chunks[tensor];
     if (k_eff) *k_eff = ctx->k_eff[tensor];
     return DEMO_OK;
-}
-
-// The 1-D kernel of a call goes to the side stream: it is ordered after everything already queued on the
-// caller's stream (fork) and the caller's stream continues only when it is done (join).
-static cudaStream_t fork_side(demo_ctx *ctx, cudaStream_t stream)
-{
-    if (!ctx->side_stream || !ctx->n2d || !ctx->n1d) return stream;
-    if (cudaEventRecord(ctx->ev_fork, stream) != cudaSuccess ||
-        cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return stream;
-    }
-    return ctx->side_stream;
-}
-static cudaError_t join_side(demo_ctx *ctx, cudaStream_t side, cudaStream_t stream)
-{
-    if (side == stream) return cudaSuccess;
-    cudaError_t err = cudaEventRecord(ctx->ev_join, side);
-    if (err == cudaSuccess) err = cudaStreamWaitEvent(stream, ctx->ev_join, 0);
-    return err;
 }
 
 // The fast kernels hard-code the DCT factorisation; any other basis takes the dense-transform kernels.
@@ -626,6 +597,8 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
         for (const DemoNdClass &k : ctx->nd_classes) {
             n.entries = ctx->d_entries_nd + k.first;
             n.cls = k;
+            n.wait_first = &k == &ctx->nd_classes.front();  // the classes run side by side
+            n.tickets = ctx->d_tickets + (&k - ctx->nd_classes.data());
             if (demo_launch_compress_nd(n, ctx->sm_count, stream) != cudaSuccess) {
                 cudaGetLastError();
                 return DEMO_ERR_CUDA;
@@ -658,14 +631,9 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
     a.n_chunks = ctx->chunks2d;
     a.k = ctx->cfg.topk;  // <= s * s
     a.momentum_dct = ctx->momentum_dct ? 1 : 0;
+    a.tickets = ctx->d_tickets;
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
-    cudaStream_t side = stream;
-    if (ctx->n1d || small_tiles) {
-        if (!small_tiles) side = fork_side(ctx, stream);
-        err = demo_launch_compress_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, side);
-        ctx->launches += 1;
-    }
-    if (err == cudaSuccess && ctx->n2d && !small_tiles) {
+    if (ctx->n2d && !small_tiles) {
         if (use_fast_path(ctx))
             err = demo_launch_compress_fast(s, a, ctx->sm_count, stream);
         else if (use_tc_path(ctx))
@@ -674,9 +642,11 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
             err = demo_launch_compress_generic(s, a, ctx->sm_count, stream);
         ctx->launches += 1;
     }
-    {
-        const cudaError_t jerr = join_side(ctx, side, stream);  // always, so that a fork never stays open
-        if (err == cudaSuccess) err = jerr;
+    if (err == cudaSuccess && (ctx->n1d || small_tiles)) {
+        // behind the kernel of the tiles, so that it fills the SMs that one leaves idle at its end
+        a1.wait_first = small_tiles || !ctx->n2d;
+        err = demo_launch_compress_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, stream);
+        ctx->launches += 1;
     }
     if (err != cudaSuccess) {
         cudaGetLastError();
@@ -756,7 +726,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     if (err == cudaSuccess && params)
         err = sync_table<float *>(ctx->d_x, ctx->h_x.data(), const_cast<float *const *>(params), T, &ctx->x_valid,
                                   stream, &x_changed);
-    if (err == cudaSuccess && params && ctx->encode && x_changed &&
+    if (err == cudaSuccess && params && ctx->d_tm_x && x_changed &&
         !upload_tensor_maps(ctx, ctx->d_tm_x, params, false, stream)) {
         err = cudaErrorInvalidValue;
         ctx->x_valid = false;
@@ -785,6 +755,8 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
         for (const DemoNdClass &k : ctx->nd_classes) {
             n.entries = ctx->d_entries_nd + k.first;
             n.cls = k;
+            n.wait_first = &k == &ctx->nd_classes.front();  // the classes run side by side
+            n.tickets = ctx->d_tickets + (&k - ctx->nd_classes.data());
             if (demo_launch_decode_nd(n, ctx->sm_count, stream) != cudaSuccess) {
                 cudaGetLastError();
                 return DEMO_ERR_CUDA;
@@ -802,7 +774,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.lr = ctx->cfg.lr;
     a.wd = ctx->cfg.weight_decay;
     a.status = ctx->d_status;
-    a.tmap_x = (ctx->encode && params) ? ctx->d_tm_x : nullptr;
+    a.tmap_x = params ? ctx->d_tm_x : nullptr;
     a.agg = ctx->aggregation;
     a.phi = ctx->phi;
     a.agg_scale = (ctx->aggregation == DEMO_AGG_MEAN) ? 1.0f / (float)W : 1.0f;
@@ -815,14 +787,9 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.entries = ctx->d_entries2d;
     a.n_entries = ctx->n2d;
     a.n_chunks = ctx->chunks2d;
+    a.tickets = ctx->d_tickets;
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
-    cudaStream_t side = stream;
-    if (ctx->n1d || small_tiles) {
-        if (!small_tiles) side = fork_side(ctx, stream);
-        err = demo_launch_decode_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, side);
-        ctx->launches += 1;
-    }
-    if (err == cudaSuccess && ctx->n2d && !small_tiles) {
+    if (ctx->n2d && !small_tiles) {
         // (a caller-supplied basis: the signs come from the dense kernels, there is no tensor-core variant)
         if (use_fast_path(ctx))
             err = demo_launch_decode_fast(s, a, ctx->sm_count, stream);
@@ -832,9 +799,11 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
             err = demo_launch_decode_generic(s, a, ctx->sm_count, stream);
         ctx->launches += 1;
     }
-    {
-        const cudaError_t jerr = join_side(ctx, side, stream);
-        if (err == cudaSuccess) err = jerr;
+    if (err == cudaSuccess && (ctx->n1d || small_tiles)) {
+        // behind the kernel of the tiles, so that it fills the SMs that one leaves idle at its end
+        a1.wait_first = small_tiles || !ctx->n2d;
+        err = demo_launch_decode_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, stream);
+        ctx->launches += 1;
     }
     if (err != cudaSuccess) {
         cudaGetLastError();
@@ -872,7 +841,7 @@ demo_status demo_apply_signs(demo_ctx *ctx, const int8_t *const *signs, float *c
     bool x_changed = false;
     cudaError_t err = sync_table<float *>(ctx->d_x, ctx->h_x.data(), const_cast<float *const *>(params), T,
                                           &ctx->x_valid, stream, &x_changed);
-    if (err == cudaSuccess && ctx->encode && x_changed && !upload_tensor_maps(ctx, ctx->d_tm_x, params, false, stream)) {
+    if (err == cudaSuccess && ctx->d_tm_x && x_changed && !upload_tensor_maps(ctx, ctx->d_tm_x, params, false, stream)) {
         err = cudaErrorInvalidValue;
         ctx->x_valid = false;
     }

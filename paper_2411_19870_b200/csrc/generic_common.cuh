@@ -3,6 +3,7 @@
 #pragma once
 
 #include "demo_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -87,16 +88,13 @@ cudaError_t launch_persistent(K kernel, size_t smem, long long n_chunks, int sm_
                               const void *args_struct_ptr)
 {
     if (n_chunks <= 0) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, GEN_THREADS, smem);
+    const cudaError_t err = demo_resident_ctas((const void *)kernel, GEN_THREADS, smem, &per_sm);
     if (err != cudaSuccess) return err;
-    if (per_sm < 1) per_sm = 1;
     long long grid = (long long)sm_count * per_sm;
     if (grid > n_chunks) grid = n_chunks;
     void *params[] = {const_cast<void *>(args_struct_ptr)};
-    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)grid), dim3(GEN_THREADS), params, smem, stream);
+    return demo_launch_kernel((const void *)kernel, grid, GEN_THREADS, smem, stream, params);
 }
 
 }  // namespace

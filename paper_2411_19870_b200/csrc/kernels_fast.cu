@@ -23,6 +23,7 @@
 #include "demo_internal.h"
 #include "fast_common.cuh"
 #include "fast_dct.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -57,6 +58,7 @@ constexpr size_t compress_slot_bytes()
 template <int S, typename GT, bool TMAP, int THREADS>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress_fast_kernel(DemoCompressArgs a)
 {
+    const StreamOrder order(a.wait_first);
     using C = Cfg<S>;
     constexpr int XS = C::XS, NW = C::NW, LOG2S = C::LOG2S;
     constexpr unsigned TILE_BYTES = S * S * sizeof(float) + S * S * sizeof(GT);
@@ -759,7 +761,7 @@ constexpr int STAGE_RECORDS = 512;  // records staged per batch of the scatter (
 template <int S>
 __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)
 {
-    return ((size_t)S * Cfg<S>::XS * 4 + 16 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + (counts ? (size_t)S * S * 2 : 0) + 127) /
+    return ((size_t)S * Cfg<S>::XS * 4 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + (counts ? (size_t)S * S * 2 : 0) + 127) /
            128 * 128;
 }
 
@@ -767,9 +769,13 @@ __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)
 // nor written (a separate instantiation, so that the update kernel keeps its size).
 // WIDE: the instantiation for fan-ins above one staging batch (sixteen workers at k <= 32): every further batch of a
 // chunk's workers is requested, like the first, while the scatter works on the batch before it.
-template <int S, bool TMAP, int THREADS, bool SIGNS = false, bool WIDE = false>
+// The x tile comes by 16-byte asynchronous copies, sixteen per thread, not by TMA: a tensor map has to be acquired by every
+// CTA that comes to a tensor, a fence that stands in front of the chunk (300M-class set, 168 matrices: 696 us with maps, 725
+// with a bulk copy per row, 624 like this; one matrix of that size: 612, 731, 597).
+template <int S, int THREADS, bool SIGNS = false, bool WIDE = false>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(DemoDecodeArgs a)
 {
+    const StreamOrder order(a.wait_first);
     using C = Cfg<S>;
     constexpr int XS = C::XS, NCH = THREADS / S;
     constexpr int M = S * S;
@@ -782,25 +788,14 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     // read back into registers -- the staging area of the x tile, fetched behind the second transform.
     float *St = reinterpret_cast<float *>(smem_raw);  // [S*XS]
     float *Xt = St;                                   // [S*S] (aliases St)
-    unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(St + S * XS);
-    DemoRecord *stage_all = reinterpret_cast<DemoRecord *>(bar_mem + 2);    // [2][STAGE_RECORDS] records of a batch of workers
+    DemoRecord *stage_all = reinterpret_cast<DemoRecord *>(St + S * XS);    // [2][STAGE_RECORDS] records of a batch of workers
     unsigned short *Cn = reinterpret_cast<unsigned short *>(stage_all + 2 * STAGE_RECORDS);  // [S*S] senders per coordinate (agg == 2)
 
     const int t = threadIdx.x % S;
-    const uint32_t bar = smem_u32(bar_mem);
-    if (t == 0) {
-        mbar_init(bar, 1);
-        fence_proxy_async();  // make the initialised barrier visible to the async proxy
-    }
-    __syncthreads();
-    fence_proxy_async();
 
     EntryCursor cur;
     float *x_ptr = nullptr;
     int cached_tensor = -1;
-    unsigned phase = 0;
-    bool failed = false;
-    const char *acquired = nullptr;
     const unsigned lr_bits = __float_as_uint(a.lr);
     const float decay = 1.f - a.lr * a.wd;
     const float neg_lr_scale = -a.lr * a.agg_scale;
@@ -842,13 +837,21 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    const long long stride = (long long)gridDim.x * NCH;
-    long long c = (long long)blockIdx.x * NCH + slot;
+    // A CTA's slots take NCH neighbouring chunks at a time (a group), the groups on demand.  The group after the current one
+    // has to be known during the current one (its records are requested), so a group is drawn two ahead: thread 0 draws at
+    // the start of a chunk and writes the result down behind the scatter; the loop-top barrier publishes it.
+    __shared__ unsigned drawn[2];
+    if (threadIdx.x == 0) drawn[0] = ticket_draw(a.tickets);
+    unsigned group = blockIdx.x, next_group, par = 0;
+    long long c = (long long)group * NCH + slot;
     int buf = 0;
     if (c < a.n_chunks) stage_ahead(0, c);
-    for (long long cb = (long long)blockIdx.x * NCH; cb < a.n_chunks; cb += stride, c += stride) {
-        if (__syncthreads_or(failed)) break;  // all slots start a chunk together (shared instruction stream)
+    for (; (long long)group * NCH < a.n_chunks; group = next_group, c = (long long)group * NCH + slot, par ^= 1u) {
+        __syncthreads();
+        next_group = gridDim.x + drawn[par];  // (NO_TICKET ends the loop: groups are fewer than 2^31)
         if (c >= a.n_chunks) continue;
+        unsigned ticket = 0;
+        if (threadIdx.x == 0) ticket = ticket_draw(a.tickets);
         cur.seek(a.entries, a.n_entries, c);
         const DemoTensorEntry te = cur.te;
         if (te.tensor != cached_tensor) {
@@ -862,13 +865,10 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         float *__restrict__ x = x_ptr;
         const int k_eff = te.k_eff;
         const long long rec_off = te.rec_begin + lc * (long long)k_eff;
-        if (TMAP && !SIGNS && t == 0) {
-            const char *tm_x = static_cast<const char *>(a.tmap_x) + (size_t)te.tensor * TMAP_BYTES;
-            if (tm_x != acquired) {  // first use of this tensor's map by the issuing thread
-                acquired = tm_x;
-                tmap_acquire(tm_x);
-            }
-            tma_prefetch_2d(tm_x, k1 * S, (int)k0 * S);
+        if (!SIGNS) {  // row t of the x tile on its way to L2
+            const float *xr = x + base + (size_t)t * te.n1;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
+            if (S == 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 32));
         }
 
         {
@@ -879,8 +879,9 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 for (int v = 0; v < S; ++v) Cn[t * S + v] = 0;
         }
         auto stage_next_chunk = [&](int into) {  // (the cursor moves on; this chunk's table entry is in `te`)
-            if (c + stride < a.n_chunks)
-                stage_ahead(into, c + stride);
+            const long long nc = (long long)next_group * NCH + slot;
+            if (nc < a.n_chunks)
+                stage_ahead(into, nc);
             else
                 asm volatile("cp.async.commit_group;" ::: "memory");
         };
@@ -987,6 +988,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 }
             }
         }
+        if (threadIdx.x == 0) drawn[par ^ 1u] = ticket;
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0 (row t is this thread's)
             for (int v = 0; v < S; ++v) {
                 const unsigned short n = Cn[t * S + v];
@@ -996,7 +998,6 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         // Two inverse passes through one copy of the unrolled transform (rolled loop): pass 0 along
         // row t in place, pass 1 down column t; the x tile is fetched while pass 1 computes.
         float r[S];
-        bool arrived = true;
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
             if (pass == 0) {
@@ -1012,19 +1013,17 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             } else {
 #pragma unroll
                 for (int u = 0; u < S; ++u) r[u] = St[u * XS + t];
-                fence_proxy_async();
                 sb.sync();  // the tile is dead: stage x into it
-                if (SIGNS) {
-                    // nothing to stage
-                } else if (TMAP) {
-                    if (t == 0) {
-                        mbar_expect_tx(bar, S * S * sizeof(float));
-                        tma_load_2d(smem_u32(Xt), static_cast<const char *>(a.tmap_x) + (size_t)te.tensor * TMAP_BYTES,
-                                    k1 * S, (int)k0 * S, bar);
-                    }
-                } else {
-                    if (t == 0) mbar_expect_tx(bar, S * S * sizeof(float));
-                    bulk_g2s(smem_u32(Xt + t * S), x + base + (size_t)t * te.n1, S * sizeof(float), bar);
+                if (!SIGNS) {
+                    constexpr int PIECES = S / 4;  // 16-byte pieces per row
+                    const float *src = x + base + (size_t)(t / PIECES) * te.n1 + (t % PIECES) * 4;
+                    const uint32_t dst = smem_u32(Xt) + t * 16;
+#pragma unroll
+                    for (int i = 0; i < PIECES; ++i)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * (S * 16)),
+                                     "l"(src + (size_t)(i * (S / PIECES)) * te.n1)
+                                     : "memory");
+                    asm volatile("cp.async.commit_group;" ::: "memory");
                 }
             }
             {
@@ -1041,9 +1040,6 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 for (int v4 = 0; v4 < S / 4; ++v4)
                     row[v4] = make_float4(r[4 * v4], r[4 * v4 + 1], r[4 * v4 + 2], r[4 * v4 + 3]);
                 sb.sync();
-            } else if (!SIGNS) {
-                arrived = mbar_wait_bounded(bar, phase);
-                phase ^= 1u;
             }
         }
         if constexpr (SIGNS) {
@@ -1053,12 +1049,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             sb.sync();  // the tile is free again
             continue;
         }
-        if (!sb.sync_and(arrived)) {
-            if (t == 0) atomicMax(a.status, DEMO_DEV_TIMEOUT);
-            mbar_wait_bounded(bar, phase ^ 1u);
-            failed = true;
-            continue;
-        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");  // (the next chunk's records, requested before, have landed too)
+        sb.sync();
         // sign and update:  x - lr (sign(R) + wd x) = x (1 - lr wd) - lr sign(R); -lr sign(R) is lr with
         // its sign flipped where R > 0, and zero where R == 0
 #pragma unroll
@@ -1072,6 +1064,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         sb.sync();  // the tile is free again
     }
     asm volatile("cp.async.wait_all;" ::: "memory");  // no copy of this thread may outlive the CTA's shared memory
+    if (threadIdx.x == 0) ticket_finish(a.tickets);
 }
 
 // CTA sizes: the compress kernel runs best with all eight slots of an SM in one CTA (one shared
@@ -1087,22 +1080,20 @@ constexpr int DECODE_THREADS = 64;
 
 // Persistent launch: CTAs of `threads` threads (threads / S slots), as many as fit the device, each
 // striding over groups of chunks.
-template <typename K>
-cudaError_t launch(K kernel, int threads, int nch, size_t smem, long long n_chunks, int sm_count, cudaStream_t stream,
-                   const void *args)
+template <typename K, typename A>
+cudaError_t launch(K kernel, int threads, int nch, size_t smem, int sm_count, cudaStream_t stream, A args)
 {
+    const long long n_chunks = args.n_chunks;
     if (n_chunks <= 0) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+    const cudaError_t err = demo_resident_ctas((const void *)kernel, threads, smem, &per_sm);
     if (err != cudaSuccess) return err;
-    if (per_sm < 1) per_sm = 1;
     const long long groups = (n_chunks + nch - 1) / nch;
     long long grid = (long long)sm_count * per_sm;
     if (grid > groups) grid = groups;
-    void *params[] = {const_cast<void *>(args)};
-    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)grid), dim3(threads), params, smem, stream);
+    if (grid == groups) args.tickets = nullptr;
+    void *params[] = {&args};
+    return demo_launch_kernel((const void *)kernel, grid, threads, smem, stream, params);
 }
 
 template <int S, typename GT>
@@ -1112,8 +1103,8 @@ cudaError_t launch_compress(const DemoCompressArgs &a, int sm_count, cudaStream_
     constexpr int NCH = TH / S;
     const size_t smem = compress_slot_bytes<S, GT>() * NCH;
     if (a.tmap_m != nullptr && a.tmap_g != nullptr)
-        return launch(compress_fast_kernel<S, GT, true, TH>, TH, NCH, smem, a.n_chunks, sm_count, stream, &a);
-    return launch(compress_fast_kernel<S, GT, false, TH>, TH, NCH, smem, a.n_chunks, sm_count, stream, &a);
+        return launch(compress_fast_kernel<S, GT, true, TH>, TH, NCH, smem, sm_count, stream, a);
+    return launch(compress_fast_kernel<S, GT, false, TH>, TH, NCH, smem, sm_count, stream, a);
 }
 
 template <int S>
@@ -1122,14 +1113,10 @@ cudaError_t launch_decode(const DemoDecodeArgs &a, int sm_count, cudaStream_t st
     constexpr int TH = DECODE_THREADS;
     constexpr int NCH = TH / S;
     const size_t smem = decode_slot_bytes<S>(a.agg == 2) * NCH;
-    if (a.sign_ptrs != nullptr)
-        return launch(decode_fast_kernel<S, false, TH, true>, TH, NCH, smem, a.n_chunks, sm_count, stream, &a);
-    if (a.tmap_x != nullptr) {
-        if (a.W > 16)  // more than one staging batch at k <= 32
-            return launch(decode_fast_kernel<S, true, TH, false, true>, TH, NCH, smem, a.n_chunks, sm_count, stream, &a);
-        return launch(decode_fast_kernel<S, true, TH>, TH, NCH, smem, a.n_chunks, sm_count, stream, &a);
-    }
-    return launch(decode_fast_kernel<S, false, TH>, TH, NCH, smem, a.n_chunks, sm_count, stream, &a);
+    if (a.sign_ptrs != nullptr) return launch(decode_fast_kernel<S, TH, true>, TH, NCH, smem, sm_count, stream, a);
+    if (a.W > 16)  // more than one staging batch at k <= 32
+        return launch(decode_fast_kernel<S, TH, false, true>, TH, NCH, smem, sm_count, stream, a);
+    return launch(decode_fast_kernel<S, TH>, TH, NCH, smem, sm_count, stream, a);
 }
 
 // One CTA arms an mbarrier with a transaction count that no copy will ever satisfy and waits for it

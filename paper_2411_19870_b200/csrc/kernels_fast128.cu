@@ -22,6 +22,7 @@
 #include "demo_internal.h"
 #include "fast_common.cuh"
 #include "fast_dct.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -88,6 +89,7 @@ constexpr size_t compress128_smem()
 template <typename GT>
 __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompressArgs a)
 {
+    const StreamOrder order(a.wait_first);
     constexpr unsigned TILE_BYTES = M * sizeof(float) + M * sizeof(GT);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *Ms = reinterpret_cast<float *>(smem_raw);  // [128*128] m tile
@@ -111,6 +113,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
     }
     // Tensor memory as storage: thread (h, j) parks its 64 elements of column j of B = beta*m + g (rows 0..63 for
     // h = 0, rows 127..64 for h = 1) in lane j, columns 64h .. 64h+63, between the forward pass and the residual.
+    if (tid == 0) tmem_slot[1] = ticket_draw(a.tickets);
     const uint32_t tmem_base = tmem_alloc_cta(tmem_slot, TMEM_COLS128);
     fence_proxy_async();
     const uint32_t taddr = tmem_base + ((uint32_t)(j & ~31) << 16) + (uint32_t)(h * H);
@@ -119,17 +122,20 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
     unsigned phase = 0;
     const char *acquired = nullptr;
 
+    auto acquire_maps = [&](const DemoTensorEntry &te) {
+        const char *tm_m = static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES;
+        if (tid == 0 && tm_m != acquired) {  // tensor maps this thread has not used yet
+            acquired = tm_m;
+            tmap_acquire(tm_m);
+            tmap_acquire(static_cast<const char *>(a.tmap_g) + (size_t)te.tensor * TMAP_BYTES);
+        }
+    };
     auto issue_tiles = [&](const DemoTensorEntry &te, long long c) {
         const unsigned lc = (unsigned)(c - te.chunk_begin);
         const unsigned k0 = lc / (unsigned)te.c1, k1 = lc - k0 * (unsigned)te.c1;
         if (tid == 0) {
             const char *tm_m = static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES;
             const char *tm_g = static_cast<const char *>(a.tmap_g) + (size_t)te.tensor * TMAP_BYTES;
-            if (tm_m != acquired) {  // a tensor map this thread has not used yet: acquire it for the tensor-map proxy
-                acquired = tm_m;
-                tmap_acquire(tm_m);
-                tmap_acquire(tm_g);
-            }
             mbar_expect_tx(bar, TILE_BYTES);
             tma_load_2d(smem_u32(Ms), tm_m, k1 * S, k0 * S, bar);
             tma_load_2d(smem_u32(Gs), tm_g, k1 * S, k0 * S, bar);
@@ -139,17 +145,25 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
     long long c = blockIdx.x;
     if (c < a.n_chunks) {
         cur.seek(a.entries, a.n_entries, c);
+        acquire_maps(cur.te);
         issue_tiles(cur.te, c);
     }
-    for (; c < a.n_chunks; c += gridDim.x) {
+    for (long long nc; c < a.n_chunks; c = nc) {
         const DemoTensorEntry te = cur.te;  // the cursor points at chunk c
         const unsigned lc = (unsigned)(c - te.chunk_begin);
         const unsigned k0 = lc / (unsigned)te.c1, k1 = lc - k0 * (unsigned)te.c1;
-        const size_t base = (size_t)k0 * S * (size_t)te.n1 + (size_t)k1 * S;
-        float *__restrict__ m = a.m_ptrs[te.tensor];
         const int k_eff = te.k_eff;
         DemoRecord *rec = a.payload + te.rec_begin + (long long)lc * k_eff;
 
+        // the next chunk (drawn during the previous one) is looked up, and its tensor maps acquired, while the tiles are on
+        // their way; the cursor moves on.  (Thread 0 wrote the ticket at the end of the previous chunk and overwrites it at
+        // the end of this one; the barrier publishes it, those below see to it that every thread has read it.)
+        __syncthreads();
+        nc = (long long)gridDim.x + tmem_slot[1];
+        if (nc < a.n_chunks) {
+            cur.seek(a.entries, a.n_entries, nc);
+            acquire_maps(cur.te);
+        }
         const bool arrived = mbar_wait_bounded(bar, phase);
         phase ^= 1u;
         if (!__syncthreads_and(arrived)) {
@@ -537,16 +551,17 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         }
         fence_proxy_async();
         __syncthreads();
-        const long long nc = c + gridDim.x;
-        if (nc < a.n_chunks) cur.seek(a.entries, a.n_entries, nc);
         if (tid == 0) {
+            const unsigned ticket = ticket_draw(a.tickets);  // the chunk after the next: drawn behind the store's wait
             tma_store_2d(static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES, (int)(k1 * S), (int)(k0 * S),
                          smem_u32(Ms));
             tma_store_commit();
             tma_store_wait_read();  // the store has read the tile: the next chunk's tiles may land
+            tmem_slot[1] = ticket;
         }
         if (nc < a.n_chunks) issue_tiles(cur.te, nc);
     }
+    if (tid == 0) ticket_finish(a.tickets);
     tmem_free_cta(tmem_base, TMEM_COLS128);
 }
 
@@ -556,6 +571,7 @@ constexpr size_t decode128_smem(bool counts) { return (size_t)S * XSD * 4 + 16 +
 template <bool SIGNS>
 __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeArgs a)
 {
+    const StreamOrder order(a.wait_first);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *St = reinterpret_cast<float *>(smem_raw);  // [128*132] aggregate / intermediate; later the x tile [128*128]
     float *Xt = St;
@@ -579,7 +595,8 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
     const bool counts = a.agg == 2;
     const char *acquired = nullptr;
 
-    for (long long c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
+    volatile unsigned *next_slot = reinterpret_cast<volatile unsigned *>(bar_mem + 1);
+    for (long long c = blockIdx.x; c < a.n_chunks; c = (long long)gridDim.x + *next_slot) {
         cur.seek(a.entries, a.n_entries, c);
         const DemoTensorEntry te = cur.te;
         const unsigned lc = (unsigned)(c - te.chunk_begin);
@@ -665,13 +682,18 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                     for (int n = 0; n < H; ++n) St[n * XSD + j] = out[n];
                 }
                 __syncthreads();
-            } else if (!SIGNS) {
+            } else if (SIGNS) {
+                if (tid == 0) *next_slot = ticket_draw(a.tickets);
+            } else {
+                unsigned ticket = 0;  // (thread 0) the CTA's next chunk, drawn behind the wait for the tile
                 if (tid == 0) {
+                    ticket = ticket_draw(a.tickets);
                     mbar_expect_tx(bar, M * sizeof(float));
                     tma_load_2d(smem_u32(Xt), tm_x, k1 * S, k0 * S, bar);
                 }
                 arrived = mbar_wait_bounded(bar, phase);
                 phase ^= 1u;
+                if (tid == 0) *next_slot = ticket;
             }
         }
         if constexpr (SIGNS) {
@@ -687,7 +709,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         if (!__syncthreads_and(arrived)) {
             if (tid == 0) atomicMax(a.status, DEMO_DEV_TIMEOUT);
             mbar_wait_bounded(bar, phase ^ 1u);
-            return;
+            break;
         }
 #pragma unroll
         for (int n = 0; n < H; ++n) {
@@ -701,13 +723,15 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         fence_proxy_async();
         __syncthreads();
     }
+    if (tid == 0) ticket_finish(a.tickets);
 }
 
-template <typename K>
-cudaError_t launch128(K kernel, size_t smem, long long n_chunks, int sm_count, cudaStream_t stream, const void *args)
+template <typename K, typename A>
+cudaError_t launch128(K kernel, size_t smem, int sm_count, cudaStream_t stream, A args)
 {
+    const long long n_chunks = args.n_chunks;
     if (n_chunks <= 0) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t err = demo_allow_smem((const void *)kernel, smem);
     if (err != cudaSuccess) return err;
     // CTAs per SM: two by the launch bounds (registers), fewer if shared memory (227 KB, 1 KB reserved per CTA) says
     // so.  The occupancy calculator is not asked: it answers 1 for a kernel that allocates tensor memory.
@@ -716,8 +740,9 @@ cudaError_t launch128(K kernel, size_t smem, long long n_chunks, int sm_count, c
     if (per_sm < 1) per_sm = 1;
     long long grid = (long long)sm_count * per_sm;
     if (grid > n_chunks) grid = n_chunks;
-    void *params[] = {const_cast<void *>(args)};
-    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)grid), dim3(THREADS), params, smem, stream);
+    if (grid == n_chunks) args.tickets = nullptr;
+    void *params[] = {&args};
+    return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
 }
 
 }  // namespace
@@ -726,14 +751,13 @@ cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, int sm_count
 {
     if (!a.tmap_m || !a.tmap_g) return cudaErrorNotSupported;
     if (a.grad_bf16)
-        return launch128(compress_fast128_kernel<__nv_bfloat16>, compress128_smem<__nv_bfloat16>(), a.n_chunks, sm_count,
-                         stream, &a);
-    return launch128(compress_fast128_kernel<float>, compress128_smem<float>(), a.n_chunks, sm_count, stream, &a);
+        return launch128(compress_fast128_kernel<__nv_bfloat16>, compress128_smem<__nv_bfloat16>(), sm_count, stream, a);
+    return launch128(compress_fast128_kernel<float>, compress128_smem<float>(), sm_count, stream, a);
 }
 
 cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
-    if (a.sign_ptrs) return launch128(decode_fast128_kernel<true>, decode128_smem(a.agg == 2), a.n_chunks, sm_count, stream, &a);
+    if (a.sign_ptrs) return launch128(decode_fast128_kernel<true>, decode128_smem(a.agg == 2), sm_count, stream, a);
     if (!a.tmap_x) return cudaErrorNotSupported;
-    return launch128(decode_fast128_kernel<false>, decode128_smem(a.agg == 2), a.n_chunks, sm_count, stream, &a);
+    return launch128(decode_fast128_kernel<false>, decode128_smem(a.agg == 2), sm_count, stream, a);
 }

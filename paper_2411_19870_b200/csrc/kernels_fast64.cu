@@ -24,6 +24,7 @@
 #include "demo_internal.h"
 #include "fast_common.cuh"
 #include "fast_dct.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -61,9 +62,40 @@ constexpr size_t region_bytes()
 template <typename GT>
 constexpr size_t slot_bytes()
 {
-    constexpr size_t raw = region_bytes<GT>() + S * 4 + (CAP + 8) * 3 * 4 + 16 * 4 + 16;
+    constexpr size_t raw = region_bytes<GT>() + S * 4 + (CAP + 8) * 3 * 4 + 16 * 4 + 16 + 128;  // (last: SlotWalk)
     return (raw + 127) / 128 * 128;
 }
+
+// Thread 0's walk over the chunks: its place in the tensor table, and of the current and the next chunk (by turns) the tile
+// and the first record.  In shared memory rather than in registers, which every thread of the kernel would have to spare.
+struct SlotWalk {
+    DemoTensorEntry te;
+    long long next_begin;  // chunk_begin of the entry after te (or "never")
+    long long rec[2];
+    int e, acquired;       // entry of te; tensor whose maps were acquired last
+    int tensor[2], x[2], y[2];
+
+    __device__ __forceinline__ void load(const DemoTensorEntry *entries, int n)
+    {
+        te = entries[e];
+        next_begin = (e + 1 < n) ? entries[e + 1].chunk_begin : 0x7fffffffffffffffLL;
+    }
+    // Moves on to chunk c (ids only grow) and notes its tile and record offset in `slot`.
+    __device__ __forceinline__ void seek(const DemoTensorEntry *entries, int n, unsigned c, int k, int slot)
+    {
+        if (c >= next_begin) {
+            while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+            load(entries, n);
+        }
+        const unsigned lc = (unsigned)(c - te.chunk_begin);
+        const unsigned k0 = lc / (unsigned)te.c1;
+        tensor[slot] = te.tensor;
+        x[slot] = (int)(lc - k0 * (unsigned)te.c1) * S;
+        y[slot] = (int)k0 * S;
+        rec[slot] = te.rec_begin + (long long)lc * k;
+    }
+};
+static_assert(sizeof(SlotWalk) <= 128, "reserved in slot_bytes");
 
 // Shared memory of one slot.
 struct SlotMem {
@@ -772,6 +804,7 @@ __device__ __forceinline__ void select_chunk_big(const SlotMem &sm, float (&q)[S
 template <typename GT, int THREADS, bool QDOM, bool BIGK>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(DemoCompressArgs a)
 {
+    const StreamOrder order(a.wait_first);
     constexpr int NCH = THREADS / S;
     constexpr int NGROUPS = (THREADS + 127) / 128;                   // groups of four warps
     constexpr int TMEM_COLS = NGROUPS * TMEM_COLS_PER_GROUP < 32 ? 32 : NGROUPS * TMEM_COLS_PER_GROUP;
@@ -795,6 +828,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
     sm.recs4 = reinterpret_cast<int4 *>(sm.raw + region_bytes<GT>()) - 65;
     sm.misc = reinterpret_cast<unsigned *>(sm.cand_key + CAP + 8);
     unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(sm.misc + 16);
+    SlotWalk &walk = *reinterpret_cast<SlotWalk *>(bar_mem + 2);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_all + (size_t)NCH * slot_bytes<GT>());
     float *X = sm.X;
     int4 *recs4 = sm.recs4;
@@ -824,61 +858,69 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
     // this thread's lane of tensor memory (a warp reaches the 32 lanes of its quadrant) and its slot's columns
     const uint32_t taddr = tmem_base + ((uint32_t)((hw_warp & 3) * 32) << 16) + (uint32_t)((hw_warp >> 2) * TMEM_COLS_PER_GROUP);
 
-    EntryCursor cur;
-    const char *acquired = nullptr;  // (thread 0) the last tensor map made visible to the tensor-map proxy
     unsigned phase = 0;
+    const int k_eff = a.k;
+    const unsigned n_chunks = (unsigned)a.n_chunks;  // (fewer than 2^31)
 
-    // Tile of chunk c: tensor maps and box coordinates (the cursor is moved to c; chunk ids only grow).
-    struct TileRef {
-        const char *tm_m, *tm_g;
-        int x, y;
+    // (thread 0) the tensor maps of the chunk in walk slot `which`
+    auto map_of = [&](const void *maps, int which) {
+        return static_cast<const char *>(maps) + (size_t)walk.tensor[which] * TMAP_BYTES;
     };
-    auto locate = [&](long long c) {
-        cur.seek(a.entries, a.n_entries, c);
-        const unsigned lc = (unsigned)(c - cur.te.chunk_begin);
-        const unsigned k0 = lc / (unsigned)cur.te.c1;
-        const int k1 = (int)(lc - k0 * (unsigned)cur.te.c1);
-        TileRef r;
-        r.x = k1 * S;
-        r.y = (int)k0 * S;
-        r.tm_m = static_cast<const char *>(a.tmap_m) + (size_t)cur.te.tensor * TMAP_BYTES;
-        r.tm_g = static_cast<const char *>(a.tmap_g) + (size_t)cur.te.tensor * TMAP_BYTES;
-        return r;
-    };
-    // (thread 0) request the tiles of a chunk; a tensor map that this thread has not used yet is acquired first
-    auto issue_loads = [&](const TileRef &r) {
-        if (r.tm_m != acquired) {
-            acquired = r.tm_m;
-            tmap_acquire(r.tm_m);
-            tmap_acquire(r.tm_g);
+    // (thread 0) maps that this thread has not used yet are acquired before their first use
+    auto acquire_maps = [&](int which) {
+        if (walk.tensor[which] != walk.acquired) {
+            walk.acquired = walk.tensor[which];
+            tmap_acquire(map_of(a.tmap_m, which));
+            tmap_acquire(map_of(a.tmap_g, which));
         }
+    };
+    // (thread 0) request the tiles of a chunk
+    auto issue_loads = [&](int which) {
         mbar_expect_tx(bar, TILE_BYTES);
-        tma_load_2d(smem_u32(Ms), r.tm_m, r.x, r.y, bar);
-        tma_load_2d(smem_u32(Gs), r.tm_g, r.x, r.y, bar);
+        tma_load_2d(smem_u32(Ms), map_of(a.tmap_m, which), walk.x[which], walk.y[which], bar);
+        tma_load_2d(smem_u32(Gs), map_of(a.tmap_g, which), walk.x[which], walk.y[which], bar);
+    };
+    // (thread 0) the new momentum tile goes out, then -- once the store has read it -- the next chunk's tiles come in
+    auto store_and_load_next = [&](int which, bool more) {
+        tma_store_2d(map_of(a.tmap_m, which), walk.x[which], walk.y[which], smem_u32(Ms));
+        tma_store_commit();
+        tma_store_wait_read();
+        if (more) issue_loads(which ^ 1);
     };
 
-    const long long stride = (long long)gridDim.x * NCH;
-    long long c = (long long)blockIdx.x * NCH + slot;
-    TileRef next{};
-    if (c < a.n_chunks) {
-        next = locate(c);
-        if (t == 0) issue_loads(next);
+    static_assert(NCH == 1, "one slot per CTA draws the chunks");
+    unsigned c = blockIdx.x;
+    if (t == 0 && c < n_chunks) {
+        walk.e = demo_find_entry(a.entries, a.n_entries, c);
+        walk.acquired = -1;
+        walk.load(a.entries, a.n_entries);
+        walk.seek(a.entries, a.n_entries, c, k_eff, 0);
+        acquire_maps(0);
+        issue_loads(0);
+        // the slot's next chunk is always known one chunk ahead: the first two rounds are fixed, the rest is drawn
+        sm.misc[8] = a.tickets ? gridDim.x + c : NO_TICKET;
     }
+    sb.sync();
 
-    for (; c < a.n_chunks; c += stride) {
-        // the cursor points at chunk c (its loads were issued last)
-        const int k_eff = cur.te.k_eff;
-        DemoRecord *rec = a.payload + cur.te.rec_begin + (c - cur.te.chunk_begin) * (long long)k_eff;
-
+    int which = 0;  // walk slot of the current chunk
+    for (unsigned nc; c < n_chunks; c = nc, which ^= 1) {
+        // The next chunk is looked up while this chunk's tiles are on their way: the reads of the tensor table and, where the
+        // tensor changes, the acquisition of its maps (a fence of about a microsecond; in a set of 168 matrices of 1024
+        // columns it is due at nearly every chunk) cost nothing here.  Behind them thread 0 draws the chunk after it, which
+        // the others get to see behind the first transform.  (One call, fixed rounds with the look-up and the fences in front
+        // of the loads -> this: 300M-class decoder set 1134 -> 990 us, one matrix of 50304 x 20480 2313 -> 2134 us.)
+        nc = sm.misc[8];
+        unsigned ticket = 0;
+        if (t == 0 && nc < n_chunks) {
+            walk.seek(a.entries, a.n_entries, nc, k_eff, which ^ 1);
+            acquire_maps(which ^ 1);
+            ticket = 2u * gridDim.x + ticket_draw(a.tickets);
+        }
         // every thread waits for the tiles by itself; whether the wait expired is settled for the whole slot
         // at the first barrier of pass 0 (no barrier lies in between)
         const bool arrived = mbar_wait_bounded(bar, phase);
         phase ^= 1u;
         bool dead = false;
-        // where this chunk's tile goes back to and where the next one comes from (moves the cursor on)
-        const TileRef mine = next;
-        const long long nc = c + stride;
-        if (nc < a.n_chunks) next = locate(nc);
         // (No L2 prefetch of the next chunk's tiles: on a single launch it gains 0.5 %, but in a step that runs at the
         // board's power limit the extra L2 requests cost 1.4 %.)
 
@@ -960,6 +1002,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
                     constexpr int p = decltype(i)::value;
                     Xc[fdct::core_index<S>(p) * XS] = y[p];
                 });
+                if (t == 0) sm.misc[8] = nc < n_chunks ? ticket : NO_TICKET;  // (all have read the last one: the barrier above)
                 sb.sync();
             } else if (BIGK && !QDOM && ph == 2) {
                 fdct::F2 rp[S / 2];  // the row of the row-stage tile in pair order
@@ -995,15 +1038,11 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
                 sb.sync();
                 {
                     // the store of this chunk, then -- once it has read the tile -- the loads of the next chunk
-                    if (t == 0) {
-                        tma_store_2d(mine.tm_m, mine.x, mine.y, smem_u32(Ms));
-                        tma_store_commit();
-                        tma_store_wait_read();
-                        if (nc < a.n_chunks) issue_loads(next);
-                    }
+                    if (t == 0) store_and_load_next(which, nc < n_chunks);
                 }
             } else {
                 // ---- coefficients of row t: q[v] = Q[t][v] ------------------------------------------
+                DemoRecord *rec = a.payload + walk.rec[which];
                 float q[S];
                 fdct::static_for<0, S>([&](auto i) {
                     constexpr int p = decltype(i)::value;
@@ -1040,12 +1079,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
                     }
                     fence_proxy_async();
                     sb.sync();
-                    if (t == 0) {
-                        tma_store_2d(mine.tm_m, mine.x, mine.y, smem_u32(Ms));
-                        tma_store_commit();
-                        tma_store_wait_read();
-                        if (nc < a.n_chunks) issue_loads(next);
-                    }
+                    if (t == 0) store_and_load_next(which, nc < n_chunks);
                     continue;
                 }
                 if constexpr (BIGK) {
@@ -1089,6 +1123,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
         }
         if (dead) break;
     }
+    if (threadIdx.x == 0) ticket_finish(a.tickets);
     // tear-down: every slot of the CTA is done with its tensor-memory columns
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -1103,7 +1138,7 @@ cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t strea
     auto kernel = compress64_kernel<GT, THREADS, QDOM, BIGK>;
     const size_t smem = slot_bytes<GT>() * NCH + 16;
     if (a.n_chunks <= 0) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t err = demo_allow_smem((const void *)kernel, smem);
     if (err != cudaSuccess) return err;
     // CTAs per SM: registers (launch bounds: 512 threads per SM), shared memory (227 KB, 1 KB reserved per CTA)
     // and tensor memory (512 columns, 64 per four warps).  The occupancy calculator is not asked: it does not
@@ -1117,8 +1152,10 @@ cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t strea
     const long long groups = (a.n_chunks + NCH - 1) / NCH;
     long long grid = (long long)sm_count * per_sm;
     if (grid > groups) grid = groups;
-    kernel<<<(unsigned)grid, THREADS, smem, stream>>>(a);
-    return cudaGetLastError();
+    DemoCompressArgs b = a;
+    if (grid == groups) b.tickets = nullptr;
+    void *params[] = {&b};
+    return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
 }
 
 }  // namespace

@@ -70,6 +70,7 @@ __device__ __forceinline__ void inverse_dct(const float *Qt, float *tmp, float *
 template <int S>
 __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompressArgs a)
 {
+    const StreamOrder order(a.wait_first);
     constexpr int M = S * S;
     extern __shared__ float smem[];
     float *Bt = smem;
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompr
 template <int S>
 __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeArgs a)
 {
+    const StreamOrder order(a.wait_first);
     constexpr int M = S * S;
     extern __shared__ float smem[];
     float *St = smem;

@@ -31,6 +31,7 @@
 
 #include "demo_internal.h"
 #include "fast_dct.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -109,7 +110,7 @@ __device__ __forceinline__ int index_of(const DemoNdEntry &e, int t)
 struct Shared {
     DemoNdEntry e[2];  // current and next chunk, looked up by one thread a chunk ahead
     size_t base[2];
-    unsigned hi, n, n_kept, bound, thr, need_eq, n_eq, state[2], warp_tot[12];
+    unsigned ticket, hi, n, n_kept, bound, thr, need_eq, n_eq, state[2], warp_tot[12];
     unsigned hist[256], fine[256];
     uint2 cand[CAND];      // candidates (value bits, tile position) in no particular order
     uint4 kept[CAND / 2];  // the kept ones, two per entry
@@ -151,6 +152,14 @@ __device__ __forceinline__ void locate(Shared *w, int slot, const DemoNdEntry *e
             e = entries[find_nd_entry(entries, n_entries, c)];
     }
     w->base[slot] = chunk_base(e, (unsigned)(c - e.chunk_begin));
+}
+
+// (one thread) the chunk of a drawn ticket becomes the next one.
+__device__ __forceinline__ void take_ticket(Shared *w, int slot, const DemoNdEntry *entries, const DemoNdClass &cls, unsigned ticket)
+{
+    const long long c = (long long)gridDim.x + ticket;
+    if (c < cls.n_chunks) locate(w, slot, entries, cls.n, c);
+    w->ticket = ticket;
 }
 
 // (all threads) another layout than the previous chunk's: offsets of its rows; the tiles are cleared, because its padding
@@ -857,6 +866,7 @@ constexpr int MAX_THREADS = 384, MAX_THREADS_BIG = 256;
 template <typename GT, bool BIG>
 __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compress_nd_kernel(DemoNdCompressArgs a)
 {
+    const StreamOrder order(a.wait_first);
     const View v = carve(a.cls, true);
     Shared *s = shared();
     float *tile0 = v.tile0, *tile1 = v.tile1;
@@ -866,7 +876,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
     if (tid == 0 && blockIdx.x < a.cls.n_chunks) locate(s, 0, a.entries, a.cls.n, blockIdx.x);
     int layout = -1, slot = 0;
 
-    for (long long c = blockIdx.x; c < a.cls.n_chunks; c += gridDim.x, slot ^= 1) {
+    for (long long c = blockIdx.x; c < a.cls.n_chunks; c = (long long)gridDim.x + s->ticket, slot ^= 1) {
         // cleared for this chunk's selection; the barriers up to it order the writes
         for (int i = tid; i < 256; i += T) s->hist[i] = s->fine[i] = 0u;
         if (tid == 0) s->hi = 0u, s->n = 0u, s->n_kept = 0u;
@@ -877,7 +887,8 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
             enter_layout(v, e, a.cls);
             __syncthreads();
         }
-        if (tid == T - 1 && c + gridDim.x < a.cls.n_chunks) locate(s, slot ^ 1, a.entries, a.cls.n, c + gridDim.x);
+        unsigned ticket = 0;  // (last thread) the CTA's next chunk, drawn now, looked up below
+        if (tid == T - 1) ticket = ticket_draw(a.tickets);
         const size_t base = s->base[slot];
         float *__restrict__ m = a.m_ptrs[e.tensor] + base;
         const GT *__restrict__ g = static_cast<const GT *>(a.g_ptrs[e.tensor]) + base;
@@ -899,6 +910,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
                     tile0[t] = b;
                 });
         }
+        if (tid == T - 1) take_ticket(s, slot ^ 1, a.entries, a.cls, ticket);
         __syncthreads();
         transform_chunk<false, BIG>(tile0, tile1, slot, a.tables);  // Q = T(B; C_0, ..., C_{d-1})
         select_topk(tile0, slot, a.payload + e.rec_begin + (c - e.chunk_begin) * (long long)e.k_eff, a.alpha);
@@ -907,11 +919,13 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
         for_elements<4>(v, e, [](int, auto) {}, [&](int, int i, auto off, int t) { m[off] = v.B[i] - tile0[t]; });
         __syncthreads();
     }
+    if (tid == T - 1) ticket_finish(a.tickets);
 }
 
 template <bool BIG>
 __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode_nd_kernel(DemoNdDecodeArgs a)
 {
+    const StreamOrder order(a.wait_first);
     const View v = carve(a.cls, false);
     Shared *s = shared();
     float *tile0 = v.tile0, *tile1 = v.tile1;
@@ -925,7 +939,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
     if (tid == 0 && blockIdx.x < a.cls.n_chunks) locate(s, 0, a.entries, a.cls.n, blockIdx.x);
     int layout = -1, slot = 0;
 
-    for (long long c = blockIdx.x; c < a.cls.n_chunks; c += gridDim.x, slot ^= 1) {
+    for (long long c = blockIdx.x; c < a.cls.n_chunks; c = (long long)gridDim.x + s->ticket, slot ^= 1) {
         __syncthreads();
         const DemoNdEntry &e = s->e[slot];
         if (e.layout != layout) {
@@ -933,7 +947,8 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
             enter_layout(v, e, a.cls);
             __syncthreads();
         }
-        if (tid == T - 1 && c + gridDim.x < a.cls.n_chunks) locate(s, slot ^ 1, a.entries, a.cls.n, c + gridDim.x);
+        unsigned ticket = 0;  // (last thread) the CTA's next chunk, drawn now, looked up below
+        if (tid == T - 1) ticket = ticket_draw(a.tickets);
         const size_t base = s->base[slot];
         const int M = e.M, k_eff = e.k_eff;
         const long long rec_off = e.rec_begin + (c - e.chunk_begin) * (long long)k_eff;
@@ -941,6 +956,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
         for (int i = tid; i < e.tile >> 2; i += T) reinterpret_cast<float4 *>(tile0)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (counts)
             for (int i = tid; i < M; i += T) Cn[i] = 0;
+        if (tid == T - 1) take_ticket(s, slot ^ 1, a.entries, a.cls, ticket);
         // S = sum over workers, in worker order: batches of records are staged by all threads, the first warp adds them
         // worker after worker (indices are unique inside one worker's chunk)
         auto add = [&](int idx, float val) {
@@ -1009,22 +1025,22 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
                 x[off] = fmaf(-a.lr, fmaf(a.wd, xv[j], sg), xv[j]);
             });
     }
+    if (tid == T - 1) ticket_finish(a.tickets);
 }
 
-template <typename K>
-cudaError_t launch_nd(K kernel, size_t smem, const DemoNdClass &cls, int sm_count, cudaStream_t stream, const void *args)
+template <typename K, typename A>
+cudaError_t launch_nd(K kernel, size_t smem, int sm_count, cudaStream_t stream, A args)
 {
+    const DemoNdClass &cls = args.cls;
     if (cls.n_chunks <= 0) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, cls.threads, smem);
+    const cudaError_t err = demo_resident_ctas((const void *)kernel, cls.threads, smem, &per_sm);
     if (err != cudaSuccess) return err;
-    if (per_sm < 1) per_sm = 1;
     long long grid = (long long)sm_count * per_sm;
     if (grid > cls.n_chunks) grid = cls.n_chunks;
-    void *params[] = {const_cast<void *>(args)};
-    return cudaLaunchKernel((const void *)kernel, dim3((unsigned)grid), dim3((unsigned)cls.threads), params, smem, stream);
+    if (grid == cls.n_chunks) args.tickets = nullptr;
+    void *params[] = {&args};
+    return demo_launch_kernel((const void *)kernel, grid, cls.threads, smem, stream, params);
 }
 
 }  // namespace
@@ -1220,15 +1236,15 @@ cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, c
 {
     const size_t smem = shared_bytes(a.cls, true);
     if (a.cls.big)
-        return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, true>, smem, a.cls, sm_count, stream, &a)
-                           : launch_nd(compress_nd_kernel<float, true>, smem, a.cls, sm_count, stream, &a);
-    return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, false>, smem, a.cls, sm_count, stream, &a)
-                       : launch_nd(compress_nd_kernel<float, false>, smem, a.cls, sm_count, stream, &a);
+        return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, true>, smem, sm_count, stream, a)
+                           : launch_nd(compress_nd_kernel<float, true>, smem, sm_count, stream, a);
+    return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, false>, smem, sm_count, stream, a)
+                       : launch_nd(compress_nd_kernel<float, false>, smem, sm_count, stream, a);
 }
 
 cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
     const size_t smem = shared_bytes(a.cls, false) + (a.agg == 2 ? align16((size_t)a.cls.max_M * 2) : 0);
-    return a.cls.big ? launch_nd(decode_nd_kernel<true>, smem, a.cls, sm_count, stream, &a)
-                     : launch_nd(decode_nd_kernel<false>, smem, a.cls, sm_count, stream, &a);
+    return a.cls.big ? launch_nd(decode_nd_kernel<true>, smem, sm_count, stream, a)
+                     : launch_nd(decode_nd_kernel<false>, smem, sm_count, stream, a);
 }

@@ -1,12 +1,12 @@
-// Kernels for the small chunks: length-s segments of 1-D tensors (any s and basis; one warp per segment) and s x s tiles with
+// Kernels for the small chunks: length-s segments of 1-D tensors (any s and basis; a thread per element) and s x s tiles with
 // s in {8, 16} (s lanes per tile, 4 or 2 tiles per warp).  A launch takes both lists: the tensors of a small model are done in
 // one launch per call, and the norm vectors of a large one beside its tiles.
 //
 // What bounds them is latency: a chunk holds 8 to 256 elements, so nothing is gained by more threads per chunk (the dense
 // kernels, a 256-thread CTA per chunk with radix select and a barrier between all steps, spent 24 us on 2048 tiles of 8 x 8
-// and 13 us on 1024 segments), and a warp needs no block barrier from the loads to the stores:
-//   * segments: every lane forms s/32 coefficients by reading rows of the basis through L1 (the sums run over n in order, so
-//     the results are those of the dense kernels bit for bit); keys in registers, the k-th by a bit-by-bit ballot search;
+// and 13 us on 1024 segments), and a warp needs (almost) no block barrier from the loads to the stores:
+//   * segments: every thread forms one coefficient by reading its row of the basis through L1 (the sums run over n in order,
+//     so the results are those of the dense kernels bit for bit); the k-th key by a bit-by-bit ballot search;
 //   * tiles: lane j holds column j, then row j, in registers (fast_dct.cuh); the transposes go through a tile of the
 //     warp's own shared memory; the k-th key by a bit-by-bit search with counts added up over the tile's lanes.
 // Measured: 256 x 512 in 8 x 8 tiles plus a vector of 512, two compress calls and a decode: 60.7 -> 30.4 us (the tiles and
@@ -17,6 +17,7 @@
 
 #include "demo_internal.h"
 #include "fast_dct.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -40,80 +41,80 @@ __device__ __forceinline__ int find_entry_warp(const DemoTensorEntry *entries, i
 }
 
 // ---- segments -------------------------------------------------------------------------------------------
-// Lane l holds elements l, l + 32, ... (E = s/32 of them, one for s < 32, where the upper lanes idle).
+// Thread i of a segment holds element i: a warp for s <= 32 (lanes above s idle), two for s = 64, a block for s = 128.  Where a
+// segment has several warps, each holds all keys (E per lane) and searches for itself; three barriers order the exchange.
 template <int S>
 struct Seg {
-    static constexpr int E = S < 32 ? 1 : S / 32;
+    static constexpr int E = S < 32 ? 1 : S / 32;             // warps per segment = keys per lane
+    static constexpr int PER_BLOCK = THREADS / (32 * E);
     static constexpr int PAD = S + 4;
+    static __device__ __forceinline__ void sync()
+    {
+        if constexpr (E == 1)
+            __syncwarp();
+        else
+            __syncthreads();
+    }
 };
 
-// r[n] = sum_u C[u][n] line[u], u in order.
+// sum_u C[u][i] line[u], u in order.
 template <int S>
-__device__ __forceinline__ void inverse_segment(const float *line, const float *__restrict__ C, float (&r)[Seg<S>::E], int lane)
+__device__ __forceinline__ float inverse_segment(const float *line, const float *__restrict__ C, int i)
 {
-    constexpr int E = Seg<S>::E;
-#pragma unroll
-    for (int e = 0; e < E; ++e) r[e] = 0.f;
-    if (lane >= S) return;
-#pragma unroll 8
-    for (int u = 0; u < S; ++u) {
-        const float q = line[u];
-#pragma unroll
-        for (int e = 0; e < E; ++e) r[e] = fmaf(q, __ldg(C + u * S + lane + 32 * e), r[e]);
-    }
+    float r = 0.f;
+#pragma unroll 16
+    for (int u = 0; u < S; ++u) r = fmaf(line[u], __ldg(C + u * S + i), r);
+    return r;
 }
 
 template <int S>
-__device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long long c, float *line)
+__device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long long c_own, float *line)
 {
     constexpr int E = Seg<S>::E;
-    const int lane = threadIdx.x & 31;
-    const bool on = lane < S;
+    const int lane = threadIdx.x & 31, i = threadIdx.x % (32 * E);  // (i >= s only for s < 32)
+    const bool valid = c_own < a.n_chunks, on = i < S && valid;
+    const long long c = valid ? c_own : a.n_chunks - 1;
     const DemoTensorEntry te = a.entries[find_entry_warp(a.entries, a.n_entries, c)];
     const long long lc = c - te.chunk_begin;
-    const size_t base = (size_t)lc * S + lane;
+    const size_t off = (size_t)lc * S + i;
     float *__restrict__ m = a.m_ptrs[te.tensor];
     const void *g = a.g_ptrs[te.tensor];
     const int k = te.k_eff;
 
     // momentum update  b = beta*m + g  (Algorithm 1, worker side)
-    float b[E], q[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        b[e] = 0.f;
-        if (on) {
-            const size_t off = base + 32 * e;
-            const float gv = a.grad_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(g)[off])
-                                         : static_cast<const float *>(g)[off];
-            b[e] = fmaf(a.beta, m[off], gv);
-            line[lane + 32 * e] = b[e];
-        }
-        q[e] = 0.f;
-    }
-    __syncwarp();
-    // q = C b
+    float b = 0.f, q = 0.f;
     if (on) {
-#pragma unroll 4
+        const float gv = a.grad_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(g)[off]) : static_cast<const float *>(g)[off];
+        b = fmaf(a.beta, m[off], gv);
+    }
+    if (i < S) line[i] = b;
+    Seg<S>::sync();
+    // q = C b
+    if (i < S) {
+#pragma unroll 8
         for (int n = 0; n < S; n += 4) {
             const float4 x = *reinterpret_cast<const float4 *>(line + n);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const float4 t = __ldg(reinterpret_cast<const float4 *>(a.C + (lane + 32 * e) * S + n));
-                q[e] = fmaf(x.x, t.x, q[e]);
-                q[e] = fmaf(x.y, t.y, q[e]);
-                q[e] = fmaf(x.z, t.z, q[e]);
-                q[e] = fmaf(x.w, t.w, q[e]);
-            }
+            const float4 t = __ldg(reinterpret_cast<const float4 *>(a.C + i * S + n));
+            q = fmaf(x.x, t.x, q);
+            q = fmaf(x.y, t.y, q);
+            q = fmaf(x.z, t.z, q);
+            q = fmaf(x.w, t.w, q);
         }
     }
-    __syncwarp();
+    Seg<S>::sync();
     // exact top-k: threshold by ballots from the highest bit any key has; keys equal to it are kept in index order
     unsigned key[E], hi = 0u;
+    if constexpr (E == 1) {
+        key[0] = i < S ? mag_key(q) : 0u;
+    } else {
+        line[i] = q;
+        Seg<S>::sync();
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        key[e] = on ? mag_key(q[e]) : 0u;
-        hi = max(hi, key[e]);
+        for (int e = 0; e < E; ++e) key[e] = mag_key(line[lane + 32 * e]);
+        Seg<S>::sync();
     }
+#pragma unroll
+    for (int e = 0; e < E; ++e) hi = max(hi, key[e]);
     unsigned thr = 0u;
     int need_eq = S;  // k = s: everything is kept
     if (k < S) {
@@ -135,104 +136,88 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
         for (int e = 0; e < E; ++e) n_gt += __popc(__ballot_sync(FULL, key[e] > thr));
         need_eq = k - n_gt;
     }
-    DemoRecord *rec = a.payload + te.rec_begin + lc * (long long)k;
+    // this thread's own key is key[i / 32]: how many are kept, and equal, before it
     const unsigned lt = (1u << lane) - 1u;
-    int gt_before = 0, eq_before = 0;
+    const unsigned own = mag_key(q);
+    int gt = 0, eq = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const unsigned gtb = __ballot_sync(FULL, on && key[e] > thr), eqb = __ballot_sync(FULL, on && key[e] == thr);
-        const int eq = eq_before + __popc(eqb & lt);
-        const bool keep = on && (key[e] > thr || (key[e] == thr && eq < need_eq));
-        if (keep) {
-            DemoRecord r;
-            r.idx = lane + 32 * e;
-            r.val = q[e];
-            rec[gt_before + __popc(gtb & lt) + min(eq, need_eq)] = r;
-        }
-        if (on) line[lane + 32 * e] = keep ? a.alpha * q[e] : 0.f;
-        gt_before += __popc(gtb);
-        eq_before += __popc(eqb);
+        const bool elem = lane + 32 * e < S;
+        const unsigned gtb = __ballot_sync(FULL, elem && key[e] > thr), eqb = __ballot_sync(FULL, elem && key[e] == thr);
+        const unsigned below = e < i / 32 ? FULL : (e == i / 32 ? lt : 0u);
+        gt += __popc(gtb & below);
+        eq += __popc(eqb & below);
     }
-    __syncwarp();
+    const bool keep = i < S && (own > thr || (own == thr && eq < need_eq));
+    if (keep && valid) {
+        DemoRecord r;
+        r.idx = i;
+        r.val = q;
+        a.payload[te.rec_begin + lc * (long long)k + gt + min(eq, need_eq)] = r;
+    }
+    if (i < S) line[i] = keep ? a.alpha * q : 0.f;
+    Seg<S>::sync();
     // m <- b - alpha C^T (kept)
-    float r[E];
-    inverse_segment<S>(line, a.C, r, lane);
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (on) m[base + 32 * e] = b[e] - r[e];
-    __syncwarp();
+    if (on) m[off] = b - inverse_segment<S>(line, a.C, i);
+    Seg<S>::sync();
 }
 
 template <int S>
-__device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long long c, float *line, unsigned short *senders)
+__device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long long c_own, float *line, unsigned short *senders)
 {
     constexpr int E = Seg<S>::E;
-    const int lane = threadIdx.x & 31;
-    const bool on = lane < S, counts = a.agg == 2;
+    const int i = threadIdx.x % (32 * E);
+    const bool counts = a.agg == 2;
+    const bool valid = c_own < a.n_chunks, on = i < S && valid;
+    const long long c = valid ? c_own : a.n_chunks - 1;
     const DemoTensorEntry te = a.entries[find_entry_warp(a.entries, a.n_entries, c)];
     const long long lc = c - te.chunk_begin;
-    const size_t base = (size_t)lc * S + lane;
+    const size_t off = (size_t)lc * S + i;
     const int k = te.k_eff;
-    const long long rec_off = te.rec_begin + lc * (long long)k;
+    const long long rec_off = te.rec_begin + lc * (long long)k + i;
+    if (i < S) {
+        line[i] = 0.f;
+        if (counts) senders[i] = 0;
+    }
+    Seg<S>::sync();
+    // sum over workers in worker order (a segment has at most as many records as threads); eight workers' records are
+    // fetched together
+    for (int w0 = 0; w0 < a.W; w0 += 8) {
+        DemoRecord rc[8];
 #pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (on) {
-            line[lane + 32 * e] = 0.f;
-            if (counts) senders[lane + 32 * e] = 0;
-        }
-    __syncwarp();
-    // sum over workers in worker order; eight records per lane are fetched together
-    constexpr int WB = 8 / E;
-    for (int w0 = 0; w0 < a.W; w0 += WB) {
-        DemoRecord rc[WB][E];
+        for (int w = 0; w < 8; ++w) rc[w] = (i < k && w0 + w < a.W) ? a.payloads[w0 + w][rec_off] : DemoRecord{-1, 0.f};
 #pragma unroll
-        for (int w = 0; w < WB; ++w)
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                rc[w][e] = (lane + 32 * e < k && w0 + w < a.W) ? a.payloads[w0 + w][rec_off + lane + 32 * e] : DemoRecord{-1, 0.f};
-#pragma unroll
-        for (int w = 0; w < WB; ++w) {
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                if (lane + 32 * e < k && w0 + w < a.W) {
-                    if ((unsigned)rc[w][e].idx < (unsigned)S) {
-                        line[rc[w][e].idx] += rc[w][e].val;
-                        if (counts) senders[rc[w][e].idx] += 1;
-                    } else {
-                        atomicMax(a.status, DEMO_DEV_PAYLOAD);
-                    }
+        for (int w = 0; w < 8; ++w) {
+            if (i < k && w0 + w < a.W) {
+                if ((unsigned)rc[w].idx < (unsigned)S) {
+                    line[rc[w].idx] += rc[w].val;
+                    if (counts) senders[rc[w].idx] += 1;
+                } else if (valid) {
+                    atomicMax(a.status, DEMO_DEV_PAYLOAD);
                 }
             }
-            __syncwarp();
+            if (w0 + w < a.W) Seg<S>::sync();
         }
     }
     if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            if (on) {
-                const unsigned short n = senders[lane + 32 * e];
-                if (n > 1) line[lane + 32 * e] = line[lane + 32 * e] / (float)n;
-            }
-        __syncwarp();
+        if (i < S) {
+            const unsigned short n = senders[i];
+            if (n > 1) line[i] = line[i] / (float)n;
+        }
+        Seg<S>::sync();
     }
-    float r[E];
-    inverse_segment<S>(line, a.C, r, lane);
     if (on) {
+        const float r = inverse_segment<S>(line, a.C, i);
         if (a.sign_ptrs) {
-            signed char *__restrict__ sg = a.sign_ptrs[te.tensor];
-#pragma unroll
-            for (int e = 0; e < E; ++e) sg[base + 32 * e] = (signed char)((r[e] > 0.f) - (r[e] < 0.f));
+            a.sign_ptrs[te.tensor][off] = (signed char)((r > 0.f) - (r < 0.f));
         } else {
             float *__restrict__ x = a.x_ptrs[te.tensor];
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const float sg = a.phi ? r[e] * a.agg_scale : (float)((r[e] > 0.f) - (r[e] < 0.f));
-                const float xv = x[base + 32 * e];
-                x[base + 32 * e] = fmaf(-a.lr, fmaf(a.wd, xv, sg), xv);
-            }
+            const float sg = a.phi ? r * a.agg_scale : (float)((r > 0.f) - (r < 0.f));
+            const float xv = x[off];
+            x[off] = fmaf(-a.lr, fmaf(a.wd, xv, sg), xv);
         }
     }
-    __syncwarp();
+    Seg<S>::sync();
 }
 
 // ---- tiles of 8 x 8 and 16 x 16 ----------------------------------------------------------------------------
@@ -478,11 +463,15 @@ constexpr int warp_floats() { return TILES && Tile<S>::FLOATS > Seg<S>::PAD ? Ti
 template <int S, typename GT, bool TILES>
 __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArgs segs, DemoCompressArgs tiles, int seg_blocks)
 {
+    const StreamOrder order(segs.wait_first);
     __shared__ __align__(16) float mem[WARPS][warp_floats<S, TILES>()];
     const int warp = threadIdx.x >> 5;
     if (!TILES || (int)blockIdx.x < seg_blocks) {
-        for (long long c = (long long)blockIdx.x * WARPS + warp; c < segs.n_chunks; c += (long long)seg_blocks * WARPS)
-            compress_segment<S>(segs, c, mem[warp]);
+        // (all threads of a block make the same rounds: a segment beyond the last is computed and not stored)
+        constexpr int PB = Seg<S>::PER_BLOCK;
+        const int own = warp / Seg<S>::E;
+        for (long long c0 = (long long)blockIdx.x * PB; c0 < segs.n_chunks; c0 += (long long)seg_blocks * PB)
+            compress_segment<S>(segs, c0 + own, mem[own]);
     } else if constexpr (TILES) {
         const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
         const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
@@ -494,12 +483,16 @@ __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArg
 template <int S, bool TILES>
 __global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs segs, DemoDecodeArgs tiles, int seg_blocks)
 {
+    const StreamOrder order(segs.wait_first);
     __shared__ __align__(16) float mem[WARPS][warp_floats<S, TILES>()];
     __shared__ unsigned short counts[WARPS][TILES ? Tile<S>::PER_WARP * S * S : S];
     const int warp = threadIdx.x >> 5;
     if (!TILES || (int)blockIdx.x < seg_blocks) {
-        for (long long c = (long long)blockIdx.x * WARPS + warp; c < segs.n_chunks; c += (long long)seg_blocks * WARPS)
-            decode_segment<S>(segs, c, mem[warp], counts[warp]);
+        // (all threads of a block make the same rounds: a segment beyond the last is computed and not stored)
+        constexpr int PB = Seg<S>::PER_BLOCK;
+        const int own = warp / Seg<S>::E;
+        for (long long c0 = (long long)blockIdx.x * PB; c0 < segs.n_chunks; c0 += (long long)seg_blocks * PB)
+            decode_segment<S>(segs, c0 + own, mem[own], counts[own]);
     } else if constexpr (TILES) {
         const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
         const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
@@ -508,22 +501,22 @@ __global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs se
     }
 }
 
-// One warp per segment or group of tiles, up to eight blocks per SM for each list (what 64 registers per thread allow).
-int blocks_for(long long warps, int sm_count)
+// Up to eight blocks per SM for each list (what 64 registers per thread allow).
+int blocks_for(long long units, int per_block, int sm_count)
 {
-    const long long b = (warps + WARPS - 1) / WARPS, cap = 8LL * sm_count;
+    const long long b = (units + per_block - 1) / per_block, cap = 8LL * sm_count;
     return (int)(b < cap ? b : cap);
 }
 template <class A>
-cudaError_t launch(const void *kernel, int per_warp, const A *segs, const A *tiles, int sm_count, cudaStream_t stream)
+cudaError_t launch(const void *kernel, int segs_per_block, int tiles_per_warp, const A *segs, const A *tiles, int sm_count, cudaStream_t stream)
 {
     A none{};
     const A &sa = segs ? *segs : none, &ta = tiles ? *tiles : none;
-    int seg_blocks = segs ? blocks_for(sa.n_chunks, sm_count) : 0;
-    const int tile_blocks = tiles ? blocks_for((ta.n_chunks + per_warp - 1) / per_warp, sm_count) : 0;
+    int seg_blocks = segs ? blocks_for(sa.n_chunks, segs_per_block, sm_count) : 0;
+    const int tile_blocks = tiles ? blocks_for(ta.n_chunks, tiles_per_warp * WARPS, sm_count) : 0;
     if (seg_blocks + tile_blocks == 0) return cudaSuccess;
     void *params[] = {const_cast<A *>(&sa), const_cast<A *>(&ta), &seg_blocks};
-    return cudaLaunchKernel(kernel, dim3((unsigned)(seg_blocks + tile_blocks)), dim3(THREADS), params, 0, stream);
+    return demo_launch_kernel(kernel, seg_blocks + tile_blocks, THREADS, 0, stream, params);
 }
 
 template <int S>
@@ -533,18 +526,18 @@ cudaError_t compress_small(const DemoCompressArgs *segs, const DemoCompressArgs 
         if (tiles)
             return launch(tiles->grad_bf16 ? (const void *)compress_small_kernel<S, __nv_bfloat16, true>
                                            : (const void *)compress_small_kernel<S, float, true>,
-                          Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
+                          Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
     }
-    return launch((const void *)compress_small_kernel<S, float, false>, 1, segs, (const DemoCompressArgs *)nullptr, sm_count, stream);
+    return launch((const void *)compress_small_kernel<S, float, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoCompressArgs *)nullptr, sm_count, stream);
 }
 template <int S>
 cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count, cudaStream_t stream)
 {
     if constexpr (S <= 16) {
         if (tiles)
-            return launch((const void *)decode_small_kernel<S, true>, Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
+            return launch((const void *)decode_small_kernel<S, true>, Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
     }
-    return launch((const void *)decode_small_kernel<S, false>, 1, segs, (const DemoDecodeArgs *)nullptr, sm_count, stream);
+    return launch((const void *)decode_small_kernel<S, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, sm_count, stream);
 }
 
 }  // namespace

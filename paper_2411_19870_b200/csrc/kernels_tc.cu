@@ -25,6 +25,7 @@
 
 #include "demo_internal.h"
 #include "fast_common.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -313,6 +314,7 @@ __device__ __forceinline__ void write_own_row(float *T, int r, const float *v)
 
 __global__ void __launch_bounds__(TC_THREADS, 1) compress_tc_kernel(DemoCompressArgs a)
 {
+    const StreamOrder order(a.wait_first);
     extern __shared__ unsigned char smem_raw[];
     TcFrame f;
     tc_setup(f, smem_raw, a.C, true);
@@ -566,6 +568,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) compress_tc_kernel(DemoCompress
 
 __global__ void __launch_bounds__(TC_THREADS, 1) decode_tc_kernel(DemoDecodeArgs a)
 {
+    const StreamOrder order(a.wait_first);
     extern __shared__ unsigned char smem_raw[];
     TcFrame f;
     tc_setup(f, smem_raw, a.C, false);
@@ -665,12 +668,12 @@ template <typename K, typename A>
 cudaError_t launch_tc(K kernel, const A &a, int sm_count, cudaStream_t stream)
 {
     if (a.n_chunks <= 0) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES);
+    const cudaError_t err = demo_allow_smem((const void *)kernel, TC_SMEM_BYTES);
     if (err != cudaSuccess) return err;
     const long long n_ctas = ((a.n_chunks + 1) / 2 + GROUPS - 1) / GROUPS;
     const long long grid = n_ctas < sm_count ? n_ctas : sm_count;  // one CTA per SM owns the tensor memory it needs
-    kernel<<<(unsigned)grid, TC_THREADS, TC_SMEM_BYTES, stream>>>(a);
-    return cudaGetLastError();
+    void *params[] = {const_cast<A *>(&a)};
+    return demo_launch_kernel((const void *)kernel, grid, TC_THREADS, TC_SMEM_BYTES, stream, params);
 }
 
 }  // namespace
