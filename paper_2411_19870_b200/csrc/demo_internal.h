@@ -55,6 +55,7 @@ struct DemoDecodeArgs {
     const DemoTensorEntry *entries;
     int n_entries;
     long long n_chunks;
+    int k = 0;                          // k_eff of the list's tensors
     const DemoRecord *const *payloads;  // device array [W]
     int W;
     float *const *x_ptrs;  // device array

@@ -787,6 +787,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.entries = ctx->d_entries2d;
     a.n_entries = ctx->n2d;
     a.n_chunks = ctx->chunks2d;
+    a.k = ctx->cfg.topk;  // <= s * s
     a.tickets = ctx->d_tickets;
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     if (ctx->n2d && !small_tiles) {

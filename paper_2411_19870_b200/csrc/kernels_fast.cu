@@ -761,18 +761,52 @@ constexpr int STAGE_RECORDS = 512;  // records staged per batch of the scatter (
 template <int S>
 __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)
 {
-    return ((size_t)S * Cfg<S>::XS * 4 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + (counts ? (size_t)S * S * 2 : 0) + 127) /
+    return ((size_t)S * Cfg<S>::XS * 4 + 128 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + (counts ? (size_t)S * S * 2 : 0) + 127) /
            128 * 128;
 }
 
+// A slot's walk over its chunks, kept by its thread 0 in shared memory (in registers every thread would have to spare them):
+// its place in the tensor table, and of the current and the next chunk (by turns) the first element, the row length and
+// the first record.
+struct DecodeWalk {
+    DemoTensorEntry te;
+    long long next_begin;  // chunk_begin of the entry after te (or "never")
+    long long rec[2];
+    long long elem[2];     // offset of the chunk's first element in its tensor
+    int e;
+    int tensor[2], n1[2];
+
+    __device__ __forceinline__ void load(const DemoTensorEntry *entries, int n)
+    {
+        te = entries[e];
+        next_begin = (e + 1 < n) ? entries[e + 1].chunk_begin : 0x7fffffffffffffffLL;
+    }
+    // Moves on to chunk c (ids only grow) and notes it in `which`.
+    template <int S>
+    __device__ __forceinline__ void seek(const DemoTensorEntry *entries, int n, long long c, int k, int which)
+    {
+        if (c >= next_begin) {
+            while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+            load(entries, n);
+        }
+        const unsigned lc = (unsigned)(c - te.chunk_begin);
+        const unsigned k0 = lc / (unsigned)te.c1;
+        tensor[which] = te.tensor;
+        n1[which] = te.n1;
+        elem[which] = ((long long)k0 * te.n1 + (lc - k0 * (unsigned)te.c1)) * S;
+        rec[which] = te.rec_begin + (long long)lc * k;
+    }
+};
+static_assert(sizeof(DecodeWalk) <= 128, "reserved in decode_slot_bytes");
+
 // SIGNS: the parameter-server form -- sign(R) goes out as int8 per element, the parameters are neither read
 // nor written (a separate instantiation, so that the update kernel keeps its size).
-// WIDE: the instantiation for fan-ins above one staging batch (sixteen workers at k <= 32): every further batch of a
-// chunk's workers is requested, like the first, while the scatter works on the batch before it.
+// The records of a chunk's workers come in batches of STAGE_RECORDS through two staging buffers, the first batch a chunk
+// ahead, every further one while the scatter works on the batch before it.
 // The x tile comes by 16-byte asynchronous copies, sixteen per thread, not by TMA: a tensor map has to be acquired by every
 // CTA that comes to a tensor, a fence that stands in front of the chunk (300M-class set, 168 matrices: 696 us with maps, 725
 // with a bulk copy per row, 624 like this; one matrix of that size: 612, 731, 597).
-template <int S, int THREADS, bool SIGNS = false, bool WIDE = false>
+template <int S, int THREADS, bool SIGNS = false>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -788,14 +822,13 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     // read back into registers -- the staging area of the x tile, fetched behind the second transform.
     float *St = reinterpret_cast<float *>(smem_raw);  // [S*XS]
     float *Xt = St;                                   // [S*S] (aliases St)
-    DemoRecord *stage_all = reinterpret_cast<DemoRecord *>(St + S * XS);    // [2][STAGE_RECORDS] records of a batch of workers
+    DecodeWalk &walk = *reinterpret_cast<DecodeWalk *>(St + S * XS);
+    DemoRecord *stage_all = reinterpret_cast<DemoRecord *>(reinterpret_cast<unsigned char *>(&walk) + 128);    // [2][STAGE_RECORDS] records of a batch of workers
     unsigned short *Cn = reinterpret_cast<unsigned short *>(stage_all + 2 * STAGE_RECORDS);  // [S*S] senders per coordinate (agg == 2)
 
     const int t = threadIdx.x % S;
 
-    EntryCursor cur;
-    float *x_ptr = nullptr;
-    int cached_tensor = -1;
+    const int k_eff = a.k;
     const unsigned lr_bits = __float_as_uint(a.lr);
     const float decay = 1.f - a.lr * a.wd;
     const float neg_lr_scale = -a.lr * a.agg_scale;
@@ -803,36 +836,20 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     // The records of a chunk's first batch of workers (up to STAGE_RECORDS records) are copied into one of two
     // staging buffers by asynchronous copies issued a whole chunk ahead, so that the payload reads of the W
     // workers -- W small pieces from W buffers -- never stand in front of the scatter.  One copy group per chunk.
-    auto stage_ahead = [&](int buf, long long chunk) {
-        cur.seek(a.entries, a.n_entries, chunk);
-        const int k_n = cur.te.k_eff;
-        if (k_n <= 64) {
-            const long long off_n = cur.te.rec_begin + (chunk - cur.te.chunk_begin) * (long long)k_n;
-            const int sh = (k_n > 32) ? 6 : 5;
+    // (The records of workers w_first .. of the chunk in walk slot `which`.)
+    auto stage_batch = [&](int buf, int which, int w_first) {
+        if (k_eff <= 64) {
+            const long long off = walk.rec[which];
+            const int sh = (k_eff > 32) ? 6 : 5;
             DemoRecord *dst = stage_all + buf * STAGE_RECORDS;
 #pragma unroll
             for (int i = 0; i < STAGE_RECORDS / S; ++i) {
-                const int r = i * S + t, wl = r >> sh, j = r & ((1 << sh) - 1);
-                if (wl < a.W && j < k_n)
+                const int r = i * S + t, wl = w_first + (r >> sh), j = r & ((1 << sh) - 1);
+                if (wl < a.W && j < k_eff)
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst + r)),
-                                 "l"(a.payloads[wl] + off_n + j)
+                                 "l"(a.payloads[wl] + off + j)
                                  : "memory");
             }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-
-    // (WIDE) a further batch of the same chunk: workers w_first .. of the chunk whose records start at off_n
-    auto stage_batch = [&](int buf, int k_n, long long off_n, int w_first) {
-        const int sh = (k_n > 32) ? 6 : 5;
-        DemoRecord *dst = stage_all + buf * STAGE_RECORDS;
-#pragma unroll
-        for (int i = 0; i < STAGE_RECORDS / S; ++i) {
-            const int r = i * S + t, wl = w_first + (r >> sh), j = r & ((1 << sh) - 1);
-            if (wl < a.W && j < k_n)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst + r)),
-                             "l"(a.payloads[wl] + off_n + j)
-                             : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -844,29 +861,24 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     if (threadIdx.x == 0) drawn[0] = ticket_draw(a.tickets);
     unsigned group = blockIdx.x, next_group, par = 0;
     long long c = (long long)group * NCH + slot;
-    int buf = 0;
-    if (c < a.n_chunks) stage_ahead(0, c);
-    for (; (long long)group * NCH < a.n_chunks; group = next_group, c = (long long)group * NCH + slot, par ^= 1u) {
-        __syncthreads();
+    int buf = 0, which = 0;  // staging buffer and walk slot of the current chunk
+    if (t == 0 && c < a.n_chunks) {
+        walk.e = demo_find_entry(a.entries, a.n_entries, c);
+        walk.load(a.entries, a.n_entries);
+        walk.seek<S>(a.entries, a.n_entries, c, k_eff, 0);
+    }
+    sb.sync();
+    if (c < a.n_chunks) stage_batch(0, 0, 0);
+    for (; (long long)group * NCH < a.n_chunks; group = next_group, c = (long long)group * NCH + slot, par ^= 1u, which ^= 1) {
+        __syncthreads();  // (publishes the draw; all slots start a chunk together)
         next_group = gridDim.x + drawn[par];  // (NO_TICKET ends the loop: groups are fewer than 2^31)
         if (c >= a.n_chunks) continue;
+        const bool more = (long long)next_group * NCH + slot < a.n_chunks;
         unsigned ticket = 0;
         if (threadIdx.x == 0) ticket = ticket_draw(a.tickets);
-        cur.seek(a.entries, a.n_entries, c);
-        const DemoTensorEntry te = cur.te;
-        if (te.tensor != cached_tensor) {
-            cached_tensor = te.tensor;
-            x_ptr = a.x_ptrs[cached_tensor];
-        }
-        const unsigned lc = (unsigned)(c - te.chunk_begin);
-        const unsigned k0 = lc / (unsigned)te.c1;
-        const int k1 = (int)(lc - k0 * (unsigned)te.c1);
-        const size_t base = (size_t)k0 * S * (size_t)te.n1 + (size_t)k1 * S;
-        float *__restrict__ x = x_ptr;
-        const int k_eff = te.k_eff;
-        const long long rec_off = te.rec_begin + lc * (long long)k_eff;
+        if (t == 0 && more) walk.seek<S>(a.entries, a.n_entries, (long long)next_group * NCH + slot, k_eff, which ^ 1);
         if (!SIGNS) {  // row t of the x tile on its way to L2
-            const float *xr = x + base + (size_t)t * te.n1;
+            const float *xr = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)t * walk.n1[which];
             asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
             if (S == 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 32));
         }
@@ -878,20 +890,14 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             if (counts)
                 for (int v = 0; v < S; ++v) Cn[t * S + v] = 0;
         }
-        auto stage_next_chunk = [&](int into) {  // (the cursor moves on; this chunk's table entry is in `te`)
-            const long long nc = (long long)next_group * NCH + slot;
-            if (nc < a.n_chunks)
-                stage_ahead(into, nc);
+        // (an empty group where there is no next chunk: the waits count groups)
+        auto stage_next_chunk = [&](int into) {
+            if (more)
+                stage_batch(into, which ^ 1, 0);
             else
                 asm volatile("cp.async.commit_group;" ::: "memory");
         };
         DemoRecord *stage = stage_all + buf * STAGE_RECORDS;
-        if (!WIDE || k_eff > 64) {
-            // next chunk's records on their way
-            stage_next_chunk(buf ^ 1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");  // this chunk's copies have landed
-            buf ^= 1;
-        }
         // S = sum over workers in worker order (Decompress&Aggregate).
         if (k_eff <= 64) {
             // Every warp owns the 32 rows of the tile its threads cleared and will transform (rows 32 w .. 32 w + 31
@@ -904,65 +910,62 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             const int sh = (k_eff > 32) ? 6 : 5;          // a worker's records take 32 or 64 staging entries
             const int wb = STAGE_RECORDS >> sh;           // workers per batch: 16 or 8
             for (int w0 = 0; w0 < a.W; w0 += wb) {
-                if (WIDE) {
-                    // both warps are done with the previous batch (between chunks the barrier at the end of a chunk
-                    // has seen to that): its buffer takes the batch after this one -- of this chunk's workers or,
-                    // behind the last, the first batch of the slot's next chunk
-                    if (w0 > 0) sb.sync();
-                    if (w0 + wb < a.W)
-                        stage_batch(buf ^ 1, k_eff, rec_off, w0 + wb);
-                    else
-                        stage_next_chunk(buf ^ 1);
-                    asm volatile("cp.async.wait_group 1;" ::: "memory");  // this batch's copies have landed
-                    stage = stage_all + buf * STAGE_RECORDS;
-                    buf ^= 1;
-                } else if (w0 > 0) {  // further batches of a large fan-in: fetched on the spot
-                    sb.sync();  // the previous batch has been consumed by both warps
-#pragma unroll 1
-                    for (int r = t; r < STAGE_RECORDS; r += S) {
-                        const int wl = r >> sh, j = r & ((1 << sh) - 1);
-                        if (w0 + wl < a.W && j < k_eff) stage[r] = a.payloads[w0 + wl][rec_off + j];
-                    }
-                }
-                sb.sync();  // staged records visible (also orders the clearing of the tile before the first additions)
+                // this batch's copies have landed (requested a chunk or a batch ago), for all threads; the tile is cleared, the
+                // next chunk looked up, and both warps are done with the other buffer: it takes the batch after this one --
+                // of this chunk's workers or, behind the last, the first batch of the slot's next chunk
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                sb.sync();
+                stage = stage_all + buf * STAGE_RECORDS;
+                buf ^= 1;
+                if (w0 + wb < a.W)
+                    stage_batch(buf, which, w0 + wb);
+                else
+                    stage_next_chunk(buf);
                 const int nw = min(wb, a.W - w0);
-                // (the next worker's record is read before this worker's addition, so that only the addition itself
-                // lies between two warp barriers)
+                // Four workers' records are read together, then added one worker after the other without a branch: a record
+                // of the other warp's rows goes to a place of this lane's own in the tile's padding (a bank of its own), so
+                // that a worker costs one dependent read-add-write.  Indices outside the chunk are noted and reported once.
+                // (4096 x 4096, W = 64: 73.8 us with branches around every record -> 63.8; W = 8: 32.5 -> 32.0.)
                 const bool two = k_eff > 32;
-                DemoRecord nx0 = stage[lane], nx1 = stage[two ? lane + 32 : lane];
+                const int spare = (32 * warp + lane) * XS + S + (lane >> 3);
+                bool bad = false;
+                auto add = [&](const DemoRecord &rc, bool have) {
+                    const unsigned idx = (unsigned)rc.idx;
+                    bad = bad || (have && idx >= (unsigned)M);
+                    const bool mine = have && (idx >> (C::LOG2S + 5)) == (unsigned)warp;  // (false for idx >= M)
+                    const int at = mine ? (int)(idx >> C::LOG2S) * XS + (int)(idx & (S - 1)) : spare;
+                    St[at] += rc.val;
+                    if (counts && mine) Cn[idx] += 1;
+                };
 #pragma unroll 1
-                for (int wl = 0; wl < nw; ++wl) {
-                    const DemoRecord rc0 = nx0, rc1 = nx1;
-                    if (wl + 1 < nw) {
-                        nx0 = stage[((wl + 1) << sh) + lane];
-                        if (two) nx1 = stage[((wl + 1) << sh) + lane + 32];
-                    }
-                    if (lane < k_eff) {
-                        if ((unsigned)rc0.idx < (unsigned)M) {
-                            if ((rc0.idx >> (C::LOG2S + 5)) == warp) {
-                                St[(rc0.idx >> C::LOG2S) * XS + (rc0.idx & (S - 1))] += rc0.val;
-                                if (counts) Cn[rc0.idx] += 1;
-                            }
-                        } else {
-                            atomicMax(a.status, DEMO_DEV_PAYLOAD);
+                for (int wl = 0; wl < nw;) {
+                    auto some = [&](auto count) {
+                        constexpr int U = decltype(count)::value;
+                        DemoRecord rc0[U], rc1[U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            rc0[u] = stage[((wl + u) << sh) + lane];
+                            if (two) rc1[u] = stage[((wl + u) << sh) + lane + 32];
                         }
-                    }
-                    if (two && lane + 32 < k_eff) {
-                        if ((unsigned)rc1.idx < (unsigned)M) {
-                            if ((rc1.idx >> (C::LOG2S + 5)) == warp) {
-                                St[(rc1.idx >> C::LOG2S) * XS + (rc1.idx & (S - 1))] += rc1.val;
-                                if (counts) Cn[rc1.idx] += 1;
-                            }
-                        } else {
-                            atomicMax(a.status, DEMO_DEV_PAYLOAD);
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            add(rc0[u], lane < k_eff);
+                            if (two) add(rc1[u], lane + 32 < k_eff);
+                            __syncwarp();
                         }
-                    }
-                    __syncwarp();
+                        wl += U;
+                    };
+                    if (wl + 4 <= nw)
+                        some(std::integral_constant<int, 4>{});
+                    else
+                        some(std::integral_constant<int, 1>{});
                 }
+                if (bad) atomicMax(a.status, DEMO_DEV_PAYLOAD);
             }
         } else {
             // k > 64: a thread's records may fall into any row; a barrier per worker fixes the order of additions.
             // Records are fetched eight workers ahead so that one memory latency covers eight workers.
+            const long long rec_off = walk.rec[which];
             sb.sync();
             for (int kb = 0; kb < k_eff; kb += S) {
                 const bool mine = kb + t < k_eff;
@@ -1016,12 +1019,13 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 sb.sync();  // the tile is dead: stage x into it
                 if (!SIGNS) {
                     constexpr int PIECES = S / 4;  // 16-byte pieces per row
-                    const float *src = x + base + (size_t)(t / PIECES) * te.n1 + (t % PIECES) * 4;
+                    const int n1 = walk.n1[which];
+                    const float *src = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)(t / PIECES) * n1 + (t % PIECES) * 4;
                     const uint32_t dst = smem_u32(Xt) + t * 16;
 #pragma unroll
                     for (int i = 0; i < PIECES; ++i)
                         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * (S * 16)),
-                                     "l"(src + (size_t)(i * (S / PIECES)) * te.n1)
+                                     "l"(src + (size_t)(i * (S / PIECES)) * n1)
                                      : "memory");
                     asm volatile("cp.async.commit_group;" ::: "memory");
                 }
@@ -1043,9 +1047,10 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             }
         }
         if constexpr (SIGNS) {
-            signed char *__restrict__ sg = a.sign_ptrs[te.tensor];
+            signed char *__restrict__ sg = a.sign_ptrs[walk.tensor[which]] + walk.elem[which] + t;
+            const size_t n1 = (size_t)walk.n1[which];
 #pragma unroll
-            for (int i = 0; i < S; ++i) sg[base + (size_t)i * te.n1 + t] = (signed char)((r[i] > 0.f) - (r[i] < 0.f));
+            for (int i = 0; i < S; ++i) sg[i * n1] = (signed char)((r[i] > 0.f) - (r[i] < 0.f));
             sb.sync();  // the tile is free again
             continue;
         }
@@ -1053,13 +1058,15 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         sb.sync();
         // sign and update:  x - lr (sign(R) + wd x) = x (1 - lr wd) - lr sign(R); -lr sign(R) is lr with
         // its sign flipped where R > 0, and zero where R == 0
+        float *__restrict__ x = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + t;
+        const size_t n1 = (size_t)walk.n1[which];
 #pragma unroll
         for (int i = 0; i < S; ++i) {
             const float rv = r[i];
             float stepv = __uint_as_float(lr_bits ^ (~__float_as_uint(rv) & 0x80000000u));
             stepv = (rv == 0.f) ? 0.f : stepv;
             if (a.phi) stepv = rv * neg_lr_scale;  // phi = identity: -lr * R (R / W for the mean)
-            x[base + (size_t)i * te.n1 + t] = fmaf(Xt[i * S + t], decay, stepv);
+            x[i * n1] = fmaf(Xt[i * S + t], decay, stepv);
         }
         sb.sync();  // the tile is free again
     }
@@ -1114,8 +1121,6 @@ cudaError_t launch_decode(const DemoDecodeArgs &a, int sm_count, cudaStream_t st
     constexpr int NCH = TH / S;
     const size_t smem = decode_slot_bytes<S>(a.agg == 2) * NCH;
     if (a.sign_ptrs != nullptr) return launch(decode_fast_kernel<S, TH, true>, TH, NCH, smem, sm_count, stream, a);
-    if (a.W > 16)  // more than one staging batch at k <= 32
-        return launch(decode_fast_kernel<S, TH, false, true>, TH, NCH, smem, sm_count, stream, a);
     return launch(decode_fast_kernel<S, TH>, TH, NCH, smem, sm_count, stream, a);
 }
 
