@@ -190,19 +190,20 @@ struct DemoNdDecodeArgs {
 
 // x <- x - lr (sign + wd x) from int8 signs, over every tensor of a context (kernels_generic.cu).
 struct DemoFlatEntry {
-    long long quad_begin;  // index of this tensor's first group of four elements in the launch
-    long long n;           // elements
-    int tensor;            // position in the pointer arrays
+    long long piece_begin;  // index of this tensor's first piece of demo_apply_piece() elements in the launch
+    long long n;            // elements
+    int tensor;             // position in the pointer arrays
     int pad;
 };
 struct DemoApplySignsArgs {
     const DemoFlatEntry *entries;  // device
     int n_entries;
-    long long n_quads;
+    long long n_pieces;
     const signed char *const *sign_ptrs;  // device array
     float *const *x_ptrs;                 // device array
     float lr, wd;
 };
+int demo_apply_piece();
 cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, cudaStream_t stream);
 
 cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, cudaStream_t stream);

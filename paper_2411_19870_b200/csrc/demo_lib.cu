@@ -60,7 +60,7 @@ struct demo_ctx {
     std::vector<signed char *> h_s;
     bool s_valid = false;
     DemoFlatEntry *d_flat = nullptr;   // [T] element ranges for demo_apply_signs
-    long long n_quads = 0;
+    long long n_pieces = 0;
     std::vector<const void *> h_g;
     std::vector<float *> h_m, h_x;
     std::vector<const DemoRecord *> h_p;
@@ -670,13 +670,13 @@ static demo_status ensure_sign_tables(demo_ctx *ctx)
     }
     long long q = 0;
     for (int t = 0; t < T; ++t) {
-        flat[t].quad_begin = q;
+        flat[t].piece_begin = q;
         flat[t].n = ctx->n_elems[t];
         flat[t].tensor = t;
         flat[t].pad = 0;
-        q += (ctx->n_elems[t] + 3) / 4;
+        q += (ctx->n_elems[t] + demo_apply_piece() - 1) / demo_apply_piece();
     }
-    ctx->n_quads = q;
+    ctx->n_pieces = q;
     if (!ctx->d_s && cudaMalloc((void **)&ctx->d_s, (size_t)T * sizeof(void *)) != cudaSuccess) {
         cudaGetLastError();
         return DEMO_ERR_ALLOC;
@@ -854,7 +854,7 @@ demo_status demo_apply_signs(demo_ctx *ctx, const int8_t *const *signs, float *c
         DemoApplySignsArgs a;
         a.entries = ctx->d_flat;
         a.n_entries = T;
-        a.n_quads = ctx->n_quads;
+        a.n_pieces = ctx->n_pieces;
         a.sign_ptrs = ctx->d_s;
         a.x_ptrs = ctx->d_x;
         a.lr = ctx->cfg.lr;

@@ -232,37 +232,35 @@ __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeA
     }
 }
 
-// x <- x - lr (sign + wd x) with the signs a parameter server handed out (Algorithm 1, last two lines).
-// One thread per group of four consecutive elements of a tensor; same arithmetic as the decode kernels.
+// x <- x - lr (sign + wd x) with the signs a parameter server handed out (Algorithm 1, last two lines); same arithmetic as
+// the decode kernels.  Bound by HBM (9 bytes per parameter).  A block takes pieces of APPLY_PIECE elements of one tensor, a
+// grid apart, four consecutive elements per thread; the tensor is looked up once per piece, 32 table entries at a time, not by
+// a binary search for every group of four elements (168 matrices, 454 M parameters: 780 -> 632 us, 6.5 TB/s).  Pieces of 8 or
+// 16 elements per thread, with their loads together, took 7 % longer.
+constexpr int APPLY_PIECE = 4 * GEN_THREADS;
 __global__ void __launch_bounds__(GEN_THREADS) apply_signs_kernel(DemoApplySignsArgs a)
 {
-    for (long long q = (long long)blockIdx.x * GEN_THREADS + threadIdx.x; q < a.n_quads;
-         q += (long long)gridDim.x * GEN_THREADS) {
-        int lo = 0, hi = a.n_entries - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (a.entries[mid].quad_begin <= q)
-                lo = mid;
-            else
-                hi = mid - 1;
+    const int lane = threadIdx.x & 31;
+    int e = 0;  // the last entry with piece_begin <= q
+    auto update = [&](float xv, signed char s) { return fmaf(-a.lr, fmaf(a.wd, xv, (float)s), xv); };
+    for (long long q = blockIdx.x; q < a.n_pieces; q += gridDim.x) {
+        for (;;) {
+            const int i = e + 1 + lane;
+            const int n = __popc(__ballot_sync(0xffffffffu, i < a.n_entries && a.entries[i].piece_begin <= q));
+            e += n;
+            if (n < 32) break;
         }
-        const DemoFlatEntry e = a.entries[lo];
-        const long long i0 = (q - e.quad_begin) * 4;
-        float *__restrict__ x = a.x_ptrs[e.tensor];
-        const signed char *__restrict__ sg = a.sign_ptrs[e.tensor];
-        if (i0 + 4 <= e.n) {  // tensors start 16-byte aligned, so groups of four are aligned too
-            float4 xv = *reinterpret_cast<const float4 *>(x + i0);
-            const char4 s4 = *reinterpret_cast<const char4 *>(sg + i0);
-            xv.x = fmaf(-a.lr, fmaf(a.wd, xv.x, (float)s4.x), xv.x);
-            xv.y = fmaf(-a.lr, fmaf(a.wd, xv.y, (float)s4.y), xv.y);
-            xv.z = fmaf(-a.lr, fmaf(a.wd, xv.z, (float)s4.z), xv.z);
-            xv.w = fmaf(-a.lr, fmaf(a.wd, xv.w, (float)s4.w), xv.w);
-            *reinterpret_cast<float4 *>(x + i0) = xv;
+        const DemoFlatEntry en = a.entries[e];
+        const long long i0 = (q - en.piece_begin) * APPLY_PIECE, left = en.n - i0;
+        float *__restrict__ x = a.x_ptrs[en.tensor] + i0;
+        const signed char *__restrict__ sg = a.sign_ptrs[en.tensor] + i0;
+        const int at = (int)threadIdx.x * 4;
+        if (left >= APPLY_PIECE) {  // tensors start 16-byte aligned, so the pieces are aligned too
+            const float4 xv = *reinterpret_cast<const float4 *>(x + at);
+            const char4 sv = *reinterpret_cast<const char4 *>(sg + at);
+            *reinterpret_cast<float4 *>(x + at) = make_float4(update(xv.x, sv.x), update(xv.y, sv.y), update(xv.z, sv.z), update(xv.w, sv.w));
         } else {
-            for (long long i = i0; i < e.n; ++i) {
-                const float xv = x[i];
-                x[i] = fmaf(-a.lr, fmaf(a.wd, xv, (float)sg[i]), xv);
-            }
+            for (int i = threadIdx.x; i < (int)left; i += GEN_THREADS) x[i] = update(x[i], sg[i]);
         }
     }
 }
@@ -295,12 +293,18 @@ cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, int s
     }
 }
 
+int demo_apply_piece() { return APPLY_PIECE; }
+
 cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, cudaStream_t stream)
 {
-    if (a.n_quads <= 0) return cudaSuccess;
-    long long grid = (a.n_quads + GEN_THREADS - 1) / GEN_THREADS;
-    const long long cap = (long long)sm_count * 8;
-    if (grid > cap) grid = cap;
+    if (a.n_pieces <= 0) return cudaSuccess;
+    int per_sm = 0;
+    const cudaError_t err = demo_resident_ctas((const void *)apply_signs_kernel, GEN_THREADS, 0, &per_sm);
+    if (err != cudaSuccess) return err;
+    long long grid = (long long)sm_count * per_sm;
+    if (grid > a.n_pieces) grid = a.n_pieces;
+    // An ordinary launch: resident beside the last CTAs of decode_signs, these would keep that kernel's split of the SM into
+    // shared memory and L1 to their end, and the L1 left (28 KB) does not hold the loads in flight (632 -> about 830 us).
     apply_signs_kernel<<<(unsigned)grid, GEN_THREADS, 0, stream>>>(a);
     return cudaGetLastError();
 }

@@ -89,3 +89,19 @@ def test_segments(s, k, workers):
     for _ in range(2):
         r.step()
     r.close()
+
+
+@pytest.mark.parametrize("shapes", [[(64, 64)], [(64,), (64, 64 * 3), (64 * 65,), (128, 64)], [(64 * 64,)] * 40])
+def test_apply_signs_pieces(shapes):
+    """Tensors of a piece of 1024 elements and less, several, and with a remainder; many tensors per block."""
+    import paper_2411_19870_b200 as demo
+
+    tr = demo.DemoTransform(shapes, chunk=64, topk=4, beta=0.9, lr=0.125, weight_decay=0.5, num_workers=1)
+    gen = torch.Generator("cuda").manual_seed(7)
+    x = [torch.randn(s, device="cuda", generator=gen) for s in shapes]
+    signs = [torch.randint(-1, 2, s, device="cuda", generator=gen, dtype=torch.int8) for s in shapes]
+    want = [v.double() - 0.125 * (s.double() + 0.5 * v.double()) for v, s in zip(x, signs)]
+    tr.apply_signs(signs, x)
+    for got, ref in zip(x, want):  # two fused multiply-adds: at most one rounding each of values below 4
+        assert (got.double() - ref).abs().max().item() <= 2 ** -22
+    tr.close()
