@@ -37,10 +37,11 @@ struct DemoTickets {
 };
 constexpr unsigned NO_TICKET = 0x80000000u;  // beyond every list
 __device__ __forceinline__ unsigned ticket_draw(DemoTickets *t) { return t ? atomicAdd(&t->next, 1u) : NO_TICKET; }
-// (one thread per CTA, after its last draw has returned)
-__device__ __forceinline__ void ticket_finish(DemoTickets *t)
+// (one thread of each of the CTA's `parties` that draw, after its last draw has returned)
+__device__ __forceinline__ void ticket_finish(DemoTickets *t, unsigned parties = 1)
 {
-    if (t && atomicInc(&t->done, gridDim.x - 1u) == gridDim.x - 1u) atomicExch(&t->next, 0u);
+    const unsigned last = gridDim.x * parties - 1u;
+    if (t && atomicInc(&t->done, last) == last) atomicExch(&t->next, 0u);
 }
 
 // Host side.  Raises the kernel's dynamic shared-memory limit to `smem` and returns how many CTAs of `threads` threads fit

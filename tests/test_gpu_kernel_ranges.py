@@ -29,6 +29,19 @@ def test_s64_list_and_dense_row_stage(k, kind):
     r.close()
 
 
+@pytest.mark.parametrize("k,agg", [(48, 0), (49, 2), (64, 2), (65, 0), (192, 0), (193, 2)])
+def test_tensor_core_pairs(k, agg):
+    """s = 64 under a random basis: listed and dense row stage, decode by warp order and by barriers, four and three groups per CTA;
+    2406 chunks, more pairs than the grid has groups, the second tensor's one chunk alone in the last pair's second half."""
+    wl = inputs.Workload("tc", [(37 * 64, 65 * 64), (64, 64)], chunk=64, topk=k, num_workers=2, grad_kind="normal", grad_std=0.01,
+                         grad_dtype=torch.float32 if k % 2 else torch.bfloat16)
+    r = parity.Runner(wl, max_chunks=300, gauss=inputs.basis_gaussian(k, 64).numpy(), agg=agg)
+    for _ in range(2):
+        r.step()
+    assert r.tr.device_status() == 0
+    r.close()
+
+
 @pytest.mark.parametrize("shapes,chunks,k", [
     ([(64, 32, 7, 7), (32,)], [(32, 4, 7, 7), (32,)], 40),         # kernel windows of 7 x 7; a lossless vector
     ([(32, 16, 2, 2), (24, 4, 6, 6)], [(16, 16, 2, 2), (8, 4, 6, 6)], 17),
