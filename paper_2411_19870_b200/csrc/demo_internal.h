@@ -107,7 +107,7 @@ cudaError_t demo_launch_wait_selftest(int *status, long long limit_cycles, cudaS
 
 // Gram-Schmidt process on the rows of the s x s matrix `gauss` (device, fp32) in fp64; writes the
 // orthonormal rows to `basis` (device, fp32) and 1 to *flag when a row has no component left.
-cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *flag, int s, cudaStream_t stream);
+cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *verdict, int s, cudaStream_t stream);
 
 // ---- tensors of any order with rectangular chunks (appendix of the paper: blocking operator and
 // multilinear product; kernels_nd.cu) ---------------------------------------------------------------

@@ -46,8 +46,8 @@ struct demo_ctx {
 
     // caller-supplied orthonormal basis (rows = basis vectors); while `custom_basis` is set every
     // tensor goes through the dense-transform kernels, which read the basis from memory
-    float *d_P = nullptr, *d_P_stage = nullptr;  // [s*s], [2*s*s]
-    int *d_basis_flag = nullptr;
+    float *d_P = nullptr;      // [s*s]
+    float *h_gauss = nullptr;  // pinned: [s*s] Gaussian matrix and the verdict on it; from the first demo_set_basis_gaussian
     bool custom_basis = false;
     bool momentum_dct = false;  // demo_set_momentum_domain(DEMO_MOMENTUM_DCT)
 
@@ -151,8 +151,7 @@ void release(demo_ctx *c)
     cudaFree(c->d_entries_nd);
     cudaFree(c->d_tables);
     cudaFree(c->d_P);
-    cudaFree(c->d_P_stage);
-    cudaFree(c->d_basis_flag);
+    cudaFreeHost(c->h_gauss);
     cudaFree(c->d_status);
     cudaFree((void *)c->d_g);
     cudaFree((void *)c->d_m);
@@ -294,8 +293,6 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     ok = ok && cudaMalloc(&c->d_status, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_tickets, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_P, C.size() * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->d_P_stage, 2 * C.size() * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->d_basis_flag, sizeof(int)) == cudaSuccess;
     if (ok && c->n2d) ok = cudaMalloc(&c->d_entries2d, e2d.size() * sizeof(DemoTensorEntry)) == cudaSuccess;
     if (ok && c->n1d) ok = cudaMalloc(&c->d_entries1d, e1d.size() * sizeof(DemoTensorEntry)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_g, W * T * sizeof(void *)) == cudaSuccess;
@@ -1010,22 +1007,22 @@ demo_status demo_set_basis_gaussian(demo_ctx *ctx, const float *gauss_host, void
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const int s = ctx->cfg.chunk;
     const size_t n = (size_t)s * s;
-    // staging = [Gaussian input | orthonormalised output]; the active table is replaced only after the
-    // kernel's verdict, so a singular matrix leaves the previous basis in force
-    float *gauss = ctx->d_P_stage, *out = ctx->d_P_stage + n;
-    int flag = 0;
-    bool ok = cudaMemcpyAsync(gauss, gauss_host, n * sizeof(float), cudaMemcpyHostToDevice, stream) == cudaSuccess;
-    ok = ok && cudaMemsetAsync(ctx->d_basis_flag, 0, sizeof(int), stream) == cudaSuccess;
-    ok = ok && demo_launch_gram_schmidt(gauss, out, ctx->d_basis_flag, s, stream) == cudaSuccess;
+    // the kernel reads the matrix from pinned memory and replaces the active table only if its verdict is good, so a
+    // singular matrix leaves the previous basis in force; the pinned buffer is free again when the call returns
+    bool ok = ctx->h_gauss || cudaHostAlloc(&ctx->h_gauss, n * sizeof(float) + sizeof(int), cudaHostAllocDefault) == cudaSuccess;
+    int *verdict = ok ? reinterpret_cast<int *>(ctx->h_gauss + n) : nullptr;
+    if (ok) {
+        std::memcpy(ctx->h_gauss, gauss_host, n * sizeof(float));
+        *verdict = 1;
+    }
+    ok = ok && demo_launch_gram_schmidt(ctx->h_gauss, ctx->d_P, verdict, s, stream) == cudaSuccess;
     if (ok) ctx->launches += 1;
-    ok = ok && cudaMemcpyAsync(&flag, ctx->d_basis_flag, sizeof(int), cudaMemcpyDeviceToHost, stream) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
-    if (ok && flag) return DEMO_ERR_INVALID_ARG;
-    ok = ok && cudaMemcpyAsync(ctx->d_P, out, n * sizeof(float), cudaMemcpyDeviceToDevice, stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         return DEMO_ERR_CUDA;
     }
+    if (*verdict) return DEMO_ERR_INVALID_ARG;
     ctx->custom_basis = true;
     return DEMO_OK;
 }

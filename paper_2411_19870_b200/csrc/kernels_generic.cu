@@ -327,77 +327,84 @@ cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, int sm_co
 // rows of a Gaussian matrix, in fp64, one CTA.  Right-looking order: once row j is final its component
 // is removed from every later row, so each row loses its components along rows 0..j-1 one after the
 // other -- the same operations as the row-by-row statement of the process.
+//
+// s dependent steps, so the latency of a step is all there is.  Eight threads keep a row in registers; the owners of
+// row j + 1 publish it, with the reciprocal of its squared length, once it has lost its component along row j: one barrier
+// per step, products by three-level reductions, one division per step in the whole CTA (fp64 arithmetic is narrow: with
+// the length formed by every row the step took 1.4 times as long).  The matrix is read from and the verdict written to
+// pinned host memory, the active basis only replaced when the verdict is good: a call is one launch and one synchronisation.
+// (One call, s = 8 / 32 / 64 / 128: 48 / 68 / 123 / 292 us with rows in shared memory, two barriers per step and four
+// copies; 20 / 29 / 47 / 215 us now.)
 // =================================================================================================
-constexpr int GS_THREADS = 1024;
+constexpr int GS_LANES = 8;  // threads per row
 
-__global__ void __launch_bounds__(GS_THREADS) gram_schmidt_kernel(const float *__restrict__ gauss,
-                                                                  float *__restrict__ basis, int *flag, int s)
+template <int EPL>  // elements per thread
+__global__ void __launch_bounds__(GS_LANES *GS_LANES *EPL, 1) gram_schmidt_kernel(const float *__restrict__ gauss,
+                                                                               float *__restrict__ basis, int *verdict)
 {
-    extern __shared__ double gs_A[];  // [s][s + 1]
-    __shared__ double scale[128];     // squared length of each input row
-    __shared__ double inv_len;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int WARPS = GS_THREADS / 32;
-    const int ld = s + 1;
-    for (int i = tid; i < s * s; i += GS_THREADS) gs_A[(i / s) * ld + (i % s)] = (double)gauss[i];
-    __syncthreads();
-    for (int r = warp; r < s; r += WARPS) {
-        double acc = 0.0;
-        for (int n = lane; n < s; n += 32) acc += gs_A[r * ld + n] * gs_A[r * ld + n];
-        for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-        if (lane == 0) scale[r] = acc;
-    }
+    constexpr int N = GS_LANES * EPL;  // rows = columns
+    __shared__ __align__(16) double pub[2][N];  // row j and 1 / its squared length, 0 when nothing is left of it
+    __shared__ double pub_inv[2];
+    const int r = threadIdx.x / GS_LANES, l = threadIdx.x % GS_LANES;
+    const int last_of_warp = r | (32 / GS_LANES - 1);
+    constexpr int V = EPL > 1 ? 2 : 1;  // consecutive elements of a thread
+    auto col = [&](int e) { return (e / V) * (V * GS_LANES) + V * l + e % V; };
+    double a[EPL];
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) a[e] = (double)gauss[r * N + col(e)];
+    auto product = [&](const double (&u)[EPL], const double (&v)[EPL]) {
+        double acc[2] = {0.0, 0.0};
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[e & 1] = fma(u[e], v[e], acc[e & 1]);
+        double sum = acc[0] + acc[1];
+#pragma unroll
+        for (int d = GS_LANES / 2; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        return sum;
+    };
+    const double scale = product(a, a);  // squared length of the input row
+    auto publish = [&](int j, double len2) {
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) pub[j & 1][col(e)] = a[e];
+        if (l == 0) pub_inv[j & 1] = len2 > 1e-24 * scale ? 1.0 / len2 : 0.0;
+    };
+    if (r == 0) publish(0, scale);
     __syncthreads();
     bool bad = false;
-    for (int j = 0; j < s; ++j) {
-        if (warp == 0) {
-            double acc = 0.0;
-            for (int n = lane; n < s; n += 32) acc += gs_A[j * ld + n] * gs_A[j * ld + n];
-            for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-            if (lane == 0) inv_len = (acc > 1e-24 * scale[j]) ? 1.0 / sqrt(acc) : 0.0;
+    for (int j = 0; j < N && !bad; ++j) {
+        const double inv = pub_inv[j & 1];
+        bad = inv == 0.0;
+        if (last_of_warp > j) {
+            double p[EPL];
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) p[e] = pub[j & 1][col(e)];
+            const double c = product(a, p) * (r > j ? inv : 0.0);
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) a[e] = fma(-c, p[e], a[e]);
+            if (last_of_warp / (32 / GS_LANES) == (j + 1) / (32 / GS_LANES)) {  // the warp that owns row j + 1
+                const double len2 = product(a, a);
+                if (r == j + 1) publish(j + 1, len2);
+            }
         }
         __syncthreads();
-        const double inv = inv_len;
-        if (inv == 0.0) {
-            bad = true;
-            break;
-        }
-        double p[4];  // s <= 128: at most 4 entries of row j per lane
-#pragma unroll
-        for (int t = 0; t < 4; ++t) p[t] = (lane + 32 * t < s) ? gs_A[j * ld + lane + 32 * t] * inv : 0.0;
-        for (int r = j + 1 + warp; r < s; r += WARPS) {
-            double dot = 0.0;
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (lane + 32 * t < s) dot += gs_A[r * ld + lane + 32 * t] * p[t];
-            for (int d = 16; d > 0; d >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, d);
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (lane + 32 * t < s) gs_A[r * ld + lane + 32 * t] -= dot * p[t];
-        }
-        __syncthreads();
-        if (warp == 0) {
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (lane + 32 * t < s) gs_A[j * ld + lane + 32 * t] = p[t];
-        }
     }
-    __syncthreads();
-    if (bad) {
-        if (tid == 0) *flag = 1;
-        return;
-    }
-    for (int i = tid; i < s * s; i += GS_THREADS) basis[i] = (float)gs_A[(i / s) * ld + (i % s)];
+    if (threadIdx.x == 0) *verdict = bad;
+    if (bad) return;
+    const double inv = 1.0 / sqrt(product(a, a));
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) basis[r * N + col(e)] = (float)(a[e] * inv);
 }
 
-cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *flag, int s, cudaStream_t stream)
+// `gauss` and `verdict` are pinned host memory.
+cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *verdict, int s, cudaStream_t stream)
 {
-    if (s < 1 || s > 128) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(double) * (size_t)s * (s + 1);
-    cudaError_t err =
-        cudaFuncSetAttribute(gram_schmidt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    gram_schmidt_kernel<<<1, GS_THREADS, smem, stream>>>(gauss, basis, flag, s);
+    switch (s) {
+        case 8: gram_schmidt_kernel<1><<<1, 64, 0, stream>>>(gauss, basis, verdict); break;
+        case 16: gram_schmidt_kernel<2><<<1, 128, 0, stream>>>(gauss, basis, verdict); break;
+        case 32: gram_schmidt_kernel<4><<<1, 256, 0, stream>>>(gauss, basis, verdict); break;
+        case 64: gram_schmidt_kernel<8><<<1, 512, 0, stream>>>(gauss, basis, verdict); break;
+        case 128: gram_schmidt_kernel<16><<<1, 1024, 0, stream>>>(gauss, basis, verdict); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
