@@ -40,8 +40,8 @@ struct DemoCompressArgs {
     float alpha;    // momentum-subtraction coefficient: m <- B - alpha * IDCT(kept)
     int grad_bf16;  // 1: gradients are bf16, 0: fp32
     int *status;    // device status word (sticky)
-    // Optional TMA tensor maps (128-byte CUtensorMap objects in device memory, indexed like the
-    // pointer arrays; box = one s x s tile).  NULL: tiles are staged row by row with 1-D bulk copies.
+    // TMA tensor maps (128-byte CUtensorMap objects in device memory, indexed like the
+    // pointer arrays; box = one s x s tile): s = 64 and 128.
     const void *tmap_m;
     const void *tmap_g;
     int wait_first = 1;  // see StreamOrder (launch.cuh)
@@ -89,6 +89,8 @@ cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const De
 bool demo_fast_supported(int s);
 cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
 cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
+// s = 32 (kernels_fast32.cu).
+cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
 // s = 64 with TMA tensor maps (kernels_fast64.cu; cudaErrorNotSupported without them).
 cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
 // s = 128 (kernels_fast128.cu); need the TMA tensor maps (cudaErrorNotSupported without them).

@@ -299,8 +299,8 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     ok = ok && cudaMalloc((void **)&c->d_m, W * T * sizeof(void *)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_x, T * sizeof(void *)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_p, W * sizeof(void *)) == cudaSuccess;
-    if (ok && c->n2d && demo_fast_supported(s)) {
-        // TMA descriptors need the driver's encoder; without it the fast kernels stage row by row
+    if (ok && c->n2d && demo_fast_supported(s) && s != 32) {
+        // TMA descriptors need the driver's encoder; without it s = 64 and 128 are left to the generic kernels
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
@@ -523,11 +523,12 @@ demo_status demo_payload_layout(const demo_ctx *ctx, int32_t tensor, int64_t *fi
     return DEMO_OK;
 }
 
-// The fast kernels hard-code the DCT factorisation; any other basis takes the dense-transform kernels.
+// The fast kernels hard-code the DCT factorisation; any other basis takes the dense-transform kernels.  s = 64 and 128
+// need tensor maps.
 static bool use_fast_path(const demo_ctx *ctx)
 {
     const int s = ctx->cfg.chunk;
-    return ctx->path == DEMO_PATH_AUTO && !ctx->custom_basis && demo_fast_supported(s) && (s != 128 || ctx->encode);
+    return ctx->path == DEMO_PATH_AUTO && !ctx->custom_basis && demo_fast_supported(s) && (s == 32 || ctx->encode);
 }
 
 static bool use_small_tiles(const demo_ctx *ctx)

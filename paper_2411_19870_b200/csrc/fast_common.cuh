@@ -43,14 +43,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, unsigned parity,
     return true;
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// 1-D bulk async copy global -> shared (16-byte aligned addresses, size a multiple of 16).
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, unsigned bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
 // 2-D tiled TMA load of one box (coordinates in elements: x along the row, y the row index).
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int x, int y, uint32_t bar)
 {
@@ -132,10 +124,8 @@ __device__ __forceinline__ unsigned warp_inclusive_scan(unsigned v, int lane)
     return v;
 }
 
-// A CTA hosts NCH independent "slots" of S threads, one chunk each.  Threads of a slot meet at the
-// slot's own named barrier (a warp-level barrier when the slot is a single warp); all slots meet once
-// per chunk at the CTA barrier, which keeps the warps of the CTA in the same region of the (large,
-// fully unrolled) code so that instruction fetches are shared instead of streamed once per warp.
+// The S threads of a "slot" own one chunk and meet at the slot's own named barrier (a warp-level barrier when the slot is a
+// single warp).
 template <int S>
 struct SlotBarrier {
     int id;  // named barrier 1..15
@@ -295,17 +285,16 @@ __device__ __forceinline__ void tmem_free_cta(uint32_t base, uint32_t cols)
 // to it in list order until k_eff are reached.  emit(pos, i) is called for every kept candidate: i its list
 // position, pos its place among the kept ones (ascending list order).
 // ------------------------------------------------------------------------------------------------
-template <int NK, class Where, class Emit>
-__device__ __forceinline__ void warp_ballot_select(const unsigned *cand_key, unsigned n_all, unsigned lmin, int k_eff,
-                                                   int lane, Where where, Emit emit)
+template <int NK, class Key, class Emit>
+__device__ __forceinline__ void warp_ballot_select(Key key_of, unsigned n_all, unsigned lmin, int k_eff, int lane, Emit emit)
 {
-    // where(i): storage position of list entry i (the list may sit in several pieces)
+    // key_of(i): magnitude key of list entry i (the list may sit in several pieces)
     unsigned keys[NK];
     unsigned hi = 0u;
 #pragma unroll
     for (int j = 0; j < NK; ++j) {
         const unsigned i = (unsigned)j * 32u + lane;
-        keys[j] = (i < n_all) ? cand_key[where(i)] : 0u;
+        keys[j] = (i < n_all) ? key_of(i) : 0u;
         hi = max(hi, keys[j]);
     }
     hi = __reduce_max_sync(0xffffffffu, hi);

@@ -29,6 +29,27 @@ def test_s64_list_and_dense_row_stage(k, kind):
     r.close()
 
 
+@pytest.mark.parametrize("kind", ["tensor_scaled", "student_t_ties"])
+@pytest.mark.parametrize("k", [1, 12, 13, 32, 33, 128, 129, 1024])
+def test_s32_bounds_list_and_search(k, kind):
+    """s = 32: bound from row and half-row maxima, listed and dense row stage, bounded and unbounded search; more chunks than
+    the grid has warps, all-zero tiles and tiles of one element."""
+    wl = inputs.Workload("s32k", [(55 * 32, 56 * 32), (32, 96)], chunk=32, topk=k, num_workers=2, grad_kind=kind,
+                         grad_dtype=torch.float32 if k % 2 else torch.bfloat16)
+    r = parity.Runner(wl, max_chunks=200, seed=k)
+    for step in range(2):
+        grads = [st.next() for st in r.streams]
+        for g in grads:
+            g[0][:32, :32] = 0
+            g[0][32:64, :32] = 0
+            g[0][40, 5] = 0.5
+            g[1][:, :32] = 0
+            g[1][:, 32:64] = 0
+            g[1][3, 40] = -0.25
+        r.step(grads=grads)
+    r.close()
+
+
 @pytest.mark.parametrize("k,agg", [(48, 0), (49, 2), (64, 2), (65, 0), (192, 0), (193, 2)])
 def test_tensor_core_pairs(k, agg):
     """s = 64 under a random basis: listed and dense row stage, decode by warp order and by barriers, four and three groups per CTA;
