@@ -8,14 +8,18 @@
 // in the second) and computes its even (h = 0) or odd (h = 1) outputs; h is warp-uniform, so the two
 // transform bodies never diverge inside a warp.  The inverse runs the transposed graph:
 //     e = DCT-III_64(X[even]),  o = DCT-IV_64(X[odd]),  x[n] = e[n] + o[n],  x[127-n] = e[n] - o[n]
-// with e and o exchanged between the two threads of a line through shared memory.
+// where thread h of a line finishes n in [32h, 32h+32): the two exchange half of e and o through shared memory.
 //
-// compress: TMA-staged m and g tiles -> B = beta*m + g (each thread parks the half column it will write back in
-// tensor memory) -> column pass -> row pass -> coefficients in shared memory -> exact top-k (bound from the 256
-// half-row maxima, candidate list, exact ranking; radix select for degenerate chunks) -> records; sparse row
-// stage of the inverse from the records, fast column stage, residual m <- B - alpha * IDCT(kept) against the
-// parked B, one TMA store of the new momentum tile.  decode: scatter-add of the W payloads in worker order,
-// two inverse passes, sign, update; the x tile is staged into the (then dead) coefficient tile.
+// compress: TMA-staged m and g tiles -> B = beta*m + g (parked in tensor memory) -> column pass -> row pass ->
+// coefficients in shared memory -> exact top-k (bound from the 256 half-row maxima, candidate list, exact ranking; radix
+// select for degenerate chunks) -> records; sparse row stage of the inverse from the records, half of them by each half of
+// the CTA, fast column stage, residual m <- B - alpha * IDCT(kept) against the parked B, one TMA store of the new momentum
+// tile.  The next chunk's g tile comes in, and its m tile to L2, as soon as B is formed.  decode: scatter-add of the W payloads
+// in worker order, two inverse passes, sign, update; the x tile is staged into the (then dead) coefficient tile.
+// Two CTAs of a serial chain of phases per SM are what registers (128 for the 64-point halves) and, for compress, shared
+// memory allow: shared-memory accesses and issue each take about half of the time.  8192 x 8192, k = 32, bf16 gradients:
+// compress 242 -> 222 us (k = 128 313 -> 272) with the halves of the row stage and the early g tile, decode 162 -> 141 us and
+// signs 235 -> 131 us with half the exchange (before, the signs form kept two sets of 64 results and spilled).
 // Tiles need the TMA tensor maps; without them the host uses the generic kernels for s = 128.
 #include <cuda_bf16.h>
 
@@ -63,22 +67,51 @@ __device__ __forceinline__ void forward_half(int h, float (&in)[H], float (&out)
         fdct::dct4_paired<H, SC>(in, out);
     }
 }
-// Inverse half-transform: in[p] = coefficient 2p (h = 0) or 2p+1 (h = 1); out = e (h = 0) or o (h = 1).
-__device__ __forceinline__ void inverse_half(int h, float (&in)[H], float (&out)[H])
+// Inverse half-transform: in[p] = coefficient 2p (h = 0) or 2p+1 (h = 1), result e (h = 0) or o (h = 1).  Thread h of the
+// line finishes the elements n and 127-n of n in [32h, 32h+32): it keeps that part of its result and sends the other.
+__device__ __forceinline__ void inverse_half(int h, float (&in)[H], float (&keep)[H / 2], float (&send)[H / 2])
 {
+    float out[H];
     if (h == 0) {
         in[0] *= fdct::dc_scale<S>();
         fdct::dct3_packed<H, SC>(in, out);
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) {
+            keep[q] = out[q];
+            send[q] = out[H / 2 + q];
+        }
     } else {
         fdct::dct4_paired<H, SC>(in, out);
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) {
+            keep[q] = out[H / 2 + q];
+            send[q] = out[q];
+        }
+    }
+}
+// Elements n (lo) and 127-n (hi) from the kept and the received part: e + o and e - o.
+__device__ __forceinline__ void inverse_join(int h, const float (&keep)[H / 2], float (&lo)[H / 2], float (&hi)[H / 2])
+{   // (in: hi = the received part)
+    if (h == 0) {
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) {
+            lo[q] = keep[q] + hi[q];
+            hi[q] = keep[q] - hi[q];
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) {
+            lo[q] = hi[q] + keep[q];
+            hi[q] = hi[q] - keep[q];
+        }
     }
 }
 
+// The g tile has a landing area of its own behind the tile that m lands in and the transform works in.
 template <typename GT>
 constexpr size_t compress128_tile_bytes()
 {
-    return (size_t)M * (sizeof(float) + sizeof(GT)) > (size_t)S * XS * 4 ? (size_t)M * (sizeof(float) + sizeof(GT))
-                                                                         : (size_t)S * XS * 4;
+    return (size_t)S * XS * sizeof(float) + (size_t)M * sizeof(GT);
 }
 template <typename GT>
 constexpr size_t compress128_smem()
@@ -93,8 +126,8 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
     constexpr unsigned TILE_BYTES = M * sizeof(float) + M * sizeof(GT);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *Ms = reinterpret_cast<float *>(smem_raw);  // [128*128] m tile
-    GT *Gs = reinterpret_cast<GT *>(Ms + M);          // [128*128] g tile
-    float *X = Ms;                                    // [128*132] transpose / coefficients / row stage (aliases the tiles)
+    float *X = Ms;                                    // [128*132] transpose / coefficients / row stage (aliases the m tile)
+    GT *Gs = reinterpret_cast<GT *>(X + S * XS);      // [128*128] g tile
     unsigned *hist = reinterpret_cast<unsigned *>(smem_raw + compress128_tile_bytes<GT>());  // [256]
     unsigned *warp_tot = hist + 256;                                                         // [8]
     unsigned *s_state = warp_tot + 8;                                                        // [4]
@@ -111,12 +144,13 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         mbar_init(bar, 1);
         fence_proxy_async();
     }
-    // Tensor memory as storage: thread (h, j) parks its 64 elements of column j of B = beta*m + g (rows 0..63 for
-    // h = 0, rows 127..64 for h = 1) in lane j, columns 64h .. 64h+63, between the forward pass and the residual.
+    // Tensor memory as storage: column j of B = beta*m + g is parked in lane j between the forward pass and the residual, by
+    // thread (0, j) its rows 0..63 in columns 0..63, by thread (1, j) its rows 127..64 in columns 64..127; each of the two
+    // reads back half of both.
     if (tid == 0) tmem_slot[1] = ticket_draw(a.tickets);
     const uint32_t tmem_base = tmem_alloc_cta(tmem_slot, TMEM_COLS128);
     fence_proxy_async();
-    const uint32_t taddr = tmem_base + ((uint32_t)(j & ~31) << 16) + (uint32_t)(h * H);
+    const uint32_t taddr = tmem_base + ((uint32_t)(j & ~31) << 16);
 
     EntryCursor cur;
     unsigned phase = 0;
@@ -130,23 +164,25 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
             tmap_acquire(static_cast<const char *>(a.tmap_g) + (size_t)te.tensor * TMAP_BYTES);
         }
     };
-    auto issue_tiles = [&](const DemoTensorEntry &te, long long c) {
+    // (thread 0) requests a chunk's g tile, which may come as soon as the one before it has been read, and with it announces
+    // both tiles; the m tile follows when the new momentum of the chunk before has left its place
+    auto issue_tile = [&](const DemoTensorEntry &te, long long c, bool g) {
         const unsigned lc = (unsigned)(c - te.chunk_begin);
         const unsigned k0 = lc / (unsigned)te.c1, k1 = lc - k0 * (unsigned)te.c1;
-        if (tid == 0) {
-            const char *tm_m = static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES;
-            const char *tm_g = static_cast<const char *>(a.tmap_g) + (size_t)te.tensor * TMAP_BYTES;
-            mbar_expect_tx(bar, TILE_BYTES);
-            tma_load_2d(smem_u32(Ms), tm_m, k1 * S, k0 * S, bar);
-            tma_load_2d(smem_u32(Gs), tm_g, k1 * S, k0 * S, bar);
-        }
+        const char *tm = static_cast<const char *>(g ? a.tmap_g : a.tmap_m) + (size_t)te.tensor * TMAP_BYTES;
+        if (g) mbar_expect_tx(bar, TILE_BYTES);
+        tma_load_2d(g ? smem_u32(Gs) : smem_u32(Ms), tm, k1 * S, k0 * S, bar);
+        if (g) tma_prefetch_2d(static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES, k1 * S, k0 * S);
     };
 
     long long c = blockIdx.x;
     if (c < a.n_chunks) {
         cur.seek(a.entries, a.n_entries, c);
         acquire_maps(cur.te);
-        issue_tiles(cur.te, c);
+        if (tid == 0) {
+            issue_tile(cur.te, c, true);
+            issue_tile(cur.te, c, false);
+        }
     }
     for (long long nc; c < a.n_chunks; c = nc) {
         const DemoTensorEntry te = cur.te;  // the cursor points at chunk c
@@ -191,9 +227,13 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                         in[n] = fmaf(sg, hi, lo);
                         park[q] = h ? hi : lo;
                     }
-                    tmem_st32(taddr + 32 * half, park);
+                    tmem_st32(taddr + h * H + 32 * half, park);
                 }
-                __syncthreads();  // the staged tiles are consumed (X aliases them)
+                tmem_wait_st();
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                fence_proxy_async();
+                __syncthreads();  // the staged tiles are consumed (X aliases the m tile)
+                if (tid == 0 && nc < a.n_chunks) issue_tile(cur.te, nc, true);
             } else {
                 // row j of the column-transformed tile, folded
                 const float4 *row = reinterpret_cast<const float4 *>(X + j * XS);
@@ -231,9 +271,10 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         // candidates are listed in index order and ranked exactly, ties to the lowest index.  Everything
         // compares integer magnitude keys, so NaN and Inf are ordered like any other bit pattern.  More
         // than CAP128 candidates (tied or degenerate chunks) or k_eff > 256: radix select below.
-        // the row-stage list is padded with zero-valued entries whose "row" is a scratch line behind the tile
+        // the row-stage list is padded with zero-valued entries whose "row" is a scratch line, the then unused histogram
         // (ordered before the record writes by the barriers below)
-        if (tid < RECS128) recs4[tid] = make_int4(S * XS, 0, 0, 0);
+        constexpr int PAD_ROW = (int)(compress128_tile_bytes<GT>() / sizeof(float));
+        if (tid < RECS128) recs4[tid] = make_int4(PAD_ROW, 0, 0, 0);
         bool use_radix = k_eff > 256;
         if (!use_radix) {
             const float4 *mine4 = reinterpret_cast<const float4 *>(X + (tid >> 1) * XS + 64 * (tid & 1));
@@ -316,10 +357,16 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                 mask = (tid & 1) ? ((mreg << 16) | (mreg >> 48)) : mreg;
             }
             const unsigned cnt = (unsigned)__popcll(mask);
-            const unsigned o = block_exclusive_scan(cnt, warp_tot);
-            if (tid == THREADS - 1) s_state[3] = o + cnt;
+            const unsigned inc = warp_inclusive_scan(cnt, lane);
+            if (lane == 31) warp_tot[warp] = inc;
             __syncthreads();
-            const unsigned n_cand = s_state[3];
+            unsigned o = inc - cnt, n_cand = 0;
+#pragma unroll
+            for (int w = 0; w < THREADS / 32; ++w) {
+                const unsigned n = warp_tot[w];
+                o += w < warp ? n : 0u;
+                n_cand += n;
+            }
             use_radix = n_cand > (unsigned)CAP128 || n_cand < (unsigned)k_eff;
             if (!use_radix) {
                 // The list is in index order: inside a row the candidates of the even-coefficient thread (lane 2r)
@@ -345,8 +392,12 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                     cand_idx[at] = S * (tid >> 1) + 2 * e + odd;
                 }
                 __syncthreads();
-                // the first warp picks the k_eff largest candidates (list order = index order) and writes the records
-                if (warp == 0) {
+                // the first warp picks the k_eff largest candidates (list order = index order) and writes the records; the
+                // others clear the tile for the row stage
+                if (warp != 0) {
+                    for (int i = tid - 32; i < S * XS / 4; i += THREADS - 32)
+                        reinterpret_cast<float4 *>(X)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                } else {
                     auto emit = [&](unsigned pos, unsigned li) {
                         DemoRecord r;
                         r.idx = cand_idx[li];
@@ -464,12 +515,18 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                 }
             }
         }
-        __syncthreads();  // records complete; the coefficient tile is dead
+        __syncthreads();  // records complete; the coefficient tile is dead or, without the radix select, already cleared
+        if (use_radix) {
+            for (int i = tid; i < S * XS / 4; i += THREADS) reinterpret_cast<float4 *>(X)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncthreads();
+        }
 
         // ---- residual: sparse row stage T[u][j] = sum over kept (u, v) of val * C[v][j] ------------
-        for (int i = tid; i < S * XS / 4; i += THREADS) reinterpret_cast<float4 *>(X)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncthreads();
-        if (h == 0 && k_eff <= 128) {
+        if (k_eff <= 128) {
+            // the two halves of the CTA take half of the list each, cut where a row ends
+            int cut = k_eff / 2;
+            while (cut > 0 && cut < k_eff && recs4[cut].x == recs4[cut - 1].x) ++cut;
+            const int r_begin = h ? cut : 0, r_end = h ? k_eff : cut;
             // The running sum of a row is stored after every entry (the last store of a row carries the whole sum)
             // and starts again from zero when the next entry belongs to another row: no branch in the loop.
             // The cosines of a whole batch of entries are requested before the dependent accumulation starts: the
@@ -480,7 +537,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
             auto row_stage = [&](auto batch_tag) {
                 constexpr int BATCH = decltype(batch_tag)::value;
 #pragma unroll 1
-                for (int r0 = 0; r0 < k_eff; r0 += BATCH) {
+                for (int r0 = r_begin; r0 < r_end; r0 += BATCH) {
                     float cv[BATCH];
 #pragma unroll
                     for (int q = 0; q < BATCH; ++q) cv[q] = __ldg(a.C + (unsigned)(recs4[r0 + q].y + j));
@@ -490,7 +547,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                         const int4 rc = nx;
                         nx = recs4[r0 + q + 1];
                         acc = fmaf(__int_as_float(rc.z), cv[q], acc);
-                        Xj[rc.x] = acc;
+                        Xj[r0 + q < r_end ? rc.x : PAD_ROW] = acc;
                         acc = (rc.x != nx.x) ? 0.f : acc;
                     }
                 }
@@ -498,7 +555,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
             if (k_eff <= ROW_AHEAD128)
                 row_stage(std::integral_constant<int, ROW_AHEAD128>{});
             else
-                row_stage(std::integral_constant<int, 4 * ROW_AHEAD128>{});
+                row_stage(std::integral_constant<int, 3 * ROW_AHEAD128>{});
         } else if (h == 0) {
             // k > 128: the records come from the payload itself
             const float *Cj = a.C + j;
@@ -523,31 +580,29 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         for (int p = 0; p < H; ++p) in[p] = X[(2 * p + h) * XS + j];
         fence_proxy_async();
         __syncthreads();  // T is in registers: the tile area is free
-        inverse_half(h, in, out);
-        // exchange e and o through the tile area
-        float *Ex = X;  // [2][64][128]
+        float keep[H / 2], lo[H / 2], hi[H / 2];
+        inverse_half(h, in, keep, lo);
+        // exchange halves of e and o through the tile area
+        float *Ex = X + j;  // [2][32][128]
 #pragma unroll
-        for (int n = 0; n < H; ++n) Ex[(h * H + n) * S + j] = out[n];
+        for (int q = 0; q < H / 2; ++q) Ex[(h * (H / 2) + q) * S] = lo[q];
         __syncthreads();
 #pragma unroll
-        for (int n = 0; n < H; ++n) {
-            const float other = Ex[((h ^ 1) * H + n) * S + j];
-            out[n] = h ? other - out[n] : out[n] + other;  // h=0: x[n] = e+o;  h=1: x[127-n] = e-o
-        }
+        for (int q = 0; q < H / 2; ++q) hi[q] = Ex[((h ^ 1) * (H / 2) + q) * S];
+        inverse_join(h, keep, lo, hi);
         __syncthreads();  // the exchange area is read: the new momentum tile takes its place
         // m <- B - alpha * IDCT(kept): B comes back from tensor memory; the dense tile goes out in one TMA store
-        tmem_wait_st();
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        {
             float b[32];
-            tmem_ld32(taddr + 32 * half, b);
-            if (h) {
+            tmem_ld32(taddr + 32 * h, b);
+            float *Mlo = Ms + (H / 2) * h * S + j, *Mhi = Ms + (S - 1 - (H / 2) * h) * S + j;
 #pragma unroll
-                for (int q = 0; q < 32; ++q) Ms[(S - 1 - (32 * half + q)) * S + j] = b[q] - out[32 * half + q];
-            } else {
+            for (int q = 0; q < 32; ++q) Mlo[q * S] = b[q] - lo[q];
+            tmem_ld32(taddr + H + 32 * h, b);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");  // (the next chunk's stores: behind barriers)
 #pragma unroll
-                for (int q = 0; q < 32; ++q) Ms[(32 * half + q) * S + j] = b[q] - out[32 * half + q];
-            }
+            for (int q = 0; q < 32; ++q) Mhi[-q * S] = b[q] - hi[q];
         }
         fence_proxy_async();
         __syncthreads();
@@ -556,10 +611,10 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
             tma_store_2d(static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES, (int)(k1 * S), (int)(k0 * S),
                          smem_u32(Ms));
             tma_store_commit();
-            tma_store_wait_read();  // the store has read the tile: the next chunk's tiles may land
+            tma_store_wait_read();  // the store has read the tile: the next chunk's m tile may land
+            if (nc < a.n_chunks) issue_tile(cur.te, nc, false);
             tmem_slot[1] = ticket;
         }
-        if (nc < a.n_chunks) issue_tiles(cur.te, nc);
     }
     if (tid == 0) ticket_finish(a.tickets);
     tmem_free_cta(tmem_base, TMEM_COLS128);
@@ -651,35 +706,34 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         }
         // two inverse passes (rolled): both walk "row j" of the tile with unit stride -- pass 0 leaves its result
         // transposed, so that the columns pass 1 needs are rows again and every access below has a fixed offset
-        float in[H], out[H];
+        float lo[H / 2], hi[H / 2];
         bool arrived = true;
         float *ln = St + j * XSD;  // line j
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
+            float in[H], keep[H / 2];
 #pragma unroll
             for (int p = 0; p < H; ++p) in[p] = ln[2 * p + h];
             fence_proxy_async();
             __syncthreads();  // every coefficient of the tile has been read
-            inverse_half(h, in, out);
-            // exchange e / o inside the line: e at elements 0..63, o at 64..127
+            inverse_half(h, in, keep, lo);
+            // exchange halves of e / o inside the line
+            float *mine = ln + (H / 2) * h, *theirs = ln + (H / 2) * (h ^ 1);
 #pragma unroll
-            for (int n = 0; n < H; ++n) ln[h * H + n] = out[n];
+            for (int q = 0; q < H / 2; ++q) mine[q] = lo[q];
             __syncthreads();
 #pragma unroll
-            for (int n = 0; n < H; ++n) {
-                const float other = ln[(h ^ 1) * H + n];
-                out[n] = h ? other - out[n] : out[n] + other;  // h=0: element n;  h=1: element 127-n
-            }
+            for (int q = 0; q < H / 2; ++q) hi[q] = theirs[q];
+            inverse_join(h, keep, lo, hi);  // elements 32h + q and 127 - 32h - q
             fence_proxy_async();
             __syncthreads();  // both halves of every line have read their partner's values
             if (pass == 0) {
-                // element n (resp. 127-n) of row j goes to row n (127-n), column j
-                if (h) {
+                // element n of row j goes to row n, column j
+                float *Slo = St + (H / 2) * h * XSD + j, *Shi = St + (S - 1 - (H / 2) * h) * XSD + j;
 #pragma unroll
-                    for (int n = 0; n < H; ++n) St[(S - 1 - n) * XSD + j] = out[n];
-                } else {
-#pragma unroll
-                    for (int n = 0; n < H; ++n) St[n * XSD + j] = out[n];
+                for (int q = 0; q < H / 2; ++q) {
+                    Slo[q * XSD] = lo[q];
+                    Shi[-q * XSD] = hi[q];
                 }
                 __syncthreads();
             } else if (SIGNS) {
@@ -696,12 +750,14 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                 if (tid == 0) *next_slot = ticket;
             }
         }
+        const ptrdiff_t n1 = te.n1;
+        const size_t at_lo = base + (size_t)((H / 2) * h) * te.n1 + j, at_hi = base + (size_t)(S - 1 - (H / 2) * h) * te.n1 + j;
         if constexpr (SIGNS) {
-            signed char *__restrict__ sg = a.sign_ptrs[te.tensor];
+            signed char *__restrict__ slo = a.sign_ptrs[te.tensor] + at_lo, *__restrict__ shi = a.sign_ptrs[te.tensor] + at_hi;
 #pragma unroll
-            for (int n = 0; n < H; ++n) {
-                const int row = h ? (S - 1 - n) : n;
-                sg[base + (size_t)row * te.n1 + j] = (signed char)((out[n] > 0.f) - (out[n] < 0.f));
+            for (int q = 0; q < H / 2; ++q) {
+                slo[q * n1] = (signed char)((lo[q] > 0.f) - (lo[q] < 0.f));
+                shi[-q * n1] = (signed char)((hi[q] > 0.f) - (hi[q] < 0.f));
             }
             __syncthreads();
             continue;
@@ -711,14 +767,18 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
             mbar_wait_bounded(bar, phase ^ 1u);
             break;
         }
-#pragma unroll
-        for (int n = 0; n < H; ++n) {
-            const int row = h ? (S - 1 - n) : n;
-            const float rv = out[n];
+        auto updated = [&](float rv, float xv) {
             float stepv = __uint_as_float(lr_bits ^ (~__float_as_uint(rv) & 0x80000000u));
             stepv = (rv == 0.f) ? 0.f : stepv;
             if (a.phi) stepv = rv * neg_lr_scale;  // phi = identity
-            x[base + (size_t)row * te.n1 + j] = fmaf(Xt[row * S + j], decay, stepv);
+            return fmaf(xv, decay, stepv);
+        };
+        const float *Xlo = Xt + (H / 2) * h * S + j, *Xhi = Xt + (S - 1 - (H / 2) * h) * S + j;
+        float *__restrict__ xlo = x + at_lo, *__restrict__ xhi = x + at_hi;
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) {
+            xlo[q * n1] = updated(lo[q], Xlo[q * S]);
+            xhi[-q * n1] = updated(hi[q], Xhi[-q * S]);
         }
         fence_proxy_async();
         __syncthreads();

@@ -50,6 +50,22 @@ def test_s32_bounds_list_and_search(k, kind):
     r.close()
 
 
+@pytest.mark.parametrize("k", [1, 2, 9, 31, 128, 129])
+def test_s128_halves_of_the_row_stage(k):
+    """s = 128: the list of records cut between the halves of a CTA where a row ends; more chunks than CTAs, chunks with all
+    their coefficients in one row or in one column."""
+    wl = inputs.Workload("s128k", [(18 * 128, 17 * 128)], chunk=128, topk=k, num_workers=2, grad_kind="tensor_scaled",
+                         grad_dtype=torch.float32 if k % 2 else torch.bfloat16)
+    r = parity.Runner(wl, max_chunks=60, seed=k)
+    for step in range(2):
+        grads = [st.next() for st in r.streams]
+        for g in grads:
+            g[0][:128, :128] = g[0][:1, :128].clone()
+            g[0][128:256, :128] = g[0][128:256, :1].clone()
+        r.step(grads=grads)
+    r.close()
+
+
 @pytest.mark.parametrize("k,agg", [(48, 0), (49, 2), (64, 2), (65, 0), (192, 0), (193, 2)])
 def test_tensor_core_pairs(k, agg):
     """s = 64 under a random basis: listed and dense row stage, decode by warp order and by barriers, four and three groups per CTA;
