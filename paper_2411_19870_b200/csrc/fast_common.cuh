@@ -333,4 +333,44 @@ __device__ __forceinline__ void warp_ballot_select(Key key_of, unsigned n_all, u
     }
 }
 
+// ------------------------------------------------------------------------------------------------
+// Decode
+// ------------------------------------------------------------------------------------------------
+constexpr int STAGE_RECORDS = 512;  // records staged per batch of the scatter (sixteen workers at k <= 32)
+// A worker's records take 2^stage_shift(k) staging entries (k <= STAGE_RECORDS).
+__device__ __forceinline__ int stage_shift(int k) { return k > 32 ? 32 - __clz(k - 1) : 5; }
+
+// A slot's walk over its chunks, kept by its thread 0 in shared memory (in registers every thread would have to spare them):
+// its place in the tensor table, and of the current and the next chunk (by turns) the first element, the row length and
+// the first record.
+struct DecodeWalk {
+    DemoTensorEntry te;
+    long long next_begin;  // chunk_begin of the entry after te (or "never")
+    long long rec[2];
+    long long elem[2];     // offset of the chunk's first element in its tensor
+    int e;
+    int tensor[2], n1[2];
+
+    __device__ __forceinline__ void load(const DemoTensorEntry *entries, int n)
+    {
+        te = entries[e];
+        next_begin = (e + 1 < n) ? entries[e + 1].chunk_begin : 0x7fffffffffffffffLL;
+    }
+    // Moves on to chunk c (ids only grow) and notes it in `which`.
+    template <int S>
+    __device__ __forceinline__ void seek(const DemoTensorEntry *entries, int n, long long c, int k, int which)
+    {
+        if (c >= next_begin) {
+            while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+            load(entries, n);
+        }
+        const unsigned lc = (unsigned)(c - te.chunk_begin);
+        const unsigned k0 = lc / (unsigned)te.c1;
+        tensor[which] = te.tensor;
+        n1[which] = te.n1;
+        elem[which] = ((long long)k0 * te.n1 + (lc - k0 * (unsigned)te.c1)) * S;
+        rec[which] = te.rec_begin + (long long)lc * k;
+    }
+};
+
 }  // namespace fastk

@@ -23,7 +23,6 @@ struct Cfg {
 
 // Bytes of one decode slot: the tile, the mbarrier and -- for the count-normalised mean -- one
 // 16-bit sender count per coordinate.
-constexpr int STAGE_RECORDS = 512;  // records staged per batch of the scatter (sixteen workers at k <= 32)
 template <int S>
 __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)
 {
@@ -31,38 +30,6 @@ __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)
            128 * 128;
 }
 
-// A slot's walk over its chunks, kept by its thread 0 in shared memory (in registers every thread would have to spare them):
-// its place in the tensor table, and of the current and the next chunk (by turns) the first element, the row length and
-// the first record.
-struct DecodeWalk {
-    DemoTensorEntry te;
-    long long next_begin;  // chunk_begin of the entry after te (or "never")
-    long long rec[2];
-    long long elem[2];     // offset of the chunk's first element in its tensor
-    int e;
-    int tensor[2], n1[2];
-
-    __device__ __forceinline__ void load(const DemoTensorEntry *entries, int n)
-    {
-        te = entries[e];
-        next_begin = (e + 1 < n) ? entries[e + 1].chunk_begin : 0x7fffffffffffffffLL;
-    }
-    // Moves on to chunk c (ids only grow) and notes it in `which`.
-    template <int S>
-    __device__ __forceinline__ void seek(const DemoTensorEntry *entries, int n, long long c, int k, int which)
-    {
-        if (c >= next_begin) {
-            while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
-            load(entries, n);
-        }
-        const unsigned lc = (unsigned)(c - te.chunk_begin);
-        const unsigned k0 = lc / (unsigned)te.c1;
-        tensor[which] = te.tensor;
-        n1[which] = te.n1;
-        elem[which] = ((long long)k0 * te.n1 + (lc - k0 * (unsigned)te.c1)) * S;
-        rec[which] = te.rec_begin + (long long)lc * k;
-    }
-};
 static_assert(sizeof(DecodeWalk) <= 128, "reserved in decode_slot_bytes");
 
 // SIGNS: the parameter-server form -- sign(R) goes out as int8 per element, the parameters are neither read
@@ -72,7 +39,14 @@ static_assert(sizeof(DecodeWalk) <= 128, "reserved in decode_slot_bytes");
 // The x tile comes by 16-byte asynchronous copies, sixteen per thread, not by TMA: a tensor map has to be acquired by every
 // CTA that comes to a tensor, a fence that stands in front of the chunk (300M-class set, 168 matrices: 696 us with maps, 725
 // with a bulk copy per row, 624 like this; one matrix of that size: 612, 731, 597).
-template <int S, int THREADS, bool SIGNS = false>
+// How the records are added up, by k.  (One instantiation each: the loops of the larger k in the same kernel cost 8 us of the
+// 96 of 8192 x 8192, k = 32.)
+//   LISTED: up to 64 records per worker, staged; STAGED: up to 512, staged, in parts of 64; BARRIERS: straight from the
+//   payloads, a barrier per worker.  4096 x 4096, k = 128, STAGED instead of BARRIERS: s = 32, W = 2 55.0 -> 40.5 us, signs
+//   39.7 -> 35.1; s = 64, W = 8 / 64 47.9 / 160 -> 42.9 / 137 us, k = 200, W = 2 44.0 -> 34.1, but signs at s = 64, W = 8
+//   31.8 -> 36.9.
+enum { LISTED, STAGED, BARRIERS };
+template <int S, int THREADS, bool SIGNS, int KMODE>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -104,9 +78,9 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     // workers -- W small pieces from W buffers -- never stand in front of the scatter.  One copy group per chunk.
     // (The records of workers w_first .. of the chunk in walk slot `which`.)
     auto stage_batch = [&](int buf, int which, int w_first) {
-        if (k_eff <= 64) {
+        if (KMODE != BARRIERS) {
             const long long off = walk.rec[which];
-            const int sh = (k_eff > 32) ? 6 : 5;
+            const int sh = KMODE == STAGED ? stage_shift(k_eff) : (k_eff > 32) ? 6 : 5;
             DemoRecord *dst = stage_all + buf * STAGE_RECORDS;
 #pragma unroll
             for (int i = 0; i < STAGE_RECORDS / S; ++i) {
@@ -165,7 +139,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         };
         DemoRecord *stage = stage_all + buf * STAGE_RECORDS;
         // S = sum over workers in worker order (Decompress&Aggregate).
-        if (k_eff <= 64) {
+        if constexpr (KMODE != BARRIERS) {
             // Every warp owns the 32 rows of the tile its threads cleared and will transform (rows 32 w .. 32 w + 31
             // for warp w of the slot).  The records of up to sixteen workers (512 records) are staged in shared
             // memory with one round of global loads; then every warp walks the staged workers in order, reads ALL
@@ -173,8 +147,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             // A coordinate is only ever touched by one warp, so the order of the additions -- worker after worker,
             // hence bit-reproducible -- needs nothing but warp-level synchronisation.
             const int lane = t & 31, warp = t >> 5;
-            const int sh = (k_eff > 32) ? 6 : 5;          // a worker's records take 32 or 64 staging entries
-            const int wb = STAGE_RECORDS >> sh;           // workers per batch: 16 or 8
+            const int sh = KMODE == STAGED ? stage_shift(k_eff) : (k_eff > 32) ? 6 : 5;  // a worker's records take 2^sh staging entries
+            const int wb = STAGE_RECORDS >> sh;           // workers per batch: 16, 8 or fewer
             for (int w0 = 0; w0 < a.W; w0 += wb) {
                 // this batch's copies have landed (requested a chunk or a batch ago), for all threads; the tile is cleared, the
                 // next chunk looked up, and both warps are done with the other buffer: it takes the batch after this one --
@@ -203,33 +177,54 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                     St[at] += rc.val;
                     if (counts && mine) Cn[idx] += 1;
                 };
+                if constexpr (KMODE == STAGED) {  // a worker's records in parts of 64, the last one short
+                    const int more_sh = sh - 6;
+                    const int n_parts = nw << more_sh, last = (1 << more_sh) - 1;
+                    DemoRecord rc[4][2];
 #pragma unroll 1
-                for (int wl = 0; wl < nw;) {
-                    auto some = [&](auto count) {
-                        constexpr int U = decltype(count)::value;
-                        DemoRecord rc0[U], rc1[U];
+                    for (int part = 0; part < n_parts; part += 4) {
 #pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            rc0[u] = stage[((wl + u) << sh) + lane];
-                            if (two) rc1[u] = stage[((wl + u) << sh) + lane + 32];
+                        for (int u = 0; u < 4; ++u) {  // (behind the last part: within the buffer, not used)
+                            rc[u][0] = stage[((part + u) << 6 & (STAGE_RECORDS - 1)) + lane];
+                            rc[u][1] = stage[((part + u) << 6 & (STAGE_RECORDS - 1)) + lane + 32];
                         }
 #pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            add(rc0[u], lane < k_eff);
-                            if (two) add(rc1[u], lane + 32 < k_eff);
+                        for (int u = 0; u < 4; ++u) {
+                            const int rest = part + u < n_parts ? k_eff - (((part + u) & last) << 6) : 0;  // records from this part on
+                            add(rc[u][0], lane < rest);
+                            add(rc[u][1], lane + 32 < rest);
                             __syncwarp();
                         }
-                        wl += U;
-                    };
-                    if (wl + 4 <= nw)
-                        some(std::integral_constant<int, 4>{});
-                    else
-                        some(std::integral_constant<int, 1>{});
+                    }
+                } else {
+#pragma unroll 1
+                    for (int wl = 0; wl < nw;) {
+                        auto some = [&](auto count) {
+                            constexpr int U = decltype(count)::value;
+                            DemoRecord rc0[U], rc1[U];
+    #pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                rc0[u] = stage[((wl + u) << sh) + lane];
+                                if (two) rc1[u] = stage[((wl + u) << sh) + lane + 32];
+                            }
+    #pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                add(rc0[u], lane < k_eff);
+                                if (two) add(rc1[u], lane + 32 < k_eff);
+                                __syncwarp();
+                            }
+                            wl += U;
+                        };
+                        if (wl + 4 <= nw)
+                            some(std::integral_constant<int, 4>{});
+                        else
+                            some(std::integral_constant<int, 1>{});
+                    }
                 }
                 if (bad) atomicMax(a.status, DEMO_DEV_PAYLOAD);
             }
         } else {
-            // k > 64: a thread's records may fall into any row; a barrier per worker fixes the order of additions.
+            // A thread's records may fall into any row; a barrier per worker fixes the order of additions.
             // Records are fetched eight workers ahead so that one memory latency covers eight workers.
             const long long rec_off = walk.rec[which];
             sb.sync();
@@ -368,8 +363,14 @@ cudaError_t launch_decode(const DemoDecodeArgs &a, int sm_count, cudaStream_t st
     constexpr int TH = DECODE_THREADS;
     constexpr int NCH = TH / S;
     const size_t smem = decode_slot_bytes<S>(a.agg == 2) * NCH;
-    if (a.sign_ptrs != nullptr) return launch(decode_fast_kernel<S, TH, true>, TH, NCH, smem, sm_count, stream, a);
-    return launch(decode_fast_kernel<S, TH>, TH, NCH, smem, sm_count, stream, a);
+    auto pick = [&](auto signs) {
+        constexpr bool SIGNS = decltype(signs)::value;
+        if (a.k <= 64) return launch(decode_fast_kernel<S, TH, SIGNS, LISTED>, TH, NCH, smem, sm_count, stream, a);
+        if constexpr (!(SIGNS && S == 64))
+            if (a.k <= STAGE_RECORDS) return launch(decode_fast_kernel<S, TH, SIGNS, STAGED>, TH, NCH, smem, sm_count, stream, a);
+        return launch(decode_fast_kernel<S, TH, SIGNS, BARRIERS>, TH, NCH, smem, sm_count, stream, a);
+    };
+    return a.sign_ptrs != nullptr ? pick(std::true_type{}) : pick(std::false_type{});
 }
 
 // One CTA arms an mbarrier with a transaction count that no copy will ever satisfy and waits for it

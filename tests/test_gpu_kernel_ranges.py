@@ -66,6 +66,18 @@ def test_s128_halves_of_the_row_stage(k):
     r.close()
 
 
+@pytest.mark.parametrize("s", [32, 64])
+@pytest.mark.parametrize("k,workers,agg", [(64, 17, 0), (65, 5, 2), (128, 5, 0), (129, 3, 1), (256, 3, 2), (512, 2, 0), (513, 2, 0)])
+def test_decode_large_k(s, k, workers, agg):
+    """Records in parts of 64 (short last part), several workers per batch, one, and none staged; colliding coordinates."""
+    wl = inputs.Workload("dk", [(2 * s, 3 * s)], chunk=s, topk=k, num_workers=workers, grad_kind="normal", grad_std=0.01)
+    r = parity.Runner(wl, max_chunks=10**9, seed=k, agg=agg)
+    base = [g.clone() for g in r.streams[0].next()]
+    grads = [[(b.float() + 0.3 * o.float()).to(b.dtype) for b, o in zip(base, st.next())] for st in r.streams]
+    r.step(grads=grads)
+    r.close()
+
+
 @pytest.mark.parametrize("k,agg", [(48, 0), (49, 2), (64, 2), (65, 0), (192, 0), (193, 2)])
 def test_tensor_core_pairs(k, agg):
     """s = 64 under a random basis: listed and dense row stage, decode by warp order and by barriers, four and three groups per CTA;
