@@ -63,7 +63,6 @@ struct DemoDecodeArgs {
     float lr;
     float wd;
     int *status;
-    const void *tmap_x;  // optional tensor maps of the parameter tensors (see DemoCompressArgs); s = 128 only
     int agg;          // 0 sum, 1 mean over workers, 2 per-coordinate count-normalised mean (0/0 = 0)
     int phi;          // 0 sign, 1 identity
     float agg_scale;  // 1/W for the mean, else 1 (only the identity update sees it)
@@ -93,7 +92,7 @@ cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, int sm_count
 cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
 // s = 64 with TMA tensor maps (kernels_fast64.cu; cudaErrorNotSupported without them).
 cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
-// s = 128 (kernels_fast128.cu); need the TMA tensor maps (cudaErrorNotSupported without them).
+// s = 128 (kernels_fast128.cu); compress needs the TMA tensor maps (cudaErrorNotSupported without them).
 cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
 cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
 

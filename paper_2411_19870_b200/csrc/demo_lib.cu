@@ -71,7 +71,6 @@ struct demo_ctx {
     // the caller's pointers change.  NULL when the driver entry point is unavailable.
     PFN_cuTensorMapEncodeTiled encode = nullptr;
     CUtensorMap *d_tm_g = nullptr, *d_tm_m = nullptr;  // [W][T]
-    CUtensorMap *d_tm_x = nullptr;                     // [T], s = 128 only
     std::vector<CUtensorMap> h_tm;                     // staging, [T]
 
     // demo_step_host: host->device gradient copies run on their own stream so that the copy of worker
@@ -161,7 +160,6 @@ void release(demo_ctx *c)
     cudaFree(c->d_flat);
     cudaFree(c->d_tm_g);
     cudaFree(c->d_tm_m);
-    cudaFree(c->d_tm_x);
     for (cudaEvent_t e : c->ev_copied)
         if (e) cudaEventDestroy(e);
     if (c->ev_start) cudaEventDestroy(c->ev_start);
@@ -313,7 +311,6 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
             }
             ok = ok && cudaMalloc(&c->d_tm_g, W * T * sizeof(CUtensorMap)) == cudaSuccess;
             ok = ok && cudaMalloc(&c->d_tm_m, W * T * sizeof(CUtensorMap)) == cudaSuccess;
-            if (s == 128) ok = ok && cudaMalloc(&c->d_tm_x, T * sizeof(CUtensorMap)) == cudaSuccess;
         } else {
             cudaGetLastError();
         }
@@ -720,15 +717,9 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     cudaError_t err = sync_table<const DemoRecord *>(ctx->d_p, ctx->h_p.data(),
                                                      reinterpret_cast<const DemoRecord *const *>(payloads), W,
                                                      &ctx->p_valid, stream);
-    bool x_changed = false;
     if (err == cudaSuccess && params)
         err = sync_table<float *>(ctx->d_x, ctx->h_x.data(), const_cast<float *const *>(params), T, &ctx->x_valid,
-                                  stream, &x_changed);
-    if (err == cudaSuccess && params && ctx->d_tm_x && x_changed &&
-        !upload_tensor_maps(ctx, ctx->d_tm_x, params, false, stream)) {
-        err = cudaErrorInvalidValue;
-        ctx->x_valid = false;
-    }
+                                  stream);
     if (err == cudaSuccess && signs)
         err = sync_table<signed char *>(ctx->d_s, ctx->h_s.data(), const_cast<signed char *const *>(signs), T,
                                         &ctx->s_valid, stream);
@@ -772,7 +763,6 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.lr = ctx->cfg.lr;
     a.wd = ctx->cfg.weight_decay;
     a.status = ctx->d_status;
-    a.tmap_x = params ? ctx->d_tm_x : nullptr;
     a.agg = ctx->aggregation;
     a.phi = ctx->phi;
     a.agg_scale = (ctx->aggregation == DEMO_AGG_MEAN) ? 1.0f / (float)W : 1.0f;
@@ -837,13 +827,8 @@ demo_status demo_apply_signs(demo_ctx *ctx, const int8_t *const *signs, float *c
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const demo_status st = ensure_sign_tables(ctx);
     if (st != DEMO_OK) return st;
-    bool x_changed = false;
     cudaError_t err = sync_table<float *>(ctx->d_x, ctx->h_x.data(), const_cast<float *const *>(params), T,
-                                          &ctx->x_valid, stream, &x_changed);
-    if (err == cudaSuccess && ctx->d_tm_x && x_changed && !upload_tensor_maps(ctx, ctx->d_tm_x, params, false, stream)) {
-        err = cudaErrorInvalidValue;
-        ctx->x_valid = false;
-    }
+                                          &ctx->x_valid, stream);
     if (err == cudaSuccess)
         err = sync_table<signed char *>(ctx->d_s, ctx->h_s.data(),
                                         const_cast<signed char *const *>(reinterpret_cast<const signed char *const *>(signs)),

@@ -338,7 +338,12 @@ __device__ __forceinline__ void warp_ballot_select(Key key_of, unsigned n_all, u
 // ------------------------------------------------------------------------------------------------
 constexpr int STAGE_RECORDS = 512;  // records staged per batch of the scatter (sixteen workers at k <= 32)
 // A worker's records take 2^stage_shift(k) staging entries (k <= STAGE_RECORDS).
-__device__ __forceinline__ int stage_shift(int k) { return k > 32 ? 32 - __clz(k - 1) : 5; }
+__host__ __device__ inline int stage_shift(int k)
+{
+    int sh = 5;
+    while ((1 << sh) < k) ++sh;
+    return sh;
+}
 
 // A slot's walk over its chunks, kept by its thread 0 in shared memory (in registers every thread would have to spare them):
 // its place in the tensor table, and of the current and the next chunk (by turns) the first element, the row length and

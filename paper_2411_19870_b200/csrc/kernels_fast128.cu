@@ -15,13 +15,16 @@
 // select for degenerate chunks) -> records; sparse row stage of the inverse from the records, half of them by each half of
 // the CTA, fast column stage, residual m <- B - alpha * IDCT(kept) against the parked B, one TMA store of the new momentum
 // tile.  The next chunk's g tile comes in, and its m tile to L2, as soon as B is formed.  decode: scatter-add of the W payloads
-// in worker order, two inverse passes, sign, update; the x tile is staged into the (then dead) coefficient tile.
+// in worker order, two inverse passes, sign, update; half of the x tile is staged into the (then dead) coefficient tile.
 // Two CTAs of a serial chain of phases per SM are what registers (128 for the 64-point halves) and, for compress, shared
 // memory allow: shared-memory accesses and issue each take about half of the time.  8192 x 8192, k = 32, bf16 gradients:
-// compress 242 -> 222 us (k = 128 313 -> 272) with the halves of the row stage and the early g tile, decode 162 -> 141 us and
-// signs 235 -> 131 us with half the exchange (before, the signs form kept two sets of 64 results and spilled).
+// compress 242 -> 222 us (k = 128 313 -> 272) with the halves of the row stage and the early g tile; decode 162 -> 141 us and
+// signs 235 -> 131 us with half the exchange (before, the signs form kept two sets of 64 results and spilled), W = 8
+// 155 -> 145 and 131 -> 121 us with staged records and the x tile in halves.
 // Tiles need the TMA tensor maps; without them the host uses the generic kernels for s = 128.
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "demo_internal.h"
 #include "fast_common.cuh"
@@ -620,101 +623,177 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
     tmem_free_cta(tmem_base, TMEM_COLS128);
 }
 
-constexpr size_t decode128_smem(bool counts) { return (size_t)S * XSD * 4 + 16 + (counts ? (size_t)M * 2 : 0); }
+// Decode: the tile, the walk, two staging buffers of records, and the landing area of the upper half of the x tile (before
+// that, of the sender counts of the count-normalised mean).
+constexpr size_t DECODE128_SMEM = (size_t)S * XSD * 4 + 128 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + M / 2 * sizeof(float);
 
 // SIGNS: the parameter-server form -- sign(R) goes out as int8, the parameters are not touched.
-template <bool SIGNS>
+// STAGED: records are staged a chunk ahead and every warp adds those of its 16 rows, worker after worker; otherwise they
+// come straight from the payloads with a barrier per worker.
+// The upper half of the x tile comes in behind the scatter and the transforms, the lower half, already in L2, into the dead
+// coefficient tile while the upper one is updated; by 16-byte asynchronous copies, without tensor maps (kernels_fast.cu).
+template <bool SIGNS, bool STAGED>
 __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    float *St = reinterpret_cast<float *>(smem_raw);  // [128*132] aggregate / intermediate; later the x tile [128*128]
-    float *Xt = St;
-    unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(St + S * XSD);
-    unsigned short *Cn = reinterpret_cast<unsigned short *>(bar_mem + 2);  // [M] senders per coordinate (agg == 2)
+    float *St = reinterpret_cast<float *>(smem_raw);  // [128*129] aggregate / intermediate; later rows 64.. of x [64*128]
+    DecodeWalk &walk = *reinterpret_cast<DecodeWalk *>(St + S * XSD);
+    DemoRecord *stage_all = reinterpret_cast<DemoRecord *>(reinterpret_cast<unsigned char *>(&walk) + 128);  // [2][STAGE_RECORDS]
+    float *Xh = reinterpret_cast<float *>(stage_all + 2 * STAGE_RECORDS);  // [64*128] rows ..63 of x
+    unsigned short *Cn = reinterpret_cast<unsigned short *>(Xh);           // [M] senders per coordinate (agg == 2)
+    __shared__ unsigned drawn[2];
 
-    const int tid = threadIdx.x, h = tid >> 7, j = tid & 127;
-    const uint32_t bar = smem_u32(bar_mem);
-    if (tid == 0) {
-        mbar_init(bar, 1);
-        fence_proxy_async();
-    }
-    __syncthreads();
-    fence_proxy_async();
-
-    EntryCursor cur;
-    unsigned phase = 0;
+    const int tid = threadIdx.x, h = tid >> 7, j = tid & 127, lane = tid & 31, warp = tid >> 5;
+    const int k_eff = a.k;
+    const unsigned n_chunks = (unsigned)a.n_chunks;  // (fewer than 2^31)
     const unsigned lr_bits = __float_as_uint(a.lr);
     const float decay = 1.f - a.lr * a.wd;
     const float neg_lr_scale = -a.lr * a.agg_scale;
     const bool counts = a.agg == 2;
-    const char *acquired = nullptr;
 
-    volatile unsigned *next_slot = reinterpret_cast<volatile unsigned *>(bar_mem + 1);
-    for (long long c = blockIdx.x; c < a.n_chunks; c = (long long)gridDim.x + *next_slot) {
-        cur.seek(a.entries, a.n_entries, c);
-        const DemoTensorEntry te = cur.te;
-        const unsigned lc = (unsigned)(c - te.chunk_begin);
-        const unsigned k0 = lc / (unsigned)te.c1, k1 = lc - k0 * (unsigned)te.c1;
-        const size_t base = (size_t)k0 * S * (size_t)te.n1 + (size_t)k1 * S;
-        float *__restrict__ x = a.x_ptrs[te.tensor];
-        const int k_eff = te.k_eff;
-        const long long rec_off = te.rec_begin + (long long)lc * k_eff;
-        const char *tm_x = static_cast<const char *>(a.tmap_x) + (size_t)te.tensor * TMAP_BYTES;
-        if (!SIGNS && tid == 0) {
-            if (tm_x != acquired) {  // first use of this tensor's map by this thread
-                acquired = tm_x;
-                tmap_acquire(tm_x);
-            }
-            tma_prefetch_2d(tm_x, k1 * S, k0 * S);
+    // the records of workers w_first .. of the chunk in walk slot `which`; one copy group per call
+    auto stage_batch = [&](int buf, int which, int w_first) {
+        const long long off = walk.rec[which];
+        const int sh = stage_shift(k_eff);
+        DemoRecord *dst = stage_all + buf * STAGE_RECORDS;
+#pragma unroll
+        for (int i = 0; i < STAGE_RECORDS / THREADS; ++i) {
+            const int r = i * THREADS + tid, wl = w_first + (r >> sh), q = r & ((1 << sh) - 1);
+            if (wl < a.W && q < k_eff)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst + r)), "l"(a.payloads[wl] + off + q)
+                             : "memory");
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
 
+    unsigned c = blockIdx.x, par = 0;
+    int buf = 0, which = 0;  // staging buffer and walk slot of the current chunk
+    if (tid == 0) {
+        drawn[0] = ticket_draw(a.tickets);
+        if (c < n_chunks) {
+            walk.e = demo_find_entry(a.entries, a.n_entries, c);
+            walk.load(a.entries, a.n_entries);
+            walk.seek<S>(a.entries, a.n_entries, c, k_eff, 0);
+        }
+    }
+    __syncthreads();
+    if (STAGED && c < n_chunks) stage_batch(0, 0, 0);
+    for (unsigned nc; c < n_chunks; c = nc, par ^= 1u, which ^= 1) {
+        __syncthreads();  // (publishes the draw; the tile and the landing area are free)
+        nc = gridDim.x + drawn[par];
+        unsigned ticket = 0;
+        if (tid == 0) {
+            ticket = ticket_draw(a.tickets);
+            if (nc < n_chunks) walk.seek<S>(a.entries, a.n_entries, nc, k_eff, which ^ 1);
+        }
+        // 64 rows of the x tile, one copy group
+        auto fetch_rows = [&](float *dst, int row0) {
+            const int n1 = walk.n1[which];
+            const float *src = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)(row0 + warp) * n1 + lane * 4;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + (warp + 8 * i) * S + lane * 4)),
+                             "l"(src + (size_t)(8 * i) * n1)
+                             : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (!SIGNS) {
+            if (!counts) fetch_rows(Xh, 0);
+            const float *xr = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)(64 + (tid >> 2)) * walk.n1[which] + (tid & 3) * 32;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
+        }
         for (int i = tid; i < S * XSD / 4; i += THREADS) reinterpret_cast<float4 *>(St)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (counts)
-            for (int i = tid; i < M; i += THREADS) Cn[i] = 0;
-        __syncthreads();
-        // S = sum over workers in worker order (a barrier per worker fixes the order of additions)
-        for (int kb = 0; kb < k_eff; kb += THREADS) {
-            const bool mine = kb + tid < k_eff;
-            for (int w0 = 0; w0 < a.W; w0 += 8) {
-                DemoRecord r[8];
+            for (int i = tid; i < M / 2; i += THREADS) reinterpret_cast<unsigned *>(Cn)[i] = 0u;
+        // S = sum over workers in worker order (Decompress&Aggregate)
+        if constexpr (STAGED) {
+            const int sh = stage_shift(k_eff), wb = STAGE_RECORDS >> sh;
+            for (int w0 = 0; w0 < a.W; w0 += wb) {
+                // the records have landed (requested a chunk or a batch ago; only the rows of x are younger), the tile is cleared,
+                // the next chunk looked up, and all warps are done with the other buffer
+                if (!SIGNS && !counts && w0 == 0)
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                else
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncthreads();
+                const DemoRecord *stage = stage_all + buf * STAGE_RECORDS;
+                buf ^= 1;
+                if (w0 + wb < a.W)
+                    stage_batch(buf, which, w0 + wb);
+                else if (nc < n_chunks)
+                    stage_batch(buf, which ^ 1, 0);
+                else
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                // branch-free as in kernels_fast.cu: a record of another warp's rows goes to a padding element
+                const int spare = (16 * warp + (lane & 15)) * XSD + S;
+                bool bad = false;
+                const int n_pieces = min(wb, a.W - w0) << (sh - 5), last = (1 << (sh - 5)) - 1;  // 32 records each
+#pragma unroll 1
+                for (int q0 = 0; q0 < n_pieces; q0 += 4) {
+                    DemoRecord rc[4];
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (mine && w0 + q < a.W) r[q] = a.payloads[w0 + q][rec_off + kb + tid];
+                    for (int u = 0; u < 4; ++u) rc[u] = stage[((q0 + u) << 5 & (STAGE_RECORDS - 1)) + lane];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (w0 + q < a.W) {
-                        if (mine) {
-                            if ((unsigned)r[q].idx < (unsigned)M) {
-                                St[(r[q].idx >> 7) * XSD + (r[q].idx & 127)] += r[q].val;
-                                if (counts) Cn[r[q].idx] += 1;
-                            } else {
-                                atomicMax(a.status, DEMO_DEV_PAYLOAD);
+                    for (int u = 0; u < 4; ++u) {
+                        const bool have = q0 + u < n_pieces && lane < k_eff - (((q0 + u) & last) << 5);
+                        const unsigned idx = (unsigned)rc[u].idx;
+                        bad = bad || (have && idx >= (unsigned)M);
+                        const bool mine = have && (idx >> 11) == (unsigned)warp;  // (false for idx >= M)
+                        const int at = mine ? (int)(idx >> 7) * XSD + (int)(idx & 127) : spare;
+                        St[at] += rc[u].val;
+                        if (counts && mine) Cn[idx] += 1;
+                        __syncwarp();
+                    }
+                }
+                if (bad) atomicMax(a.status, DEMO_DEV_PAYLOAD);
+            }
+        } else {
+            const long long rec_off = walk.rec[which];
+            __syncthreads();
+            for (int kb = 0; kb < k_eff; kb += THREADS) {
+                const bool mine = kb + tid < k_eff;
+                for (int w0 = 0; w0 < a.W; w0 += 8) {  // fetched eight workers ahead
+                    DemoRecord r[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        if (mine && w0 + q < a.W) r[q] = a.payloads[w0 + q][rec_off + kb + tid];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if (w0 + q < a.W) {
+                            if (mine) {
+                                if ((unsigned)r[q].idx < (unsigned)M) {
+                                    St[(r[q].idx >> 7) * XSD + (r[q].idx & 127)] += r[q].val;
+                                    if (counts) Cn[r[q].idx] += 1;
+                                } else {
+                                    atomicMax(a.status, DEMO_DEV_PAYLOAD);
+                                }
                             }
+                            __syncthreads();
                         }
-                        __syncthreads();
                     }
                 }
             }
         }
+        if (tid == 0) drawn[par ^ 1u] = ticket;
+        __syncthreads();
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
             for (int i = tid; i < M; i += THREADS) {
                 const unsigned short n = Cn[i];
                 if (n > 1) St[(i >> 7) * XSD + (i & 127)] /= (float)n;
             }
             __syncthreads();
+            if (!SIGNS) fetch_rows(Xh, 0);
         }
         // two inverse passes (rolled): both walk "row j" of the tile with unit stride -- pass 0 leaves its result
         // transposed, so that the columns pass 1 needs are rows again and every access below has a fixed offset
         float lo[H / 2], hi[H / 2];
-        bool arrived = true;
         float *ln = St + j * XSD;  // line j
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
             float in[H], keep[H / 2];
 #pragma unroll
             for (int p = 0; p < H; ++p) in[p] = ln[2 * p + h];
-            fence_proxy_async();
             __syncthreads();  // every coefficient of the tile has been read
             inverse_half(h, in, keep, lo);
             // exchange halves of e / o inside the line
@@ -725,7 +804,6 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
 #pragma unroll
             for (int q = 0; q < H / 2; ++q) hi[q] = theirs[q];
             inverse_join(h, keep, lo, hi);  // elements 32h + q and 127 - 32h - q
-            fence_proxy_async();
             __syncthreads();  // both halves of every line have read their partner's values
             if (pass == 0) {
                 // element n of row j goes to row n, column j
@@ -736,53 +814,40 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                     Shi[-q * XSD] = hi[q];
                 }
                 __syncthreads();
-            } else if (SIGNS) {
-                if (tid == 0) *next_slot = ticket_draw(a.tickets);
-            } else {
-                unsigned ticket = 0;  // (thread 0) the CTA's next chunk, drawn behind the wait for the tile
-                if (tid == 0) {
-                    ticket = ticket_draw(a.tickets);
-                    mbar_expect_tx(bar, M * sizeof(float));
-                    tma_load_2d(smem_u32(Xt), tm_x, k1 * S, k0 * S, bar);
-                }
-                arrived = mbar_wait_bounded(bar, phase);
-                phase ^= 1u;
-                if (tid == 0) *next_slot = ticket;
             }
         }
-        const ptrdiff_t n1 = te.n1;
-        const size_t at_lo = base + (size_t)((H / 2) * h) * te.n1 + j, at_hi = base + (size_t)(S - 1 - (H / 2) * h) * te.n1 + j;
+        // thread (h, j) holds rows 32h + q and 127 - 32h - q of column j
+        const ptrdiff_t n1 = walk.n1[which];
+        const size_t at_lo = walk.elem[which] + (size_t)((H / 2) * h) * n1 + j, at_hi = walk.elem[which] + (size_t)(S - 1 - (H / 2) * h) * n1 + j;
         if constexpr (SIGNS) {
-            signed char *__restrict__ slo = a.sign_ptrs[te.tensor] + at_lo, *__restrict__ shi = a.sign_ptrs[te.tensor] + at_hi;
+            signed char *__restrict__ slo = a.sign_ptrs[walk.tensor[which]] + at_lo, *__restrict__ shi = a.sign_ptrs[walk.tensor[which]] + at_hi;
 #pragma unroll
             for (int q = 0; q < H / 2; ++q) {
                 slo[q * n1] = (signed char)((lo[q] > 0.f) - (lo[q] < 0.f));
                 shi[-q * n1] = (signed char)((hi[q] > 0.f) - (hi[q] < 0.f));
             }
-            __syncthreads();
             continue;
         }
-        if (!__syncthreads_and(arrived)) {
-            if (tid == 0) atomicMax(a.status, DEMO_DEV_TIMEOUT);
-            mbar_wait_bounded(bar, phase ^ 1u);
-            break;
-        }
+        fetch_rows(St, 64);
         auto updated = [&](float rv, float xv) {
             float stepv = __uint_as_float(lr_bits ^ (~__float_as_uint(rv) & 0x80000000u));
             stepv = (rv == 0.f) ? 0.f : stepv;
             if (a.phi) stepv = rv * neg_lr_scale;  // phi = identity
             return fmaf(xv, decay, stepv);
         };
-        const float *Xlo = Xt + (H / 2) * h * S + j, *Xhi = Xt + (S - 1 - (H / 2) * h) * S + j;
-        float *__restrict__ xlo = x + at_lo, *__restrict__ xhi = x + at_hi;
-#pragma unroll
-        for (int q = 0; q < H / 2; ++q) {
-            xlo[q * n1] = updated(lo[q], Xlo[q * S]);
-            xhi[-q * n1] = updated(hi[q], Xhi[-q * S]);
-        }
-        fence_proxy_async();
+        float *__restrict__ xlo = a.x_ptrs[walk.tensor[which]] + at_lo, *__restrict__ xhi = a.x_ptrs[walk.tensor[which]] + at_hi;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");  // all but the lower rows
         __syncthreads();
+        const float *Xlo = Xh + (H / 2) * h * S + j;
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) xlo[q * n1] = updated(lo[q], Xlo[q * S]);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const float *Xhi = St + (63 - (H / 2) * h) * S + j;
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) xhi[-q * n1] = updated(hi[q], Xhi[-q * S]);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");  // no copy may outlive the CTA's shared memory
     if (tid == 0) ticket_finish(a.tickets);
 }
 
@@ -817,7 +882,15 @@ cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, int sm_count
 
 cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
-    if (a.sign_ptrs) return launch128(decode_fast128_kernel<true>, decode128_smem(a.agg == 2), sm_count, stream, a);
-    if (!a.tmap_x) return cudaErrorNotSupported;
-    return launch128(decode_fast128_kernel<false>, decode128_smem(a.agg == 2), sm_count, stream, a);
+    // Staged while the additions are short (k <= 64) or all workers' records fit one batch; a further batch of longer lists
+    // comes too late.  8192 x 8192, staged / with barriers: k = 32, W = 1 139 / 149 us, W = 8 145 / 169 us, k = 64, W = 8
+    // 156 / 164, k = 128, W = 1 139 / 149, W = 8 182 / 165 us; 4096 x 4096, k = 32, W = 64 62 / 103 us, k = 128, W = 32
+    // 85 / 75 us.
+    const bool staged = a.k <= 64 || (a.k <= STAGE_RECORDS && (long long)a.W << stage_shift(a.k) <= STAGE_RECORDS);
+    auto pick = [&](auto signs) {
+        constexpr bool SIGNS = decltype(signs)::value;
+        return staged ? launch128(decode_fast128_kernel<SIGNS, true>, DECODE128_SMEM, sm_count, stream, a)
+                      : launch128(decode_fast128_kernel<SIGNS, false>, DECODE128_SMEM, sm_count, stream, a);
+    };
+    return a.sign_ptrs ? pick(std::true_type{}) : pick(std::false_type{});
 }

@@ -579,7 +579,6 @@ extern "C" demo_status demo_decode_apply_static(const demo_config *cfg, const de
         a.lr = cfg->lr;
         a.wd = cfg->weight_decay;
         a.status = reinterpret_cast<int *>(base + OFF_STATUS);
-        a.tmap_x = nullptr;
         a.agg = 0;
         a.phi = 0;
         a.agg_scale = 1.f;

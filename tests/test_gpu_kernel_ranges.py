@@ -66,7 +66,7 @@ def test_s128_halves_of_the_row_stage(k):
     r.close()
 
 
-@pytest.mark.parametrize("s", [32, 64])
+@pytest.mark.parametrize("s", [32, 64, 128])
 @pytest.mark.parametrize("k,workers,agg", [(64, 17, 0), (65, 5, 2), (128, 5, 0), (129, 3, 1), (256, 3, 2), (512, 2, 0), (513, 2, 0)])
 def test_decode_large_k(s, k, workers, agg):
     """Records in parts of 64 (short last part), several workers per batch, one, and none staged; colliding coordinates."""
