@@ -17,9 +17,11 @@
 //     coalesced row piece per load; a transpose through the tile gives the second stage its rows; the inverse's row stage is
 //     k rank-1 updates on the CUDA cores (as in kernels_fast64.cu), its column stage one more tensor-core stage whose result
 //     is column j of the residual update: loads and stores of the momentum are coalesced and B is formed again from L2.
-// 4096 x 8192, bf16 gradients, two workers: compress k = 32 199 us, k = 128 247 us, decode 108 / 123 us (378 and 236 us at
-// k = 32 with both operands in shared memory, 64 KB per pair, two pairs per SM and four stages).  Every wait is bounded: on expiry the group records DEMO_DEV_TIMEOUT and stops, the CTA frees its tensor
-// memory and returns.
+// 4096 x 8192, bf16 gradients, two workers: compress k = 32 185 us, k = 128 234 us, decode 108 / 123 us (378 and 236 us at
+// k = 32 with both operands in shared memory, 64 KB per pair, two pairs per SM and four stages).  A third of compress
+// is the two passes over the momentum: the next pair's tiles are brought to L2 during the selection and read 32 rows at a
+// time (without: 199 us).  Every wait is bounded: on expiry the group records DEMO_DEV_TIMEOUT and stops, the CTA frees its
+// tensor memory and returns.
 #include <cuda_bf16.h>
 
 #include "demo_internal.h"
@@ -289,8 +291,8 @@ __device__ __forceinline__ void write_row(float *X, int r, const float (&v)[S])
 }
 
 // BIGK (k > MAX_K_LISTED): selection from quarter-row maxima with the wide list (3 groups fit), both inverse stages dense.
-// The same sizes as above: from the list k = 40 / 48 204 / 244 us (at 48 part of the lists overflow into the radix select),
-// dense k = 49 / 128 / 300 240 / 247 / 605 us.
+// Without the prefetch, the same sizes: from the list k = 40 / 48 204 / 244 us (at 48 part of the lists overflow into the radix
+// select), dense k = 49 / 128 / 300 240 / 247 / 605 us.
 template <typename GT, int GROUPS, bool BIGK>
 __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(DemoCompressArgs a)
 {
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
             cr = locate(a.entries, a.n_entries, chunk, k_eff, e);
             m = a.m_ptrs[cr.tensor] + cr.elem + r;
             g = static_cast<const GT *>(a.g_ptrs[cr.tensor]) + cr.elem + r;
-            each_b<16>(m, g, cr.n1, a.beta, [&](int i, float b) { v[i] = b; });
+            each_b<32>(m, g, cr.n1, a.beta, [&](int i, float b) { v[i] = b; });
         } else {
 #pragma unroll
             for (int i = 0; i < S; ++i) v[i] = 0.f;
@@ -349,6 +351,17 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         ok = tc_stage(f, pb, v, 0);
         if (!ok) break;
         const unsigned next = *f.drawn;  // (written before the barriers of the stages; overwritten behind those below)
+        if (2u * next + c < n_chunks) {  // row r of the group's next tiles on its way to L2
+            int e2 = e;
+            const ChunkRef nr = locate(a.entries, a.n_entries, 2u * next + c, k_eff, e2);
+            const size_t at = nr.elem + (size_t)r * nr.n1;
+            const float *nm = a.m_ptrs[nr.tensor] + at;
+            const GT *ng = static_cast<const GT *>(a.g_ptrs[nr.tensor]) + at;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(nm));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(nm + 32));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(ng));
+            if (sizeof(GT) == 4) asm volatile("prefetch.global.L2 [%0];" ::"l"(ng + 32));
+        }
 
         // ---- exact top-k, records, and the row stage of the inverse -------------------------------------------
         if constexpr (BIGK) {
@@ -395,7 +408,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         // ---- column stage; momentum subtraction  m <- B - alpha R  (Section 2.1) --------------------------------
         ok = tc_stage(f, pb, v, 1);
         if (!ok) break;
-        if (valid) each_b<8>(m, g, cr.n1, a.beta, [&](int i, float b) { m[(size_t)i * cr.n1] = b - v[i]; });
+        if (valid) each_b<BIGK ? 16 : 8>(m, g, cr.n1, a.beta, [&](int i, float b) { m[(size_t)i * cr.n1] = b - v[i]; });
         p = next;
     }
     if (!ok && f.pt == 0) atomicMax(a.status, DEMO_DEV_TIMEOUT);
