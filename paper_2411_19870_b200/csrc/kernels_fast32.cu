@@ -4,7 +4,7 @@
 //
 // A chunk is small enough that no step needs more than a warp-level barrier, so the chunks of an SM (twenty with bf16
 // gradients, sixteen with fp32) run in phases of their own and their loads, transforms, selections and stores overlap.
-// Instruction issue bounds it: about 1600 instructions per chunk, issued in 65 % of the cycles, next to which the 10 KB
+// Instruction issue bounds it: about 1660 instructions per chunk, issued in 62 % of the cycles, next to which the 10 KB
 // that a chunk moves cost less.  The next chunk's tiles come in by 16-byte asynchronous copies (they need no tensor map,
 // whose acquisition costs about a microsecond per tensor) as soon as this chunk's have been read; B is parked in tensor
 // memory between the load and the residual (in registers only sixteen warps fit: 8192 x 8192 154 us instead of 144); the new
