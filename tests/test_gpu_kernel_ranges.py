@@ -1,5 +1,7 @@
 """Edges of the size ranges the kernel variants are chosen by, against the fp64 oracle (rules and tolerances of
 tests/parity.py, every chunk)."""
+import ctypes
+import math
 import types
 
 import pytest
@@ -167,3 +169,84 @@ def test_apply_signs_pieces(shapes):
     for got, ref in zip(x, want):  # two fused multiply-adds: at most one rounding each of values below 4
         assert (got.double() - ref).abs().max().item() <= 2 ** -22
     tr.close()
+
+
+class Flat:
+    """A set of equal tensors laid one behind the other in flat buffers, and the calls on it through the C ABI with pointer
+    arrays made once (the binding would look at every tensor in every call)."""
+
+    def __init__(self, count, shape, chunk, topk, basis=None):
+        import paper_2411_19870_b200 as demo
+
+        self.tr = demo.DemoTransform([shape] * count, chunk=chunk, topk=topk, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=1)
+        if basis is not None:
+            self.tr.set_basis(basis)
+        n, gen = count * math.prod(shape), torch.Generator("cuda").manual_seed(11)
+        self.m = torch.randn(n, device="cuda", generator=gen)
+        self.g = torch.randn(n, device="cuda", generator=gen).bfloat16()
+        self.x = torch.randn(n, device="cuda", generator=gen)
+        each = math.prod(shape)
+        rows = torch.zeros(count, -(-each // 16) * 16, dtype=torch.int8, device="cuda")  # tensors start on 16-byte boundaries
+        self.signs = rows[:, :each]
+        self.payload = torch.zeros(self.tr.payload_bytes, dtype=torch.uint8, device="cuda")
+
+        def pointers(t):
+            step = (rows.shape[1] if t is self.signs else each) * t.element_size()
+            return (ctypes.c_void_p * count)(*range(t.data_ptr(), t.data_ptr() + count * step, step))
+
+        self.ptr = {k: pointers(getattr(self, k)) for k in ("m", "g", "x", "signs")}
+        self.payloads = (ctypes.c_void_p * 1)(self.payload.data_ptr())
+
+    def call(self, what):
+        lib, ctx, p = self.tr.lib, self.tr._ctx, self.ptr
+        stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if what == "compress":
+            st = lib.demo_compress(ctx, 0, p["g"], p["m"], ctypes.c_void_p(self.payload.data_ptr()), stream)
+        elif what == "decode":
+            st = lib.demo_decode_apply(ctx, self.payloads, 1, p["x"], stream)
+        elif what == "signs":
+            st = lib.demo_decode_signs(ctx, self.payloads, 1, p["signs"], stream)
+        else:
+            st = lib.demo_apply_signs(ctx, p["signs"], p["x"], stream)
+        assert st == 0, what
+
+    def device_us(self, what):
+        """Time of one call on the device (calls of a captured graph), the best of several."""
+        self.call(what)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(4):
+                self.call(what)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        best = math.inf
+        for _ in range(8):
+            t0.record()
+            graph.replay()
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1) / 4 * 1e3)
+        return best
+
+
+def check_many_tensors(count, shape, chunk, calls, slower, topk=4, basis=None):
+    """`count` tensors against one tensor of the same chunks: the same bits, and a call at most `slower` times as long (a call
+    looks its tensors up in a table; a search one entry after the other makes it tens of times as long)."""
+    many = Flat(count, shape, chunk, topk, basis)
+    one = Flat(1, (count * shape[0],) + shape[1:], chunk, topk, basis)
+    for what in ("compress", "decode", "signs", "apply"):
+        many.call(what)
+        one.call(what)
+    for k in ("m", "payload", "x", "signs"):
+        assert torch.equal(getattr(many, k).reshape(-1), getattr(one, k).reshape(-1)), k
+    for what in calls:
+        a, b = many.device_us(what), one.device_us(what)
+        assert a <= slower * b + 5.0, "%s: %.1f us, one tensor %.1f us" % (what, a, b)
+    many.tr.close()
+    one.tr.close()
+
+
+@pytest.mark.parametrize("count", [2, 32, 33, 1024, 1025, 20000])
+@pytest.mark.parametrize("s", [8, 64, 128])
+def test_many_vectors(s, count):
+    check_many_tensors(count, (s,), s, ["compress", "decode"] if count == 20000 else [], 5.0)
