@@ -191,7 +191,7 @@ struct DemoNdDecodeArgs {
 
 // x <- x - lr (sign + wd x) from int8 signs, over every tensor of a context (kernels_generic.cu).
 struct DemoFlatEntry {
-    long long piece_begin;  // index of this tensor's first piece of demo_apply_piece() elements in the launch
+    long long piece_begin;  // index of this tensor's first piece in the launch
     long long n;            // elements
     int tensor;             // position in the pointer arrays
     int pad;
@@ -200,11 +200,12 @@ struct DemoApplySignsArgs {
     const DemoFlatEntry *entries;  // device
     int n_entries;
     long long n_pieces;
+    int piece;                            // elements per piece: one of demo_apply_pieces
     const signed char *const *sign_ptrs;  // device array
     float *const *x_ptrs;                 // device array
     float lr, wd;
 };
-int demo_apply_piece();
+constexpr int demo_apply_pieces[2] = {1024, 4};  // a block's, a thread's
 cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, cudaStream_t stream);
 
 cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, cudaStream_t stream);
@@ -223,6 +224,24 @@ __device__ __forceinline__ int demo_find_entry(const DemoTensorEntry *entries, i
     }
     return lo;
 }
+
+// (warp) the last i of lo .. lo + n - 1 with below(i), which holds for lo and up to some i.  32 places are compared at once, so up to
+// 32 entries take one round of loads, up to 2^20 four.  (In steps of 32 entries instead: decode of 20000 vectors of 64 elements 647 us
+// instead of 44, of 100000 15.2 ms instead of 0.22.)
+#ifdef __CUDACC__
+template <class Below>
+__device__ __forceinline__ int demo_find_warp(int lo, int n, Below below)
+{
+    const int lane = threadIdx.x & 31;
+    while (n > 1) {
+        const int step = (n + 31) / 32, i = lane * step;
+        const int last = __popc(__ballot_sync(0xffffffffu, i < n && below(lo + i))) - 1;
+        lo += last * step;
+        n = n - last * step < step ? n - last * step : step;
+    }
+    return lo;
+}
+#endif
 
 // Status values written by kernels (match demo_status in include/demo.h).
 #define DEMO_DEV_TIMEOUT 7

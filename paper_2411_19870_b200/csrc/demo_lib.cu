@@ -61,6 +61,7 @@ struct demo_ctx {
     bool s_valid = false;
     DemoFlatEntry *d_flat = nullptr;   // [T] element ranges for demo_apply_signs
     long long n_pieces = 0;
+    int piece = 0;                     // elements per piece
     std::vector<const void *> h_g;
     std::vector<float *> h_m, h_x;
     std::vector<const DemoRecord *> h_p;
@@ -663,13 +664,19 @@ static demo_status ensure_sign_tables(demo_ctx *ctx)
     } catch (const std::bad_alloc &) {
         return DEMO_ERR_ALLOC;
     }
-    long long q = 0;
-    for (int t = 0; t < T; ++t) {
-        flat[t].piece_begin = q;
-        flat[t].n = ctx->n_elems[t];
-        flat[t].tensor = t;
-        flat[t].pad = 0;
-        q += (ctx->n_elems[t] + demo_apply_piece() - 1) / demo_apply_piece();
+    long long q = 0, elems = 0;
+    for (const int piece : demo_apply_pieces) {
+        q = elems = 0;
+        for (int t = 0; t < T; ++t) {
+            flat[t].piece_begin = q;
+            flat[t].n = ctx->n_elems[t];
+            flat[t].tensor = t;
+            flat[t].pad = 0;
+            q += (ctx->n_elems[t] + piece - 1) / piece;
+            elems += ctx->n_elems[t];
+        }
+        ctx->piece = piece;
+        if (2 * elems >= piece * q) break;  // pieces of a block at least half full on average; otherwise those of a thread
     }
     ctx->n_pieces = q;
     if (!ctx->d_s && cudaMalloc((void **)&ctx->d_s, (size_t)T * sizeof(void *)) != cudaSuccess) {
@@ -838,6 +845,7 @@ demo_status demo_apply_signs(demo_ctx *ctx, const int8_t *const *signs, float *c
         a.entries = ctx->d_flat;
         a.n_entries = T;
         a.n_pieces = ctx->n_pieces;
+        a.piece = ctx->piece;
         a.sign_ptrs = ctx->d_s;
         a.x_ptrs = ctx->d_x;
         a.lr = ctx->cfg.lr;

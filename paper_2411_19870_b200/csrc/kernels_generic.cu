@@ -233,34 +233,48 @@ __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeA
 }
 
 // x <- x - lr (sign + wd x) with the signs a parameter server handed out (Algorithm 1, last two lines); same arithmetic as
-// the decode kernels.  Bound by HBM (9 bytes per parameter).  A block takes pieces of APPLY_PIECE elements of one tensor, a
-// grid apart, four consecutive elements per thread; the tensor is looked up once per piece, 32 table entries at a time, not by
-// a binary search for every group of four elements (168 matrices, 454 M parameters: 780 -> 632 us, 6.5 TB/s).  Pieces of 8 or
-// 16 elements per thread, with their loads together, took 7 % longer.
-constexpr int APPLY_PIECE = 4 * GEN_THREADS;
+// the decode kernels.  Bound by HBM (9 bytes per parameter).  Four consecutive elements per thread.
+// BLOCKS: a block takes pieces of 1024 elements of one tensor, a grid apart, and looks the tensor up once per piece (168 matrices,
+// 454 M parameters: 632 us, 6.5 TB/s, against 780 us with a search for every four elements; pieces of 8 or 16 elements per thread,
+// with their loads together, 7 % longer).  Otherwise a thread takes pieces of four elements and searches for each: for sets whose
+// small tensors would leave blocks mostly idle (20000 vectors of 8 / 64 / 128 elements 5.5 / 8.2 / 11 us against 158 with a block per
+// vector).
+template <bool BLOCKS>
 __global__ void __launch_bounds__(GEN_THREADS) apply_signs_kernel(DemoApplySignsArgs a)
 {
-    const int lane = threadIdx.x & 31;
+    constexpr int PIECE = demo_apply_pieces[BLOCKS ? 0 : 1];
+    static_assert(PIECE == (BLOCKS ? 4 * GEN_THREADS : 4), "four elements per thread");
+    const int lane = threadIdx.x & 31, at = BLOCKS ? (int)threadIdx.x * 4 : 0;
+    const long long first = BLOCKS ? blockIdx.x : (long long)blockIdx.x * GEN_THREADS + threadIdx.x;
+    const long long stride = BLOCKS ? gridDim.x : (long long)gridDim.x * GEN_THREADS;
     int e = 0;  // the last entry with piece_begin <= q
     auto update = [&](float xv, signed char s) { return fmaf(-a.lr, fmaf(a.wd, xv, (float)s), xv); };
-    for (long long q = blockIdx.x; q < a.n_pieces; q += gridDim.x) {
-        for (;;) {
-            const int i = e + 1 + lane;
-            const int n = __popc(__ballot_sync(0xffffffffu, i < a.n_entries && a.entries[i].piece_begin <= q));
+    for (long long q = first; q < a.n_pieces; q += stride) {
+        auto below = [&](int i) { return a.entries[i].piece_begin <= q; };
+        if constexpr (BLOCKS) {
+            const int next = e + 1 + lane, n = __popc(__ballot_sync(0xffffffffu, next < a.n_entries && below(next)));
             e += n;
-            if (n < 32) break;
+            if (n == 32) e = demo_find_warp(e, a.n_entries - e, below);
+        } else {
+            int hi = a.n_entries - 1;
+            while (e < hi) {
+                const int mid = (e + hi + 1) >> 1;
+                if (below(mid))
+                    e = mid;
+                else
+                    hi = mid - 1;
+            }
         }
         const DemoFlatEntry en = a.entries[e];
-        const long long i0 = (q - en.piece_begin) * APPLY_PIECE, left = en.n - i0;
+        const long long i0 = (q - en.piece_begin) * PIECE, left = en.n - i0;
         float *__restrict__ x = a.x_ptrs[en.tensor] + i0;
         const signed char *__restrict__ sg = a.sign_ptrs[en.tensor] + i0;
-        const int at = (int)threadIdx.x * 4;
-        if (left >= APPLY_PIECE) {  // tensors start 16-byte aligned, so the pieces are aligned too
+        if (left >= PIECE) {  // tensors start 16-byte aligned, so the pieces are aligned too
             const float4 xv = *reinterpret_cast<const float4 *>(x + at);
             const char4 sv = *reinterpret_cast<const char4 *>(sg + at);
             *reinterpret_cast<float4 *>(x + at) = make_float4(update(xv.x, sv.x), update(xv.y, sv.y), update(xv.z, sv.z), update(xv.w, sv.w));
         } else {
-            for (int i = threadIdx.x; i < (int)left; i += GEN_THREADS) x[i] = update(x[i], sg[i]);
+            for (int i = BLOCKS ? threadIdx.x : 0; i < (int)left; i += BLOCKS ? GEN_THREADS : 1) x[i] = update(x[i], sg[i]);
         }
     }
 }
@@ -293,19 +307,20 @@ cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, int s
     }
 }
 
-int demo_apply_piece() { return APPLY_PIECE; }
-
 cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, cudaStream_t stream)
 {
     if (a.n_pieces <= 0) return cudaSuccess;
+    const bool blocks = a.piece == demo_apply_pieces[0];
+    const auto kernel = blocks ? apply_signs_kernel<true> : apply_signs_kernel<false>;
+    const long long need = blocks ? a.n_pieces : (a.n_pieces + GEN_THREADS - 1) / GEN_THREADS;
     int per_sm = 0;
-    const cudaError_t err = demo_resident_ctas((const void *)apply_signs_kernel, GEN_THREADS, 0, &per_sm);
+    const cudaError_t err = demo_resident_ctas((const void *)kernel, GEN_THREADS, 0, &per_sm);
     if (err != cudaSuccess) return err;
     long long grid = (long long)sm_count * per_sm;
-    if (grid > a.n_pieces) grid = a.n_pieces;
+    if (grid > need) grid = need;
     // An ordinary launch: resident beside the last CTAs of decode_signs, these would keep that kernel's split of the SM into
     // shared memory and L1 to their end, and the L1 left (28 KB) does not hold the loads in flight (632 -> about 830 us).
-    apply_signs_kernel<<<(unsigned)grid, GEN_THREADS, 0, stream>>>(a);
+    kernel<<<(unsigned)grid, GEN_THREADS, 0, stream>>>(a);
     return cudaGetLastError();
 }
 

@@ -26,20 +26,10 @@ constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ unsigned mag_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 
-// (warp) the tensor that owns chunk id c: the last entry with chunk_begin <= c.  32 entries are compared at once, so sets of up to
-// 32 tensors take one round of loads, of up to 2^20 tensors four.  (One after the other in steps of 32 entries: 20000 vectors of
-// 64 elements, decode 647 us instead of 44; 100000 15.2 ms instead of 0.22.)
+// (warp) the tensor that owns chunk id c.
 __device__ __forceinline__ int find_entry_warp(const DemoTensorEntry *entries, int n, long long c)
 {
-    const int lane = threadIdx.x & 31;
-    int lo = 0;  // the entry is one of lo .. lo + n - 1
-    while (n > 1) {
-        const int step = (n + 31) / 32, i = lane * step;
-        const int last = __popc(__ballot_sync(FULL, i < n && entries[lo + i].chunk_begin <= c)) - 1;  // (chunk_begin ascends; entry lo is below)
-        lo += last * step;
-        n = min(step, n - last * step);
-    }
-    return lo;
+    return demo_find_warp(0, n, [&](int i) { return entries[i].chunk_begin <= c; });
 }
 
 // ---- segments -------------------------------------------------------------------------------------------

@@ -250,3 +250,9 @@ def check_many_tensors(count, shape, chunk, calls, slower, topk=4, basis=None):
 @pytest.mark.parametrize("s", [8, 64, 128])
 def test_many_vectors(s, count):
     check_many_tensors(count, (s,), s, ["compress", "decode"] if count == 20000 else [], 5.0)
+
+
+@pytest.mark.parametrize("count,shape", [(33, (64,)), (20000, (8,)), (20000, (64,)), (3000, (128,)), (5000, (32, 32)), (20000, (64, 64))])
+def test_apply_signs_many_tensors(count, shape):
+    """Pieces of a thread (less than half a block's piece on average) and of a block, each with more than 32 tensors to skip."""
+    check_many_tensors(count, shape, shape[0], ["apply"] if count > 1000 else [], 5.0)
