@@ -225,6 +225,17 @@ __device__ __forceinline__ int demo_find_entry(const DemoTensorEntry *entries, i
     return lo;
 }
 
+// The last entry at or behind e with chunk_begin <= c (which holds for e): strides that double, then halve, so that the entry after e
+// costs one comparison and one d entries away about 2 log2 d.
+__device__ __forceinline__ int demo_seek_entry(const DemoTensorEntry *entries, int n, int e, long long c)
+{
+    int step = 1;
+    for (; step < n - e && entries[e + step].chunk_begin <= c; step <<= 1) e += step;
+    while (step >>= 1)
+        if (step < n - e && entries[e + step].chunk_begin <= c) e += step;
+    return e;
+}
+
 // (warp) the last i of lo .. lo + n - 1 with below(i), which holds for lo and up to some i.  32 places are compared at once, so up to
 // 32 entries take one round of loads, up to 2^20 four.  (In steps of 32 entries instead: decode of 20000 vectors of 64 elements 647 us
 // instead of 44, of 100000 15.2 ms instead of 0.22.)

@@ -108,7 +108,7 @@ struct EntryCursor {
             return;
         }
         if (c < next_begin) return;
-        while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+        e = demo_seek_entry(entries, n, e + 1, c);
         load(entries, n);
     }
 };
@@ -366,7 +366,7 @@ struct DecodeWalk {
     __device__ __forceinline__ void seek(const DemoTensorEntry *entries, int n, long long c, int k, int which)
     {
         if (c >= next_begin) {
-            while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+            e = demo_seek_entry(entries, n, e + 1, c);
             load(entries, n);
         }
         const unsigned lc = (unsigned)(c - te.chunk_begin);

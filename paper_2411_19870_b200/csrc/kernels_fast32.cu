@@ -115,8 +115,7 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) compress32_kernel(DemoCompre
     unsigned next_begin = 0;  // first chunk of the next tensor
     auto locate = [&](unsigned c) {
         if (c >= next_begin) {
-            e = next_begin ? e + 1 : demo_find_entry(a.entries, a.n_entries, c);
-            while (e + 1 < a.n_entries && a.entries[e + 1].chunk_begin <= c) ++e;
+            e = next_begin ? demo_seek_entry(a.entries, a.n_entries, e + 1, c) : demo_find_entry(a.entries, a.n_entries, c);
             next_begin = e + 1 < a.n_entries ? (unsigned)a.entries[e + 1].chunk_begin : ~0u;
             const DemoTensorEntry te = a.entries[e];
             if (t == 0) {

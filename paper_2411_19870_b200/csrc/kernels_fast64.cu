@@ -73,7 +73,7 @@ struct SlotWalk {
     __device__ __forceinline__ void seek(const DemoTensorEntry *entries, int n, unsigned c, int k, int slot)
     {
         if (c >= next_begin) {
-            while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+            e = demo_seek_entry(entries, n, e + 1, c);
             load(entries, n);
         }
         const unsigned lc = (unsigned)(c - te.chunk_begin);

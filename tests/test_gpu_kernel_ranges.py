@@ -256,3 +256,11 @@ def test_many_vectors(s, count):
 def test_apply_signs_many_tensors(count, shape):
     """Pieces of a thread (less than half a block's piece on average) and of a block, each with more than 32 tensors to skip."""
     check_many_tensors(count, shape, shape[0], ["apply"] if count > 1000 else [], 5.0)
+
+
+@pytest.mark.parametrize("count,s,basis", [(3, 64, False), (1000, 64, False), (20000, 64, False), (5000, 32, False), (2000, 128, False)])
+def test_many_matrices(count, s, basis):
+    """One chunk per tensor: the walks over the tensor table skip a grid's worth of entries between two chunks of a CTA."""
+    b = torch.linalg.qr(torch.randn(s, s, dtype=torch.float64, generator=torch.Generator().manual_seed(5)))[0].float() if basis else None
+    # (s = 64 and 128 acquire two tensor maps for every chunk, about a microsecond each; a few tensors per chunk slot only)
+    check_many_tensors(count, (s, s), s, ["compress", "decode"] if count >= 1000 else [], 5.0, basis=b)
