@@ -235,15 +235,22 @@ __device__ __forceinline__ bool tc_stage(TcFrame &f, const SlotBarrier<PAIR_THRE
     return true;
 }
 
-// Where a chunk lies; the entry index only grows.
+// Where a chunk lies; the entry index only grows.  MANY (more tensors than MANY_TENSORS): the walk over the table skips entries; an
+// instantiation of its own, because in the kernels at the register limit the longer code costs 1 % of 4096 x 8192 even with one
+// tensor.  (One entry after the other, one chunk per tensor: 1000 tensors compress 219 us instead of 31, 20000 8.1 ms instead of 0.49.)
+constexpr int MANY_TENSORS = 32;
 struct ChunkRef {
     int tensor, n1;
     size_t elem;         // of the tile's first element
     long long first_rec;
 };
+template <bool MANY>
 __device__ __forceinline__ ChunkRef locate(const DemoTensorEntry *entries, int n, unsigned c, int k, int &e)
 {
-    while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
+    if constexpr (MANY)
+        e = demo_seek_entry(entries, n, e, c);
+    else
+        while (e + 1 < n && entries[e + 1].chunk_begin <= c) ++e;
     const DemoTensorEntry te = entries[e];
     const unsigned lc = (unsigned)(c - te.chunk_begin), k0 = lc / (unsigned)te.c1;
     ChunkRef r;
@@ -293,7 +300,7 @@ __device__ __forceinline__ void write_row(float *X, int r, const float (&v)[S])
 // BIGK (k > MAX_K_LISTED): selection from quarter-row maxima with the wide list (3 groups fit), both inverse stages dense.
 // Without the prefetch, the same sizes: from the list k = 40 / 48 204 / 244 us (at 48 part of the lists overflow into the radix
 // select), dense k = 49 / 128 / 300 240 / 247 / 605 us.
-template <typename GT, int GROUPS, bool BIGK>
+template <typename GT, int GROUPS, bool BIGK, bool MANY>
 __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(DemoCompressArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -333,7 +340,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         float *m = nullptr;
         const GT *g = nullptr;
         if (valid) {
-            cr = locate(a.entries, a.n_entries, chunk, k_eff, e);
+            cr = locate<MANY>(a.entries, a.n_entries, chunk, k_eff, e);
             m = a.m_ptrs[cr.tensor] + cr.elem + r;
             g = static_cast<const GT *>(a.g_ptrs[cr.tensor]) + cr.elem + r;
             each_b<32>(m, g, cr.n1, a.beta, [&](int i, float b) { v[i] = b; });
@@ -353,7 +360,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         const unsigned next = *f.drawn;  // (written before the barriers of the stages; overwritten behind those below)
         if (2u * next + c < n_chunks) {  // row r of the group's next tiles on its way to L2
             int e2 = e;
-            const ChunkRef nr = locate(a.entries, a.n_entries, 2u * next + c, k_eff, e2);
+            const ChunkRef nr = locate<MANY>(a.entries, a.n_entries, 2u * next + c, k_eff, e2);
             const size_t at = nr.elem + (size_t)r * nr.n1;
             const float *nm = a.m_ptrs[nr.tensor] + at;
             const GT *ng = static_cast<const GT *>(a.g_ptrs[nr.tensor]) + at;
@@ -416,7 +423,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
     tmem_free_cta(f.tmem, TMEM_COLS);
 }
 
-template <int GROUPS>
+template <int GROUPS, bool MANY>
 __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -445,7 +452,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
 #pragma unroll
         for (int j = 0; j < S; ++j) v[j] = 0.f;
         if (valid) {
-            cr = locate(a.entries, a.n_entries, chunk, k_eff, e);
+            cr = locate<MANY>(a.entries, a.n_entries, chunk, k_eff, e);
             x = a.x_ptrs[cr.tensor] + cr.elem + r;
             // the x tile on its way to L2
             const float *xr = a.x_ptrs[cr.tensor] + cr.elem + (size_t)r * cr.n1;
@@ -561,20 +568,25 @@ bool demo_tc_supported(int s) { return s == S; }
 cudaError_t demo_launch_compress_tc(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
 {
     constexpr int FIXED = 8 * BLK + bars_bytes + 1024;  // (last: alignment slack)
-    if (a.k > MAX_K_LISTED) {
-        const int smem = FIXED + 6 * chunk_bytes(true);
-        return a.grad_bf16 ? launch_tc(compress_tc_kernel<__nv_bfloat16, 3, true>, 3, smem, a, sm_count, stream)
-                           : launch_tc(compress_tc_kernel<float, 3, true>, 3, smem, a, sm_count, stream);
-    }
-    const int smem = FIXED + 8 * chunk_bytes(false);
-    return a.grad_bf16 ? launch_tc(compress_tc_kernel<__nv_bfloat16, 4, false>, 4, smem, a, sm_count, stream)
-                       : launch_tc(compress_tc_kernel<float, 4, false>, 4, smem, a, sm_count, stream);
+    auto pick = [&](auto gt, auto many) {
+        using GT = decltype(gt);
+        constexpr bool MANY = decltype(many)::value;
+        return a.k > MAX_K_LISTED ? launch_tc(compress_tc_kernel<GT, 3, true, MANY>, 3, FIXED + 6 * chunk_bytes(true), a, sm_count, stream)
+                                  : launch_tc(compress_tc_kernel<GT, 4, false, MANY>, 4, FIXED + 8 * chunk_bytes(false), a, sm_count, stream);
+    };
+    if (a.n_entries > MANY_TENSORS)
+        return a.grad_bf16 ? pick(__nv_bfloat16{}, std::true_type{}) : pick(float{}, std::true_type{});
+    return a.grad_bf16 ? pick(__nv_bfloat16{}, std::false_type{}) : pick(float{}, std::false_type{});
 }
 
 cudaError_t demo_launch_decode_tc(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
     constexpr int FIXED = 4 * BLK + bars_bytes + 1024;
-    if (a.agg == 2)  // the sender counts leave room for three groups
-        return launch_tc(decode_tc_kernel<3>, 3, FIXED + 6 * (X_BYTES + M * 2), a, sm_count, stream);
-    return launch_tc(decode_tc_kernel<4>, 4, FIXED + 8 * X_BYTES, a, sm_count, stream);
+    auto pick = [&](auto many) {
+        constexpr bool MANY = decltype(many)::value;
+        if (a.agg == 2)  // the sender counts leave room for three groups
+            return launch_tc(decode_tc_kernel<3, MANY>, 3, FIXED + 6 * (X_BYTES + M * 2), a, sm_count, stream);
+        return launch_tc(decode_tc_kernel<4, MANY>, 4, FIXED + 8 * X_BYTES, a, sm_count, stream);
+    };
+    return a.n_entries > MANY_TENSORS ? pick(std::true_type{}) : pick(std::false_type{});
 }

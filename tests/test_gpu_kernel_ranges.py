@@ -258,7 +258,8 @@ def test_apply_signs_many_tensors(count, shape):
     check_many_tensors(count, shape, shape[0], ["apply"] if count > 1000 else [], 5.0)
 
 
-@pytest.mark.parametrize("count,s,basis", [(3, 64, False), (1000, 64, False), (20000, 64, False), (5000, 32, False), (2000, 128, False)])
+@pytest.mark.parametrize("count,s,basis", [(3, 64, False), (1000, 64, False), (20000, 64, False), (5000, 32, False), (2000, 128, False),
+                                           (32, 64, True), (33, 64, True), (1000, 64, True), (20000, 64, True)])
 def test_many_matrices(count, s, basis):
     """One chunk per tensor: the walks over the tensor table skip a grid's worth of entries between two chunks of a CTA."""
     b = torch.linalg.qr(torch.randn(s, s, dtype=torch.float64, generator=torch.Generator().manual_seed(5)))[0].float() if basis else None
