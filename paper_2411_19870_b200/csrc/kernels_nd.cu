@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
+#include <cstddef>
 #include <type_traits>
 
 #include "demo_internal.h"
@@ -112,8 +113,8 @@ struct Shared {
     size_t base[2];
     unsigned ticket, hi, n, n_kept, bound, thr, need_eq, n_eq, state[2], warp_tot[12];
     unsigned hist[256], fine[256];
-    uint2 cand[CAND];      // candidates (value bits, tile position) in no particular order
-    uint4 kept[CAND / 2];  // the kept ones, two per entry
+    alignas(16) uint2 cand[CAND];  // candidates (value bits, tile position) in no particular order
+    uint4 kept[CAND / 2];          // the kept ones, two per entry; decode: with cand, two batches of records
 };
 extern __shared__ __align__(16) unsigned char smem_raw[];
 __device__ __forceinline__ Shared *shared() { return reinterpret_cast<Shared *>(smem_raw); }
@@ -860,6 +861,11 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
     __syncthreads();
 }
 
+// Decode: records of one of the two batches; place of a record outside its chunk; longest list that one warp adds.
+constexpr int STAGE = CAND, WARP_K = 32;
+constexpr unsigned SKIP = 0xffffffffu;
+static_assert(offsetof(Shared, kept) == offsetof(Shared, cand) + STAGE * sizeof(uint2), "the batches are neighbours");
+
 // Registers: 80 per thread (768 threads per SM); 128 with extents of 128.
 constexpr int MAX_THREADS = 384, MAX_THREADS_BIG = 256;
 
@@ -930,8 +936,6 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
     Shared *s = shared();
     float *tile0 = v.tile0, *tile1 = v.tile1;
     unsigned short *Cn = reinterpret_cast<unsigned short *>(v.tile0 + (size_t)a.cls.tile * (a.cls.dense_axes ? 2 : 1));  // senders (agg == 2)
-    constexpr int STAGE = CAND;  // records staged at once (in the place of the selection's list)
-    uint2 *stage = s->cand;
     const int tid = threadIdx.x, T = blockDim.x;
     const bool counts = a.agg == 2;
     if (tid < 2) s->e[tid].chunk_begin = 1, s->e[tid].chunk_end = 0;
@@ -953,53 +957,105 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
         const int M = e.M, k_eff = e.k_eff;
         const long long rec_off = e.rec_begin + (c - e.chunk_begin) * (long long)k_eff;
 
+        // S = sum over workers in worker order (indices are unique inside one worker's chunk).  k <= STAGE: batches of several
+        // workers' records come through two buffers, the next batch while this one is added; a thread turns the records that it
+        // requested into tile positions, then one warp adds short lists and all threads long ones, with a barrier per worker.  Larger k:
+        // straight from the payloads.  (One warp for every k, with the positions inside its serial loop: 2048 x 2048 in 32 x 128, W = 64,
+        // k = 8 / 128 / 512 78 / 228 / 828 us instead of 44 / 107 / 236; W = 16, k = 256 111 instead of 60.)
+        const int wb = STAGE / k_eff;
+        auto request = [&](int w0, int buf) {
+            const int n = min(wb, a.W - w0) * k_eff;  // (negative behind the last)
+            for (int r = tid; r < n; r += T) {
+                const int w = r / k_eff;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(s->cand + buf + r)),
+                             "l"(a.payloads[w0 + w] + rec_off + (r - w * k_eff))
+                             : "memory");
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (wb) request(0, 0);
         for (int i = tid; i < e.tile >> 2; i += T) reinterpret_cast<float4 *>(tile0)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (counts)
-            for (int i = tid; i < M; i += T) Cn[i] = 0;
+            for (int i = tid; i < e.tile; i += T) Cn[i] = 0;
         if (tid == T - 1) take_ticket(s, slot ^ 1, a.entries, a.cls, ticket);
-        // S = sum over workers, in worker order: batches of records are staged by all threads, the first warp adds them
-        // worker after worker (indices are unique inside one worker's chunk)
-        auto add = [&](int idx, float val) {
-            if ((unsigned)idx < (unsigned)M) {
-                tile0[place_of(e, idx).t] += val;
-                if (counts) Cn[idx] += 1;
-            } else {
-                atomicMax(a.status, DEMO_DEV_PAYLOAD);
-            }
+        auto position = [&](unsigned idx) {
+            if (idx < (unsigned)M) return (unsigned)place_of(e, (int)idx).t;
+            atomicMax(a.status, DEMO_DEV_PAYLOAD);
+            return SKIP;
         };
-        if (k_eff <= STAGE) {
-            const int wb = STAGE / k_eff;
-            for (int w0 = 0; w0 < a.W; w0 += wb) {
-                const int nw = min(wb, a.W - w0);
-                for (int r = tid; r < nw * k_eff; r += T) {
-                    const int w = r / k_eff;
-                    const DemoRecord rc = a.payloads[w0 + w][rec_off + (r - w * k_eff)];
-                    stage[r] = make_uint2((unsigned)rc.idx, __float_as_uint(rc.val));
+        // several records of one worker, their tile accesses side by side
+        auto add = [&](const uint2 (&r)[4]) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = r[u].x != SKIP ? tile0[r[u].x] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (r[u].x != SKIP) {
+                    tile0[r[u].x] = v[u] + __uint_as_float(r[u].y);
+                    if (counts) Cn[r[u].x] += 1;
                 }
-                __syncthreads();
-                if (tid < 32) {
-                    for (int w = 0; w < nw; ++w) {
-                        for (int i = tid; i < k_eff; i += 32) {
-                            const uint2 r = stage[w * k_eff + i];
-                            add((int)r.x, __uint_as_float(r.y));
+        };
+        const uint2 none = make_uint2(SKIP, 0u);
+        if (wb) {
+            for (int w0 = 0, buf = 0; w0 < a.W; w0 += wb, buf ^= STAGE) {
+                uint2 *stage = s->cand + buf;
+                const int n = min(wb, a.W - w0) * k_eff;
+                request(w0 + wb, buf ^ STAGE);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+                for (int r = tid; r < n; r += T) stage[r].x = position(stage[r].x);
+                __syncthreads();  // (the first time: the tile is cleared too)
+                if (k_eff <= WARP_K) {
+                    if (tid < 32) {
+                        for (int r0 = 0; r0 < n; r0 += 4 * k_eff) {  // four workers' records are read together
+                            uint2 r[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int i = r0 + u * k_eff + tid;
+                                r[u] = tid < k_eff && i < n ? stage[i] : none;
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                if (r[u].x != SKIP) {
+                                    tile0[r[u].x] += __uint_as_float(r[u].y);
+                                    if (counts) Cn[r[u].x] += 1;
+                                }
+                                __syncwarp();
+                            }
                         }
-                        __syncwarp();
+                    }
+                    __syncthreads();
+                } else {
+                    for (int r0 = 0; r0 < n; r0 += k_eff) {
+                        for (int i0 = tid; i0 < k_eff; i0 += 4 * T) {
+                            uint2 r[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) r[u] = i0 + u * T < k_eff ? stage[r0 + i0 + u * T] : none;
+                            add(r);
+                        }
+                        __syncthreads();
                     }
                 }
-                __syncthreads();
             }
         } else {
             __syncthreads();
             for (int w = 0; w < a.W; ++w) {
                 const DemoRecord *rec = a.payloads[w] + rec_off;
-                for (int i = tid; i < k_eff; i += T) add(rec[i].idx, rec[i].val);
+                for (int i0 = tid; i0 < k_eff; i0 += 4 * T) {
+                    uint2 r[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) r[u] = i0 + u * T < k_eff ? *reinterpret_cast<const uint2 *>(rec + i0 + u * T) : none;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (i0 + u * T < k_eff) r[u].x = position(r[u].x);
+                    add(r);
+                }
                 __syncthreads();
             }
         }
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
             for (int i = tid; i < M; i += T) {
-                const unsigned short n = Cn[i];
                 const int t = place_of(e, i).t;
+                const unsigned short n = Cn[t];
                 if (n > 1) tile0[t] = tile0[t] / (float)n;
             }
             __syncthreads();
@@ -1244,7 +1300,7 @@ cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, c
 
 cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, int sm_count, cudaStream_t stream)
 {
-    const size_t smem = shared_bytes(a.cls, false) + (a.agg == 2 ? align16((size_t)a.cls.max_M * 2) : 0);
+    const size_t smem = shared_bytes(a.cls, false) + (a.agg == 2 ? align16((size_t)a.cls.tile * 2) : 0);
     return a.cls.big ? launch_nd(decode_nd_kernel<true>, smem, sm_count, stream, a)
                      : launch_nd(decode_nd_kernel<false>, smem, sm_count, stream, a);
 }

@@ -265,3 +265,47 @@ def test_many_matrices(count, s, basis):
     b = torch.linalg.qr(torch.randn(s, s, dtype=torch.float64, generator=torch.Generator().manual_seed(5)))[0].float() if basis else None
     # (s = 64 and 128 acquire two tensor maps for every chunk, about a microsecond each; a few tensors per chunk slot only)
     check_many_tensors(count, (s, s), s, ["compress", "decode"] if count >= 1000 else [], 5.0, basis=b)
+
+
+@pytest.mark.parametrize("chunk,k,workers,agg", [
+    ((16, 32), 32, 17, 0), ((16, 32), 33, 17, 2), ((16, 32), 256, 3, 2), ((16, 32), 257, 3, 0), ((16, 32), 511, 2, 1),  # a warp, one list per batch
+    ((32, 64), 32, 19, 2), ((32, 64), 100, 11, 0), ((32, 64), 512, 3, 2), ((32, 64), 513, 3, 2), ((32, 64), 1500, 2, 0),  # more threads, no batches
+    ((4, 8, 6, 5), 40, 5, 2), ((13, 64), 90, 6, 2),                                  # an odd number of dense axes: the tiles change places
+])
+def test_nd_decode_batches(chunk, k, workers, agg):
+    """Records of several workers per batch, two and more batches, a short last one, lists longer than a batch; colliding coordinates."""
+    r = parity.NdRunner([tuple(3 * c for c in chunk)], [chunk], topk=k, num_workers=workers, grad_std=0.02, agg=agg)
+    for _ in range(2):
+        r.step()
+    r.close()
+
+
+def nd_device_us(shape, chunk, k, workers, what):
+    """Time of one call on an N-D context, the best of several."""
+    import paper_2411_19870_b200 as demo
+
+    tr = demo.DemoTransform([shape], chunk_shapes=[chunk], topk=k, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=workers)
+    gen = torch.Generator("cuda").manual_seed(3)
+    g = [torch.randn(shape, device="cuda", generator=gen).bfloat16()]
+    m, x = [torch.zeros(shape, device="cuda")], [torch.zeros(shape, device="cuda")]
+    pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(workers)]
+    for w in range(workers):
+        tr.compress(w, g, m, pay[w])
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = math.inf
+    for _ in range(8):
+        t0.record()
+        for _ in range(10):
+            tr.compress(0, g, m, pay[0]) if what == "compress" else tr.decode_apply(pay, x)
+        t1.record()
+        torch.cuda.synchronize()
+        best = min(best, t0.elapsed_time(t1) / 10 * 1e3)
+    tr.close()
+    return best
+
+
+@pytest.mark.parametrize("shape,chunk", [((2048, 2048), (32, 128)), ((512, 512, 3, 3), (32, 32, 3, 3))])
+def test_nd_decode_time_of_long_lists(shape, chunk):
+    """512 records per chunk and 64 workers are 64 times the records of k = 8: added by one warp they took 7 and 11 times as long, by all threads 3 and 5."""
+    short, long_ = nd_device_us(shape, chunk, 8, 64, "decode"), nd_device_us(shape, chunk, 512, 64, "decode")
+    assert long_ <= 6 * short, "k = 8 %.1f us, k = 512 %.1f us" % (short, long_)
