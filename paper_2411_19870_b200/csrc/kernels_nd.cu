@@ -36,7 +36,8 @@
 
 namespace {
 
-constexpr int CAND = 512;  // candidate list
+constexpr int CAND = 512;       // candidate list
+constexpr int DENSE_SHARE = 24;  // select_topk
 
 __device__ __forceinline__ unsigned mag_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 
@@ -598,13 +599,73 @@ __device__ __forceinline__ void find_bin(const unsigned *hist, unsigned rank, un
     *before_bin = __shfl_sync(0xffffffffu, bb, src);
 }
 
-// Exact top-k by radix select on the magnitude bits, index-ordered compaction; leaves alpha * kept in X, zero elsewhere.
+// Records of the coefficients with keys above thr (>= 1: never the padding) and of the first need_eq equal to it, in index order; X
+// left with alpha * kept, zero elsewhere; ends with a barrier.  A warp has neighbouring quads of the tile (tile positions are in
+// index order): the warps count theirs, then number them.
+__device__ __noinline__ void compact(unsigned tile, int slot, DemoRecord *rec, float alpha, unsigned thr, unsigned need_eq)
+{
+    Shared *s = shared();
+    const DemoNdEntry &e = s->e[slot];
+    float4 *X4 = reinterpret_cast<float4 *>(tile_at(tile));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, quads = e.tile >> 2;
+    const int rounds = (quads + (int)blockDim.x - 1) / (int)blockDim.x, q0 = warp * rounds * 32 + lane;
+    auto count = [&](const float4 &f) {  // above | equal << 16
+        const unsigned k[4] = {mag_key(f.x), mag_key(f.y), mag_key(f.z), mag_key(f.w)};
+        unsigned n = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) n += (k[j] > thr ? 1u : 0u) + (k[j] == thr ? 0x10000u : 0u);
+        return n;
+    };
+    unsigned n = 0;
+    for (int r = 0; r < rounds; ++r)
+        if (q0 + 32 * r < quads) n += count(X4[q0 + 32 * r]);
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) s->warp_tot[warp] = n;
+    __syncthreads();
+    unsigned before = 0;
+    for (int w = 0; w < warp; ++w) before += s->warp_tot[w];
+    for (int r = 0; r < rounds; ++r) {
+        const int q = q0 + 32 * r;
+        const bool have = q < quads;
+        float4 f = have ? X4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const unsigned own = count(f);
+        unsigned inc = own;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned v = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += v;
+        }
+        unsigned gt = (before + inc - own) & 0xffffu, eq = (before + inc - own) >> 16;
+        before += __shfl_sync(0xffffffffu, inc, 31);
+        float v[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned key = mag_key(v[j]);
+            const bool above = key > thr, equal = key == thr;
+            const bool keep = above || (equal && eq < need_eq);
+            if (keep) {
+                DemoRecord out;
+                out.idx = index_of(e, 4 * q + j);
+                out.val = v[j];
+                rec[gt + min(eq, need_eq)] = out;
+            }
+            gt += above;
+            eq += equal;
+            v[j] = keep ? alpha * v[j] : 0.f;
+        }
+        if (have) X4[q] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    __syncthreads();
+}
+
+// Exact top-k by radix select on the magnitude bits (the padding's zeros are taken out of the counts), index-ordered compaction; leaves
+// alpha * kept in X, zero elsewhere.
 __device__ __noinline__ void select_radix(unsigned tile, int slot, DemoRecord *rec, float alpha)
 {
     float *X = tile_at(tile);
     Shared *s = shared();
     const DemoNdEntry &e = s->e[slot];
-    const int tid = threadIdx.x, T = blockDim.x, M = e.M, k_eff = e.k_eff;
+    const int tid = threadIdx.x, T = blockDim.x, M = e.M, k_eff = e.k_eff, quads = e.tile >> 2;
     if (tid == 0) {
         s->state[0] = 0u;               // prefix of the key found so far
         s->state[1] = (unsigned)k_eff;  // rank still to resolve inside the prefix class
@@ -615,14 +676,23 @@ __device__ __noinline__ void select_radix(unsigned tile, int slot, DemoRecord *r
         for (int i = tid; i < 256; i += T) s->hist[i] = 0u;
         __syncthreads();
         const unsigned prefix = s->state[0];
-        for (int i = tid; i < M; i += T) {
-            const unsigned key = mag_key(X[place_of(e, i).t]);
+        auto note = [&](float v) {
+            const unsigned key = mag_key(v);
             if ((key & mask) == prefix) atomicAdd(&s->hist[255u - ((key >> shift) & 255u)], 1u);
+        };
+        for (int i = tid; i < quads; i += T) {
+            const float4 f = reinterpret_cast<const float4 *>(X)[i];
+            note(f.x);
+            note(f.y);
+            note(f.z);
+            note(f.w);
         }
         __syncthreads();
         if (tid < 32) {
             unsigned bin, before;
             const unsigned rem = s->state[1];
+            if (tid == 0 && prefix == 0u) s->hist[255] -= (unsigned)(4 * quads - M);
+            __syncwarp();
             find_bin(s->hist, rem, &bin, &before);
             __syncwarp();
             if (tid == 0) {
@@ -633,6 +703,11 @@ __device__ __noinline__ void select_radix(unsigned tile, int slot, DemoRecord *r
         __syncthreads();
     }
     const unsigned thr = s->state[0], need_eq = s->state[1];
+    if (thr) {
+        compact(tile, slot, rec, alpha, thr, need_eq);
+        return;
+    }
+    // fewer than k coefficients are not zero: zeros are kept too, but not those of the padding
     const int per = (M + T - 1) / T;
     const int start = tid * per;
     const int stop = min(M, start + per);
@@ -720,6 +795,22 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
     const DemoNdEntry &e = s->e[slot];
     const int k_eff = e.k_eff, quads = e.tile >> 2;
     float4 *X4 = reinterpret_cast<float4 *>(X);
+    if (k_eff == e.M) {  // everything is kept
+        for (int i = tid; i < e.M; i += T) {
+            const int t = place_of(e, i).t;
+            DemoRecord r;
+            r.idx = i;
+            r.val = X[t];
+            rec[i] = r;
+            X[t] = alpha * r.val;
+        }
+        __syncthreads();
+        return;
+    }
+    // Long lists of a small chunk are numbered by going over the tile twice, short ones by counting the records below each: k^2 / 2
+    // comparisons, which pays up to k^2 = 24 M (one call, counting / numbering: 512 x 512 x 3 x 3 in 16 x 16 x 3 x 3 k = 192 / 256 56 / 66
+    // and 64 / 66 us; 1024 x 1024 in 16 x 32 k = 64 / 128 / 256 34 / 48 / 81 and 34 / 38 / 37 us).
+    const bool dense = k_eff * k_eff > DENSE_SHARE * e.M;
     // group maxima: a thread's quads as one group, or -- where k is not well below the number of threads -- as four
     const bool four = 2 * k_eff > T;
     unsigned key[4] = {0u, 0u, 0u, 0u};
@@ -820,7 +911,8 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
         else
             find_threshold<16>((unsigned)n, bound, k_eff);
     }
-    if (T == 32) {
+    if (dense) {
+    } else if (T == 32) {
         for (int i = tid; i < quads; i += 32) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else if (tid >= 32) {
         for (int i = tid - 32; i < quads; i += T - 32) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -829,6 +921,10 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
     if (tid == 0 && (k_eff & 1)) kept[k_eff] = make_uint2(0u, 0xffffffffu);  // completes the last pair: behind everything
     __syncthreads();
     const unsigned thr = s->thr, need_eq = s->need_eq;
+    if (dense) {  // (thr < bound: exactly the candidates are kept)
+        compact(tile_offset(X), slot, rec, alpha, thr < bound ? bound - 1u : thr, thr < bound ? 0u : need_eq);
+        return;
+    }
     const bool ties = need_eq != s->n_eq;
     for (int i = tid; i < n; i += T) {
         const uint2 c = s->cand[i];
@@ -1280,6 +1376,11 @@ void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vect
             e.layout = k.n_chunks > n && same_layout(entries.back(), e) ? entries.back().layout : (int)entries.size();
             entries.push_back(e);
         }
+        // chunks that leave the device's threads idle get more of them, down to eight elements each (256 chunks of 32 x 32, k = 32 / 128:
+        // compress 21 / 56 -> 14 / 18 us, decode of 16 workers 18 / 37 -> 13 / 16)
+        const long long places = (long long)sm_count * 2 * MAX_THREADS / k.n_chunks, useful = (k.max_M / 8 + 31) / 32 * 32;
+        const long long more = (places < useful ? places : useful) / 32 * 32;
+        if (more > k.threads) k.threads = (int)(more < MAX_THREADS ? more : MAX_THREADS);
         if (split) k.threads = (k.threads + 63) / 64 * 64;  // two warps per 32 lines
         if (k.big && k.threads > MAX_THREADS_BIG) k.threads = MAX_THREADS_BIG;
         classes->push_back(k);

@@ -284,10 +284,11 @@ def nd_device_us(shape, chunk, k, workers, what):
     """Time of one call on an N-D context, the best of several."""
     import paper_2411_19870_b200 as demo
 
-    tr = demo.DemoTransform([shape], chunk_shapes=[chunk], topk=k, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=workers)
+    shapes = [shape, (48, 48)]  # (the second keeps square chunks on the N-D kernels)
+    tr = demo.DemoTransform(shapes, chunk_shapes=[chunk, (3, 16)], topk=k, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=workers)
     gen = torch.Generator("cuda").manual_seed(3)
-    g = [torch.randn(shape, device="cuda", generator=gen).bfloat16()]
-    m, x = [torch.zeros(shape, device="cuda")], [torch.zeros(shape, device="cuda")]
+    g = [torch.randn(s, device="cuda", generator=gen).bfloat16() for s in shapes]
+    m, x = ([torch.zeros(s, device="cuda") for s in shapes] for _ in range(2))
     pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(workers)]
     for w in range(workers):
         tr.compress(w, g, m, pay[w])
@@ -309,3 +310,32 @@ def test_nd_decode_time_of_long_lists(shape, chunk):
     """512 records per chunk and 64 workers are 64 times the records of k = 8: added by one warp they took 7 and 11 times as long, by all threads 3 and 5."""
     short, long_ = nd_device_us(shape, chunk, 8, 64, "decode"), nd_device_us(shape, chunk, 512, 64, "decode")
     assert long_ <= 6 * short, "k = 8 %.1f us, k = 512 %.1f us" % (short, long_)
+
+
+@pytest.mark.parametrize("shape,chunk,k", [((512, 512, 1, 1), (32, 32, 1, 1), 128), ((512, 512, 1, 1), (32, 32, 1, 1), 1000), ((1024, 1024), (16, 32), 256),
+                                           ((1024, 1024), (16, 32), 512), ((7475, 512), (13, 32), 300)])
+def test_nd_compress_time_of_large_k(shape, chunk, k):
+    """Much of a small chunk kept: ordering the records by counting pairs, and the radix select with 32 threads, took 2.7 to 7 times as
+    long as k = 32."""
+    short, long_ = nd_device_us(shape, chunk, 32, 1, "compress"), nd_device_us(shape, chunk, k, 1, "compress")
+    assert long_ <= 2.2 * short, "k = 32 %.1f us, k = %d %.1f us" % (short, k, long_)
+
+
+@pytest.mark.parametrize("k", [108, 111, 135, 136, 150, 400, 767, 768])
+def test_nd_numbered_records(k):
+    """Chunks of 768 elements around k^2 = 24 M and up to all of them, padded tiles, equal magnitudes at the k-th place, a tile with few
+    non-zero coefficients, an all-zero one."""
+    r = parity.NdRunner([(96, 48)], [(32, 24)], topk=k, num_workers=1, grad_dtype=torch.float32)
+    gen = torch.Generator("cuda").manual_seed(k)
+    sign = torch.where(torch.rand(96, 48, device="cuda", generator=gen) < 0.5, -1.0, 1.0)
+    g = torch.randn(96, 48, device="cuda", generator=gen)
+    g[:32, 24:] = 0.0
+    g[32:64, :24] = 0.125 * sign[32:64, :24]
+    g[32:64, 24:] = 0.25
+    # With most of a chunk kept the residual is the rounding of both transforms: some 5 * 2^-23 of the largest |B|, here about 4 * 2^-6, which
+    # stays below the absolute tolerance of 1e-7.
+    g *= 2.0 ** -6 if k > 300 else 1.0
+    r.inputs = types.SimpleNamespace(random_tensor=lambda *a: g)
+    for _ in range(2):
+        r.step()
+    r.close()
