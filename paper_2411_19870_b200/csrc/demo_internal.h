@@ -148,9 +148,13 @@ struct DemoNdClass {
     int dense_axes;      // some extent is a dense contraction from a table (second tile)
     int big;             // some extent is 128: the variant with 64 registers per half line
 };
-// Coefficient tables of the dense extents in use.
+// Coefficient tables of the dense extents in use, and the tile layouts of the chunk shapes planned so far.
 struct DemoNdTables {
+    struct Layout {
+        int s[DEMO_ND_DIMS], p[DEMO_ND_DIMS], tile;
+    };
     std::vector<float> data;
+    std::vector<Layout> layouts;
     int of[129];
     DemoNdTables() { for (int &v : of) v = -1; }
     int get(int s);  // offset of the tables of extent s (made on first use)

@@ -1218,7 +1218,8 @@ int DemoNdTables::get(int s)
 
 // Tile strides: the innermost axis is dense, every outer stride may be padded by a few words.  The padding is the one with
 // the fewest bank conflicts of a warp's accesses over the axis passes (32 neighbouring lines at a time), the smaller tile
-// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it.
+// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it.  The search takes 10 to 50 us of the host's time, so
+// tensors of the same chunk shape share one.
 void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
 {
     const int *s = e->s;
@@ -1246,11 +1247,14 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
         }
         return cost;
     };
+    const DemoNdTables::Layout *known = nullptr;
+    for (const DemoNdTables::Layout &l : tables->layouts)
+        if (l.s[0] == s[0] && l.s[1] == s[1] && l.s[2] == s[2] && l.s[3] == s[3]) known = &l;
     const int room = e->M / 16 > 64 ? e->M / 16 : 64;
     long long best = -1;
     int p[DEMO_ND_DIMS];
     p[3] = 1;
-    for (int pad2 = 0; pad2 <= (s[2] > 1 && !e->tail ? 8 : 0); ++pad2) {
+    for (int pad2 = 0; !known && pad2 <= (s[2] > 1 && !e->tail ? 8 : 0); ++pad2) {
         p[2] = s[3] + pad2;
         for (int pad1 = 0; pad1 <= (s[1] > 1 && s[2] * s[3] > 1 ? 8 : 0); ++pad1) {
             p[1] = p[2] * s[2] + pad1;
@@ -1266,6 +1270,18 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
                 }
             }
         }
+    }
+    if (known) {
+        for (int a = 0; a < DEMO_ND_DIMS; ++a) e->p[a] = known->p[a];
+        e->tile = known->tile;
+    } else {
+        DemoNdTables::Layout l;
+        for (int a = 0; a < DEMO_ND_DIMS; ++a) {
+            l.s[a] = s[a];
+            l.p[a] = e->p[a];
+        }
+        l.tile = e->tile;
+        tables->layouts.push_back(l);
     }
     // rows: the trailing elements that follow one another in the tensor and in the tile
     long long run = 1, span = 0;

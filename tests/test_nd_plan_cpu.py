@@ -1,0 +1,77 @@
+"""The host side of the N-D contexts without a device: a small program linked against the library drives the planner."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2411_19870_b200 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA_INCLUDE = "/usr/local/cuda/include"
+
+PRELUDE = """
+#include <chrono>
+#include <cstdio>
+#include "demo_internal.h"
+static DemoNdEntry entry(const int (&s)[4], const long long (&n)[4], int k)
+{
+    DemoNdEntry e{};
+    long long stride = 1, chunks = 1;
+    e.M = 1;
+    for (int a = 3; a >= 0; --a) {
+        e.s[a] = s[a];
+        e.c[a] = (int)(n[a] / s[a]);
+        e.stride[a] = stride;
+        stride *= n[a];
+        chunks *= e.c[a];
+        e.M *= s[a];
+        e.inv[a] = s[a] > 1 ? (unsigned)(((1ULL << 32) + s[a] - 1) / s[a]) : 0u;
+    }
+    e.k_eff = k < e.M ? k : e.M;
+    e.chunk_end = chunks;
+    return e;
+}
+"""
+
+
+def run(tmp_path, main):
+    lib = build.build_library()
+    if shutil.which("g++") is None or not os.path.isdir(CUDA_INCLUDE):
+        pytest.skip("no host compiler or CUDA headers")
+    src, exe = tmp_path / "plan.cc", tmp_path / "plan"
+    src.write_text(PRELUDE + "int main()\n{\n" + main + "\n}\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", CUDA_INCLUDE, "-I", os.path.join(os.path.dirname(lib), "csrc"), str(src), lib,
+                    "-Wl,-rpath," + os.path.dirname(lib), "-o", str(exe)], check=True, capture_output=True, text=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True, timeout=120).stdout.split()
+
+
+def test_tensors_of_one_chunk_shape_are_planned_once(tmp_path):
+    """The layout search of a chunk shape runs once per context, and a later tensor of the shape gets the same layout."""
+    out = run(tmp_path, """
+    using clock = std::chrono::steady_clock;
+    const int s[4] = {16, 12, 5, 7};
+    const long long n[4] = {64, 24, 10, 14}, n2[4] = {16, 12, 50, 70};
+    double first = 1e9, later = 1e9;
+    bool same = true;
+    for (int r = 0; r < 5; ++r) {
+        DemoNdTables tables;
+        DemoNdEntry a = entry(s, n, 32), b;
+        auto t0 = clock::now();
+        demo_nd_plan(&a, &tables);
+        auto t1 = clock::now();
+        for (int i = 0; i < 100; ++i) {
+            b = entry(s, i % 2 ? n : n2, 32);
+            demo_nd_plan(&b, &tables);
+            for (int d = 0; d < 4; ++d) same = same && a.p[d] == b.p[d];
+            same = same && a.tile == b.tile && a.tail == b.tail && a.threads == b.threads;
+        }
+        auto t2 = clock::now();
+        const double x = std::chrono::duration<double>(t1 - t0).count(), y = std::chrono::duration<double>(t2 - t1).count();
+        if (x < first) first = x;
+        if (y < later) later = y;
+    }
+    std::printf("%d %g %g", (int)same, first, later);
+    """)
+    assert out[0] == "1"
+    assert float(out[2]) < 20 * float(out[1])  # a hundred further tensors
