@@ -155,7 +155,9 @@ demo_status demo_payload_layout(const demo_ctx *ctx, int32_t tensor, int64_t *fi
  *   cuda_stream  cudaStream_t (NULL = default stream)
  * Device buffers must be 16-byte aligned and must not alias each other.  The pointer arrays are
  * host memory, read during the call and not retained.  Calls on one context must be issued in
- * stream order (one stream, or streams the caller orders).  Gradients or momenta that hold NaN or Inf
+ * stream order (one stream, or streams the caller orders): calls that run at the same time overwrite each other's device
+ * tables and chunk counters, and chunks may be left out.  The exception are demo_compress calls of different workers, which
+ * share nothing that they write; they may overlap.  Gradients or momenta that hold NaN or Inf
  * give unspecified values for the chunks they touch, but every chunk still gets k_eff records with
  * distinct, ascending, in-range indices, other chunks are unaffected and nothing hangs or traps.
  * Errors: INVALID_ARG, CUDA.

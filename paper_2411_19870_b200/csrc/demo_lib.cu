@@ -12,8 +12,6 @@
 #include "demo_internal.h"
 #include "launch.cuh"
 
-constexpr int TICKETS = 32;  // one per kernel of a call that may run beside another: tiles, N-D classes
-
 struct demo_ctx {
     demo_config cfg;
     int device = 0;
@@ -33,7 +31,10 @@ struct demo_ctx {
     long long chunks2d = 0, chunks1d = 0;
     DemoTensorEntry *d_entries2d = nullptr, *d_entries1d = nullptr;
 
-    DemoTickets *d_tickets = nullptr;  // [TICKETS] chunk counters, zero between launches
+    // [W + 1][slots] chunk counters, zero between launches: a row for each worker's compress calls and one for decode, so that compress
+    // calls of different workers may overlap; in a row one per kernel of a call that may run beside another (tiles, N-D classes)
+    DemoTickets *d_tickets = nullptr;
+    int ticket_slots = 1;
     float *d_C = nullptr;
     int *d_status = nullptr;
 
@@ -84,6 +85,14 @@ struct demo_ctx {
 static_assert(DEMO_ND_DIMS == DEMO_ND_MAX_DIMS, "public and internal axis limits disagree");
 
 namespace {
+
+cudaError_t make_tickets(demo_ctx *c)
+{
+    const size_t bytes = ((size_t)c->cfg.num_workers + 1) * (size_t)c->ticket_slots * sizeof(DemoTickets);
+    const cudaError_t err = cudaMalloc(&c->d_tickets, bytes);
+    return err == cudaSuccess ? cudaMemset(c->d_tickets, 0, bytes) : err;
+}
+DemoTickets *tickets_of(const demo_ctx *c, int row) { return c->d_tickets + (size_t)row * (size_t)c->ticket_slots; }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -290,7 +299,7 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     bool ok = true;
     ok = ok && cudaMalloc(&c->d_C, C.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_status, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->d_tickets, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
+    ok = ok && make_tickets(c) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_P, C.size() * sizeof(float)) == cudaSuccess;
     if (ok && c->n2d) ok = cudaMalloc(&c->d_entries2d, e2d.size() * sizeof(DemoTensorEntry)) == cudaSuccess;
     if (ok && c->n1d) ok = cudaMalloc(&c->d_entries1d, e1d.size() * sizeof(DemoTensorEntry)) == cudaSuccess;
@@ -323,7 +332,6 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     }
     ok = ok && cudaMemcpy(c->d_C, C.data(), C.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMemset(c->d_tickets, 0, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     if (ok && c->n2d)
         ok = cudaMemcpy(c->d_entries2d, e2d.data(), e2d.size() * sizeof(DemoTensorEntry), cudaMemcpyHostToDevice) ==
              cudaSuccess;
@@ -485,7 +493,8 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
     ok = ok && cudaMalloc(&c->d_tables, tables.data.size() * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_entries_nd, entries.size() * sizeof(DemoNdEntry)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_status, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->d_tickets, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
+    c->ticket_slots = (int)c->nd_classes.size();
+    ok = ok && make_tickets(c) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_g, W * T * sizeof(void *)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_m, W * T * sizeof(void *)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->d_x, T * sizeof(void *)) == cudaSuccess;
@@ -499,7 +508,6 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
     ok = ok && cudaMemcpy(c->d_entries_nd, entries.data(), entries.size() * sizeof(DemoNdEntry),
                           cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(c->d_status, 0, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMemset(c->d_tickets, 0, TICKETS * sizeof(DemoTickets)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         release(c);
@@ -594,7 +602,7 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
             n.entries = ctx->d_entries_nd + k.first;
             n.cls = k;
             n.wait_first = &k == &ctx->nd_classes.front();  // the classes run side by side
-            n.tickets = ctx->d_tickets + (&k - ctx->nd_classes.data());
+            n.tickets = tickets_of(ctx, worker) + (&k - ctx->nd_classes.data());
             if (demo_launch_compress_nd(n, ctx->sm_count, stream) != cudaSuccess) {
                 cudaGetLastError();
                 return DEMO_ERR_CUDA;
@@ -627,7 +635,7 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
     a.n_chunks = ctx->chunks2d;
     a.k = ctx->cfg.topk;  // <= s * s
     a.momentum_dct = ctx->momentum_dct ? 1 : 0;
-    a.tickets = ctx->d_tickets;
+    a.tickets = tickets_of(ctx, worker);
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     if (ctx->n2d && !small_tiles) {
         if (use_fast_path(ctx))
@@ -752,7 +760,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
             n.entries = ctx->d_entries_nd + k.first;
             n.cls = k;
             n.wait_first = &k == &ctx->nd_classes.front();  // the classes run side by side
-            n.tickets = ctx->d_tickets + (&k - ctx->nd_classes.data());
+            n.tickets = tickets_of(ctx, W) + (&k - ctx->nd_classes.data());
             if (demo_launch_decode_nd(n, ctx->sm_count, stream) != cudaSuccess) {
                 cudaGetLastError();
                 return DEMO_ERR_CUDA;
@@ -783,7 +791,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.n_entries = ctx->n2d;
     a.n_chunks = ctx->chunks2d;
     a.k = ctx->cfg.topk;  // <= s * s
-    a.tickets = ctx->d_tickets;
+    a.tickets = tickets_of(ctx, W);
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     if (ctx->n2d && !small_tiles) {
         // (a caller-supplied basis: the signs come from the dense kernels, there is no tensor-core variant)

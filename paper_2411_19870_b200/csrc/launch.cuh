@@ -29,7 +29,8 @@ struct StreamOrder {
 // Chunks of a persistent grid are handed out on demand: a CTA starts with chunk blockIdx.x and draws every further one from
 // a counter, so that a CTA that falls behind (another part of the memory system, a chunk with ties) gets fewer of them, and
 // the launch does not depend on which SM the CTAs came to.  The counter is zero between launches: the last CTA that is done
-// with it clears it.  One pair of words per kernel that may be in flight beside others of its context.  A grid with a CTA for
+// with it clears it.  One pair of words per kernel that may be in flight beside others of its context: two that drew from one counter
+// would leave chunks out.  A grid with a CTA for
 // every chunk has nothing to hand out and makes do without (NULL): an atomic operation and a wait for it less at either end
 // (256 x 256, s = 64: compress 9.1 -> 8.3 us, decode 6.6 -> 5.6).
 struct DemoTickets {

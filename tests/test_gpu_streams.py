@@ -1,0 +1,87 @@
+"""Calls of one context on several streams: compress calls of different workers side by side, and whole steps on streams that the
+caller orders by events.  Every run is compared bit for bit with the same calls one after the other."""
+import pytest
+import torch
+
+import paper_2411_19870_b200 as demo
+
+pytestmark = pytest.mark.gpu
+
+W = 3
+# name, shapes, chunk size or chunk shapes, k, caller-supplied basis: more chunks than a grid has CTAs or slots (chunks on demand)
+SETS = {
+    "s64_and_vectors": ([(4096, 2048), (2048,), (128, 64)], 64, 32, False),
+    "s32": ([(2048, 4096)], 32, 8, False),
+    "s128": ([(4096, 4096), (512,)], 128, 32, False),
+    "s64_basis": ([(4096, 4096)], 64, 32, True),
+    "nd_classes": ([(1024, 512, 3, 3), (9000, 512), (640,)], [(16, 16, 3, 3), (15, 64), (20,)], 12, False),
+}
+
+
+class Run:
+    def __init__(self, name):
+        shapes, chunk, k, basis = SETS[name]
+        kw = dict(chunk=chunk) if isinstance(chunk, int) else dict(chunk_shapes=chunk)
+        self.tr = demo.DemoTransform(shapes, topk=k, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=W, **kw)
+        if basis:
+            gen = torch.Generator().manual_seed(1)
+            self.tr.set_basis(torch.linalg.qr(torch.randn(64, 64, generator=gen, dtype=torch.float64))[0].float())
+        gen = torch.Generator("cuda").manual_seed(2)
+        self.g = [[torch.randn(s, device="cuda", generator=gen).bfloat16() for s in shapes] for _ in range(W)]
+        self.m = [[torch.randn(s, device="cuda", generator=gen) for s in shapes] for _ in range(W)]
+        self.x = [torch.randn(s, device="cuda", generator=gen) for s in shapes]
+        self.p = [torch.zeros(self.tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(W)]
+
+    def compress(self, w):
+        self.tr.compress(w, self.g[w], self.m[w], self.p[w])
+
+    def results(self):
+        torch.cuda.synchronize()
+        assert self.tr.device_status() == 0
+        return [v for m in self.m for v in m] + self.x + self.p
+
+
+def same(a, b):
+    return all(torch.equal(u, v) for u, v in zip(a.results(), b.results()))
+
+
+@pytest.mark.parametrize("name", SETS)
+def test_compress_of_different_workers_side_by_side(name):
+    ref, run = Run(name), Run(name)
+    streams = [torch.cuda.Stream() for _ in range(W)]
+    for r in (ref, run):
+        for w in range(W):
+            r.compress(w)  # (the pointer tables of this worker are on the device from here on)
+    torch.cuda.synchronize()
+    for _ in range(6):
+        for w in range(W):
+            ref.compress(w)
+    for _ in range(6):
+        for w, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                run.compress(w)
+    for r in (ref, run):
+        torch.cuda.synchronize()
+        r.tr.decode_apply(r.p, r.x)
+    assert same(ref, run)
+
+
+@pytest.mark.parametrize("name", SETS)
+def test_steps_on_streams_ordered_by_events(name):
+    ref, run = Run(name), Run(name)
+    torch.cuda.synchronize()
+    for _ in range(4):
+        for w in range(W):
+            ref.compress(w)
+        ref.tr.decode_apply(ref.p, ref.x)
+    streams, last = [torch.cuda.Stream() for _ in range(2)], None
+    for step in range(4):
+        for call in range(W + 1):
+            st = streams[(step + call) % 2]
+            if last is not None:
+                st.wait_event(last)
+            with torch.cuda.stream(st):
+                run.compress(call) if call < W else run.tr.decode_apply(run.p, run.x)
+                last = torch.cuda.Event()
+                last.record()
+    assert same(ref, run)
