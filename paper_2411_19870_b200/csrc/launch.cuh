@@ -5,7 +5,11 @@
 // finished.  A StreamOrder, the first object of the kernel, keeps the order:
 //   wait_first = 1: it touches nothing before everything queued earlier has finished;
 //   wait_first = 0: the kernel before it belongs to the same call, works on other data and itself waited for everything
-//     earlier; the two run side by side, and this one finishes last, so that whatever follows sees both complete.
+//     earlier; the two run side by side, and this one finishes last, so that whatever follows sees both complete.  It reads
+//     what earlier kernels wrote (momentum, records) before any wait of its own.  The wait instruction promises such writes to the
+//     grid that executes it, here the kernel before; that this one sees them too rests on two things: its CTAs start after every CTA of that
+//     kernel is past its wait, when those writes have reached the L2; and the fence below, without which an SM might still hold older
+//     lines of its own L1.
 // A CTA lets the next kernel be launched once it is itself past its wait, and the next kernel's CTAs come only when every
 // CTA of this one has come so far: they take registers and shared memory that nothing of this kernel still needs.  Tensor
 // memory is allocated behind the wait, so no CTA holds any while it waits for another kernel.
@@ -17,7 +21,10 @@ struct StreamOrder {
     const int wait_first;
     __device__ __forceinline__ explicit StreamOrder(int w) : wait_first(w)
     {
-        if (wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (wait_first)
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+        else
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     __device__ __forceinline__ ~StreamOrder()

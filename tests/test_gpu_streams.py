@@ -85,3 +85,21 @@ def test_steps_on_streams_ordered_by_events(name):
                 last = torch.cuda.Event()
                 last.record()
     assert same(ref, run)
+
+
+@pytest.mark.parametrize("name", SETS)
+def test_queued_steps_equal_steps_waited_for(name):
+    """Kernels may be resident before the work queued before them has finished, and the second kernel of a call runs beside the first:
+    many calls with nothing waited for in between against the same calls each waited for."""
+    ref, run = Run(name), Run(name)
+    torch.cuda.synchronize()
+    for r, wait in ((ref, True), (run, False)):
+        for _ in range(12):
+            for w in range(W):
+                r.compress(w)
+                if wait:
+                    torch.cuda.synchronize()
+            r.tr.decode_apply(r.p, r.x)
+            if wait:
+                torch.cuda.synchronize()
+    assert same(ref, run)
