@@ -1312,6 +1312,9 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
     e->threads = threads > MAX_THREADS ? MAX_THREADS : threads;
 }
 
+// Chunks of a class are drawn from a 32-bit counter.
+constexpr long long MAX_CLASS_CHUNKS = (1LL << 31) - 1;
+
 // A class is a size bucket with or without extents of 128 (registers) and with or without dense axes (shared memory), so
 // that a few chunks of one kind do not set the resources of all others.  Classes that would not fill the device (fewer than
 // two chunks per SM) are merged, with one another and, where it has all that they need, with the largest of the others:
@@ -1376,14 +1379,14 @@ void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vect
             if (x.s[a] != y.s[a] || x.stride[a] != y.stride[a]) return false;  // (the tile follows from these)
         return true;
     };
-    auto emit = [&](Group &d) {
-        if (d.list.empty()) return;
+    auto emit_part = [&](const Group &d, size_t first, size_t last) {  // tensors first .. last - 1
         DemoNdClass k = d.k;
         k.first = (int)entries.size();
-        k.n = (int)d.list.size();
+        k.n = (int)(last - first);
         k.n_chunks = 0;
         bool split = false;
-        for (DemoNdEntry e : d.list) {
+        for (size_t i = first; i < last; ++i) {
+            DemoNdEntry e = d.list[i];
             const long long n = e.chunk_end;
             e.chunk_begin = k.n_chunks;
             k.n_chunks += n;
@@ -1400,6 +1403,19 @@ void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vect
         if (split) k.threads = (k.threads + 63) / 64 * 64;  // two warps per 32 lines
         if (k.big && k.threads > MAX_THREADS_BIG) k.threads = MAX_THREADS_BIG;
         classes->push_back(k);
+    };
+    auto emit = [&](const Group &d) {
+        long long chunks = 0;
+        size_t first = 0;
+        for (size_t i = 0; i < d.list.size(); ++i) {
+            if (chunks + d.list[i].chunk_end > MAX_CLASS_CHUNKS) {  // (no tensor is larger than that)
+                emit_part(d, first, i);
+                first = i;
+                chunks = 0;
+            }
+            chunks += d.list[i].chunk_end;
+        }
+        if (first < d.list.size()) emit_part(d, first, d.list.size());
     };
     for (Group &d : g) emit(d);
     emit(rest);

@@ -358,7 +358,9 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         ok = tc_stage(f, pb, v, 0);
         if (!ok) break;
         const unsigned next = *f.drawn;  // (written before the barriers of the stages; overwritten behind those below)
-        if (2u * next + c < n_chunks) {  // row r of the group's next tiles on its way to L2
+        // row r of the group's next tiles on its way to L2.  (Without a counter next is NO_TICKET = 2^31 behind the grid, which then has a
+        // group for every pair: 2 next wraps to twice the grid's groups, past the last chunk.)
+        if (2u * next + c < n_chunks) {
             int e2 = e;
             const ChunkRef nr = locate<MANY>(a.entries, a.n_entries, 2u * next + c, k_eff, e2);
             const size_t at = nr.elem + (size_t)r * nr.n1;

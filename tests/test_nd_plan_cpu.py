@@ -75,3 +75,39 @@ def test_tensors_of_one_chunk_shape_are_planned_once(tmp_path):
     """)
     assert out[0] == "1"
     assert float(out[2]) < 20 * float(out[1])  # a hundred further tensors
+
+
+def test_classes_stay_below_the_range_of_the_chunk_counters(tmp_path):
+    """Three tensors of 2^31 - 1 chunks and a small one, all of one kind: no class of 2^31 chunks or more, every tensor in one class, its
+    chunks consecutive."""
+    out = run(tmp_path, """
+    const int s[4] = {1, 1, 1, 2};
+    const long long n[4] = {1, 1, 1, 2 * ((1LL << 31) - 1)}, few[4] = {1, 1, 1, 2000};
+    DemoNdTables tables;
+    std::vector<DemoNdEntry> entries;
+    for (int t = 0; t < 4; ++t) {
+        entries.push_back(entry(s, t == 2 ? few : n, 1));
+        entries.back().tensor = t;
+        demo_nd_plan(&entries.back(), &tables);
+    }
+    std::vector<DemoNdClass> classes;
+    demo_nd_classify(entries, 148, &classes);
+    bool in_order = true;
+    int next = 0;
+    for (const DemoNdClass &k : classes) {
+        long long at = 0;
+        in_order = in_order && k.first == next;
+        for (int i = 0; i < k.n; ++i) {
+            const DemoNdEntry &e = entries[k.first + i];
+            in_order = in_order && e.chunk_begin == at && e.layout <= k.first + i;
+            at = e.chunk_end;
+        }
+        in_order = in_order && at == k.n_chunks;
+        next += k.n;
+        std::printf("%lld ", k.n_chunks);
+    }
+    std::printf("%d %d", next, (int)in_order);
+    """)
+    chunks, (tensors, in_order) = [int(v) for v in out[:-2]], out[-2:]
+    assert max(chunks) <= 2 ** 31 - 1 and sum(chunks) == 3 * (2 ** 31 - 1) + 1000
+    assert tensors == "4" and in_order == "1"
