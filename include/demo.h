@@ -306,11 +306,12 @@ demo_status demo_set_decode_mode(demo_ctx *ctx, int32_t aggregation, int32_t phi
  * paper seeds them with the step number so that all workers agree).  Its rows are orthonormalised in
  * order by the Gram-Schmidt process on the device (fp64, one small kernel) and the result becomes the
  * active basis.  Synchronises cuda_stream.  INVALID_ARG when a row has no component left (singular
- * matrix); the previous basis then stays in force.
+ * matrix); the previous basis then stays in force.  The first call of a context allocates a small pinned host buffer
+ * (ALLOC when that fails), which may wait for other work of the device.
  *
  * demo_get_basis: copies the active basis (DCT or caller-supplied) to basis_host_out (HOST, s*s floats)
  * and synchronises cuda_stream.
- * Errors: INVALID_ARG, CUDA. */
+ * Errors: INVALID_ARG, ALLOC (demo_set_basis_gaussian), CUDA. */
 demo_status demo_set_basis(demo_ctx *ctx, const float *basis_host, void *cuda_stream);
 demo_status demo_set_basis_gaussian(demo_ctx *ctx, const float *gauss_host, void *cuda_stream);
 demo_status demo_get_basis(demo_ctx *ctx, float *basis_host_out, void *cuda_stream);

@@ -1010,14 +1010,17 @@ demo_status demo_set_basis_gaussian(demo_ctx *ctx, const float *gauss_host, void
     const int s = ctx->cfg.chunk;
     const size_t n = (size_t)s * s;
     // the kernel reads the matrix from pinned memory and replaces the active table only if its verdict is good, so a
-    // singular matrix leaves the previous basis in force; the pinned buffer is free again when the call returns
-    bool ok = ctx->h_gauss || cudaHostAlloc(&ctx->h_gauss, n * sizeof(float) + sizeof(int), cudaHostAllocDefault) == cudaSuccess;
-    int *verdict = ok ? reinterpret_cast<int *>(ctx->h_gauss + n) : nullptr;
-    if (ok) {
-        std::memcpy(ctx->h_gauss, gauss_host, n * sizeof(float));
-        *verdict = 1;
+    // singular matrix leaves the previous basis in force; the pinned buffer is free again when the call returns.  It is made on the first
+    // call: in demo_init it would cost every context up to 0.9 ms
+    if (!ctx->h_gauss && cudaHostAlloc(&ctx->h_gauss, n * sizeof(float) + sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->h_gauss = nullptr;
+        return DEMO_ERR_ALLOC;
     }
-    ok = ok && demo_launch_gram_schmidt(ctx->h_gauss, ctx->d_P, verdict, s, stream) == cudaSuccess;
+    int *verdict = reinterpret_cast<int *>(ctx->h_gauss + n);
+    std::memcpy(ctx->h_gauss, gauss_host, n * sizeof(float));
+    *verdict = 1;
+    bool ok = demo_launch_gram_schmidt(ctx->h_gauss, ctx->d_P, verdict, s, stream) == cudaSuccess;
     if (ok) ctx->launches += 1;
     ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
     if (!ok) {
