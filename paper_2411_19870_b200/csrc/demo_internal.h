@@ -8,6 +8,7 @@
 #include <vector>
 
 struct DemoTickets;  // launch.cuh
+struct DemoLaunch;   // launch.cuh
 
 // One payload record: flat index inside the chunk + fp32 coefficient (8 bytes, little-endian).
 struct DemoRecord {
@@ -75,32 +76,32 @@ struct DemoDecodeArgs {
 
 // Launchers (defined in the kernel translation units).  `s` is the chunk size.  Return the CUDA error of the launch.
 // Dense transforms of s x s tiles, any basis (kernels_generic.cu).
-cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
-cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);
 // Segments of 1-D tensors (any s, any basis) and, where `demo_small_tiles_supported` and the basis is the DCT, s x s tiles, in
 // one launch (kernels_small.cu).  Either list may be NULL.
 bool demo_small_tiles_supported(int s);
-cudaError_t demo_launch_compress_small(int s, const DemoCompressArgs *segs, const DemoCompressArgs *tiles, int sm_count,
+cudaError_t demo_launch_compress_small(int s, const DemoCompressArgs *segs, const DemoCompressArgs *tiles, DemoLaunch &dev,
                                        cudaStream_t stream);
-cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count,
+cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, DemoLaunch &dev,
                                      cudaStream_t stream);
 // Fast-DCT kernels for 2-D tensors; `supported` tells whether chunk size s has one.
 bool demo_fast_supported(int s);
-cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
-cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);
 // s = 32 (kernels_fast32.cu).
-cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
 // s = 64 with TMA tensor maps (kernels_fast64.cu; cudaErrorNotSupported without them).
-cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
 // s = 128 (kernels_fast128.cu); compress needs the TMA tensor maps (cudaErrorNotSupported without them).
-cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
-cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);
 
 // Tensor-core kernels for 2-D tensors under a caller-supplied basis (kernels_tc.cu): tcgen05 MMAs with
 // 3xTF32 splitting, chunk size 64 only.
 bool demo_tc_supported(int s);
-cudaError_t demo_launch_compress_tc(const DemoCompressArgs &a, int sm_count, cudaStream_t stream);
-cudaError_t demo_launch_decode_tc(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_tc(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+cudaError_t demo_launch_decode_tc(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);
 
 // Self-test of the bounded wait (kernels_fast.cu): one CTA waits, for at most `limit_cycles`, on an
 // mbarrier that nothing completes, records DEMO_DEV_TIMEOUT in *status and returns.
@@ -210,10 +211,10 @@ struct DemoApplySignsArgs {
     float lr, wd;
 };
 constexpr int demo_apply_pieces[2] = {1024, 4};  // a block's, a thread's
-cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, DemoLaunch &dev, cudaStream_t stream);
 
-cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, cudaStream_t stream);
-cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, int sm_count, cudaStream_t stream);
+cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);
 
 // Locate the tensor that owns chunk id c: the last entry with chunk_begin <= c.
 __device__ __forceinline__ int demo_find_entry(const DemoTensorEntry *entries, int n, long long c)

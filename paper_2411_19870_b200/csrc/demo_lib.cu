@@ -15,7 +15,7 @@
 struct demo_ctx {
     demo_config cfg;
     int device = 0;
-    int sm_count = 0;
+    DemoLaunch launch;
     int n_tensors = 0;
     int path = DEMO_PATH_AUTO;
     float alpha = 1.0f;  // momentum-subtraction coefficient
@@ -233,7 +233,7 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
     c->cfg = *cfg;
     c->device = cuda_device;
     c->n_tensors = n_tensors;
-    if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
+    if (cudaDeviceGetAttribute(&c->launch.sm_count, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
         release(c);
         return DEMO_ERR_CUDA;
     }
@@ -430,7 +430,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
     c->device = cuda_device;
     c->n_tensors = n_tensors;
     c->nd = true;
-    if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
+    if (cudaDeviceGetAttribute(&c->launch.sm_count, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
         release(c);
         return DEMO_ERR_CUDA;
     }
@@ -475,7 +475,7 @@ demo_status demo_init_nd(demo_ctx **out, const demo_config *cfg, const demo_nd_t
             rec += n_ch * e.k_eff;
         }
         c->total_records = rec;
-        demo_nd_classify(entries, c->sm_count, &c->nd_classes);
+        demo_nd_classify(entries, c->launch.sm_count, &c->nd_classes);
         if (tables.data.empty()) tables.data.push_back(1.0f);  // no dense extent: never read
         const size_t W = (size_t)cfg->num_workers, T = (size_t)n_tensors;
         c->h_g.assign(W * T, nullptr);
@@ -603,7 +603,7 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
             n.cls = k;
             n.wait_first = &k == &ctx->nd_classes.front();  // the classes run side by side
             n.tickets = tickets_of(ctx, worker) + (&k - ctx->nd_classes.data());
-            if (demo_launch_compress_nd(n, ctx->sm_count, stream) != cudaSuccess) {
+            if (demo_launch_compress_nd(n, ctx->launch, stream) != cudaSuccess) {
                 cudaGetLastError();
                 return DEMO_ERR_CUDA;
             }
@@ -639,17 +639,17 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     if (ctx->n2d && !small_tiles) {
         if (use_fast_path(ctx))
-            err = demo_launch_compress_fast(s, a, ctx->sm_count, stream);
+            err = demo_launch_compress_fast(s, a, ctx->launch, stream);
         else if (use_tc_path(ctx))
-            err = demo_launch_compress_tc(a, ctx->sm_count, stream);
+            err = demo_launch_compress_tc(a, ctx->launch, stream);
         else
-            err = demo_launch_compress_generic(s, a, ctx->sm_count, stream);
+            err = demo_launch_compress_generic(s, a, ctx->launch, stream);
         ctx->launches += 1;
     }
     if (err == cudaSuccess && (ctx->n1d || small_tiles)) {
         // behind the kernel of the tiles, so that it fills the SMs that one leaves idle at its end
         a1.wait_first = small_tiles || !ctx->n2d;
-        err = demo_launch_compress_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, stream);
+        err = demo_launch_compress_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->launch, stream);
         ctx->launches += 1;
     }
     if (err != cudaSuccess) {
@@ -761,7 +761,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
             n.cls = k;
             n.wait_first = &k == &ctx->nd_classes.front();  // the classes run side by side
             n.tickets = tickets_of(ctx, W) + (&k - ctx->nd_classes.data());
-            if (demo_launch_decode_nd(n, ctx->sm_count, stream) != cudaSuccess) {
+            if (demo_launch_decode_nd(n, ctx->launch, stream) != cudaSuccess) {
                 cudaGetLastError();
                 return DEMO_ERR_CUDA;
             }
@@ -796,17 +796,17 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     if (ctx->n2d && !small_tiles) {
         // (a caller-supplied basis: the signs come from the dense kernels, there is no tensor-core variant)
         if (use_fast_path(ctx))
-            err = demo_launch_decode_fast(s, a, ctx->sm_count, stream);
+            err = demo_launch_decode_fast(s, a, ctx->launch, stream);
         else if (use_tc_path(ctx) && !signs)
-            err = demo_launch_decode_tc(a, ctx->sm_count, stream);
+            err = demo_launch_decode_tc(a, ctx->launch, stream);
         else
-            err = demo_launch_decode_generic(s, a, ctx->sm_count, stream);
+            err = demo_launch_decode_generic(s, a, ctx->launch, stream);
         ctx->launches += 1;
     }
     if (err == cudaSuccess && (ctx->n1d || small_tiles)) {
         // behind the kernel of the tiles, so that it fills the SMs that one leaves idle at its end
         a1.wait_first = small_tiles || !ctx->n2d;
-        err = demo_launch_decode_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->sm_count, stream);
+        err = demo_launch_decode_small(s, ctx->n1d ? &a1 : nullptr, small_tiles ? &a : nullptr, ctx->launch, stream);
         ctx->launches += 1;
     }
     if (err != cudaSuccess) {
@@ -858,7 +858,7 @@ demo_status demo_apply_signs(demo_ctx *ctx, const int8_t *const *signs, float *c
         a.x_ptrs = ctx->d_x;
         a.lr = ctx->cfg.lr;
         a.wd = ctx->cfg.weight_decay;
-        err = demo_launch_apply_signs(a, ctx->sm_count, stream);
+        err = demo_launch_apply_signs(a, ctx->launch, stream);
         ctx->launches += 1;
     }
     if (err != cudaSuccess) {

@@ -84,14 +84,14 @@ __device__ __forceinline__ void radix_select(const float *Q, int M, int k_eff, u
 }
 
 template <typename K>
-cudaError_t launch_persistent(K kernel, size_t smem, long long n_chunks, int sm_count, cudaStream_t stream,
+cudaError_t launch_persistent(K kernel, size_t smem, long long n_chunks, DemoLaunch &dev, cudaStream_t stream,
                               const void *args_struct_ptr)
 {
     if (n_chunks <= 0) return cudaSuccess;
     int per_sm = 0;
-    const cudaError_t err = demo_resident_ctas((const void *)kernel, GEN_THREADS, smem, &per_sm);
+    const cudaError_t err = demo_resident_ctas(dev, (const void *)kernel, GEN_THREADS, smem, &per_sm);
     if (err != cudaSuccess) return err;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid > n_chunks) grid = n_chunks;
     void *params[] = {const_cast<void *>(args_struct_ptr)};
     return demo_launch_kernel((const void *)kernel, grid, GEN_THREADS, smem, stream, params);

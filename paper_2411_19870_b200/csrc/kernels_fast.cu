@@ -342,15 +342,15 @@ constexpr int DECODE_THREADS = 64;
 // Persistent launch: CTAs of `threads` threads (threads / S slots), as many as fit the device, each
 // striding over groups of chunks.
 template <typename K, typename A>
-cudaError_t launch(K kernel, int threads, int nch, size_t smem, int sm_count, cudaStream_t stream, A args)
+cudaError_t launch(K kernel, int threads, int nch, size_t smem, DemoLaunch &dev, cudaStream_t stream, A args)
 {
     const long long n_chunks = args.n_chunks;
     if (n_chunks <= 0) return cudaSuccess;
     int per_sm = 0;
-    const cudaError_t err = demo_resident_ctas((const void *)kernel, threads, smem, &per_sm);
+    const cudaError_t err = demo_resident_ctas(dev, (const void *)kernel, threads, smem, &per_sm);
     if (err != cudaSuccess) return err;
     const long long groups = (n_chunks + nch - 1) / nch;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid > groups) grid = groups;
     if (grid == groups) args.tickets = nullptr;
     void *params[] = {&args};
@@ -358,17 +358,17 @@ cudaError_t launch(K kernel, int threads, int nch, size_t smem, int sm_count, cu
 }
 
 template <int S>
-cudaError_t launch_decode(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t launch_decode(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     constexpr int TH = DECODE_THREADS;
     constexpr int NCH = TH / S;
     const size_t smem = decode_slot_bytes<S>(a.agg == 2) * NCH;
     auto pick = [&](auto signs) {
         constexpr bool SIGNS = decltype(signs)::value;
-        if (a.k <= 64) return launch(decode_fast_kernel<S, TH, SIGNS, LISTED>, TH, NCH, smem, sm_count, stream, a);
+        if (a.k <= 64) return launch(decode_fast_kernel<S, TH, SIGNS, LISTED>, TH, NCH, smem, dev, stream, a);
         if constexpr (!(SIGNS && S == 64))
-            if (a.k <= STAGE_RECORDS) return launch(decode_fast_kernel<S, TH, SIGNS, STAGED>, TH, NCH, smem, sm_count, stream, a);
-        return launch(decode_fast_kernel<S, TH, SIGNS, BARRIERS>, TH, NCH, smem, sm_count, stream, a);
+            if (a.k <= STAGE_RECORDS) return launch(decode_fast_kernel<S, TH, SIGNS, STAGED>, TH, NCH, smem, dev, stream, a);
+        return launch(decode_fast_kernel<S, TH, SIGNS, BARRIERS>, TH, NCH, smem, dev, stream, a);
     };
     return a.sign_ptrs != nullptr ? pick(std::true_type{}) : pick(std::false_type{});
 }
@@ -399,18 +399,18 @@ cudaError_t demo_launch_wait_selftest(int *status, long long limit_cycles, cudaS
 
 bool demo_fast_supported(int s) { return s == 128 || s == 64 || s == 32; }
 
-cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
-    if (s == 128) return demo_launch_compress_fast128(a, sm_count, stream);
-    if (s == 64) return demo_launch_compress_fast64(a, sm_count, stream);
-    if (s == 32) return demo_launch_compress_fast32(a, sm_count, stream);
+    if (s == 128) return demo_launch_compress_fast128(a, dev, stream);
+    if (s == 64) return demo_launch_compress_fast64(a, dev, stream);
+    if (s == 32) return demo_launch_compress_fast32(a, dev, stream);
     return cudaErrorInvalidValue;
 }
 
-cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
-    if (s == 128) return demo_launch_decode_fast128(a, sm_count, stream);
-    if (s == 64) return launch_decode<64>(a, sm_count, stream);
-    if (s == 32) return launch_decode<32>(a, sm_count, stream);
+    if (s == 128) return demo_launch_decode_fast128(a, dev, stream);
+    if (s == 64) return launch_decode<64>(a, dev, stream);
+    if (s == 32) return launch_decode<32>(a, dev, stream);
     return cudaErrorInvalidValue;
 }

@@ -852,18 +852,18 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
 }
 
 template <typename K, typename A>
-cudaError_t launch128(K kernel, size_t smem, int sm_count, cudaStream_t stream, A args)
+cudaError_t launch128(K kernel, size_t smem, DemoLaunch &dev, cudaStream_t stream, A args)
 {
     const long long n_chunks = args.n_chunks;
     if (n_chunks <= 0) return cudaSuccess;
-    const cudaError_t err = demo_allow_smem((const void *)kernel, smem);
+    const cudaError_t err = demo_allow_smem(dev, (const void *)kernel);
     if (err != cudaSuccess) return err;
     // CTAs per SM: two by the launch bounds (registers), fewer if shared memory (227 KB, 1 KB reserved per CTA) says
     // so.  The occupancy calculator is not asked: it answers 1 for a kernel that allocates tensor memory.
     int per_sm = (int)((227u * 1024u) / (smem + 1024u));
     if (per_sm > 2) per_sm = 2;
     if (per_sm < 1) per_sm = 1;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid > n_chunks) grid = n_chunks;
     if (grid == n_chunks) args.tickets = nullptr;
     void *params[] = {&args};
@@ -872,15 +872,15 @@ cudaError_t launch128(K kernel, size_t smem, int sm_count, cudaStream_t stream, 
 
 }  // namespace
 
-cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (!a.tmap_m || !a.tmap_g) return cudaErrorNotSupported;
     if (a.grad_bf16)
-        return launch128(compress_fast128_kernel<__nv_bfloat16>, compress128_smem<__nv_bfloat16>(), sm_count, stream, a);
-    return launch128(compress_fast128_kernel<float>, compress128_smem<float>(), sm_count, stream, a);
+        return launch128(compress_fast128_kernel<__nv_bfloat16>, compress128_smem<__nv_bfloat16>(), dev, stream, a);
+    return launch128(compress_fast128_kernel<float>, compress128_smem<float>(), dev, stream, a);
 }
 
-cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     // Staged while the additions are short (k <= 64) or all workers' records fit one batch; a further batch of longer lists
     // comes too late.  8192 x 8192, staged / with barriers: k = 32, W = 1 139 / 149 us, W = 8 145 / 169 us, k = 64, W = 8
@@ -889,8 +889,8 @@ cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, int sm_count, cu
     const bool staged = a.k <= 64 || (a.k <= STAGE_RECORDS && (long long)a.W << stage_shift(a.k) <= STAGE_RECORDS);
     auto pick = [&](auto signs) {
         constexpr bool SIGNS = decltype(signs)::value;
-        return staged ? launch128(decode_fast128_kernel<SIGNS, true>, DECODE128_SMEM, sm_count, stream, a)
-                      : launch128(decode_fast128_kernel<SIGNS, false>, DECODE128_SMEM, sm_count, stream, a);
+        return staged ? launch128(decode_fast128_kernel<SIGNS, true>, DECODE128_SMEM, dev, stream, a)
+                      : launch128(decode_fast128_kernel<SIGNS, false>, DECODE128_SMEM, dev, stream, a);
     };
     return a.sign_ptrs ? pick(std::true_type{}) : pick(std::false_type{});
 }

@@ -375,18 +375,18 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) compress32_kernel(DemoCompre
 }
 
 template <typename GT, bool BIGK>
-cudaError_t launch32(DemoCompressArgs a, int sm_count, cudaStream_t stream)
+cudaError_t launch32(DemoCompressArgs a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.n_chunks <= 0) return cudaSuccess;
     const void *kernel = (const void *)compress32_kernel<GT, BIGK>;
     const size_t smem = sizeof(Area<GT>) * WARPS + 16;
-    const cudaError_t err = demo_allow_smem(kernel, smem);
+    const cudaError_t err = demo_allow_smem(dev, kernel);
     if (err != cudaSuccess) return err;
     // by registers and shared memory (1 KB reserved per CTA; tensor memory has room for sixteen, the occupancy calculator
     // does not know about it)
     const int by_smem = (int)(227u * 1024u / (smem + 1024u)), per_sm = by_smem < CTAS ? by_smem : CTAS;
     const long long n_ctas = (a.n_chunks + WARPS - 1) / WARPS;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid >= n_ctas) {
         grid = n_ctas;
         a.tickets = nullptr;
@@ -397,9 +397,9 @@ cudaError_t launch32(DemoCompressArgs a, int sm_count, cudaStream_t stream)
 
 }  // namespace
 
-cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.k > MAX_K_LISTED)
-        return a.grad_bf16 ? launch32<__nv_bfloat16, true>(a, sm_count, stream) : launch32<float, true>(a, sm_count, stream);
-    return a.grad_bf16 ? launch32<__nv_bfloat16, false>(a, sm_count, stream) : launch32<float, false>(a, sm_count, stream);
+        return a.grad_bf16 ? launch32<__nv_bfloat16, true>(a, dev, stream) : launch32<float, true>(a, dev, stream);
+    return a.grad_bf16 ? launch32<__nv_bfloat16, false>(a, dev, stream) : launch32<float, false>(a, dev, stream);
 }

@@ -423,13 +423,13 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
 }
 
 template <typename GT, int THREADS, bool QDOM, bool BIGK>
-cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     constexpr int NCH = THREADS / S;
     auto kernel = compress64_kernel<GT, THREADS, QDOM, BIGK>;
     const size_t smem = slot_bytes<GT>() * NCH + 16;
     if (a.n_chunks <= 0) return cudaSuccess;
-    const cudaError_t err = demo_allow_smem((const void *)kernel, smem);
+    const cudaError_t err = demo_allow_smem(dev, (const void *)kernel);
     if (err != cudaSuccess) return err;
     // CTAs per SM: registers (launch bounds: 512 threads per SM), shared memory (227 KB, 1 KB reserved per CTA)
     // and tensor memory (512 columns, 64 per four warps).  The occupancy calculator is not asked: it does not
@@ -441,7 +441,7 @@ cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t strea
     if (per_sm > tmem_limit) per_sm = tmem_limit;
     if (per_sm < 1) per_sm = 1;
     const long long groups = (a.n_chunks + NCH - 1) / NCH;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid > groups) grid = groups;
     DemoCompressArgs b = a;
     if (grid == groups) b.tickets = nullptr;
@@ -452,13 +452,13 @@ cudaError_t launch64(const DemoCompressArgs &a, int sm_count, cudaStream_t strea
 }  // namespace
 
 // Needs the TMA tensor maps of both tensors.
-cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.tmap_m == nullptr || a.tmap_g == nullptr) return cudaErrorNotSupported;
     auto pick = [&](auto gt, auto qdom) {
         using GT = decltype(gt);
         constexpr bool Q = decltype(qdom)::value;
-        return a.k > MAX_K_LISTED ? launch64<GT, 64, Q, true>(a, sm_count, stream) : launch64<GT, 64, Q, false>(a, sm_count, stream);
+        return a.k > MAX_K_LISTED ? launch64<GT, 64, Q, true>(a, dev, stream) : launch64<GT, 64, Q, false>(a, dev, stream);
     };
     if (a.momentum_dct)
         return a.grad_bf16 ? pick(__nv_bfloat16{}, std::true_type{}) : pick(float{}, std::true_type{});

@@ -280,43 +280,43 @@ __global__ void __launch_bounds__(GEN_THREADS) apply_signs_kernel(DemoApplySigns
 }
 
 template <int S>
-cudaError_t compress_dispatch(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t compress_dispatch(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     const size_t extra = (256 + 8 + 2) * sizeof(unsigned);
-    return launch_persistent(compress_generic_kernel<S>, 3 * S * S * sizeof(float) + extra, a.n_chunks, sm_count, stream, &a);
+    return launch_persistent(compress_generic_kernel<S>, 3 * S * S * sizeof(float) + extra, a.n_chunks, dev, stream, &a);
 }
 
 template <int S>
-cudaError_t decode_dispatch(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t decode_dispatch(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
-    return launch_persistent(decode_generic_kernel<S>, 2 * S * S * sizeof(float) + S * S * 2, a.n_chunks, sm_count, stream, &a);
+    return launch_persistent(decode_generic_kernel<S>, 2 * S * S * sizeof(float) + S * S * 2, a.n_chunks, dev, stream, &a);
 }
 
 }  // namespace
 
-cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, int sm_count,
+cudaError_t demo_launch_compress_generic(int s, const DemoCompressArgs &a, DemoLaunch &dev,
                                          cudaStream_t stream)
 {
     switch (s) {
-        case 8: return compress_dispatch<8>(a, sm_count, stream);
-        case 16: return compress_dispatch<16>(a, sm_count, stream);
-        case 32: return compress_dispatch<32>(a, sm_count, stream);
-        case 64: return compress_dispatch<64>(a, sm_count, stream);
-        case 128: return compress_dispatch<128>(a, sm_count, stream);
+        case 8: return compress_dispatch<8>(a, dev, stream);
+        case 16: return compress_dispatch<16>(a, dev, stream);
+        case 32: return compress_dispatch<32>(a, dev, stream);
+        case 64: return compress_dispatch<64>(a, dev, stream);
+        case 128: return compress_dispatch<128>(a, dev, stream);
         default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.n_pieces <= 0) return cudaSuccess;
     const bool blocks = a.piece == demo_apply_pieces[0];
     const auto kernel = blocks ? apply_signs_kernel<true> : apply_signs_kernel<false>;
     const long long need = blocks ? a.n_pieces : (a.n_pieces + GEN_THREADS - 1) / GEN_THREADS;
     int per_sm = 0;
-    const cudaError_t err = demo_resident_ctas((const void *)kernel, GEN_THREADS, 0, &per_sm);
+    const cudaError_t err = demo_resident_ctas(dev, (const void *)kernel, GEN_THREADS, 0, &per_sm);
     if (err != cudaSuccess) return err;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid > need) grid = need;
     // An ordinary launch: resident beside the last CTAs of decode_signs, these would keep that kernel's split of the SM into
     // shared memory and L1 to their end, and the L1 left (28 KB) does not hold the loads in flight (632 -> about 830 us).
@@ -324,15 +324,15 @@ cudaError_t demo_launch_apply_signs(const DemoApplySignsArgs &a, int sm_count, c
     return cudaGetLastError();
 }
 
-cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, int sm_count,
+cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, DemoLaunch &dev,
                                        cudaStream_t stream)
 {
     switch (s) {
-        case 8: return decode_dispatch<8>(a, sm_count, stream);
-        case 16: return decode_dispatch<16>(a, sm_count, stream);
-        case 32: return decode_dispatch<32>(a, sm_count, stream);
-        case 64: return decode_dispatch<64>(a, sm_count, stream);
-        case 128: return decode_dispatch<128>(a, sm_count, stream);
+        case 8: return decode_dispatch<8>(a, dev, stream);
+        case 16: return decode_dispatch<16>(a, dev, stream);
+        case 32: return decode_dispatch<32>(a, dev, stream);
+        case 64: return decode_dispatch<64>(a, dev, stream);
+        case 128: return decode_dispatch<128>(a, dev, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -528,8 +528,8 @@ extern "C" demo_status demo_decode_apply_static(const demo_config *cfg, const de
             }
             base = g_static_base[cuda_device];
         }
-        int sm_count = 0;
-        if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
+        DemoLaunch dev;
+        if (cudaDeviceGetAttribute(&dev.sm_count, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
             result = DEMO_ERR_CUDA;
             break;
         }
@@ -602,13 +602,13 @@ extern "C" demo_status demo_decode_apply_static(const demo_config *cfg, const de
             a.entries = reinterpret_cast<const DemoTensorEntry *>(base + OFF_ENTRIES);
             a.n_entries = n2d;
             a.n_chunks = chunks2d;
-            err = demo_launch_decode_generic(s, a, sm_count, stream);
+            err = demo_launch_decode_generic(s, a, dev, stream);
         }
         if (err == cudaSuccess && n1d) {
             a.entries = reinterpret_cast<const DemoTensorEntry *>(base + OFF_ENTRIES) + n2d;
             a.n_entries = n1d;
             a.n_chunks = chunks1d;
-            err = demo_launch_decode_small(s, &a, nullptr, sm_count, stream);
+            err = demo_launch_decode_small(s, &a, nullptr, dev, stream);
         }
         if (err != cudaSuccess) {
             cudaGetLastError();

@@ -1181,14 +1181,14 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
 }
 
 template <typename K, typename A>
-cudaError_t launch_nd(K kernel, size_t smem, int sm_count, cudaStream_t stream, A args)
+cudaError_t launch_nd(K kernel, size_t smem, DemoLaunch &dev, cudaStream_t stream, A args)
 {
     const DemoNdClass &cls = args.cls;
     if (cls.n_chunks <= 0) return cudaSuccess;
     int per_sm = 0;
-    const cudaError_t err = demo_resident_ctas((const void *)kernel, cls.threads, smem, &per_sm);
+    const cudaError_t err = demo_resident_ctas(dev, (const void *)kernel, cls.threads, smem, &per_sm);
     if (err != cudaSuccess) return err;
-    long long grid = (long long)sm_count * per_sm;
+    long long grid = (long long)dev.sm_count * per_sm;
     if (grid > cls.n_chunks) grid = cls.n_chunks;
     if (grid == cls.n_chunks) args.tickets = nullptr;
     void *params[] = {&args};
@@ -1421,19 +1421,19 @@ void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vect
     emit(rest);
 }
 
-cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_compress_nd(const DemoNdCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     const size_t smem = shared_bytes(a.cls, true);
     if (a.cls.big)
-        return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, true>, smem, sm_count, stream, a)
-                           : launch_nd(compress_nd_kernel<float, true>, smem, sm_count, stream, a);
-    return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, false>, smem, sm_count, stream, a)
-                       : launch_nd(compress_nd_kernel<float, false>, smem, sm_count, stream, a);
+        return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, true>, smem, dev, stream, a)
+                           : launch_nd(compress_nd_kernel<float, true>, smem, dev, stream, a);
+    return a.grad_bf16 ? launch_nd(compress_nd_kernel<__nv_bfloat16, false>, smem, dev, stream, a)
+                       : launch_nd(compress_nd_kernel<float, false>, smem, dev, stream, a);
 }
 
-cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_decode_nd(const DemoNdDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     const size_t smem = shared_bytes(a.cls, false) + (a.agg == 2 ? align16((size_t)a.cls.tile * 2) : 0);
-    return a.cls.big ? launch_nd(decode_nd_kernel<true>, smem, sm_count, stream, a)
-                     : launch_nd(decode_nd_kernel<false>, smem, sm_count, stream, a);
+    return a.cls.big ? launch_nd(decode_nd_kernel<true>, smem, dev, stream, a)
+                     : launch_nd(decode_nd_kernel<false>, smem, dev, stream, a);
 }

@@ -500,64 +500,64 @@ int blocks_for(long long units, int per_block, int sm_count)
     return (int)(b < cap ? b : cap);
 }
 template <class A>
-cudaError_t launch(const void *kernel, int segs_per_block, int tiles_per_warp, const A *segs, const A *tiles, int sm_count, cudaStream_t stream)
+cudaError_t launch(const void *kernel, int segs_per_block, int tiles_per_warp, const A *segs, const A *tiles, DemoLaunch &dev, cudaStream_t stream)
 {
     A none{};
     const A &sa = segs ? *segs : none, &ta = tiles ? *tiles : none;
-    int seg_blocks = segs ? blocks_for(sa.n_chunks, segs_per_block, sm_count) : 0;
-    const int tile_blocks = tiles ? blocks_for(ta.n_chunks, tiles_per_warp * WARPS, sm_count) : 0;
+    int seg_blocks = segs ? blocks_for(sa.n_chunks, segs_per_block, dev.sm_count) : 0;
+    const int tile_blocks = tiles ? blocks_for(ta.n_chunks, tiles_per_warp * WARPS, dev.sm_count) : 0;
     if (seg_blocks + tile_blocks == 0) return cudaSuccess;
     void *params[] = {const_cast<A *>(&sa), const_cast<A *>(&ta), &seg_blocks};
     return demo_launch_kernel(kernel, seg_blocks + tile_blocks, THREADS, 0, stream, params);
 }
 
 template <int S>
-cudaError_t compress_small(const DemoCompressArgs *segs, const DemoCompressArgs *tiles, int sm_count, cudaStream_t stream)
+cudaError_t compress_small(const DemoCompressArgs *segs, const DemoCompressArgs *tiles, DemoLaunch &dev, cudaStream_t stream)
 {
     if constexpr (S <= 16) {
         if (tiles)
             return launch(tiles->grad_bf16 ? (const void *)compress_small_kernel<S, __nv_bfloat16, true>
                                            : (const void *)compress_small_kernel<S, float, true>,
-                          Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
+                          Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, dev, stream);
     }
-    return launch((const void *)compress_small_kernel<S, float, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoCompressArgs *)nullptr, sm_count, stream);
+    return launch((const void *)compress_small_kernel<S, float, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoCompressArgs *)nullptr, dev, stream);
 }
 template <int S>
-cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count, cudaStream_t stream)
+cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, DemoLaunch &dev, cudaStream_t stream)
 {
     if constexpr (S <= 16) {
         if (tiles)
-            return launch((const void *)decode_small_kernel<S, true>, Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, sm_count, stream);
+            return launch((const void *)decode_small_kernel<S, true>, Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, dev, stream);
     }
-    return launch((const void *)decode_small_kernel<S, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, sm_count, stream);
+    return launch((const void *)decode_small_kernel<S, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, dev, stream);
 }
 
 }  // namespace
 
 bool demo_small_tiles_supported(int s) { return s == 8 || s == 16; }
 
-cudaError_t demo_launch_compress_small(int s, const DemoCompressArgs *segs, const DemoCompressArgs *tiles, int sm_count,
+cudaError_t demo_launch_compress_small(int s, const DemoCompressArgs *segs, const DemoCompressArgs *tiles, DemoLaunch &dev,
                                        cudaStream_t stream)
 {
     switch (s) {
-        case 8: return compress_small<8>(segs, tiles, sm_count, stream);
-        case 16: return compress_small<16>(segs, tiles, sm_count, stream);
-        case 32: return compress_small<32>(segs, nullptr, sm_count, stream);
-        case 64: return compress_small<64>(segs, nullptr, sm_count, stream);
-        case 128: return compress_small<128>(segs, nullptr, sm_count, stream);
+        case 8: return compress_small<8>(segs, tiles, dev, stream);
+        case 16: return compress_small<16>(segs, tiles, dev, stream);
+        case 32: return compress_small<32>(segs, nullptr, dev, stream);
+        case 64: return compress_small<64>(segs, nullptr, dev, stream);
+        case 128: return compress_small<128>(segs, nullptr, dev, stream);
         default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, int sm_count,
+cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, DemoLaunch &dev,
                                      cudaStream_t stream)
 {
     switch (s) {
-        case 8: return decode_small<8>(segs, tiles, sm_count, stream);
-        case 16: return decode_small<16>(segs, tiles, sm_count, stream);
-        case 32: return decode_small<32>(segs, nullptr, sm_count, stream);
-        case 64: return decode_small<64>(segs, nullptr, sm_count, stream);
-        case 128: return decode_small<128>(segs, nullptr, sm_count, stream);
+        case 8: return decode_small<8>(segs, tiles, dev, stream);
+        case 16: return decode_small<16>(segs, tiles, dev, stream);
+        case 32: return decode_small<32>(segs, nullptr, dev, stream);
+        case 64: return decode_small<64>(segs, nullptr, dev, stream);
+        case 128: return decode_small<128>(segs, nullptr, dev, stream);
         default: return cudaErrorInvalidValue;
     }
 }

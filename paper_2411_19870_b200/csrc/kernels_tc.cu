@@ -551,13 +551,13 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
 }
 
 template <typename K, typename A>
-cudaError_t launch_tc(K kernel, int groups, int smem, A a, int sm_count, cudaStream_t stream)
+cudaError_t launch_tc(K kernel, int groups, int smem, A a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.n_chunks <= 0) return cudaSuccess;
-    const cudaError_t err = demo_allow_smem((const void *)kernel, (size_t)smem);
+    const cudaError_t err = demo_allow_smem(dev, (const void *)kernel);
     if (err != cudaSuccess) return err;
     const long long n_ctas = ((a.n_chunks + 1) / 2 + groups - 1) / groups;
-    const long long grid = n_ctas < sm_count ? n_ctas : sm_count;  // one CTA per SM: it takes all of the tensor memory
+    const long long grid = n_ctas < dev.sm_count ? n_ctas : dev.sm_count;  // one CTA per SM: it takes all of the tensor memory
     if (grid == n_ctas) a.tickets = nullptr;
     void *params[] = {&a};
     return demo_launch_kernel((const void *)kernel, grid, groups * PAIR_THREADS, (size_t)smem, stream, params);
@@ -567,28 +567,28 @@ cudaError_t launch_tc(K kernel, int groups, int smem, A a, int sm_count, cudaStr
 
 bool demo_tc_supported(int s) { return s == S; }
 
-cudaError_t demo_launch_compress_tc(const DemoCompressArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_compress_tc(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     constexpr int FIXED = 8 * BLK + bars_bytes + 1024;  // (last: alignment slack)
     auto pick = [&](auto gt, auto many) {
         using GT = decltype(gt);
         constexpr bool MANY = decltype(many)::value;
-        return a.k > MAX_K_LISTED ? launch_tc(compress_tc_kernel<GT, 3, true, MANY>, 3, FIXED + 6 * chunk_bytes(true), a, sm_count, stream)
-                                  : launch_tc(compress_tc_kernel<GT, 4, false, MANY>, 4, FIXED + 8 * chunk_bytes(false), a, sm_count, stream);
+        return a.k > MAX_K_LISTED ? launch_tc(compress_tc_kernel<GT, 3, true, MANY>, 3, FIXED + 6 * chunk_bytes(true), a, dev, stream)
+                                  : launch_tc(compress_tc_kernel<GT, 4, false, MANY>, 4, FIXED + 8 * chunk_bytes(false), a, dev, stream);
     };
     if (a.n_entries > MANY_TENSORS)
         return a.grad_bf16 ? pick(__nv_bfloat16{}, std::true_type{}) : pick(float{}, std::true_type{});
     return a.grad_bf16 ? pick(__nv_bfloat16{}, std::false_type{}) : pick(float{}, std::false_type{});
 }
 
-cudaError_t demo_launch_decode_tc(const DemoDecodeArgs &a, int sm_count, cudaStream_t stream)
+cudaError_t demo_launch_decode_tc(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     constexpr int FIXED = 4 * BLK + bars_bytes + 1024;
     auto pick = [&](auto many) {
         constexpr bool MANY = decltype(many)::value;
         if (a.agg == 2)  // the sender counts leave room for three groups
-            return launch_tc(decode_tc_kernel<3, MANY>, 3, FIXED + 6 * (X_BYTES + M * 2), a, sm_count, stream);
-        return launch_tc(decode_tc_kernel<4, MANY>, 4, FIXED + 8 * X_BYTES, a, sm_count, stream);
+            return launch_tc(decode_tc_kernel<3, MANY>, 3, FIXED + 6 * (X_BYTES + M * 2), a, dev, stream);
+        return launch_tc(decode_tc_kernel<4, MANY>, 4, FIXED + 8 * X_BYTES, a, dev, stream);
     };
     return a.n_entries > MANY_TENSORS ? pick(std::true_type{}) : pick(std::false_type{});
 }

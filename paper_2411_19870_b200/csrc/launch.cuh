@@ -1,4 +1,4 @@
-// Launching: the resident-CTA count and the shared-memory limit of a kernel are asked for once per device, and consecutive
+// Launching: the resident-CTA count and the shared-memory limit of a kernel are asked for once per demo_ctx, and consecutive
 // kernels of this library overlap one kernel's launch with the end of the one before (programmatic dependent launch).
 //
 // Device side.  A kernel launched with demo_launch_kernel may be resident before the previous work of its stream has
@@ -16,6 +16,8 @@
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <mutex>
 
 struct StreamOrder {
     const int wait_first;
@@ -52,10 +54,24 @@ __device__ __forceinline__ void ticket_finish(DemoTickets *t, unsigned parties =
     if (t && atomicInc(&t->done, last) == last) atomicExch(&t->next, 0u);
 }
 
-// Host side.  Raises the kernel's dynamic shared-memory limit to `smem` and returns how many CTAs of `threads` threads fit
-// an SM (at least 1); both are looked up once per device, kernel and size.
-cudaError_t demo_resident_ctas(const void *kernel, int threads, size_t smem, int *per_sm);
+// Host side.  What launches on a device need: its SM count, and what is known about kernels launched before.  One per demo_ctx: the
+// limits set on a kernel belong to the CUDA context, so they must not outlive it or serve another one.  Calls of several threads may
+// share it.
+struct DemoLaunch {
+    struct Known {
+        const void *kernel;
+        int threads;  // 0: the kernel's shared-memory limit is set
+        size_t smem;
+        int per_sm;
+    };
+    int sm_count = 0;
+    std::mutex mutex;
+    Known known[64];  // kernels x sizes; a full table only means asking again
+    int n_known = 0;
+};
+// Raises the kernel's dynamic shared-memory limit to what the device has and returns how many CTAs of `threads` threads fit an SM (at least 1).
+cudaError_t demo_resident_ctas(DemoLaunch &dev, const void *kernel, int threads, size_t smem, int *per_sm);
 // The limit alone, for kernels whose residency is computed by hand.
-cudaError_t demo_allow_smem(const void *kernel, size_t smem);
+cudaError_t demo_allow_smem(DemoLaunch &dev, const void *kernel);
 // Launch of a kernel with a StreamOrder.
 cudaError_t demo_launch_kernel(const void *kernel, long long grid, int threads, size_t smem, cudaStream_t stream, void **params);

@@ -1,5 +1,9 @@
 """Calls of one context on several streams: compress calls of different workers side by side, and whole steps on streams that the
 caller orders by events.  Every run is compared bit for bit with the same calls one after the other."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -103,3 +107,60 @@ def test_queued_steps_equal_steps_waited_for(name):
             if wait:
                 torch.cuda.synchronize()
     assert same(ref, run)
+
+
+RESET = """
+import ctypes, glob, sys
+from paper_2411_19870_b200 import binding
+
+rt = ctypes.CDLL(glob.glob(sys.prefix + "/lib/python3*/site-packages/nvidia/cuda_runtime/lib/libcudart.so*")[0])
+lib = binding.load_library()
+
+
+def compress():
+    ctx, bufs = ctypes.c_void_p(), []
+    desc = (binding.DemoTensorDesc * 1)()
+    desc[0].ndim, desc[0].shape[0], desc[0].shape[1] = 2, 256, 256
+    assert lib.demo_init(ctypes.byref(ctx), ctypes.byref(binding.DemoConfig(0.9, 128, 32, 1e-3, 0.1, 1, 0)), desc, 1, 0) == 0
+    for n in (4 * 256 * 256, 4 * 256 * 256, lib.demo_payload_bytes(ctx)):
+        p = ctypes.c_void_p()
+        assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(n)) == 0 and rt.cudaMemset(p, 0, ctypes.c_size_t(n)) == 0
+        bufs.append(p)
+    one = lambda p: (ctypes.c_void_p * 1)(p.value)
+    status = lib.demo_compress(ctx, 0, one(bufs[0]), one(bufs[1]), bufs[2], None), lib.demo_device_status(ctx, None)
+    lib.demo_free(ctx)
+    for p in bufs:
+        rt.cudaFree(p)
+    return status
+
+
+assert compress() == (0, 0)
+assert rt.cudaDeviceReset() == 0
+assert compress() == (0, 0)
+print("both")
+"""
+
+
+def test_a_context_made_after_the_process_reset_its_cuda_context():
+    """The limit on a kernel's shared memory goes with the CUDA context of the process: it is set again after cudaDeviceReset (in a process
+    of its own: torch's memory would go too)."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.stdout.split() == ["both"], r.stdout + r.stderr
+
+
+def test_contexts_of_different_sizes_do_not_lower_each_other_s_limits():
+    """The same N-D kernels with much and with little shared memory, by turns."""
+    made = []
+    for chunk in ((128, 64), (16, 32), (64, 127), (8, 128)):
+        shape = tuple(2 * c for c in chunk)
+        tr = demo.DemoTransform([shape], chunk_shapes=[chunk], topk=32, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=1)
+        m, x = torch.zeros(shape, device="cuda"), torch.zeros(shape, device="cuda")
+        made.append((tr, [torch.ones(shape, device="cuda").bfloat16()], [m], [x], torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda")))
+    for _ in range(2):
+        for tr, g, m, x, p in made:
+            tr.compress(0, g, m, p)
+            tr.decode_apply([p], x)
+            assert tr.device_status() == 0
+    for tr, *_ in made:
+        tr.close()
