@@ -29,6 +29,12 @@ FAMILIES = [
     ("generic_s64", 64, 32, torch.bfloat16, "generic", False, None),
     ("generic_s8_f32", 8, 4, torch.float32, None, False, None),
     ("tensor_core_s64", 64, 32, torch.bfloat16, None, True, None),
+    ("generic_path_s8", 8, 4, torch.float32, "generic", False, None),
+    ("small_tiles_s16", 16, 20, torch.bfloat16, None, False, None),
+    ("fast_s128_f32_k_above_s", 128, 130, torch.float32, None, False, None),
+    ("tensor_core_s64_k_above_list", 64, 100, torch.float32, None, True, None),
+    ("nd_numbered", 0, 400, torch.float32, None, False, [(32, 64), (64, 32), (64,), (128,)]),
+    ("nd_long_lists", 0, 600, torch.bfloat16, None, False, [(32, 64), (64, 32), (64,), (128,)]),
     ("nd_rectangular", 0, 16, torch.bfloat16, None, False, [(32, 64), (64, 32), (64,), (128,)]),
 ]
 

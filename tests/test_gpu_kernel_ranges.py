@@ -4,6 +4,7 @@ import ctypes
 import math
 import types
 
+import numpy as np
 import pytest
 import torch
 
@@ -97,7 +98,7 @@ def test_tensor_core_pairs(k, agg):
     ([(64, 32, 7, 7), (32,)], [(32, 4, 7, 7), (32,)], 40),         # kernel windows of 7 x 7; a lossless vector
     ([(32, 16, 2, 2), (24, 4, 6, 6)], [(16, 16, 2, 2), (8, 4, 6, 6)], 17),
     ([(32, 48, 3)], [(32, 48, 1)], 33),                            # 1536 rows of one element: no row table
-    ([(128, 64), (64, 384)], [(64, 32), (32, 128)], 64),           # two threads per line; two classes in one context
+    ([(128, 64), (64, 384)], [(64, 32), (32, 128)], 64),           # two threads per line; ten chunks in one class with extents of 128
     ([(58, 128), (62, 93)], [(29, 64), (31, 31)], 32),             # odd dense extents, one and two lines per thread
     ([(127, 127)], [(127, 127)], 300),                             # the largest dense chunk: both tiles and B fill the SM
     ([(64, 96)], [(16, 32)], 400),                                 # k close to the chunk: the list overflows
@@ -339,3 +340,91 @@ def test_nd_numbered_records(k):
     for _ in range(2):
         r.step()
     r.close()
+
+
+@pytest.mark.parametrize("shapes,chunks,classes,agg", [
+    # one class, 4900 chunks, a CTA takes several and changes between one dense axis (the tiles change places) and two
+    ([(60 * 13, 40 * 32), (50 * 9, 50 * 40)], [(13, 32), (9, 40)], 1, 0),
+    ([(60 * 13, 40 * 32), (50 * 9, 50 * 40)], [(13, 32), (9, 40)], 1, 2),
+    # a class of 2400 chunks and one of 400 beside it
+    ([(60 * 13, 40 * 32), (160, 640, 3, 3)], [(13, 32), (16, 16, 3, 3)], 2, 2),
+])
+def test_nd_many_chunks_and_classes(shapes, chunks, classes, agg):
+    """Chunks on demand, changes of layout inside a CTA and classes side by side, every chunk against the oracle; the signs handed out and
+    applied leave the parameters of decode_apply."""
+    r = parity.NdRunner(shapes, chunks, topk=12, num_workers=2, grad_std=0.02, agg=agg)
+    for _ in range(2):
+        n = r.tr.launch_count
+        x = [p.clone() for p in r.params]
+        r.step()
+        assert r.tr.launch_count - n == classes * (r.W + 1)
+        signs = [torch.zeros(s, dtype=torch.int8, device="cuda") for s in r.shapes]
+        r.tr.decode_signs(r.payloads, signs)
+        r.tr.apply_signs(signs, x)
+        assert all(torch.equal(a, b) for a, b in zip(x, r.params))
+    r.close()
+
+
+@pytest.mark.parametrize("shapes,s,k", [([(20001 * 8,), (19321 * 8,)], 8, 3), ([(2501 * 64,)], 64, 9), ([(1301 * 128,)], 128, 17),
+                                        ([(139 * 8, 139 * 8)], 8, 5), ([(99 * 16, 97 * 16), (5000 * 16,)], 16, 7)])
+def test_small_chunks_beyond_one_round(shapes, s, k):
+    """More segments and tiles than the grid takes in one round, the last round and the last warp partly filled."""
+    wl = inputs.Workload("small", shapes, chunk=s, topk=k, num_workers=2, grad_kind="student_t_ties")
+    r = parity.Runner(wl, max_chunks=400, seed=s)
+    for _ in range(2):
+        r.step()
+    # (the sample holds the last chunk; the energy identity covers all of them)
+    r.step(invariants=True)
+    r.close()
+
+
+def steps_with(shapes, chunk, k, f32, basis, domain, bad):
+    import paper_2411_19870_b200 as demo
+
+    kw = dict(chunk=chunk) if isinstance(chunk, int) else dict(chunk_shapes=chunk)
+    tr = demo.DemoTransform(shapes, topk=k, beta=0.9, lr=1e-3, weight_decay=0.1, num_workers=2,
+                            grad_dtype=demo.DEMO_F32 if f32 else demo.DEMO_BF16, **kw)
+    if basis:
+        tr.set_basis(torch.linalg.qr(torch.randn(64, 64, dtype=torch.float64, generator=torch.Generator().manual_seed(2)))[0].float())
+    if domain:
+        tr.set_momentum_domain(demo.DEMO_MOMENTUM_DCT)
+    gen = torch.Generator("cuda").manual_seed(9)
+    m = [[torch.zeros(s, device="cuda") for s in shapes] for _ in range(2)]
+    x = [torch.randn(s, device="cuda", generator=gen) for s in shapes]
+    p = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    for step in range(2):
+        for w in range(2):
+            g = [torch.randn(s, device="cuda", generator=gen) for s in shapes]
+            if bad and step == 0:
+                flat = g[0].view(-1)
+                flat[3], flat[flat.numel() // 2], flat[-2] = float("nan"), float("inf"), float("-inf")
+            tr.compress(w, [v if f32 else v.bfloat16() for v in g], m[w], p[w])
+        tr.decode_apply(p, x)
+    assert tr.device_status() == 0
+    layout = [tr.payload_layout(t) for t in range(len(shapes))]
+    tr.close()
+    return m, x, p, layout
+
+
+@pytest.mark.parametrize("chunk,k,f32,basis,domain", [
+    (8, 20, True, False, False), (16, 5, False, False, False), (16, 100, True, False, False), (32, 20, True, False, False),
+    (32, 40, False, False, False), (64, 64, False, False, False), (64, 200, True, False, False), (64, 64, True, False, True), (128, 130, True, False, False),
+    (128, 300, False, False, False), (64, 32, False, True, False), (64, 60, True, True, False),
+    ([(12, 29), (7, 3, 3)], 20, True, False, False), ([(12, 29), (7, 3, 3)], 100, False, False, False), ([(32, 64), (16, 4, 4)], 600, True, False, False),
+])
+def test_non_finite_gradients_per_variant(chunk, k, f32, basis, domain):
+    """NaN and infinities in the first tensor, in every variant of the selection: records still distinct, ascending and in range, the
+    second tensor the same bits as without them."""
+    square = isinstance(chunk, int)
+    shapes = [(4 * chunk, 3 * chunk), (2 * chunk, 2 * chunk)] if square else [tuple(3 * c for c in ch) for ch in chunk]
+    per = [chunk * chunk] * 2 if square else [math.prod(c) for c in chunk]
+    clean = steps_with(shapes, chunk, k, f32, basis, domain, False)
+    dirty = steps_with(shapes, chunk, k, f32, basis, domain, True)
+    assert torch.equal(clean[1][1], dirty[1][1])
+    for w in range(2):
+        assert torch.equal(clean[0][w][1], dirty[0][w][1])
+        rec = dirty[2][w].view(torch.int32).view(-1, 2)[:, 0].cpu().numpy()
+        for (first, n, k_eff), elems in zip(dirty[3], per):
+            idx = rec[first:first + n * k_eff].reshape(n, k_eff)
+            assert idx.min() >= 0 and idx.max() < elems
+            assert k_eff == 1 or np.all(np.diff(idx, axis=1) > 0)
