@@ -64,9 +64,8 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, int x, int y, uin
                  : "memory");
 }
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// Waits (the issuing thread's own bulk groups; completes by itself): source read out / fully done.
+// Waits until the issuing thread's own bulk groups have read their source (completes by itself).
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // The tensor maps live in global memory and are rewritten by the host (a stream-ordered copy) when the
 // caller's buffers change: the thread that is about to use one acquires it for the tensor-map proxy first.
 __device__ __forceinline__ void tmap_acquire(const void *tmap)

@@ -139,52 +139,8 @@ FDCT_HD void dct4(const float (&v)[N], float (&V)[N])
     }
 }
 
-// x[n] = sum_k w_k X[k] cos(pi (2n+1) k / (2N)),  w_0 = 1, w_k = SC   (transpose of dct2)
-template <int N, class SC>
-FDCT_HD void dct3(const float (&X)[N], float (&x)[N])
-{
-    if constexpr (N == 1) {
-        x[0] = X[0];
-    } else {
-        constexpr int H = N / 2;
-        float Xe[H], Xo[H], e[H], o[H];
-        static_for<0, H>([&](auto i) {
-            constexpr int j = decltype(i)::value;
-            Xe[j] = X[2 * j];
-            Xo[j] = X[2 * j + 1];
-        });
-        dct3<H, SC>(Xe, e);
-        dct4<H, SC>(Xo, o);
-        static_for<0, H>([&](auto i) {
-            constexpr int n = decltype(i)::value;
-            x[n] = e[n] + o[n];
-            x[N - 1 - n] = e[n] - o[n];
-        });
-    }
-}
-
-// Orthonormal DCT-II of x (in place): X[k] = a_k sum_n x[n] cos(pi (2n+1) k / (2N)).
-template <int N>
-FDCT_HD void dct2_ortho(float (&x)[N])
-{
-    float X[N];
-    dct2<N, ScaleOrtho<N>>(x, X);
-    X[0] *= dc_scale<N>();
-    static_for<0, N>([&](auto i) { x[decltype(i)::value] = X[decltype(i)::value]; });
-}
-
-// Inverse of dct2_ortho (orthonormal DCT-III), in place.
-template <int N>
-FDCT_HD void dct3_ortho(float (&X)[N])
-{
-    float x[N];
-    X[0] *= dc_scale<N>();
-    dct3<N, ScaleOrtho<N>>(X, x);
-    static_for<0, N>([&](auto i) { X[decltype(i)::value] = x[decltype(i)::value]; });
-}
-
 // ------------------------------------------------------------------------------------------------
-// The same two transforms split so that the forward and the inverse share ONE copy of their
+// DCT-II and DCT-III split so that the forward and the inverse share ONE copy of their
 // multiplications.  DCT-II_N is a cascade of butterflies (sums go down, differences are the inputs of
 // DCT-IV_{N/2}, DCT-IV_{N/4}, ..., DCT-IV_1) and DCT-III_N is the same DCT-IV blocks followed by the
 // transposed cascade, so both are  [butterflies] o core  /  core o [butterflies]  with
@@ -200,77 +156,6 @@ constexpr int core_index(int p)
     while (2 * h <= p) h *= 2;
     return (N / h) * (p - h) + N / (2 * h);
 }
-// inverse map: position of coefficient v
-template <int N>
-constexpr int core_pos(int v)
-{
-    for (int p = 0; p < N; ++p)
-        if (core_index<N>(p) == v) return p;
-    return -1;
-}
-
-template <int H, int N, class SC>
-FDCT_HD void core_blocks(const float (&w)[N], float (&y)[N])
-{
-    float v[H], V[H];
-    static_for<0, H>([&](auto i) { v[decltype(i)::value] = w[H + decltype(i)::value]; });
-    dct4<H, SC>(v, V);
-    static_for<0, H>([&](auto i) { y[H + decltype(i)::value] = V[decltype(i)::value]; });
-    if constexpr (H > 1) core_blocks<H / 2, N, SC>(w, y);
-}
-template <int N>
-FDCT_HD void dct_core_ortho(const float (&w)[N], float (&y)[N])
-{
-    y[0] = w[0] * dc_scale<N>();
-    core_blocks<N / 2, N, ScaleOrtho<N>>(w, y);
-}
-
-// Forward butterflies: natural-order input x -> core input w.
-template <int L, int N>
-FDCT_HD void fwd_cascade(const float (&u)[L], float (&w)[N])
-{
-    if constexpr (L == 1) {
-        w[0] = u[0];
-    } else {
-        constexpr int H = L / 2;
-        float s[H];
-        static_for<0, H>([&](auto i) {
-            constexpr int n = decltype(i)::value;
-            s[n] = u[n] + u[L - 1 - n];
-            w[H + n] = u[n] - u[L - 1 - n];
-        });
-        fwd_cascade<H, N>(s, w);
-    }
-}
-template <int N>
-FDCT_HD void dct2_pre(const float (&x)[N], float (&w)[N])
-{
-    fwd_cascade<N, N>(x, w);
-}
-
-// Inverse butterflies: core output y -> natural-order output x.
-template <int H, int N>
-FDCT_HD void inv_cascade(const float (&e)[H], const float (&y)[N], float (&x)[N])
-{
-    if constexpr (H == N) {
-        static_for<0, N>([&](auto i) { x[decltype(i)::value] = e[decltype(i)::value]; });
-    } else {
-        float f[2 * H];
-        static_for<0, H>([&](auto i) {
-            constexpr int n = decltype(i)::value;
-            f[n] = e[n] + y[H + n];
-            f[2 * H - 1 - n] = e[n] - y[H + n];
-        });
-        inv_cascade<2 * H, N>(f, y, x);
-    }
-}
-template <int N>
-FDCT_HD void dct3_post(const float (&y)[N], float (&x)[N])
-{
-    float e[1] = {y[0]};
-    inv_cascade<1, N>(e, y, x);
-}
-
 // ------------------------------------------------------------------------------------------------
 // Two floats per operation.  sm_100 adds packed fp32 arithmetic (add / sub on a register pair, one issue
 // slot for two results, each result rounded exactly like the scalar operation).  A kernel whose limit is
@@ -470,7 +355,7 @@ FDCT_HD void core_blocks_paired(const float (&w)[N], float (&y)[N])
     static_for<0, H>([&](auto i) { y[H + decltype(i)::value] = V[decltype(i)::value]; });
     if constexpr (H > 1) core_blocks_paired<H / 2, N, SC>(w, y);
 }
-// dct_core_ortho with packed arithmetic (same results).
+// The core of the orthonormal transforms.
 template <int N>
 FDCT_HD void dct_core_ortho_paired(const float (&w)[N], float (&y)[N])
 {
@@ -537,8 +422,7 @@ FDCT_HD void dct3_post_paired(const float (&y)[N], float (&x)[N])
     const F2 e[1] = {f2_make(y[0] + y[1], y[0] - y[1])};
     inv_cascade_paired<2, N>(e, y, x);
 }
-// dct2<N, SC> / dct3<N, SC> (any output scale SC, DC term unscaled) through the packed cascades and blocks: same
-// results, about a third fewer instructions.
+// DCT-II and DCT-III with any output scale SC (DC term unscaled) through the packed cascades and blocks.
 template <int N, class SC>
 FDCT_HD void dct2_packed(const float (&x)[N], float (&X)[N])
 {

@@ -293,7 +293,6 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             }
             {
                 // inverse transform: the DCT-IV blocks and the butterfly cascade with two sums per instruction
-                // (same results as the scalar form)
                 float w[S], y[S];
                 fdct::static_for<0, S>([&](auto i) { w[decltype(i)::value] = r[fdct::core_index<S>(decltype(i)::value)]; });
                 fdct::dct_core_ortho_paired<S>(w, y);
