@@ -377,4 +377,59 @@ struct DecodeWalk {
     }
 };
 
+// Adds the workers' records of a chunk straight from the payloads: THREADS threads, thread t takes the records t, t + THREADS, ...
+// of a worker, a barrier behind every worker keeps the order of the additions (indices are unique inside one worker's chunk).
+// Eight rounds of THREADS records are fetched together, of whichever workers come next.  add(record) for each; barrier() is the block's.
+// ONE: k <= THREADS, a single round per worker.
+template <int THREADS, bool ONE, class Add, class Barrier>
+__device__ __forceinline__ void add_from_payloads(const DemoRecord *const *payloads, int n_workers, long long first_rec, int k, int t,
+                                                  Add add, Barrier barrier)
+{
+    if constexpr (ONE) {
+        const bool mine = t < k;
+        for (int w0 = 0; w0 < n_workers; w0 += 8) {
+            DemoRecord r[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (mine && w0 + u < n_workers) r[u] = payloads[w0 + u][first_rec + t];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (w0 + u < n_workers) {
+                    if (mine) add(r[u]);
+                    barrier();
+                }
+        }
+    } else {
+        struct Place {  // of a round
+            int w, kb;
+            __device__ __forceinline__ void next(int k)
+            {
+                kb += THREADS;
+                if (kb >= k) {
+                    kb = 0;
+                    ++w;
+                }
+            }
+        };
+        Place p{0, 0};
+        while (p.w < n_workers) {
+            DemoRecord r[8];
+            Place f = p;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (f.w < n_workers && f.kb + t < k) r[u] = payloads[f.w][first_rec + f.kb + t];
+                f.next(k);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (p.w < n_workers) {
+                    if (p.kb + t < k) add(r[u]);
+                    if (p.kb + THREADS >= k) barrier();
+                }
+                p.next(k);
+            }
+        }
+    }
+}
+
 }  // namespace fastk

@@ -224,33 +224,18 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 if (bad) atomicMax(a.status, DEMO_DEV_PAYLOAD);
             }
         } else {
-            // A thread's records may fall into any row; a barrier per worker fixes the order of additions.
-            // Records are fetched eight workers ahead so that one memory latency covers eight workers.
-            const long long rec_off = walk.rec[which];
-            sb.sync();
-            for (int kb = 0; kb < k_eff; kb += S) {
-                const bool mine = kb + t < k_eff;
-                for (int w0 = 0; w0 < a.W; w0 += 8) {
-                    DemoRecord r[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (mine && w0 + j < a.W) r[j] = a.payloads[w0 + j][rec_off + kb + t];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (w0 + j < a.W) {
-                            if (mine) {
-                                if ((unsigned)r[j].idx < (unsigned)M) {
-                                    St[(r[j].idx >> C::LOG2S) * XS + (r[j].idx & (S - 1))] += r[j].val;
-                                    if (counts) Cn[r[j].idx] += 1;
-                                } else {
-                                    atomicMax(a.status, DEMO_DEV_PAYLOAD);
-                                }
-                            }
-                            sb.sync();
-                        }
+            sb.sync();  // the tile is cleared
+            add_from_payloads<S, false>(
+                a.payloads, a.W, walk.rec[which], k_eff, t,
+                [&](const DemoRecord &rc) {
+                    if ((unsigned)rc.idx < (unsigned)M) {
+                        St[(rc.idx >> C::LOG2S) * XS + (rc.idx & (S - 1))] += rc.val;
+                        if (counts) Cn[rc.idx] += 1;
+                    } else {
+                        atomicMax(a.status, DEMO_DEV_PAYLOAD);
                     }
-                }
-            }
+                },
+                [&] { sb.sync(); });
         }
         if (threadIdx.x == 0) drawn[par ^ 1u] = ticket;
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0 (row t is this thread's)

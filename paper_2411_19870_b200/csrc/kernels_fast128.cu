@@ -629,10 +629,12 @@ constexpr size_t DECODE128_SMEM = (size_t)S * XSD * 4 + 128 + 2 * STAGE_RECORDS 
 
 // SIGNS: the parameter-server form -- sign(R) goes out as int8, the parameters are not touched.
 // STAGED: records are staged a chunk ahead and every warp adds those of its 16 rows, worker after worker; otherwise they
-// come straight from the payloads with a barrier per worker.
+// come straight from the payloads with a barrier per worker, ROUND for lists that one round of the threads covers, ROUNDS for longer
+// ones (in one instantiation the loop of the longer lists cost signs 4 %).
 // The upper half of the x tile comes in behind the scatter and the transforms, the lower half, already in L2, into the dead
 // coefficient tile while the upper one is updated; by 16-byte asynchronous copies, without tensor maps (kernels_fast.cu).
-template <bool SIGNS, bool STAGED>
+enum { STAGED, ROUND, ROUNDS };
+template <bool SIGNS, int KMODE>
 __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -678,7 +680,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         }
     }
     __syncthreads();
-    if (STAGED && c < n_chunks) stage_batch(0, 0, 0);
+    if (KMODE == STAGED && c < n_chunks) stage_batch(0, 0, 0);
     for (unsigned nc; c < n_chunks; c = nc, par ^= 1u, which ^= 1) {
         __syncthreads();  // (publishes the draw; the tile and the landing area are free)
         nc = gridDim.x + drawn[par];
@@ -707,7 +709,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         if (counts)
             for (int i = tid; i < M / 2; i += THREADS) reinterpret_cast<unsigned *>(Cn)[i] = 0u;
         // S = sum over workers in worker order (Decompress&Aggregate)
-        if constexpr (STAGED) {
+        if constexpr (KMODE == STAGED) {
             const int sh = stage_shift(k_eff), wb = STAGE_RECORDS >> sh;
             for (int w0 = 0; w0 < a.W; w0 += wb) {
                 // the records have landed (requested a chunk or a batch ago; only the rows of x are younger), the tile is cleared,
@@ -749,31 +751,18 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                 if (bad) atomicMax(a.status, DEMO_DEV_PAYLOAD);
             }
         } else {
-            const long long rec_off = walk.rec[which];
             __syncthreads();
-            for (int kb = 0; kb < k_eff; kb += THREADS) {
-                const bool mine = kb + tid < k_eff;
-                for (int w0 = 0; w0 < a.W; w0 += 8) {  // fetched eight workers ahead
-                    DemoRecord r[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (mine && w0 + q < a.W) r[q] = a.payloads[w0 + q][rec_off + kb + tid];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        if (w0 + q < a.W) {
-                            if (mine) {
-                                if ((unsigned)r[q].idx < (unsigned)M) {
-                                    St[(r[q].idx >> 7) * XSD + (r[q].idx & 127)] += r[q].val;
-                                    if (counts) Cn[r[q].idx] += 1;
-                                } else {
-                                    atomicMax(a.status, DEMO_DEV_PAYLOAD);
-                                }
-                            }
-                            __syncthreads();
-                        }
+            add_from_payloads<THREADS, KMODE == ROUND>(
+                a.payloads, a.W, walk.rec[which], k_eff, tid,
+                [&](const DemoRecord &rc) {
+                    if ((unsigned)rc.idx < (unsigned)M) {
+                        St[(rc.idx >> 7) * XSD + (rc.idx & 127)] += rc.val;
+                        if (counts) Cn[rc.idx] += 1;
+                    } else {
+                        atomicMax(a.status, DEMO_DEV_PAYLOAD);
                     }
-                }
-            }
+                },
+                [] { __syncthreads(); });
         }
         if (tid == 0) drawn[par ^ 1u] = ticket;
         __syncthreads();
@@ -889,8 +878,9 @@ cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev,
     const bool staged = a.k <= 64 || (a.k <= STAGE_RECORDS && (long long)a.W << stage_shift(a.k) <= STAGE_RECORDS);
     auto pick = [&](auto signs) {
         constexpr bool SIGNS = decltype(signs)::value;
-        return staged ? launch128(decode_fast128_kernel<SIGNS, true>, DECODE128_SMEM, dev, stream, a)
-                      : launch128(decode_fast128_kernel<SIGNS, false>, DECODE128_SMEM, dev, stream, a);
+        if (staged) return launch128(decode_fast128_kernel<SIGNS, STAGED>, DECODE128_SMEM, dev, stream, a);
+        if (a.k <= THREADS) return launch128(decode_fast128_kernel<SIGNS, ROUND>, DECODE128_SMEM, dev, stream, a);
+        return launch128(decode_fast128_kernel<SIGNS, ROUNDS>, DECODE128_SMEM, dev, stream, a);
     };
     return a.sign_ptrs ? pick(std::true_type{}) : pick(std::false_type{});
 }

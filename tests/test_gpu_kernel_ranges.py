@@ -428,3 +428,35 @@ def test_non_finite_gradients_per_variant(chunk, k, f32, basis, domain):
             idx = rec[first:first + n * k_eff].reshape(n, k_eff)
             assert idx.min() >= 0 and idx.max() < elems
             assert k_eff == 1 or np.all(np.diff(idx, axis=1) > 0)
+
+
+@pytest.mark.parametrize("s", [8, 16, 32, 64, 128])
+@pytest.mark.parametrize("k", [1, 40, 64, 65, 128, 129, 200, 256, 257, 512, 513])
+def test_decode_adds_in_the_order_of_the_workers(s, k):
+    """2^25 + 1 - 2^25 is 0 in fp32 in this order and 1 or 0 in others: three workers send these values for one coordinate that stands
+    first in the lists of workers 0 and 2 and last in worker 1's, all other values are zero.  The signs and the update agree."""
+    import paper_2411_19870_b200 as demo
+
+    M = s * s
+    if k > M // 4:
+        pytest.skip("the lists need room on both sides of the coordinate")
+    lr = 2.0 ** -3
+    tr = demo.DemoTransform([(2 * s, s)], chunk=s, topk=k, beta=0.9, lr=lr, weight_decay=0.0, num_workers=3)
+    at = M // 2
+    pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    for w, (value, first) in enumerate(((2.0 ** 25, True), (1.0, False), (-2.0 ** 25, True))):
+        idx = torch.arange(k) + (at if first else at - k + 1)
+        rec = pay[w].view(torch.int32).view(2, k, 2)
+        rec[:, :, 0] = idx.int().cuda()
+        pay[w].view(torch.float32).view(2, k, 2)[:, 0 if first else k - 1, 1] = value
+    signs = [torch.ones(2 * s, s, dtype=torch.int8, device="cuda")]
+    tr.decode_signs(pay, signs)
+    assert int(signs[0].abs().sum()) == 0
+    x = [torch.randn(2 * s, s, device="cuda")]
+    before = x[0].clone()
+    tr.decode_apply(pay, x)
+    assert torch.equal(x[0], before)
+    tr.set_decode_mode(demo.DEMO_AGG_SUM, demo.DEMO_PHI_IDENTITY)
+    tr.decode_apply(pay, x)
+    assert torch.equal(x[0], before)
+    tr.close()
