@@ -40,11 +40,12 @@ static_assert(sizeof(DecodeWalk) <= 128, "reserved in decode_slot_bytes");
 // CTA that comes to a tensor, a fence that stands in front of the chunk (300M-class set, 168 matrices: 696 us with maps, 725
 // with a bulk copy per row, 624 like this; one matrix of that size: 612, 731, 597).
 // How the records are added up, by k.  (One instantiation each: the loops of the larger k in the same kernel cost 8 us of the
-// 96 of 8192 x 8192, k = 32.)
-//   LISTED: up to 64 records per worker, staged; STAGED: up to 512, staged, in parts of 64; BARRIERS: straight from the
-//   payloads, a barrier per worker.  4096 x 4096, k = 128, STAGED instead of BARRIERS: s = 32, W = 2 55.0 -> 40.5 us, signs
-//   39.7 -> 35.1; s = 64, W = 8 / 64 47.9 / 160 -> 42.9 / 137 us, k = 200, W = 2 44.0 -> 34.1, but signs at s = 64, W = 8
-//   31.8 -> 36.9.
+// 96 of 8192 x 8192, k = 32.)  In all of them a coordinate gets its workers' values in the order of the workers.
+//   LISTED: up to 64 records per worker, staged; STAGED: up to 512, staged, in parts of 64, unless they are few enough (s = 32,
+//   W k < 256) or only the signs are wanted (s = 64); BARRIERS: straight from the payloads, a barrier per worker.
+// 4096 x 4096, STAGED / BARRIERS: s = 64, k = 96 / 129 / 257 W = 8 41 / 42, 49 / 51, 65 / 69 us, W = 32 80 / 92, 112 / 122, 171 / 182;
+// s = 32, k = 65 W = 1 36 / 34, W = 2 39 / 39, W = 8 60 / 70, k = 129 W = 1 38 / 37, W = 2 44 / 50; signs, s = 64, k = 96 / 128
+// W = 8 36 / 33, k = 200 W = 2 / 8 / 32 29 / 26, 50 / 39, 144 / 138.
 enum { LISTED, STAGED, BARRIERS };
 template <int S, int THREADS, bool SIGNS, int KMODE>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(DemoDecodeArgs a)
@@ -178,22 +179,40 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                     if (counts && mine) Cn[idx] += 1;
                 };
                 if constexpr (KMODE == STAGED) {  // a worker's records in parts of 64, the last one short
-                    const int more_sh = sh - 6;
-                    const int n_parts = nw << more_sh, last = (1 << more_sh) - 1;
-                    DemoRecord rc[4][2];
-#pragma unroll 1
-                    for (int part = 0; part < n_parts; part += 4) {
+                    const int per = (k_eff + 63) >> 6;  // parts of a worker
+                    int at = 0, left = k_eff, wl = 0;   // staging place and remaining records of the next part, its worker
+                    auto some = [&](auto count) {
+                        constexpr int U = decltype(count)::value;
+                        DemoRecord rc[U][2];
+                        int n[U];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {  // (behind the last part: within the buffer, not used)
-                            rc[u][0] = stage[((part + u) << 6 & (STAGE_RECORDS - 1)) + lane];
-                            rc[u][1] = stage[((part + u) << 6 & (STAGE_RECORDS - 1)) + lane + 32];
+                        for (int u = 0; u < U; ++u) {
+                            n[u] = left;
+                            rc[u][0] = stage[at + lane];
+                            rc[u][1] = stage[at + lane + 32];
+                            at += 64;
+                            left -= 64;
+                            if (left <= 0) {
+                                ++wl;
+                                at = wl << sh;
+                                left = k_eff;
+                            }
                         }
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int rest = part + u < n_parts ? k_eff - (((part + u) & last) << 6) : 0;  // records from this part on
-                            add(rc[u][0], lane < rest);
-                            add(rc[u][1], lane + 32 < rest);
+                        for (int u = 0; u < U; ++u) {
+                            add(rc[u][0], lane < n[u]);
+                            add(rc[u][1], lane + 32 < n[u]);
                             __syncwarp();
+                        }
+                    };
+#pragma unroll 1
+                    for (int parts = nw * per; parts > 0;) {
+                        if (parts >= 4) {
+                            some(std::integral_constant<int, 4>{});
+                            parts -= 4;
+                        } else {
+                            some(std::integral_constant<int, 1>{});
+                            --parts;
                         }
                     }
                 } else {
@@ -351,7 +370,7 @@ cudaError_t launch_decode(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t
         constexpr bool SIGNS = decltype(signs)::value;
         if (a.k <= 64) return launch(decode_fast_kernel<S, TH, SIGNS, LISTED>, TH, NCH, smem, dev, stream, a);
         if constexpr (!(SIGNS && S == 64))
-            if (a.k <= STAGE_RECORDS) return launch(decode_fast_kernel<S, TH, SIGNS, STAGED>, TH, NCH, smem, dev, stream, a);
+            if (a.k <= STAGE_RECORDS && (S == 64 || (long long)a.W * a.k >= 256)) return launch(decode_fast_kernel<S, TH, SIGNS, STAGED>, TH, NCH, smem, dev, stream, a);
         return launch(decode_fast_kernel<S, TH, SIGNS, BARRIERS>, TH, NCH, smem, dev, stream, a);
     };
     return a.sign_ptrs != nullptr ? pick(std::true_type{}) : pick(std::false_type{});

@@ -871,11 +871,11 @@ cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, DemoLaunch &
 
 cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
-    // Staged while the additions are short (k <= 64) or all workers' records fit one batch; a further batch of longer lists
+    // Staged while the additions are short (k <= 64), and one worker's up to k = 128 in the update form; a further batch of longer lists
     // comes too late.  8192 x 8192, staged / with barriers: k = 32, W = 1 139 / 149 us, W = 8 145 / 169 us, k = 64, W = 8
-    // 156 / 164, k = 128, W = 1 139 / 149, W = 8 182 / 165 us; 4096 x 4096, k = 32, W = 64 62 / 103 us, k = 128, W = 32
-    // 85 / 75 us.
-    const bool staged = a.k <= 64 || (a.k <= STAGE_RECORDS && (long long)a.W << stage_shift(a.k) <= STAGE_RECORDS);
+    // 156 / 164, k = 128, W = 1 139 / 149, W = 8 182 / 165 us; 4096 x 4096, k = 32, W = 64 62 / 103 us, k = 65 .. 128, W = 1
+    // 37.3 / 38.1, W = 4 42 / 39, signs W = 1 33.2 / 32.5, W = 4 37.4 / 32.7.
+    const bool staged = a.k <= 64 || (a.k <= 128 && a.W == 1 && !a.sign_ptrs);
     auto pick = [&](auto signs) {
         constexpr bool SIGNS = decltype(signs)::value;
         if (staged) return launch128(decode_fast128_kernel<SIGNS, STAGED>, DECODE128_SMEM, dev, stream, a);
