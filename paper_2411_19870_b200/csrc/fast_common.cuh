@@ -151,62 +151,6 @@ struct SlotBarrier {
     }
 };
 
-// ------------------------------------------------------------------------------------------------
-// Exact radix select over the S x S coefficient tile stored at X[u*XS + v] (S threads).  Returns the
-// magnitude key of the k-th largest and how many coefficients equal to it belong to the top-k.
-// ------------------------------------------------------------------------------------------------
-template <int S, int XS>
-__device__ __forceinline__ void radix_select_tile(const float *X, int k_eff, unsigned *hist, unsigned *s_state,
-                                                  unsigned *thr, unsigned *need_eq, int t, SlotBarrier<S> sb)
-{
-    if (t == 0) {
-        s_state[0] = 0u;
-        s_state[1] = (unsigned)k_eff;
-    }
-#pragma unroll 1
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 24 - 8 * pass;
-        const unsigned mask = (pass == 0) ? 0u : (0xffffffffu << (shift + 8));
-        for (int i = t; i < 256; i += S) hist[i] = 0u;
-        sb.sync();
-        const unsigned prefix = s_state[0];
-#pragma unroll 1
-        for (int v = 0; v < S; ++v) {
-            const unsigned key = mag_key(X[t * XS + v]);
-            if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-        }
-        sb.sync();
-        if (t < 32) {
-            const unsigned rem = s_state[1];
-            unsigned local = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) local += hist[255 - 8 * t - j];
-            unsigned inc = local;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                unsigned n = __shfl_up_sync(0xffffffffu, inc, d);
-                if (t >= d) inc += n;
-            }
-            const unsigned before = inc - local;
-            if (before < rem && rem <= inc) {
-                unsigned cum = before;
-                int b = 255 - 8 * t;
-                for (int j = 0; j < 8; ++j, --b) {
-                    const unsigned h = hist[b];
-                    if (cum + h >= rem) break;
-                    cum += h;
-                }
-                s_state[1] = rem - cum;
-                s_state[0] = prefix | ((unsigned)b << shift);
-            }
-        }
-        sb.sync();
-    }
-    *thr = s_state[0];
-    *need_eq = s_state[1];
-}
-
-
 // 64 / 32 consecutive fp32 columns of this thread's tensor-memory lane.
 __device__ __forceinline__ void tmem_st64(uint32_t taddr, const float (&v)[64])
 {

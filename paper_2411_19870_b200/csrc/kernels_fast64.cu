@@ -115,7 +115,6 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
     sm.cand_idx = reinterpret_cast<int *>(sm.tmax + S);
     sm.cand_val = reinterpret_cast<float *>(sm.cand_idx + CAP + 8);
     sm.cand_key = reinterpret_cast<unsigned *>(sm.cand_val + CAP + 8);
-    sm.hist = reinterpret_cast<unsigned *>(sm.cand_idx);
     sm.recs4 = reinterpret_cast<int4 *>(sm.raw + region_bytes<GT>()) - 65;
     sm.misc = reinterpret_cast<unsigned *>(sm.cand_key + CAP + 8);
     unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(sm.misc + 16);

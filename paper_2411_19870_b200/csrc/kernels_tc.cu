@@ -320,7 +320,6 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
     sm.cand_idx = reinterpret_cast<int *>(sm.tmax + S);
     sm.cand_val = reinterpret_cast<float *>(sm.cand_idx + CAP + 8);
     sm.cand_key = reinterpret_cast<unsigned *>(sm.cand_val + CAP + 8);
-    sm.hist = reinterpret_cast<unsigned *>(sm.cand_idx);
     sm.misc = reinterpret_cast<unsigned *>(sm.cand_key + CAP + 8);
     sm.wkey = sm.misc + 16;  // (BIGK only)
     sm.widx = sm.wkey + WCAP + 4;

@@ -34,7 +34,6 @@ struct SlotMem {
     int *cand_idx;       // [CAP + 8]
     float *cand_val;     // [CAP + 8]
     unsigned *cand_key;  // [CAP + 8]
-    unsigned *hist;      // [256] aliases the candidate arrays
     int4 *recs4;         // [65] kept records, pre-decoded for the row stage; entry 64 is always padding
     unsigned *misc;      // [16]
     unsigned *wkey;      // [WCAP + 4] wide list, behind the tile
@@ -47,61 +46,88 @@ struct SlotMem {
 enum { SELECT_LISTED, SELECT_QDOM, SELECT_DENSE };
 
 // ------------------------------------------------------------------------------------------------
-// Exact 4 x 8-bit radix select over the coefficient tile in X (complete for every thread of the slot), any k: the
-// last resort of both variants below (tied or degenerate chunks, non-finite values, k > 256).
+// Exact selection over the coefficient tile in X (row t complete for thread t), any k: the last resort of both variants below (tied or
+// degenerate chunks, non-finite values, k above the bounds of the lists).  Row t goes into registers; a threshold with exactly k keys
+// at or above it is searched bit by bit from the highest that any key has, one barrier per bit; if the bits run out, equal keys
+// straddle the k-th place and the first ones are kept.  (A radix select over histograms in shared memory, where most keys meet in a few
+// bins: 4096 x 4096, k = 193 / 256 / 512 196 us instead of 119, all-zero tiles 399 instead of 82; 1024 x 1024 under a caller's basis,
+// k = 256 65 instead of 43.)
 // ------------------------------------------------------------------------------------------------
-static __device__ __noinline__ void select_radix(const SlotMem sm, int k_eff, DemoRecord *rec, float alpha, int t, int bar_id, int mode)
+static __device__ __noinline__ void select_search(const SlotMem sm, int k_eff, DemoRecord *rec, float alpha, int t, int bar_id, int mode)
 {
     const SlotBarrier<S> sb{bar_id};
     const int lane = t & 31, warp = t >> 5;
-    float *X = sm.X;
-    unsigned *misc = sm.misc;
-    unsigned thr, need_eq;
-    sb.sync();
-    radix_select_tile<S, XS>(X, k_eff, sm.hist, misc, &thr, &need_eq, t, sb);
-    unsigned gt = 0, eq = 0;
-#pragma unroll 1
-    for (int v = 0; v < S; ++v) {
-        const unsigned key = mag_key(X[t * XS + v]);
-        gt += key > thr;
-        eq += key == thr;
+    float *row = sm.X + t * XS;
+    unsigned *misc = sm.misc;  // [2][2]: the warps' values, by turns
+    float q[S];
+#pragma unroll
+    for (int v4 = 0; v4 < S / 4; ++v4) {
+        const float4 f = reinterpret_cast<const float4 *>(row)[v4];
+        q[4 * v4] = f.x;
+        q[4 * v4 + 1] = f.y;
+        q[4 * v4 + 2] = f.z;
+        q[4 * v4 + 3] = f.w;
     }
-    const unsigned packed = gt | (eq << 16);
-    const unsigned inc = warp_inclusive_scan(packed, lane);
-    sb.sync();  // radix_select_tile's last reads of misc are done
-    if (lane == 31) misc[warp] = inc;
+    sb.sync();  // earlier readers of misc are done
+    int turn = 0;
+    auto both = [&](unsigned v, auto join) {  // v of this warp and of the other
+        if (lane == 0) misc[2 * turn + warp] = v;
+        sb.sync();
+        const unsigned r = join(misc[2 * turn], misc[2 * turn + 1]);
+        turn ^= 1;
+        return r;
+    };
+    auto sum = [](unsigned x, unsigned y) { return x + y; };
+    unsigned top = 0u;
+#pragma unroll
+    for (int v = 0; v < S; ++v) top = max(top, mag_key(q[v]));
+    top = both(__reduce_max_sync(0xffffffffu, top), [](unsigned x, unsigned y) { return max(x, y); });
+    unsigned thr = 0u, n_ge = (unsigned)(S * S);
+#pragma unroll 1
+    for (int b = 31 - __clz(top | 1u); b >= 0 && n_ge != (unsigned)k_eff; --b) {
+        const unsigned cand = thr | (1u << b);
+        unsigned n = 0u;
+#pragma unroll
+        for (int v = 0; v < S; ++v) n += mag_key(q[v]) >= cand;
+        n = both(__reduce_add_sync(0xffffffffu, n), sum);
+        if (n >= (unsigned)k_eff) {
+            thr = cand;
+            n_ge = n;
+        }
+    }
+    // (n_ge = k: all at or above the threshold are kept, whatever lies between equal keys)
+    unsigned gt = 0u, eq = 0u;
+#pragma unroll
+    for (int v = 0; v < S; ++v) {
+        gt += mag_key(q[v]) > thr;
+        eq += mag_key(q[v]) == thr;
+    }
+    const unsigned packed = gt | (eq << 16), inc = warp_inclusive_scan(packed, lane);
+    const unsigned last = __shfl_sync(0xffffffffu, inc, 31);
+    if (lane == 0) misc[2 * turn + warp] = last;
     sb.sync();
-    unsigned before = inc - packed;
-    if (warp == 1) before += misc[0];
+    const unsigned first_warp = misc[2 * turn], need_eq = (unsigned)k_eff - ((first_warp + misc[2 * turn + 1]) & 0xffffu);
+    const unsigned before = inc - packed + (warp ? first_warp : 0u);
     unsigned gb = before & 0xffffu, eb = before >> 16;
 #pragma unroll 1
     for (int v = 0; v < S; ++v) {
-        const float val = X[t * XS + v];
+        const float val = row[v];
         const unsigned key = mag_key(val);
-        bool s = false;
-        unsigned pos = 0;
-        if (key > thr) {
-            pos = gb + min(eb, need_eq);
-            ++gb;
-            s = true;
-        } else if (key == thr) {
-            if (eb < need_eq) {
-                pos = gb + eb;
-                s = true;
-            }
-            ++eb;
-        }
+        const bool s = key > thr || (key == thr && eb < need_eq);
         if (s) {
+            const unsigned pos = gb + min(eb, need_eq);
             DemoRecord r;
             r.idx = t * S + v;
             r.val = val;
             rec[pos] = r;
             if (mode == SELECT_QDOM)
-                X[t * XS + v] = fmaf(-alpha, val, val);
+                row[v] = fmaf(-alpha, val, val);
             else if (mode == SELECT_LISTED)
                 sm.recs4[pos] = make_int4(t * XS, v * S, __float_as_int(alpha * val), 0);
         }
-        if (mode == SELECT_DENSE) X[t * XS + v] = s ? alpha * val : 0.f;
+        if (mode == SELECT_DENSE) row[v] = s ? alpha * val : 0.f;
+        gb += key > thr;
+        eb += key == thr;
     }
 }
 
@@ -115,7 +141,7 @@ static __device__ __noinline__ void select_radix(const SlotMem sm, int k_eff, De
 //      bit-by-bit ballot search;
 //   2. if the list overflows: a tighter bound from the 256 quarter-row and the 256 quarter-column
 //      maxima, then 1. again;
-//   3. otherwise an exact 4 x 8-bit radix select over the whole tile.
+//   3. otherwise select_search over the whole tile.
 // ------------------------------------------------------------------------------------------------
 static __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, DemoRecord *rec, float alpha, int t, int bar_id,
                                          unsigned lmin_w, bool qdom)
@@ -286,7 +312,7 @@ static __device__ __noinline__ void select_slow(const SlotMem sm, int k_eff, Dem
             done = true;
         }
     }
-    if (!done) select_radix(sm, k_eff, rec, alpha, t, bar_id, qdom ? SELECT_QDOM : SELECT_LISTED);
+    if (!done) select_search(sm, k_eff, rec, alpha, t, bar_id, qdom ? SELECT_QDOM : SELECT_LISTED);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -370,8 +396,8 @@ __device__ __forceinline__ void ballot_select(const SlotMem &sm, unsigned n_w0, 
 // Exact top-k of one chunk (Section 2.1 "Top-k Sparsification"): thread t holds the coefficients q[v] = Q[t][v] of
 // row t.  Writes the k_eff records in ascending index order to `rec`; ends before the barrier that makes them
 // visible.  QDOM = false (momentum kept in the spatial domain): also leaves the pre-decoded row-stage list and the
-// tile X cleared for the row stage.  (WIDE = false: no room for the wide list, such chunks go to the radix select.)  QDOM = true (momentum kept in the transform domain): leaves in X the
-// coefficient tile with every transmitted coefficient q replaced by q - alpha q.
+// tile X cleared for the row stage.  (WIDE = false: no room for the wide list, such chunks go to select_search.)  QDOM = true
+// (momentum kept in the transform domain): leaves in X the coefficient tile with every transmitted coefficient q replaced by q - alpha q.
 // ------------------------------------------------------------------------------------------------
 template <bool QDOM, bool WIDE = true>
 __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], int k_eff, DemoRecord *rec, float alpha,
@@ -524,7 +550,7 @@ __device__ __forceinline__ void select_chunk(const SlotMem &sm, float (&q)[S], i
             if constexpr (WIDE)
                 select_slow(sm, k_eff, rec, alpha, t, bar_id, lmin_w, QDOM);
             else
-                select_radix(sm, k_eff, rec, alpha, t, bar_id, QDOM ? SELECT_QDOM : SELECT_LISTED);
+                select_search(sm, k_eff, rec, alpha, t, bar_id, QDOM ? SELECT_QDOM : SELECT_LISTED);
             sb.sync();  // every thread is done with the coefficient tile
             zero_row();
         }
@@ -707,7 +733,7 @@ __device__ __forceinline__ void select_chunk_big(const SlotMem &sm, float (&q)[S
         stash_row();
     }
     if (slow) {
-        select_radix(sm, k_eff, rec, alpha, t, bar_id, QDOM ? SELECT_QDOM : SELECT_DENSE);
+        select_search(sm, k_eff, rec, alpha, t, bar_id, QDOM ? SELECT_QDOM : SELECT_DENSE);
         if (!QDOM) {  // index order -> core order (this thread's row)
             float4 *row = reinterpret_cast<float4 *>(my_row);
 #pragma unroll

@@ -460,3 +460,42 @@ def test_decode_adds_in_the_order_of_the_workers(s, k):
     tr.decode_apply(pay, x)
     assert torch.equal(x[0], before)
     tr.close()
+
+
+@pytest.mark.parametrize("kind", ["normal", "ties", "zero", "one", "full"])
+@pytest.mark.parametrize("k", [193, 255, 1000, 4095, 4096])
+def test_s64_search_of_the_threshold(k, kind):
+    """s = 64 above the bound of the lists: all keys equal, all zero, a single non-zero coefficient, fewer than k of them, everything kept;
+    on DCT and caller-supplied basis, every chunk against the oracle."""
+    for gauss in (None, inputs.basis_gaussian(3, 64).numpy()):
+        wl = inputs.Workload("s64s", [(2 * 64, 3 * 64)], chunk=64, topk=k, num_workers=1, grad_kind="normal", grad_dtype=torch.float32)
+        r = parity.Runner(wl, max_chunks=10**9, seed=k, gauss=gauss)
+        g = r.streams[0].next()
+        # (most of a chunk kept leaves the rounding of both transforms, some 5 * 2^-23 of the largest |B|, as the residual: inputs below
+        # 2^-4 keep it under the absolute tolerance of 1e-7)
+        g[0].mul_(2.0 ** -6 / max(1e-30, float(g[0].abs().max())))
+        if kind == "ties":
+            g[0].copy_(torch.where(g[0] < 0, -(2.0 ** -8), 2.0 ** -8))
+        if kind in ("zero", "one"):
+            g[0].zero_()
+        if kind == "one":
+            g[0][::64, ::64] = 2.0 ** -6
+        if kind == "full":
+            g[0][64:] = 2.0 ** -6
+        r.step(grads=[g])
+        r.close()
+
+
+@pytest.mark.parametrize("basis", [False, True])
+def test_s64_compress_time_above_the_lists(basis):
+    """k = 193 is searched among all coefficients, k = 192 among a list: by a radix select it took 2.7 times as long, on all-zero tiles nine
+    times."""
+    times = {}
+    for k in (192, 193):
+        f = Flat(1, (4096, 4096), 64, k, torch.linalg.qr(torch.randn(64, 64, dtype=torch.float64))[0].float() if basis else None)
+        times[k] = f.device_us("compress")
+        f.g.zero_()
+        f.m.zero_()
+        times[-k] = f.device_us("compress")
+        f.tr.close()
+    assert times[193] <= 2.0 * times[192] and times[-193] <= 2.2 * times[-192], times
