@@ -96,27 +96,13 @@ __device__ __forceinline__ uint32_t op_off(int c, int cb, int r, int q)
     if (MN) return (2 * c + cb) * BLK + r * 128 + ((((q >> 1) ^ (r & 3)) << 5) | ((q & 1) << 4));
     return (2 * c + cb) * BLK + r * 128 + ((q ^ (r & 7)) << 4);
 }
-// Row r of chunk c (64 floats) split into the hi and lo operand tiles.
+// Piece p (four floats) of row r of the basis, split into the hi and lo operand tiles.
 template <bool MN>
-__device__ __forceinline__ void write_split_row(unsigned char *hi, unsigned char *lo, int c, int r, const float *v)
+__device__ __forceinline__ void write_split(unsigned char *hi, unsigned char *lo, int r, int p, const float4 &h, const float4 &l)
 {
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float *p = v + cb * 32 + q * 4;
-            float4 h, l;
-            h.x = tf32_rn(p[0]);
-            h.y = tf32_rn(p[1]);
-            h.z = tf32_rn(p[2]);
-            h.w = tf32_rn(p[3]);
-            l.x = tf32_rn(p[0] - h.x);
-            l.y = tf32_rn(p[1] - h.y);
-            l.z = tf32_rn(p[2] - h.z);
-            l.w = tf32_rn(p[3] - h.w);
-            *reinterpret_cast<float4 *>(hi + op_off<MN>(c, cb, r, q)) = h;
-            *reinterpret_cast<float4 *>(lo + op_off<MN>(c, cb, r, q)) = l;
-        }
+    const uint32_t at = op_off<MN>(0, p >> 3, r, p & 7);
+    *reinterpret_cast<float4 *>(hi + at) = h;
+    *reinterpret_cast<float4 *>(lo + at) = l;
 }
 
 // One product, issued by one thread: D (+)= A * basis part, K = 64 in eight steps of 8 (8 columns of A; 32 bytes inside a
@@ -162,18 +148,14 @@ __device__ __forceinline__ void tc_setup(TcFrame &f, unsigned char *raw, const f
         mbar_init(f.bar, 1);
         fence_proxy_async();
     }
-    if (tid < S) {
-        float v[S];
-#pragma unroll
-        for (int j4 = 0; j4 < S / 4; ++j4) {
-            const float4 p = __ldg(reinterpret_cast<const float4 *>(basis + tid * S) + j4);
-            v[4 * j4] = p.x;
-            v[4 * j4 + 1] = p.y;
-            v[4 * j4 + 2] = p.z;
-            v[4 * j4 + 3] = p.w;
-        }
-        if (need_k_major) write_split_row<false>(f.sm + OFF_BK_HI, f.sm + OFF_BK_LO, 0, tid, v);
-        write_split_row<true>(f.sm + OFF_BM_HI, f.sm + OFF_BM_LO, 0, tid, v);
+    // (all threads: by 64 of them, a row each, decode of 1024 x 1024 takes 18.3 us instead of 17.9)
+    for (int i = tid; i < S * S / 4; i += GROUPS * PAIR_THREADS) {
+        const int r = i % S, p = i / S;
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(basis + r * S) + p);
+        const float4 h = make_float4(tf32_rn(v.x), tf32_rn(v.y), tf32_rn(v.z), tf32_rn(v.w));
+        const float4 l = make_float4(tf32_rn(v.x - h.x), tf32_rn(v.y - h.y), tf32_rn(v.z - h.z), tf32_rn(v.w - h.w));
+        if (need_k_major) write_split<false>(f.sm + OFF_BK_HI, f.sm + OFF_BK_LO, r, p, h, l);
+        write_split<true>(f.sm + OFF_BM_HI, f.sm + OFF_BM_LO, r, p, h, l);
     }
     fence_proxy_async();  // generic-proxy writes -> visible to the tensor core's reads
     f.tmem = tmem_alloc_cta(tmem_slot, TMEM_COLS);
@@ -297,9 +279,10 @@ __device__ __forceinline__ void write_row(float *X, int r, const float (&v)[S])
         reinterpret_cast<float4 *>(X + r * XS)[j4] = make_float4(v[4 * j4], v[4 * j4 + 1], v[4 * j4 + 2], v[4 * j4 + 3]);
 }
 
-// BIGK (k > MAX_K_LISTED): selection from quarter-row maxima with the wide list (3 groups fit), both inverse stages dense.
-// Without the prefetch, the same sizes: from the list k = 40 / 48 204 / 244 us (at 48 part of the lists overflow into the radix
-// select), dense k = 49 / 128 / 300 240 / 247 / 605 us.
+// BIGK (k > TC_MAX_K_LISTED): selection from quarter-row maxima with the wide list (3 groups fit), both inverse stages dense.
+// From the list / dense, 4096 x 4096, one worker: k = 44 118 / 127 us, k = 48 127 / 127 (part of the lists overflow: there is no room for a
+// wide list); 1024 x 1024: 30 / 28 and 40 / 28 us.
+constexpr int TC_MAX_K_LISTED = 44;
 template <typename GT, int GROUPS, bool BIGK, bool MANY>
 __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(DemoCompressArgs a)
 {
@@ -572,7 +555,7 @@ cudaError_t demo_launch_compress_tc(const DemoCompressArgs &a, DemoLaunch &dev, 
     auto pick = [&](auto gt, auto many) {
         using GT = decltype(gt);
         constexpr bool MANY = decltype(many)::value;
-        return a.k > MAX_K_LISTED ? launch_tc(compress_tc_kernel<GT, 3, true, MANY>, 3, FIXED + 6 * chunk_bytes(true), a, dev, stream)
+        return a.k > TC_MAX_K_LISTED ? launch_tc(compress_tc_kernel<GT, 3, true, MANY>, 3, FIXED + 6 * chunk_bytes(true), a, dev, stream)
                                   : launch_tc(compress_tc_kernel<GT, 4, false, MANY>, 4, FIXED + 8 * chunk_bytes(false), a, dev, stream);
     };
     if (a.n_entries > MANY_TENSORS)
