@@ -542,6 +542,16 @@ static bool use_small_tiles(const demo_ctx *ctx)
     return ctx->path == DEMO_PATH_AUTO && !ctx->custom_basis && demo_small_tiles_supported(ctx->cfg.chunk);
 }
 
+// Decode of long lists from many workers on few tiles is a serial chain of additions per tile: a CTA of the dense kernels has 256
+// threads for it, a tile of the small-chunk kernels 8 or 16.  s = 16, 256 tiles, small-chunk / dense kernels: k = 17 W = 64 63 / 35 us,
+// k = 64 W = 16 / 64 19 / 13, 66 / 33, k = 128 W = 8 13 / 10; s = 8, 256 tiles, k = 64, W = 8 / 64 9.8 / 9.4, 56 / 33; four times the tiles,
+// s = 16, k = 128, W = 8 / 16 13 / 15, 22 / 21, s = 8, k = 64, W = 16 17 / 17.
+static bool use_small_tiles_decode(const demo_ctx *ctx)
+{
+    const bool crowded = ctx->cfg.num_workers >= 8 && ctx->cfg.topk > ctx->cfg.chunk && ctx->chunks2d <= 2LL * ctx->launch.sm_count;
+    return use_small_tiles(ctx) && !crowded;
+}
+
 // A caller-supplied basis has no fast factorisation: its dense transforms run on the tensor cores where
 // there is a kernel for the chunk size, else on the CUDA cores.
 static bool use_tc_path(const demo_ctx *ctx)
@@ -792,7 +802,7 @@ static demo_status decode_common(demo_ctx *ctx, const void *const *payloads, int
     a.n_chunks = ctx->chunks2d;
     a.k = ctx->cfg.topk;  // <= s * s
     a.tickets = tickets_of(ctx, W);
-    const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
+    const bool small_tiles = ctx->n2d && use_small_tiles_decode(ctx);
     if (ctx->n2d && !small_tiles) {
         // (a caller-supplied basis: the signs come from the dense kernels, there is no tensor-core variant)
         if (use_fast_path(ctx))

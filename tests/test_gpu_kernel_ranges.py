@@ -499,3 +499,37 @@ def test_s64_compress_time_above_the_lists(basis):
         times[-k] = f.device_us("compress")
         f.tr.close()
     assert times[193] <= 2.0 * times[192] and times[-193] <= 2.2 * times[-192], times
+
+
+@pytest.mark.parametrize("shapes,s,k,workers,agg", [([(8 * 8, 37 * 8), (40,)], 8, 9, 8, 0), ([(8 * 8, 38 * 8), (40,)], 8, 20, 9, 2),
+                                                    ([(4 * 16, 5 * 16)], 16, 17, 8, 2), ([(18 * 16, 17 * 16)], 16, 40, 8, 0)])
+def test_small_tiles_many_workers(shapes, s, k, workers, agg):
+    """Eight workers and lists longer than a tile's lanes: up to 296 tiles on the dense kernels, more on the small-chunk ones."""
+    wl = inputs.Workload("st", shapes, chunk=s, topk=k, num_workers=workers, grad_kind="student_t_ties")
+    r = parity.Runner(wl, max_chunks=10**9, seed=k, agg=agg)
+    for _ in range(2):
+        r.step()
+    r.close()
+
+
+def test_decode_time_of_long_lists_on_few_small_tiles():
+    """64 workers' lists of half a tile, 256 tiles of 16 x 16: with 16 threads per tile 2.4 times as long as with 256."""
+    import paper_2411_19870_b200 as demo
+
+    wl = inputs.Workload("st", [(256, 256)], chunk=16, topk=128, num_workers=64, grad_kind="normal")
+    r = parity.Runner(wl, max_chunks=4)
+    r.step(check=False)
+    times = {}
+    for path in (demo.DEMO_PATH_AUTO, demo.DEMO_PATH_GENERIC):
+        r.tr.set_path(path)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        times[path] = math.inf
+        for _ in range(8):
+            t0.record()
+            for _ in range(8):
+                r.tr.decode_apply(r.payloads, r.params)
+            t1.record()
+            torch.cuda.synchronize()
+            times[path] = min(times[path], t0.elapsed_time(t1))
+    assert times[demo.DEMO_PATH_AUTO] <= 1.4 * times[demo.DEMO_PATH_GENERIC], times
+    r.close()
