@@ -8,7 +8,7 @@
  * (DCT tables, chunk tables, pointer tables, one status word).  Every call enqueues work on the
  * given CUDA stream and returns; argument errors are reported synchronously before any launch,
  * device-side problems through demo_device_status().  No C++ exception crosses this boundary,
- * there is no global state and no CPU fallback: without a CUDA device every compute entry point
+ * there is no global state (but for the array of demo_decode_apply_static) and no CPU fallback: without a CUDA device every compute entry point
  * fails with DEMO_ERR_CUDA.
  *
  * Streams: everything of a call runs on cuda_stream.  When a context holds both 2-D and 1-D tensors, the kernels of the
@@ -75,9 +75,10 @@ typedef struct {
     int32_t grad_dtype;    /* demo_dtype of the gradient tensors (momentum/params: f32) */
 } demo_config;
 
-/* Kernel family used for 2-D tensors.  AUTO picks the register-resident fast-DCT kernels where
- * they exist (s in {32, 64}) and the generic dense-contraction kernels elsewhere; GENERIC forces
- * the latter everywhere (used by tests to cross-check the two).  Both are CUDA paths. */
+/* Kernel family used for 2-D tensors.  AUTO picks the register-resident fast-DCT kernels (every s; 64 and 128 need the driver's
+ * tensor-map encoder; decode of a few 8 x 8 or 16 x 16 tiles with long lists from many workers uses the dense ones) and, under a
+ * caller-supplied basis, the tensor-core kernels where they exist; GENERIC forces the dense-contraction kernels everywhere (used by
+ * tests to cross-check the two).  1-D tensors have one family of kernels.  All are CUDA paths. */
 typedef enum { DEMO_PATH_AUTO = 0, DEMO_PATH_GENERIC = 1 } demo_path;
 
 /*
@@ -111,9 +112,9 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
  * DEMO_ND_MAX_CHUNK_ELEMS, k_eff = min(k, M) per tensor).  Every other entry point takes the context
  * unchanged, with these differences: a record's idx is the row-major position inside the chunk
  * (((j_0 * s_1 + j_1) * s_2 + j_2) ...), chunks are ordered row-major over the chunk grid
- * (k_0, ..., k_{d-1}); all tensors run on one family of kernels that apply the transform axis by axis as
- * dense contractions on the CUDA cores (no fast-DCT, tensor-core or side-stream path; demo_set_path has
- * no effect); demo_set_basis, demo_set_basis_gaussian and demo_get_basis return UNSUPPORTED (one basis
+ * (k_0, ..., k_{d-1}); all tensors run on one family of kernels that apply the transform axis by axis on the
+ * CUDA cores, extents up to 8 and powers of two in registers, others as dense contractions (no tensor-core path;
+ * demo_set_path has no effect), one launch per class of chunk sizes; demo_set_basis, demo_set_basis_gaussian and demo_get_basis return UNSUPPORTED (one basis
  * per chunk extent: only the DCT is built).  A descriptor whose chunk is an s x s tile of its last two axes
  * or a length-s segment of its last axis (all other chunk extents 1) gives the payload layout of demo_init
  * with chunk size s on the tensor flattened to its last two axes / last axis and, up to the fp32 rounding of a
@@ -186,9 +187,8 @@ demo_status demo_decode_apply(demo_ctx *ctx, const void *const *payloads, int32_
  * parameters writes sign(R) in {-1, 0, +1} as one int8 per parameter.
  *   signs_out    host array of n_tensors DEVICE pointers (int8, each shaped and ordered like its
  *                parameter tensor), overwritten; 16-byte aligned
- * Needs phi = DEMO_PHI_SIGN (INVALID_ARG otherwise).  2-D tensors run on the fast kernels where
- * demo_decode_apply does, everything else (and every tensor under a caller-supplied basis) on the dense
- * kernels.
+ * Needs phi = DEMO_PHI_SIGN (INVALID_ARG otherwise).  Every tensor runs on the kernels that demo_decode_apply uses for it,
+ * except 2-D tensors under a caller-supplied basis at chunk size 64, which run on the dense kernels.
  *
  * demo_apply_signs -- x <- x - lr (sign + weight_decay x) for every parameter, from such int8 tensors
  * (the broadcast's payload), with the context's current lr.
@@ -258,7 +258,7 @@ demo_status demo_step_host(demo_ctx *ctx, const void *const *host_grads, void *c
  * happen before any stream capture begins).  Every call copies its tables from host memory that is
  * gone when the call returns, so the call must not be recorded into a CUDA graph: a stream that is
  * capturing is refused with DEMO_ERR_INVALID_ARG before anything is enqueued.  The 2-D and 1-D
- * tensors run through the generic decode kernels.  Errors: INVALID_ARG, SHAPE, K, UNSUPPORTED, CUDA.
+ * tensors run through the decode kernels that DEMO_PATH_GENERIC uses.  Errors: INVALID_ARG, SHAPE, K, UNSUPPORTED, CUDA.
  */
 #define DEMO_STATIC_MAX_TENSORS 256
 #define DEMO_STATIC_MAX_WORKERS 64
@@ -296,7 +296,7 @@ demo_status demo_set_decode_mode(demo_ctx *ctx, int32_t aggregation, int32_t phi
  * vectors; it replaces the DCT matrix on both axes of a 2-D chunk (Q = P B P^T, inverse P^T Q P) and on
  * 1-D segments (q = P b).  While a caller-supplied basis is active the fast kernels (which hard-code the
  * DCT factorisation) are out: 2-D tensors at chunk size 64 run on tensor-core kernels (3xTF32, fp32
- * accuracy), everything else on the dense CUDA-core kernels; DEMO_PATH_GENERIC forces the latter.
+ * accuracy), other 2-D tensors on the dense CUDA-core kernels (DEMO_PATH_GENERIC: all), 1-D tensors on the kernels they always use.
  *
  * demo_set_basis: basis_host = HOST pointer to P, read during the call and not retained; NULL restores
  * the DCT.  The rows must be orthonormal to 1e-5 (INVALID_ARG otherwise).  The upload is enqueued on

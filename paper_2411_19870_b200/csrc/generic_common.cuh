@@ -1,5 +1,4 @@
-// Helpers shared by the dense-transform kernels (kernels_generic.cu, kernels_nd.cu): magnitude keys, a
-// CTA-wide prefix sum, the exact radix select behind the top-k, and the persistent-grid launcher.
+// Helpers of the dense-transform kernels (kernels_generic.cu): magnitude keys, a CTA-wide prefix sum, the exact radix select behind the top-k, and the persistent-grid launcher.
 #pragma once
 
 #include "demo_internal.h"

@@ -21,7 +21,7 @@ struct Cfg {
     static constexpr int LOG2S = (S == 64) ? 6 : 5;
 };
 
-// Bytes of one decode slot: the tile, the mbarrier and -- for the count-normalised mean -- one
+// Bytes of one decode slot: the tile, the walk, the staged records and -- for the count-normalised mean -- one
 // 16-bit sender count per coordinate.
 template <int S>
 __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)

@@ -11,7 +11,7 @@
 // where thread h of a line finishes n in [32h, 32h+32): the two exchange half of e and o through shared memory.
 //
 // compress: TMA-staged m and g tiles -> B = beta*m + g (parked in tensor memory) -> column pass -> row pass ->
-// coefficients in shared memory -> exact top-k (bound from the 256 half-row maxima, candidate list, exact ranking; radix
+// coefficients in shared memory -> exact top-k (bound from the 256 half-row maxima, candidate list, ballot search; radix
 // select for degenerate chunks) -> records; sparse row stage of the inverse from the records, half of them by each half of
 // the CTA, fast column stage, residual m <- B - alpha * IDCT(kept) against the parked B, one TMA store of the new momentum
 // tile.  The next chunk's g tile comes in, and its m tile to L2, as soon as B is formed.  decode: scatter-add of the W payloads
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         // odd ones (tid odd); element e of its half is coefficient 2e + (tid & 1), flat index 128*(tid/2) + 2e + (tid&1).
         // Fast path (k_eff <= 256): the k_eff-th largest of the 256 per-thread maxima is a lower bound L of
         // the k_eff-th largest coefficient (256 groups: the bound is tight, a few dozen candidates); the
-        // candidates are listed in index order and ranked exactly, ties to the lowest index.  Everything
+        // candidates are listed in index order and searched by ballots, ties to the lowest index.  Everything
         // compares integer magnitude keys, so NaN and Inf are ordered like any other bit pattern.  More
         // than CAP128 candidates (tied or degenerate chunks) or k_eff > 256: radix select below.
         // the row-stage list is padded with zero-valued entries whose "row" is a scratch line, the then unused histogram
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         }
         __syncthreads();
 
-        // ---- column stage of the inverse (split), second fetch of the tiles, residual --------------
+        // ---- column stage of the inverse (split), residual --------------
 #pragma unroll
         for (int p = 0; p < H; ++p) in[p] = X[(2 * p + h) * XS + j];
         fence_proxy_async();

@@ -14,8 +14,9 @@
 //     the residual, instead of fetching and recombining the two tiles a second time;
 //   * the next chunk's tiles are requested as soon as the transpose tile is dead, so they land behind
 //     the inverse transform and the store burst of the current chunk;
-//   * everything rare (tied or degenerate chunks, tiles of low rank, k > 64) lives in one out-of-line
-//     routine that works from the coefficient tile in shared memory.
+//   * k > 48 has an instantiation of its own (select64.cuh); everything rare (tied or degenerate chunks, tiles of low
+//     rank, k above the bounds of the lists) lives in out-of-line routines that work from the coefficient tile in
+//     shared memory.
 // Every wait on an mbarrier is bounded: on expiry the slot records DEMO_DEV_TIMEOUT and stops.
 #include <cuda_bf16.h>
 

@@ -18,8 +18,8 @@
 //     of eight elements per thread are issued together;
 //   * top-k: the k-th largest of the threads' maxima (from a histogram relative to the largest) bounds the k-th coefficient;
 //     the few dozen to few hundred coefficients above it are listed, one warp finds the k-th among them, and the kept ones
-//     are put in index order by counting; radix select only when the list overflows (chunks with many equal magnitudes, k
-//     beyond the bound).
+//     are put in index order by counting or, where much of a chunk is kept, by going over the tile; radix select only when the
+//     list overflows (chunks with many equal magnitudes, k beyond the bound).
 // Measured (one call, bf16 gradients, k = 32; dense contractions on every axis with radix select -> this): four
 // 512 x 512 x 3 x 3 weights in 32 x 32 x 3 x 3 chunks (9.4 M parameters) compress 381 -> 115 us, decode 219 -> 63;
 // 7511 x 512 in 29 x 64: 243 -> 83 / 122 -> 36; 8192 x 8192 in 32 x 128: 2424 -> 1050 / 1155 -> 379; in 16 x 32 (k = 4):
