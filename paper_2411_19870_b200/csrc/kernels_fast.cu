@@ -99,7 +99,6 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     // has to be known during the current one (its records are requested), so a group is drawn two ahead: thread 0 draws at
     // the start of a chunk and writes the result down behind the scatter; the loop-top barrier publishes it.
     __shared__ unsigned drawn[2];
-    if (threadIdx.x == 0) drawn[0] = ticket_draw(a.tickets);
     unsigned group = blockIdx.x, next_group, par = 0;
     long long c = (long long)group * NCH + slot;
     int buf = 0, which = 0;  // staging buffer and walk slot of the current chunk
@@ -109,6 +108,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         walk.seek<S>(a.entries, a.n_entries, c, k_eff, 0);
     }
     sb.sync();
+    order.begin();
+    if (threadIdx.x == 0) drawn[0] = second_ticket(a.tickets, (unsigned)((a.n_chunks + NCH - 1) / NCH));
     if (c < a.n_chunks) stage_batch(0, 0, 0);
     for (; (long long)group * NCH < a.n_chunks; group = next_group, c = (long long)group * NCH + slot, par ^= 1u, which ^= 1) {
         __syncthreads();  // (publishes the draw; all slots start a chunk together)
@@ -120,8 +121,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
         if (t == 0 && more) walk.seek<S>(a.entries, a.n_entries, (long long)next_group * NCH + slot, k_eff, which ^ 1);
         if (!SIGNS) {  // row t of the x tile on its way to L2
             const float *xr = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)t * walk.n1[which];
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
-            if (S == 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 32));
+            prefetch_l2(xr);
+            if (S == 64) prefetch_l2(xr + 32);
         }
 
         {
@@ -256,7 +257,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 },
                 [&] { sb.sync(); });
         }
-        if (threadIdx.x == 0) drawn[par ^ 1u] = ticket;
+        if (threadIdx.x == 0) drawn[par ^ 1u] = ticket + tickets_from((unsigned)((a.n_chunks + NCH - 1) / NCH));
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0 (row t is this thread's)
             for (int v = 0; v < S; ++v) {
                 const unsigned short n = Cn[t * S + v];

@@ -143,18 +143,6 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
 
     const int tid = threadIdx.x, h = tid >> 7, j = tid & 127;
     const uint32_t bar = smem_u32(bar_mem);
-    if (tid == 0) {
-        mbar_init(bar, 1);
-        fence_proxy_async();
-    }
-    // Tensor memory as storage: column j of B = beta*m + g is parked in lane j between the forward pass and the residual, by
-    // thread (0, j) its rows 0..63 in columns 0..63, by thread (1, j) its rows 127..64 in columns 64..127; each of the two
-    // reads back half of both.
-    if (tid == 0) tmem_slot[1] = ticket_draw(a.tickets);
-    const uint32_t tmem_base = tmem_alloc_cta(tmem_slot, TMEM_COLS128);
-    fence_proxy_async();
-    const uint32_t taddr = tmem_base + ((uint32_t)(j & ~31) << 16);
-
     EntryCursor cur;
     unsigned phase = 0;
     const char *acquired = nullptr;
@@ -168,25 +156,45 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
         }
     };
     // (thread 0) requests a chunk's g tile, which may come as soon as the one before it has been read, and with it announces
-    // both tiles; the m tile follows when the new momentum of the chunk before has left its place
-    auto issue_tile = [&](const DemoTensorEntry &te, long long c, bool g) {
+    // both tiles; the m tile follows when the new momentum of the chunk before has left its place.  `ahead`: both only to L2.
+    auto issue_tile = [&](const DemoTensorEntry &te, long long c, bool g, bool ahead) {
         const unsigned lc = (unsigned)(c - te.chunk_begin);
         const unsigned k0 = lc / (unsigned)te.c1, k1 = lc - k0 * (unsigned)te.c1;
-        const char *tm = static_cast<const char *>(g ? a.tmap_g : a.tmap_m) + (size_t)te.tensor * TMAP_BYTES;
-        if (g) mbar_expect_tx(bar, TILE_BYTES);
-        tma_load_2d(g ? smem_u32(Gs) : smem_u32(Ms), tm, k1 * S, k0 * S, bar);
-        if (g) tma_prefetch_2d(static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES, k1 * S, k0 * S);
+        const char *tm_g = static_cast<const char *>(a.tmap_g) + (size_t)te.tensor * TMAP_BYTES;
+        const char *tm_m = static_cast<const char *>(a.tmap_m) + (size_t)te.tensor * TMAP_BYTES;
+        if (ahead) {
+            tma_prefetch_2d(tm_g, k1 * S, k0 * S);
+        } else {
+            if (g) mbar_expect_tx(bar, TILE_BYTES);
+            tma_load_2d(g ? smem_u32(Gs) : smem_u32(Ms), g ? tm_g : tm_m, k1 * S, k0 * S, bar);
+        }
+        if (g || ahead) tma_prefetch_2d(tm_m, k1 * S, k0 * S);
     };
 
     long long c = blockIdx.x;
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        fence_proxy_async();
+    }
     if (c < a.n_chunks) {
         cur.seek(a.entries, a.n_entries, c);
         acquire_maps(cur.te);
-        if (tid == 0) {
-            issue_tile(cur.te, c, true);
-            issue_tile(cur.te, c, false);
-        }
+        if (tid == 0) issue_tile(cur.te, c, false, true);
     }
+    order.begin();
+    if (tid == 0 && c < a.n_chunks) {
+        issue_tile(cur.te, c, true, false);
+        issue_tile(cur.te, c, false, false);
+    }
+    __syncwarp();
+    // Tensor memory as storage: column j of B = beta*m + g is parked in lane j between the forward pass and the residual, by
+    // thread (0, j) its rows 0..63 in columns 0..63, by thread (1, j) its rows 127..64 in columns 64..127; each of the two
+    // reads back half of both.
+    if (tid == 0) tmem_slot[1] = ticket_draw(a.tickets);
+    const uint32_t tmem_base = tmem_alloc_cta(tmem_slot, TMEM_COLS128);
+    fence_proxy_async();
+    const uint32_t taddr = tmem_base + ((uint32_t)(j & ~31) << 16);
+
     for (long long nc; c < a.n_chunks; c = nc) {
         const DemoTensorEntry te = cur.te;  // the cursor points at chunk c
         const unsigned lc = (unsigned)(c - te.chunk_begin);
@@ -236,7 +244,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 fence_proxy_async();
                 __syncthreads();  // the staged tiles are consumed (X aliases the m tile)
-                if (tid == 0 && nc < a.n_chunks) issue_tile(cur.te, nc, true);
+                if (tid == 0 && nc < a.n_chunks) issue_tile(cur.te, nc, true, false);
             } else {
                 // row j of the column-transformed tile, folded
                 const float4 *row = reinterpret_cast<const float4 *>(X + j * XS);
@@ -615,7 +623,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                          smem_u32(Ms));
             tma_store_commit();
             tma_store_wait_read();  // the store has read the tile: the next chunk's m tile may land
-            if (nc < a.n_chunks) issue_tile(cur.te, nc, false);
+            if (nc < a.n_chunks) issue_tile(cur.te, nc, false, false);
             tmem_slot[1] = ticket;
         }
     }
@@ -671,15 +679,19 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
 
     unsigned c = blockIdx.x, par = 0;
     int buf = 0, which = 0;  // staging buffer and walk slot of the current chunk
-    if (tid == 0) {
-        drawn[0] = ticket_draw(a.tickets);
-        if (c < n_chunks) {
-            walk.e = demo_find_entry(a.entries, a.n_entries, c);
-            walk.load(a.entries, a.n_entries);
-            walk.seek<S>(a.entries, a.n_entries, c, k_eff, 0);
-        }
+    if (tid == 0 && c < n_chunks) {
+        walk.e = demo_find_entry(a.entries, a.n_entries, c);
+        walk.load(a.entries, a.n_entries);
+        walk.seek<S>(a.entries, a.n_entries, c, k_eff, 0);
     }
     __syncthreads();
+    if (!SIGNS && c < n_chunks && tid < 128) {  // half a row per thread of the rows that are fetched first on their way to L2
+        const float *xr = a.x_ptrs[walk.tensor[0]] + walk.elem[0] + (size_t)(tid >> 1) * walk.n1[0] + (tid & 1) * 64;
+        prefetch_l2(xr);
+        prefetch_l2(xr + 32);
+    }
+    order.begin();
+    if (tid == 0) drawn[0] = second_ticket(a.tickets, n_chunks);
     if (KMODE == STAGED && c < n_chunks) stage_batch(0, 0, 0);
     for (unsigned nc; c < n_chunks; c = nc, par ^= 1u, which ^= 1) {
         __syncthreads();  // (publishes the draw; the tile and the landing area are free)
@@ -703,7 +715,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         if (!SIGNS) {
             if (!counts) fetch_rows(Xh, 0);
             const float *xr = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)(64 + (tid >> 2)) * walk.n1[which] + (tid & 3) * 32;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
+            prefetch_l2(xr);
         }
         for (int i = tid; i < S * XSD / 4; i += THREADS) reinterpret_cast<float4 *>(St)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (counts)
@@ -764,7 +776,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                 },
                 [] { __syncthreads(); });
         }
-        if (tid == 0) drawn[par ^ 1u] = ticket;
+        if (tid == 0) drawn[par ^ 1u] = ticket + tickets_from(n_chunks);
         __syncthreads();
         if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
             for (int i = tid; i < M; i += THREADS) {

@@ -71,6 +71,7 @@ template <int S>
 __global__ void __launch_bounds__(GEN_THREADS) compress_generic_kernel(DemoCompressArgs a)
 {
     const StreamOrder order(a.wait_first);
+    order.begin();
     constexpr int M = S * S;
     extern __shared__ float smem[];
     float *Bt = smem;
@@ -168,6 +169,7 @@ template <int S>
 __global__ void __launch_bounds__(GEN_THREADS) decode_generic_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
+    order.begin();
     constexpr int M = S * S;
     extern __shared__ float smem[];
     float *St = smem;

@@ -179,6 +179,17 @@ __device__ __forceinline__ void enter_layout(const View &v, const DemoNdEntry &e
         v.tile1[i] = 0.f;
     }
 }
+// A chunk's rows on their way to L2, a row per thread.
+template <typename T>
+__device__ __forceinline__ void prefetch_chunk(const View &v, const DemoNdEntry &e, const T *base)
+{
+    if (!e.row_table) return;
+    for (int r = threadIdx.x; r * e.row < e.M; r += blockDim.x) {
+        const T *p = base + v.rows[r].x, *end = p + e.row;
+        for (; p < end; p += 128 / sizeof(T)) prefetch_l2(p);
+        prefetch_l2(end - 1);
+    }
+}
 // Runs over the chunk's elements, U per thread and round: every thread calls load(j, offset in the tensor) U times without
 // a branch in between (the last element again where there is none left), then use(j, index, offset, tile position) for
 // those that exist.
@@ -976,7 +987,16 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
     if (tid < 2) s->e[tid].chunk_begin = 1, s->e[tid].chunk_end = 0;  // no tensor yet
     __syncthreads();
     if (tid == 0 && blockIdx.x < a.cls.n_chunks) locate(s, 0, a.entries, a.cls.n, blockIdx.x);
+    __syncthreads();
     int layout = -1, slot = 0;
+    if (!BIG && blockIdx.x < a.cls.n_chunks) {  // (in the kernels of the large extents it spills registers of the loop below)
+        layout = s->e[0].layout;
+        enter_layout(v, s->e[0], a.cls);
+        __syncthreads();
+        prefetch_chunk(v, s->e[0], a.m_ptrs[s->e[0].tensor] + s->base[0]);
+        prefetch_chunk(v, s->e[0], static_cast<const GT *>(a.g_ptrs[s->e[0].tensor]) + s->base[0]);
+    }
+    order.begin();
 
     for (long long c = blockIdx.x; c < a.cls.n_chunks; c = (long long)gridDim.x + s->ticket, slot ^= 1) {
         // cleared for this chunk's selection; the barriers up to it order the writes
@@ -1037,7 +1057,15 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
     if (tid < 2) s->e[tid].chunk_begin = 1, s->e[tid].chunk_end = 0;
     __syncthreads();
     if (tid == 0 && blockIdx.x < a.cls.n_chunks) locate(s, 0, a.entries, a.cls.n, blockIdx.x);
+    __syncthreads();
     int layout = -1, slot = 0;
+    if (!BIG && blockIdx.x < a.cls.n_chunks) {  // (in the kernels of the large extents it spills registers of the loop below)
+        layout = s->e[0].layout;
+        enter_layout(v, s->e[0], a.cls);
+        __syncthreads();
+        if (!a.sign_ptrs) prefetch_chunk(v, s->e[0], a.x_ptrs[s->e[0].tensor] + s->base[0]);
+    }
+    order.begin();
 
     for (long long c = blockIdx.x; c < a.cls.n_chunks; c = (long long)gridDim.x + s->ticket, slot ^= 1) {
         __syncthreads();

@@ -59,8 +59,19 @@ __device__ __forceinline__ float inverse_segment(const float *line, const float 
     return r;
 }
 
+// A warp's first round looks its chunk up and prefetches it in front of the line that StreamOrder draws (launch.cuh).
+struct FirstRound {
+    const StreamOrder &order;
+    bool left;
+    __device__ __forceinline__ void begin()
+    {
+        if (left) order.begin();
+        left = false;
+    }
+};
+
 template <int S>
-__device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long long c_own, float *line)
+__device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long long c_own, float *line, FirstRound &first)
 {
     constexpr int E = Seg<S>::E;
     const int lane = threadIdx.x & 31, i = threadIdx.x % (32 * E);  // (i >= s only for s < 32)
@@ -72,6 +83,11 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     float *__restrict__ m = a.m_ptrs[te.tensor];
     const void *g = a.g_ptrs[te.tensor];
     const int k = te.k_eff;
+    if (first.left && on) {
+        prefetch_l2(m + off);
+        prefetch_l2(static_cast<const char *>(g) + off * (a.grad_bf16 ? 2 : 4));
+    }
+    first.begin();
 
     // momentum update  b = beta*m + g  (Algorithm 1, worker side)
     float b = 0.f, q = 0.f;
@@ -155,7 +171,7 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
 }
 
 template <int S>
-__device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long long c_own, float *line, unsigned short *senders)
+__device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long long c_own, float *line, unsigned short *senders, FirstRound &first)
 {
     constexpr int E = Seg<S>::E;
     const int i = threadIdx.x % (32 * E);
@@ -167,6 +183,8 @@ __device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long lon
     const size_t off = (size_t)lc * S + i;
     const int k = te.k_eff;
     const long long rec_off = te.rec_begin + lc * (long long)k + i;
+    if (first.left && on && !a.sign_ptrs) prefetch_l2(a.x_ptrs[te.tensor] + off);
+    first.begin();
     if (i < S) {
         line[i] = 0.f;
         if (counts) senders[i] = 0;
@@ -270,7 +288,7 @@ __device__ __forceinline__ void inverse_tile(float (&q)[S], float *X, int j)
 }
 
 template <int S, typename GT>
-__device__ __forceinline__ void compress_tiles(const DemoCompressArgs &a, long long group, float *warp_mem)
+__device__ __forceinline__ void compress_tiles(const DemoCompressArgs &a, long long group, float *warp_mem, FirstRound &first)
 {
     constexpr int XS = Tile<S>::XS, M = S * S;
     const int lane = threadIdx.x & 31, j = lane % S, sub = lane / S;
@@ -281,6 +299,11 @@ __device__ __forceinline__ void compress_tiles(const DemoCompressArgs &a, long l
     const int n1 = t.te.n1, k = t.te.k_eff;
     float *__restrict__ m = a.m_ptrs[t.te.tensor] + t.base;
     const GT *__restrict__ g = static_cast<const GT *>(a.g_ptrs[t.te.tensor]) + t.base;
+    if (first.left) {  // row j
+        prefetch_l2(m + (size_t)j * n1 - j);
+        prefetch_l2(g + (size_t)j * n1 - j);
+    }
+    first.begin();
 
     // momentum update  B = beta*m + g, column j  (Algorithm 1, worker side)
     float B[S], q[S];
@@ -363,7 +386,7 @@ __device__ __forceinline__ void compress_tiles(const DemoCompressArgs &a, long l
 }
 
 template <int S>
-__device__ __forceinline__ void decode_tiles(const DemoDecodeArgs &a, long long group, float *warp_mem, unsigned short *warp_counts)
+__device__ __forceinline__ void decode_tiles(const DemoDecodeArgs &a, long long group, float *warp_mem, unsigned short *warp_counts, FirstRound &first)
 {
     constexpr int XS = Tile<S>::XS, M = S * S;
     const int lane = threadIdx.x & 31, j = lane % S, sub = lane / S;
@@ -375,6 +398,8 @@ __device__ __forceinline__ void decode_tiles(const DemoDecodeArgs &a, long long 
     const TileRef<S> t = tile_ref<S>(a.entries, a.n_entries, on ? c_own : a.n_chunks - 1, j);
     const int n1 = t.te.n1, k = t.te.k_eff;
     const long long rec_off = t.te.rec_begin + t.lc * (long long)k;
+    if (first.left && !a.sign_ptrs) prefetch_l2(a.x_ptrs[t.te.tensor] + t.base + (size_t)j * n1 - j);
+    first.begin();
 #pragma unroll
     for (int v = 0; v < S; ++v) {
         X[j * XS + v] = 0.f;
@@ -456,6 +481,7 @@ template <int S, typename GT, bool TILES>
 __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArgs segs, DemoCompressArgs tiles, int seg_blocks)
 {
     const StreamOrder order(segs.wait_first);
+    FirstRound first{order, true};
     __shared__ __align__(16) float mem[WARPS][warp_floats<S, TILES>()];
     const int warp = threadIdx.x >> 5;
     if (!TILES || (int)blockIdx.x < seg_blocks) {
@@ -463,19 +489,21 @@ __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArg
         constexpr int PB = Seg<S>::PER_BLOCK;
         const int own = warp / Seg<S>::E;
         for (long long c0 = (long long)blockIdx.x * PB; c0 < segs.n_chunks; c0 += (long long)seg_blocks * PB)
-            compress_segment<S>(segs, c0 + own, mem[own]);
+            compress_segment<S>(segs, c0 + own, mem[own], first);
     } else if constexpr (TILES) {
         const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
         const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
         for (long long p = (long long)(blockIdx.x - seg_blocks) * WARPS + warp; p < groups; p += stride)
-            compress_tiles<S, GT>(tiles, p, mem[warp]);
+            compress_tiles<S, GT>(tiles, p, mem[warp], first);
     }
+    first.begin();  // (a warp without a round)
 }
 
 template <int S, bool TILES>
 __global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs segs, DemoDecodeArgs tiles, int seg_blocks)
 {
     const StreamOrder order(segs.wait_first);
+    FirstRound first{order, true};
     __shared__ __align__(16) float mem[WARPS][warp_floats<S, TILES>()];
     __shared__ unsigned short counts[WARPS][TILES ? Tile<S>::PER_WARP * S * S : S];
     const int warp = threadIdx.x >> 5;
@@ -484,13 +512,14 @@ __global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs se
         constexpr int PB = Seg<S>::PER_BLOCK;
         const int own = warp / Seg<S>::E;
         for (long long c0 = (long long)blockIdx.x * PB; c0 < segs.n_chunks; c0 += (long long)seg_blocks * PB)
-            decode_segment<S>(segs, c0 + own, mem[own], counts[own]);
+            decode_segment<S>(segs, c0 + own, mem[own], counts[own], first);
     } else if constexpr (TILES) {
         const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
         const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
         for (long long p = (long long)(blockIdx.x - seg_blocks) * WARPS + warp; p < groups; p += stride)
-            decode_tiles<S>(tiles, p, mem[warp], counts[warp]);
+            decode_tiles<S>(tiles, p, mem[warp], counts[warp], first);
     }
+    first.begin();
 }
 
 // Up to eight blocks per SM for each list (what 64 registers per thread allow).

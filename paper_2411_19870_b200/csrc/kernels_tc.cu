@@ -131,7 +131,8 @@ struct TcFrame {
 };
 
 template <int GROUPS>
-__device__ __forceinline__ void tc_setup(TcFrame &f, unsigned char *raw, const float *basis, bool need_k_major, int chunk_area)
+__device__ __forceinline__ void tc_setup(TcFrame &f, unsigned char *raw, const float *basis, bool need_k_major, int chunk_area,
+                                         const StreamOrder &order)
 {
     const int tid = threadIdx.x, warp = tid >> 5;
     const uint32_t raw_s = smem_u32(raw);
@@ -148,6 +149,7 @@ __device__ __forceinline__ void tc_setup(TcFrame &f, unsigned char *raw, const f
         mbar_init(f.bar, 1);
         fence_proxy_async();
     }
+    order.begin();  // (the basis is written by earlier work)
     // (all threads: by 64 of them, a row each, decode of 1024 x 1024 takes 18.3 us instead of 17.9)
     for (int i = tid; i < S * S / 4; i += GROUPS * PAIR_THREADS) {
         const int r = i % S, p = i / S;
@@ -289,8 +291,25 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
     const StreamOrder order(a.wait_first);
     extern __shared__ unsigned char smem_raw[];
     constexpr int AREA = chunk_bytes(BIGK);
+    const unsigned n_chunks = (unsigned)a.n_chunks, n_pairs = (n_chunks + 1u) / 2u;
+    const int k_eff = a.k;
+    // row `row` of a chunk's tiles on its way to L2; e0: an entry at or in front of the chunk's
+    auto prefetch_row = [&](unsigned chunk, int row, int e0) {
+        const ChunkRef nr = locate<MANY>(a.entries, a.n_entries, chunk, k_eff, e0);
+        const size_t at = nr.elem + (size_t)row * nr.n1;
+        const float *nm = a.m_ptrs[nr.tensor] + at;
+        const GT *ng = static_cast<const GT *>(a.g_ptrs[nr.tensor]) + at;
+        prefetch_l2(nm);
+        prefetch_l2(nm + 32);
+        prefetch_l2(ng);
+        if (sizeof(GT) == 4) prefetch_l2(ng + 32);
+    };
+    {
+        const unsigned first = 2u * (blockIdx.x * GROUPS + threadIdx.x / PAIR_THREADS) + (threadIdx.x >> 6 & 1);
+        if (first < n_chunks) prefetch_row(first, threadIdx.x & 63, 0);
+    }
     TcFrame f;
-    tc_setup<GROUPS>(f, smem_raw, a.C, true, AREA);
+    tc_setup<GROUPS>(f, smem_raw, a.C, true, AREA, order);
     const int c = f.pt >> 6, r = f.pt & 63;
     const SlotBarrier<PAIR_THREADS> pb{1 + f.g};        // the 128 threads of the pair
     const int bar_id = 1 + GROUPS + 2 * f.g + c;
@@ -308,8 +327,6 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
     sm.widx = sm.wkey + WCAP + 4;
     constexpr int PAD_ROW = (X_BYTES + 65 * 16) / 4;  // the scratch line tmax[0..S) seen from X
     float *X = sm.X;
-    const int k_eff = a.k;
-    const unsigned n_chunks = (unsigned)a.n_chunks, n_pairs = (n_chunks + 1u) / 2u;
     bool ok = true;
     int e = 0;
 
@@ -342,17 +359,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         const unsigned next = *f.drawn;  // (written before the barriers of the stages; overwritten behind those below)
         // row r of the group's next tiles on its way to L2.  (Without a counter next is NO_TICKET = 2^31 behind the grid, which then has a
         // group for every pair: 2 next wraps to twice the grid's groups, past the last chunk.)
-        if (2u * next + c < n_chunks) {
-            int e2 = e;
-            const ChunkRef nr = locate<MANY>(a.entries, a.n_entries, 2u * next + c, k_eff, e2);
-            const size_t at = nr.elem + (size_t)r * nr.n1;
-            const float *nm = a.m_ptrs[nr.tensor] + at;
-            const GT *ng = static_cast<const GT *>(a.g_ptrs[nr.tensor]) + at;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(nm));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(nm + 32));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(ng));
-            if (sizeof(GT) == 4) asm volatile("prefetch.global.L2 [%0];" ::"l"(ng + 32));
-        }
+        if (2u * next + c < n_chunks) prefetch_row(2u * next + c, r, e);
 
         // ---- exact top-k, records, and the row stage of the inverse -------------------------------------------
         if constexpr (BIGK) {
@@ -414,15 +421,26 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
     extern __shared__ unsigned char smem_raw[];
     const bool counts = a.agg == 2;
     const int area = X_BYTES + (counts ? M * 2 : 0);
+    const unsigned n_chunks = (unsigned)a.n_chunks, n_pairs = (n_chunks + 1u) / 2u;
+    const int k_eff = a.k;
+    // row `row` of a chunk's x tile on its way to L2
+    auto prefetch_row = [&](const ChunkRef &cr, int row) {
+        const float *xr = a.x_ptrs[cr.tensor] + cr.elem + (size_t)row * cr.n1;
+        prefetch_l2(xr);
+        prefetch_l2(xr + 32);
+    };
+    {
+        const unsigned first = 2u * (blockIdx.x * GROUPS + threadIdx.x / PAIR_THREADS) + (threadIdx.x >> 6 & 1);
+        int e0 = 0;
+        if (first < n_chunks) prefetch_row(locate<MANY>(a.entries, a.n_entries, first, k_eff, e0), threadIdx.x & 63);
+    }
     TcFrame f;
-    tc_setup<GROUPS>(f, smem_raw, a.C, false, area);
+    tc_setup<GROUPS>(f, smem_raw, a.C, false, area, order);
     const int c = f.pt >> 6, r = f.pt & 63, lane = f.pt & 31, warp = (f.pt >> 5) & 1;
     const SlotBarrier<PAIR_THREADS> pb{1 + f.g};
     const SlotBarrier<S> sb{1 + GROUPS + 2 * f.g + c};
     float *X = reinterpret_cast<float *>(f.sm + 4 * BLK + (2 * f.g + c) * area);
     unsigned short *Cn = reinterpret_cast<unsigned short *>(X + S * XS);  // senders per coordinate (agg == 2)
-    const int k_eff = a.k;
-    const unsigned n_chunks = (unsigned)a.n_chunks, n_pairs = (n_chunks + 1u) / 2u;
     bool ok = true;
     int e = 0;
 
@@ -438,10 +456,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
         if (valid) {
             cr = locate<MANY>(a.entries, a.n_entries, chunk, k_eff, e);
             x = a.x_ptrs[cr.tensor] + cr.elem + r;
-            // the x tile on its way to L2
-            const float *xr = a.x_ptrs[cr.tensor] + cr.elem + (size_t)r * cr.n1;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 32));
+            prefetch_row(cr, r);
             write_row(X, r, v);
             if (counts)
                 for (int i = 0; i < S; ++i) Cn[r * S + i] = 0;

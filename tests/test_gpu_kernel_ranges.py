@@ -533,3 +533,31 @@ def test_decode_time_of_long_lists_on_few_small_tiles():
             times[path] = min(times[path], t0.elapsed_time(t1))
     assert times[demo.DEMO_PATH_AUTO] <= 1.4 * times[demo.DEMO_PATH_GENERIC], times
     r.close()
+
+
+@pytest.mark.parametrize("s,grid", [(32, 148 * 8), (64, 148 * 8), (128, 148 * 2)])
+@pytest.mark.parametrize("rounds,extra", [(1, 0), (1, 1), (2, -1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 3)])
+def test_chunks_of_the_first_rounds(s, grid, rounds, extra):
+    """Every chunk is processed once whether a CTA's second chunk is fixed or drawn (up to three rounds of the grid of the decode kernels, or
+    more): one row of chunks in one call against the same chunks as tensors of one to four chunks each, bit for bit, over two calls."""
+    import paper_2411_19870_b200 as demo
+
+    n, k = rounds * grid + extra, 3
+    cut = [n // 2, n - n // 2]
+    g = torch.randn(s, n * s, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+
+    def run(widths):
+        tr = demo.DemoTransform([(s, w * s) for w in widths], chunk=s, topk=k, beta=0.9, lr=0.125, weight_decay=0.1, num_workers=1,
+                                grad_dtype=demo.DEMO_F32)
+        split = lambda t: [v.contiguous() for v in t.split([w * s for w in widths], dim=1)]  # noqa: E731
+        gs, ms, xs = split(g), split(0.5 * g), split(0.25 * g)
+        pay = torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda")
+        for _ in range(2):
+            tr.compress(0, gs, ms, pay)
+            tr.decode_apply([pay], xs)
+        assert tr.device_status() == 0
+        tr.close()
+        return pay, torch.cat(ms, 1), torch.cat(xs, 1)
+
+    for a, b in zip(run([n]), run(cut)):
+        assert torch.equal(a, b)
