@@ -19,6 +19,10 @@ struct Cfg {
     static constexpr int XS = S + 4;  // row stride of the transpose tile: conflict-free scalar
                                       // column access and 128-bit row access
     static constexpr int LOG2S = (S == 64) ? 6 : 5;
+    // Row stride of the sender counts (16 bit): a thread goes over its row 16 bytes at a time, and rows 16 bytes apart in their banks keep
+    // the threads out of each other's way.  (Rows end to end and one count per access, 32 threads on one bank: 4096 x 4096, W = 1 / 16,
+    // count-normalised 92 / 105 us, now 31 / 50; the sum 30 / 36.)
+    static constexpr int CS = S + 8;
 };
 
 // Bytes of one decode slot: the tile, the walk, the staged records and -- for the count-normalised mean -- one
@@ -26,7 +30,7 @@ struct Cfg {
 template <int S>
 __host__ __device__ constexpr size_t decode_slot_bytes(bool counts)
 {
-    return ((size_t)S * Cfg<S>::XS * 4 + 128 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + (counts ? (size_t)S * S * 2 : 0) + 127) /
+    return ((size_t)S * Cfg<S>::XS * 4 + 128 + 2 * STAGE_RECORDS * sizeof(DemoRecord) + (counts ? (size_t)S * Cfg<S>::CS * 2 : 0) + 127) /
            128 * 128;
 }
 
@@ -46,8 +50,10 @@ static_assert(sizeof(DecodeWalk) <= 128, "reserved in decode_slot_bytes");
 // 4096 x 4096, STAGED / BARRIERS: s = 64, k = 96 / 129 / 257 W = 8 41 / 42, 49 / 51, 65 / 69 us, W = 32 80 / 92, 112 / 122, 171 / 182;
 // s = 32, k = 65 W = 1 36 / 34, W = 2 39 / 39, W = 8 60 / 70, k = 129 W = 1 38 / 37, W = 2 44 / 50; signs, s = 64, k = 96 / 128
 // W = 8 36 / 33, k = 200 W = 2 / 8 / 32 29 / 26, 50 / 39, 144 / 138.
+// COUNTS: the count-normalised mean.  (As a branch of the same kernels its code cost the sum 2 to 12 %: 4096 x 4096, k = 32, W = 64
+// 61.9 -> 55.6 us, s = 32, k = 8, W = 64 101 -> 88, 16 chunks 4.4 -> 4.2.)
 enum { LISTED, STAGED, BARRIERS };
-template <int S, int THREADS, bool SIGNS, int KMODE>
+template <int S, int THREADS, bool SIGNS, int KMODE, bool COUNTS>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -56,8 +62,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     constexpr int M = S * S;
     extern __shared__ __align__(128) unsigned char smem_all[];
     const int slot = threadIdx.x / S;
-    const bool counts = a.agg == 2;
-    unsigned char *smem_raw = smem_all + (size_t)slot * decode_slot_bytes<S>(counts);
+    unsigned char *smem_raw = smem_all + (size_t)slot * decode_slot_bytes<S>(COUNTS);
     const SlotBarrier<S> sb{slot + 1};
     // One tile per slot: the aggregate S, then the row-stage output, and -- once column t has been
     // read back into registers -- the staging area of the x tile, fetched behind the second transform.
@@ -65,7 +70,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
     float *Xt = St;                                   // [S*S] (aliases St)
     DecodeWalk &walk = *reinterpret_cast<DecodeWalk *>(St + S * XS);
     DemoRecord *stage_all = reinterpret_cast<DemoRecord *>(reinterpret_cast<unsigned char *>(&walk) + 128);    // [2][STAGE_RECORDS] records of a batch of workers
-    unsigned short *Cn = reinterpret_cast<unsigned short *>(stage_all + 2 * STAGE_RECORDS);  // [S*S] senders per coordinate (agg == 2)
+    unsigned short *Cn = reinterpret_cast<unsigned short *>(stage_all + 2 * STAGE_RECORDS);  // [S*CS] senders per coordinate
 
     const int t = threadIdx.x % S;
 
@@ -129,8 +134,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
             float4 *row = reinterpret_cast<float4 *>(St + t * XS);
 #pragma unroll
             for (int v4 = 0; v4 < S / 4; ++v4) row[v4] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (counts)
-                for (int v = 0; v < S; ++v) Cn[t * S + v] = 0;
+            if constexpr (COUNTS)
+                for (int v = 0; v < S; v += 8) *reinterpret_cast<uint4 *>(Cn + t * C::CS + v) = make_uint4(0u, 0u, 0u, 0u);
         }
         // (an empty group where there is no next chunk: the waits count groups)
         auto stage_next_chunk = [&](int into) {
@@ -177,7 +182,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                     const bool mine = have && (idx >> (C::LOG2S + 5)) == (unsigned)warp;  // (false for idx >= M)
                     const int at = mine ? (int)(idx >> C::LOG2S) * XS + (int)(idx & (S - 1)) : spare;
                     St[at] += rc.val;
-                    if (counts && mine) Cn[idx] += 1;
+                    if (COUNTS && mine) Cn[(idx >> C::LOG2S) * C::CS + (idx & (S - 1))] += 1;
                 };
                 if constexpr (KMODE == STAGED) {  // a worker's records in parts of 64, the last one short
                     const int per = (k_eff + 63) >> 6;  // parts of a worker
@@ -250,7 +255,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 [&](const DemoRecord &rc) {
                     if ((unsigned)rc.idx < (unsigned)M) {
                         St[(rc.idx >> C::LOG2S) * XS + (rc.idx & (S - 1))] += rc.val;
-                        if (counts) Cn[rc.idx] += 1;
+                        if (COUNTS) Cn[(rc.idx >> C::LOG2S) * C::CS + (rc.idx & (S - 1))] += 1;
                     } else {
                         atomicMax(a.status, DEMO_DEV_PAYLOAD);
                     }
@@ -258,10 +263,16 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) decode_fast_kernel(Dem
                 [&] { sb.sync(); });
         }
         if (threadIdx.x == 0) drawn[par ^ 1u] = ticket + tickets_from((unsigned)((a.n_chunks + NCH - 1) / NCH));
-        if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0 (row t is this thread's)
-            for (int v = 0; v < S; ++v) {
-                const unsigned short n = Cn[t * S + v];
-                if (n > 1) St[t * XS + v] = St[t * XS + v] / (float)n;
+        if constexpr (COUNTS) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0 (row t is this thread's)
+#pragma unroll 1
+            for (int v = 0; v < S; v += 8) {
+                const uint4 n8 = *reinterpret_cast<const uint4 *>(Cn + t * C::CS + v);
+                if (((n8.x | n8.y | n8.z | n8.w) & 0xfffefffeu) == 0u) continue;  // at most one sender each
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const unsigned n = ((i >> 1) == 0 ? n8.x : (i >> 1) == 1 ? n8.y : (i >> 1) == 2 ? n8.z : n8.w) >> (16 * (i & 1)) & 0xffffu;
+                    if (n > 1u) St[t * XS + v + i] = St[t * XS + v + i] / (float)n;
+                }
             }
         }
         // Two inverse passes through one copy of the unrolled transform (rolled loop): pass 0 along
@@ -366,15 +377,17 @@ cudaError_t launch_decode(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t
 {
     constexpr int TH = DECODE_THREADS;
     constexpr int NCH = TH / S;
-    const size_t smem = decode_slot_bytes<S>(a.agg == 2) * NCH;
-    auto pick = [&](auto signs) {
-        constexpr bool SIGNS = decltype(signs)::value;
-        if (a.k <= 64) return launch(decode_fast_kernel<S, TH, SIGNS, LISTED>, TH, NCH, smem, dev, stream, a);
+    auto pick = [&](auto signs, auto counts) {
+        constexpr bool SIGNS = decltype(signs)::value, COUNTS = decltype(counts)::value;
+        const size_t smem = decode_slot_bytes<S>(COUNTS) * NCH;
+        if (a.k <= 64) return launch(decode_fast_kernel<S, TH, SIGNS, LISTED, COUNTS>, TH, NCH, smem, dev, stream, a);
         if constexpr (!(SIGNS && S == 64))
-            if (a.k <= STAGE_RECORDS && (S == 64 || (long long)a.W * a.k >= 256)) return launch(decode_fast_kernel<S, TH, SIGNS, STAGED>, TH, NCH, smem, dev, stream, a);
-        return launch(decode_fast_kernel<S, TH, SIGNS, BARRIERS>, TH, NCH, smem, dev, stream, a);
+            if (a.k <= STAGE_RECORDS && (S == 64 || (long long)a.W * a.k >= 256))
+                return launch(decode_fast_kernel<S, TH, SIGNS, STAGED, COUNTS>, TH, NCH, smem, dev, stream, a);
+        return launch(decode_fast_kernel<S, TH, SIGNS, BARRIERS, COUNTS>, TH, NCH, smem, dev, stream, a);
     };
-    return a.sign_ptrs != nullptr ? pick(std::true_type{}) : pick(std::false_type{});
+    if (a.agg == 2) return a.sign_ptrs != nullptr ? pick(std::true_type{}, std::true_type{}) : pick(std::false_type{}, std::true_type{});
+    return a.sign_ptrs != nullptr ? pick(std::true_type{}, std::false_type{}) : pick(std::false_type{}, std::false_type{});
 }
 
 // One CTA arms an mbarrier with a transaction count that no copy will ever satisfy and waits for it

@@ -641,8 +641,9 @@ constexpr size_t DECODE128_SMEM = (size_t)S * XSD * 4 + 128 + 2 * STAGE_RECORDS 
 // ones (in one instantiation the loop of the longer lists cost signs 4 %).
 // The upper half of the x tile comes in behind the scatter and the transforms, the lower half, already in L2, into the dead
 // coefficient tile while the upper one is updated; by 16-byte asynchronous copies, without tensor maps (kernels_fast.cu).
+// COUNTS: the count-normalised mean (an instantiation of its own, as at s = 32 / 64, where the code for it cost the sum up to 12 %).
 enum { STAGED, ROUND, ROUNDS };
-template <bool SIGNS, int KMODE>
+template <bool SIGNS, int KMODE, bool COUNTS>
 __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -660,7 +661,6 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
     const unsigned lr_bits = __float_as_uint(a.lr);
     const float decay = 1.f - a.lr * a.wd;
     const float neg_lr_scale = -a.lr * a.agg_scale;
-    const bool counts = a.agg == 2;
 
     // the records of workers w_first .. of the chunk in walk slot `which`; one copy group per call
     auto stage_batch = [&](int buf, int which, int w_first) {
@@ -713,12 +713,12 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         if (!SIGNS) {
-            if (!counts) fetch_rows(Xh, 0);
+            if (!COUNTS) fetch_rows(Xh, 0);
             const float *xr = a.x_ptrs[walk.tensor[which]] + walk.elem[which] + (size_t)(64 + (tid >> 2)) * walk.n1[which] + (tid & 3) * 32;
             prefetch_l2(xr);
         }
         for (int i = tid; i < S * XSD / 4; i += THREADS) reinterpret_cast<float4 *>(St)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (counts)
+        if constexpr (COUNTS)
             for (int i = tid; i < M / 2; i += THREADS) reinterpret_cast<unsigned *>(Cn)[i] = 0u;
         // S = sum over workers in worker order (Decompress&Aggregate)
         if constexpr (KMODE == STAGED) {
@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
             for (int w0 = 0; w0 < a.W; w0 += wb) {
                 // the records have landed (requested a chunk or a batch ago; only the rows of x are younger), the tile is cleared,
                 // the next chunk looked up, and all warps are done with the other buffer
-                if (!SIGNS && !counts && w0 == 0)
+                if (!SIGNS && !COUNTS && w0 == 0)
                     asm volatile("cp.async.wait_group 1;" ::: "memory");
                 else
                     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                         const bool mine = have && (idx >> 11) == (unsigned)warp;  // (false for idx >= M)
                         const int at = mine ? (int)(idx >> 7) * XSD + (int)(idx & 127) : spare;
                         St[at] += rc[u].val;
-                        if (counts && mine) Cn[idx] += 1;
+                        if (COUNTS && mine) Cn[idx] += 1;
                         __syncwarp();
                     }
                 }
@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
                 [&](const DemoRecord &rc) {
                     if ((unsigned)rc.idx < (unsigned)M) {
                         St[(rc.idx >> 7) * XSD + (rc.idx & 127)] += rc.val;
-                        if (counts) Cn[rc.idx] += 1;
+                        if (COUNTS) Cn[rc.idx] += 1;
                     } else {
                         atomicMax(a.status, DEMO_DEV_PAYLOAD);
                     }
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(THREADS, 2) decode_fast128_kernel(DemoDecodeAr
         }
         if (tid == 0) drawn[par ^ 1u] = ticket + tickets_from(n_chunks);
         __syncthreads();
-        if (counts) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
+        if constexpr (COUNTS) {  // Sparse Top-k Averaging: sum / number of senders, 0/0 = 0
             for (int i = tid; i < M; i += THREADS) {
                 const unsigned short n = Cn[i];
                 if (n > 1) St[(i >> 7) * XSD + (i & 127)] /= (float)n;
@@ -888,11 +888,12 @@ cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev,
     // 156 / 164, k = 128, W = 1 139 / 149, W = 8 182 / 165 us; 4096 x 4096, k = 32, W = 64 62 / 103 us, k = 65 .. 128, W = 1
     // 37.3 / 38.1, W = 4 42 / 39, signs W = 1 33.2 / 32.5, W = 4 37.4 / 32.7.
     const bool staged = a.k <= 64 || (a.k <= 128 && a.W == 1 && !a.sign_ptrs);
-    auto pick = [&](auto signs) {
-        constexpr bool SIGNS = decltype(signs)::value;
-        if (staged) return launch128(decode_fast128_kernel<SIGNS, STAGED>, DECODE128_SMEM, dev, stream, a);
-        if (a.k <= THREADS) return launch128(decode_fast128_kernel<SIGNS, ROUND>, DECODE128_SMEM, dev, stream, a);
-        return launch128(decode_fast128_kernel<SIGNS, ROUNDS>, DECODE128_SMEM, dev, stream, a);
+    auto pick = [&](auto signs, auto counts) {
+        constexpr bool SIGNS = decltype(signs)::value, COUNTS = decltype(counts)::value;
+        if (staged) return launch128(decode_fast128_kernel<SIGNS, STAGED, COUNTS>, DECODE128_SMEM, dev, stream, a);
+        if (a.k <= THREADS) return launch128(decode_fast128_kernel<SIGNS, ROUND, COUNTS>, DECODE128_SMEM, dev, stream, a);
+        return launch128(decode_fast128_kernel<SIGNS, ROUNDS, COUNTS>, DECODE128_SMEM, dev, stream, a);
     };
-    return a.sign_ptrs ? pick(std::true_type{}) : pick(std::false_type{});
+    if (a.agg == 2) return a.sign_ptrs ? pick(std::true_type{}, std::true_type{}) : pick(std::false_type{}, std::true_type{});
+    return a.sign_ptrs ? pick(std::true_type{}, std::false_type{}) : pick(std::false_type{}, std::false_type{});
 }

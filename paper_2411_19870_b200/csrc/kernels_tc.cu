@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
 {
     const StreamOrder order(a.wait_first);
     extern __shared__ unsigned char smem_raw[];
-    const bool counts = a.agg == 2;
+    constexpr bool counts = GROUPS == 3;  // the count-normalised mean: its counters leave room for three groups
     const int area = X_BYTES + (counts ? M * 2 : 0);
     const unsigned n_chunks = (unsigned)a.n_chunks, n_pairs = (n_chunks + 1u) / 2u;
     const int k_eff = a.k;

@@ -561,3 +561,13 @@ def test_chunks_of_the_first_rounds(s, grid, rounds, extra):
 
     for a, b in zip(run([n]), run(cut)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("s,k,workers", [(32, 1, 2), (32, 40, 9), (64, 1, 3), (64, 33, 17), (64, 70, 5), (64, 600, 3)])
+def test_senders_of_every_place_of_a_row(s, k, workers):
+    """Count-normalised mean: coordinates of every column sent by none, one and several workers."""
+    wl = inputs.Workload("cm", [(2 * s, 3 * s)], chunk=s, topk=k, num_workers=workers, grad_kind="normal", grad_std=0.01)
+    r = parity.Runner(wl, max_chunks=10**9, seed=k, agg=2)
+    base = [g.clone() for g in r.streams[0].next()]
+    r.step(grads=[[(b.float() + 0.2 * o.float()).to(b.dtype) for b, o in zip(base, st.next())] for st in r.streams])
+    r.close()
