@@ -57,6 +57,7 @@ class DemoError(RuntimeError):
 
 
 _lib = None
+_calls = None
 
 
 def load_library(path: Optional[str] = None) -> ctypes.CDLL:
@@ -124,6 +125,18 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     return lib
 
 
+def load_calls():
+    """The extension module of the per-step calls (csrc/calls.cpp).  Raises if it is absent."""
+    global _calls
+    if _calls is None:
+        path = os.path.join(os.path.dirname(LIB_PATH), "_calls.so")
+        if not os.path.exists(path):
+            raise RuntimeError("%s is missing: build it with `python -m paper_2411_19870_b200.build`" % path)
+        from . import _calls as module
+        _calls = module
+    return _calls
+
+
 def demo_status_string(status: int) -> str:
     return load_library().demo_status_string(int(status)).decode()
 
@@ -179,6 +192,7 @@ class DemoTransform:
     def __init__(self, shapes, *, chunk: int = 0, topk: int, beta: float, lr: float, weight_decay: float,
                  num_workers: int, grad_dtype: int = DEMO_BF16, device: int = 0, chunk_shapes=None):
         self.lib = load_library()
+        self._calls = load_calls()
         self.shapes = [tuple(int(d) for d in s) for s in shapes]
         self.chunk_shapes = None if chunk_shapes is None else [tuple(int(d) for d in s) for s in chunk_shapes]
         self.cfg = DemoConfig(beta, chunk, topk, lr, weight_decay, num_workers, grad_dtype)
@@ -210,6 +224,10 @@ class DemoTransform:
         self._payload_bytes = int(self.lib.demo_payload_bytes(self._ctx))
         self._payload_ok = set()   # (data pointer, size) of payload buffers already checked
         self._gdtype = torch.bfloat16 if grad_dtype == DEMO_BF16 else torch.float32
+        # what the calls of csrc/calls.cpp are given: entry points, context, keys of the pointer arrays
+        address = lambda f: ctypes.cast(f, ctypes.c_void_p).value  # noqa: E731
+        self._fn = {n: address(getattr(self.lib, n)) for n in ("demo_compress", "demo_decode_apply", "demo_decode_signs", "demo_apply_signs")}
+        self._keys = [(("g", w), ("m", w)) for w in range(num_workers)]
 
     # --- queries -------------------------------------------------------------------------------
     @property
@@ -262,8 +280,23 @@ class DemoTransform:
             return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
         return ctypes.c_void_p(int(getattr(stream, "cuda_stream", stream)))
 
+    @staticmethod
+    def _raw_stream(stream):
+        """The stream as csrc/calls.cpp takes it: None for the current one, else its handle."""
+        return None if stream is None else int(getattr(stream, "cuda_stream", stream))
+
     # --- the ABI calls -------------------------------------------------------------------------
+    # Tensors that lie where they were checked last go straight to the library (csrc/calls.cpp); the others, which it answers with None,
+    # are checked and their pointers noted.
     def compress(self, worker: int, grads, momentum, payload_out, stream=None) -> None:
+        if type(worker) is int and 0 <= worker < self.num_workers:
+            kg, km = self._keys[worker]
+            st = self._calls.compress(self._fn["demo_compress"], self._ctx.value or 0, self._ptr_cache, self._payload_ok, worker,
+                                      kg, grads, km, momentum, payload_out, self._raw_stream(stream))
+            if st is not None:
+                if st != 0:
+                    raise DemoError(st, "demo_compress")
+                return
         self._check_payload(payload_out, "payload_out")
         st = self.lib.demo_compress(self._ctx, worker, self._array(("g", worker), grads, (self.shapes, self._gdtype, True)),
                                     self._array(("m", worker), momentum, (self.shapes, torch.float32, True)),
@@ -272,6 +305,12 @@ class DemoTransform:
             raise DemoError(st, "demo_compress")
 
     def decode_apply(self, payloads, params, stream=None) -> None:
+        st = self._calls.decode(self._fn["demo_decode_apply"], self._ctx.value or 0, self._ptr_cache, self._payload_ok, payloads, "x", params,
+                                self._raw_stream(stream))
+        if st is not None:
+            if st != 0:
+                raise DemoError(st, "demo_decode_apply")
+            return
         self._check_payloads(payloads)
         st = self.lib.demo_decode_apply(self._ctx, self._array("p", payloads), len(payloads),
                                         self._array("x", params, (self.shapes, torch.float32, True)), self._stream(stream))
@@ -280,6 +319,12 @@ class DemoTransform:
 
     def decode_signs(self, payloads, signs_out, stream=None) -> None:
         """Parameter-server form: sign of the reconstructed momentum as int8 tensors shaped like the parameters."""
+        st = self._calls.decode(self._fn["demo_decode_signs"], self._ctx.value or 0, self._ptr_cache, self._payload_ok, payloads, "s", signs_out,
+                                self._raw_stream(stream))
+        if st is not None:
+            if st != 0:
+                raise DemoError(st, "demo_decode_signs")
+            return
         self._check_payloads(payloads)
         st = self.lib.demo_decode_signs(self._ctx, self._array("p", payloads), len(payloads),
                                         self._array("s", signs_out, (self.shapes, torch.int8, True)), self._stream(stream))
@@ -287,6 +332,11 @@ class DemoTransform:
             raise DemoError(st, "demo_decode_signs")
 
     def apply_signs(self, signs, params, stream=None) -> None:
+        st = self._calls.apply_signs(self._fn["demo_apply_signs"], self._ctx.value or 0, self._ptr_cache, signs, params, self._raw_stream(stream))
+        if st is not None:
+            if st != 0:
+                raise DemoError(st, "demo_apply_signs")
+            return
         st = self.lib.demo_apply_signs(self._ctx, self._array("s", signs, (self.shapes, torch.int8, True)),
                                        self._array("x", params, (self.shapes, torch.float32, True)), self._stream(stream))
         if st != 0:

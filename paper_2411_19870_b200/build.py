@@ -1,7 +1,8 @@
 """Build the CUDA library in-tree for sm_100a with nvcc (no JIT cache, no torch extension).
 
 ``python -m paper_2411_19870_b200.build`` or ``build_library()`` compiles every ``csrc/*.cu`` into
-``build/*.o`` and links ``libdemo_b200.so`` next to this file.  Objects are rebuilt only when a
+``build/*.o`` and links ``libdemo_b200.so`` next to this file; ``build_calls()`` compiles ``csrc/calls.cpp``, the
+extension module behind the per-step calls of ``binding.py``, into ``_calls.so``.  Objects are rebuilt only when a
 source or header is newer.
 """
 from __future__ import annotations
@@ -12,11 +13,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libdemo_b200.so")
+CALLS = os.path.join(HERE, "_calls.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 NVCC_FLAGS = [
@@ -72,5 +75,31 @@ def build_library(force: bool = False, verbose: bool = False, ptxas_info: bool =
     return LIB
 
 
+def build_calls(force: bool = False) -> str:
+    src = os.path.join(CSRC, "calls.cpp")
+    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= os.path.getmtime(src):
+        return CALLS
+    import torch
+    from torch.utils import cpp_extension
+
+    cxx = shutil.which(os.environ.get("CXX", "g++"))
+    if cxx is None:
+        raise RuntimeError("no C++ compiler: the call module cannot be built")
+    torch_lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    tmp = CALLS + ".tmp.%d" % os.getpid()
+    cmd = [cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+    for inc in cpp_extension.include_paths() + [os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]:
+        cmd += ["-isystem", inc]
+    cmd += [src, "-o", tmp, "-L" + torch_lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+        raise RuntimeError("the C++ compiler failed for " + src)
+    os.replace(tmp, CALLS)
+    return CALLS
+
+
 if __name__ == "__main__":
+    print(build_calls(force="--force" in sys.argv))
     print(build_library(force="--force" in sys.argv, verbose=True, ptxas_info="--ptxas" in sys.argv))

@@ -1,0 +1,185 @@
+// The per-step calls of binding.py without Python between the tensors and the library: a call whose tensors are where they were the last
+// time (their pointers are compared with the arrays that binding.py made and checked then) takes the current stream and enters the
+// library; anything else returns None, and binding.py takes its checked way.
+//
+// What it saves is host time, which is all that a step of small tensors costs: compress of one matrix 5.9 -> 3.9 us, of 50 matrices and 12
+// vectors (two launches) 23.9 -> 5.9, decode of the same set 16.7 -> 5.8, of 64 payloads 30.3 -> 10.3 (one attribute look-up and method call
+// per tensor and list, the comparison of two Python lists, ctypes' conversion of the arguments, the device and stream queries).
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <cstdint>
+
+namespace {
+
+// A reference that is given up at the end of the scope.
+struct Ref {
+    PyObject *p;
+    explicit Ref(PyObject *o) : p(o) {}
+    ~Ref() { Py_XDECREF(p); }
+    Ref(const Ref &) = delete;
+    Ref &operator=(const Ref &) = delete;
+    explicit operator bool() const { return p != nullptr; }
+};
+
+// data_ptr() of a tensor; false with a Python error set.  Subclasses of Tensor are asked through their own method.
+bool data_pointer(PyObject *t, std::uintptr_t *out)
+{
+    if (THPVariable_CheckExact(t)) {
+        *out = reinterpret_cast<std::uintptr_t>(THPVariable_Unpack(t).data_ptr());
+        return true;
+    }
+    Ref v(PyObject_CallMethod(t, "data_ptr", nullptr));
+    if (!v) return false;
+    *out = reinterpret_cast<std::uintptr_t>(PyLong_AsVoidPtr(v.p));
+    return !PyErr_Occurred();
+}
+
+enum class Found { error, no, yes };
+
+// The array of pointers that cache[key] = (list, array) holds, if `tensors` lie exactly there.  `hold` keeps it alive.
+struct Array {
+    Py_buffer view{};
+    ~Array()
+    {
+        if (view.obj) PyBuffer_Release(&view);
+    }
+    void **data() const { return static_cast<void **>(view.buf); }
+};
+Found lookup(PyObject *cache, PyObject *key, PyObject *tensors, Array *array)
+{
+    PyObject *hit = PyDict_GetItemWithError(cache, key);  // (borrowed; the view below keeps the array)
+    if (!hit) return PyErr_Occurred() ? Found::error : Found::no;
+    if (!PyTuple_Check(hit) || PyTuple_GET_SIZE(hit) != 2) return Found::no;
+    if (PyObject_GetBuffer(PyTuple_GET_ITEM(hit, 1), &array->view, PyBUF_SIMPLE) != 0) return Found::error;
+    if (!PyList_Check(tensors) && !PyTuple_Check(tensors)) return Found::no;  // (an iterator is left to the checked way)
+    const Py_ssize_t n = PySequence_Fast_GET_SIZE(tensors);
+    if (array->view.len != n * (Py_ssize_t)sizeof(void *)) return Found::no;
+    for (Py_ssize_t i = 0; i < n; ++i) {
+        std::uintptr_t p;
+        if (i >= PySequence_Fast_GET_SIZE(tensors)) return Found::no;  // (a subclass's data_ptr may have changed the list)
+        Ref t(Py_NewRef(PySequence_Fast_GET_ITEM(tensors, i)));
+        if (!data_pointer(t.p, &p)) return Found::error;
+        if (reinterpret_cast<std::uintptr_t>(array->data()[i]) != p) return Found::no;
+    }
+    return Found::yes;
+}
+
+// Whether (data pointer, size) of a payload is among those that were checked.
+Found payload_known(PyObject *known, PyObject *payload, std::uintptr_t *ptr)
+{
+    if (!THPVariable_CheckExact(payload)) return Found::no;
+    const at::Tensor &t = THPVariable_Unpack(payload);
+    *ptr = reinterpret_cast<std::uintptr_t>(t.data_ptr());
+    Ref key(Py_BuildValue("(KL)", (unsigned long long)*ptr, (long long)t.numel()));
+    if (!key) return Found::error;
+    const int in = PySet_Contains(known, key.p);
+    return in < 0 ? Found::error : in ? Found::yes : Found::no;
+}
+
+bool stream_of(PyObject *stream, void **out)
+{
+    if (stream == Py_None) {
+        *out = c10::cuda::getCurrentCUDAStream().stream();
+        return true;
+    }
+    *out = PyLong_AsVoidPtr(stream);
+    return !PyErr_Occurred();
+}
+
+PyObject *slow(Found f)
+{
+    if (f == Found::error) return nullptr;
+    Py_RETURN_NONE;
+}
+
+using CompressFn = int (*)(void *, std::int32_t, void **, void **, void *, void *);
+using DecodeFn = int (*)(void *, void **, std::int32_t, void **, void *);
+using ApplyFn = int (*)(void *, void **, void **, void *);
+
+// compress(function, context, cache, known payloads, worker, key of grads, grads, key of momentum, momentum, payload, stream or None)
+PyObject *compress(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    if (n != 11) return PyErr_Format(PyExc_TypeError, "compress: 11 arguments");
+    void *fn = PyLong_AsVoidPtr(a[0]), *ctx = PyLong_AsVoidPtr(a[1]), *stream = nullptr;
+    const long worker = PyLong_AsLong(a[4]);
+    if (PyErr_Occurred()) return nullptr;
+    std::uintptr_t payload = 0;
+    Array g, m;
+    Found f = payload_known(a[3], a[9], &payload);
+    if (f == Found::yes) f = lookup(a[2], a[5], a[6], &g);
+    if (f == Found::yes) f = lookup(a[2], a[7], a[8], &m);
+    if (f != Found::yes) return slow(f);
+    if (!stream_of(a[10], &stream)) return nullptr;
+    int st;
+    Py_BEGIN_ALLOW_THREADS
+    st = reinterpret_cast<CompressFn>(fn)(ctx, (std::int32_t)worker, g.data(), m.data(), reinterpret_cast<void *>(payload), stream);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(st);
+    END_HANDLE_TH_ERRORS
+}
+
+// decode(function, context, cache, known payloads, payloads, key of tensors, tensors, stream or None)
+PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    if (n != 8) return PyErr_Format(PyExc_TypeError, "decode: 8 arguments");
+    void *fn = PyLong_AsVoidPtr(a[0]), *ctx = PyLong_AsVoidPtr(a[1]), *stream = nullptr;
+    if (PyErr_Occurred()) return nullptr;
+    static PyObject *const key_p = PyUnicode_InternFromString("p");
+    if (!key_p) return nullptr;
+    Array p, x;
+    Found f = lookup(a[2], key_p, a[4], &p);
+    for (Py_ssize_t i = 0; f == Found::yes && i < PySequence_Fast_GET_SIZE(a[4]); ++i) {
+        std::uintptr_t ptr;
+        f = payload_known(a[3], PySequence_Fast_GET_ITEM(a[4], i), &ptr);
+    }
+    if (f == Found::yes) f = lookup(a[2], a[5], a[6], &x);
+    if (f != Found::yes) return slow(f);
+    if (!stream_of(a[7], &stream)) return nullptr;
+    const std::int32_t count = (std::int32_t)(p.view.len / (Py_ssize_t)sizeof(void *));
+    int st;
+    Py_BEGIN_ALLOW_THREADS
+    st = reinterpret_cast<DecodeFn>(fn)(ctx, p.data(), count, x.data(), stream);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(st);
+    END_HANDLE_TH_ERRORS
+}
+
+// apply_signs(function, context, cache, signs, params, stream or None)
+PyObject *apply_signs(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    if (n != 6) return PyErr_Format(PyExc_TypeError, "apply_signs: 6 arguments");
+    void *fn = PyLong_AsVoidPtr(a[0]), *ctx = PyLong_AsVoidPtr(a[1]), *stream = nullptr;
+    if (PyErr_Occurred()) return nullptr;
+    static PyObject *const key_s = PyUnicode_InternFromString("s"), *const key_x = PyUnicode_InternFromString("x");
+    if (!key_s || !key_x) return nullptr;
+    Array s, x;
+    Found f = lookup(a[2], key_s, a[3], &s);
+    if (f == Found::yes) f = lookup(a[2], key_x, a[4], &x);
+    if (f != Found::yes) return slow(f);
+    if (!stream_of(a[5], &stream)) return nullptr;
+    int st;
+    Py_BEGIN_ALLOW_THREADS
+    st = reinterpret_cast<ApplyFn>(fn)(ctx, s.data(), x.data(), stream);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(st);
+    END_HANDLE_TH_ERRORS
+}
+
+PyMethodDef methods[] = {
+    {"compress", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(compress)), METH_FASTCALL, nullptr},
+    {"decode", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(decode)), METH_FASTCALL, nullptr},
+    {"apply_signs", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(apply_signs)), METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__calls() { return PyModule_Create(&module); }

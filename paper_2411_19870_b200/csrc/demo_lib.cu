@@ -98,15 +98,16 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 struct DeviceGuard {
     int prev = -1;
-    bool ok = false;
+    bool ok = false, changed = false;
     explicit DeviceGuard(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) return;
-        ok = (prev == dev) || (cudaSetDevice(dev) == cudaSuccess);
+        changed = prev != dev;
+        ok = !changed || cudaSetDevice(dev) == cudaSuccess;
     }
     ~DeviceGuard()
     {
-        if (ok && prev >= 0) cudaSetDevice(prev);
+        if (ok && changed) cudaSetDevice(prev);
     }
 };
 
