@@ -36,7 +36,7 @@ struct DemoCompressArgs {
     const void *const *g_ptrs;  // device array indexed by DemoTensorEntry::tensor
     float *const *m_ptrs;       // device array
     DemoRecord *payload;        // device, whole payload of this worker
-    const float *C;             // device, s x s orthonormal DCT-II, C[u*s + n]
+    const float *C;             // device, s x s orthonormal DCT-II, C[u*s + n], and behind it its transpose
     float beta;
     float alpha;    // momentum-subtraction coefficient: m <- B - alpha * IDCT(kept)
     int grad_bf16;  // 1: gradients are bf16, 0: fp32
@@ -108,8 +108,10 @@ cudaError_t demo_launch_decode_tc(const DemoDecodeArgs &a, DemoLaunch &dev, cuda
 cudaError_t demo_launch_wait_selftest(int *status, long long limit_cycles, cudaStream_t stream);
 
 // Gram-Schmidt process on the rows of the s x s matrix `gauss` (device, fp32) in fp64; writes the
-// orthonormal rows to `basis` (device, fp32) and 1 to *flag when a row has no component left.
+// orthonormal rows to `basis` (device, fp32, the transpose behind them) and 1 to *flag when a row has no component left.
 cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *verdict, int s, cudaStream_t stream);
+// basis[s*s .. 2 s*s) <- the transpose of basis[0 .. s*s) (kernels_generic.cu; the launcher above writes both)
+cudaError_t demo_launch_transpose_basis(float *basis, int s, cudaStream_t stream);
 
 // ---- tensors of any order with rectangular chunks (appendix of the paper: blocking operator and
 // multilinear product; kernels_nd.cu) ---------------------------------------------------------------

@@ -47,7 +47,7 @@ struct demo_ctx {
 
     // caller-supplied orthonormal basis (rows = basis vectors); while `custom_basis` is set every
     // tensor goes through the dense-transform kernels, which read the basis from memory
-    float *d_P = nullptr;      // [s*s]
+    float *d_P = nullptr;      // [2][s*s]: the matrix and its transpose, as in d_C
     float *h_gauss = nullptr;  // pinned: [s*s] Gaussian matrix and the verdict on it; from the first demo_set_basis_gaussian
     bool custom_basis = false;
     bool momentum_dct = false;  // demo_set_momentum_domain(DEMO_MOMENTUM_DCT)
@@ -286,13 +286,13 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
 
     // orthonormal DCT-II basis, built in fp64 and rounded once to fp32:
     // C[u][n] = a_u cos(pi (2n+1) u / (2s)), a_0 = sqrt(1/s), a_u = sqrt(2/s)
-    std::vector<float> C((size_t)s * s);
+    std::vector<float> C(2 * (size_t)s * s);  // (and behind it the transpose)
     {
         const double pi = 3.141592653589793238462643383279502884;
         for (int u = 0; u < s; ++u)
             for (int n = 0; n < s; ++n) {
                 const double a = (u == 0) ? std::sqrt(1.0 / s) : std::sqrt(2.0 / s);
-                C[(size_t)u * s + n] = (float)(a * std::cos(pi * (2.0 * n + 1.0) * u / (2.0 * s)));
+                C[(size_t)u * s + n] = C[(size_t)(s + n) * s + u] = (float)(a * std::cos(pi * (2.0 * n + 1.0) * u / (2.0 * s)));
             }
     }
 
@@ -1003,7 +1003,8 @@ demo_status demo_set_basis(demo_ctx *ctx, const float *basis_host, void *cuda_st
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return DEMO_ERR_CUDA;
     if (cudaMemcpyAsync(ctx->d_P, basis_host, sizeof(float) * (size_t)s * s, cudaMemcpyHostToDevice,
-                        static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
+                        static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess ||
+        demo_launch_transpose_basis(ctx->d_P, s, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
         cudaGetLastError();
         return DEMO_ERR_CUDA;
     }

@@ -408,7 +408,13 @@ __global__ void __launch_bounds__(GS_LANES *GS_LANES *EPL, 1) gram_schmidt_kerne
     if (bad) return;
     const double inv = 1.0 / sqrt(product(a, a));
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) basis[r * N + col(e)] = (float)(a[e] * inv);
+    for (int e = 0; e < EPL; ++e) basis[r * N + col(e)] = basis[N * N + col(e) * N + r] = (float)(a[e] * inv);
+}
+
+__global__ void transpose_basis_kernel(float *basis, int s)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < s * s) basis[s * s + i] = basis[i % s * s + i / s];
 }
 
 // `gauss` and `verdict` are pinned host memory.
@@ -422,6 +428,12 @@ cudaError_t demo_launch_gram_schmidt(const float *gauss, float *basis, int *verd
         case 128: gram_schmidt_kernel<16><<<1, 1024, 0, stream>>>(gauss, basis, verdict); break;
         default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t demo_launch_transpose_basis(float *basis, int s, cudaStream_t stream)
+{
+    transpose_basis_kernel<<<(s * s + 255) / 256, 256, 0, stream>>>(basis, s);
     return cudaGetLastError();
 }
 

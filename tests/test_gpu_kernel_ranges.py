@@ -571,3 +571,17 @@ def test_senders_of_every_place_of_a_row(s, k, workers):
     base = [g.clone() for g in r.streams[0].next()]
     r.step(grads=[[(b.float() + 0.2 * o.float()).to(b.dtype) for b, o in zip(base, st.next())] for st in r.streams])
     r.close()
+
+
+@pytest.mark.parametrize("s", [8, 16, 32, 64, 128])
+def test_vectors_under_a_callers_basis(s):
+    """1-D tensors read the basis by columns on the way there and by rows on the way back: a matrix that is not symmetric, set twice."""
+    wl = inputs.Workload("vb", [(3 * s,), (s, 2 * s), (s,)], chunk=s, topk=max(1, s // 4), num_workers=2, grad_kind="normal", grad_std=0.01)
+    r = parity.Runner(wl, max_chunks=10**9)
+    for seed in (1, 2):
+        q = np.linalg.qr(np.random.default_rng(seed).standard_normal((s, s)))[0]
+        r.set_basis(basis=np.ascontiguousarray(q, dtype=np.float32))
+        r.step()
+    r.set_basis()
+    r.step()
+    r.close()
