@@ -47,6 +47,7 @@ struct DemoCompressArgs {
     const void *tmap_g;
     int wait_first = 1;  // see StreamOrder (launch.cuh)
     DemoTickets *tickets = nullptr;  // device; the counter of this kernel's chunks
+    int late_lookup = 0;  // s = 64: the first chunk is looked up behind the tensor-memory allocation (kernels_fast64.cu)
     // 1: the momentum tensors hold the chunk-wise DCT of the momentum (tiles transposed); only the s = 64 tile
     // kernel with tensor maps implements it
     int momentum_dct = 0;
