@@ -341,17 +341,16 @@ cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, DemoLaunc
 
 // =================================================================================================
 // Random orthonormal basis (Section 4.2, "Choice of Linear Projections"): Gram-Schmidt process on the
-// rows of a Gaussian matrix, in fp64, one CTA.  Right-looking order: once row j is final its component
-// is removed from every later row, so each row loses its components along rows 0..j-1 one after the
-// other -- the same operations as the row-by-row statement of the process.
+// rows of a Gaussian matrix, in fp64, one CTA.  Right-looking order by blocks of four rows: the warp that holds them makes them
+// orthogonal among themselves, one after the other, then every later row loses its components along the four, which are orthogonal to
+// each other, at once.
 //
-// s dependent steps, so the latency of a step is all there is.  Eight threads keep a row in registers; the owners of
-// row j + 1 publish it, with the reciprocal of its squared length, once it has lost its component along row j: one barrier
-// per step, products by three-level reductions, one division per step in the whole CTA (fp64 arithmetic is narrow: with
-// the length formed by every row the step took 1.4 times as long).  The matrix is read from and the verdict written to
-// pinned host memory, the active basis only replaced when the verdict is good: a call is one launch and one synchronisation.
-// (One call, s = 8 / 32 / 64 / 128: 48 / 68 / 123 / 292 us with rows in shared memory, two barriers per step and four
-// copies; 20 / 29 / 47 / 215 us now.)
+// s dependent steps, so the latency of a step is all there is.  Eight threads keep a row in registers, a warp a block: inside it a step is
+// a row published in shared memory and two three-level reductions side by side, without a barrier; one barrier per block, one division per
+// step in the whole CTA (fp64 arithmetic is narrow).  At s = 128 the registers hold one published row at a time.  The matrix is read from and
+// the verdict written to pinned host memory, the active basis only replaced when the verdict is good: a call is one launch and one
+// synchronisation.  (One call, s = 64: 123 us with rows in shared memory, two barriers per step and four copies, 44.6 with a barrier per
+// row, 40.9 now.)
 // =================================================================================================
 constexpr int GS_LANES = 8;  // threads per row
 
@@ -360,53 +359,79 @@ __global__ void __launch_bounds__(GS_LANES *GS_LANES *EPL, 1) gram_schmidt_kerne
                                                                                float *__restrict__ basis, int *verdict)
 {
     constexpr int N = GS_LANES * EPL;  // rows = columns
-    __shared__ __align__(16) double pub[2][N];  // row j and 1 / its squared length, 0 when nothing is left of it
-    __shared__ double pub_inv[2];
-    const int r = threadIdx.x / GS_LANES, l = threadIdx.x % GS_LANES;
-    const int last_of_warp = r | (32 / GS_LANES - 1);
+    constexpr int R = 32 / GS_LANES;   // rows of a warp, a block
+    __shared__ __align__(16) double pub[2][R][N];  // the rows of a block and 1 / their squared lengths, 0 when nothing is left of one
+    __shared__ double pub_inv[2][R];
+    const int r = threadIdx.x / GS_LANES, l = threadIdx.x % GS_LANES, warp = threadIdx.x / 32, own = r % R;
     constexpr int V = EPL > 1 ? 2 : 1;  // consecutive elements of a thread
     auto col = [&](int e) { return (e / V) * (V * GS_LANES) + V * l + e % V; };
     double a[EPL];
 #pragma unroll
     for (int e = 0; e < EPL; ++e) a[e] = (double)gauss[r * N + col(e)];
-    auto product = [&](const double (&u)[EPL], const double (&v)[EPL]) {
+    // product of u with a published row, or of the row with itself; all threads of the eight get it
+    auto along = [&](const double *u, const double *row) {
         double acc[2] = {0.0, 0.0};
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[e & 1] = fma(u[e], v[e], acc[e & 1]);
+        for (int e = 0; e < EPL; ++e) {
+            const double p = row[col(e)];
+            acc[e & 1] = fma(u ? u[e] : p, p, acc[e & 1]);
+        }
         double sum = acc[0] + acc[1];
 #pragma unroll
         for (int d = GS_LANES / 2; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
         return sum;
     };
-    const double scale = product(a, a);  // squared length of the input row
-    auto publish = [&](int j, double len2) {
+    auto length2 = [&]() {
+        double acc[2] = {0.0, 0.0};
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) pub[j & 1][col(e)] = a[e];
-        if (l == 0) pub_inv[j & 1] = len2 > 1e-24 * scale ? 1.0 / len2 : 0.0;
+        for (int e = 0; e < EPL; ++e) acc[e & 1] = fma(a[e], a[e], acc[e & 1]);
+        double sum = acc[0] + acc[1];
+#pragma unroll
+        for (int d = GS_LANES / 2; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        return sum;
     };
-    if (r == 0) publish(0, scale);
-    __syncthreads();
+    const double scale = length2();  // squared length of the input row
     bool bad = false;
-    for (int j = 0; j < N && !bad; ++j) {
-        const double inv = pub_inv[j & 1];
-        bad = inv == 0.0;
-        if (last_of_warp > j) {
-            double p[EPL];
+    for (int b = 0; b < N / R && !bad; ++b) {
+        if (warp == b) {  // this warp's rows among themselves, one after the other, without a barrier
+#pragma unroll 1
+            for (int i = 0; i < R; ++i) {
+                const double *row = pub[b & 1][i];
+                if (own == i) {
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) p[e] = pub[j & 1][col(e)];
-            const double c = product(a, p) * (r > j ? inv : 0.0);
+                    for (int e = 0; e < EPL; ++e) pub[b & 1][i][col(e)] = a[e];
+                }
+                __syncwarp();
+                const double len2 = along(nullptr, row), dot = along(a, row), scale_i = __shfl_sync(0xffffffffu, scale, i * GS_LANES);
+                const double inv = len2 > 1e-24 * scale_i ? 1.0 / len2 : 0.0;
+                if (own == i && l == 0) pub_inv[b & 1][i] = inv;
+                const double c = own > i ? dot * inv : 0.0;
+                if (EPL > 8) asm volatile("" ::: "memory");
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) a[e] = fma(-c, p[e], a[e]);
-            if (last_of_warp / (32 / GS_LANES) == (j + 1) / (32 / GS_LANES)) {  // the warp that owns row j + 1
-                const double len2 = product(a, a);
-                if (r == j + 1) publish(j + 1, len2);
+                for (int e = 0; e < EPL; ++e) a[e] = fma(-c, row[col(e)], a[e]);
             }
         }
         __syncthreads();
+#pragma unroll
+        for (int i = 0; i < R; ++i) bad = bad || pub_inv[b & 1][i] == 0.0;
+        if (warp > b) {  // the block's rows are orthogonal to each other: their parts are taken off together
+            constexpr int G = EPL > 8 ? 1 : R;  // (s = 128: one after the other, there are 64 registers)
+#pragma unroll 1
+            for (int i0 = 0; i0 < R; i0 += G) {
+                double c[G];
+#pragma unroll
+                for (int i = 0; i < G; ++i) c[i] = along(a, pub[b & 1][i0 + i]) * pub_inv[b & 1][i0 + i];
+                if (G == 1) asm volatile("" ::: "memory");  // (the row is read again rather than kept)
+#pragma unroll
+                for (int i = 0; i < G; ++i)
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) a[e] = fma(-c[i], pub[b & 1][i0 + i][col(e)], a[e]);
+            }
+        }
     }
     if (threadIdx.x == 0) *verdict = bad;
     if (bad) return;
-    const double inv = 1.0 / sqrt(product(a, a));
+    const double inv = 1.0 / sqrt(length2());
 #pragma unroll
     for (int e = 0; e < EPL; ++e) basis[r * N + col(e)] = basis[N * N + col(e) * N + r] = (float)(a[e] * inv);
 }
