@@ -137,6 +137,8 @@ struct DemoNdEntry {
     int tail;                        // > 0: the last two axes are both of this extent and transformed together
     int row;                         // elements that are contiguous both in the tensor and in the tile
     unsigned inv_row;                // ceil(2^32 / row) for row > 1, else 0
+    int quads;                       // 1: rows are whole 16-byte pieces of the tensor, 2: and of the tile
+    unsigned inv_row4;               // ceil(2^32 / (row / 4)) for row > 4, else 0 (quads only)
     int row_table;                   // 1: the chunk's rows are few and their offsets fit 32 bits
     int threads;                     // CTA size this chunk would choose
     int layout;                      // same number: same strides in the tensor and in the tile

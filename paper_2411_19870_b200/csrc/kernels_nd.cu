@@ -15,7 +15,10 @@
 //     constant stride apart; the padding is always zero, so that sweeps over the tile run over plain memory, 16 bytes at a
 //     time;
 //   * global offsets come from a table of the chunk's contiguous rows, not from four divisions per element, and the loads
-//     of eight elements per thread are issued together;
+//     of eight elements per thread -- of sixteen, in quads, where the rows are whole 16-byte pieces -- are issued together; the next
+//     chunk's rows are on their way to L2 during the selection;
+//   * addresses along a line are byte offsets, one instruction each, and on a last axis of whole quads four elements one access;
+//   * the first axis of the inverse is transformed only along the lines that hold kept coefficients;
 //   * top-k: the k-th largest of the threads' maxima (from a histogram relative to the largest) bounds the k-th coefficient;
 //     the few dozen to few hundred coefficients above it are listed, one warp finds the k-th among them, and the kept ones
 //     are put in index order by counting or, where much of a chunk is kept, by going over the tile; radix select only when the
@@ -23,7 +26,8 @@
 // Measured (one call, bf16 gradients, k = 32; dense contractions on every axis with radix select -> this): four
 // 512 x 512 x 3 x 3 weights in 32 x 32 x 3 x 3 chunks (9.4 M parameters) compress 381 -> 115 us, decode 219 -> 63;
 // 7511 x 512 in 29 x 64: 243 -> 83 / 122 -> 36; 8192 x 8192 in 32 x 128: 2424 -> 1050 / 1155 -> 379; in 16 x 32 (k = 4):
-// 3254 -> 1017 / 1509 -> 409.
+// 3254 -> 1017 / 1509 -> 409.  Quads, byte offsets, L2 ahead and listed lines: in 16 x 32 again 988 -> 882 us, 1024 x 1024 20.5 -> 17.6;
+// a set of both kinds (13 M parameters) compress 188 -> 176, decode 80 -> 77.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -113,11 +117,16 @@ struct Shared {
     DemoNdEntry e[2];  // current and next chunk, looked up by one thread a chunk ahead
     size_t base[2];
     unsigned ticket, hi, n, n_kept, bound, thr, need_eq, n_eq, state[2], warp_tot[12];
-    unsigned hist[256], fine[256];
+    int n_list;                    // lines in the list, -1: none was made
+    unsigned hist[256], fine[256];  // then, together, a bit per line of the first axis
     alignas(16) uint2 cand[CAND];  // candidates (value bits, tile position) in no particular order
+    __device__ __forceinline__ unsigned *bits();  // both histograms as one bit map
+    __device__ __forceinline__ unsigned *list() { return reinterpret_cast<unsigned *>(cand); }  // tile positions; the candidates are dead
     uint4 kept[CAND / 2];          // the kept ones, two per entry; decode: with cand, two batches of records
 };
 extern __shared__ __align__(16) unsigned char smem_raw[];
+static_assert(offsetof(Shared, fine) == offsetof(Shared, hist) + 256 * sizeof(unsigned), "one bit map");
+__device__ __forceinline__ unsigned *Shared::bits() { return reinterpret_cast<unsigned *>(smem_raw + offsetof(Shared, hist)); }
 __device__ __forceinline__ Shared *shared() { return reinterpret_cast<Shared *>(smem_raw); }
 struct View {
     uint2 *rows;  // (offset in the tensor, offset in the tile) of every row
@@ -231,11 +240,82 @@ __device__ __forceinline__ void for_elements(const View &v, const DemoNdEntry &e
         walk(std::false_type{});
 }
 
+// The same by quads of four neighbouring elements (e.quads): load(j, offset), then use(j, first index, offset, tile position).
+template <int U, class Load, class Use>
+__device__ __forceinline__ void for_quads(const View &v, const DemoNdEntry &e, Load load, Use use)
+{
+    const int n = e.M >> 2, T = blockDim.x;
+    const unsigned row = (unsigned)e.row >> 2, inv_row = e.inv_row4;
+    for (int i0 = threadIdx.x; i0 < n; i0 += U * T) {
+        unsigned g[U];
+        int t[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const int i = min(i0 + j * T, n - 1);
+            const unsigned r = inv_row ? __umulhi((unsigned)i, inv_row) : (unsigned)i;
+            const unsigned d = 4u * ((unsigned)i - r * row);
+            const uint2 o = v.rows[r];
+            g[j] = o.x + d;
+            t[j] = (int)(o.y + d);
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) load(j, g[j]);
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (i0 + j * T < n) use(j, 4 * (i0 + j * T), g[j], t[j]);
+    }
+}
+// Four elements of the tile: in one access where its rows allow, else in four, whose order turns with the thread, so that a warp's 32
+// neighbouring quads do not meet in eight banks.
+__device__ __forceinline__ float4 turned(float4 f, int r)  // its element j is element (j + r) mod 4 of f
+{
+    if (r & 1) f = make_float4(f.y, f.z, f.w, f.x);
+    if (r & 2) f = make_float4(f.z, f.w, f.x, f.y);
+    return f;
+}
+__device__ __forceinline__ float4 tile_quad(const float *tile, int t, bool whole)
+{
+    if (whole) return *reinterpret_cast<const float4 *>(tile + t);
+    const int r = threadIdx.x >> 3 & 3;
+    const float *q = tile + t;
+    return turned(make_float4(q[r], q[(r + 1) & 3], q[(r + 2) & 3], q[(r + 3) & 3]), (4 - r) & 3);
+}
+__device__ __forceinline__ void set_tile_quad(float *tile, int t, bool whole, const float4 &f)
+{
+    if (whole) {
+        *reinterpret_cast<float4 *>(tile + t) = f;
+    } else {
+        const int r = threadIdx.x >> 3 & 3;
+        const float4 v = turned(f, r);
+        float *q = tile + t;
+        q[r] = v.x;
+        q[(r + 1) & 3] = v.y;
+        q[(r + 2) & 3] = v.z;
+        q[(r + 3) & 3] = v.w;
+    }
+}
+__device__ __forceinline__ float4 grad_quad(const float *g) { return *reinterpret_cast<const float4 *>(g); }
+__device__ __forceinline__ uint2 grad_quad(const __nv_bfloat16 *g) { return *reinterpret_cast<const uint2 *>(g); }
+__device__ __forceinline__ float4 grad_floats(const float4 &v) { return v; }
+__device__ __forceinline__ float4 grad_floats(const uint2 &v)
+{   // (bf16 is the upper half of a float)
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                       __uint_as_float(v.y & 0xffff0000u));
+}
+
 // ---- one axis of the multilinear product ------------------------------------------------------------
 // Every extent is a function of its own (not inlined: dozens of register-resident bodies in one kernel cost each other
 // registers).  They get the byte offset of the tile and the slot of the entry, so that the accesses stay shared-memory
 // accesses.
 __device__ __forceinline__ float *tile_at(unsigned off) { return reinterpret_cast<float *>(smem_raw + off); }
+// A line by the byte offsets of its first element and between elements: one instruction per address (as floats, an index
+// and a shift each).
+struct Line {
+    unsigned at, step;
+    __device__ __forceinline__ Line(unsigned tile, int first, int p) : at(tile + 4u * (unsigned)first), step(4u * (unsigned)p) {}
+    __device__ __forceinline__ float &operator[](int n) const { return *reinterpret_cast<float *>(smem_raw + at + (unsigned)n * step); }
+    __device__ __forceinline__ float4 &quad(int n) const { return *reinterpret_cast<float4 *>(smem_raw + at + 16u * (unsigned)n); }
+};
 __device__ __forceinline__ unsigned tile_offset(const float *X)
 {
     return (unsigned)(reinterpret_cast<const unsigned char *>(X) - smem_raw);
@@ -277,36 +357,96 @@ __device__ __forceinline__ void line_transform(float (&x)[S])
         else
             fdct::dct2_ortho_dense4<S>(x);
     } else {
+        // even outputs from x[n] + x[S-1-n], odd ones from x[n] - x[S-1-n]: half the products.  (Errors against 64 bits, 5 / 6 / 7 points a
+        // side, folded / plain: 8.5 / 7.8 / 6.8e-8 and 8.5 / 8.0 / 7.1e-8; 3 points 7.5 and 7.3e-8: those stay plain.)
+        constexpr int H = S / 2;
         float y[S];
-        fdct::static_for<0, S>([&](auto uu) {
-            constexpr int u = decltype(uu)::value;
-            float acc = 0.f;
-            fdct::static_for<0, S>([&](auto nn) {
-                constexpr int n = decltype(nn)::value;
-                constexpr float c = (float)(INV ? dct_entry<S>(n, u) : dct_entry<S>(u, n));
-                acc = n == 0 ? c * x[0] : fmaf(c, x[n], acc);
+        if constexpr (S == 3) {
+            fdct::static_for<0, S>([&](auto uu) {
+                constexpr int u = decltype(uu)::value;
+                float acc = 0.f;
+                fdct::static_for<0, S>([&](auto nn) {
+                    constexpr int n = decltype(nn)::value;
+                    constexpr float c = (float)(INV ? dct_entry<S>(n, u) : dct_entry<S>(u, n));
+                    acc = n == 0 ? c * x[0] : fmaf(c, x[n], acc);
+                });
+                y[u] = acc;
             });
-            y[u] = acc;
-        });
+        } else if constexpr (!INV) {
+            float u[H + 1], v[H];
+            fdct::static_for<0, H>([&](auto nn) {
+                constexpr int n = decltype(nn)::value;
+                u[n] = x[n] + x[S - 1 - n];
+                v[n] = x[n] - x[S - 1 - n];
+            });
+            u[H] = x[H];  // (odd S: the middle; even S: not used)
+            fdct::static_for<0, S>([&](auto uu) {
+                constexpr int k = decltype(uu)::value, terms = (k & 1) ? H : (S + 1) / 2;
+                float acc = 0.f;
+                fdct::static_for<0, terms>([&](auto nn) {
+                    constexpr int n = decltype(nn)::value;
+                    constexpr float c = (float)dct_entry<S>(k, n);
+                    const float t = (k & 1) ? v[n] : u[n];
+                    acc = n == 0 ? c * t : fmaf(c, t, acc);
+                });
+                y[k] = acc;
+            });
+        } else {
+            fdct::static_for<0, (S + 1) / 2>([&](auto nn) {
+                constexpr int n = decltype(nn)::value;
+                float ev = 0.f, od = 0.f;
+                fdct::static_for<0, S>([&](auto uu) {
+                    constexpr int k = decltype(uu)::value;
+                    constexpr float c = (float)dct_entry<S>(k, n);
+                    if constexpr (k & 1)
+                        od = k == 1 ? c * x[1] : fmaf(c, x[k], od);
+                    else
+                        ev = k == 0 ? c * x[0] : fmaf(c, x[k], ev);
+                });
+                if constexpr (2 * n + 1 == S) {
+                    y[n] = ev;
+                } else {
+                    y[n] = ev + od;
+                    y[S - 1 - n] = ev - od;
+                }
+            });
+        }
 #pragma unroll
         for (int n = 0; n < S; ++n) x[n] = y[n];
     }
 }
 
-template <int S, bool INV>
-__device__ __noinline__ void lines_whole(unsigned tile, int slot, int a)
+// QUADS: the last axis, its lines in whole quads of the tile.  `list`: only the lines that start at these tile positions.
+template <int S, bool INV, bool QUADS>
+__device__ __noinline__ void lines_whole(unsigned tile, int slot, int a, int n_list)
 {
-    float *X = tile_at(tile);
-    const DemoNdEntry &e = shared()->e[slot];
-    const int lines = e.M / S, p = e.p[a];
+    Shared *s = shared();
+    const DemoNdEntry &e = s->e[slot];
+    const int lines = n_list >= 0 ? n_list : e.M / S, p = e.p[a];
     for (int L = threadIdx.x; L < lines; L += blockDim.x) {
-        float *q = X + line_base(e, a, a, L);
+        const Line q(tile, n_list >= 0 ? (int)s->list()[L] : line_base(e, a, a, L), p);
         float x[S];
+        if constexpr (QUADS) {
 #pragma unroll
-        for (int n = 0; n < S; ++n) x[n] = q[n * p];
+            for (int n = 0; n < S / 4; ++n) {
+                const float4 f = q.quad(n);
+                x[4 * n] = f.x;
+                x[4 * n + 1] = f.y;
+                x[4 * n + 2] = f.z;
+                x[4 * n + 3] = f.w;
+            }
+        } else {
+#pragma unroll
+            for (int n = 0; n < S; ++n) x[n] = q[n];
+        }
         line_transform<S, INV>(x);
+        if constexpr (QUADS) {
 #pragma unroll
-        for (int n = 0; n < S; ++n) q[n * p] = x[n];
+            for (int n = 0; n < S / 4; ++n) q.quad(n) = make_float4(x[4 * n], x[4 * n + 1], x[4 * n + 2], x[4 * n + 3]);
+        } else {
+#pragma unroll
+            for (int n = 0; n < S; ++n) q[n] = x[n];
+        }
     }
 }
 
@@ -343,7 +483,6 @@ __device__ __noinline__ void lines_tail(unsigned tile, int slot)
 template <int H, bool INV>
 __device__ __noinline__ void lines_split(unsigned tile, int slot, int a)
 {
-    float *X = tile_at(tile);
     const DemoNdEntry &e = shared()->e[slot];
     using SC = fdct::ScaleOrtho<2 * H>;
     constexpr float DC = (float)fdct::c_sqrt(0.5);
@@ -352,13 +491,13 @@ __device__ __noinline__ void lines_split(unsigned tile, int slot, int a)
     const int l0 = (threadIdx.x >> 6) * 32 + (threadIdx.x & 31), per_round = blockDim.x >> 1;
     for (int r0 = 0; r0 < lines; r0 += per_round) {
         const bool active = r0 + l0 < lines;
-        float *q = X + (active ? line_base(e, a, a, r0 + l0) : 0);
+        const Line q(tile, active ? line_base(e, a, a, r0 + l0) : 0, p);
         float x[H], y[H];
         if (active) {
             if constexpr (!INV) {
 #pragma unroll
                 for (int n = 0; n < H; ++n) {
-                    const float lo = q[n * p], hi = q[(2 * H - 1 - n) * p];
+                    const float lo = q[n], hi = q[2 * H - 1 - n];
                     x[n] = h ? lo - hi : lo + hi;
                 }
                 if (h == 0) {
@@ -369,7 +508,7 @@ __device__ __noinline__ void lines_split(unsigned tile, int slot, int a)
                 }
             } else {
 #pragma unroll
-                for (int n = 0; n < H; ++n) x[n] = q[(2 * n + h) * p];
+                for (int n = 0; n < H; ++n) x[n] = q[2 * n + h];
                 if (h == 0) {
                     x[0] *= DC;
                     fdct::dct3_dense4<H, SC>(x, y);
@@ -382,14 +521,14 @@ __device__ __noinline__ void lines_split(unsigned tile, int slot, int a)
         if (active) {
             if constexpr (!INV) {
 #pragma unroll
-                for (int n = 0; n < H; ++n) q[(2 * n + h) * p] = y[n];
+                for (int n = 0; n < H; ++n) q[2 * n + h] = y[n];
             } else {
                 if (h == 0) {
 #pragma unroll
-                    for (int n = 0; n < H; ++n) q[n * p] = y[n];
+                    for (int n = 0; n < H; ++n) q[n] = y[n];
                 } else {
 #pragma unroll
-                    for (int n = 0; n < H; ++n) q[(2 * H - 1 - n) * p] = y[n];
+                    for (int n = 0; n < H; ++n) q[2 * H - 1 - n] = y[n];
                 }
             }
         }
@@ -399,9 +538,9 @@ __device__ __noinline__ void lines_split(unsigned tile, int slot, int a)
 #pragma unroll
                 for (int i = 0; i < H / 2; ++i) {
                     const int n = i + h * (H / 2);
-                    const float ev = q[n * p], od = q[(2 * H - 1 - n) * p];
-                    q[n * p] = ev + od;
-                    q[(2 * H - 1 - n) * p] = ev - od;
+                    const float ev = q[n], od = q[2 * H - 1 - n];
+                    q[n] = ev + od;
+                    q[2 * H - 1 - n] = ev - od;
                 }
             }
         }
@@ -417,10 +556,10 @@ __host__ __device__ constexpr int up8(int v) { return (v + 7) & ~7; }
 template <int LPT, bool INV>
 __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, const float *__restrict__ table, int slot, int a)
 {
-    float *__restrict__ dst = tile_at(dst_tile);
-    const float *__restrict__ src = tile_at(src_tile);
     const DemoNdEntry &e = shared()->e[slot];
     const int s = e.s[a], p = e.p[a], lines = e.M / s;
+    const unsigned step = 4u * (unsigned)p;
+    auto at = [](unsigned byte) -> float & { return *reinterpret_cast<float *>(smem_raw + byte); };
     const int h = (s + 1) >> 1, pe = up8(h), po = up8(s >> 1);
     const int groups = INV ? pe >> 3 : (pe + po) >> 3;
     const float *Tb = INV ? table + h * (pe + po) : table;
@@ -428,9 +567,9 @@ __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, c
     const int items = groups * Q;
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
         const int g = it / Q, l0 = it - g * Q;
-        int b[LPT];
+        unsigned b[LPT];  // bytes into the tile
 #pragma unroll
-        for (int v = 0; v < LPT; ++v) b[v] = line_base(e, a, a, min(l0 + v * Q, lines - 1));
+        for (int v = 0; v < LPT; ++v) b[v] = 4u * (unsigned)line_base(e, a, a, min(l0 + v * Q, lines - 1));
         if constexpr (!INV) {
             const bool odd = 8 * g >= pe;
             const float sign = odd ? -1.f : 1.f;
@@ -440,15 +579,22 @@ __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, c
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[v][j] = 0.f;
             const float *tp = Tb + 8 * g;
-            int lo = 0, hi = (s - 1) * p;
+            unsigned lo[LPT], hi[LPT];
+#pragma unroll
+            for (int v = 0; v < LPT; ++v) {
+                lo[v] = src_tile + b[v];
+                hi[v] = lo[v] + (unsigned)(s - 1) * step;
+            }
 #pragma unroll 4
-            for (int n = 0; n < h; ++n, tp += pe + po, lo += p, hi -= p) {
+            for (int n = 0; n < h; ++n, tp += pe + po) {
                 const float4 t0 = __ldg(reinterpret_cast<const float4 *>(tp));
                 const float4 t1 = __ldg(reinterpret_cast<const float4 *>(tp + 4));
                 const float t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
 #pragma unroll
                 for (int v = 0; v < LPT; ++v) {
-                    const float xv = fmaf(sign, src[b[v] + hi], src[b[v] + lo]);
+                    const float xv = fmaf(sign, at(hi[v]), at(lo[v]));
+                    lo[v] += step;
+                    hi[v] -= step;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) acc[v][j] = fmaf(t[j], xv, acc[v][j]);
                 }
@@ -456,11 +602,11 @@ __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, c
 #pragma unroll
             for (int v = 0; v < LPT; ++v) {
                 if (l0 + v * Q < lines) {
+                    const int u0 = odd ? 2 * (8 * g - pe) + 1 : 16 * g;
+                    const unsigned q = dst_tile + b[v] + (unsigned)u0 * step;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int u = odd ? 2 * (8 * g - pe + j) + 1 : 2 * (8 * g + j);
-                        if (u < s) dst[b[v] + u * p] = acc[v][j];
-                    }
+                    for (int j = 0; j < 8; ++j)
+                        if (u0 + 2 * j < s) at(q + 2u * (unsigned)j * step) = acc[v][j];
                 }
             }
         } else {
@@ -470,13 +616,17 @@ __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, c
 #pragma unroll
                 for (int j = 0; j < 8; ++j) ev[v][j] = od[v][j] = 0.f;
             const float *tp = Tb + 8 * g;
+            unsigned q[LPT];
+#pragma unroll
+            for (int v = 0; v < LPT; ++v) q[v] = src_tile + b[v];
             auto term = [&](int u, float (&acc)[LPT][8]) {
                 const float4 t0 = __ldg(reinterpret_cast<const float4 *>(tp + u * pe));
                 const float4 t1 = __ldg(reinterpret_cast<const float4 *>(tp + u * pe + 4));
                 const float t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
 #pragma unroll
                 for (int v = 0; v < LPT; ++v) {
-                    const float xv = src[b[v] + u * p];
+                    const float xv = at(q[v]);
+                    q[v] += step;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) acc[v][j] = fmaf(t[j], xv, acc[v][j]);
                 }
@@ -490,12 +640,13 @@ __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, c
 #pragma unroll
             for (int v = 0; v < LPT; ++v) {
                 if (l0 + v * Q < lines) {
+                    const unsigned lo = dst_tile + b[v] + (unsigned)(8 * g) * step, hi = dst_tile + b[v] + (unsigned)(s - 1 - 8 * g) * step;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int n = 8 * g + j;
                         if (n < h) {
-                            dst[b[v] + n * p] = ev[v][j] + od[v][j];
-                            if (n != s - 1 - n) dst[b[v] + (s - 1 - n) * p] = ev[v][j] - od[v][j];
+                            at(lo + (unsigned)j * step) = ev[v][j] + od[v][j];
+                            if (n != s - 1 - n) at(hi - (unsigned)j * step) = ev[v][j] - od[v][j];
                         }
                     }
                 }
@@ -507,9 +658,20 @@ __device__ __noinline__ void lines_dense(unsigned dst_tile, unsigned src_tile, c
 // Extents that are transformed in registers.
 constexpr bool in_place_extent(int s) { return s <= 8 || s == 16 || s == 32 || s == 64 || s == 128; }
 
+// The first axis that is transformed, if the kept coefficients' lines along it are worth listing (those it is transformed in by a thread
+// per line); else -1.
+__device__ __forceinline__ int first_listed(const DemoNdEntry &e)
+{
+    int a = 0;
+    while (a < DEMO_ND_DIMS && e.s[a] == 1) ++a;
+    if (a == DEMO_ND_DIMS || (e.tail && a == 2) || !in_place_extent(e.s[a]) || e.s[a] > 32) return -1;
+    return a;
+}
+
 // All axes in turn.  cur / spare: the tile and the second tile (used by dense axes only); swapped as needed.
+// n_list >= 0: only the lines in the list are not zero along the first axis (first_listed).
 template <bool INV, bool BIG>
-__device__ __forceinline__ void transform_chunk(float *&cur, float *&spare, int slot, const float *tables)
+__device__ __forceinline__ void transform_chunk(float *&cur, float *&spare, int slot, const float *tables, int n_list)
 {
     const DemoNdEntry &e = shared()->e[slot];
     unsigned tile = tile_offset(cur), other = tile_offset(spare);
@@ -529,16 +691,28 @@ __device__ __forceinline__ void transform_chunk(float *&cur, float *&spare, int 
             __syncthreads();
             break;
         }
+        const int list = n_list;
+        n_list = -1;
+        auto whole = [&](auto extent) {
+            constexpr int S = decltype(extent)::value;
+            if constexpr (S % 4 == 0) {
+                if (a == DEMO_ND_DIMS - 1 && e.quads == 2) {
+                    lines_whole<S, INV, true>(tile, slot, a, list);
+                    return;
+                }
+            }
+            lines_whole<S, INV, false>(tile, slot, a, list);
+        };
         switch (s) {
-            case 2: lines_whole<2, INV>(tile, slot, a); break;
-            case 3: lines_whole<3, INV>(tile, slot, a); break;
-            case 4: lines_whole<4, INV>(tile, slot, a); break;
-            case 5: lines_whole<5, INV>(tile, slot, a); break;
-            case 6: lines_whole<6, INV>(tile, slot, a); break;
-            case 7: lines_whole<7, INV>(tile, slot, a); break;
-            case 8: lines_whole<8, INV>(tile, slot, a); break;
-            case 16: lines_whole<16, INV>(tile, slot, a); break;
-            case 32: lines_whole<32, INV>(tile, slot, a); break;
+            case 2: whole(std::integral_constant<int, 2>{}); break;
+            case 3: whole(std::integral_constant<int, 3>{}); break;
+            case 4: whole(std::integral_constant<int, 4>{}); break;
+            case 5: whole(std::integral_constant<int, 5>{}); break;
+            case 6: whole(std::integral_constant<int, 6>{}); break;
+            case 7: whole(std::integral_constant<int, 7>{}); break;
+            case 8: whole(std::integral_constant<int, 8>{}); break;
+            case 16: whole(std::integral_constant<int, 16>{}); break;
+            case 32: whole(std::integral_constant<int, 32>{}); break;
             case 64: lines_split<32, INV>(tile, slot, a); break;
             case 128:
                 if constexpr (BIG) lines_split<64, INV>(tile, slot, a);
@@ -889,20 +1063,21 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
     }
     __syncthreads();
     const unsigned bound = s->bound;  // (>= 1: the padding is never a candidate)
-    auto append = [&](float f, int t) {
-        if (mag_key(f) >= bound) {
-            const unsigned at = atomicAdd(&s->n, 1u);
-            if (at < (unsigned)CAND) s->cand[at] = make_uint2(__float_as_uint(f), (unsigned)t);
-        }
-    };
+    // (a thread whose maximum is below the bound has none; the quads of a thread take their places in the list together)
+    if (mine >= bound) {
 #pragma unroll 2
-    for (int i = tid; i < quads; i += T) {
-        const float4 f = X4[i];
-        if (max(max(mag_key(f.x), mag_key(f.y)), max(mag_key(f.z), mag_key(f.w))) >= bound) {
-            append(f.x, 4 * i);
-            append(f.y, 4 * i + 1);
-            append(f.z, 4 * i + 2);
-            append(f.w, 4 * i + 3);
+        for (int i = tid; i < quads; i += T) {
+            const float4 f = X4[i];
+            const bool c[4] = {mag_key(f.x) >= bound, mag_key(f.y) >= bound, mag_key(f.z) >= bound, mag_key(f.w) >= bound};
+            if (c[0] || c[1] || c[2] || c[3]) {
+                unsigned at = atomicAdd(&s->n, (unsigned)c[0] + (unsigned)c[1] + (unsigned)c[2] + (unsigned)c[3]);
+                const float v[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (c[j] && at < (unsigned)CAND) s->cand[at] = make_uint2(__float_as_uint(v[j]), (unsigned)(4 * i + j));
+                    at += c[j];
+                }
+            }
         }
     }
     __syncthreads();
@@ -922,11 +1097,13 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
         else
             find_threshold<16>((unsigned)n, bound, k_eff);
     }
-    if (dense) {
-    } else if (T == 32) {
-        for (int i = tid; i < quads; i += 32) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else if (tid >= 32) {
-        for (int i = tid - 32; i < quads; i += T - 32) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int listed = first_listed(e);
+    if (!dense && (T == 32 || tid >= 32)) {
+        const int first = T == 32 ? tid : tid - 32, step = T == 32 ? 32 : T - 32;
+        for (int i = first; i < quads; i += step) X4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (listed >= 0)
+            for (int i = first; i < 512; i += step) s->bits()[i] = 0u;
+        if (tid == T - 1 && listed >= 0) s->n_list = 0;
     }
     uint2 *kept = reinterpret_cast<uint2 *>(s->kept);
     if (tid == 0 && (k_eff & 1)) kept[k_eff] = make_uint2(0u, 0xffffffffu);  // completes the last pair: behind everything
@@ -964,6 +1141,10 @@ __device__ __forceinline__ void select_topk(float *X, int slot, DemoRecord *rec,
         r.val = __uint_as_float(c.x);
         rec[pos] = r;
         X[c.y] = alpha * r.val;
+        if (listed >= 0) {  // the line's first place identifies it: the first axis has the largest stride
+            const unsigned line = c.y % (unsigned)e.p[listed];
+            if (!(atomicOr(&s->bits()[line >> 5], 1u << (line & 31u)) >> (line & 31u) & 1u)) s->list()[atomicAdd(&s->n_list, 1)] = line;
+        }
     }
     __syncthreads();
 }
@@ -1001,7 +1182,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
     for (long long c = blockIdx.x; c < a.cls.n_chunks; c = (long long)gridDim.x + s->ticket, slot ^= 1) {
         // cleared for this chunk's selection; the barriers up to it order the writes
         for (int i = tid; i < 256; i += T) s->hist[i] = s->fine[i] = 0u;
-        if (tid == 0) s->hi = 0u, s->n = 0u, s->n_kept = 0u;
+        if (tid == 0) s->hi = 0u, s->n = 0u, s->n_kept = 0u, s->n_list = -1;
         __syncthreads();
         const DemoNdEntry &e = s->e[slot];
         if (e.layout != layout) {
@@ -1016,7 +1197,25 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
         const GT *__restrict__ g = static_cast<const GT *>(a.g_ptrs[e.tensor]) + base;
 
         // momentum update  B = beta*m + g  on the chunk (Algorithm 1, worker side)
-        {
+        const bool whole = e.quads == 2;
+        if (e.quads) {
+            constexpr int U = BIG ? 2 : 4;
+            float4 mv[U];
+            decltype(grad_quad(g)) gv[U];
+            for_quads<U>(
+                v, e,
+                [&](int j, unsigned off) {
+                    mv[j] = *reinterpret_cast<const float4 *>(m + off);
+                    gv[j] = grad_quad(g + off);
+                },
+                [&](int j, int i, unsigned, int t) {
+                    const float4 gf = grad_floats(gv[j]);
+                    const float4 b = make_float4(fmaf(a.beta, mv[j].x, gf.x), fmaf(a.beta, mv[j].y, gf.y), fmaf(a.beta, mv[j].z, gf.z),
+                                                 fmaf(a.beta, mv[j].w, gf.w));
+                    *reinterpret_cast<float4 *>(v.B + i) = b;
+                    set_tile_quad(tile0, t, whole, b);
+                });
+        } else {
             constexpr int U = 8;
             float mv[U];
             GT gv[U];
@@ -1034,11 +1233,22 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
         }
         if (tid == T - 1) take_ticket(s, slot ^ 1, a.entries, a.cls, ticket);
         __syncthreads();
-        transform_chunk<false, BIG>(tile0, tile1, slot, a.tables);  // Q = T(B; C_0, ..., C_{d-1})
+        transform_chunk<false, BIG>(tile0, tile1, slot, a.tables, -1);  // Q = T(B; C_0, ..., C_{d-1})
+        if ((long long)gridDim.x + s->ticket < a.cls.n_chunks && s->e[slot ^ 1].layout == layout) {  // the next chunk on its way to L2
+            const DemoNdEntry &ne = s->e[slot ^ 1];
+            prefetch_chunk(v, ne, a.m_ptrs[ne.tensor] + s->base[slot ^ 1]);
+            prefetch_chunk(v, ne, static_cast<const GT *>(a.g_ptrs[ne.tensor]) + s->base[slot ^ 1]);
+        }
         select_topk(tile0, slot, a.payload + e.rec_begin + (c - e.chunk_begin) * (long long)e.k_eff, a.alpha);
         // momentum subtraction  m <- B - alpha * T(kept; C_0^T, ..., C_{d-1}^T)
-        transform_chunk<true, BIG>(tile0, tile1, slot, a.tables);
-        for_elements<4>(v, e, [](int, auto) {}, [&](int, int i, auto off, int t) { m[off] = v.B[i] - tile0[t]; });
+        transform_chunk<true, BIG>(tile0, tile1, slot, a.tables, s->n_list);
+        if (e.quads)
+            for_quads<2>(v, e, [](int, unsigned) {}, [&](int, int i, unsigned off, int t) {
+                const float4 b = *reinterpret_cast<const float4 *>(v.B + i), r = tile_quad(tile0, t, whole);
+                *reinterpret_cast<float4 *>(m + off) = make_float4(b.x - r.x, b.y - r.y, b.z - r.z, b.w - r.w);
+            });
+        else
+            for_elements<4>(v, e, [](int, auto) {}, [&](int, int i, auto off, int t) { m[off] = v.B[i] - tile0[t]; });
         __syncthreads();
     }
     if (tid == T - 1) ticket_finish(a.tickets);
@@ -1077,7 +1287,6 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
         }
         unsigned ticket = 0;  // (last thread) the CTA's next chunk, drawn now, looked up below
         if (tid == T - 1) ticket = ticket_draw(a.tickets);
-        const size_t base = s->base[slot];
         const int M = e.M, k_eff = e.k_eff;
         const long long rec_off = e.rec_begin + (c - e.chunk_begin) * (long long)k_eff;
 
@@ -1184,9 +1393,9 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
             }
             __syncthreads();
         }
-        transform_chunk<true, BIG>(tile0, tile1, slot, a.tables);
+        transform_chunk<true, BIG>(tile0, tile1, slot, a.tables, -1);
         if (a.sign_ptrs) {  // parameter-server form: hand out sign(R), the workers apply it
-            signed char *__restrict__ sg = a.sign_ptrs[e.tensor] + base;
+            signed char *__restrict__ sg = a.sign_ptrs[e.tensor] + s->base[slot];
             for_elements<4>(v, e, [](int, auto) {}, [&](int, int, auto off, int t) {
                 const float rv = tile0[t];
                 sg[off] = (signed char)((rv > 0.f) - (rv < 0.f));
@@ -1194,15 +1403,29 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
             continue;
         }
         // x <- x - lr * (phi(R) + wd * x), sign(0) = 0
-        float *__restrict__ x = a.x_ptrs[e.tensor] + base;
+        float *__restrict__ x = a.x_ptrs[e.tensor] + s->base[slot];
+        auto updated = [&](float xv, float rv) {
+            const float sg = a.phi ? rv * a.agg_scale : (float)((rv > 0.f) - (rv < 0.f));
+            return fmaf(-a.lr, fmaf(a.wd, xv, sg), xv);
+        };
+        if (e.quads) {
+            constexpr int U = BIG ? 2 : 4;
+            float4 xv[U];
+            for_quads<U>(
+                v, e, [&](int j, unsigned off) { xv[j] = *reinterpret_cast<const float4 *>(x + off); },
+                [&](int j, int, unsigned off, int t) {
+                    const float4 r = tile_quad(tile0, t, e.quads == 2);
+                    *reinterpret_cast<float4 *>(x + off) =
+                        make_float4(updated(xv[j].x, r.x), updated(xv[j].y, r.y), updated(xv[j].z, r.z), updated(xv[j].w, r.w));
+                });
+            continue;
+        }
         constexpr int U = 8;
         float xv[U];
         for_elements<U>(
             v, e, [&](int j, auto off) { xv[j] = x[off]; },
             [&](int j, int, auto off, int t) {
-                const float rv = tile0[t];
-                const float sg = a.phi ? rv * a.agg_scale : (float)((rv > 0.f) - (rv < 0.f));
-                x[off] = fmaf(-a.lr, fmaf(a.wd, xv[j], sg), xv[j]);
+                x[off] = updated(xv[j], tile0[t]);
             });
     }
     if (tid == T - 1) ticket_finish(a.tickets);
@@ -1246,39 +1469,67 @@ int DemoNdTables::get(int s)
 
 // Tile strides: the innermost axis is dense, every outer stride may be padded by a few words.  The padding is the one with
 // the fewest bank conflicts of a warp's accesses over the axis passes (32 neighbouring lines at a time), the smaller tile
-// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it.  The search takes 10 to 50 us of the host's time, so
+// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it, an eighth where it makes the rows whole quads.  The search takes 10 to 50 us of the host's time, so
 // tensors of the same chunk shape share one.
 void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
 {
     const int *s = e->s;
     e->tail = s[2] == s[3] && s[3] >= 2 && s[3] <= 7 ? s[3] : 0;
-    auto conflicts = [&](const int *p) {
+    // how many trailing elements follow one another in the tensor and, with strides p, in the tile
+    auto run_of = [&](const int *p) {
+        long long run = 1;
+        for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
+            if (s[a] > 1 && (e->stride[a] != run || p[a] != run)) break;
+            run *= s[a];
+        }
+        return (int)run;
+    };
+    // 1: the rows are whole 16-byte pieces of the tensor, 2: of the tile too
+    auto quads_of = [&](const int *p) {
+        const int run = run_of(p);
+        if (run % 4) return 0;
+        bool tile = true;
+        long long in = 1;  // elements of the axes behind a
+        for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
+            if (e->c[a] > 1 && s[a] * e->stride[a] % 4) return 0;  // chunks start on a piece
+            if (s[a] > 1 && in >= run) {
+                if (e->stride[a] % 4) return 0;
+                tile = tile && p[a] % 4 == 0;
+            }
+            in *= s[a];
+        }
+        return tile ? 2 : 1;
+    };
+    auto conflicts = [&](const int *p, bool whole) {
         long long cost = 0;
         for (int a = 0; a < DEMO_ND_DIMS; ++a) {
             if (s[a] == 1 || (e->tail && a == 3)) continue;
             const int last = e->tail && a == 2 ? 3 : a;
             const int lines = e->M / (s[a] * (last > a ? s[last] : 1));
+            const bool pieces = whole && a == 3 && s[a] % 4 == 0 && in_place_extent(s[a]) && s[a] <= 32;  // 16 bytes per thread, eight threads at a time
+            const int lanes = pieces ? 8 : 32, banks = pieces ? 8 : 32;
             for (int w = 0; w < 3 && w * 32 < lines; ++w) {  // the first, second and third warp's lines
                 int bank[32] = {0}, worst = 0;
-                for (int l = 32 * w; l < lines && l < 32 * w + 32; ++l) {
+                for (int l = 32 * w; l < lines && l < 32 * w + lanes; ++l) {
                     int r = l, t = 0;
                     for (int b = DEMO_ND_DIMS - 1; b >= 0; --b)
                         if (b < a || b > last) {
                             t += (r % s[b]) * p[b];
                             r /= s[b];
                         }
-                    const int v = ++bank[t & 31];
+                    const int v = ++bank[(pieces ? t / 4 : t) % banks];
                     worst = worst > v ? worst : v;
                 }
                 cost += worst * (last > a ? 2 : 1);
             }
         }
-        return cost;
+        // (rows that are not whole pieces cost four accesses instead of one where the chunk comes and goes)
+        return 2 * cost + (whole ? 0 : 2);
     };
     const DemoNdTables::Layout *known = nullptr;
     for (const DemoNdTables::Layout &l : tables->layouts)
         if (l.s[0] == s[0] && l.s[1] == s[1] && l.s[2] == s[2] && l.s[3] == s[3]) known = &l;
-    const int room = e->M / 16 > 64 ? e->M / 16 : 64;
+    const int room = e->M / 16 > 64 ? e->M / 16 : 64, room_quads = e->M / 8 > room ? e->M / 8 : room;
     long long best = -1;
     int p[DEMO_ND_DIMS];
     p[3] = 1;
@@ -1289,8 +1540,9 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
             for (int pad0 = 0; pad0 <= (s[0] > 1 && s[1] * s[2] * s[3] > 1 ? 31 : 0); ++pad0) {
                 p[0] = p[1] * s[1] + pad0;
                 const int floats = p[0] * s[0];
-                if (floats > e->M + room) break;
-                const long long cost = conflicts(p) * (1LL << 20) + floats;
+                if (floats > e->M + room_quads) break;
+                if (floats > e->M + room && quads_of(p) != 2) continue;
+                const long long cost = conflicts(p, quads_of(p) == 2) * (1LL << 20) + floats;
                 if (best < 0 || cost < best) {
                     best = cost;
                     for (int a = 0; a < DEMO_ND_DIMS; ++a) e->p[a] = p[a];
@@ -1311,19 +1563,14 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
         l.tile = e->tile;
         tables->layouts.push_back(l);
     }
-    // rows: the trailing elements that follow one another in the tensor and in the tile
-    long long run = 1, span = 0;
-    bool joined = true;
-    for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
-        if (joined && (s[a] == 1 || (e->stride[a] == run && e->p[a] == run)))
-            run *= s[a];
-        else
-            joined = joined && s[a] == 1;
-        span += (s[a] - 1) * e->stride[a];
-    }
-    e->row = (int)run;
+    long long span = 0;
+    for (int a = 0; a < DEMO_ND_DIMS; ++a) span += (s[a] - 1) * e->stride[a];
+    const int run = run_of(e->p);
+    e->row = run;
     e->inv_row = run > 1 ? (unsigned)(((1ULL << 32) + (unsigned long long)run - 1) / (unsigned long long)run) : 0u;
+    e->inv_row4 = run > 4 ? (unsigned)(((1ULL << 32) + (unsigned long long)run / 4 - 1) / (unsigned long long)(run / 4)) : 0u;
     e->row_table = e->M / run <= DEMO_ND_MAX_ROWS && span < (1LL << 32);
+    e->quads = e->row_table ? quads_of(e->p) : 0;
     // threads: enough for every pass over the long axes in whole rounds, and for 32 elements each
     int threads = (e->M + 31) / 32;
     for (int a = 0; a < DEMO_ND_DIMS; ++a) {

@@ -585,3 +585,25 @@ def test_vectors_under_a_callers_basis(s):
     r.set_basis()
     r.step()
     r.close()
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("shape,chunk,k", [
+    ((32, 128), (16, 32), 5),            # rows of whole quads in the tensor and in the tile, the last axis read by quads
+    ((24, 80), (8, 16), 128),            # the same, everything kept: no list of lines
+    ((64, 24), (32, 8), 12), ((48, 12), (3, 4), 3),
+    ((48, 64, 3, 3), (16, 32, 3, 3), 31),  # rows of 288 elements across two axes, the tile's rows not quads
+    ((4, 48, 3, 3), (4, 16, 3, 3), 9),   # one chunk deep: the rows are the chunk
+    ((32, 36, 5, 5), (8, 12, 5, 5), 20), ((14, 21, 6, 6), (7, 7, 6, 6), 17),
+    ((30, 33), (6, 11), 7),              # rows of 11: element by element
+    ((30, 36), (5, 12), 7), ((29 * 3, 128), (29, 64), 32), ((64, 62), (32, 31), 40),
+    ((128, 8), (128, 4), 30),
+])
+def test_nd_rows_and_lines(shape, chunk, k, f32):
+    """Chunks whose rows are whole 16-byte pieces of the tensor, of the tile, of both, or not; odd and even extents multiplied out;
+    first axes whose kept lines are listed (several records per line among them) and others."""
+    r = parity.NdRunner([shape, (shape[-1] * 4,)], [chunk, (chunk[-1],)], topk=k, num_workers=2, grad_std=0.02,
+                        grad_dtype=torch.float32 if f32 else torch.bfloat16)
+    for _ in range(2):
+        r.step()
+    r.close()
