@@ -10,7 +10,8 @@
 //     e = DCT-III_64(X[even]),  o = DCT-IV_64(X[odd]),  x[n] = e[n] + o[n],  x[127-n] = e[n] - o[n]
 // where thread h of a line finishes n in [32h, 32h+32): the two exchange half of e and o through shared memory.
 //
-// compress: TMA-staged m and g tiles -> B = beta*m + g (parked in tensor memory) -> column pass -> row pass ->
+// compress: TMA-staged m and g tiles -> B = beta*m + g (half a column per thread, parked in tensor memory, from where the
+// other thread of the column reads it) -> column pass -> row pass ->
 // coefficients in shared memory -> exact top-k (bound from the 256 half-row maxima, candidate list, ballot search; radix
 // select for degenerate chunks) -> records; sparse row stage of the inverse from the records, half of them by each half of
 // the CTA, fast column stage, residual m <- B - alpha * IDCT(kept) against the parked B, one TMA store of the new momentum
@@ -20,7 +21,8 @@
 // memory allow: shared-memory accesses and issue each take about half of the time.  8192 x 8192, k = 32, bf16 gradients:
 // compress 242 -> 222 us (k = 128 313 -> 272) with the halves of the row stage and the early g tile; decode 162 -> 141 us and
 // signs 235 -> 131 us with half the exchange (before, the signs form kept two sets of 64 results and spilled), W = 8
-// 155 -> 145 and 131 -> 121 us with staged records and the x tile in halves.
+// 155 -> 145 and 131 -> 121 us with staged records and the x tile in halves; compress of 2368 chunks 134.0 -> 133.3 us, 592
+// 39.6 -> 39.0 with half a column of B per thread (both halves by both before).
 // Tiles need the TMA tensor maps; without them the host uses the generic kernels for s = 128.
 #include <cuda_bf16.h>
 
@@ -224,19 +226,17 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
             if (pass == 0) {
-                // column j of B = beta*m + g, folded: in[n] = B[n][j] +/- B[127-n][j]; the half of the column that
-                // this thread will write back is parked in tensor memory (two stores of 32 columns)
-                const float sg = h ? -1.f : 1.f;
+                // Column j of B = beta*m + g: thread h forms the half of it that it will write back (rows 0 .. 63 or 127 .. 64) and parks
+                // it in tensor memory (two stores of 32 columns), where the other thread of the column reads it for its own fold,
+                // in[n] = B[n][j] +/- B[127-n][j].  (With both halves formed by both threads: twice the shared-memory reads,
+                // conversions and multiply-adds.)
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     float park[32];
 #pragma unroll
                     for (int q = 0; q < 32; ++q) {
-                        const int n = 32 * half + q;
-                        const float lo = fmaf(a.beta, Ms[n * S + j], to_f32(Gs[n * S + j]));
-                        const float hi = fmaf(a.beta, Ms[(S - 1 - n) * S + j], to_f32(Gs[(S - 1 - n) * S + j]));
-                        in[n] = fmaf(sg, hi, lo);
-                        park[q] = h ? hi : lo;
+                        const int n = 32 * half + q, at = (h ? S - 1 - n : n) * S + j;
+                        park[q] = in[n] = fmaf(a.beta, Ms[at], to_f32(Gs[at]));
                     }
                     tmem_st32(taddr + h * H + 32 * half, park);
                 }
@@ -245,6 +245,17 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
                 fence_proxy_async();
                 __syncthreads();  // the staged tiles are consumed (X aliases the m tile)
                 if (tid == 0 && nc < a.n_chunks) issue_tile(cur.te, nc, true, false);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    float other[32];
+                    tmem_ld32(taddr + (h ^ 1) * H + 32 * half, other);
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) {
+                        const int n = 32 * half + q;
+                        in[n] = h ? other[q] - in[n] : in[n] + other[q];
+                    }
+                }
             } else {
                 // row j of the column-transformed tile, folded
                 const float4 *row = reinterpret_cast<const float4 *>(X + j * XS);
