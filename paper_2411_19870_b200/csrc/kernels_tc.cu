@@ -17,7 +17,8 @@
 //     coalesced row piece per load; a transpose through the tile gives the second stage its rows; the inverse's row stage is
 //     k rank-1 updates on the CUDA cores (as in kernels_fast64.cu), its column stage one more tensor-core stage whose result
 //     is column j of the residual update: loads and stores of the momentum are coalesced and B is formed again from L2.
-// 4096 x 8192, bf16 gradients, two workers: compress k = 32 185 us, k = 128 234 us, decode 108 / 123 us (378 and 236 us at
+// 4096 x 8192, bf16 gradients, two workers: compress k = 32 177 us, decode 102 us (185 and 108 before the look-up in front of the
+// wait and the descriptors that move on; 378 and 236 us at
 // k = 32 with both operands in shared memory, 64 KB per pair, two pairs per SM and four stages).  A third of compress
 // is the two passes over the momentum: the next pair's tiles are brought to L2 during the selection and read 32 rows at a
 // time (without: 199 us).  Every wait is bounded: on expiry the group records DEMO_DEV_TIMEOUT and stops, the CTA frees its
@@ -71,7 +72,7 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;
 }
 // Instruction descriptor: D fp32, A (tensor memory) and B tf32, B K- or MN-major, N = 64, M = 128.
-__device__ __forceinline__ constexpr uint32_t instr_desc(int b_mn)
+__host__ __device__ constexpr uint32_t instr_desc(int b_mn)
 {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)b_mn << 16) | ((uint32_t)(S >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
@@ -106,16 +107,24 @@ __device__ __forceinline__ void write_split(unsigned char *hi, unsigned char *lo
 }
 
 // One product, issued by one thread: D (+)= A * basis part, K = 64 in eight steps of 8 (8 columns of A; 32 bytes inside a
-// 128-byte row of the K-major basis, second half of K one block further, or 8 K-rows of the MN-major one).
-__device__ __forceinline__ void issue_product(uint32_t d_tmem, uint32_t a_tmem, uint32_t b, int b_mn, uint32_t acc)
+// 128-byte row of the K-major basis, second half of K one block further, or 8 K-rows of the MN-major one).  The descriptor is formed once
+// and moved on: a thread that builds one per step takes longer than the tensor core for the product.  Rolled: unrolled, its temporaries
+// spill the 64 values that every thread holds.
+template <bool MN>
+__device__ __forceinline__ void issue_product(uint32_t d_tmem, uint32_t a_tmem, uint32_t b, uint32_t acc)
 {
-    const uint32_t idesc = instr_desc(b_mn);
+    constexpr uint32_t idesc = instr_desc(MN);
+    uint64_t desc = MN ? smem_desc(b, BLK, 512, 1) : smem_desc(b, 16, 1024, 2);  // (addresses stay below 2^18: no carry out of the field)
 #pragma unroll 1
-    for (int kk = 0; kk < 8; ++kk) {
-        const uint64_t bd = b_mn ? smem_desc(b + kk * 1024, BLK, 512, 1)
-                                 : smem_desc(b + (kk >> 2) * BLK + (kk & 3) * 32, 16, 1024, 2);
-        umma_tf32(d_tmem, a_tmem + kk * 8, bd, idesc, acc);
-        acc = 1;
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll 1
+        for (int kk = 0; kk < 4; ++kk) {
+            umma_tf32(d_tmem, a_tmem, desc, idesc, acc);
+            acc = 1u;
+            a_tmem += 8;
+            desc += (MN ? 1024 : 32) >> 4;
+        }
+        if (!MN) desc += (BLK - 4 * 32) >> 4;
     }
 }
 
@@ -168,9 +177,10 @@ __device__ __forceinline__ void tc_setup(TcFrame &f, unsigned char *raw, const f
 }
 
 // One stage on the pair: v becomes this thread's row of (the pair's vectors) * basis, 3xTF32.  False if a wait expired.
-__device__ __forceinline__ bool tc_stage(TcFrame &f, const SlotBarrier<PAIR_THREADS> &pb, float (&v)[S], int b_mn)
+template <bool MN>
+__device__ __forceinline__ bool tc_stage(TcFrame &f, const SlotBarrier<PAIR_THREADS> &pb, float (&v)[S])
 {
-    const uint32_t b_hi = smem_u32(f.sm + (b_mn ? OFF_BM_HI : OFF_BK_HI)), b_lo = smem_u32(f.sm + (b_mn ? OFF_BM_LO : OFF_BK_LO));
+    const uint32_t b_hi = smem_u32(f.sm + (MN ? OFF_BM_HI : OFF_BK_HI)), b_lo = smem_u32(f.sm + (MN ? OFF_BM_LO : OFF_BK_LO));
     bool ok = true;
     auto product = [&](auto last) {
         tmem_wait_st();
@@ -178,8 +188,8 @@ __device__ __forceinline__ bool tc_stage(TcFrame &f, const SlotBarrier<PAIR_THRE
         pb.sync();
         if (f.pt == 0) {
             tc_fence_after();
-            issue_product(f.d_mma, f.a_mma, decltype(last)::value ? b_lo : b_hi, b_mn, decltype(last)::value);
-            if (decltype(last)::value) issue_product(f.d_mma, f.a_mma, b_hi, b_mn, 1);
+            issue_product<MN>(f.d_mma, f.a_mma, decltype(last)::value ? b_lo : b_hi, decltype(last)::value);
+            if (decltype(last)::value) issue_product<MN>(f.d_mma, f.a_mma, b_hi, 1);
             umma_commit(f.bar);
         }
         ok = mbar_wait_bounded(f.bar, f.phase) && ok;
@@ -348,13 +358,13 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
             for (int i = 0; i < S; ++i) v[i] = 0.f;
         }
         // ---- Q = P B P^T: column j of B -> column j of P B -> row u of P B -> row u of Q ----------------------
-        ok = tc_stage(f, pb, v, 0);
+        ok = tc_stage<false>(f, pb, v);
         if (!ok) break;
 #pragma unroll
         for (int u = 0; u < S; ++u) X[u * XS + r] = v[u];
         sb.sync();
         read_row(X, r, v);
-        ok = tc_stage(f, pb, v, 0);
+        ok = tc_stage<false>(f, pb, v);
         if (!ok) break;
         const unsigned next = *f.drawn;  // (written before the barriers of the stages; overwritten behind those below)
         // row r of the group's next tiles on its way to L2.  (Without a counter next is NO_TICKET = 2^31 behind the grid, which then has a
@@ -370,7 +380,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
                 read_row(X, r, w);  // (core order)
                 fdct::static_for<0, S>([&](auto q) { v[fdct::core_index<S>(decltype(q)::value)] = w[decltype(q)::value]; });
             }
-            ok = tc_stage(f, pb, v, 1);  // row u of S P
+            ok = tc_stage<true>(f, pb, v);  // row u of S P
             if (!ok) break;
             write_row(X, r, v);
             sb.sync();
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
             for (int u = 0; u < S; ++u) v[u] = Xt[u * XS];  // (written by this thread only)
         }
         // ---- column stage; momentum subtraction  m <- B - alpha R  (Section 2.1) --------------------------------
-        ok = tc_stage(f, pb, v, 1);
+        ok = tc_stage<true>(f, pb, v);
         if (!ok) break;
         if (valid) each_b<BIGK ? 16 : 8>(m, g, cr.n1, a.beta, [&](int i, float b) { m[(size_t)i * cr.n1] = b - v[i]; });
         p = next;
@@ -517,14 +527,14 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
             }
         }
         // ---- R = P^T S P: row u of S -> row u of S P -> column j of S P -> column j of R; x <- x - lr (phi(R) + wd x)
-        ok = tc_stage(f, pb, v, 1);
+        ok = tc_stage<true>(f, pb, v);
         if (!ok) break;
         const unsigned next = *f.drawn;  // (written before the barriers of this stage, overwritten behind the next one's)
         write_row(X, r, v);
         sb.sync();
 #pragma unroll
         for (int u = 0; u < S; ++u) v[u] = X[u * XS + r];
-        ok = tc_stage(f, pb, v, 1);
+        ok = tc_stage<true>(f, pb, v);
         if (!ok) break;
         if (valid) {
 #pragma unroll
