@@ -120,6 +120,9 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.demo_status_string.restype = ctypes.c_char_p
     lib.demo_free.argtypes = [vp]
     lib.demo_free.restype = None
+    # addresses of the per-step calls, for csrc/calls.cpp
+    lib.entry_points = {n: ctypes.cast(getattr(lib, n), ctypes.c_void_p).value
+                        for n in ("demo_compress", "demo_decode_apply", "demo_decode_signs", "demo_apply_signs")}
     if path is None:
         _lib = lib
     return lib
@@ -225,8 +228,7 @@ class DemoTransform:
         self._payload_ok = set()   # (data pointer, size) of payload buffers already checked
         self._gdtype = torch.bfloat16 if grad_dtype == DEMO_BF16 else torch.float32
         # what the calls of csrc/calls.cpp are given: entry points, context, keys of the pointer arrays
-        address = lambda f: ctypes.cast(f, ctypes.c_void_p).value  # noqa: E731
-        self._fn = {n: address(getattr(self.lib, n)) for n in ("demo_compress", "demo_decode_apply", "demo_decode_signs", "demo_apply_signs")}
+        self._fn = self.lib.entry_points
         self._keys = [(("g", w), ("m", w)) for w in range(num_workers)]
 
     # --- queries -------------------------------------------------------------------------------

@@ -5,7 +5,7 @@
 // What bounds them is latency: a chunk holds 8 to 256 elements, so nothing is gained by more threads per chunk (the dense
 // kernels, a 256-thread CTA per chunk with radix select and a barrier between all steps, spent 24 us on 2048 tiles of 8 x 8
 // and 13 us on 1024 segments), and a warp needs (almost) no block barrier from the loads to the stores:
-//   * segments: every thread forms one coefficient by reading its row of the basis through L1 (the sums run over n in order,
+//   * segments: every thread forms one coefficient, a warp reading the basis by rows of its transpose (the sums run over n in order,
 //     so the results are those of the dense kernels bit for bit); the k-th key by a bit-by-bit ballot search;
 //   * tiles: lane j holds column j, then row j, in registers (fast_dct.cuh); the transposes go through a tile of the
 //     warp's own shared memory; the k-th key by a bit-by-bit search with counts added up over the tile's lanes.
