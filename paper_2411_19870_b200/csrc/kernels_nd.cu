@@ -1469,8 +1469,8 @@ int DemoNdTables::get(int s)
 
 // Tile strides: the innermost axis is dense, every outer stride may be padded by a few words.  The padding is the one with
 // the fewest bank conflicts of a warp's accesses over the axis passes (32 neighbouring lines at a time), the smaller tile
-// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it, an eighth where it makes the rows whole quads.  The search takes 10 to 50 us of the host's time, so
-// tensors of the same chunk shape share one.
+// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it, an eighth where it makes the rows whole quads.  The search takes 10
+// to 130 us of the host's time, so tensors of the same chunk shape share one.
 void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
 {
     const int *s = e->s;
@@ -1517,7 +1517,7 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
                             t += (r % s[b]) * p[b];
                             r /= s[b];
                         }
-                    const int v = ++bank[(pieces ? t / 4 : t) % banks];
+                    const int v = ++bank[(pieces ? t >> 2 : t) & (banks - 1)];
                     worst = worst > v ? worst : v;
                 }
                 cost += worst * (last > a ? 2 : 1);
@@ -1541,8 +1541,9 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
                 p[0] = p[1] * s[1] + pad0;
                 const int floats = p[0] * s[0];
                 if (floats > e->M + room_quads) break;
-                if (floats > e->M + room && quads_of(p) != 2) continue;
-                const long long cost = conflicts(p, quads_of(p) == 2) * (1LL << 20) + floats;
+                const bool whole = quads_of(p) == 2;
+                if (floats > e->M + room && !whole) continue;
+                const long long cost = conflicts(p, whole) * (1LL << 20) + floats;
                 if (best < 0 || cost < best) {
                     best = cost;
                     for (int a = 0; a < DEMO_ND_DIMS; ++a) e->p[a] = p[a];
