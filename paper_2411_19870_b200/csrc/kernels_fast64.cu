@@ -453,11 +453,12 @@ cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t st
     if (grid > groups) grid = groups;
     DemoCompressArgs b = a;
     if (grid == groups) b.tickets = nullptr;
-    // The look-up in front of the wait spares every call its latency, except where a set of several tensors nearly fills the device once:
-    // there all tiles would be requested in the same moment, by many maps, and land late; behind the allocation the look-ups spread the
-    // requests.  Steps, early / late / before both: 976 chunks of 57 tensors, six workers 135 / 120 / 120 us; 800 of 23, two workers 48.1 /
-    // 44.3 / 46.0; 280 of 9, seven workers 92.5 / 99.9 / 101.7; 3328 of 58, three workers 171 / 178 / 173.
-    b.late_lookup = a.n_entries > 1 && grid == groups && grid > 4LL * dev.sm_count;
+    // The look-up in front of the wait spares every call its latency, except where a set of several tensors nearly fills the device, up to
+    // two and a half times: there all tiles would be requested in the same moment, by many maps, and land late; behind the allocation the
+    // look-ups spread the requests.  Steps, early / late / before both: 280 chunks of 9 tensors, seven workers 92.5 / 99.9 / 101.7 us; 800 of
+    // 23, two workers 48.1 / 44.3 / 46.0; 976 of 57, six workers 135 / 120 / 120; 1424 of 30, six workers 170.5 / 158.5 / 167.1; 2400 of 65,
+    // two workers 91.8 / 85.3 / 88.0; 2640 of 72, one worker 60.3 / 60.2 / 63.1; 3328 of 58, three workers 171 / 178 / 173.
+    b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > 4LL * dev.sm_count;
     void *params[] = {&b};
     return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
 }
