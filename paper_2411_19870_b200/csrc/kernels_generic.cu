@@ -342,15 +342,19 @@ cudaError_t demo_launch_decode_generic(int s, const DemoDecodeArgs &a, DemoLaunc
 // =================================================================================================
 // Random orthonormal basis (Section 4.2, "Choice of Linear Projections"): Gram-Schmidt process on the
 // rows of a Gaussian matrix, in fp64, one CTA.  Right-looking order by blocks of four rows: the warp that holds them makes them
-// orthogonal among themselves, one after the other, then every later row loses its components along the four, which are orthogonal to
-// each other, at once.
+// orthogonal among themselves, one after the other, then every later row loses its components along the four at once.  The four are
+// orthogonal to each other only up to rounding times their condition, so the products of a later row with them are not yet its
+// components: those follow by a triangular substitution with the four rows' own products, which the block's warp has formed anyway (the
+// inverse compact WY form of the modified process; Swirydowicz, Langou, Ananthan, Yang, Thomas, "Low synchronization Gram-Schmidt and
+// generalized minimal residual algorithms", 2021).  Taken without it, rows that differ by 1e-5 of their length came out with products of
+// 4e-4; with it |P P^T - I| is that of the process row by row, about the rounding times the condition of the matrix.
 //
 // s dependent steps, so the latency of a step is all there is.  Eight threads keep a row in registers, a warp a block: inside it a step is
 // a row published in shared memory and two three-level reductions side by side, without a barrier; one barrier per block, one division per
 // step in the whole CTA (fp64 arithmetic is narrow).  At s = 128 the registers hold one published row at a time.  The matrix is read from and
 // the verdict written to pinned host memory, the active basis only replaced when the verdict is good: a call is one launch and one
 // synchronisation.  (One call, s = 64: 123 us with rows in shared memory, two barriers per step and four copies, 44.6 with a barrier per
-// row, 40.9 now.)
+// row, 41 now.)
 // =================================================================================================
 constexpr int GS_LANES = 8;  // threads per row
 
@@ -361,7 +365,7 @@ __global__ void __launch_bounds__(GS_LANES *GS_LANES *EPL, 1) gram_schmidt_kerne
     constexpr int N = GS_LANES * EPL;  // rows = columns
     constexpr int R = 32 / GS_LANES;   // rows of a warp, a block
     __shared__ __align__(16) double pub[2][R][N];  // the rows of a block and 1 / their squared lengths, 0 when nothing is left of one
-    __shared__ double pub_inv[2][R];
+    __shared__ double pub_inv[2][R], pub_dot[2][R][R];  // [i][j]: product of the block's rows j < i
     const int r = threadIdx.x / GS_LANES, l = threadIdx.x % GS_LANES, warp = threadIdx.x / 32, own = r % R;
     constexpr int V = EPL > 1 ? 2 : 1;  // consecutive elements of a thread
     auto col = [&](int e) { return (e / V) * (V * GS_LANES) + V * l + e % V; };
@@ -405,6 +409,7 @@ __global__ void __launch_bounds__(GS_LANES *GS_LANES *EPL, 1) gram_schmidt_kerne
                 const double len2 = along(nullptr, row), dot = along(a, row), scale_i = __shfl_sync(0xffffffffu, scale, i * GS_LANES);
                 const double inv = len2 > 1e-24 * scale_i ? 1.0 / len2 : 0.0;
                 if (own == i && l == 0) pub_inv[b & 1][i] = inv;
+                if (EPL <= 8 && own < i && l == 0) pub_dot[b & 1][i][own] = dot;  // (both rows are final)
                 const double c = own > i ? dot * inv : 0.0;
                 if (EPL > 8) asm volatile("" ::: "memory");
 #pragma unroll
@@ -414,13 +419,19 @@ __global__ void __launch_bounds__(GS_LANES *GS_LANES *EPL, 1) gram_schmidt_kerne
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < R; ++i) bad = bad || pub_inv[b & 1][i] == 0.0;
-        if (warp > b) {  // the block's rows are orthogonal to each other: their parts are taken off together
+        if (warp > b) {  // the block's rows: their parts are taken off together
             constexpr int G = EPL > 8 ? 1 : R;  // (s = 128: one after the other, there are 64 registers)
 #pragma unroll 1
             for (int i0 = 0; i0 < R; i0 += G) {
                 double c[G];
 #pragma unroll
-                for (int i = 0; i < G; ++i) c[i] = along(a, pub[b & 1][i0 + i]) * pub_inv[b & 1][i0 + i];
+                for (int i = 0; i < G; ++i) c[i] = along(a, pub[b & 1][i0 + i]);
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+#pragma unroll
+                    for (int j = 0; j < i; ++j) c[i] = fma(-c[j], pub_dot[b & 1][i][j], c[i]);
+                    c[i] *= pub_inv[b & 1][i0 + i];
+                }
                 if (G == 1) asm volatile("" ::: "memory");  // (the row is read again rather than kept)
 #pragma unroll
                 for (int i = 0; i < G; ++i)
