@@ -226,7 +226,9 @@ class DemoTransform:
         self._ptr_cache = {}
         self._payload_bytes = int(self.lib.demo_payload_bytes(self._ctx))
         self._payload_ok = set()   # (data pointer, size) of payload buffers already checked
-        self._gdtype = torch.bfloat16 if grad_dtype == DEMO_BF16 else torch.float32
+        self._grad, self._f32, self._i8 = (
+            (d, self._calls.layouts(d, device, self.shapes))
+            for d in (torch.bfloat16 if grad_dtype == DEMO_BF16 else torch.float32, torch.float32, torch.int8))
         # what the calls of csrc/calls.cpp are given: entry points, context, keys of the pointer arrays
         self._fn = self.lib.entry_points
         self._keys = [(("g", w), ("m", w)) for w in range(num_workers)]
@@ -249,16 +251,16 @@ class DemoTransform:
         return int(self.lib.demo_launch_count(self._ctx))
 
     # --- marshalling helpers -------------------------------------------------------------------
-    def _array(self, key, tensors, check=None):
-        """Pointer array for a list of tensors, cached per key and data pointers.  ``check`` = (shapes,
-        dtype, on_device) is verified whenever the pointers are new."""
+    def _array(self, key, tensors, layouts=None):
+        """Pointer array for a list of tensors, cached per key and data pointers.  ``layouts`` = (dtype, what csrc/calls.cpp
+        compares): the tensors are checked, in every call, since an address says nothing about a tensor's type or shape."""
+        tensors = list(tensors)
         ptrs = [t.data_ptr() for t in tensors]
+        if layouts is not None:
+            validate_tensors(tensors, self.shapes, layouts[0], self.device, str(key))
         hit = self._ptr_cache.get(key)
         if hit is None or hit[0] != ptrs:
-            if check is not None:
-                shapes, dtype, on_device = check
-                validate_tensors(tensors, shapes, dtype, self.device if on_device else None, str(key))
-            hit = (ptrs, _ptr_array(ptrs))
+            hit = (ptrs, _ptr_array(ptrs)) if layouts is None else (ptrs, _ptr_array(ptrs), layouts[1])
             self._ptr_cache[key] = hit
         return hit[1]
 
@@ -267,14 +269,11 @@ class DemoTransform:
             self._check_payload(p, "payloads[%d]" % i)
 
     def _check_payload(self, p, what: str) -> None:
-        ptr = (p.data_ptr(), p.numel())
-        if ptr in self._payload_ok:
-            return
         if p.dtype != torch.uint8 or not p.is_contiguous() or p.numel() < self.payload_bytes or not p.is_cuda \
                 or p.device.index != self.device:
             raise ValueError("%s: need a contiguous uint8 tensor of at least %d bytes on cuda:%d"
                              % (what, self.payload_bytes, self.device))
-        self._payload_ok.add(ptr)
+        self._payload_ok.add((p.data_ptr(), p.numel()))
 
     @staticmethod
     def _stream(stream) -> ctypes.c_void_p:
@@ -288,8 +287,8 @@ class DemoTransform:
         return None if stream is None else int(getattr(stream, "cuda_stream", stream))
 
     # --- the ABI calls -------------------------------------------------------------------------
-    # Tensors that lie where they were checked last go straight to the library (csrc/calls.cpp); the others, which it answers with None,
-    # are checked and their pointers noted.
+    # Tensors that lie where they lay last, with the layout the library assumes, go straight to it (csrc/calls.cpp); the others, which that
+    # module answers with None, are checked and their pointers noted.
     def compress(self, worker: int, grads, momentum, payload_out, stream=None) -> None:
         if type(worker) is int and 0 <= worker < self.num_workers:
             kg, km = self._keys[worker]
@@ -300,8 +299,8 @@ class DemoTransform:
                     raise DemoError(st, "demo_compress")
                 return
         self._check_payload(payload_out, "payload_out")
-        st = self.lib.demo_compress(self._ctx, worker, self._array(("g", worker), grads, (self.shapes, self._gdtype, True)),
-                                    self._array(("m", worker), momentum, (self.shapes, torch.float32, True)),
+        st = self.lib.demo_compress(self._ctx, worker, self._array(("g", worker), grads, self._grad),
+                                    self._array(("m", worker), momentum, self._f32),
                                     ctypes.c_void_p(payload_out.data_ptr()), self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_compress")
@@ -315,7 +314,7 @@ class DemoTransform:
             return
         self._check_payloads(payloads)
         st = self.lib.demo_decode_apply(self._ctx, self._array("p", payloads), len(payloads),
-                                        self._array("x", params, (self.shapes, torch.float32, True)), self._stream(stream))
+                                        self._array("x", params, self._f32), self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_decode_apply")
 
@@ -329,7 +328,7 @@ class DemoTransform:
             return
         self._check_payloads(payloads)
         st = self.lib.demo_decode_signs(self._ctx, self._array("p", payloads), len(payloads),
-                                        self._array("s", signs_out, (self.shapes, torch.int8, True)), self._stream(stream))
+                                        self._array("s", signs_out, self._i8), self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_decode_signs")
 
@@ -339,8 +338,8 @@ class DemoTransform:
             if st != 0:
                 raise DemoError(st, "demo_apply_signs")
             return
-        st = self.lib.demo_apply_signs(self._ctx, self._array("s", signs, (self.shapes, torch.int8, True)),
-                                       self._array("x", params, (self.shapes, torch.float32, True)), self._stream(stream))
+        st = self.lib.demo_apply_signs(self._ctx, self._array("s", signs, self._i8),
+                                       self._array("x", params, self._f32), self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_apply_signs")
 
@@ -349,8 +348,8 @@ class DemoTransform:
         flat = lambda ll: [t for l in ll for t in l]  # noqa: E731
         out = ctypes.c_void_p(host_payloads_out.data_ptr()) if host_payloads_out is not None else ctypes.c_void_p()
         st = self.lib.demo_step_host(self._ctx, self._array("hg", flat(host_grads)), self._array("dg", flat(dev_grads)),
-                                     self._array("mm", flat(momentum)), self._array("p", payloads),
-                                     self._array("x", params), out, self._stream(stream))
+                                     self._array("mm", flat(momentum)), self._array("hp", payloads),
+                                     self._array("hx", params), out, self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_step_host")
 

@@ -1,5 +1,6 @@
 // The per-step calls of binding.py without Python between the tensors and the library: a call whose tensors are where they were the last
-// time (their pointers are compared with the arrays that binding.py made and checked then) takes the current stream and enters the
+// time (their pointers are compared with the arrays that binding.py made then) and have the layout that the library assumes (number, type,
+// shape, device, contiguous: looked at in every call, since an address says nothing about them) takes the current stream and enters the
 // library; anything else returns None, and binding.py takes its checked way.
 //
 // What it saves is host time, which is all that a step of small tensors costs: compress of one matrix 5.9 -> 3.9 us, of 50 matrices and 12
@@ -9,10 +10,13 @@
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <cstdint>
+#include <memory>
+#include <vector>
 
 namespace {
 
@@ -41,39 +45,89 @@ bool data_pointer(PyObject *t, std::uintptr_t *out)
 
 enum class Found { error, no, yes };
 
-// The array of pointers that cache[key] = (list, array) holds, if `tensors` lie exactly there.  `hold` keeps it alive.
+// What the library assumes of a list of tensors: contiguous, of one type, on one device (-1: any), of these shapes.
+struct Layouts {
+    at::ScalarType dtype;
+    int device;
+    std::vector<std::vector<std::int64_t>> shapes;
+    bool placed(const at::Tensor &t) const { return device < 0 || (t.is_cuda() && t.device().index() == device); }
+    bool fits(const at::Tensor &t, std::size_t i) const
+    {
+        return i < shapes.size() && t.scalar_type() == dtype && t.sizes() == at::IntArrayRef(shapes[i]) && t.is_contiguous() && placed(t);
+    }
+};
+constexpr const char *LAYOUTS = "paper_2411_19870_b200.layouts";
+void free_layouts(PyObject *capsule) { delete static_cast<Layouts *>(PyCapsule_GetPointer(capsule, LAYOUTS)); }
+
+// layouts(dtype, device index or -1, sequence of shapes): the third part of a cache entry, against which every call's tensors are held
+PyObject *make_layouts(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    if (n != 3 || !THPDtype_Check(a[0])) return PyErr_Format(PyExc_TypeError, "layouts: a dtype, a device index and shapes");
+    auto l = std::make_unique<Layouts>();
+    l->dtype = reinterpret_cast<THPDtype *>(a[0])->scalar_type;
+    l->device = (int)PyLong_AsLong(a[1]);
+    Ref shapes(PySequence_Fast(a[2], "layouts: shapes"));
+    if (!shapes || PyErr_Occurred()) return nullptr;
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(shapes.p); ++i) {
+        Ref shape(PySequence_Fast(PySequence_Fast_GET_ITEM(shapes.p, i), "layouts: a shape"));
+        if (!shape) return nullptr;
+        l->shapes.emplace_back();
+        for (Py_ssize_t d = 0; d < PySequence_Fast_GET_SIZE(shape.p); ++d)
+            l->shapes.back().push_back(PyLong_AsLongLong(PySequence_Fast_GET_ITEM(shape.p, d)));
+    }
+    if (PyErr_Occurred()) return nullptr;
+    PyObject *capsule = PyCapsule_New(l.get(), LAYOUTS, free_layouts);
+    if (capsule) l.release();
+    return capsule;
+    END_HANDLE_TH_ERRORS
+}
+
+// The array of pointers that cache[key] = (list, array, layouts) holds, if `tensors` lie exactly there and fit the layouts.  (An entry
+// without layouts is for tensors that are looked at elsewhere: the payloads.)
 struct Array {
+    PyObject *entry = nullptr;
+    const Layouts *layouts = nullptr;
     Py_buffer view{};
     ~Array()
     {
         if (view.obj) PyBuffer_Release(&view);
+        Py_XDECREF(entry);
     }
     void **data() const { return static_cast<void **>(view.buf); }
 };
 Found lookup(PyObject *cache, PyObject *key, PyObject *tensors, Array *array)
 {
-    PyObject *hit = PyDict_GetItemWithError(cache, key);  // (borrowed; the view below keeps the array)
+    PyObject *hit = PyDict_GetItemWithError(cache, key);  // (borrowed; kept by `array` below)
     if (!hit) return PyErr_Occurred() ? Found::error : Found::no;
-    if (!PyTuple_Check(hit) || PyTuple_GET_SIZE(hit) != 2) return Found::no;
+    if (!PyTuple_Check(hit) || PyTuple_GET_SIZE(hit) < 2 || PyTuple_GET_SIZE(hit) > 3) return Found::no;
+    array->entry = Py_NewRef(hit);
+    if (PyTuple_GET_SIZE(hit) == 3) {
+        array->layouts = static_cast<const Layouts *>(PyCapsule_GetPointer(PyTuple_GET_ITEM(hit, 2), LAYOUTS));
+        if (!array->layouts) return Found::error;
+    }
     if (PyObject_GetBuffer(PyTuple_GET_ITEM(hit, 1), &array->view, PyBUF_SIMPLE) != 0) return Found::error;
     if (!PyList_Check(tensors) && !PyTuple_Check(tensors)) return Found::no;  // (an iterator is left to the checked way)
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(tensors);
     if (array->view.len != n * (Py_ssize_t)sizeof(void *)) return Found::no;
+    if (array->layouts && array->layouts->shapes.size() != (std::size_t)n) return Found::no;
     for (Py_ssize_t i = 0; i < n; ++i) {
         std::uintptr_t p;
         if (i >= PySequence_Fast_GET_SIZE(tensors)) return Found::no;  // (a subclass's data_ptr may have changed the list)
         Ref t(Py_NewRef(PySequence_Fast_GET_ITEM(tensors, i)));
+        if (array->layouts && (!THPVariable_Check(t.p) || !array->layouts->fits(THPVariable_Unpack(t.p), (std::size_t)i))) return Found::no;
         if (!data_pointer(t.p, &p)) return Found::error;
         if (reinterpret_cast<std::uintptr_t>(array->data()[i]) != p) return Found::no;
     }
     return Found::yes;
 }
 
-// Whether (data pointer, size) of a payload is among those that were checked.
-Found payload_known(PyObject *known, PyObject *payload, std::uintptr_t *ptr)
+// Whether a payload is bytes end to end, on the tensors' device, and its (data pointer, size) among those that were checked.
+Found payload_known(PyObject *known, PyObject *payload, const Layouts *tensors, std::uintptr_t *ptr)
 {
     if (!THPVariable_CheckExact(payload)) return Found::no;
     const at::Tensor &t = THPVariable_Unpack(payload);
+    if (t.scalar_type() != at::kByte || !t.is_contiguous() || (tensors && !tensors->placed(t))) return Found::no;
     *ptr = reinterpret_cast<std::uintptr_t>(t.data_ptr());
     Ref key(Py_BuildValue("(KL)", (unsigned long long)*ptr, (long long)t.numel()));
     if (!key) return Found::error;
@@ -111,9 +165,9 @@ PyObject *compress(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (PyErr_Occurred()) return nullptr;
     std::uintptr_t payload = 0;
     Array g, m;
-    Found f = payload_known(a[3], a[9], &payload);
-    if (f == Found::yes) f = lookup(a[2], a[5], a[6], &g);
+    Found f = lookup(a[2], a[5], a[6], &g);
     if (f == Found::yes) f = lookup(a[2], a[7], a[8], &m);
+    if (f == Found::yes) f = payload_known(a[3], a[9], g.layouts, &payload);
     if (f != Found::yes) return slow(f);
     if (!stream_of(a[10], &stream)) return nullptr;
     int st;
@@ -134,12 +188,12 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
     static PyObject *const key_p = PyUnicode_InternFromString("p");
     if (!key_p) return nullptr;
     Array p, x;
-    Found f = lookup(a[2], key_p, a[4], &p);
+    Found f = lookup(a[2], a[5], a[6], &x);
+    if (f == Found::yes) f = lookup(a[2], key_p, a[4], &p);
     for (Py_ssize_t i = 0; f == Found::yes && i < PySequence_Fast_GET_SIZE(a[4]); ++i) {
         std::uintptr_t ptr;
-        f = payload_known(a[3], PySequence_Fast_GET_ITEM(a[4], i), &ptr);
+        f = payload_known(a[3], PySequence_Fast_GET_ITEM(a[4], i), x.layouts, &ptr);
     }
-    if (f == Found::yes) f = lookup(a[2], a[5], a[6], &x);
     if (f != Found::yes) return slow(f);
     if (!stream_of(a[7], &stream)) return nullptr;
     const std::int32_t count = (std::int32_t)(p.view.len / (Py_ssize_t)sizeof(void *));
@@ -174,6 +228,7 @@ PyObject *apply_signs(PyObject *, PyObject *const *a, Py_ssize_t n)
 }
 
 PyMethodDef methods[] = {
+    {"layouts", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(make_layouts)), METH_FASTCALL, nullptr},
     {"compress", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(compress)), METH_FASTCALL, nullptr},
     {"decode", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(decode)), METH_FASTCALL, nullptr},
     {"apply_signs", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(apply_signs)), METH_FASTCALL, nullptr},

@@ -1,5 +1,6 @@
 """The native per-step calls (csrc/calls.cpp) without a device: which calls they take, and what reaches the library."""
 import ctypes
+import types
 
 import pytest
 import torch
@@ -68,3 +69,79 @@ def test_errors_of_the_arguments_are_raised():
         calls.decode("no address", 0, {}, set(), [], "x", [], 0)
     with pytest.raises(AttributeError):
         calls.apply_signs(1, 0, {"s": ([1], (ctypes.c_void_p * 1)(1))}, [object()], [], 0)
+
+
+def views(t):
+    """Tensors at t's address that are not t: another shape, order, type, or part of it."""
+    return {"transposed": t.t(), "columns": t[:, :4], "rows": t[:1], "reshaped": t.view(8, 4), "flat": t.view(-1), "type": t.view(torch.int32),
+            "half": t.view(torch.float16)[:, :8]}
+
+
+@pytest.mark.parametrize("view", sorted(views(torch.zeros(4, 8))))
+def test_a_known_address_with_another_layout_is_not_taken(view):
+    calls, seen = binding.load_calls(), []
+    g, m, x = (torch.zeros(4, 8) for _ in range(3))
+    p = torch.zeros(16, dtype=torch.uint8)
+    f32 = calls.layouts(torch.float32, -1, [(4, 8)])
+    cache = {k: array([t]) + (f32,) for k, t in ((("g", 0), g), (("m", 0), m), ("x", x), ("s", m))}
+    cache["p"] = array([p])
+    known = {(p.data_ptr(), p.numel())}
+    fn = [f(lambda *a: seen.append(a) or 0) for f in (COMPRESS, DECODE, APPLY)]
+    at = [ctypes.cast(f, ctypes.c_void_p).value for f in fn]
+    go = lambda g, m, x, p: (calls.compress(at[0], 0, cache, known, 0, ("g", 0), [g], ("m", 0), [m], p, 0),  # noqa: E731
+                             calls.decode(at[1], 0, cache, known, [p], "x", [x], 0), calls.apply_signs(at[2], 0, cache, [m], [x], 0))
+    assert go(g, m, x, p) == (0, 0, 0) and len(seen) == 3
+    assert go(views(g)[view], m, x, p) == (None, 0, 0)
+    assert go(g, views(m)[view], x, p) == (None, 0, None)
+    assert go(g, m, views(x)[view], p) == (0, None, None)
+    assert go(g, m, x, p.view(torch.int8)) == (None, None, 0)
+    assert go(g, m, x, torch.zeros(32, dtype=torch.uint8).set_(p.untyped_storage(), 0, (4, 4), (1, 4))) == (None, None, 0)
+    assert go(g.as_subclass(Sub), m, x, p) == (0, 0, 0) and go(views(g)[view].as_subclass(Sub), m, x, p) == (None, 0, 0)
+    # the payload is held to the tensors' device as well
+    cache["x"] = cache["x"][:2] + (calls.layouts(torch.float32, 0, [(4, 8)]),)
+    assert go(g, m, x, p)[1:] == (None, None)
+
+
+def test_layouts_refuses_what_it_cannot_read():
+    calls = binding.load_calls()
+    for bad in ((1, -1, []), (torch.float32, "0", []), (torch.float32, -1, 3), (torch.float32, -1, [("a",)]), (torch.float32, -1, [(1 << 70,)])):
+        with pytest.raises((TypeError, OverflowError)):
+            calls.layouts(*bad)
+    with pytest.raises(ValueError):
+        calls.apply_signs(1, 0, {"s": ([], (ctypes.c_void_p * 0)(), "not layouts")}, [], [], 0)
+
+
+@pytest.fixture
+def host_only(monkeypatch):
+    """A DemoTransform of one 4 x 8 tensor around functions that write down what reaches the library."""
+    seen = []
+    apply = APPLY(lambda *a: seen.append("apply") or 0)
+    note = lambda name: lambda *a: seen.append(name) or 0  # noqa: E731
+    lib = types.SimpleNamespace(demo_init=lambda *a: 0, demo_payload_bytes=lambda c: 16, demo_apply_signs=note("apply"), demo_step_host=note("host"),
+                                demo_free=lambda c: None, entry_points={"demo_apply_signs": ctypes.cast(apply, ctypes.c_void_p).value})
+    monkeypatch.setattr(binding, "load_library", lambda: lib)
+    tr = binding.DemoTransform([(4, 8)], chunk=4, topk=1, beta=0.9, lr=0.1, weight_decay=0.0, num_workers=1, device=-1)
+    tr.device, tr.keep, tr.seen = None, apply, seen
+    return tr
+
+
+@pytest.mark.parametrize("view", sorted(views(torch.zeros(4, 8))))
+def test_every_call_checks_the_layout(host_only, view):
+    x, s = torch.zeros(4, 8), torch.zeros(4, 8, dtype=torch.int8)
+    for _ in range(3):
+        host_only.apply_signs([s], [x], stream=1)
+    assert host_only.seen == ["apply"] * 3
+    for args in (([s], [views(x)[view]]), ([s.t()], [x]), ([views(x)[view].as_subclass(Sub)], [x]), ([s], iter([views(x)[view]]))):
+        with pytest.raises(ValueError):
+            host_only.apply_signs(*args, stream=1)
+    assert len(host_only.seen) == 3
+
+
+def test_tensors_of_step_host_are_not_taken_as_checked(host_only):
+    x, s = torch.zeros(4, 8, dtype=torch.int32), torch.zeros(4, 8, dtype=torch.int8)
+    p = torch.zeros(16, dtype=torch.uint8)
+    host_only.apply_signs([s], [torch.zeros(4, 8)], stream=1)
+    host_only.step_host([[x]], [[x]], [[x]], [p], [x], stream=1)
+    with pytest.raises(ValueError):
+        host_only.apply_signs([s], [x], stream=1)
+    assert host_only.seen == ["apply", "host"]
