@@ -223,15 +223,18 @@ class DemoTransform:
         if st != 0:
             self._ctx = ctypes.c_void_p()
             raise DemoError(st, "demo_init" if self.chunk_shapes is None else "demo_init_nd")
-        self._ptr_cache = {}
         self._payload_bytes = int(self.lib.demo_payload_bytes(self._ctx))
-        self._payload_ok = set()   # (data pointer, size) of payload buffers already checked
+        self._payload_ok = set()   # (data pointer, size) of payload buffers whose size was checked
         self._grad, self._f32, self._i8 = (
             (d, self._calls.layouts(d, device, self.shapes))
             for d in (torch.bfloat16 if grad_dtype == DEMO_BF16 else torch.float32, torch.float32, torch.int8))
         # what the calls of csrc/calls.cpp are given: entry points, context, keys of the pointer arrays
         self._fn = self.lib.entry_points
         self._keys = [(("g", w), ("m", w)) for w in range(num_workers)]
+        nowhere = ([], _ptr_array([]))
+        self._ptr_cache = {"x": nowhere + self._f32[1:], "s": nowhere + self._i8[1:]}
+        for kg, km in self._keys:
+            self._ptr_cache[kg], self._ptr_cache[km] = nowhere + self._grad[1:], nowhere + self._f32[1:]
 
     # --- queries -------------------------------------------------------------------------------
     @property
@@ -269,11 +272,11 @@ class DemoTransform:
             self._check_payload(p, "payloads[%d]" % i)
 
     def _check_payload(self, p, what: str) -> None:
-        if p.dtype != torch.uint8 or not p.is_contiguous() or p.numel() < self.payload_bytes or not p.is_cuda \
-                or p.device.index != self.device:
+        n = p.numel()
+        if p.dtype != torch.uint8 or not p.is_contiguous() or n < self._payload_bytes or not p.is_cuda or p.device.index != self.device:
             raise ValueError("%s: need a contiguous uint8 tensor of at least %d bytes on cuda:%d"
                              % (what, self.payload_bytes, self.device))
-        self._payload_ok.add((p.data_ptr(), p.numel()))
+        self._payload_ok.add((p.data_ptr(), n))
 
     @staticmethod
     def _stream(stream) -> ctypes.c_void_p:
@@ -287,8 +290,8 @@ class DemoTransform:
         return None if stream is None else int(getattr(stream, "cuda_stream", stream))
 
     # --- the ABI calls -------------------------------------------------------------------------
-    # Tensors that lie where they lay last, with the layout the library assumes, go straight to it (csrc/calls.cpp); the others, which that
-    # module answers with None, are checked and their pointers noted.
+    # Tensors with the layout the library assumes go straight to it (csrc/calls.cpp); what that module answers with None -- payload buffers not
+    # seen before, subclasses of Tensor that moved, tensors that do not fit -- is checked here.
     def compress(self, worker: int, grads, momentum, payload_out, stream=None) -> None:
         if type(worker) is int and 0 <= worker < self.num_workers:
             kg, km = self._keys[worker]
@@ -313,7 +316,7 @@ class DemoTransform:
                 raise DemoError(st, "demo_decode_apply")
             return
         self._check_payloads(payloads)
-        st = self.lib.demo_decode_apply(self._ctx, self._array("p", payloads), len(payloads),
+        st = self.lib.demo_decode_apply(self._ctx, _ptr_array(_tensor_ptrs(payloads)), len(payloads),
                                         self._array("x", params, self._f32), self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_decode_apply")
@@ -327,7 +330,7 @@ class DemoTransform:
                 raise DemoError(st, "demo_decode_signs")
             return
         self._check_payloads(payloads)
-        st = self.lib.demo_decode_signs(self._ctx, self._array("p", payloads), len(payloads),
+        st = self.lib.demo_decode_signs(self._ctx, _ptr_array(_tensor_ptrs(payloads)), len(payloads),
                                         self._array("s", signs_out, self._i8), self._stream(stream))
         if st != 0:
             raise DemoError(st, "demo_decode_signs")

@@ -1,15 +1,17 @@
-// The per-step calls of binding.py without Python between the tensors and the library: a call whose tensors are where they were the last
-// time (their pointers are compared with the arrays that binding.py made then) and have the layout that the library assumes (number, type,
-// shape, device, contiguous: looked at in every call, since an address says nothing about them) takes the current stream and enters the
-// library; anything else returns None, and binding.py takes its checked way.
+// The per-step calls of binding.py without Python between the tensors and the library: a call whose tensors have the layout that the
+// library assumes (number, type, shape, device, contiguous: looked at in every call, wherever they lie) takes the current stream and enters
+// the library; anything else returns None, and binding.py takes its own way, which says what is wrong.
 //
-// What it saves is host time, which is all that a step of small tensors costs: compress of one matrix 5.9 -> 3.9 us, of 50 matrices and 12
-// vectors (two launches) 23.9 -> 5.9, decode of the same set 16.7 -> 5.8, of 64 payloads 30.3 -> 10.3 (one attribute look-up and method call
-// per tensor and list, the comparison of two Python lists, ctypes' conversion of the arguments, the device and stream queries).
+// What it saves is host time, which is all that a step of small tensors costs (one attribute look-up and method call per tensor and list,
+// the checks in Python, ctypes' conversion of the arguments, the device and stream queries).  Without it -> with it, tensors where the call
+// before had them / tensors elsewhere, whose pointers the library copies to the device: compress of one matrix 5.6 -> 3.0 / 15.5 -> 9.6 us,
+// of 50 matrices and 12 vectors (two launches) 16.3 -> 7.1 / 93 -> 20, decode of the same set 12.2 -> 6.4 / 48 -> 9.8, of 64 payloads
+// 28.4 -> 8.1 / 38.4 -> 11.6.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <c10/util/SmallVector.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -49,11 +51,14 @@ enum class Found { error, no, yes };
 struct Layouts {
     at::ScalarType dtype;
     int device;
-    std::vector<std::vector<std::int64_t>> shapes;
-    bool placed(const at::Tensor &t) const { return device < 0 || (t.is_cuda() && t.device().index() == device); }
-    bool fits(const at::Tensor &t, std::size_t i) const
+    std::vector<std::int64_t> dims;         // shape after shape
+    std::vector<std::size_t> starts = {0};  // of the shapes, and the end
+    Py_ssize_t size() const { return (Py_ssize_t)starts.size() - 1; }
+    bool placed(const at::Tensor &t) const { return device < 0 || t.device() == at::Device(at::kCUDA, (at::DeviceIndex)device); }
+    bool fits(const at::Tensor &t, Py_ssize_t i) const  // (i < size())
     {
-        return i < shapes.size() && t.scalar_type() == dtype && t.sizes() == at::IntArrayRef(shapes[i]) && t.is_contiguous() && placed(t);
+        return t.scalar_type() == dtype && t.sizes() == at::IntArrayRef(dims.data() + starts[i], starts[i + 1] - starts[i]) && t.is_contiguous() &&
+               placed(t);
     }
 };
 constexpr const char *LAYOUTS = "paper_2411_19870_b200.layouts";
@@ -72,9 +77,9 @@ PyObject *make_layouts(PyObject *, PyObject *const *a, Py_ssize_t n)
     for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(shapes.p); ++i) {
         Ref shape(PySequence_Fast(PySequence_Fast_GET_ITEM(shapes.p, i), "layouts: a shape"));
         if (!shape) return nullptr;
-        l->shapes.emplace_back();
         for (Py_ssize_t d = 0; d < PySequence_Fast_GET_SIZE(shape.p); ++d)
-            l->shapes.back().push_back(PyLong_AsLongLong(PySequence_Fast_GET_ITEM(shape.p, d)));
+            l->dims.push_back(PyLong_AsLongLong(PySequence_Fast_GET_ITEM(shape.p, d)));
+        l->starts.push_back(l->dims.size());
     }
     if (PyErr_Occurred()) return nullptr;
     PyObject *capsule = PyCapsule_New(l.get(), LAYOUTS, free_layouts);
@@ -83,19 +88,21 @@ PyObject *make_layouts(PyObject *, PyObject *const *a, Py_ssize_t n)
     END_HANDLE_TH_ERRORS
 }
 
-// The array of pointers that cache[key] = (list, array, layouts) holds, if `tensors` lie exactly there and fit the layouts.  (An entry
-// without layouts is for tensors that are looked at elsewhere: the payloads.)
+// The pointers of a list of tensors, and the cache entry that they were held against.
 struct Array {
     PyObject *entry = nullptr;
     const Layouts *layouts = nullptr;
+    c10::SmallVector<void *, 64> pointers;
     Py_buffer view{};
     ~Array()
     {
         if (view.obj) PyBuffer_Release(&view);
         Py_XDECREF(entry);
     }
-    void **data() const { return static_cast<void **>(view.buf); }
+    void **data() { return pointers.data(); }
 };
+// cache[key] = (list, array of pointers, layouts).  Tensors proper are held against the layouts.  A subclass answers for itself, in Python:
+// it has to lie where it lay when binding.py asked it last, which is what the array says.  (So does everything under an entry without layouts.)
 Found lookup(PyObject *cache, PyObject *key, PyObject *tensors, Array *array)
 {
     PyObject *hit = PyDict_GetItemWithError(cache, key);  // (borrowed; kept by `array` below)
@@ -106,18 +113,33 @@ Found lookup(PyObject *cache, PyObject *key, PyObject *tensors, Array *array)
         array->layouts = static_cast<const Layouts *>(PyCapsule_GetPointer(PyTuple_GET_ITEM(hit, 2), LAYOUTS));
         if (!array->layouts) return Found::error;
     }
-    if (PyObject_GetBuffer(PyTuple_GET_ITEM(hit, 1), &array->view, PyBUF_SIMPLE) != 0) return Found::error;
-    if (!PyList_Check(tensors) && !PyTuple_Check(tensors)) return Found::no;  // (an iterator is left to the checked way)
+    const Layouts *l = array->layouts;
+    if (!PyList_Check(tensors) && !PyTuple_Check(tensors)) return Found::no;  // (an iterator is left to binding.py)
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(tensors);
-    if (array->view.len != n * (Py_ssize_t)sizeof(void *)) return Found::no;
-    if (array->layouts && array->layouts->shapes.size() != (std::size_t)n) return Found::no;
+    if (l && l->size() != n) return Found::no;
+    auto known = [&]() {  // the array, asked for once; null with a Python error set
+        if (!array->view.obj && PyObject_GetBuffer(PyTuple_GET_ITEM(array->entry, 1), &array->view, PyBUF_SIMPLE) != 0) return false;
+        return true;
+    };
+    if (!l) {
+        if (!known()) return Found::error;
+        if (array->view.len != n * (Py_ssize_t)sizeof(void *)) return Found::no;
+    }
     for (Py_ssize_t i = 0; i < n; ++i) {
-        std::uintptr_t p;
         if (i >= PySequence_Fast_GET_SIZE(tensors)) return Found::no;  // (a subclass's data_ptr may have changed the list)
-        Ref t(Py_NewRef(PySequence_Fast_GET_ITEM(tensors, i)));
-        if (array->layouts && (!THPVariable_Check(t.p) || !array->layouts->fits(THPVariable_Unpack(t.p), (std::size_t)i))) return Found::no;
-        if (!data_pointer(t.p, &p)) return Found::error;
-        if (reinterpret_cast<std::uintptr_t>(array->data()[i]) != p) return Found::no;
+        PyObject *t = PySequence_Fast_GET_ITEM(tensors, i);
+        if (l && THPVariable_CheckExact(t)) {
+            const at::Tensor &v = THPVariable_Unpack(t);
+            if (!l->fits(v, i)) return Found::no;
+            array->pointers.push_back(v.data_ptr());
+            continue;
+        }
+        Ref hold(Py_NewRef(t));
+        std::uintptr_t p;
+        if (l && (!THPVariable_Check(t) || !l->fits(THPVariable_Unpack(t), i))) return Found::no;
+        if (!known() || !data_pointer(t, &p)) return Found::error;
+        if ((i + 1) * (Py_ssize_t)sizeof(void *) > array->view.len || static_cast<std::uintptr_t *>(array->view.buf)[i] != p) return Found::no;
+        array->pointers.push_back(reinterpret_cast<void *>(p));
     }
     return Found::yes;
 }
@@ -185,18 +207,18 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (n != 8) return PyErr_Format(PyExc_TypeError, "decode: 8 arguments");
     void *fn = PyLong_AsVoidPtr(a[0]), *ctx = PyLong_AsVoidPtr(a[1]), *stream = nullptr;
     if (PyErr_Occurred()) return nullptr;
-    static PyObject *const key_p = PyUnicode_InternFromString("p");
-    if (!key_p) return nullptr;
-    Array p, x;
+    if (!PyList_Check(a[4]) && !PyTuple_Check(a[4])) Py_RETURN_NONE;
+    Array x;
+    c10::SmallVector<void *, 64> p;
     Found f = lookup(a[2], a[5], a[6], &x);
-    if (f == Found::yes) f = lookup(a[2], key_p, a[4], &p);
     for (Py_ssize_t i = 0; f == Found::yes && i < PySequence_Fast_GET_SIZE(a[4]); ++i) {
         std::uintptr_t ptr;
         f = payload_known(a[3], PySequence_Fast_GET_ITEM(a[4], i), x.layouts, &ptr);
+        if (f == Found::yes) p.push_back(reinterpret_cast<void *>(ptr));
     }
     if (f != Found::yes) return slow(f);
     if (!stream_of(a[7], &stream)) return nullptr;
-    const std::int32_t count = (std::int32_t)(p.view.len / (Py_ssize_t)sizeof(void *));
+    const std::int32_t count = (std::int32_t)p.size();
     int st;
     Py_BEGIN_ALLOW_THREADS
     st = reinterpret_cast<DecodeFn>(fn)(ctx, p.data(), count, x.data(), stream);

@@ -115,9 +115,9 @@ def test_layouts_refuses_what_it_cannot_read():
 def host_only(monkeypatch):
     """A DemoTransform of one 4 x 8 tensor around functions that write down what reaches the library."""
     seen = []
-    apply = APPLY(lambda *a: seen.append("apply") or 0)
+    apply = APPLY(lambda *a: seen.append("native") or 0)
     note = lambda name: lambda *a: seen.append(name) or 0  # noqa: E731
-    lib = types.SimpleNamespace(demo_init=lambda *a: 0, demo_payload_bytes=lambda c: 16, demo_apply_signs=note("apply"), demo_step_host=note("host"),
+    lib = types.SimpleNamespace(demo_init=lambda *a: 0, demo_payload_bytes=lambda c: 16, demo_apply_signs=note("python"), demo_step_host=note("host"),
                                 demo_free=lambda c: None, entry_points={"demo_apply_signs": ctypes.cast(apply, ctypes.c_void_p).value})
     monkeypatch.setattr(binding, "load_library", lambda: lib)
     tr = binding.DemoTransform([(4, 8)], chunk=4, topk=1, beta=0.9, lr=0.1, weight_decay=0.0, num_workers=1, device=-1)
@@ -130,7 +130,7 @@ def test_every_call_checks_the_layout(host_only, view):
     x, s = torch.zeros(4, 8), torch.zeros(4, 8, dtype=torch.int8)
     for _ in range(3):
         host_only.apply_signs([s], [x], stream=1)
-    assert host_only.seen == ["apply"] * 3
+    assert host_only.seen == ["native"] * 3
     for args in (([s], [views(x)[view]]), ([s.t()], [x]), ([views(x)[view].as_subclass(Sub)], [x]), ([s], iter([views(x)[view]]))):
         with pytest.raises(ValueError):
             host_only.apply_signs(*args, stream=1)
@@ -144,4 +144,39 @@ def test_tensors_of_step_host_are_not_taken_as_checked(host_only):
     host_only.step_host([[x]], [[x]], [[x]], [p], [x], stream=1)
     with pytest.raises(ValueError):
         host_only.apply_signs([s], [x], stream=1)
-    assert host_only.seen == ["apply", "host"]
+    assert host_only.seen == ["native", "host"]
+
+
+@pytest.mark.parametrize("n", [1, 5, 70])
+def test_tensors_at_new_addresses_take_the_native_way(n):
+    calls, seen = binding.load_calls(), []
+    f32 = calls.layouts(torch.float32, -1, [(4, 8 + i) for i in range(n)])
+    cache = {k: ([], (ctypes.c_void_p * 0)(), f32) for k in (("g", 0), ("m", 0), "x", "s")}
+    fn = (COMPRESS(lambda *a: seen.append([a[1], pointers(a[2], n), pointers(a[3], n), a[4]]) or 0),
+          DECODE(lambda *a: seen.append([pointers(a[1], a[2]), pointers(a[3], n)]) or 0), APPLY(lambda *a: seen.append([pointers(a[1], n), pointers(a[2], n)]) or 0))
+    at = [ctypes.cast(f, ctypes.c_void_p).value for f in fn]
+    keep = []
+    for _ in range(3):
+        g, m, x = ([torch.zeros(4, 8 + i) for i in range(n)] for _ in range(3))
+        p = [torch.zeros(16, dtype=torch.uint8) for _ in range(n)]
+        known = {(t.data_ptr(), t.numel()) for t in p}
+        keep += [g, m, x, p]  # (so that the next ones lie elsewhere)
+        G, M, X, P = ([t.data_ptr() for t in v] for v in (g, m, x, p))
+        assert calls.compress(at[0], 0, cache, known, 0, ("g", 0), g, ("m", 0), tuple(m), p[-1], 0) == 0 and seen.pop() == [0, G, M, P[-1]]
+        assert calls.decode(at[1], 0, cache, known, tuple(p), "x", x, 0) == 0 and seen.pop() == [P, X]
+        assert calls.apply_signs(at[2], 0, cache, m, x, 0) == 0 and seen.pop() == [M, X]
+        # a payload not seen before, a subclass that was never asked, a list that is too short or too long
+        assert calls.decode(at[1], 0, cache, known, p + [torch.zeros(16, dtype=torch.uint8)], "x", x, 0) is None
+        assert calls.apply_signs(at[2], 0, cache, m[:-1] + [m[-1].as_subclass(Sub)], x, 0) is None
+        assert calls.apply_signs(at[2], 0, cache, m[:-1], x, 0) is None and calls.apply_signs(at[2], 0, cache, m, x + x[:1], 0) is None
+    assert not seen
+
+
+def test_a_subclass_takes_the_native_way_where_it_was_asked(host_only):
+    s, x = torch.zeros(4, 8, dtype=torch.int8), torch.zeros(4, 8).as_subclass(Sub)
+    for _ in range(3):
+        host_only.apply_signs([s], [x], stream=1)
+    x.shift = 16
+    host_only.apply_signs([s], [x], stream=1)
+    host_only.apply_signs([s], [torch.zeros(4, 8)], stream=1)
+    assert host_only.seen == ["python", "native", "native", "python", "native"]
