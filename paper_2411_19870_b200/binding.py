@@ -1,4 +1,5 @@
-"""ctypes binding of the C ABI in ``include/demo.h`` -- argument marshalling only.
+"""Binding of the C ABI in ``include/demo.h`` -- argument checks and marshalling only: through ctypes, and for the per-step
+calls through an extension module (``csrc/calls.cpp``, ``load_calls()``) that spares them the Python between the tensors and the library.
 
 ``load_library()`` opens ``libdemo_b200.so`` (built in-tree by ``build.py``) and fails loudly if it
 is missing: there is no CPU or eager fallback.  ``DemoTransform`` wraps one ``demo_ctx`` and turns
@@ -8,6 +9,7 @@ lists of torch tensors into the pointer arrays the ABI takes; method names follo
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import List, Optional, Sequence
 
@@ -129,13 +131,18 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
 
 
 def load_calls():
-    """The extension module of the per-step calls (csrc/calls.cpp).  Raises if it is absent."""
+    """The extension module of the per-step calls (csrc/calls.cpp) for the running Python and torch, whose internals are
+    compiled into it.  Raises if it is absent; one that was built for others is not loaded."""
     global _calls
     if _calls is None:
-        path = os.path.join(os.path.dirname(LIB_PATH), "_calls.so")
+        from .build import calls_path
+
+        path = calls_path()
         if not os.path.exists(path):
             raise RuntimeError("%s is missing: build it with `python -m paper_2411_19870_b200.build`" % path)
-        from . import _calls as module
+        spec = importlib.util.spec_from_file_location(__package__ + "._calls", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
         _calls = module
     return _calls
 

@@ -2,8 +2,9 @@
 
 ``python -m paper_2411_19870_b200.build`` or ``build_library()`` compiles every ``csrc/*.cu`` into
 ``build/*.o`` and links ``libdemo_b200.so`` next to this file; ``build_calls()`` compiles ``csrc/calls.cpp``, the
-extension module behind the per-step calls of ``binding.py``, into ``_calls.so``.  Objects are rebuilt only when a
-source or header is newer.
+extension module behind the per-step calls of ``binding.py``, into ``_calls.<python>.<torch>.so``.  Objects are rebuilt only
+when a source or header is newer.  The library needs nvcc; the module needs a C++ compiler, Python's headers and a CUDA build
+of torch, and belongs to the Python and torch that its name says: their internals are compiled into it.
 """
 from __future__ import annotations
 
@@ -19,7 +20,6 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libdemo_b200.so")
-CALLS = os.path.join(HERE, "_calls.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 NVCC_FLAGS = [
@@ -75,10 +75,17 @@ def build_library(force: bool = False, verbose: bool = False, ptxas_info: bool =
     return LIB
 
 
+def calls_path() -> str:
+    """Where the call module of the running Python and torch lies."""
+    import torch
+
+    return os.path.join(HERE, "_calls.%s.torch-%s.so" % (sysconfig.get_config_var("SOABI"), torch.__version__.replace("+", "-")))
+
+
 def build_calls(force: bool = False) -> str:
-    src = os.path.join(CSRC, "calls.cpp")
-    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= os.path.getmtime(src):
-        return CALLS
+    src, out = os.path.join(CSRC, "calls.cpp"), calls_path()
+    if not force and os.path.exists(out) and os.path.getmtime(out) >= max(os.path.getmtime(src), os.path.getmtime(os.path.abspath(__file__))):
+        return out
     import torch
     from torch.utils import cpp_extension
 
@@ -87,7 +94,7 @@ def build_calls(force: bool = False) -> str:
         raise RuntimeError("no C++ compiler: the call module cannot be built")
     torch_lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     cuda = os.path.dirname(os.path.dirname(_nvcc()))
-    tmp = CALLS + ".tmp.%d" % os.getpid()
+    tmp = out + ".tmp.%d" % os.getpid()
     cmd = [cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
     for inc in cpp_extension.include_paths() + [os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]:
         cmd += ["-isystem", inc]
@@ -96,8 +103,8 @@ def build_calls(force: bool = False) -> str:
     if r.returncode != 0:
         sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         raise RuntimeError("the C++ compiler failed for " + src)
-    os.replace(tmp, CALLS)
-    return CALLS
+    os.replace(tmp, out)
+    return out
 
 
 if __name__ == "__main__":

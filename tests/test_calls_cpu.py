@@ -5,7 +5,7 @@ import types
 import pytest
 import torch
 
-from paper_2411_19870_b200 import binding
+from paper_2411_19870_b200 import binding, build
 
 COMPRESS = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
 DECODE = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p)
@@ -109,6 +109,26 @@ def test_layouts_refuses_what_it_cannot_read():
             calls.layouts(*bad)
     with pytest.raises(ValueError):
         calls.apply_signs(1, 0, {"s": ([], (ctypes.c_void_p * 0)(), "not layouts")}, [], [], 0)
+
+
+def test_a_module_of_another_python_or_torch_is_not_loaded(monkeypatch):
+    """Their internals are compiled into it: only the one whose name says the running versions counts as built, and is loaded."""
+    binding.load_calls()
+    own = build.calls_path()
+    ran = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **k: ran.append(cmd) or types.SimpleNamespace(returncode=1, stdout="", stderr=""))
+    assert build.build_calls() == own and not ran
+    for target, name, value in ((torch, "__version__", "9.9.0+cu999"), (build.sysconfig, "get_config_var", lambda n: "cpython-399-x86_64-linux-gnu")):
+        with monkeypatch.context() as m:
+            m.setattr(target, name, value)
+            assert build.calls_path() != own
+            with pytest.raises(RuntimeError):
+                build.build_calls()
+            assert len(ran) == 1 and ran.pop()[0].endswith("g++")
+            m.setattr(binding, "_calls", None)
+            with pytest.raises(RuntimeError, match="missing"):
+                binding.load_calls()
+    assert build.calls_path() == own
 
 
 @pytest.fixture
