@@ -1008,6 +1008,7 @@ demo_status demo_set_basis(demo_ctx *ctx, const float *basis_host, void *cuda_st
         cudaGetLastError();
         return DEMO_ERR_CUDA;
     }
+    ctx->launches += 1;
     ctx->custom_basis = true;
     return DEMO_OK;
 }

@@ -545,6 +545,17 @@ def test_tensor_core_kernels_on_tie_maker_chunks(basis_kind):
     r.close()
 
 
+def test_launches_of_the_basis_calls_are_counted():
+    """One kernel each for a caller's basis (its transpose) and a Gaussian one; none for the way back to the DCT."""
+    tr = demo.DemoTransform([(16, 16)], chunk=8, topk=4, beta=0.9, lr=0.1, weight_decay=0.0, num_workers=1)
+    counts = [tr.launch_count]
+    for call in (lambda: tr.set_basis(torch.eye(8)), lambda: tr.set_basis_gaussian(inputs.basis_gaussian(1, 8)), tr.set_basis, tr.get_basis):
+        call()
+        counts.append(tr.launch_count)
+    assert counts == [0, 1, 2, 2, 2]
+    tr.close()
+
+
 def test_basis_argument_errors_keep_the_previous_basis():
     s = 8
     wl = inputs.Workload("basis-err", [(2 * s, 2 * s)], chunk=s, topk=4, num_workers=1, grad_kind="normal", grad_std=0.01)
