@@ -458,7 +458,10 @@ cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t st
     // look-ups spread the requests.  Steps, early / late / before both: 280 chunks of 9 tensors, seven workers 92.5 / 99.9 / 101.7 us; 800 of
     // 23, two workers 48.1 / 44.3 / 46.0; 976 of 57, six workers 135 / 120 / 120; 1424 of 30, six workers 170.5 / 158.5 / 167.1; 2400 of 65,
     // two workers 91.8 / 85.3 / 88.0; 2640 of 72, one worker 60.3 / 60.2 / 63.1; 3328 of 58, three workers 171 / 178 / 173.
-    b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > 4LL * dev.sm_count;
+    // The line lies at two chunks per SM, with up to four tensors, whose maps are few, at four: two workers, 320 of 64 32.9 / 30.8 / 32.7,
+    // 448 of 64 35.9 / 31.5 / 33.2, 560 of 16 37.0 / 33.3 / 34.9, 350 of 10 30.9 / 30.6 / 32.3, 348 of 3 29.0 / 29.1 / 30.8; four workers,
+    // 576 of 36 67.7 / 60.8 / 63.0, 396 of 9 53.4 / 53.5 / 55.4, 400 of 4 51.3 / 55.4 / 56.0.
+    b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > (a.n_entries > 4 ? 2LL : 4LL) * dev.sm_count;
     void *params[] = {&b};
     return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
 }

@@ -1,5 +1,6 @@
 """Edges of the size ranges the kernel variants are chosen by, against the fp64 oracle (rules and tolerances of
 tests/parity.py, every chunk)."""
+import contextlib
 import ctypes
 import math
 import types
@@ -607,3 +608,32 @@ def test_nd_rows_and_lines(shape, chunk, k, f32):
     for _ in range(2):
         r.step()
     r.close()
+
+
+def test_compress_time_of_several_tensors_below_four_chunks_per_sm():
+    """s = 64, sets of 16-chunk tensors: 576 chunks are compressed in 0.91 of the time of 640, as their number says.  (1.01 where their first
+    chunks, below four per SM, were all looked up and requested in the same moment.)"""
+    import paper_2411_19870_b200 as demo
+
+    times = {}
+    for n in (36, 40):
+        tr = demo.DemoTransform([(256, 256)] * n, chunk=64, topk=32, beta=0.9, lr=0.1, weight_decay=0.1, num_workers=4)
+        sets = [[[torch.randn((256, 256), device="cuda").to(d) for _ in range(n)] for d in (torch.bfloat16, torch.float32)] for _ in range(4)]
+        pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(4)]
+        graph = torch.cuda.CUDAGraph()
+        for captured in (False, True):
+            with torch.cuda.graph(graph) if captured else contextlib.nullcontext():
+                for w, (g, m) in enumerate(sets):
+                    tr.compress(w, g, m, pay[w])
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        times[n] = math.inf
+        for _ in range(10):
+            t0.record()
+            for _ in range(20):
+                graph.replay()
+            t1.record()
+            torch.cuda.synchronize()
+            times[n] = min(times[n], t0.elapsed_time(t1))
+        del graph
+        tr.close()
+    assert times[36] <= 0.96 * times[40], times
