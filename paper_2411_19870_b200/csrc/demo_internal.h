@@ -154,10 +154,11 @@ struct DemoNdClass {
     int dense_axes;      // some extent is a dense contraction from a table (second tile)
     int big;             // some extent is 128: the variant with 64 registers per half line
 };
-// Coefficient tables of the dense extents in use, and the tile layouts of the chunk shapes planned so far.
+// Coefficient tables of the dense extents in use, and the tile layouts of the chunk shapes planned so far: `rows` is what the search reads of
+// the tensor beside them (demo_nd_plan).
 struct DemoNdTables {
     struct Layout {
-        int s[DEMO_ND_DIMS], p[DEMO_ND_DIMS], tile;
+        int s[DEMO_ND_DIMS], p[DEMO_ND_DIMS], tile, rows;
     };
     std::vector<float> data;
     std::vector<Layout> layouts;

@@ -1470,7 +1470,7 @@ int DemoNdTables::get(int s)
 // Tile strides: the innermost axis is dense, every outer stride may be padded by a few words.  The padding is the one with
 // the fewest bank conflicts of a warp's accesses over the axis passes (32 neighbouring lines at a time), the smaller tile
 // where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it, an eighth where it makes the rows whole quads.  The search takes 10
-// to 130 us of the host's time, so tensors of the same chunk shape share one.
+// to 130 us of the host's time, so tensors of the same chunk shape, whose rows are pieces of the tensor alike, share one.
 void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
 {
     const int *s = e->s;
@@ -1526,9 +1526,25 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
         // (rows that are not whole pieces cost four accesses instead of one where the chunk comes and goes)
         return 2 * cost + (whole ? 0 : 2);
     };
+    // What quads_of reads of the tensor, so that a layout does not depend on which tensor of a chunk shape came first: the first axis from which
+    // on the chunk is one piece of the tensor and the strides that are whole quads; 0 where chunks start off the pieces, whatever the tile.
+    int rows = 1;
+    {
+        long long in = 1;
+        int axis = DEMO_ND_DIMS;
+        bool joined = true;
+        for (int a = DEMO_ND_DIMS - 1; a >= 0; --a) {
+            if (e->c[a] > 1 && s[a] * e->stride[a] % 4) rows = 0;
+            joined = joined && (s[a] == 1 || e->stride[a] == in);
+            if (joined) axis = a;
+            if (rows && s[a] > 1 && e->stride[a] % 4 == 0) rows |= 16 << a;
+            in *= s[a];
+        }
+        if (rows) rows |= axis << 1;
+    }
     const DemoNdTables::Layout *known = nullptr;
     for (const DemoNdTables::Layout &l : tables->layouts)
-        if (l.s[0] == s[0] && l.s[1] == s[1] && l.s[2] == s[2] && l.s[3] == s[3]) known = &l;
+        if (l.s[0] == s[0] && l.s[1] == s[1] && l.s[2] == s[2] && l.s[3] == s[3] && l.rows == rows) known = &l;
     const int room = e->M / 16 > 64 ? e->M / 16 : 64, room_quads = e->M / 8 > room ? e->M / 8 : room;
     long long best = -1;
     int p[DEMO_ND_DIMS];
@@ -1562,6 +1578,7 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
             l.p[a] = e->p[a];
         }
         l.tile = e->tile;
+        l.rows = rows;
         tables->layouts.push_back(l);
     }
     long long span = 0;
@@ -1652,7 +1669,7 @@ void demo_nd_classify(std::vector<DemoNdEntry> &entries, int sm_count, std::vect
     classes->clear();
     auto same_layout = [](const DemoNdEntry &x, const DemoNdEntry &y) {
         for (int a = 0; a < DEMO_ND_DIMS; ++a)
-            if (x.s[a] != y.s[a] || x.stride[a] != y.stride[a]) return false;  // (the tile follows from these)
+            if (x.s[a] != y.s[a] || x.stride[a] != y.stride[a] || x.p[a] != y.p[a]) return false;
         return true;
     };
     auto emit_part = [&](const Group &d, size_t first, size_t last) {  // tensors first .. last - 1

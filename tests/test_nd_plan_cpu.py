@@ -77,6 +77,40 @@ def test_tensors_of_one_chunk_shape_are_planned_once(tmp_path):
     assert float(out[2]) < 20 * float(out[1])  # a hundred further tensors
 
 
+def test_a_layout_does_not_depend_on_the_order_of_the_tensors(tmp_path):
+    """Chunks of one shape whose rows are whole 16-byte pieces of one tensor and not of the other: planned alone, first and second, every tensor
+    gets the same tile and the same rows."""
+    out = run(tmp_path, """
+    const int s[][4] = {{1, 1, 32, 6}, {1, 1, 16, 12}, {1, 4, 6, 10}, {1, 8, 12, 5}};
+    const long long n[][4][4] = {{{1, 1, 4096, 6}, {1, 1, 64, 18}, {1, 1, 32, 6}, {1, 1, 64, 12}},
+                                 {{1, 1, 64, 24}, {1, 1, 64, 12}, {1, 1, 16, 36}, {1, 1, 32, 12}},
+                                 {{1, 8, 12, 20}, {1, 8, 6, 10}, {1, 4, 6, 30}, {1, 16, 18, 10}},
+                                 {{1, 64, 12, 5}, {1, 8, 24, 5}, {1, 16, 12, 10}, {1, 8, 12, 5}}};
+    auto same = [](const DemoNdEntry &a, const DemoNdEntry &b) {
+        for (int d = 0; d < 4; ++d)
+            if (a.p[d] != b.p[d]) return false;
+        return a.tile == b.tile && a.row == b.row && a.quads == b.quads && a.row_table == b.row_table && a.threads == b.threads;
+    };
+    int differ = 0, kinds = 0;
+    for (int k = 0; k < 4; ++k)
+        for (int i = 0; i < 4; ++i) {
+            DemoNdTables own;
+            DemoNdEntry alone = entry(s[k], n[k][i], 32);
+            demo_nd_plan(&alone, &own);
+            kinds |= 1 << alone.quads;
+            for (int j = 0; j < 4; ++j) {
+                DemoNdTables tables;
+                DemoNdEntry first = entry(s[k], n[k][j], 32), second = entry(s[k], n[k][i], 32);
+                demo_nd_plan(&first, &tables);
+                demo_nd_plan(&second, &tables);
+                differ += !same(alone, second);
+            }
+        }
+    std::printf("%d %d", differ, kinds);
+    """)
+    assert out == ["0", "5"]
+
+
 def test_classes_stay_below_the_range_of_the_chunk_counters(tmp_path):
     """Three tensors of 2^31 - 1 chunks and a small one, all of one kind: no class of 2^31 chunks or more, every tensor in one class, its
     chunks consecutive."""
