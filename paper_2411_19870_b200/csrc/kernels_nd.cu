@@ -1469,8 +1469,9 @@ int DemoNdTables::get(int s)
 
 // Tile strides: the innermost axis is dense, every outer stride may be padded by a few words.  The padding is the one with
 // the fewest bank conflicts of a warp's accesses over the axis passes (32 neighbouring lines at a time), the smaller tile
-// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it, an eighth where it makes the rows whole quads.  The search takes 10
-// to 130 us of the host's time, so tensors of the same chunk shape, whose rows are pieces of the tensor alike, share one.
+// where that is equal; at most a sixteenth of the chunk (or 64 words) is spent on it, an eighth where it makes the rows whole quads.  The
+// search takes 1 to 60 us of the host's time, 190 for 4 x 8 x 8 x 16, so tensors of the same chunk shape, whose rows are pieces of the tensor
+// alike, share one.  (The lines' indices are found once: with the divisions in every trial, fourteen shapes took 1070 us instead of 550.)
 void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
 {
     const int *s = e->s;
@@ -1500,27 +1501,46 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
         }
         return tile ? 2 : 1;
     };
-    auto conflicts = [&](const int *p, bool whole) {
-        long long cost = 0;
+    // The lines of the first, second and third warp of each axis pass, as indices along the axes (which the strides tried below do not change).
+    struct Pass {
+        bool pieces;  // may be 16 bytes per thread, eight threads at a time
+        int weight, lines, index[96][DEMO_ND_DIMS];
+    };
+    auto passes_of = [&](Pass *passes) {
+        int n = 0;
         for (int a = 0; a < DEMO_ND_DIMS; ++a) {
             if (s[a] == 1 || (e->tail && a == 3)) continue;
             const int last = e->tail && a == 2 ? 3 : a;
-            const int lines = e->M / (s[a] * (last > a ? s[last] : 1));
-            const bool pieces = whole && a == 3 && s[a] % 4 == 0 && in_place_extent(s[a]) && s[a] <= 32;  // 16 bytes per thread, eight threads at a time
+            Pass &q = passes[n++];
+            q.pieces = a == 3 && s[a] % 4 == 0 && in_place_extent(s[a]) && s[a] <= 32;
+            q.weight = last > a ? 2 : 1;
+            q.lines = e->M / (s[a] * (last > a ? s[last] : 1));
+            if (q.lines > 96) q.lines = 96;
+            for (int l = 0; l < q.lines; ++l) {
+                int r = l;
+                for (int b = DEMO_ND_DIMS - 1; b >= 0; --b) {
+                    const bool across = b < a || b > last;
+                    q.index[l][b] = across ? r % s[b] : 0;
+                    if (across) r /= s[b];
+                }
+            }
+        }
+        return n;
+    };
+    auto conflicts = [](const Pass *passes, int n, const int *p, bool whole) {
+        long long cost = 0;
+        for (const Pass *q = passes; q < passes + n; ++q) {
+            const bool pieces = whole && q->pieces;
             const int lanes = pieces ? 8 : 32, banks = pieces ? 8 : 32;
-            for (int w = 0; w < 3 && w * 32 < lines; ++w) {  // the first, second and third warp's lines
-                int bank[32] = {0}, worst = 0;
-                for (int l = 32 * w; l < lines && l < 32 * w + lanes; ++l) {
-                    int r = l, t = 0;
-                    for (int b = DEMO_ND_DIMS - 1; b >= 0; --b)
-                        if (b < a || b > last) {
-                            t += (r % s[b]) * p[b];
-                            r /= s[b];
-                        }
+            for (int first = 0; first < q->lines; first += 32) {
+                unsigned char bank[32] = {0};
+                int worst = 0;
+                for (int l = first; l < q->lines && l < first + lanes; ++l) {
+                    const int *x = q->index[l], t = x[0] * p[0] + x[1] * p[1] + x[2] * p[2] + x[3] * p[3];
                     const int v = ++bank[(pieces ? t >> 2 : t) & (banks - 1)];
                     worst = worst > v ? worst : v;
                 }
-                cost += worst * (last > a ? 2 : 1);
+                cost += worst * q->weight;
             }
         }
         // (rows that are not whole pieces cost four accesses instead of one where the chunk comes and goes)
@@ -1549,6 +1569,8 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
     long long best = -1;
     int p[DEMO_ND_DIMS];
     p[3] = 1;
+    Pass passes[DEMO_ND_DIMS];
+    const int n_passes = known ? 0 : passes_of(passes);
     for (int pad2 = 0; !known && pad2 <= (s[2] > 1 && !e->tail ? 8 : 0); ++pad2) {
         p[2] = s[3] + pad2;
         for (int pad1 = 0; pad1 <= (s[1] > 1 && s[2] * s[3] > 1 ? 8 : 0); ++pad1) {
@@ -1557,9 +1579,9 @@ void demo_nd_plan(DemoNdEntry *e, DemoNdTables *tables)
                 p[0] = p[1] * s[1] + pad0;
                 const int floats = p[0] * s[0];
                 if (floats > e->M + room_quads) break;
-                const bool whole = quads_of(p) == 2;
+                const bool whole = rows && quads_of(p) == 2;
                 if (floats > e->M + room && !whole) continue;
-                const long long cost = conflicts(p, whole) * (1LL << 20) + floats;
+                const long long cost = conflicts(passes, n_passes, p, whole) * (1LL << 20) + floats;
                 if (best < 0 || cost < best) {
                     best = cost;
                     for (int a = 0; a < DEMO_ND_DIMS; ++a) e->p[a] = p[a];
