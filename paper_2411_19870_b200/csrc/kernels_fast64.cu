@@ -461,12 +461,7 @@ cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t st
     // The line lies at two chunks per SM, with up to four tensors, whose maps are few, at four: two workers, 320 of 64 32.9 / 30.8 / 32.7,
     // 448 of 64 35.9 / 31.5 / 33.2, 560 of 16 37.0 / 33.3 / 34.9, 350 of 10 30.9 / 30.6 / 32.3, 348 of 3 29.0 / 29.1 / 30.8; four workers,
     // 576 of 36 67.7 / 60.8 / 63.0, 396 of 9 53.4 / 53.5 / 55.4, 400 of 4 51.3 / 55.4 / 56.0.
-    // Transform-domain kernels, with half the work per chunk behind the tiles, lose by the early look-up on sets of more than eight tensors of
-    // any length (up to 1.9 % against none; late, at most 0.3 %): 10240 chunks of 16 tensors, two workers 238.7 / 235.0 / 236.6, 8192 of 9, four
-    // 333.7 / 328.9 / 330.0, 6400 of 64 159.3 / 155.8 / 159.0, 40960 of 16 834.9 / 827.0 / 833.1; against it 10752 of 30 244.9 /
-    // 247.2 / 249.5 and 5120 of 5 135.5 / 136.9 / 136.2.
-    const bool nearly_full = 2 * groups <= 5 * grid && grid > (a.n_entries > 4 ? 2LL : 4LL) * dev.sm_count;
-    b.late_lookup = a.n_entries > 1 && (nearly_full || (a.momentum_dct && a.n_entries > 8 && 2 * groups > 5 * grid));
+    b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > (a.n_entries > 4 ? 2LL : 4LL) * dev.sm_count;
     void *params[] = {&b};
     return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
 }
