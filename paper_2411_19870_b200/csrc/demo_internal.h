@@ -88,12 +88,13 @@ cudaError_t demo_launch_decode_small(int s, const DemoDecodeArgs *segs, const De
                                      cudaStream_t stream);
 // Fast-DCT kernels for 2-D tensors; `supported` tells whether chunk size s has one.
 bool demo_fast_supported(int s);
-cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+// largest: chunks of the list's largest tensor
+cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, long long largest, DemoLaunch &dev, cudaStream_t stream);
 cudaError_t demo_launch_decode_fast(int s, const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);
 // s = 32 (kernels_fast32.cu).
 cudaError_t demo_launch_compress_fast32(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
 // s = 64 with TMA tensor maps (kernels_fast64.cu; cudaErrorNotSupported without them).
-cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
+cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, long long largest, DemoLaunch &dev, cudaStream_t stream);
 // s = 128 (kernels_fast128.cu); compress needs the TMA tensor maps (cudaErrorNotSupported without them).
 cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream);
 cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream);

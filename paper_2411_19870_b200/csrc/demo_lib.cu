@@ -28,7 +28,7 @@ struct demo_ctx {
 
     // work lists
     int n2d = 0, n1d = 0;
-    long long chunks2d = 0, chunks1d = 0;
+    long long chunks2d = 0, chunks1d = 0, largest2d = 0;
     DemoTensorEntry *d_entries2d = nullptr, *d_entries1d = nullptr;
 
     // [W + 1][slots] chunk counters, zero between launches: a row for each worker's compress calls and one for decode, so that compress
@@ -262,6 +262,7 @@ demo_status demo_init(demo_ctx **out, const demo_config *cfg, const demo_tensor_
             e.rec_begin = rec;
             e.chunk_begin = two ? c->chunks2d : c->chunks1d;
             (two ? c->chunks2d : c->chunks1d) += c0 * c1;
+            if (two && c0 * c1 > c->largest2d) c->largest2d = c0 * c1;
             (two ? e2d : e1d).push_back(e);
             c->first_record[t] = rec;
             c->n_chunks[t] = c0 * c1;
@@ -650,7 +651,7 @@ demo_status demo_compress(demo_ctx *ctx, int32_t worker, const void *const *grad
     const bool small_tiles = ctx->n2d && use_small_tiles(ctx);
     if (ctx->n2d && !small_tiles) {
         if (use_fast_path(ctx))
-            err = demo_launch_compress_fast(s, a, ctx->launch, stream);
+            err = demo_launch_compress_fast(s, a, ctx->largest2d, ctx->launch, stream);
         else if (use_tc_path(ctx))
             err = demo_launch_compress_tc(a, ctx->launch, stream);
         else

@@ -416,10 +416,10 @@ cudaError_t demo_launch_wait_selftest(int *status, long long limit_cycles, cudaS
 
 bool demo_fast_supported(int s) { return s == 128 || s == 64 || s == 32; }
 
-cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
+cudaError_t demo_launch_compress_fast(int s, const DemoCompressArgs &a, long long largest, DemoLaunch &dev, cudaStream_t stream)
 {
     if (s == 128) return demo_launch_compress_fast128(a, dev, stream);
-    if (s == 64) return demo_launch_compress_fast64(a, dev, stream);
+    if (s == 64) return demo_launch_compress_fast64(a, largest, dev, stream);
     if (s == 32) return demo_launch_compress_fast32(a, dev, stream);
     return cudaErrorInvalidValue;
 }

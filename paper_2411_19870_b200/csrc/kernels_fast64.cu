@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) compress64_kernel(Demo
 }
 
 template <typename GT, int THREADS, bool QDOM, bool BIGK>
-cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
+cudaError_t launch64(const DemoCompressArgs &a, long long largest, DemoLaunch &dev, cudaStream_t stream)
 {
     constexpr int NCH = THREADS / S;
     auto kernel = compress64_kernel<GT, THREADS, QDOM, BIGK>;
@@ -458,10 +458,14 @@ cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t st
     // look-ups spread the requests.  Steps, early / late / before both: 280 chunks of 9 tensors, seven workers 92.5 / 99.9 / 101.7 us; 800 of
     // 23, two workers 48.1 / 44.3 / 46.0; 976 of 57, six workers 135 / 120 / 120; 1424 of 30, six workers 170.5 / 158.5 / 167.1; 2400 of 65,
     // two workers 91.8 / 85.3 / 88.0; 2640 of 72, one worker 60.3 / 60.2 / 63.1; 3328 of 58, three workers 171 / 178 / 173.
-    // The line lies at two chunks per SM, with up to four tensors, whose maps are few, at four: two workers, 320 of 64 32.9 / 30.8 / 32.7,
-    // 448 of 64 35.9 / 31.5 / 33.2, 560 of 16 37.0 / 33.3 / 34.9, 350 of 10 30.9 / 30.6 / 32.3, 348 of 3 29.0 / 29.1 / 30.8; four workers,
-    // 576 of 36 67.7 / 60.8 / 63.0, 396 of 9 53.4 / 53.5 / 55.4, 400 of 4 51.3 / 55.4 / 56.0.
-    b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > (a.n_entries > 4 ? 2LL : 4LL) * dev.sm_count;
+    // The line lies at four chunks per SM; the more maps, the lower: at three with more than four tensors, at two with more than sixteen, where no
+    // tensor holds more than three quarters of the chunks (few maps again).  Three workers, 540 of 60 46.0 / 39.1 / 39.2, of 9 41.1 / 39.1 /
+    // 39.2, 360 of 60 39.2 / 36.9 / 37.0, 375 of 5 35.1 / 36.9 / 37.0, 432 of 15 39.0 / 41.1 / 41.1 (but 340 of 15 37.0 / 35.1 / 35.2); two, 448 of 64
+    // 35.9 / 31.5 / 33.2, 556 of 15, 500 of them in one, 35.4 / 36.7 / 37.4; four, 576 of 36 67.7 / 60.8 / 63.0, 400 of 4 51.3 / 55.4 / 56.0.  (Not
+    // in the transform domain: 440 of 15, three workers 42.4 early, 43.6 late.)
+    const bool spread = 4 * largest <= 3 * a.n_chunks && !a.momentum_dct;
+    const long long line = (spread && a.n_entries > 16 ? 2LL : spread && a.n_entries > 4 ? 3LL : 4LL) * dev.sm_count;
+    b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > line;
     void *params[] = {&b};
     return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
 }
@@ -469,13 +473,13 @@ cudaError_t launch64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t st
 }  // namespace
 
 // Needs the TMA tensor maps of both tensors.
-cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
+cudaError_t demo_launch_compress_fast64(const DemoCompressArgs &a, long long largest, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.tmap_m == nullptr || a.tmap_g == nullptr) return cudaErrorNotSupported;
     auto pick = [&](auto gt, auto qdom) {
         using GT = decltype(gt);
         constexpr bool Q = decltype(qdom)::value;
-        return a.k > MAX_K_LISTED ? launch64<GT, 64, Q, true>(a, dev, stream) : launch64<GT, 64, Q, false>(a, dev, stream);
+        return a.k > MAX_K_LISTED ? launch64<GT, 64, Q, true>(a, largest, dev, stream) : launch64<GT, 64, Q, false>(a, largest, dev, stream);
     };
     if (a.momentum_dct)
         return a.grad_bf16 ? pick(__nv_bfloat16{}, std::true_type{}) : pick(float{}, std::true_type{});

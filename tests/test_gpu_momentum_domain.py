@@ -113,3 +113,28 @@ def test_refused_where_no_kernel_implements_it():
     r.mom_dct = False  # (the buffers are still all zero: no conversion needed)
     r.step(grads=g)
     r.close()
+
+
+@pytest.mark.parametrize("domain", [demo.DEMO_MOMENTUM_SPATIAL, DCT])
+@pytest.mark.parametrize("tensors,chunks", [(8, 400), (17, 18), (8, 56), (3, 200)])
+def test_one_set_of_tensors_or_each_alone(tensors, chunks, domain):
+    """Where the first chunks are looked up depends on the number of tensors and chunks; records and momentum do not, bit for bit."""
+    gen = torch.Generator("cuda").manual_seed(tensors)
+    g = [torch.randn((64 * chunks, 64), device="cuda", generator=gen).bfloat16() for _ in range(tensors)]
+    m = [torch.randn((64 * chunks, 64), device="cuda", generator=gen) for _ in range(tensors)]
+
+    def run(gs, ms):
+        tr = demo.DemoTransform([t.shape for t in gs], chunk=64, topk=5, beta=0.9, lr=0.1, weight_decay=0.0, num_workers=1)
+        tr.set_momentum_domain(domain)
+        ms = [t.clone() for t in ms]
+        pay = torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda")
+        for _ in range(2):
+            tr.compress(0, gs, ms, pay)
+        assert tr.device_status() == 0
+        tr.close()
+        return torch.cat(ms), pay
+
+    together = run(g, m)
+    alone = [run([a], [b]) for a, b in zip(g, m)]
+    assert torch.equal(together[0], torch.cat([v[0] for v in alone]))
+    assert torch.equal(together[1], torch.cat([v[1] for v in alone]))
