@@ -536,32 +536,38 @@ def test_decode_time_of_long_lists_on_few_small_tiles():
     r.close()
 
 
-@pytest.mark.parametrize("s,grid", [(32, 148 * 8), (64, 148 * 8), (128, 148 * 2)])
-@pytest.mark.parametrize("rounds,extra", [(1, 0), (1, 1), (2, -1), (2, 0), (2, 1), (3, 0), (3, 1), (4, 3)])
-def test_chunks_of_the_first_rounds(s, grid, rounds, extra):
-    """Every chunk is processed once whether a CTA's second chunk is fixed or drawn (up to three rounds of the grid of the decode kernels, or
-    more): one row of chunks in one call against the same chunks as tensors of one to four chunks each, bit for bit, over two calls."""
+@pytest.mark.parametrize("s,per_sm", [(32, 16), (64, 6), (64, 8), (128, 2)])
+@pytest.mark.parametrize("rounds,extra", [(1, 0), (1, 1), (2, -1), (2, 0), (2, 1), (3, -1), (3, 0), (3, 1), (4, 3)])
+def test_chunks_of_the_first_rounds(s, per_sm, rounds, extra):
+    """Every chunk is processed once whether a CTA's second chunk is fixed or drawn (up to three rounds of the decode kernels' grid, or more): one
+    row of chunks in one call against the same chunks in contexts of at most one chunk per SM, whose grids hold them all at once and draw
+    nothing, bit for bit, over two calls.  ``per_sm``: chunks of a round per SM (s = 32: eight CTAs of two; s = 64: eight, six where the senders
+    are counted)."""
     import paper_2411_19870_b200 as demo
 
-    n, k = rounds * grid + extra, 3
-    cut = [n // 2, n - n // 2]
+    sms, k = torch.cuda.get_device_properties(0).multi_processor_count, 3
+    n = rounds * per_sm * sms + extra
     g = torch.randn(s, n * s, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
 
-    def run(widths):
-        tr = demo.DemoTransform([(s, w * s) for w in widths], chunk=s, topk=k, beta=0.9, lr=0.125, weight_decay=0.1, num_workers=1,
-                                grad_dtype=demo.DEMO_F32)
-        split = lambda t: [v.contiguous() for v in t.split([w * s for w in widths], dim=1)]  # noqa: E731
-        gs, ms, xs = split(g), split(0.5 * g), split(0.25 * g)
+    def run(first, count):
+        tr = demo.DemoTransform([(s, count * s)], chunk=s, topk=k, beta=0.9, lr=0.125, weight_decay=0.1, num_workers=1, grad_dtype=demo.DEMO_F32)
+        if per_sm == 6:
+            tr.set_decode_mode(demo.DEMO_AGG_COUNT_MEAN, demo.DEMO_PHI_SIGN)
+        part = g[:, first * s:(first + count) * s].contiguous()
+        gs, ms, xs = [part], [0.5 * part], [0.25 * part]
         pay = torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda")
         for _ in range(2):
             tr.compress(0, gs, ms, pay)
             tr.decode_apply([pay], xs)
         assert tr.device_status() == 0
         tr.close()
-        return pay, torch.cat(ms, 1), torch.cat(xs, 1)
+        return pay, ms[0], xs[0]
 
-    for a, b in zip(run([n]), run(cut)):
-        assert torch.equal(a, b)
+    whole = run(0, n)
+    parts = [run(first, min(sms, n - first)) for first in range(0, n, sms)]
+    assert torch.equal(whole[0], torch.cat([p[0] for p in parts]))
+    assert torch.equal(whole[1], torch.cat([p[1] for p in parts], 1))
+    assert torch.equal(whole[2], torch.cat([p[2] for p in parts], 1))
 
 
 @pytest.mark.parametrize("s,k,workers", [(32, 1, 2), (32, 40, 9), (64, 1, 3), (64, 33, 17), (64, 70, 5), (64, 600, 3)])
