@@ -49,13 +49,34 @@ struct Seg {
     }
 };
 
-// sum_u C[u][i] line[u], u in order.
+// Elements of a row of the basis that a thread has under way together on the way forward: a launch of few segments is the latency of the
+// table's lines.  (Not more at s = 64: with 64 elements a block's 80 registers per thread no longer fit beside the tiles' kernel where one of
+// its CTAs has left.)
 template <int S>
+constexpr int BATCH = S == 128 ? 64 : S < 32 ? S : 32;
+template <int B>
+__device__ __forceinline__ void load_column(float (&t)[B], const float *__restrict__ at, int stride)
+{
+#pragma unroll
+    for (int u = 0; u < B; ++u) t[u] = __ldg(at + u * stride);
+}
+// sum_u C[u][i] line[u], u in order.  AHEAD: 64 elements under way together (s = 128).
+template <int S, bool AHEAD>
 __device__ __forceinline__ float inverse_segment(const float *line, const float *__restrict__ C, int i)
 {
     float r = 0.f;
+    if constexpr (AHEAD) {
+#pragma unroll 1
+        for (int u0 = 0; u0 < S; u0 += 64) {
+            float t[64];
+            load_column(t, C + u0 * S + i, S);
+#pragma unroll
+            for (int u = 0; u < 64; ++u) r = fmaf(line[u0 + u], t[u], r);
+        }
+    } else {
 #pragma unroll 16
-    for (int u = 0; u < S; ++u) r = fmaf(line[u], __ldg(C + u * S + i), r);
+        for (int u = 0; u < S; ++u) r = fmaf(line[u], __ldg(C + u * S + i), r);
+    }
     return r;
 }
 
@@ -89,6 +110,15 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     }
     first.begin();
 
+    // row i of the basis, as a column of the transposed table (a warp reads 128 consecutive bytes; from the rows, 32 lines per read, sets with
+    // many segments of 128 took up to a third longer: 296 tiles of 128 x 128 and a vector of 37888, compress 43.4 us instead of 32.8), the
+    // first batch on its way beside the tensors' elements (32 elements at a time, none ahead: one segment of 128 10.8 us a call, now 5.2; from the
+    // rows 8.2; 5000 segments 41.0 / 40.8 / 103; of 64 4.6 / 3.6 / 5.2 and 14.8 / 13.3 / 37.8)
+    constexpr int B = BATCH<S>;
+    const float *Ct = a.C + S * S + (i < S ? i : 0);
+    float t[B];
+    load_column(t, Ct, S);
+
     // momentum update  b = beta*m + g  (Algorithm 1, worker side)
     float b = 0.f, q = 0.f;
     if (on) {
@@ -99,16 +129,17 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     Seg<S>::sync();
     // q = C b
     if (i < S) {
-        // (the transposed table: a warp reads 128 consecutive bytes; from the rows, 32 lines per read, sets with many segments of 128 took
-        // up to a third longer: 296 tiles of 128 x 128 and a vector of 37888, compress 43.4 us instead of 32.8)
-        const float *Ct = a.C + S * S + i;
-#pragma unroll 8
-        for (int n = 0; n < S; n += 4) {
-            const float4 x = *reinterpret_cast<const float4 *>(line + n);
-            q = fmaf(x.x, __ldg(Ct + n * S), q);
-            q = fmaf(x.y, __ldg(Ct + (n + 1) * S), q);
-            q = fmaf(x.z, __ldg(Ct + (n + 2) * S), q);
-            q = fmaf(x.w, __ldg(Ct + (n + 3) * S), q);
+#pragma unroll
+        for (int n0 = 0; n0 < S; n0 += B) {
+#pragma unroll
+            for (int n = 0; n < B; n += 4) {
+                const float4 x = *reinterpret_cast<const float4 *>(line + n0 + n);
+                q = fmaf(x.x, t[n], q);
+                q = fmaf(x.y, t[n + 1], q);
+                q = fmaf(x.z, t[n + 2], q);
+                q = fmaf(x.w, t[n + 3], q);
+            }
+            if (n0 + B < S) load_column(t, Ct + (n0 + B) * S, S);
         }
     }
     Seg<S>::sync();
@@ -168,11 +199,11 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     if (i < S) line[i] = keep ? a.alpha * q : 0.f;
     Seg<S>::sync();
     // m <- b - alpha C^T (kept)
-    if (on) m[off] = b - inverse_segment<S>(line, a.C, i);
+    if (on) m[off] = b - inverse_segment<S, S == 128>(line, a.C, i);
     Seg<S>::sync();
 }
 
-template <int S>
+template <int S, bool AHEAD>
 __device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long long c_own, float *line, unsigned short *senders, FirstRound &first)
 {
     constexpr int E = Seg<S>::E;
@@ -219,7 +250,7 @@ __device__ __forceinline__ void decode_segment(const DemoDecodeArgs &a, long lon
         Seg<S>::sync();
     }
     if (on) {
-        const float r = inverse_segment<S>(line, a.C, i);
+        const float r = inverse_segment<S, AHEAD>(line, a.C, i);
         if (a.sign_ptrs) {
             a.sign_ptrs[te.tensor][off] = (signed char)((r > 0.f) - (r < 0.f));
         } else {
@@ -501,7 +532,7 @@ __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArg
     first.begin();  // (a warp without a round)
 }
 
-template <int S, bool TILES>
+template <int S, bool TILES, bool AHEAD>
 __global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs segs, DemoDecodeArgs tiles, int seg_blocks)
 {
     const StreamOrder order(segs.wait_first);
@@ -514,7 +545,7 @@ __global__ void __launch_bounds__(THREADS) decode_small_kernel(DemoDecodeArgs se
         constexpr int PB = Seg<S>::PER_BLOCK;
         const int own = warp / Seg<S>::E;
         for (long long c0 = (long long)blockIdx.x * PB; c0 < segs.n_chunks; c0 += (long long)seg_blocks * PB)
-            decode_segment<S>(segs, c0 + own, mem[own], counts[own], first);
+            decode_segment<S, AHEAD>(segs, c0 + own, mem[own], counts[own], first);
     } else if constexpr (TILES) {
         const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
         const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
@@ -558,9 +589,16 @@ cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles
 {
     if constexpr (S <= 16) {
         if (tiles)
-            return launch((const void *)decode_small_kernel<S, true>, Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, dev, stream);
+            return launch((const void *)decode_small_kernel<S, true, false>, Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, dev, stream);
     }
-    return launch((const void *)decode_small_kernel<S, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, dev, stream);
+    // s = 128, up to two rounds of blocks: the inverse reads 64 elements of the basis ahead, with 46 registers per thread; beyond, other segments
+    // cover that latency, and with 32 registers the next kernel's blocks find room beside this one's (a decode call, ahead / not: one segment
+    // 4.1 / 5.2 us, 600 5.2 / 5.7, 1200 7.5 / 8.3, 2400 13.4 / 11.8, 5000 24.9 / 21.5).  Nor beside tiles, which cover it too (804 tiles and 32
+    // segments 44.9 / 44.2).
+    if constexpr (S == 128)
+        if (segs && segs->wait_first && segs->n_chunks <= 2LL * blocks_for(segs->n_chunks, Seg<S>::PER_BLOCK, dev.sm_count) * Seg<S>::PER_BLOCK)
+            return launch((const void *)decode_small_kernel<S, false, true>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, dev, stream);
+    return launch((const void *)decode_small_kernel<S, false, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, dev, stream);
 }
 
 }  // namespace

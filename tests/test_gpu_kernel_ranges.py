@@ -643,3 +643,65 @@ def test_compress_time_of_several_tensors_below_four_chunks_per_sm():
         del graph
         tr.close()
     assert times[36] <= 0.96 * times[40], times
+
+
+def _graph_time(calls, repeats=20):
+    """Device time of the captured calls, the shortest of ten loops."""
+    graph = torch.cuda.CUDAGraph()
+    calls()
+    with torch.cuda.graph(graph):
+        calls()
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = math.inf
+    for _ in range(10):
+        t0.record()
+        for _ in range(repeats):
+            graph.replay()
+        t1.record()
+        torch.cuda.synchronize()
+        best = min(best, t0.elapsed_time(t1))
+    return best
+
+
+def test_time_of_a_few_segments_of_128():
+    """Compress of one segment of 128 elements takes 1.4 times as long as of one of 64, whose table is a quarter as large (2.3 times where its
+    elements of the basis were fetched in four turns behind one another)."""
+    import paper_2411_19870_b200 as demo
+
+    times = {}
+    for s in (64, 128):
+        tr = demo.DemoTransform([(s,)], chunk=s, topk=8, beta=0.9, lr=0.1, weight_decay=0.1, num_workers=1)
+        g, m = [torch.randn(s, device="cuda").bfloat16()], [torch.randn(s, device="cuda")]
+        pay = torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda")
+        times[s] = _graph_time(lambda: [tr.compress(0, g, m, pay) for _ in range(4)])
+        tr.close()
+    assert times[128] <= 1.9 * times[64], times
+
+
+@pytest.mark.parametrize("counted", [False, True])
+def test_segments_of_128_in_two_rounds_and_more(counted):
+    """Decode of vectors at s = 128 has a form for up to two rounds of blocks and one for more: one vector of both kinds of length, and in halves
+    that take the first form, bit for bit."""
+    import paper_2411_19870_b200 as demo
+
+    sms, s, W = torch.cuda.get_device_properties(0).multi_processor_count, 128, 3
+    n = 16 * sms + 7
+    gen = torch.Generator("cuda").manual_seed(n)
+    g = [torch.randn(n * s, device="cuda", generator=gen) for _ in range(W)]
+
+    def run(first, count):
+        tr = demo.DemoTransform([(count * s,)], chunk=s, topk=9, beta=0.9, lr=0.125, weight_decay=0.1, num_workers=W, grad_dtype=demo.DEMO_F32)
+        tr.set_decode_mode(demo.DEMO_AGG_COUNT_MEAN if counted else demo.DEMO_AGG_SUM, demo.DEMO_PHI_IDENTITY)
+        gs = [v[first * s:(first + count) * s].contiguous() for v in g]
+        ms, x = [0.5 * v for v in gs], 0.25 * gs[0]
+        pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(W)]
+        for _ in range(2):
+            for w in range(W):
+                tr.compress(w, [gs[w]], [ms[w]], pay[w])
+            tr.decode_apply(pay, [x])
+        tr.close()
+        return torch.cat(ms), x
+
+    whole, parts = run(0, n), [run(0, n // 2), run(n // 2, n - n // 2)]
+    assert torch.equal(whole[1], torch.cat([p[1] for p in parts]))
+    assert torch.equal(whole[0].view(W, -1), torch.cat([p[0].view(W, -1) for p in parts], 1))
