@@ -665,6 +665,7 @@ __device__ __forceinline__ int first_listed(const DemoNdEntry &e)
     int a = 0;
     while (a < DEMO_ND_DIMS && e.s[a] == 1) ++a;
     if (a == DEMO_ND_DIMS || (e.tail && a == 2) || !in_place_extent(e.s[a]) || e.s[a] > 32) return -1;
+    if (e.M <= 128 * e.s[a]) return -1;  // a round of lines or less (8192 x 8192 in 16 x 32 2033 us listed, 1952 not; 28 M in 32 x 32 x 3 x 3 496 / 511)
     return a;
 }
 
