@@ -1175,10 +1175,8 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
         layout = s->e[0].layout;
         enter_layout(v, s->e[0], a.cls);
         __syncthreads();
-        if (a.tickets) {  // (where every chunk has a CTA, all would be requested in one moment: two calls, 296 of 64 x 48 52.0 us, 50.7 without)
-            prefetch_chunk(v, s->e[0], a.m_ptrs[s->e[0].tensor] + s->base[0]);
-            prefetch_chunk(v, s->e[0], static_cast<const GT *>(a.g_ptrs[s->e[0].tensor]) + s->base[0]);
-        }
+        prefetch_chunk(v, s->e[0], a.m_ptrs[s->e[0].tensor] + s->base[0]);
+        prefetch_chunk(v, s->e[0], static_cast<const GT *>(a.g_ptrs[s->e[0].tensor]) + s->base[0]);
     }
     order.begin();
 
@@ -1237,9 +1235,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) compre
         if (tid == T - 1) take_ticket(s, slot ^ 1, a.entries, a.cls, ticket);
         __syncthreads();
         transform_chunk<false, BIG>(tile0, tile1, slot, a.tables, -1);  // Q = T(B; C_0, ..., C_{d-1})
-        // the next chunk on its way to L2, where the chunks are large and the class does not stay there (two calls: 8192 x 8192 in 32 x 128 1865 us,
-        // 1911 without, 28 M elements in 32 x 32 x 3 x 3 496 / 506; 4096 x 4096 in 8 x 16 1397 / 1337, 4.7 M in 16 x 16 x 3 x 3 116.7 / 113.3)
-        if (e.M >= 1024 && a.cls.n_chunks * e.M >= 7 << 20 && (long long)gridDim.x + s->ticket < a.cls.n_chunks && s->e[slot ^ 1].layout == layout) {
+        if ((long long)gridDim.x + s->ticket < a.cls.n_chunks && s->e[slot ^ 1].layout == layout) {  // the next chunk on its way to L2
             const DemoNdEntry &ne = s->e[slot ^ 1];
             prefetch_chunk(v, ne, a.m_ptrs[ne.tensor] + s->base[slot ^ 1]);
             prefetch_chunk(v, ne, static_cast<const GT *>(a.g_ptrs[ne.tensor]) + s->base[slot ^ 1]);
@@ -1278,7 +1274,7 @@ __global__ void __launch_bounds__(BIG ? MAX_THREADS_BIG : MAX_THREADS, 2) decode
         layout = s->e[0].layout;
         enter_layout(v, s->e[0], a.cls);
         __syncthreads();
-        if (!a.sign_ptrs && a.tickets) prefetch_chunk(v, s->e[0], a.x_ptrs[s->e[0].tensor] + s->base[0]);
+        if (!a.sign_ptrs) prefetch_chunk(v, s->e[0], a.x_ptrs[s->e[0].tensor] + s->base[0]);
     }
     order.begin();
 
