@@ -315,10 +315,8 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) compress_tc_kernel(De
         if (sizeof(GT) == 4) prefetch_l2(ng + 32);
     };
     {
-        // (calls of several rounds only: where every pair has a group, all rows are requested in one moment and land late: two calls, 1184 chunks of
-        // 16 tensors 64.1 us, 58.5 without, 900 60.8 / 58.0, of one 54.5 / 53.7; 2400 of 40 158.9 / 168.4)
         const unsigned first = 2u * (blockIdx.x * GROUPS + threadIdx.x / PAIR_THREADS) + (threadIdx.x >> 6 & 1);
-        if (a.tickets && first < n_chunks) prefetch_row(first, threadIdx.x & 63, 0);
+        if (first < n_chunks) prefetch_row(first, threadIdx.x & 63, 0);
     }
     TcFrame f;
     tc_setup<GROUPS>(f, smem_raw, a.C, true, AREA, order);
@@ -441,7 +439,11 @@ __global__ void __launch_bounds__(GROUPS *PAIR_THREADS, 1) decode_tc_kernel(Demo
         prefetch_l2(xr);
         prefetch_l2(xr + 32);
     };
-    // (nothing of the first chunks in front of the wait: 592 chunks, k = 128 18.4 us, 17.8 without, 1184 19.2 / 18.5)
+    {
+        const unsigned first = 2u * (blockIdx.x * GROUPS + threadIdx.x / PAIR_THREADS) + (threadIdx.x >> 6 & 1);
+        int e0 = 0;
+        if (first < n_chunks) prefetch_row(locate<MANY>(a.entries, a.n_entries, first, k_eff, e0), threadIdx.x & 63);
+    }
     TcFrame f;
     tc_setup<GROUPS>(f, smem_raw, a.C, false, area, order);
     const int c = f.pt >> 6, r = f.pt & 63, lane = f.pt & 31, warp = (f.pt >> 5) & 1;

@@ -756,21 +756,3 @@ def test_first_chunks_of_128(n, tensors):
     parts = [run(g[128 * a:128 * b], m[128 * a:128 * b], [0, b - a]) for a, b in zip(ends, ends[1:])]
     assert torch.equal(whole[0], torch.cat([p[0] for p in parts]))
     assert torch.equal(whole[1], torch.cat([p[1] for p in parts]))
-
-
-def test_compress_time_of_a_full_round_of_pairs_under_a_callers_basis():
-    """1184 chunks, a group of the tensor-core kernel for every pair: of 16 tensors 1.07 of the time of one matrix (1.15 where the rows of all
-    pairs were sent to L2 in front of the wait)."""
-    import paper_2411_19870_b200 as demo
-
-    q = torch.from_numpy(np.linalg.qr(np.random.default_rng(3).standard_normal((64, 64)))[0]).float()
-    times = []
-    for tensors in (16, 1):
-        shapes = [(64 * (1184 // tensors), 64)] * tensors
-        tr = demo.DemoTransform(shapes, chunk=64, topk=32, beta=0.9, lr=0.1, weight_decay=0.1, num_workers=2)
-        tr.set_basis(q)
-        sets = [[[torch.randn(shape, device="cuda").to(d) for shape in shapes] for d in (torch.bfloat16, torch.float32)] for _ in range(2)]
-        pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(2)]
-        times.append(_graph_time(lambda: [tr.compress(w, g, m, pay[w]) for w, (g, m) in enumerate(sets)]))
-        tr.close()
-    assert times[0] <= 1.11 * times[1], times
