@@ -124,8 +124,7 @@ constexpr size_t compress128_smem()
     return compress128_tile_bytes<GT>() + (256 + 8 + 4) * 4 + RECS128 * 16 + 3 * CAP128P * 4 + 16 + 16;
 }
 
-// AHEAD: the first tiles go to L2 in front of the wait (demo_launch_compress_fast128 says when).
-template <typename GT, bool AHEAD>
+template <typename GT>
 __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompressArgs a)
 {
     const StreamOrder order(a.wait_first);
@@ -182,7 +181,7 @@ __global__ void __launch_bounds__(THREADS, 2) compress_fast128_kernel(DemoCompre
     if (c < a.n_chunks) {
         cur.seek(a.entries, a.n_entries, c);
         acquire_maps(cur.te);
-        if (AHEAD && tid == 0) issue_tile(cur.te, c, false, true);
+        if (tid == 0) issue_tile(cur.te, c, false, true);
     }
     order.begin();
     if (tid == 0 && c < a.n_chunks) {
@@ -888,13 +887,9 @@ cudaError_t launch128(K kernel, size_t smem, DemoLaunch &dev, cudaStream_t strea
 cudaError_t demo_launch_compress_fast128(const DemoCompressArgs &a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (!a.tmap_m || !a.tmap_g) return cudaErrorNotSupported;
-    if (!a.grad_bf16) return launch128(compress_fast128_kernel<float, true>, compress128_smem<float>(), dev, stream, a);
-    // Tiles sent to L2 in front of the wait spare every call their latency, except where the two CTAs of every SM request their first ones in one
-    // moment, up to one and a half rounds, from one or two tensors with bf16 gradients (two calls, ahead / not: 248 chunks, k = 16 39.1 / 36.8 us,
-    // 296, k = 24 40.0 / 38.1, 440, k = 4 56.5 / 55.0; of 16 tensors 240 37.1 / 38.0; fp32, one CTA per SM, 440 74.1 / 77.1; 592, k = 4 71.5 / 72.0).
-    const bool ahead = a.n_entries > 2 || a.n_chunks <= dev.sm_count || a.n_chunks > 3LL * dev.sm_count;
-    return launch128(ahead ? compress_fast128_kernel<__nv_bfloat16, true> : compress_fast128_kernel<__nv_bfloat16, false>,
-                     compress128_smem<__nv_bfloat16>(), dev, stream, a);
+    if (a.grad_bf16)
+        return launch128(compress_fast128_kernel<__nv_bfloat16>, compress128_smem<__nv_bfloat16>(), dev, stream, a);
+    return launch128(compress_fast128_kernel<float>, compress128_smem<float>(), dev, stream, a);
 }
 
 cudaError_t demo_launch_decode_fast128(const DemoDecodeArgs &a, DemoLaunch &dev, cudaStream_t stream)

@@ -722,37 +722,3 @@ def test_compress_time_of_a_full_round_of_chunks_of_32():
     """2960 chunks of 16 tensors, a warp each on the whole device, take 0.42 of the time of 9000 (0.52 where all of them were requested at once)."""
     times = [_compress_time([(32 * 185, 32)] * 16, 32, 4), _compress_time([(32 * 9000, 32)], 32, 4)]
     assert times[0] <= 0.47 * times[1], times
-
-
-def test_compress_time_of_less_than_a_round_of_chunks_of_128():
-    """248 chunks, two on most SMs, take 0.49 of the time of 592 (0.52 where their tiles were sent to L2 at once in front of the wait)."""
-    times = [_compress_time([(128 * n // 8, 1024)], 128, 16) for n in (248, 592)]
-    assert times[0] <= 0.506 * times[1], times
-
-
-@pytest.mark.parametrize("n", [148, 149, 296, 297, 444, 445])
-@pytest.mark.parametrize("tensors", [1, 2, 3])
-def test_first_chunks_of_128(n, tensors):
-    """bf16 gradients: where the first tiles are requested depends on the number of chunks and tensors, records and momentum do not, bit for bit."""
-    import paper_2411_19870_b200 as demo
-
-    gen = torch.Generator("cuda").manual_seed(n)
-    g = torch.randn((128 * n, 128), device="cuda", generator=gen).bfloat16()
-    m = torch.randn((128 * n, 128), device="cuda", generator=gen)
-
-    def run(g, m, cuts):
-        shapes = [(128 * (b - a), 128) for a, b in zip(cuts, cuts[1:])]
-        tr = demo.DemoTransform(shapes, chunk=128, topk=5, beta=0.9, lr=0.1, weight_decay=0.0, num_workers=1)
-        gs, ms = ([t[128 * a:128 * b].clone() for a, b in zip(cuts, cuts[1:])] for t in (g, m))
-        pay = torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda")
-        for _ in range(2):
-            tr.compress(0, gs, ms, pay)
-        assert tr.device_status() == 0
-        tr.close()
-        return torch.cat(ms), pay
-
-    whole = run(g, m, [n * i // tensors for i in range(tensors)] + [n])
-    ends = list(range(0, n, 100)) + [n]
-    parts = [run(g[128 * a:128 * b], m[128 * a:128 * b], [0, b - a]) for a, b in zip(ends, ends[1:])]
-    assert torch.equal(whole[0], torch.cat([p[0] for p in parts]))
-    assert torch.equal(whole[1], torch.cat([p[1] for p in parts]))
