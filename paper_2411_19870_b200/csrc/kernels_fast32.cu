@@ -95,13 +95,10 @@ __device__ __forceinline__ unsigned search_all(const float (&q)[S], unsigned bou
     return gt | eq;
 }
 
-// LATE: the first chunk is looked up and requested behind the tensor-memory allocation (launch32 says when), an instantiation of its own: as a
-// branch it cost 2 to 5 %.
-template <typename GT, bool BIGK, bool LATE>
+template <typename GT, bool BIGK>
 __global__ void __launch_bounds__(WARPS * 32, CTAS) compress32_kernel(DemoCompressArgs a)
 {
     const StreamOrder order(a.wait_first);
-    if constexpr (LATE) order.begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int t = threadIdx.x & 31;
     Area<GT> &w = reinterpret_cast<Area<GT> *>(smem_raw)[threadIdx.x >> 5];
@@ -155,19 +152,17 @@ __global__ void __launch_bounds__(WARPS * 32, CTAS) compress32_kernel(DemoCompre
 
     unsigned c = blockIdx.x * WARPS + (threadIdx.x >> 5);
     Place<GT> p;
-    if constexpr (!LATE) {
-        if (c < n_chunks) {
-            p = locate(c);
-            prefetch_l2(p.m + (size_t)t * p.n1);
-            prefetch_l2(p.g + (size_t)t * p.n1);
-        }
-        order.begin();
-        if (!BIGK && c < n_chunks) fetch(p);
-        __syncwarp();
+    if (c < n_chunks) {
+        p = locate(c);
+        prefetch_l2(p.m + (size_t)t * p.n1);
+        prefetch_l2(p.g + (size_t)t * p.n1);
     }
+    order.begin();
+    if (!BIGK && c < n_chunks) fetch(p);
+    __syncwarp();
     const uint32_t tmem = tmem_alloc_cta(tmem_slot, S);
     const uint32_t taddr = tmem + ((threadIdx.x & ~31u) << 16);  // this warp's lanes: column t of B, parked for the residual
-    if ((BIGK || LATE) && c < n_chunks) {  // (with the place kept across the allocation the code comes out 5 to 20 % slower)
+    if (BIGK && c < n_chunks) {  // (with the place kept across the allocation the code comes out 5 to 20 % slower)
         p = locate(c);
         fetch(p);
     }
@@ -391,7 +386,10 @@ template <typename GT, bool BIGK>
 cudaError_t launch32(DemoCompressArgs a, DemoLaunch &dev, cudaStream_t stream)
 {
     if (a.n_chunks <= 0) return cudaSuccess;
+    const void *kernel = (const void *)compress32_kernel<GT, BIGK>;
     const size_t smem = sizeof(Area<GT>) * WARPS + 16;
+    const cudaError_t err = demo_allow_smem(dev, kernel);
+    if (err != cudaSuccess) return err;
     // by registers and shared memory (1 KB reserved per CTA; tensor memory has room for sixteen, the occupancy calculator
     // does not know about it)
     const int by_smem = (int)(227u * 1024u / (smem + 1024u)), per_sm = by_smem < CTAS ? by_smem : CTAS;
@@ -401,16 +399,6 @@ cudaError_t launch32(DemoCompressArgs a, DemoLaunch &dev, cudaStream_t stream)
         grid = n_ctas;
         a.tickets = nullptr;
     }
-    // The look-up in front of the wait and the tiles' way to L2 from there spare every call their latency, except where the warps of the first
-    // round request so many tiles in one moment that they land late: from two CTAs per SM (below, 1000 chunks of one tensor, k = 24 13.9 us early,
-    // 14.2 late) up to two and a half rounds (beyond, the call is long enough: 9000 50.7 / 51.7).  Two calls, early / late:
-    // 1200 chunks of one tensor 14.4 / 13.9, 2960 21.6 / 20.0, of 16 tensors 26.0 / 21.4, 5500 34.7 / 32.8, 7300 40.5 / 39.9.  Not above k = 32
-    // (6500, k = 100 65.0 / 68.2), where the tiles are requested behind the allocation anyway.
-    const void *kernel = (const void *)compress32_kernel<GT, BIGK, false>;
-    if constexpr (!BIGK)
-        if (n_ctas > 2LL * dev.sm_count && 2 * n_ctas <= 5LL * dev.sm_count * per_sm) kernel = (const void *)compress32_kernel<GT, false, true>;
-    const cudaError_t err = demo_allow_smem(dev, kernel);
-    if (err != cudaSuccess) return err;
     void *params[] = {&a};
     return demo_launch_kernel(kernel, grid, WARPS * 32, smem, stream, params);
 }

@@ -705,20 +705,3 @@ def test_segments_of_128_in_two_rounds_and_more(counted):
     whole, parts = run(0, n), [run(0, n // 2), run(n // 2, n - n // 2)]
     assert torch.equal(whole[1], torch.cat([p[1] for p in parts]))
     assert torch.equal(whole[0].view(W, -1), torch.cat([p[0].view(W, -1) for p in parts], 1))
-
-
-def _compress_time(shapes, s, k):
-    import paper_2411_19870_b200 as demo
-
-    tr = demo.DemoTransform(shapes, chunk=s, topk=k, beta=0.9, lr=0.1, weight_decay=0.1, num_workers=2)
-    sets = [[[torch.randn(shape, device="cuda").to(d) for shape in shapes] for d in (torch.bfloat16, torch.float32)] for _ in range(2)]
-    pay = [torch.zeros(tr.payload_bytes, dtype=torch.uint8, device="cuda") for _ in range(2)]
-    best = _graph_time(lambda: [tr.compress(w, g, m, pay[w]) for w, (g, m) in enumerate(sets)])
-    tr.close()
-    return best
-
-
-def test_compress_time_of_a_full_round_of_chunks_of_32():
-    """2960 chunks of 16 tensors, a warp each on the whole device, take 0.42 of the time of 9000 (0.52 where all of them were requested at once)."""
-    times = [_compress_time([(32 * 185, 32)] * 16, 32, 4), _compress_time([(32 * 9000, 32)], 32, 4)]
-    assert times[0] <= 0.47 * times[1], times
