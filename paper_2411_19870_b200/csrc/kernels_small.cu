@@ -91,7 +91,7 @@ struct FirstRound {
     }
 };
 
-template <int S>
+template <int S, bool AHEAD>
 __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long long c_own, float *line, FirstRound &first)
 {
     constexpr int E = Seg<S>::E;
@@ -113,11 +113,10 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     // row i of the basis, as a column of the transposed table (a warp reads 128 consecutive bytes; from the rows, 32 lines per read, sets with
     // many segments of 128 took up to a third longer: 296 tiles of 128 x 128 and a vector of 37888, compress 43.4 us instead of 32.8), the
     // first batch on its way beside the tensors' elements (32 elements at a time, none ahead: one segment of 128 10.8 us a call, now 5.2; from the
-    // rows 8.2; 5000 segments 41.0 / 40.8 / 103; of 64 4.6 / 3.6 / 5.2 and 14.8 / 13.3 / 37.8)
-    constexpr int B = BATCH<S>;
+    // rows 8.2; of 64 1 / 5000 segments 4.6 / 14.8, 3.6 / 13.3, 5.2 / 37.8)
     const float *Ct = a.C + S * S + (i < S ? i : 0);
-    float t[B];
-    load_column(t, Ct, S);
+    float t[BATCH<S>];
+    if constexpr (AHEAD) load_column(t, Ct, S);
 
     // momentum update  b = beta*m + g  (Algorithm 1, worker side)
     float b = 0.f, q = 0.f;
@@ -129,17 +128,29 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     Seg<S>::sync();
     // q = C b
     if (i < S) {
+        if constexpr (AHEAD) {
+            constexpr int B = BATCH<S>;
 #pragma unroll
-        for (int n0 = 0; n0 < S; n0 += B) {
+            for (int n0 = 0; n0 < S; n0 += B) {
 #pragma unroll
-            for (int n = 0; n < B; n += 4) {
-                const float4 x = *reinterpret_cast<const float4 *>(line + n0 + n);
-                q = fmaf(x.x, t[n], q);
-                q = fmaf(x.y, t[n + 1], q);
-                q = fmaf(x.z, t[n + 2], q);
-                q = fmaf(x.w, t[n + 3], q);
+                for (int n = 0; n < B; n += 4) {
+                    const float4 x = *reinterpret_cast<const float4 *>(line + n0 + n);
+                    q = fmaf(x.x, t[n], q);
+                    q = fmaf(x.y, t[n + 1], q);
+                    q = fmaf(x.z, t[n + 2], q);
+                    q = fmaf(x.w, t[n + 3], q);
+                }
+                if (n0 + B < S) load_column(t, Ct + (n0 + B) * S, S);
             }
-            if (n0 + B < S) load_column(t, Ct + (n0 + B) * S, S);
+        } else {
+#pragma unroll 8
+            for (int n = 0; n < S; n += 4) {
+                const float4 x = *reinterpret_cast<const float4 *>(line + n);
+                q = fmaf(x.x, __ldg(Ct + n * S), q);
+                q = fmaf(x.y, __ldg(Ct + (n + 1) * S), q);
+                q = fmaf(x.z, __ldg(Ct + (n + 2) * S), q);
+                q = fmaf(x.w, __ldg(Ct + (n + 3) * S), q);
+            }
         }
     }
     Seg<S>::sync();
@@ -199,7 +210,7 @@ __device__ __forceinline__ void compress_segment(const DemoCompressArgs &a, long
     if (i < S) line[i] = keep ? a.alpha * q : 0.f;
     Seg<S>::sync();
     // m <- b - alpha C^T (kept)
-    if (on) m[off] = b - inverse_segment<S, S == 128>(line, a.C, i);
+    if (on) m[off] = b - inverse_segment<S, S == 128 && AHEAD>(line, a.C, i);
     Seg<S>::sync();
 }
 
@@ -510,7 +521,7 @@ __device__ __forceinline__ void decode_tiles(const DemoDecodeArgs &a, long long 
 template <int S, bool TILES>
 constexpr int warp_floats() { return TILES && Tile<S>::FLOATS > Seg<S>::PAD ? Tile<S>::FLOATS : Seg<S>::PAD; }
 
-template <int S, typename GT, bool TILES>
+template <int S, typename GT, bool TILES, bool AHEAD>
 __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArgs segs, DemoCompressArgs tiles, int seg_blocks)
 {
     const StreamOrder order(segs.wait_first);
@@ -522,7 +533,7 @@ __global__ void __launch_bounds__(THREADS) compress_small_kernel(DemoCompressArg
         constexpr int PB = Seg<S>::PER_BLOCK;
         const int own = warp / Seg<S>::E;
         for (long long c0 = (long long)blockIdx.x * PB; c0 < segs.n_chunks; c0 += (long long)seg_blocks * PB)
-            compress_segment<S>(segs, c0 + own, mem[own], first);
+            compress_segment<S, AHEAD>(segs, c0 + own, mem[own], first);
     } else if constexpr (TILES) {
         const long long groups = (tiles.n_chunks + Tile<S>::PER_WARP - 1) / Tile<S>::PER_WARP;
         const long long stride = (long long)(gridDim.x - seg_blocks) * WARPS;
@@ -573,16 +584,28 @@ cudaError_t launch(const void *kernel, int segs_per_block, int tiles_per_warp, c
     return demo_launch_kernel(kernel, seg_blocks + tile_blocks, THREADS, 0, stream, params);
 }
 
+// At most two rounds of blocks.
+template <int S>
+bool few_rounds(long long n_segs, const DemoLaunch &dev)
+{
+    return n_segs <= 2LL * blocks_for(n_segs, Seg<S>::PER_BLOCK, dev.sm_count) * Seg<S>::PER_BLOCK;
+}
+
 template <int S>
 cudaError_t compress_small(const DemoCompressArgs *segs, const DemoCompressArgs *tiles, DemoLaunch &dev, cudaStream_t stream)
 {
     if constexpr (S <= 16) {
         if (tiles)
-            return launch(tiles->grad_bf16 ? (const void *)compress_small_kernel<S, __nv_bfloat16, true>
-                                           : (const void *)compress_small_kernel<S, float, true>,
+            return launch(tiles->grad_bf16 ? (const void *)compress_small_kernel<S, __nv_bfloat16, true, true>
+                                           : (const void *)compress_small_kernel<S, float, true, true>,
                           Seg<S>::PER_BLOCK, Tile<S>::PER_WARP, segs, tiles, dev, stream);
     }
-    return launch((const void *)compress_small_kernel<S, float, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoCompressArgs *)nullptr, dev, stream);
+    // s = 128: a batch of 64 elements ahead up to two rounds of blocks; beyond, other segments cover the latency, and with half the registers
+    // sixteen blocks of an SM instead of eight do (two calls and a decode, data not in L2, 4000 segments 101 us ahead, 92 not, 1000 28 / 29).
+    if constexpr (S == 128)
+        if (segs && !few_rounds<S>(segs->n_chunks, dev))
+            return launch((const void *)compress_small_kernel<S, float, false, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoCompressArgs *)nullptr, dev, stream);
+    return launch((const void *)compress_small_kernel<S, float, false, true>, Seg<S>::PER_BLOCK, 1, segs, (const DemoCompressArgs *)nullptr, dev, stream);
 }
 template <int S>
 cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles, DemoLaunch &dev, cudaStream_t stream)
@@ -596,7 +619,7 @@ cudaError_t decode_small(const DemoDecodeArgs *segs, const DemoDecodeArgs *tiles
     // 4.1 / 5.2 us, 600 5.2 / 5.7, 1200 7.5 / 8.3, 2400 13.4 / 11.8, 5000 24.9 / 21.5).  Nor beside tiles, which cover it too (804 tiles and 32
     // segments 44.9 / 44.2).
     if constexpr (S == 128)
-        if (segs && segs->wait_first && segs->n_chunks <= 2LL * blocks_for(segs->n_chunks, Seg<S>::PER_BLOCK, dev.sm_count) * Seg<S>::PER_BLOCK)
+        if (segs && segs->wait_first && few_rounds<S>(segs->n_chunks, dev))
             return launch((const void *)decode_small_kernel<S, false, true>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, dev, stream);
     return launch((const void *)decode_small_kernel<S, false, false>, Seg<S>::PER_BLOCK, 1, segs, (const DemoDecodeArgs *)nullptr, dev, stream);
 }
