@@ -458,13 +458,13 @@ cudaError_t launch64(const DemoCompressArgs &a, long long largest, DemoLaunch &d
     // look-ups spread the requests.  Steps, early / late / before both: 280 chunks of 9 tensors, seven workers 92.5 / 99.9 / 101.7 us; 800 of
     // 23, two workers 48.1 / 44.3 / 46.0; 976 of 57, six workers 135 / 120 / 120; 1424 of 30, six workers 170.5 / 158.5 / 167.1; 2400 of 65,
     // two workers 91.8 / 85.3 / 88.0; 2640 of 72, one worker 60.3 / 60.2 / 63.1; 3328 of 58, three workers 171 / 178 / 173.
-    // The line lies at four chunks per SM; the more maps, the lower: at three with more than four tensors, at two with more than sixteen, where no
-    // tensor holds more than three quarters of the chunks (few maps again).  Three workers, 540 of 60 46.0 / 39.1 / 39.2, of 9 41.1 / 39.1 /
-    // 39.2, 360 of 60 39.2 / 36.9 / 37.0, 375 of 5 35.1 / 36.9 / 37.0, 432 of 15 39.0 / 41.1 / 41.1 (but 340 of 15 37.0 / 35.1 / 35.2); two, 448 of 64
-    // 35.9 / 31.5 / 33.2, 556 of 15, 500 of them in one, 35.4 / 36.7 / 37.4; four, 576 of 36 67.7 / 60.8 / 63.0, 400 of 4 51.3 / 55.4 / 56.0.  (Not
-    // in the transform domain: 440 of 15, three workers 42.4 early, 43.6 late.)
-    const bool spread = 4 * largest <= 3 * a.n_chunks && !a.momentum_dct;
-    const long long line = (spread && a.n_entries > 16 ? 2LL : spread && a.n_entries > 4 ? 3LL : 4LL) * dev.sm_count;
+    // The line lies at four chunks per SM, with more than four tensors at three and a quarter, where no tensor holds more than three quarters of
+    // the chunks (few maps again).  Steps of two workers, data not in L2: 540 chunks of 60 37.9 / 35.3 / 37.3, of 9 34.7 / 33.6 / 34.9, 500 of 20
+    // 34.6 / 33.7 / 35.3, but 450 of 10 31.7 / 32.3 / 33.9, 360 of 40 31.4 / 32.4 / 34.3; compress of three, data in L2: 540 of 60 46.0 / 39.1 /
+    // 39.2, 375 of 5 35.1 / 36.9 / 37.0, two, 556 of 15, 500 of them in one, 35.4 / 36.7 / 37.4.  (Not in the transform domain: 440 of 15, three
+    // workers 42.4 early, 43.6 late.)
+    const bool spread = a.n_entries > 4 && 4 * largest <= 3 * a.n_chunks && !a.momentum_dct;
+    const long long line = (spread ? 13LL : 16LL) * dev.sm_count / 4;
     b.late_lookup = a.n_entries > 1 && 2 * groups <= 5 * grid && grid > line;
     void *params[] = {&b};
     return demo_launch_kernel((const void *)kernel, grid, THREADS, smem, stream, params);
