@@ -13,7 +13,9 @@
  *
  * Streams: everything of a call runs on cuda_stream.  When a context holds both 2-D and 1-D tensors, the kernels of the
  * two run side by side (programmatic dependent launch), and a kernel of this library may be resident on the device before
- * the work queued before it has finished, but touches nothing until then: the caller sees plain stream order.
+ * the work queued before it has finished.  Until then it reads the context's own tables (tensors, pointers, tensor maps: which no
+ * kernel writes) and asks for the first tiles of the caller's tensors to be brought to L2; it loads nothing of theirs into an SM and
+ * writes nothing, so the caller sees plain stream order.
  *
  * CUDA graphs: demo_compress and demo_decode_apply copy their pointer arrays to device tables only
  * when a pointer differs from the previous call with the same worker index.  After one ordinary call
