@@ -18,7 +18,7 @@
 //     of eight elements per thread -- of sixteen, in quads, where the rows are whole 16-byte pieces -- are issued together; the next
 //     chunk's rows are on their way to L2 during the selection;
 //   * addresses along a line are byte offsets, one instruction each, and on a last axis of whole quads four elements one access;
-//   * the first axis of the inverse is transformed only along the lines that hold kept coefficients;
+//   * the first axis of the inverse is transformed only along the lines that hold kept coefficients, where it has more than 128 lines;
 //   * top-k: the k-th largest of the threads' maxima (from a histogram relative to the largest) bounds the k-th coefficient;
 //     the few dozen to few hundred coefficients above it are listed, one warp finds the k-th among them, and the kept ones
 //     are put in index order by counting or, where much of a chunk is kept, by going over the tile; radix select only when the
